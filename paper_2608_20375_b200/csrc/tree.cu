@@ -649,7 +649,9 @@ __global__ void __launch_bounds__(TREE_THREADS) tree_kernel(const TreeParams p) 
     __shared__ int rows_abort;
     const int rows_pre = p.rows_pre;
     const int ne = rows_pre * K * K;  // entries that come from the edge-score kernel for every sequence
-    const bool bulk = ne > 0 && (ne % 16) == 0;
+    // (a bulk copy's source and size are multiples of 16 bytes: the child ranks are bytes, so the entries copied and the
+    // entries between two sequences both have to be multiples of 16 -- L = 11, K = 10 with 8 rows ahead has 800 and 1100)
+    const bool bulk = ne > 0 && (ne % 16) == 0 && (L * K * K) % 16 == 0;
     // the prologue's loads from global memory are all issued before the first of them is used: one round trip
     const int root = p.root_token[b];
     const float lp_top = p.rows_adaptive ? deep_tree_load(p.topk_lp + (size_t)b * L * K, L, K) : 0.f;

@@ -547,6 +547,25 @@ def test_round_does_not_depend_on_the_edge_rows_split(kw):
     g.destroy()
 
 
+@pytest.mark.parametrize("L,K", [(11, 10), (9, 6), (13, 18), (12, 10)])
+@pytest.mark.parametrize("beta", [0.2, 0.0])
+def test_round_rows_of_a_sequence_off_the_16_byte_grid(L, K, beta):
+    """Eight depths scored ahead are a multiple of 16 entries while a sequence's rows, L K K entries, are not (the last
+    shape: both are): the rows of every second sequence then start off the grid that bulk copies need."""
+    w = gi.small(batch=5, L=L, V=5003, K=K, budget_min=16, budget_max=128, budget_step=16, logits_dtype="bf16", m=64,
+                 hidden_dim=40, beta=beta)
+    g = _graft(w)
+    tb, saba_kw, keep = _setup(w, g)
+    x = gi.batch_inputs(w)
+    out, gpu = gpu_round(g, w, x)
+    compare_round(oracle, w, x, tb, saba_kw, gpu, oracle_round(oracle, w, x, tb, saba_kw))
+    _, gpu2 = gpu_round(g, w, x, debug=False)  # (eight rows ahead; with the score array asked for, all L)
+    for k in ("n_nodes", "budget", "status", "token", "parent", "depth", "position", "path_score", "mask"):
+        assert np.array_equal(gpu[k], gpu2[k]), k
+    compare_accept(oracle, gi, g, w, out, gpu)
+    g.destroy()
+
+
 @pytest.mark.parametrize("kw", _SPLIT_CASES[:3] + [
     dict(batch=3, L=16, V=6000, K=32, budget_min=32, budget_max=512, budget_step=16, m=512, hidden_dim=64)])
 @pytest.mark.parametrize("rows", [0, None])
