@@ -248,31 +248,31 @@ graft_status graft_tdes_precompute(graft_ctx* ctx, const void* d_emb, graft_dtyp
                                    const float* d_W, const float* d_b, float* d_out, void* stream) {
     if (!ctx || !d_emb || !d_W || !d_out || E < 1) return GRAFT_ERR_INVALID_ARG;
     if (emb_dtype != GRAFT_F32 && emb_dtype != GRAFT_BF16) return GRAFT_ERR_INVALID_ARG;
-    // bf16 embeddings: the tensor cores (the embeddings are exact operands, W goes in as three bf16 parts); its
-    // scratch is allocated on the first such call (this is the once-per-model setup step, not the round)
-    if (emb_dtype == GRAFT_BF16) {
-        const size_t need = tables_tc_scratch_bytes(ctx->cfg.V, E, ctx->cfg.m);
-        if (need > 0) {
-            if (ctx->tables_scratch_bytes < need) {
-                if (ctx->tables_scratch) cudaFree(ctx->tables_scratch);
-                ctx->tables_scratch = nullptr;
-                ctx->tables_scratch_bytes = 0;
-                if (cudaMalloc(&ctx->tables_scratch, need) != cudaSuccess) {
-                    cudaGetLastError();
-                    return GRAFT_ERR_WORKSPACE;
-                }
-                ctx->tables_scratch_bytes = need;
+    // the tensor cores (bf16 parts of the inputs, exact products); their scratch is allocated on the first call (this is
+    // the once-per-model setup step, not the round)
+    if (tables_mma_fits(d_emb, emb_dtype, E, d_out)) {
+        const size_t need = tables_mma_scratch_bytes(ctx->num_sms, E, ctx->cfg.m);
+        if (ctx->tables_scratch_bytes < need) {
+            if (ctx->tables_scratch) cudaFree(ctx->tables_scratch);
+            ctx->tables_scratch = nullptr;
+            ctx->tables_scratch_bytes = 0;
+            if (cudaMalloc(&ctx->tables_scratch, need) != cudaSuccess) {
+                cudaGetLastError();
+                return GRAFT_ERR_WORKSPACE;
             }
-            int n = 0;
-            const cudaError_t e = tables_tc_launch(d_emb, ctx->cfg.V, E, ctx->cfg.m, d_W, d_b, d_out, ctx->tables_scratch, &n,
-                                               (cudaStream_t)stream);
-            ctx->launches += (uint64_t)n;
-            if (e == cudaSuccess) return GRAFT_OK;
-            if (e != cudaErrorNotSupported) {
+            ctx->tables_scratch_bytes = need;
+            if (cudaMemsetAsync(ctx->tables_scratch, 0, tables_mma_counter_bytes(ctx->num_sms), (cudaStream_t)stream) !=
+                cudaSuccess) {
                 cudaGetLastError();
                 return GRAFT_ERR_CUDA;
             }
         }
+        if (tables_mma_launch(ctx, d_emb, emb_dtype, E, d_W, d_b, d_out, ctx->tables_scratch, (cudaStream_t)stream) !=
+            cudaSuccess) {
+            cudaGetLastError();
+            return GRAFT_ERR_CUDA;
+        }
+        return GRAFT_OK;
     }
     if (tdes_precompute_launch(ctx, d_emb, emb_dtype, E, d_W, d_b, d_out, (cudaStream_t)stream) != cudaSuccess)
         return GRAFT_ERR_CUDA;
