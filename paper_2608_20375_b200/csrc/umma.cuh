@@ -54,6 +54,14 @@ __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst_smem, const void* 
         "l"(map), "r"(x), "r"(y), "r"(bar)
         : "memory");
 }
+// The same with a barrier of this CTA.
+__device__ __forceinline__ void tma_load_2d(uint32_t dst_smem, const void* map, int x, int y, uint32_t bar) {
+    asm volatile(
+        "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(
+            dst_smem),
+        "l"(map), "r"(x), "r"(y), "r"(bar)
+        : "memory");
+}
 __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
 // ---- TMEM ------------------------------------------------------------------------------------------------------
