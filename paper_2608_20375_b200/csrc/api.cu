@@ -261,11 +261,6 @@ graft_status graft_tdes_precompute(graft_ctx* ctx, const void* d_emb, graft_dtyp
                 return GRAFT_ERR_WORKSPACE;
             }
             ctx->tables_scratch_bytes = need;
-            if (cudaMemsetAsync(ctx->tables_scratch, 0, tables_mma_counter_bytes(ctx->num_sms), (cudaStream_t)stream) !=
-                cudaSuccess) {
-                cudaGetLastError();
-                return GRAFT_ERR_CUDA;
-            }
         }
         if (tables_mma_launch(ctx, d_emb, emb_dtype, E, d_W, d_b, d_out, ctx->tables_scratch, (cudaStream_t)stream) !=
             cudaSuccess) {

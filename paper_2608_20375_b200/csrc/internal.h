@@ -91,7 +91,7 @@ struct graft_ctx {
     double* w_fit;                // [32] normal equations of graft_saba_fit and its arrival counter, zero between calls
     int32_t* w_errflag;           // [1] device-side internal error flag
     graft::VpPlan vp_plan;
-    // scratch of the tensor-core table precompute (allocated on its first use: counters, pieces of split tiles, W's bf16 parts)
+    // scratch of the tensor-core table precompute (allocated on its first use: pieces of split tiles, W's bf16 parts)
     void* tables_scratch;
     size_t tables_scratch_bytes;
     // host-buffer staging (allocated on first use of graft_build_trees_host)
@@ -138,7 +138,6 @@ cudaError_t tdes_precompute_launch(graft_ctx* ctx, const void* d_emb, graft_dtyp
                                    const float* d_b, float* d_out, cudaStream_t st);
 // table precompute on the tensor cores (csrc/tables_mma.cu); inputs that do not fit go to tdes_precompute_launch
 bool tables_mma_fits(const void* d_emb, graft_dtype dt, int E, const void* d_out);
-size_t tables_mma_counter_bytes(int num_sms);
 size_t tables_mma_scratch_bytes(int num_sms, int E, int m);
 cudaError_t tables_mma_launch(graft_ctx* ctx, const void* d_emb, graft_dtype dt, int E, const float* d_W, const float* d_b,
                               float* d_out, void* scratch, cudaStream_t st);

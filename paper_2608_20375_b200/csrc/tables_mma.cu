@@ -18,7 +18,7 @@
 // W1 and W2 stand side by side as one operand of N = 256 (M = 256, N = 128 takes as long as N = 256: 128 cycles measured),
 // W3 is an N = 128 of its own.  Tiles of 512 rows halve the passes over W, which comes from L2 every time.  The
 // embeddings are read from memory once; nothing but the tables is written.  What is left when the tiles do not divide
-// by the pairs is dealt out along E in equal shares, and the pair that finishes a tile's last piece adds them up in order.
+// by the pairs is dealt out along E in equal shares, whose sums a small kernel adds up in order.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -29,26 +29,53 @@
 namespace graft {
 namespace {
 
-constexpr int kTmBlk = 64;            // columns of E per ring stage: one 128-byte row of bf16
-constexpr int kTmPart = 128 * 128;    // bytes of 128 rows of bf16 in a stage
-constexpr int kTmW = 3 * 64 * 128;    // bytes of W in a stage: W1 (even CTA) or W2 (odd CTA), and half of W3
 constexpr int kTmEpiWarps = 8;
 constexpr int kTmConvWarps = 8;
-constexpr int kTmMaxSplit = 8;        // pairs that share a left-over tile, about
+constexpr int kTmMaxSplit = 16;  // pairs that share a left-over tile, about
 
+// Ring sizes: what a block's copies need in flight (about 2 us of them) beside the blocks being worked on, in 227 KB.
 template <bool F32>
 struct TablesCfg {
-    static constexpr int MT = F32 ? 1 : 2;          // row blocks of 128 a CTA works on at a time
-    static constexpr int ROWS = 256 * MT;           // rows of V per tile
-    static constexpr int CHUNK = F32 ? 2 : 8;       // ring stages between two emptyings of an accumulator
-    static constexpr int STAGES = F32 ? 2 : 4;
-    static constexpr int A_BYTES = (F32 ? 3 : MT) * kTmPart;
-    static constexpr int STAGE = A_BYTES + kTmW;
-    static constexpr int RAW_STAGES = F32 ? 2 : 0;  // blocks of fp32 embeddings on their way
-    static constexpr int RAW = 2 * kTmPart;
-    static constexpr int THREADS = (kTmEpiWarps + 2 + (F32 ? kTmConvWarps : 0)) * 32;
-    static constexpr int SLOT = 32 * 64 * MT;       // running sums of one epilogue warp
-    static constexpr size_t SMEM = (size_t)STAGES * STAGE + (size_t)RAW_STAGES * RAW + 1024;  // (ring on a 1024-byte boundary)
+    static constexpr int MT = F32 ? 1 : 2;     // row blocks of 128 a CTA works on at a time
+    static constexpr int ROWS = 256 * MT;      // rows of V per tile
+    static constexpr int BLK = F32 ? 32 : 64;  // columns of E per block: rows of 64 or 128 bytes of bf16
+    static constexpr int CHUNK = F32 ? 4 : 8;  // blocks between two emptyings of an accumulator
+    static constexpr int PART = 128 * BLK * 2;                // bytes of 128 rows of bf16
+    static constexpr int A_BYTES = (F32 ? 3 : MT) * PART;     // a block's embeddings
+    static constexpr int W_BYTES = 3 * 64 * BLK * 2;          // a block's W: W1 (even CTA) or W2 (odd CTA), and half of W3
+    static constexpr int RAW = 128 * BLK * 4;                 // a block's fp32 embeddings
+    static constexpr int A_STAGES = F32 ? 3 : 4, W_STAGES = F32 ? 5 : 4, RAW_STAGES = F32 ? 5 : 1;
+    static constexpr int THREADS = (kTmEpiWarps + 2 + (F32 ? 1 + kTmConvWarps : 0)) * 32;
+    // (the rings start on a 1024-byte boundary)
+    static constexpr size_t SMEM = (size_t)A_STAGES * A_BYTES + (size_t)W_STAGES * W_BYTES + (F32 ? (size_t)RAW_STAGES * RAW : 0) + 1024;
+    static __device__ __forceinline__ uint64_t desc(uint32_t addr) { return F32 ? umma_desc_sw64(addr) : umma_desc_sw128(addr); }
+};
+
+// A walk over the N stages of a ring: stages passed so far, the stage, the parity to wait for.
+template <uint32_t N>
+struct TablesRing {
+    uint32_t t = 0, st = 0, ph;
+    __device__ __forceinline__ explicit TablesRing(uint32_t parity) : ph(parity) {}
+    __device__ __forceinline__ void next() {
+        ++t;
+        if (++st == N) {
+            st = 0;
+            ph ^= 1;
+        }
+    }
+    // Wait (bounded) until the stages passed last have been released; after an abort also, where `full` is given, until
+    // their copies have landed.
+    __device__ __forceinline__ void drain(uint32_t empty, uint32_t full, volatile int* abort_flag) const {
+        const uint32_t back = t < N ? t : N;
+        for (uint32_t b = 0; b < back; ++b) {
+            const uint32_t tt = t - back + b, at = 8 * (tt % N), parity = (tt / N) & 1;
+            for (uint32_t tries = 0; !mbar_try_wait_cluster(empty + at, parity) && tries < GRAFT_SPIN_LIMIT; ++tries)
+                if (*abort_flag && tries > 4096u) break;
+            if (*abort_flag && full != 0u)
+                for (uint32_t tries = 0; !mbar_try_wait_cluster(full + at, parity) && tries < 65536u; ++tries) {
+                }
+        }
+    }
 };
 
 struct __align__(64) TablesParams {
@@ -56,16 +83,16 @@ struct __align__(64) TablesParams {
     CUtensorMap map_e;  // [V, E] embeddings
     const float* bias;  // [m] or NULL
     float* out;         // [V, m]
-    float* pieces;      // [pairs][2 pieces][2 CTAs][kTmEpiWarps][SLOT]
-    int* counters;      // [pairs][2 CTAs][kTmEpiWarps], zero between calls
+    float* pieces;      // [pairs][2 pieces][ROWS][128]
     int32_t* errflag;
     int V, m, m_pad, n_mb, n_kb;
     int pairs, full_rounds;
     int left, share_pairs;  // left-over tiles, pairs that share them
+    int wide;               // rows of the table are whole 32-byte sectors
 };
 
-// What a pair works on: whole tiles, one in every round, then its share of the left-over tiles' blocks (the share is no
-// longer than a tile, so it lies in two tiles at most).
+// What a pair works on: its share of the left-over tiles' blocks (no longer than a tile, so it lies in two tiles at most;
+// tiles 0 .. left - 1), then whole tiles, one in every round.
 struct TablesItem {
     int tile, kb0, kb1;
     int q0, q1;  // a piece: the first and the last pair that work on the tile (q0 == q1: the whole tile)
@@ -79,24 +106,25 @@ __device__ __forceinline__ int tables_owner(const TablesParams& p, int block) {
     return (int)(((long long)(block + 1) * p.share_pairs + T - 1) / T - 1);
 }
 __device__ __forceinline__ bool tables_item(const TablesParams& p, int pair, int i, TablesItem& it) {
-    if (i < p.full_rounds) {
-        it.tile = pair + i * p.pairs;
-        it.kb0 = 0;
-        it.kb1 = p.n_kb;
-        it.q0 = it.q1 = pair;
-        return true;
+    if (pair < p.share_pairs) {
+        const int x0 = tables_share(p, pair), x1 = tables_share(p, pair + 1);
+        const int t = x0 / p.n_kb + i, b0 = t * p.n_kb, b1 = b0 + p.n_kb;
+        if (b0 < x1) {
+            it.tile = t;
+            it.kb0 = x0 > b0 ? x0 - b0 : 0;
+            it.kb1 = x1 < b1 ? x1 - b0 : p.n_kb;
+            it.seg = i;
+            it.q0 = tables_owner(p, b0);
+            it.q1 = tables_owner(p, b1 - 1);
+            return true;
+        }
+        i -= (x1 - 1) / p.n_kb - x0 / p.n_kb + 1;
     }
-    if (p.left == 0 || pair >= p.share_pairs) return false;
-    const int x0 = tables_share(p, pair), x1 = tables_share(p, pair + 1);
-    const int t = x0 / p.n_kb + (i - p.full_rounds);
-    const int b0 = t * p.n_kb, b1 = b0 + p.n_kb;
-    if (b0 >= x1) return false;
-    it.tile = p.full_rounds * p.pairs + t;
-    it.kb0 = x0 > b0 ? x0 - b0 : 0;
-    it.kb1 = x1 < b1 ? x1 - b0 : p.n_kb;
-    it.seg = i - p.full_rounds;
-    it.q0 = tables_owner(p, b0);
-    it.q1 = tables_owner(p, b1 - 1);
+    if (i >= p.full_rounds) return false;
+    it.tile = p.left + pair + i * p.pairs;
+    it.kb0 = 0;
+    it.kb1 = p.n_kb;
+    it.q0 = it.q1 = pair;
     return true;
 }
 
@@ -130,8 +158,13 @@ __device__ __forceinline__ void split3(float x0, float x1, uint32_t& a, uint32_t
     x1 -= __uint_as_float(b & 0xFFFF0000u);
     asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(c) : "f"(x1), "f"(x0));
 }
-__device__ __forceinline__ void st_shared_v4(uint32_t at, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
-    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(at), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
+__device__ __forceinline__ void st_shared_v4(uint32_t at, const uint32_t (&v)[4]) {
+    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(at), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]) : "memory");
+}
+__device__ __forceinline__ void st_global_v8(float* dst, const float* v) {
+    asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst), "f"(v[0]), "f"(v[1]), "f"(v[2]),
+                 "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7])
+                 : "memory");
 }
 __device__ __forceinline__ float4 ld_shared_f4(uint32_t at) {
     float4 v;
@@ -143,29 +176,32 @@ template <bool F32>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TablesCfg<F32>::THREADS, 1)
     tables_mma_kernel(const __grid_constant__ TablesParams p) {
     using C = TablesCfg<F32>;
-    constexpr uint32_t NST = C::STAGES, NRAW = F32 ? C::RAW_STAGES : 1;
+    constexpr uint32_t NA = C::A_STAGES, NW = C::W_STAGES, NR = C::RAW_STAGES;
     extern __shared__ unsigned char smem_raw[];
-    __shared__ __align__(8) uint64_t bars[3 * NST + 2 * NRAW + 4];
+    __shared__ __align__(8) uint64_t bars[2 * (NA + NW + NR) + 4];
     __shared__ uint32_t s_tmem;
     __shared__ volatile int s_abort;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const uint32_t rank = cluster_ctarank();
     const int pair = (int)blockIdx.x >> 1;
-    const uint32_t ring = (smem_u32(smem_raw) + 1023u) & ~1023u, raw_ring = ring + NST * C::STAGE;
-    // full: a stage's copies have landed in both CTAs (fp32: and the odd CTA's parts are written) -- the even CTA's;
-    // empty: its matrix instructions are done; conv: this CTA's parts of a stage are written (fp32)
-    const uint32_t full0 = smem_u32(bars), empty0 = full0 + 8 * NST, conv0 = empty0 + 8 * NST;
-    const uint32_t rawfull0 = conv0 + 8 * NST, rawempty0 = rawfull0 + 8 * NRAW;
-    const uint32_t accfull0 = rawempty0 + 8 * NRAW, accempty0 = accfull0 + 16;
+    const uint32_t a_ring = (smem_u32(smem_raw) + 1023u) & ~1023u;
+    const uint32_t w_ring = a_ring + NA * C::A_BYTES, raw_ring = w_ring + NW * C::W_BYTES;
+    // afull / wfull: a block's rows, W's are there in both CTAs (the even CTA's barriers), aempty / wempty: the instructions that read them are done, raw: fp32 rows as loaded
+    const uint32_t afull0 = smem_u32(bars), aempty0 = afull0 + 8 * NA, wfull0 = aempty0 + 8 * NA, wempty0 = wfull0 + 8 * NW;
+    const uint32_t rfull0 = wempty0 + 8 * NW, rempty0 = rfull0 + 8 * NR;
+    const uint32_t accfull0 = rempty0 + 8 * NR, accempty0 = accfull0 + 16;
     if (tid == 0) {
-        for (uint32_t s = 0; s < NST; ++s) {
-            mbar_init(full0 + 8 * s, F32 ? 2 : 1);
-            mbar_init(empty0 + 8 * s, 1);
-            mbar_init(conv0 + 8 * s, kTmConvWarps);
+        for (uint32_t s = 0; s < NA; ++s) {
+            mbar_init(afull0 + 8 * s, F32 ? 2 * kTmConvWarps : 1);
+            mbar_init(aempty0 + 8 * s, 1);
         }
-        for (uint32_t s = 0; s < NRAW; ++s) {
-            mbar_init(rawfull0 + 8 * s, 1);
-            mbar_init(rawempty0 + 8 * s, kTmConvWarps);
+        for (uint32_t s = 0; s < NW; ++s) {
+            mbar_init(wfull0 + 8 * s, 1);
+            mbar_init(wempty0 + 8 * s, 1);
+        }
+        for (uint32_t s = 0; s < NR; ++s) {
+            mbar_init(rfull0 + 8 * s, 1);
+            mbar_init(rempty0 + 8 * s, kTmConvWarps);
         }
         for (int s = 0; s < 2; ++s) {
             mbar_init(accfull0 + 8 * s, 1);
@@ -174,6 +210,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TablesCfg<F32>::THRE
         mbar_fence_init();
         s_abort = 0;
     }
+    pdl_launch_dependents();  // (the kernel that adds up the pieces; it waits for this grid)
     if (warp == 9) tmem_alloc_pair(smem_u32(&s_tmem), 512);
     tc_fence_before();
     cluster_sync();
@@ -220,144 +257,81 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TablesCfg<F32>::THRE
                     if (lane == 0) mbar_arrive_cluster(accempty_even + 8 * slot);
                 }
             }
-            bool write = true;
-            if (it.q0 != it.q1) {  // a piece of a left-over tile: the warp that arrives last adds the pieces up
-                auto piece = [&](int q, int seg) {
-                    return p.pieces + ((size_t)((q * 2 + seg) * 2 + (int)rank) * kTmEpiWarps + warp) * C::SLOT + lane;
-                };
-                float* mine = piece(pair, it.seg);
-#pragma unroll
-                for (int h = 0; h < C::MT; ++h)
-#pragma unroll
-                    for (int c = 0; c < 64; ++c) mine[(h * 64 + c) * 32] = acc[h][c];
-                __threadfence();
-                __syncwarp();
-                int* cnt = p.counters + ((it.tile - p.full_rounds * p.pairs) * 2 + (int)rank) * kTmEpiWarps + warp;
-                int old = 0;
-                if (lane == 0) old = atomicAdd(cnt, 1);
-                old = __shfl_sync(0xFFFFFFFFu, old, 0);
-                write = old == it.q1 - it.q0;
-                if (write) {
-                    __threadfence();
-                    if (lane == 0) *cnt = 0;  // ready for the next call
-                    const int b0 = (it.tile - p.full_rounds * p.pairs) * p.n_kb;
-#pragma unroll
-                    for (int h = 0; h < C::MT; ++h)
-#pragma unroll
-                        for (int c = 0; c < 64; ++c) acc[h][c] = 0.f;
-                    for (int q = it.q0; q <= it.q1; ++q) {
-                        const float* src = piece(q, tables_share(p, q) < b0 ? 1 : 0);
-#pragma unroll
-                        for (int h = 0; h < C::MT; ++h)
-#pragma unroll
-                            for (int c = 0; c < 64; ++c) acc[h][c] += __ldcg(src + (h * 64 + c) * 32);
-                    }
-                }
-            }
+            // a piece of a left-over tile goes to scratch, [ROWS][128], without the bias
+            const bool piece = it.q0 != it.q1;
+            const int ld = piece ? 128 : p.m, rows = piece ? C::ROWS : p.V - rt * C::ROWS, cols = piece ? 64 : p.m - mb * 128 - half * 64;
+            const bool wide = piece || p.wide;
+            float* base = piece ? p.pieces + (size_t)(pair * 2 + it.seg) * C::ROWS * 128
+                                : p.out + (size_t)rt * C::ROWS * p.m + mb * 128;
+            const float* bias = piece || p.bias == nullptr ? nullptr : p.bias + mb * 128 + half * 64;
 #pragma unroll
             for (int h = 0; h < C::MT; ++h) {
-                const int v = rt * C::ROWS + h * 256 + (int)rank * 128 + quarter * 32 + lane;
-                if (write && v < p.V) {
-                    const int col0 = mb * 128 + half * 64;
-                    float* dst = p.out + (size_t)v * p.m + col0;
+                const int v = h * 256 + (int)rank * 128 + quarter * 32 + lane;
+                if (v < rows) {
+                    float* dst = base + (size_t)v * ld + half * 64;
 #pragma unroll
-                    for (int c = 0; c < 64; c += 4) {
-                        if (col0 + c < p.m) {
-                            float4 b = make_float4(0.f, 0.f, 0.f, 0.f);
-                            if (p.bias)
-                                b = make_float4(__ldg(p.bias + col0 + c), __ldg(p.bias + col0 + c + 1),
-                                                __ldg(p.bias + col0 + c + 2), __ldg(p.bias + col0 + c + 3));
-                            *(float4*)(dst + c) = make_float4(acc[h][c] + b.x, acc[h][c + 1] + b.y, acc[h][c + 2] + b.z,
-                                                              acc[h][c + 3] + b.w);
+                    for (int c = 0; c < 64; c += 8) {
+                        if (c >= cols) break;
+                        const bool both = c + 4 < cols;
+                        if (bias) {
+#pragma unroll
+                            for (int k = 0; k < 8; ++k)
+                                if (k < 4 || both) acc[h][c + k] += __ldg(bias + c + k);
+                        }
+                        if (wide) {  // (both: m is a multiple of 8)
+                            st_global_v8(dst + c, &acc[h][c]);
+                        } else {
+                            *(float4*)(dst + c) = make_float4(acc[h][c], acc[h][c + 1], acc[h][c + 2], acc[h][c + 3]);
+                            if (both)
+                                *(float4*)(dst + c + 4) = make_float4(acc[h][c + 4], acc[h][c + 5], acc[h][c + 6], acc[h][c + 7]);
                         }
                     }
                 }
             }
         }
     } else if (warp == 8) {
-        // ------------------------------ TMA loads ------------------------------------------------
+        // ------------------------------ TMA loads: W, bf16 embeddings ----------------------------
         if (lane == 0) {
-            const uint32_t full_even = mapa_u32(full0, 0);
-            uint32_t t = 0, st = 0, ph = 1, rst = 0, rph = 1;
-            // fp32: an iterator of the raw blocks, which run ahead of W's
-            int ri = 0, rkb = 0;
-            uint32_t rt_ = 0;
-            TablesItem rit;
-            bool rvalid = F32 && tables_item(p, pair, 0, rit);
-            if (rvalid) rkb = rit.kb0;
-            auto raw_load = [&]() {
-                if (!rvalid || s_abort) return;
-                if (rt_ >= NRAW) mbar_wait_bounded(rawempty0 + 8 * rst, rph, &s_abort);
-                if (s_abort) return;
-                const int row = rit.tile / p.n_mb * C::ROWS + (int)rank * 128;
-                mbar_arrive_expect_tx(rawfull0 + 8 * rst, C::RAW);
-                tma_load_2d(raw_ring + rst * C::RAW, &p.map_e, rkb * kTmBlk, row, rawfull0 + 8 * rst);
-                tma_load_2d(raw_ring + rst * C::RAW + kTmPart, &p.map_e, rkb * kTmBlk + 32, row, rawfull0 + 8 * rst);
-                ++rt_;
-                if (++rst == NRAW) {
-                    rst = 0;
-                    rph ^= 1;
-                }
-                if (++rkb == rit.kb1) {
-                    rvalid = tables_item(p, pair, ++ri, rit);
-                    if (rvalid) rkb = rit.kb0;
-                }
-            };
-            if (F32) raw_load();
+            const uint32_t afull_even = mapa_u32(afull0, 0), wfull_even = mapa_u32(wfull0, 0);
+            TablesRing<NA> a(1);
+            TablesRing<NW> w(1);
             for (int i = 0; tables_item(p, pair, i, it); ++i) {
                 const int rt = it.tile / p.n_mb, mb = it.tile - rt * p.n_mb;
                 const int n = ((p.m - mb * 128 < 128 ? p.m - mb * 128 : 128) + 31) & ~31;
                 const int w12 = (int)rank * p.m_pad + mb * 128, w3 = 2 * p.m_pad + mb * 128 + (int)rank * (n >> 1);
-                for (int kb = it.kb0; kb < it.kb1; ++kb, ++t) {
-                    if (F32) raw_load();
-                    if (t >= NST) mbar_wait_cluster(empty0 + 8 * st, ph, &s_abort);
-                    if (s_abort) break;  // (no copy is started any more)
-                    const uint32_t dst = ring + st * C::STAGE, dw = dst + C::A_BYTES, fb = full_even + 8 * st;
-                    const int x = kb * kTmBlk;
-                    if (rank == 0) mbar_arrive_expect_tx(full0 + 8 * st, 2u * (F32 ? kTmW : C::STAGE));
+                for (int kb = it.kb0; kb < it.kb1; ++kb) {
+                    const int x = kb * C::BLK;
                     if (!F32) {
+                        if (a.t >= NA) mbar_wait_cluster(aempty0 + 8 * a.st, a.ph, &s_abort);
+                        if (s_abort) break;  // (no copy is started any more)
+                        if (rank == 0) mbar_arrive_expect_tx(afull0 + 8 * a.st, 2u * C::A_BYTES);
 #pragma unroll
                         for (int h = 0; h < C::MT; ++h)
-                            tma_load_2d_pair(dst + h * kTmPart, &p.map_e, x, rt * C::ROWS + h * 256 + (int)rank * 128, fb);
+                            tma_load_2d_pair(a_ring + a.st * C::A_BYTES + h * C::PART, &p.map_e, x,
+                                             rt * C::ROWS + h * 256 + (int)rank * 128, afull_even + 8 * a.st);
+                        a.next();
                     }
+                    if (w.t >= NW) mbar_wait_cluster(wempty0 + 8 * w.st, w.ph, &s_abort);
+                    if (s_abort) break;
+                    const uint32_t dw = w_ring + w.st * C::W_BYTES, fb = wfull_even + 8 * w.st;
+                    if (rank == 0) mbar_arrive_expect_tx(wfull0 + 8 * w.st, 2u * C::W_BYTES);
                     tma_load_2d_pair(dw, &p.map_w, x, w12, fb);
-                    tma_load_2d_pair(dw + 8192, &p.map_w, x, w12 + 64, fb);
-                    tma_load_2d_pair(dw + 16384, &p.map_w, x, w3, fb);
-                    if (++st == NST) {
-                        st = 0;
-                        ph ^= 1;
-                    }
+                    tma_load_2d_pair(dw + C::W_BYTES / 3, &p.map_w, x, w12 + 64, fb);
+                    tma_load_2d_pair(dw + 2 * (C::W_BYTES / 3), &p.map_w, x, w3, fb);
+                    w.next();
                 }
             }
-            // every stage has been read before the CTA retires (its barriers are arrived at from the other CTA); after
-            // an abort: no copy of this pair may still be in flight
-            const uint32_t back = t < NST ? t : NST;
-            for (uint32_t b = 0; b < back; ++b) {
-                const uint32_t tt = t - back + b;
-                uint32_t tries = 0;
-                while (!mbar_try_wait_cluster(empty0 + 8 * (tt % NST), (tt / NST) & 1) && ++tries < GRAFT_SPIN_LIMIT) {
-                    if (s_abort && tries > 4096u) break;
-                }
-                if (s_abort && rank == 0) {
-                    tries = 0;
-                    while (!mbar_try_wait_cluster(full0 + 8 * (tt % NST), (tt / NST) & 1) && ++tries < 65536u) {
-                    }
-                }
-            }
-            if (F32 && s_abort) {
-                const uint32_t rback = rt_ < NRAW ? rt_ : NRAW;
-                for (uint32_t b = 0; b < rback; ++b) {
-                    const uint32_t tt = rt_ - rback + b;
-                    uint32_t tries = 0;
-                    while (!mbar_try_wait(rawfull0 + 8 * (tt % NRAW), (tt / NRAW) & 1) && ++tries < 65536u) {
-                    }
-                }
-            }
+            // the last arrivals from the other CTA have come before this CTA retires; after an abort: no copy of the pair
+            // is in flight any more
+            if (!F32) a.drain(aempty0, rank == 0 ? afull0 : 0u, &s_abort);
+            w.drain(wempty0, rank == 0 ? wfull0 : 0u, &s_abort);
         }
     } else if (warp == 9) {
         // ------------------------------ matrix instructions --------------------------------------
         if (rank == 0 && lane == 0) {
-            uint32_t st = 0, ph = 0, cc = 0;
+            TablesRing<NA> a(0);
+            TablesRing<NW> w(0);
+            uint32_t cc = 0;
             for (int i = 0; tables_item(p, pair, i, it); ++i) {
                 const int mb = it.tile % p.n_mb;
                 const int n = ((p.m - mb * 128 < 128 ? p.m - mb * 128 : 128) + 31) & ~31;
@@ -365,32 +339,31 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TablesCfg<F32>::THRE
                 for (int kb = it.kb0; kb < it.kb1; ++kb) {
                     const bool first = (kb - it.kb0) % C::CHUNK == 0;
                     const bool last = kb + 1 == it.kb1 || (kb + 1 - it.kb0) % C::CHUNK == 0;
-                    mbar_wait_cluster(full0 + 8 * st, ph, &s_abort);
-                    if (F32) mbar_wait_cluster(conv0 + 8 * st, ph, &s_abort);
+                    mbar_wait_cluster(wfull0 + 8 * w.st, w.ph, &s_abort);
+                    mbar_wait_cluster(afull0 + 8 * a.st, a.ph, &s_abort);
                     tc_fence_after();
-                    const uint32_t a0 = ring + st * C::STAGE, b0 = a0 + C::A_BYTES;
+                    const uint32_t a0 = a_ring + a.st * C::A_BYTES, b0 = w_ring + w.st * C::W_BYTES;
                     // An instruction whose accumulator columns the one just ahead of it wrote waits for those; with two row
                     // blocks their instructions alternate, except in the first and the last block of a chunk, where the
                     // first row block goes ahead (its accumulators are emptied, or were, while the second's are filled).
-                    const bool alternate = C::MT == 2 && !first && !last;
                     auto mma = [&](int h, int ks, bool w3) {
                         const uint32_t d = tmem + (C::MT == 1 ? (cc & 1u) : (uint32_t)h) * 256u;
-                        const uint64_t a1 = umma_desc_sw128(a0 + h * kTmPart + 32 * ks);
+                        const uint64_t a1 = C::desc(a0 + h * C::PART + 32 * ks);
                         if (w3) {
-                            umma_pair(d + (uint32_t)n, a1, umma_desc_sw128(b0 + 16384 + 32 * ks), idesc1, true);
+                            umma_pair(d + (uint32_t)n, a1, C::desc(b0 + 2 * (C::W_BYTES / 3) + 32 * ks), idesc1, true);
                         } else {
-                            const uint64_t w12 = umma_desc_sw128(b0 + 32 * ks);
+                            const uint64_t w12 = C::desc(b0 + 32 * ks);
                             umma_pair(d, a1, w12, idesc2, !first || ks > 0);
                             if (F32) {
-                                umma_pair(d, umma_desc_sw128(a0 + kTmPart + 32 * ks), w12, idesc2, true);
-                                umma_pair(d, umma_desc_sw128(a0 + 2 * kTmPart + 32 * ks), w12, idesc2, true);
+                                umma_pair(d, C::desc(a0 + C::PART + 32 * ks), w12, idesc2, true);
+                                umma_pair(d, C::desc(a0 + 2 * C::PART + 32 * ks), w12, idesc2, true);
                             }
                         }
                     };
-                    if (alternate) {
+                    if (C::MT == 2 && !first && !last) {
                         if (!s_abort) {
 #pragma unroll
-                            for (int ks = 0; ks < 4; ++ks) {
+                            for (int ks = 0; ks < C::BLK / 16; ++ks) {
                                 mma(0, ks, false);
                                 mma(1, ks, false);
                                 mma(0, ks, true);
@@ -408,7 +381,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TablesCfg<F32>::THRE
                             }
                             if (!s_abort) {
 #pragma unroll
-                                for (int ks = 0; ks < 4; ++ks) {
+                                for (int ks = 0; ks < C::BLK / 16; ++ks) {
                                     mma(h, ks, false);
                                     mma(h, ks, true);
                                 }
@@ -416,84 +389,74 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TablesCfg<F32>::THRE
                             if (last) umma_commit_pair(accfull0 + 8 * slot);
                         }
                     }
-                    umma_commit_pair(empty0 + 8 * st);
+                    umma_commit_pair(aempty0 + 8 * a.st);
+                    umma_commit_pair(wempty0 + 8 * w.st);
                     if (last) ++cc;
-                    if (++st == NST) {
-                        st = 0;
-                        ph ^= 1;
-                    }
+                    a.next();
+                    w.next();
                 }
             }
-        } else if (F32 && rank == 1 && lane == 0) {
-            // the odd CTA's parts of a stage are written: tell the even CTA
-            const uint32_t full_even = mapa_u32(full0, 0);
-            uint32_t st = 0, ph = 0;
-            for (int i = 0; tables_item(p, pair, i, it); ++i)
+        }
+    } else if (F32 && warp == 10) {
+        // ------------------------------ TMA loads: fp32 embeddings -------------------------------
+        if (lane == 0) {
+            TablesRing<NR> r(1);
+            for (int i = 0; tables_item(p, pair, i, it); ++i) {
+                const int row = it.tile / p.n_mb * C::ROWS + (int)rank * 128;
                 for (int kb = it.kb0; kb < it.kb1; ++kb) {
-                    mbar_wait_cluster(conv0 + 8 * st, ph, &s_abort);
-                    mbar_arrive_cluster(full_even + 8 * st);
-                    if (++st == NST) {
-                        st = 0;
-                        ph ^= 1;
-                    }
+                    if (r.t >= NR) mbar_wait_bounded(rempty0 + 8 * r.st, r.ph, &s_abort);
+                    if (s_abort) break;
+                    mbar_arrive_expect_tx(rfull0 + 8 * r.st, C::RAW);
+                    tma_load_2d(raw_ring + r.st * C::RAW, &p.map_e, kb * C::BLK, row, rfull0 + 8 * r.st);
+                    r.next();
                 }
+            }
+            r.drain(rempty0, rfull0, &s_abort);
         }
     } else if (F32) {
         // ------------------------------ fp32 embeddings -> bf16 parts ----------------------------
-        const int ct = tid - (kTmEpiWarps + 2) * 32;
-        const int c8 = ct & 7, r0 = ct >> 3;  // columns 8 c8 .. 8 c8 + 7 of rows r0, r0 + 32, ...
-        uint32_t t = 0, st = 0, ph = 1, rst = 0, rph = 0;
+        const int ct = tid - (kTmEpiWarps + 3) * 32;
+        const int c8 = ct & 3, r0 = ct >> 2;  // columns 8 c8 .. 8 c8 + 7 of rows r0 and r0 + 64
+        const uint32_t afull_even = mapa_u32(afull0, 0);
+        TablesRing<NA> a(1);
+        TablesRing<NR> r(0);
         for (int i = 0; tables_item(p, pair, i, it); ++i) {
-            for (int kb = it.kb0; kb < it.kb1; ++kb, ++t) {
-                mbar_wait_bounded(rawfull0 + 8 * rst, rph, &s_abort);
-                // a block is two boxes of 32 columns; the lanes of the second read their halves in the other order, so
-                // that the eight lanes of a row touch every bank once
-                const uint32_t src = raw_ring + rst * C::RAW + (uint32_t)(c8 >> 2) * kTmPart;
-                float x[4][8];
+            for (int kb = it.kb0; kb < it.kb1; ++kb) {
+                mbar_wait_bounded(rfull0 + 8 * r.st, r.ph, &s_abort);
+                const uint32_t src = raw_ring + r.st * C::RAW;
+                float4 x[2][2];
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const int row = r0 + 32 * q;
+                for (int q = 0; q < 2; ++q) {
+                    const int row = r0 + 64 * q;
 #pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        const int hh = h ^ (c8 >> 2);
-                        const float4 v = ld_shared_f4(src + (uint32_t)row * 128u + (uint32_t)(((2 * (c8 & 3) + hh) ^ (row & 7)) * 16));
-                        x[q][4 * h] = v.x, x[q][4 * h + 1] = v.y, x[q][4 * h + 2] = v.z, x[q][4 * h + 3] = v.w;
-                    }
+                    for (int h = 0; h < 2; ++h)  // (128-byte rows in the 128-byte swizzle)
+                        x[q][h] = ld_shared_f4(src + (uint32_t)row * 128u + (uint32_t)(((2 * c8 + h) ^ (row & 7)) * 16));
                 }
                 __syncwarp();
-                if (lane == 0) mbar_arrive(rawempty0 + 8 * rst);
-                if (++rst == NRAW) {
-                    rst = 0;
-                    rph ^= 1;
-                }
-                if (t >= NST) mbar_wait_bounded(empty0 + 8 * st, ph, &s_abort);
-                const uint32_t dst = ring + st * C::STAGE;
+                if (lane == 0) mbar_arrive(rempty0 + 8 * r.st);
+                r.next();
+                if (a.t >= NA) mbar_wait_bounded(aempty0 + 8 * a.st, a.ph, &s_abort);
+                const uint32_t dst = a_ring + a.st * C::A_BYTES;
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const int row = r0 + 32 * q;
-                    const uint32_t at = dst + (uint32_t)row * 128u + (uint32_t)((c8 ^ (row & 7)) * 16);
-                    uint32_t a[4], b[4], c[4];
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) split3(x[q][2 * k], x[q][2 * k + 1], a[k], b[k], c[k]);
-                    if (c8 >> 2) {  // (the halves were read in the other order)
-                        st_shared_v4(at, a[2], a[3], a[0], a[1]);
-                        st_shared_v4(at + kTmPart, b[2], b[3], b[0], b[1]);
-                        st_shared_v4(at + 2 * kTmPart, c[2], c[3], c[0], c[1]);
-                    } else {
-                        st_shared_v4(at, a[0], a[1], a[2], a[3]);
-                        st_shared_v4(at + kTmPart, b[0], b[1], b[2], b[3]);
-                        st_shared_v4(at + 2 * kTmPart, c[0], c[1], c[2], c[3]);
-                    }
+                for (int q = 0; q < 2; ++q) {
+                    const int row = r0 + 64 * q;  // (64-byte rows in the 64-byte swizzle)
+                    const uint32_t at = dst + (uint32_t)row * 64u + (uint32_t)((c8 ^ ((row >> 1) & 3)) * 16);
+                    uint32_t b1[4], b2[4], b3[4];
+                    split3(x[q][0].x, x[q][0].y, b1[0], b2[0], b3[0]);
+                    split3(x[q][0].z, x[q][0].w, b1[1], b2[1], b3[1]);
+                    split3(x[q][1].x, x[q][1].y, b1[2], b2[2], b3[2]);
+                    split3(x[q][1].z, x[q][1].w, b1[3], b2[3], b3[3]);
+                    st_shared_v4(at, b1);
+                    st_shared_v4(at + C::PART, b2);
+                    st_shared_v4(at + 2 * C::PART, b3);
                 }
                 fence_proxy_async();
                 __syncwarp();
-                if (lane == 0) mbar_arrive(conv0 + 8 * st);
-                if (++st == NST) {
-                    st = 0;
-                    ph ^= 1;
-                }
+                if (lane == 0) mbar_arrive_cluster(afull_even + 8 * a.st);
+                a.next();
             }
         }
+        a.drain(aempty0, 0u, &s_abort);
     }
     __syncwarp();
     tc_fence_before();
@@ -501,6 +464,29 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TablesCfg<F32>::THRE
     tc_fence_after();
     if (warp == 9) tmem_free_pair(tmem, 512);
     if (tid == 0 && s_abort) atomicOr(p.errflag, 1);
+}
+
+// The left-over tiles' pieces, added up in order: one thread per four columns of a row.
+template <bool F32>
+__global__ void __launch_bounds__(256) tables_pieces_kernel(const __grid_constant__ TablesParams p) {
+    using C = TablesCfg<F32>;
+    pdl_wait();
+    const int tile = (int)blockIdx.y, rt = tile / p.n_mb, mb = tile - rt * p.n_mb;
+    const int q0 = tables_owner(p, tile * p.n_kb), q1 = tables_owner(p, (tile + 1) * p.n_kb - 1);
+    const int v = (int)blockIdx.x * 8 + (threadIdx.x >> 5), c = (threadIdx.x & 31) * 4;
+    if (q0 == q1 || rt * C::ROWS + v >= p.V || mb * 128 + c >= p.m) return;  // (q0 == q1: written whole)
+    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 4
+    for (int q = q0; q <= q1; ++q) {
+        const int seg = tables_share(p, q) < tile * p.n_kb ? 1 : 0;
+        const float4 x = __ldcs((const float4*)(p.pieces + ((size_t)(q * 2 + seg) * C::ROWS + v) * 128 + c));
+        s.x += x.x, s.y += x.y, s.z += x.z, s.w += x.w;
+    }
+    if (p.bias) {
+        const float* b = p.bias + mb * 128 + c;
+        s.x += b[0], s.y += b[1], s.z += b[2], s.w += b[3];
+    }
+    *(float4*)(p.out + (size_t)(rt * C::ROWS + v) * p.m + mb * 128 + c) = s;
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
@@ -519,29 +505,42 @@ EncodeTiledFn encode_tiled() {
     }();
     return fn;
 }
-// [rows, cols], boxes of box_rows rows of 128 bytes, 128-byte swizzle, zeros outside
-bool encode_map(CUtensorMap* map, const void* base, bool f32, uint64_t rows, uint64_t cols, uint32_t box_rows) {
-    const cuuint64_t dims[2] = {cols, rows}, strides[1] = {cols * (f32 ? 4 : 2)};
-    const cuuint32_t box[2] = {f32 ? 32u : 64u, box_rows}, step[2] = {1, 1};
-    return encode_tiled()(map, f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, step,
-                          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+// [rows, cols], boxes of box_rows rows of box_bytes, in the swizzle of that width, zeros outside
+bool encode_map(CUtensorMap* map, const void* base, bool f32, uint64_t rows, uint64_t cols, uint32_t box_rows, uint32_t box_bytes) {
+    const uint32_t esz = f32 ? 4 : 2;
+    const cuuint64_t dims[2] = {cols, rows}, strides[1] = {cols * esz};
+    const cuuint32_t box[2] = {box_bytes / esz, box_rows}, step[2] = {1, 1};
+    return encode_tiled()(map, f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2,
+                          const_cast<void*>(base), dims, strides, box, step, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                          box_bytes == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
+                          CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 struct TablesSizes {
     int n_mb, m_pad, E_pad, pairs;
-    size_t o_pieces, o_w, total;  // (the counters stand first: their place does not depend on E)
+    size_t o_w, total;
 };
 TablesSizes tables_sizes(int num_sms, int E, int m) {
     TablesSizes s;
     s.n_mb = (m + 127) / 128;
     s.m_pad = 128 * s.n_mb;
-    s.E_pad = (E + kTmBlk - 1) / kTmBlk * kTmBlk;
+    s.E_pad = (E + 63) / 64 * 64;
     s.pairs = num_sms / 2;
-    s.o_pieces = ((size_t)s.pairs * 2 * kTmEpiWarps * sizeof(int) + 255) & ~(size_t)255;
-    s.o_w = s.o_pieces + (size_t)s.pairs * 2 * 2 * kTmEpiWarps * TablesCfg<false>::SLOT * sizeof(float);
+    s.o_w = (size_t)s.pairs * 2 * TablesCfg<false>::ROWS * 128 * sizeof(float);
     s.total = s.o_w + (size_t)3 * s.m_pad * s.E_pad * 2;
     return s;
+}
+template <bool F32>
+cudaError_t tables_run(const TablesParams& p, cudaStream_t st, int* launches) {
+    using C = TablesCfg<F32>;
+    cudaError_t e = cudaFuncSetAttribute(tables_mma_kernel<F32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
+    if (e == cudaSuccess) e = launch_pdl(tables_mma_kernel<F32>, dim3(2 * p.pairs), dim3(C::THREADS), C::SMEM, st, p);
+    *launches += 1;
+    if (e == cudaSuccess && p.share_pairs > p.left) {
+        e = launch_pdl(tables_pieces_kernel<F32>, dim3(C::ROWS / 8, p.left), dim3(256), 0, st, p);
+        *launches += 1;
+    }
+    return e;
 }
 
 }  // namespace
@@ -550,11 +549,9 @@ TablesSizes tables_sizes(int num_sms, int E, int m) {
 bool tables_mma_fits(const void* d_emb, graft_dtype dt, int E, const void* d_out) {
     return E % (dt == GRAFT_BF16 ? 8 : 4) == 0 && (((uintptr_t)d_emb | (uintptr_t)d_out) & 15) == 0 && encode_tiled() != nullptr;
 }
-size_t tables_mma_counter_bytes(int num_sms) { return tables_sizes(num_sms, 1, 1).o_pieces; }
 size_t tables_mma_scratch_bytes(int num_sms, int E, int m) { return tables_sizes(num_sms, E, m).total; }
 
-// out [V, m] = emb [V, E] . W^T + bias.  scratch: tables_mma_scratch_bytes, 256-byte aligned; its first
-// tables_mma_counter_bytes are zero when it is first used.
+// out [V, m] = emb [V, E] . W^T + bias.  scratch: tables_mma_scratch_bytes, 256-byte aligned.
 cudaError_t tables_mma_launch(graft_ctx* ctx, const void* d_emb, graft_dtype dt, int E, const float* d_W, const float* d_b,
                               float* d_out, void* scratch, cudaStream_t st) {
     const int V = ctx->cfg.V, m = ctx->cfg.m;
@@ -562,42 +559,36 @@ cudaError_t tables_mma_launch(graft_ctx* ctx, const void* d_emb, graft_dtype dt,
     const bool f32 = dt == GRAFT_F32;
     __nv_bfloat16* w = (__nv_bfloat16*)((char*)scratch + s.o_w);
     TablesParams p;
-    if (!encode_map(&p.map_w, w, false, (uint64_t)3 * s.m_pad, s.E_pad, 64) || !encode_map(&p.map_e, d_emb, f32, V, E, 128))
+    const int blk = f32 ? TablesCfg<true>::BLK : TablesCfg<false>::BLK;
+    if (!encode_map(&p.map_w, w, false, (uint64_t)3 * s.m_pad, s.E_pad, 64, 2 * blk) ||
+        !encode_map(&p.map_e, d_emb, f32, V, E, 128, 128))
         return cudaErrorUnknown;
     p.bias = d_b;
     p.out = d_out;
-    p.pieces = (float*)((char*)scratch + s.o_pieces);
-    p.counters = (int*)scratch;
+    p.pieces = (float*)scratch;
     p.errflag = ctx->w_errflag;
     p.V = V;
     p.m = m;
     p.m_pad = s.m_pad;
     p.n_mb = s.n_mb;
-    p.n_kb = s.E_pad / kTmBlk;
+    p.n_kb = (E + blk - 1) / blk;
     p.pairs = s.pairs;
     const int rows = f32 ? TablesCfg<true>::ROWS : TablesCfg<false>::ROWS;
     const int tiles = (V + rows - 1) / rows * s.n_mb;
     p.full_rounds = tiles / s.pairs;
     p.left = tiles - p.full_rounds * s.pairs;
-    // a share of the left-over tiles: at least an eighth of a tile and four ring stages, at most a tile
+    // a share of the left-over tiles: at least a sixteenth of a tile and 256 columns, at most a tile
     long long sp = s.pairs;
     if (sp > (long long)p.left * kTmMaxSplit) sp = (long long)p.left * kTmMaxSplit;
-    if (sp > (long long)p.left * p.n_kb / 4) sp = (long long)p.left * p.n_kb / 4;
+    if (sp > (long long)p.left * p.n_kb * blk / 256) sp = (long long)p.left * p.n_kb * blk / 256;
     p.share_pairs = (int)(sp < p.left ? p.left : sp);
-    if (p.left == 0) p.share_pairs = 1;
+    p.wide = m % 8 == 0 && ((uintptr_t)d_out & 31) == 0;
     weight_split_kernel<<<dim3((s.E_pad + 511) / 512, s.m_pad), 256, 0, st>>>(d_W, m, E, s.m_pad, s.E_pad, w);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    if (f32) {
-        e = cudaFuncSetAttribute(tables_mma_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TablesCfg<true>::SMEM);
-        if (e == cudaSuccess)
-            e = launch_pdl(tables_mma_kernel<true>, dim3(2 * s.pairs), dim3(TablesCfg<true>::THREADS), TablesCfg<true>::SMEM, st, p);
-    } else {
-        e = cudaFuncSetAttribute(tables_mma_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TablesCfg<false>::SMEM);
-        if (e == cudaSuccess)
-            e = launch_pdl(tables_mma_kernel<false>, dim3(2 * s.pairs), dim3(TablesCfg<false>::THREADS), TablesCfg<false>::SMEM, st, p);
-    }
-    ctx->launches += 2;
+    int launches = 1;
+    e = f32 ? tables_run<true>(p, st, &launches) : tables_run<false>(p, st, &launches);
+    ctx->launches += (uint64_t)launches;
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
