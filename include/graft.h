@@ -134,10 +134,11 @@ int32_t graft_edge_rows(const graft_ctx* ctx);
 
 /* Table precompute (same passage): d_out[v] = W e_v + b for one tower.  d_emb [V, E] (dtype as given),
  * d_W [m, E] fp32, d_b [m] fp32 or NULL, d_out [V, m] fp32.  fp32 accumulation.  Call once per tower.
- * With bf16 embeddings (16-byte aligned, E a multiple of 8) the products run on the tensor cores: the embeddings are
- * exact operands and W enters as three bf16 parts, so the result differs from the fp32 one only by the order of
- * the additions; the first such call allocates scratch in the context (3 m E bf16 values and the GEMM's
- * workspace; GRAFT_ERR_WORKSPACE if that fails).  This is the once-per-model setup step, not the round. */
+ * With d_emb and d_out 16-byte aligned and E a multiple of 8 (bf16) or 4 (fp32) the products run on the tensor cores:
+ * fp32 numbers enter as three bf16 parts, whose products are exact, so the result differs from a fp32 FMA one only by
+ * the order of the additions (an infinite entry gives NaN); the first such call allocates scratch in the context (3 m E
+ * bf16 values and up to 40 MB of partial sums; GRAFT_ERR_WORKSPACE if that fails).  This is the once-per-model setup
+ * step, not the round. */
 graft_status graft_tdes_precompute(graft_ctx* ctx, const void* d_emb, graft_dtype emb_dtype, int32_t E,
                                    const float* d_W, const float* d_b, float* d_out, void* stream);
 

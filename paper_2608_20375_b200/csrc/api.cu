@@ -251,7 +251,7 @@ graft_status graft_tdes_precompute(graft_ctx* ctx, const void* d_emb, graft_dtyp
     // the tensor cores (bf16 parts of the inputs, exact products); their scratch is allocated on the first call (this is
     // the once-per-model setup step, not the round)
     if (tables_mma_fits(d_emb, emb_dtype, E, d_out)) {
-        const size_t need = tables_mma_scratch_bytes(ctx->num_sms, E, ctx->cfg.m);
+        const size_t need = tables_mma_scratch_bytes(ctx->num_sms, E, ctx->cfg.m, emb_dtype);
         if (ctx->tables_scratch_bytes < need) {
             if (ctx->tables_scratch) cudaFree(ctx->tables_scratch);
             ctx->tables_scratch = nullptr;

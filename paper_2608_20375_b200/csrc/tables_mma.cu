@@ -9,16 +9,25 @@
 // round less carefully than an FMA chain: they are emptied into fp32 registers after 32 (bf16) or 24 (fp32
 // embeddings) additions to the large products' accumulators, which W2's and W3's do not share.
 //
-// One kernel, persistent, a cluster of two CTAs per pair of SMs (tcgen05, cta_group::2): a pair owns a tile of 512 rows
-// of V (fp32 embeddings: 256) times up to 128 columns of m, and streams E in blocks of 64 through a shared-memory ring.
-//   warps 0-7   empty the accumulators (TMEM, two sets of 2 x 128 columns), keep the running sums and write the tile
-//   warp 8      TMA loads: W's parts (split once per call into scratch by weight_split_kernel) and the embeddings
-//   warp 9      issues the matrix instructions (even CTA only)
-//   warps 10-17 fp32 embeddings only: raw rows -> bf16 parts in the operands' layout
-// W1 and W2 stand side by side as one operand of N = 256 (M = 256, N = 128 takes as long as N = 256: 128 cycles measured),
-// W3 is an N = 128 of its own.  Tiles of 512 rows halve the passes over W, which comes from L2 every time.  The
-// embeddings are read from memory once; nothing but the tables is written.  What is left when the tiles do not divide
-// by the pairs is dealt out along E in equal shares, whose sums a small kernel adds up in order.
+// One persistent kernel.  A worker -- a pair of CTAs (cluster of two, tcgen05 cta_group::2) for bf16 embeddings, one CTA
+// for fp32 -- owns a tile of 512 (fp32: 128) rows of V times up to 128 columns of m, and streams E in blocks of 64 (32)
+// columns through shared-memory rings.
+//   warps 0-7    empty the accumulators (TMEM, two sets of 2 x 128 columns), keep the running sums and write the tile
+//   warp 8       TMA loads: W's parts (split once per call into scratch by weight_split_kernel), bf16 embeddings
+//   warp 9       issues the matrix instructions
+//   warp 10      fp32 only: TMA loads of the raw rows;  warps 11-18  raw rows -> bf16 parts in the operands' layout
+// W1 and W2 stand side by side as one operand of N = 256, W3 is an N = 128 of its own (three of N = 128 in a row on one
+// accumulator took 122 cycles each: an instruction waits for the one ahead of it on the same columns).  Tiles of 512
+// rows halve the passes over W, which comes from L2 every time.  The fp32 kernel works on single CTAs because its rows
+// go through threads: telling the other CTA of a pair about every block cost more (136 - 160 us at V = 32,000, E = 2048)
+// than the second CTA's half of W saves (120 us).  The embeddings are read from memory once; nothing but the tables is
+// written.  What is left when the tiles do not divide by the workers is dealt out along E in equal shares, whose sums a
+// small kernel adds up in order (summing them inside, by the warp that came last, stalled its tile: 462 against 370 us).
+//
+// Measured (one tower, back to back, B200): V = 151,936, E = 4096, m = 128, bf16: 373 us (798 us with the library
+// template's GEMMs, whose partial sums went through memory); its products take 287 us at the measured dense rate, the
+// loads alone 258 us.  V = 32,000, E = 2048, fp32: 120 us (1180 us by the FMA kernel; the loads and the splitting 82 us).
+// Largest error against fp64 products at those sizes: 3.2e-6 and 3.0e-6 (library template 6.3e-6, FMA kernel 1.2e-5).
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -36,15 +45,16 @@ constexpr int kTmMaxSplit = 16;  // pairs that share a left-over tile, about
 // Ring sizes: what a block's copies need in flight (about 2 us of them) beside the blocks being worked on, in 227 KB.
 template <bool F32>
 struct TablesCfg {
+    static constexpr bool PAIR = !F32;         // two CTAs work on a tile together
     static constexpr int MT = F32 ? 1 : 2;     // row blocks of 128 a CTA works on at a time
-    static constexpr int ROWS = 256 * MT;      // rows of V per tile
+    static constexpr int ROWS = F32 ? 128 : 512;  // rows of V per tile
     static constexpr int BLK = F32 ? 32 : 64;  // columns of E per block: rows of 64 or 128 bytes of bf16
     static constexpr int CHUNK = F32 ? 4 : 8;  // blocks between two emptyings of an accumulator
     static constexpr int PART = 128 * BLK * 2;                // bytes of 128 rows of bf16
     static constexpr int A_BYTES = (F32 ? 3 : MT) * PART;     // a block's embeddings
-    static constexpr int W_BYTES = 3 * 64 * BLK * 2;          // a block's W: W1 (even CTA) or W2 (odd CTA), and half of W3
+    static constexpr int W_BYTES = (F32 ? 384 : 192) * BLK * 2;  // a block's W; a pair: W1 (even CTA) or W2 (odd), half of W3
     static constexpr int RAW = 128 * BLK * 4;                 // a block's fp32 embeddings
-    static constexpr int A_STAGES = F32 ? 3 : 4, W_STAGES = F32 ? 5 : 4, RAW_STAGES = F32 ? 5 : 1;
+    static constexpr int A_STAGES = F32 ? 3 : 4, W_STAGES = F32 ? 3 : 4, RAW_STAGES = F32 ? 4 : 1;
     static constexpr int THREADS = (kTmEpiWarps + 2 + (F32 ? 1 + kTmConvWarps : 0)) * 32;
     // (the rings start on a 1024-byte boundary)
     static constexpr size_t SMEM = (size_t)A_STAGES * A_BYTES + (size_t)W_STAGES * W_BYTES + (F32 ? (size_t)RAW_STAGES * RAW : 0) + 1024;
@@ -88,6 +98,7 @@ struct __align__(64) TablesParams {
     int V, m, m_pad, n_mb, n_kb;
     int pairs, full_rounds;
     int left, share_pairs;  // left-over tiles, pairs that share them
+    int box_n;              // fp32 embeddings: rows of W's boxes
     int wide;               // rows of the table are whole 32-byte sectors
 };
 
@@ -95,7 +106,7 @@ struct __align__(64) TablesParams {
 // tiles 0 .. left - 1), then whole tiles, one in every round.
 struct TablesItem {
     int tile, kb0, kb1;
-    int q0, q1;  // a piece: the first and the last pair that work on the tile (q0 == q1: the whole tile)
+    int q0, q1;  // a piece: the first and the last worker that work on the tile (q0 == q1: the whole tile)
     int seg;     // 0: the pair's share begins in this tile, 1: it began in the tile before
 };
 __device__ __forceinline__ int tables_share(const TablesParams& p, int pair) {
@@ -126,6 +137,14 @@ __device__ __forceinline__ bool tables_item(const TablesParams& p, int pair, int
     it.kb1 = p.n_kb;
     it.q0 = it.q1 = pair;
     return true;
+}
+
+// Columns of an accumulator: those of the tile's block of m, a multiple of 32.  (One CTA: W's parts stand one behind the
+// other in a stage, copied in boxes of n rows, so n is the same for every block.)
+template <bool F32>
+__device__ __forceinline__ int tables_n(const TablesParams& p, int mb) {
+    if (F32) return p.box_n;
+    return ((p.m - mb * 128 < 128 ? p.m - mb * 128 : 128) + 31) & ~31;
 }
 
 // W (fp32, [m, E]) -> three bf16 parts [3][m_pad][E_pad], zero where padded
@@ -173,7 +192,7 @@ __device__ __forceinline__ float4 ld_shared_f4(uint32_t at) {
 }
 
 template <bool F32>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TablesCfg<F32>::THREADS, 1)
+__global__ void __cluster_dims__(F32 ? 1 : 2, 1, 1) __launch_bounds__(TablesCfg<F32>::THREADS, 1)
     tables_mma_kernel(const __grid_constant__ TablesParams p) {
     using C = TablesCfg<F32>;
     constexpr uint32_t NA = C::A_STAGES, NW = C::W_STAGES, NR = C::RAW_STAGES;
@@ -182,17 +201,24 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TablesCfg<F32>::THRE
     __shared__ uint32_t s_tmem;
     __shared__ volatile int s_abort;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const uint32_t rank = cluster_ctarank();
-    const int pair = (int)blockIdx.x >> 1;
+    const uint32_t rank = C::PAIR ? cluster_ctarank() : 0u;
+    const int pair = C::PAIR ? (int)blockIdx.x >> 1 : (int)blockIdx.x;
+    auto wait = [&](uint32_t bar, uint32_t parity) {
+        if (C::PAIR)
+            mbar_wait_cluster(bar, parity, &s_abort);
+        else
+            mbar_wait_bounded(bar, parity, &s_abort);
+    };
     const uint32_t a_ring = (smem_u32(smem_raw) + 1023u) & ~1023u;
     const uint32_t w_ring = a_ring + NA * C::A_BYTES, raw_ring = w_ring + NW * C::W_BYTES;
-    // afull / wfull: a block's rows, W's are there in both CTAs (the even CTA's barriers), aempty / wempty: the instructions that read them are done, raw: fp32 rows as loaded
+    // afull / wfull: a block's rows, its W are there (a pair: in both CTAs; the even CTA's barriers), aempty / wempty: the
+    // instructions that read them are done, rfull / rempty: fp32 rows as loaded
     const uint32_t afull0 = smem_u32(bars), aempty0 = afull0 + 8 * NA, wfull0 = aempty0 + 8 * NA, wempty0 = wfull0 + 8 * NW;
     const uint32_t rfull0 = wempty0 + 8 * NW, rempty0 = rfull0 + 8 * NR;
     const uint32_t accfull0 = rempty0 + 8 * NR, accempty0 = accfull0 + 16;
     if (tid == 0) {
         for (uint32_t s = 0; s < NA; ++s) {
-            mbar_init(afull0 + 8 * s, F32 ? 2 * kTmConvWarps : 1);
+            mbar_init(afull0 + 8 * s, F32 ? kTmConvWarps : 1);
             mbar_init(aempty0 + 8 * s, 1);
         }
         for (uint32_t s = 0; s < NW; ++s) {
@@ -205,13 +231,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TablesCfg<F32>::THRE
         }
         for (int s = 0; s < 2; ++s) {
             mbar_init(accfull0 + 8 * s, 1);
-            mbar_init(accempty0 + 8 * s, 2 * kTmEpiWarps);  // (the even CTA's)
+            mbar_init(accempty0 + 8 * s, (C::PAIR ? 2 : 1) * kTmEpiWarps);  // (the even CTA's)
         }
         mbar_fence_init();
         s_abort = 0;
     }
     pdl_launch_dependents();  // (the kernel that adds up the pieces; it waits for this grid)
-    if (warp == 9) tmem_alloc_pair(smem_u32(&s_tmem), 512);
+    if (warp == 9) tmem_alloc<C::PAIR>(smem_u32(&s_tmem), 512);
     tc_fence_before();
     cluster_sync();
     tc_fence_after();
@@ -228,7 +254,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TablesCfg<F32>::THRE
         uint32_t cc = 0;  // chunks emptied so far
         for (int i = 0; tables_item(p, pair, i, it); ++i) {
             const int rt = it.tile / p.n_mb, mb = it.tile - rt * p.n_mb;
-            const uint32_t n = (uint32_t)((p.m - mb * 128 < 128 ? p.m - mb * 128 : 128) + 31) & ~31u;
+            const uint32_t n = (uint32_t)tables_n<F32>(p, mb);
             float acc[C::MT][64];
 #pragma unroll
             for (int h = 0; h < C::MT; ++h)
@@ -238,7 +264,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TablesCfg<F32>::THRE
 #pragma unroll
                 for (int h = 0; h < C::MT; ++h) {
                     const uint32_t slot = C::MT == 1 ? (cc & 1u) : (uint32_t)h;
-                    mbar_wait_cluster(accfull0 + 8 * slot, (C::MT == 1 ? cc >> 1 : cc) & 1u, &s_abort);
+                    wait(accfull0 + 8 * slot, (C::MT == 1 ? cc >> 1 : cc) & 1u);
                     tc_fence_after();
                     const uint32_t t0 = tmem + ((uint32_t)(32 * quarter) << 16) + slot * 256u + (uint32_t)half * 64u;
 #pragma unroll
@@ -254,7 +280,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TablesCfg<F32>::THRE
                     }
                     tc_fence_before();
                     __syncwarp();
-                    if (lane == 0) mbar_arrive_cluster(accempty_even + 8 * slot);
+                    if (lane == 0) {
+                        if (C::PAIR)
+                            mbar_arrive_cluster(accempty_even + 8 * slot);
+                        else
+                            mbar_arrive(accempty0 + 8 * slot);
+                    }
                 }
             }
             // a piece of a left-over tile goes to scratch, [ROWS][128], without the bias
@@ -297,12 +328,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TablesCfg<F32>::THRE
             TablesRing<NW> w(1);
             for (int i = 0; tables_item(p, pair, i, it); ++i) {
                 const int rt = it.tile / p.n_mb, mb = it.tile - rt * p.n_mb;
-                const int n = ((p.m - mb * 128 < 128 ? p.m - mb * 128 : 128) + 31) & ~31;
+                const int n = tables_n<F32>(p, mb);
                 const int w12 = (int)rank * p.m_pad + mb * 128, w3 = 2 * p.m_pad + mb * 128 + (int)rank * (n >> 1);
                 for (int kb = it.kb0; kb < it.kb1; ++kb) {
                     const int x = kb * C::BLK;
                     if (!F32) {
-                        if (a.t >= NA) mbar_wait_cluster(aempty0 + 8 * a.st, a.ph, &s_abort);
+                        if (a.t >= NA) wait(aempty0 + 8 * a.st, a.ph);
                         if (s_abort) break;  // (no copy is started any more)
                         if (rank == 0) mbar_arrive_expect_tx(afull0 + 8 * a.st, 2u * C::A_BYTES);
 #pragma unroll
@@ -311,13 +342,21 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TablesCfg<F32>::THRE
                                              rt * C::ROWS + h * 256 + (int)rank * 128, afull_even + 8 * a.st);
                         a.next();
                     }
-                    if (w.t >= NW) mbar_wait_cluster(wempty0 + 8 * w.st, w.ph, &s_abort);
+                    if (w.t >= NW) wait(wempty0 + 8 * w.st, w.ph);
                     if (s_abort) break;
                     const uint32_t dw = w_ring + w.st * C::W_BYTES, fb = wfull_even + 8 * w.st;
-                    if (rank == 0) mbar_arrive_expect_tx(wfull0 + 8 * w.st, 2u * C::W_BYTES);
-                    tma_load_2d_pair(dw, &p.map_w, x, w12, fb);
-                    tma_load_2d_pair(dw + C::W_BYTES / 3, &p.map_w, x, w12 + 64, fb);
-                    tma_load_2d_pair(dw + 2 * (C::W_BYTES / 3), &p.map_w, x, w3, fb);
+                    if (C::PAIR) {
+                        if (rank == 0) mbar_arrive_expect_tx(wfull0 + 8 * w.st, 2u * C::W_BYTES);
+                        tma_load_2d_pair(dw, &p.map_w, x, w12, fb);
+                        tma_load_2d_pair(dw + C::W_BYTES / 3, &p.map_w, x, w12 + 64, fb);
+                        tma_load_2d_pair(dw + 2 * (C::W_BYTES / 3), &p.map_w, x, w3, fb);
+                    } else {
+                        const uint32_t part = (uint32_t)n * C::BLK * 2;
+                        mbar_arrive_expect_tx(wfull0 + 8 * w.st, 3u * part);
+#pragma unroll
+                        for (int j = 0; j < 3; ++j)
+                            tma_load_2d(dw + j * part, &p.map_w, x, j * p.m_pad + mb * 128, wfull0 + 8 * w.st);
+                    }
                     w.next();
                 }
             }
@@ -334,13 +373,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TablesCfg<F32>::THRE
             uint32_t cc = 0;
             for (int i = 0; tables_item(p, pair, i, it); ++i) {
                 const int mb = it.tile % p.n_mb;
-                const int n = ((p.m - mb * 128 < 128 ? p.m - mb * 128 : 128) + 31) & ~31;
-                const uint32_t idesc2 = umma_idesc_bf16(256, 2 * n), idesc1 = umma_idesc_bf16(256, n);
+                const int n = tables_n<F32>(p, mb);
+                constexpr int M = C::PAIR ? 256 : 128;
+                const uint32_t idesc2 = umma_idesc_bf16(M, 2 * n), idesc1 = umma_idesc_bf16(M, n);
+                const uint32_t o_w3 = C::PAIR ? 2 * (C::W_BYTES / 3) : (uint32_t)n * (2 * C::BLK * 2);
                 for (int kb = it.kb0; kb < it.kb1; ++kb) {
                     const bool first = (kb - it.kb0) % C::CHUNK == 0;
                     const bool last = kb + 1 == it.kb1 || (kb + 1 - it.kb0) % C::CHUNK == 0;
-                    mbar_wait_cluster(wfull0 + 8 * w.st, w.ph, &s_abort);
-                    mbar_wait_cluster(afull0 + 8 * a.st, a.ph, &s_abort);
+                    wait(wfull0 + 8 * w.st, w.ph);
+                    wait(afull0 + 8 * a.st, a.ph);
                     tc_fence_after();
                     const uint32_t a0 = a_ring + a.st * C::A_BYTES, b0 = w_ring + w.st * C::W_BYTES;
                     // An instruction whose accumulator columns the one just ahead of it wrote waits for those; with two row
@@ -350,13 +391,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TablesCfg<F32>::THRE
                         const uint32_t d = tmem + (C::MT == 1 ? (cc & 1u) : (uint32_t)h) * 256u;
                         const uint64_t a1 = C::desc(a0 + h * C::PART + 32 * ks);
                         if (w3) {
-                            umma_pair(d + (uint32_t)n, a1, C::desc(b0 + 2 * (C::W_BYTES / 3) + 32 * ks), idesc1, true);
+                            umma<C::PAIR>(d + (uint32_t)n, a1, C::desc(b0 + o_w3 + 32 * ks), idesc1, true);
                         } else {
                             const uint64_t w12 = C::desc(b0 + 32 * ks);
-                            umma_pair(d, a1, w12, idesc2, !first || ks > 0);
+                            umma<C::PAIR>(d, a1, w12, idesc2, !first || ks > 0);
                             if (F32) {
-                                umma_pair(d, C::desc(a0 + C::PART + 32 * ks), w12, idesc2, true);
-                                umma_pair(d, C::desc(a0 + 2 * C::PART + 32 * ks), w12, idesc2, true);
+                                umma<C::PAIR>(d, C::desc(a0 + C::PART + 32 * ks), w12, idesc2, true);
+                                umma<C::PAIR>(d, C::desc(a0 + 2 * C::PART + 32 * ks), w12, idesc2, true);
                             }
                         }
                     };
@@ -376,7 +417,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TablesCfg<F32>::THRE
                             const uint32_t slot = C::MT == 1 ? (cc & 1u) : (uint32_t)h;
                             const uint32_t turn = C::MT == 1 ? cc >> 1 : cc;  // how often the set has been filled before
                             if (first && turn >= 1) {
-                                mbar_wait_cluster(accempty0 + 8 * slot, (turn - 1u) & 1u, &s_abort);
+                                wait(accempty0 + 8 * slot, (turn - 1u) & 1u);
                                 tc_fence_after();
                             }
                             if (!s_abort) {
@@ -386,11 +427,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TablesCfg<F32>::THRE
                                     mma(h, ks, true);
                                 }
                             }
-                            if (last) umma_commit_pair(accfull0 + 8 * slot);
+                            if (last) umma_commit<C::PAIR>(accfull0 + 8 * slot);
                         }
                     }
-                    umma_commit_pair(aempty0 + 8 * a.st);
-                    umma_commit_pair(wempty0 + 8 * w.st);
+                    umma_commit<C::PAIR>(aempty0 + 8 * a.st);
+                    umma_commit<C::PAIR>(wempty0 + 8 * w.st);
                     if (last) ++cc;
                     a.next();
                     w.next();
@@ -404,7 +445,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TablesCfg<F32>::THRE
             for (int i = 0; tables_item(p, pair, i, it); ++i) {
                 const int row = it.tile / p.n_mb * C::ROWS + (int)rank * 128;
                 for (int kb = it.kb0; kb < it.kb1; ++kb) {
-                    if (r.t >= NR) mbar_wait_bounded(rempty0 + 8 * r.st, r.ph, &s_abort);
+                    if (r.t >= NR) wait(rempty0 + 8 * r.st, r.ph);
                     if (s_abort) break;
                     mbar_arrive_expect_tx(rfull0 + 8 * r.st, C::RAW);
                     tma_load_2d(raw_ring + r.st * C::RAW, &p.map_e, kb * C::BLK, row, rfull0 + 8 * r.st);
@@ -417,12 +458,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TablesCfg<F32>::THRE
         // ------------------------------ fp32 embeddings -> bf16 parts ----------------------------
         const int ct = tid - (kTmEpiWarps + 3) * 32;
         const int c8 = ct & 3, r0 = ct >> 2;  // columns 8 c8 .. 8 c8 + 7 of rows r0 and r0 + 64
-        const uint32_t afull_even = mapa_u32(afull0, 0);
         TablesRing<NA> a(1);
         TablesRing<NR> r(0);
         for (int i = 0; tables_item(p, pair, i, it); ++i) {
             for (int kb = it.kb0; kb < it.kb1; ++kb) {
-                mbar_wait_bounded(rfull0 + 8 * r.st, r.ph, &s_abort);
+                wait(rfull0 + 8 * r.st, r.ph);
                 const uint32_t src = raw_ring + r.st * C::RAW;
                 float4 x[2][2];
 #pragma unroll
@@ -435,7 +475,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TablesCfg<F32>::THRE
                 __syncwarp();
                 if (lane == 0) mbar_arrive(rempty0 + 8 * r.st);
                 r.next();
-                if (a.t >= NA) mbar_wait_bounded(aempty0 + 8 * a.st, a.ph, &s_abort);
+                if (a.t >= NA) wait(aempty0 + 8 * a.st, a.ph);
                 const uint32_t dst = a_ring + a.st * C::A_BYTES;
 #pragma unroll
                 for (int q = 0; q < 2; ++q) {
@@ -452,7 +492,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TablesCfg<F32>::THRE
                 }
                 fence_proxy_async();
                 __syncwarp();
-                if (lane == 0) mbar_arrive_cluster(afull_even + 8 * a.st);
+                if (lane == 0) mbar_arrive(afull0 + 8 * a.st);
                 a.next();
             }
         }
@@ -462,7 +502,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TablesCfg<F32>::THRE
     tc_fence_before();
     cluster_sync();  // (the other CTA's last arrivals on this CTA's barriers, and its reads of this CTA's memory, are done)
     tc_fence_after();
-    if (warp == 9) tmem_free_pair(tmem, 512);
+    if (warp == 9) tmem_free<C::PAIR>(tmem, 512);
     if (tid == 0 && s_abort) atomicOr(p.errflag, 1);
 }
 
@@ -520,13 +560,13 @@ struct TablesSizes {
     int n_mb, m_pad, E_pad, pairs;
     size_t o_w, total;
 };
-TablesSizes tables_sizes(int num_sms, int E, int m) {
+TablesSizes tables_sizes(int num_sms, int E, int m, bool f32) {
     TablesSizes s;
     s.n_mb = (m + 127) / 128;
     s.m_pad = 128 * s.n_mb;
     s.E_pad = (E + 63) / 64 * 64;
-    s.pairs = num_sms / 2;
-    s.o_w = (size_t)s.pairs * 2 * TablesCfg<false>::ROWS * 128 * sizeof(float);
+    s.pairs = f32 ? num_sms : num_sms / 2;
+    s.o_w = (size_t)s.pairs * 2 * (f32 ? TablesCfg<true>::ROWS : TablesCfg<false>::ROWS) * 128 * sizeof(float);
     s.total = s.o_w + (size_t)3 * s.m_pad * s.E_pad * 2;
     return s;
 }
@@ -534,7 +574,7 @@ template <bool F32>
 cudaError_t tables_run(const TablesParams& p, cudaStream_t st, int* launches) {
     using C = TablesCfg<F32>;
     cudaError_t e = cudaFuncSetAttribute(tables_mma_kernel<F32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
-    if (e == cudaSuccess) e = launch_pdl(tables_mma_kernel<F32>, dim3(2 * p.pairs), dim3(C::THREADS), C::SMEM, st, p);
+    if (e == cudaSuccess) e = launch_pdl(tables_mma_kernel<F32>, dim3((C::PAIR ? 2 : 1) * p.pairs), dim3(C::THREADS), C::SMEM, st, p);
     *launches += 1;
     if (e == cudaSuccess && p.share_pairs > p.left) {
         e = launch_pdl(tables_pieces_kernel<F32>, dim3(C::ROWS / 8, p.left), dim3(256), 0, st, p);
@@ -549,18 +589,21 @@ cudaError_t tables_run(const TablesParams& p, cudaStream_t st, int* launches) {
 bool tables_mma_fits(const void* d_emb, graft_dtype dt, int E, const void* d_out) {
     return E % (dt == GRAFT_BF16 ? 8 : 4) == 0 && (((uintptr_t)d_emb | (uintptr_t)d_out) & 15) == 0 && encode_tiled() != nullptr;
 }
-size_t tables_mma_scratch_bytes(int num_sms, int E, int m) { return tables_sizes(num_sms, E, m).total; }
+size_t tables_mma_scratch_bytes(int num_sms, int E, int m, graft_dtype dt) {
+    return tables_sizes(num_sms, E, m, dt == GRAFT_F32).total;
+}
 
 // out [V, m] = emb [V, E] . W^T + bias.  scratch: tables_mma_scratch_bytes, 256-byte aligned.
 cudaError_t tables_mma_launch(graft_ctx* ctx, const void* d_emb, graft_dtype dt, int E, const float* d_W, const float* d_b,
                               float* d_out, void* scratch, cudaStream_t st) {
     const int V = ctx->cfg.V, m = ctx->cfg.m;
-    const TablesSizes s = tables_sizes(ctx->num_sms, E, m);
     const bool f32 = dt == GRAFT_F32;
+    const TablesSizes s = tables_sizes(ctx->num_sms, E, m, f32);
     __nv_bfloat16* w = (__nv_bfloat16*)((char*)scratch + s.o_w);
     TablesParams p;
     const int blk = f32 ? TablesCfg<true>::BLK : TablesCfg<false>::BLK;
-    if (!encode_map(&p.map_w, w, false, (uint64_t)3 * s.m_pad, s.E_pad, 64, 2 * blk) ||
+    p.box_n = s.n_mb > 1 ? 128 : (m + 31) / 32 * 32;
+    if (!encode_map(&p.map_w, w, false, (uint64_t)3 * s.m_pad, s.E_pad, f32 ? p.box_n : 64, 2 * blk) ||
         !encode_map(&p.map_e, d_emb, f32, V, E, 128, 128))
         return cudaErrorUnknown;
     p.bias = d_b;

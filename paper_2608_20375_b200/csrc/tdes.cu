@@ -1,6 +1,7 @@
 // TDES (Sec. 3.2): the cached bi-tower projections and the per-round edge scores.
 //
-//   tdes_precompute_kernel   out[v] = W e_v + b            (text after Eq. 6: computed once per model)
+//   tdes_precompute_kernel   out[v] = W e_v + b            (text after Eq. 6: computed once per model; rows the tensor
+//                            cores cannot load, see tables_mma.cu)
 //   tdes_edges_kernel        edge[d][i][c] = log q_d(c) + beta * (f - mean_c f),
 //                            f = s (P[p_i] + u_d) . (C[c] + u_d) / sqrt(m)          (Eq. 4-6)
 //                            for the first depths of every sequence (the arithmetic is in edge_score.cuh,
