@@ -89,6 +89,7 @@ struct graft_ctx {
     double* w_cos;                // [max_batch, L] adjacent-position cosines (Eq. 15)
     graft::SabaResult* w_saba;    // [max_batch] budgets worked out by the edge-score kernel
     double* w_fit;                // [32] normal equations of graft_saba_fit and its arrival counter, zero between calls
+    double* w_loss;               // [8] sums of graft_tdes_loss and its arrival counter, zero between calls
     int32_t* w_errflag;           // [1] device-side internal error flag
     graft::VpPlan vp_plan;
     // scratch of the tensor-core table precompute (allocated on its first use: pieces of split tiles, W's bf16 parts)
