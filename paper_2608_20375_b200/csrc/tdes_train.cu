@@ -378,32 +378,45 @@ __device__ __forceinline__ void smem_add4(float4* q, const float4& v) { *q = add
 
 // What the warps of a CTA share, and this warp's place in it.
 struct TrainCtx {
-    const float4* u;  // [L][m / 4] shared copy of the depth embeddings
+    const float* u;   // [L][m] shared copy of the depth embeddings
     float* gu;        // [L][m] this warp's sums (or the CTA's, with atomics)
     float4* hot;      // [2][kTsSlots][32] this warp's sums of the hot rows
     bool gu_shared, on;  // on: this lane holds a part of a row
-    int lane;
+    int lane, m;
 };
+// FULL: m = 128, every lane holds a part of a row
+template <bool FULL>
+__device__ __forceinline__ float4* ctx_at(const TrainCtx& c, const float* table, int tok) {
+    return (float4*)(table + (size_t)tok * (FULL ? 128 : c.m)) + c.lane;
+}
+template <bool FULL>
 __device__ __forceinline__ void ctx_add_row(const TrainParams& p, const TrainCtx& c, int t, int tok, int slot, const float4& v) {
     if (slot >= 0)  // (uniform)
         smem_add4(c.hot + (t * kTsSlots + slot) * 32 + c.lane, v);
-    else if (c.on)
-        atomicAdd((float4*)((t == 0 ? p.gP : p.gC) + (size_t)tok * p.m) + c.lane, v);
+    else if (FULL || c.on)
+        atomicAdd(ctx_at<FULL>(c, t == 0 ? p.gP : p.gC, tok), v);
 }
-__device__ __forceinline__ void ctx_add_u(const TrainParams& p, const TrainCtx& c, int d, const float4& v) {
-    if (!c.on) return;
-    float* q = c.gu + (size_t)(d - 1) * p.m + 4 * c.lane;
+template <bool FULL>
+__device__ __forceinline__ void ctx_add_u(const TrainCtx& c, int d, const float4& v) {
+    if (!FULL && !c.on) return;
+    float4* q = ctx_at<FULL>(c, c.gu, d - 1);
     if (!c.gu_shared) {
-        smem_add4((float4*)q, v);
+        smem_add4(q, v);
     } else {
-        atomicAdd(q + 0, v.x);
-        atomicAdd(q + 1, v.y);
-        atomicAdd(q + 2, v.z);
-        atomicAdd(q + 3, v.w);
+        float* f = (float*)q;
+        atomicAdd(f + 0, v.x);
+        atomicAdd(f + 1, v.y);
+        atomicAdd(f + 2, v.z);
+        atomicAdd(f + 3, v.w);
     }
 }
-__device__ __forceinline__ float4 ctx_load(const TrainParams& p, const TrainCtx& c, const float* table, int tok) {
-    return c.on ? __ldg((const float4*)(table + (size_t)tok * p.m) + c.lane) : make_float4(0.f, 0.f, 0.f, 0.f);
+template <bool FULL>
+__device__ __forceinline__ float4 ctx_load(const TrainCtx& c, const float* table, int tok) {
+    return FULL || c.on ? __ldg(ctx_at<FULL>(c, table, tok)) : make_float4(0.f, 0.f, 0.f, 0.f);
+}
+template <bool FULL>
+__device__ __forceinline__ float4 ctx_u(const TrainCtx& c, int d) {
+    return FULL || c.on ? *ctx_at<FULL>(c, c.u, d - 1) : make_float4(0.f, 0.f, 0.f, 0.f);
 }
 
 // The i-th of kTsSample tokens spread evenly over the references to a table (0: P, 1: C), or -1.
@@ -424,7 +437,7 @@ __device__ __forceinline__ int train_sample(const TrainParams& p, int t, int i) 
 }
 
 // KC: children held in registers, a multiple of 8 (K <= KC)
-template <int KC>
+template <int KC, bool FULL>
 __global__ void __launch_bounds__(kTsThreads, 1) tdes_loss_rows_kernel(const TrainParams p) {
     extern __shared__ __align__(16) float smem_f[];
     __shared__ TrainHot s_hot;
@@ -439,12 +452,13 @@ __global__ void __launch_bounds__(kTsThreads, 1) tdes_loss_rows_kernel(const Tra
     float* s_gu = smem_f + Lm;
     float* s_rows = s_gu + (size_t)Lm * p.gu_copies;
     TrainCtx c;
-    c.u = (const float4*)smem_f;
+    c.u = smem_f;
     c.gu_shared = p.gu_copies == 1;
     c.gu = s_gu + (c.gu_shared ? 0 : (size_t)warp * Lm);
     c.hot = (float4*)(s_rows + (size_t)warp * 2 * kTsSlots * 128);
     c.on = lane < p.m / 4;
     c.lane = lane;
+    c.m = p.m;
     for (int i = tid; i < Lm; i += kTsThreads) smem_f[i] = p.u[i];
     if (grad) {
         for (int i = tid; i < Lm * p.gu_copies; i += kTsThreads) s_gu[i] = 0.f;
@@ -487,32 +501,43 @@ __global__ void __launch_bounds__(kTsThreads, 1) tdes_loss_rows_kernel(const Tra
     float gs = 0.f;
     int skipped = 0;
 
-    // ---- distribution level (Eq. 7-9): lane i owns child i
+    // ---- distribution level (Eq. 7-9): lane i owns child i; the next group's ids are on their way while one is worked on
+    int n_tp = 0, n_d = 0, n_tc = 0;
+    float n_z = 0.f, n_lq = 0.f;
+    auto fetch = [&](int g) {
+        if (g >= p.n_groups) return;
+        n_tp = p.g_parent[g];
+        n_d = p.g_depth[g];
+        const size_t at = (size_t)g * p.K + lane;
+        n_tc = lane < p.K ? p.g_child[at] : 0;
+        n_z = lane < p.K ? p.g_ztgt[at] : -INFINITY;
+        n_lq = lane < p.K ? p.g_logq[at] : -INFINITY;
+    };
+    fetch(wid);
     for (int g = wid; g < p.n_groups; g += nw) {
-        const int tp = p.g_parent[g], d = p.g_depth[g];
-        const int tc = lane < p.K ? p.g_child[(size_t)g * p.K + lane] : 0;
-        const float z = lane < p.K ? p.g_ztgt[(size_t)g * p.K + lane] : -INFINITY;
-        const float lq = lane < p.K ? p.g_logq[(size_t)g * p.K + lane] : -INFINITY;
+        const int tp = n_tp, d = n_d, tc = n_tc;
+        const float z = n_z, lq = n_lq;
+        fetch(g + nw);
         if (!(tok_ok(tp, p.V) && d >= 1 && d <= p.L && __all_sync(0xFFFFFFFFu, tok_ok(tc, p.V)))) {
             skipped += lane == 0 ? 1 : 0;
             continue;
         }
+        const float4 prow = ctx_load<FULL>(c, p.P, tp);
         float4 rows[KC];
 #pragma unroll
         for (int i = 0; i < KC; ++i) {
             const int t = __shfl_sync(0xFFFFFFFFu, tc, i);
-            rows[i] = i < p.K ? ctx_load(p, c, p.C, t) : zero4;
+            rows[i] = i < p.K ? ctx_load<FULL>(c, p.C, t) : zero4;
         }
-        const float4 u = c.on ? c.u[(size_t)(d - 1) * (p.m / 4) + lane] : zero4;
-        const float4 a = add4(ctx_load(p, c, p.P, tp), u);
+        const float4 u = ctx_u<FULL>(c, d), a = add4(prow, u);
         // f = k0 (a . C + a . u)
+        const float au = dot4(a, u);
         float part[KC];
 #pragma unroll
-        for (int i = 0; i < KC; ++i) part[i] = dot4(a, rows[i]);
-        const float au = warp_sum(dot4(a, u));
+        for (int i = 0; i < KC; ++i) part[i] = au + dot4(a, rows[i]);
         const float dots = warp_sums<KC>(part, lane);
         constexpr int SH = KC == 32 ? 0 : (KC == 16 ? 1 : 2);
-        const float dot_c = (SH == 0 ? dots : __shfl_sync(0xFFFFFFFFu, dots, (lane << SH) & 31)) + au;
+        const float dot_c = SH == 0 ? dots : __shfl_sync(0xFFFFFFFFu, dots, (lane << SH) & 31);
         const float al = lane < p.K ? lq + p.k0 * dot_c : -INFINITY;
         float zmax = z, amax = al;
 #pragma unroll
@@ -527,25 +552,26 @@ __global__ void __launch_bounds__(kTsThreads, 1) tdes_loss_rows_kernel(const Tra
         if (!grad) continue;
         const float gf = lane < p.K ? p.w_kl * (ph - pt) : 0.f;  // d L / d f
         if (lane < p.K) gs += gf * dot_c * p.inv_sqrt_m;
-        const float coef = gf * p.k0, csum = warp_sum(coef);
+        const float coef = gf * p.k0;
         const int slot = lane < p.K ? hot_slot(hot, 1, tc) : -1;
         const uint32_t hots = __ballot_sync(0xFFFFFFFFu, slot >= 0);
-        float4 acc = mul4(csum, u);  // sum_c coef_c (C_c + u)
+        // sum_c coef_c (C_c + u) = sum_c coef_c C_c: the coefficients, differences of two distributions, add up to 0
+        float4 acc = zero4;
 #pragma unroll
         for (int i = 0; i < KC; ++i) {
             if (i < p.K) {
                 const float cf = __shfl_sync(0xFFFFFFFFu, coef, i);
                 const int t = __shfl_sync(0xFFFFFFFFu, tc, i);
                 acc = fma4(cf, rows[i], acc);
-                const float4 v = mul4(cf, a);
-                if ((hots >> i) & 1u)
-                    ctx_add_row(p, c, 1, t, __shfl_sync(0xFFFFFFFFu, slot, i), v);
-                else
-                    ctx_add_row(p, c, 1, t, -1, v);
+                if (!((hots >> i) & 1u) && (FULL || c.on)) atomicAdd(ctx_at<FULL>(c, p.gC, t), mul4(cf, a));
             }
         }
-        ctx_add_row(p, c, 0, tp, hot_slot(hot, 0, tp), acc);
-        ctx_add_u(p, c, d, fma4(csum, a, acc));
+        for (uint32_t left = hots; left != 0u; left &= left - 1u) {  // (uniform)
+            const int i = __ffs(left) - 1;
+            smem_add4(c.hot + (kTsSlots + __shfl_sync(0xFFFFFFFFu, slot, i)) * 32 + lane, mul4(__shfl_sync(0xFFFFFFFFu, coef, i), a));
+        }
+        ctx_add_row<FULL>(p, c, 0, tp, hot_slot(hot, 0, tp), acc);
+        ctx_add_u<FULL>(c, d, acc);
     }
     // ---- pairwise level (Eq. 10): blocks of eight pairs, four at a time; lanes 0-7 hold the block's ids
     for (int b0 = wid * 8; b0 < p.n_pairs; b0 += nw * 8) {
@@ -572,17 +598,17 @@ __global__ void __launch_bounds__(kTsThreads, 1) tdes_loss_rows_kernel(const Tra
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 const int s = 4 * h + i;
-                a1[i] = ctx_load(p, c, p.P, __shfl_sync(0xFFFFFFFFu, id[0], s));
-                b1[i] = ctx_load(p, c, p.C, __shfl_sync(0xFFFFFFFFu, id[1], s));
-                a2[i] = ctx_load(p, c, p.P, __shfl_sync(0xFFFFFFFFu, id[3], s));
-                b2[i] = ctx_load(p, c, p.C, __shfl_sync(0xFFFFFFFFu, id[4], s));
+                a1[i] = ctx_load<FULL>(c, p.P, __shfl_sync(0xFFFFFFFFu, id[0], s));
+                b1[i] = ctx_load<FULL>(c, p.C, __shfl_sync(0xFFFFFFFFu, id[1], s));
+                a2[i] = ctx_load<FULL>(c, p.P, __shfl_sync(0xFFFFFFFFu, id[3], s));
+                b2[i] = ctx_load<FULL>(c, p.C, __shfl_sync(0xFFFFFFFFu, id[4], s));
             }
             float part[8];
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 const int s = 4 * h + i, d1 = __shfl_sync(0xFFFFFFFFu, id[2], s), d2 = __shfl_sync(0xFFFFFFFFu, id[5], s);
-                const float4 u1 = c.on ? c.u[(size_t)(d1 - 1) * (p.m / 4) + lane] : zero4;
-                const float4 u2 = c.on ? c.u[(size_t)(d2 - 1) * (p.m / 4) + lane] : zero4;
+                const float4 u1 = ctx_u<FULL>(c, d1);
+                const float4 u2 = ctx_u<FULL>(c, d2);
                 a1[i] = add4(a1[i], u1);
                 b1[i] = add4(b1[i], u1);
                 a2[i] = add4(a2[i], u2);
@@ -611,23 +637,23 @@ __global__ void __launch_bounds__(kTsThreads, 1) tdes_loss_rows_kernel(const Tra
                 const int p2 = __shfl_sync(0xFFFFFFFFu, id[3], s), c2 = __shfl_sync(0xFFFFFFFFu, id[4], s), d2 = __shfl_sync(0xFFFFFFFFu, id[5], s);
                 const int h1 = __shfl_sync(0xFFFFFFFFu, sp1, s), h2 = __shfl_sync(0xFFFFFFFFu, sc1, s);
                 if (p1 == p2) {  // (uniform; an alternative keeps the pair's parent or its child: one addition for both)
-                    ctx_add_row(p, c, 0, p1, h1, mul4(cf, sub4(b2[i], b1[i])));
+                    ctx_add_row<FULL>(p, c, 0, p1, h1, mul4(cf, sub4(b2[i], b1[i])));
                 } else {
-                    ctx_add_row(p, c, 0, p1, h1, mul4(-cf, b1[i]));
-                    ctx_add_row(p, c, 0, p2, __shfl_sync(0xFFFFFFFFu, sp2, s), mul4(cf, b2[i]));
+                    ctx_add_row<FULL>(p, c, 0, p1, h1, mul4(-cf, b1[i]));
+                    ctx_add_row<FULL>(p, c, 0, p2, __shfl_sync(0xFFFFFFFFu, sp2, s), mul4(cf, b2[i]));
                 }
                 if (c1 == c2) {
-                    ctx_add_row(p, c, 1, c1, h2, mul4(cf, sub4(a2[i], a1[i])));
+                    ctx_add_row<FULL>(p, c, 1, c1, h2, mul4(cf, sub4(a2[i], a1[i])));
                 } else {
-                    ctx_add_row(p, c, 1, c1, h2, mul4(-cf, a1[i]));
-                    ctx_add_row(p, c, 1, c2, __shfl_sync(0xFFFFFFFFu, sc2, s), mul4(cf, a2[i]));
+                    ctx_add_row<FULL>(p, c, 1, c1, h2, mul4(-cf, a1[i]));
+                    ctx_add_row<FULL>(p, c, 1, c2, __shfl_sync(0xFFFFFFFFu, sc2, s), mul4(cf, a2[i]));
                 }
                 const float4 s1 = add4(a1[i], b1[i]), s2 = add4(a2[i], b2[i]);
                 if (d1 == d2) {
-                    ctx_add_u(p, c, d1, mul4(cf, sub4(s2, s1)));
+                    ctx_add_u<FULL>(c, d1, mul4(cf, sub4(s2, s1)));
                 } else {
-                    ctx_add_u(p, c, d1, mul4(-cf, s1));
-                    ctx_add_u(p, c, d2, mul4(cf, s2));
+                    ctx_add_u<FULL>(c, d1, mul4(-cf, s1));
+                    ctx_add_u<FULL>(c, d2, mul4(cf, s2));
                 }
             }
         }
@@ -651,14 +677,14 @@ __global__ void __launch_bounds__(kTsThreads, 1) tdes_loss_rows_kernel(const Tra
         float4 a[8], b[8];
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
-            a[i] = ctx_load(p, c, p.P, __shfl_sync(0xFFFFFFFFu, tp, i));
-            b[i] = ctx_load(p, c, p.C, __shfl_sync(0xFFFFFFFFu, tc, i));
+            a[i] = ctx_load<FULL>(c, p.P, __shfl_sync(0xFFFFFFFFu, tp, i));
+            b[i] = ctx_load<FULL>(c, p.C, __shfl_sync(0xFFFFFFFFu, tc, i));
         }
         float part[8];
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
             const int dd = __shfl_sync(0xFFFFFFFFu, d, i);
-            const float4 u = c.on ? c.u[(size_t)(dd - 1) * (p.m / 4) + lane] : zero4;
+            const float4 u = ctx_u<FULL>(c, dd);
             a[i] = add4(a[i], u);
             b[i] = add4(b[i], u);
             part[i] = dot4(a[i], b[i]);
@@ -677,9 +703,9 @@ __global__ void __launch_bounds__(kTsThreads, 1) tdes_loss_rows_kernel(const Tra
         for (int i = 0; i < 8; ++i) {
             if (!((oks >> i) & 1u)) continue;  // (uniform)
             const float cf = __shfl_sync(0xFFFFFFFFu, coef, 4 * i);
-            ctx_add_row(p, c, 0, __shfl_sync(0xFFFFFFFFu, tp, i), __shfl_sync(0xFFFFFFFFu, sp, i), mul4(cf, b[i]));
-            ctx_add_row(p, c, 1, __shfl_sync(0xFFFFFFFFu, tc, i), __shfl_sync(0xFFFFFFFFu, sc, i), mul4(cf, a[i]));
-            ctx_add_u(p, c, __shfl_sync(0xFFFFFFFFu, d, i), mul4(cf, add4(a[i], b[i])));
+            ctx_add_row<FULL>(p, c, 0, __shfl_sync(0xFFFFFFFFu, tp, i), __shfl_sync(0xFFFFFFFFu, sp, i), mul4(cf, b[i]));
+            ctx_add_row<FULL>(p, c, 1, __shfl_sync(0xFFFFFFFFu, tc, i), __shfl_sync(0xFFFFFFFFu, sc, i), mul4(cf, a[i]));
+            ctx_add_u<FULL>(c, __shfl_sync(0xFFFFFFFFu, d, i), mul4(cf, add4(a[i], b[i])));
         }
     }
     // ---- per-CTA sums, then one round of global atomics
@@ -746,7 +772,8 @@ static size_t tdes_loss_smem(const graft_config& cfg) {
     return (lm * (1 + rows_gu_copies(cfg)) + (size_t)kTsWarps * 2 * kTsSlots * 128) * sizeof(float);
 }
 static void (*rows_kernel(const graft_config& cfg))(const TrainParams) {
-    return cfg.K <= 8 ? tdes_loss_rows_kernel<8> : (cfg.K <= 16 ? tdes_loss_rows_kernel<16> : tdes_loss_rows_kernel<32>);
+    if (cfg.m == 128) return cfg.K <= 8 ? tdes_loss_rows_kernel<8, true> : (cfg.K <= 16 ? tdes_loss_rows_kernel<16, true> : tdes_loss_rows_kernel<32, true>);
+    return cfg.K <= 8 ? tdes_loss_rows_kernel<8, false> : (cfg.K <= 16 ? tdes_loss_rows_kernel<16, false> : tdes_loss_rows_kernel<32, false>);
 }
 
 cudaError_t tdes_loss_launch(graft_ctx* ctx, const graft_tdes_traces* tr, const graft_tdes_loss_config* lc,
