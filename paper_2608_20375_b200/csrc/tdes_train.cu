@@ -315,11 +315,16 @@ __global__ void __launch_bounds__(kTrThreads) tdes_loss_kernel(const TrainParams
 //   * every warp adds into a copy of gu of its own (a plain load, add and store);
 //   * the few hottest tokens' gradient rows (additions to one row serialise in L2) are picked once per CTA from a sample of
 //     the tokens, and every warp keeps its sums of them in shared memory; everything else is a 16-byte vector atomic.
-// Measured (B200, V = 151,936, m = 128, 32,768 groups of 32, 131,072 pairs, 262,144 edges): LOSS_FIGURES
+// Measured (B200, V = 151,936, m = 128, L = 16, 32,768 groups of 32, 131,072 pairs, 262,144 edges): 337 us (434 us by the
+// one-item-a-warp kernel with replaced cached rows).  What bounds it now: the vector atomics -- a million rows spread
+// evenly take 96 us whether from 8 or from 32 warps an SM or as bulk reductions from shared memory, a million with the
+// Zipf(1.1) tokens of these traces 790 us, without their eight hottest 152 us -- and, in front of them in the same
+// queue, 1.6 million row loads (138 us for the losses alone).  One copy of gu with atomics instead of one a warp leaves
+// more L1 for the rows but costs more than it saves (360 us).
 constexpr int kTsThreads = 384;
 constexpr int kTsWarps = kTsThreads / 32;
 constexpr int kTsSample = 256;
-constexpr int kTsSampleMin = 16384;  // references to rows from which the sample is worth its 2 us
+constexpr int kTsSampleMin = 16384;  // references to rows from which looking for hot ones (about 2 us) is worth it
 
 constexpr int kTsSlots = 8;  // hot rows per table
 struct __align__(16) TrainHot {

@@ -66,6 +66,11 @@ def _compare(got, ref, grad=True):
     (1500, 4, 8, 256, 200, 300, 0),         # two 128-float chunks per row, no edges
     (1200, 3, 7, 384, 150, 150, 150),       # three chunks
     (900, 32, 1, 8, 100, 100, 100),         # K = 1: pi = 1, the distribution term vanishes
+    (5000, 16, 8, 128, 1801, 3001, 4007),   # children held eight at a time, enough rows to look for hot ones
+    (5000, 16, 9, 128, 1500, 2500, 3003),   # sixteen
+    (5000, 32, 16, 128, 1500, 2500, 3003),  # one copy of gu (L m > 2048)
+    (5000, 16, 17, 124, 1000, 2500, 3003),  # thirty-two, lanes without a part of a row
+    (400, 16, 4, 64, 7, 9, 17),             # less than a block of items
 ])
 def test_loss_and_gradients(V, L, K, m, ng, npair, ne):
     g, P, Ct, u, s, keep = _ctx(V, L, K, m, seed=V + m)
@@ -79,6 +84,25 @@ def test_loss_and_gradients(V, L, K, m, ng, npair, ne):
     # losses only: the same losses, nothing else written
     lo = _run(g, V, L, m, tr, grad=False)
     assert np.array_equal(lo["loss"], got["loss"]) or np.allclose(lo["loss"], got["loss"], rtol=1e-12)
+    g.destroy()
+
+
+@pytest.mark.parametrize("same", ["parent", "child", "both", "none"])
+def test_pairs_that_share_a_row(same):
+    """An alternative that keeps the pair's parent or child: one addition stands for two."""
+    V, L, K, m = 300, 16, 4, 128
+    g, P, Ct, u, s, keep = _ctx(V, L, K, m, seed=31)
+    tr = gi.tdes_traces(V, L, K, 8, 5000, 8, seed=32)
+    pr = tr["pairs"]
+    rng = np.random.default_rng(33)
+    pr[:, 3:] = np.stack([rng.integers(0, V, 5000), rng.integers(0, V, 5000), rng.integers(1, L + 1, 5000)], 1)
+    if same in ("parent", "both"):
+        pr[:, 3] = pr[:, 0]
+    if same in ("child", "both"):
+        pr[:, 4] = pr[:, 1]
+    pr[::3, 5] = pr[::3, 2]
+    got = _run(g, V, L, m, tr)
+    _compare(got, oracle.tdes_loss(P, Ct, u, s, tr["groups"], tr["pairs"], tr["edges"], **CFG))
     g.destroy()
 
 
