@@ -393,6 +393,7 @@ struct __align__(16) EpiShared {  // private to one epilogue group
     uint32_t hits[kVpHitCap];
     uint16_t hthreads[NT];  // streaming threads whose maximum reaches T
     int nhits, ncand, nht, ovf;
+    int arrived;    // records of a shared row that were there before this CTA's
     int tie_groups;  // groups of threads whose maximum is T (to 16 bits): many of them means bulk ties at T
     int fill_ninf;  // the threshold fell on -inf: the candidates are the finite elements plus the first -inf ones
     int fill_tie;   // too many chunks reach the threshold T (bulk ties at T): the candidates are the elements above T
@@ -1189,98 +1190,124 @@ __global__ void __launch_bounds__(kVpThreads, 1) vocab_pass_kernel(const VpParam
                 nk = warp_fallback_select<BF16>(es, p, sg, cmx, lane, es->fill_ninf ? 0ull : ((uint64_t)Tv << 32) - 1ull);
             }
             epi_bar(grp);
-            if (ew != 0) continue;
             // the double-buffered arrays of parity pb may be reused from here on
-            __syncwarp();
-            if (lane == 0) mbar_arrive(done0 + 8 * pb);
+            if (ew == 0) {
+                __syncwarp();
+                if (lane == 0) mbar_arrive(done0 + 8 * pb);
+            }
             // (g) finish the row, or leave a record for the CTA that arrives last
             // (a whole row is nobody else's: the divisions that find a shared row's CTAs are for partial rows only)
             const bool whole_row = sg.e0 == 0 && sg.e1 == p.V;
-            const long long x0 = (long long)sg.row * p.nq;
-            const int c_first = whole_row ? (int)blockIdx.x : cta_of(x0, p.Q, G);
-            const int c_last = whole_row ? (int)blockIdx.x : cta_of(x0 + p.nq - 1, p.Q, G);
-            const int nseg = c_last - c_first + 1;
             double Cd = (double)c, Sd = (double)s;
             uint32_t Vm = vmo;
-            bool finish = (nseg == 1);
+            bool finish = whole_row;
             int rec_internal = 0;  // a bounded wait ran out in one of the CTAs that left a record for this row
-            if (nseg > 1) {
+            if (!whole_row) {
+                const long long x0 = (long long)sg.row * p.nq;
+                const int c_first = cta_of(x0, p.Q, G), nseg = cta_of(x0 + p.nq - 1, p.Q, G) - c_first + 1;
                 const int my_first_row = (int)(q0 / p.nq);
-                VpRecord* rec = p.records + (size_t)blockIdx.x * 2 + (sg.row == my_first_row ? 0 : 1);
-                if (lane < kMaxK) rec->keys[lane] = lane < nk ? es->outk[lane] : 0ull;
-                if (lane == 0) {
-                    rec->c = c;
-                    rec->s = s;
-                    rec->vmax = __uint_as_float(vmo);
-                    rec->nkeys = (uint32_t)nk | (sh->abort_flag ? 0x80000000u : 0u);
-                }
-                __threadfence();
-                __syncwarp();
-                int old = 0;
-                if (lane == 0) {
-                    old = atomicAdd(p.row_counter + sg.row, 1);
+                if (ew == 0) {
+                    VpRecord* rec = p.records + (size_t)blockIdx.x * 2 + (sg.row == my_first_row ? 0 : 1);
+                    if (lane < kMaxK) rec->keys[lane] = lane < nk ? es->outk[lane] : 0ull;
+                    if (lane == 0) {
+                        rec->c = c;
+                        rec->s = s;
+                        rec->vmax = __uint_as_float(vmo);
+                        rec->nkeys = (uint32_t)nk | (sh->abort_flag ? 0x80000000u : 0u);
+                    }
                     __threadfence();
+                    __syncwarp();
+                    if (lane == 0) {
+                        es->arrived = nseg == 1 ? 0 : atomicAdd(p.row_counter + sg.row, 1);
+                        __threadfence();
+                    }
                 }
-                old = __shfl_sync(0xFFFFFFFFu, old, 0);
-                if (old == nseg - 1) {
+                epi_bar(grp);
+                if (es->arrived == nseg - 1) {  // (uniform)
                     finish = true;
-                    // merge the records of CTAs c_first..c_last, a round at a time
-                    const int per_round = (kVpCandCap - kMaxK) / kMaxK;
-                    int have = 0;
-                    for (int c0 = c_first; c0 <= c_last; c0 += per_round) {
-                        const int c1 = c0 + per_round - 1 < c_last ? c0 + per_round - 1 : c_last;
-                        int n = have, ovf = 0;
-                        for (int i0 = 0; i0 < (c1 - c0 + 1) * kMaxK; i0 += 32) {
-                            const int i = i0 + lane;
-                            const int cc = c0 + i / kMaxK, kk = i % kMaxK;
-                            const int c_row0 = (int)(cta_start(cc, p.Q, G) / p.nq);
-                            const VpRecord* r = p.records + (size_t)cc * 2 + (sg.row == c_row0 ? 0 : 1);
-                            const uint64_t key = __ldcg((const unsigned long long*)&r->keys[kk]);
-                            n = warp_append(es->cand, n, kVpCandCap, key != 0ull, key, lane, &ovf);
+                    // Merge the records of the row's CTAs, the group's 128 threads together.  Every CTA after the first
+                    // starts inside the row, so the row is its first and its record the first of its two; every record's
+                    // keys are in descending order (empty ones, 0, last): a key's rank is its place in its own record plus
+                    // the places that a binary search finds for it in the others.  (One warp that ranked all keys against
+                    // each other took 10 us of a batch-1 round.)
+                    const VpRecord* rec0 = p.records + (size_t)c_first * 2 + ((int)(cta_start(c_first, p.Q, G) / p.nq) == sg.row ? 0 : 1);
+                    auto record = [&](int i) { return i == 0 ? rec0 : p.records + (size_t)(c_first + i) * 2; };
+                    // the log-sum-exp pieces (warp 0), on their way while the keys are ranked
+                    float rc = -INFINITY, rs = 0.f;
+                    uint32_t rv = 0u;
+                    int have_all = 0;
+                    if (ew == 0 && lane < nseg) {
+                        const VpRecord* r = record(lane);
+                        rc = __ldcg(&r->c);
+                        rs = __ldcg(&r->s);
+                        rv = __float_as_uint(__ldcg(&r->vmax));
+                        const uint32_t kn = __ldcg(&r->nkeys);
+                        have_all = (int)(kn & 0x7FFFFFFFu);
+                        rec_internal = (int)(kn >> 31);
+                    }
+                    constexpr int kRound = kVpCandCap / kMaxK - 1;  // records a round, behind the best of the rounds before
+                    int have = 0;                                   // lists of kMaxK keys carried over: 0 or 1
+                    for (int r0 = 0; r0 < nseg; r0 += kRound) {
+                        const int cnt = nseg - r0 < kRound ? nseg - r0 : kRound, n = (have + cnt) * kMaxK;
+                        for (int i = etid; i < cnt * kMaxK; i += kVpEpiThreads)
+                            es->cand[have * kMaxK + i] = __ldcg((const unsigned long long*)&record(r0 + i / kMaxK)->keys[i % kMaxK]);
+                        if (etid < kMaxK) es->outk[etid] = 0ull;
+                        epi_bar(grp);
+                        for (int i = etid; i < n; i += kVpEpiThreads) {
+                            const uint64_t key = es->cand[i];
+                            int rank = i % kMaxK;
+                            for (int l = 0; l < n; l += kMaxK) {
+                                if (l == i - i % kMaxK) continue;
+                                int pos = 0;  // keys of list l above this one
+#pragma unroll
+                                for (int step = kMaxK / 2; step >= 1; step >>= 1)
+                                    if (es->cand[l + pos + step - 1] > key) pos += step;
+                                rank += pos + (es->cand[l + pos] > key ? 1 : 0);
+                            }
+                            if (key != 0ull && rank < p.K) es->outk[rank] = key;
                         }
-                        warp_select_topk(es, n, p.K, lane);
-                        have = n < p.K ? n : p.K;
-                        if (lane < have) es->cand[lane] = es->outk[lane];
-                        __syncwarp();
+                        epi_bar(grp);
+                        if (r0 + kRound < nseg) {  // (uniform)
+                            if (etid < kMaxK) es->cand[etid] = es->outk[etid];
+                            have = 1;
+                            epi_bar(grp);
+                        }
                     }
-                    nk = have;
-                    // log-sum-exp pieces, folded in double
-                    double Cm = -INFINITY;
-                    uint32_t vm = 0;
-                    for (int cc = c_first + lane; cc <= c_last; cc += 32) {
-                        const int c_row0 = (int)(cta_start(cc, p.Q, G) / p.nq);
-                        const VpRecord* r = p.records + (size_t)cc * 2 + (sg.row == c_row0 ? 0 : 1);
-                        if (__ldcg(&r->nkeys) & 0x80000000u) rec_internal = 1;
-                        const float rc = __ldcg(&r->c);
-                        const uint32_t rv = __float_as_uint(__ldcg(&r->vmax));
-                        Cm = fmax(Cm, (double)rc);
-                        vm = vm > rv ? vm : rv;
-                    }
+                    if (ew == 0) {
+                        // log-sum-exp pieces, folded in double
+                        double Cm = (double)rc, S = 0.0;
+                        uint32_t vm = rv;
+                        for (int i = lane + 32; i < nseg; i += 32) {
+                            const VpRecord* r = record(i);
+                            const uint32_t kn = __ldcg(&r->nkeys), v2 = __float_as_uint(__ldcg(&r->vmax));
+                            have_all += (int)(kn & 0x7FFFFFFFu);
+                            rec_internal |= (int)(kn >> 31);
+                            Cm = fmax(Cm, (double)__ldcg(&r->c));
+                            vm = vm > v2 ? vm : v2;
+                        }
 #pragma unroll
-                    for (int d = 16; d > 0; d >>= 1) {
-                        Cm = fmax(Cm, __shfl_xor_sync(0xFFFFFFFFu, Cm, d));
-                        const uint32_t v2 = __shfl_xor_sync(0xFFFFFFFFu, vm, d);
-                        vm = vm > v2 ? vm : v2;
-                    }
-                    double S = 0.0;
-                    for (int cc = c_first + lane; cc <= c_last; cc += 32) {
-                        const int c_row0 = (int)(cta_start(cc, p.Q, G) / p.nq);
-                        const VpRecord* r = p.records + (size_t)cc * 2 + (sg.row == c_row0 ? 0 : 1);
-                        const float rc = __ldcg(&r->c), rs = __ldcg(&r->s);
-                        if (rc != -INFINITY)
-                            S += (double)rs * exp2((double)rc - Cm);
-                        else if (rs != rs)
-                            S += (double)rs;
-                    }
+                        for (int d = 16; d > 0; d >>= 1) Cm = fmax(Cm, __shfl_xor_sync(0xFFFFFFFFu, Cm, d));
+                        vm = __reduce_max_sync(0xFFFFFFFFu, vm);
+                        have_all = __reduce_add_sync(0xFFFFFFFFu, have_all);
+                        for (int i = lane; i < nseg; i += 32) {
+                            const float c2 = i < 32 ? rc : __ldcg(&record(i)->c), s2 = i < 32 ? rs : __ldcg(&record(i)->s);
+                            if (c2 != -INFINITY)
+                                S += (double)s2 * exp2((double)c2 - Cm);
+                            else if (s2 != s2)
+                                S += (double)s2;
+                        }
 #pragma unroll
-                    for (int d = 16; d > 0; d >>= 1) S += __shfl_xor_sync(0xFFFFFFFFu, S, d);
-                    rec_internal = __any_sync(0xFFFFFFFFu, rec_internal);
-                    Cd = Cm;
-                    Sd = S;
-                    Vm = vm;
-                    if (lane == 0) p.row_counter[sg.row] = 0;
+                        for (int d = 16; d > 0; d >>= 1) S += __shfl_xor_sync(0xFFFFFFFFu, S, d);
+                        rec_internal = __any_sync(0xFFFFFFFFu, rec_internal);
+                        nk = have_all < p.K ? have_all : p.K;
+                        Cd = Cm;
+                        Sd = S;
+                        Vm = vm;
+                        if (lane == 0) p.row_counter[sg.row] = 0;
+                    }
                 }
             }
+            if (ew != 0) continue;
             if (finish && p.partial_out != nullptr) {
                 graft_vocab_partial* po = p.partial_out + sg.row;
                 if (lane < kMaxK) po->keys[lane] = lane < nk ? es->outk[lane] : 0ull;
@@ -1303,6 +1330,10 @@ __global__ void __launch_bounds__(kVpThreads, 1) vocab_pass_kernel(const VpParam
 }
 
 // ---- vocabulary-parallel merge: one CTA of 128 threads per row ---------------------------------------------------
+// A latency chain (1024 rows of 8 shards are 2.3 MB): every load is issued at once, a key's rank is its place in its own
+// shard's descending list plus the places a binary search finds for it in the others (ranking all keys against each
+// other, 256 x 256 compares a row, and folding the log-sum-exp pieces one after the other took 19 us of 49), and the
+// pieces are folded by a lane each.
 constexpr int kMergeMaxShards = 64;
 struct MergeParams {
     const graft_vocab_partial* parts;  // [n_shards, rows]
@@ -1313,62 +1344,77 @@ struct MergeParams {
     float* lse;
     int32_t* row_status;
 };
-__global__ void __launch_bounds__(128) vocab_merge_kernel(const MergeParams p) {
-    __shared__ uint64_t cand[kMergeMaxShards * kMaxK];
+__global__ void __launch_bounds__(128) vocab_merge_kernel(const __grid_constant__ MergeParams p) {
+    extern __shared__ uint64_t merge_cand[];  // [n_shards][kMaxK]
     __shared__ uint64_t outk[kMaxK];
-    __shared__ double sC[kMergeMaxShards], sS[kMergeMaxShards];
-    __shared__ uint32_t sV[kMergeMaxShards], sN[kMergeMaxShards];
     const int row = blockIdx.x, tid = threadIdx.x, lane = tid & 31;
     const int n = p.n_shards * kMaxK;
+    pdl_launch_dependents();
+    pdl_wait();
+    // warp 0: the shards' pieces (two a lane: up to 64 shards)
+    double c2[2] = {-INFINITY, -INFINITY}, s2[2] = {0.0, 0.0};
+    uint32_t vm = 0u;
+    int have = 0, internal = 0;
+    if (tid < 32) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int i = lane + 32 * h;
+            if (i < p.n_shards) {
+                const graft_vocab_partial* r = p.parts + (size_t)i * p.rows + row;
+                c2[h] = r->c;
+                s2[h] = r->s;
+                const uint32_t v = r->vmax_ord, kn = r->nkeys;  // bit 31: a bounded wait ran out while the shard was scanned
+                vm = vm > v ? vm : v;
+                have += (int)(kn & 0x7FFFFFFFu);
+                internal |= (int)(kn >> 31);
+            }
+        }
+    }
     // the shards' keys with global token ids (an empty slot stays 0 and ranks below every key)
     for (int i = tid; i < n; i += 128) {
         const int sidx = i / kMaxK, kk = i % kMaxK;
         const graft_vocab_partial* r = p.parts + (size_t)sidx * p.rows + row;
-        uint64_t key = kk < (int)(r->nkeys & 0x7FFFFFFFu) ? r->keys[kk] : 0ull;
+        const uint32_t kn = r->nkeys;
+        uint64_t key = r->keys[kk];
+        if (kk >= (int)(kn & 0x7FFFFFFFu)) key = 0ull;
         if (key != 0ull) key = make_key(bits_from_ord((uint32_t)(key >> 32)), key_id(key) + (uint32_t)p.v_offset[sidx]);
-        cand[i] = key;
-    }
-    if (tid < p.n_shards) {
-        const graft_vocab_partial* r = p.parts + (size_t)tid * p.rows + row;
-        sC[tid] = r->c;
-        sS[tid] = r->s;
-        sV[tid] = r->vmax_ord;
-        sN[tid] = r->nkeys;  // bit 31: a bounded wait ran out while the shard was scanned
+        merge_cand[i] = key;
     }
     if (tid < kMaxK) outk[tid] = 0ull;
     __syncthreads();
-    // exact top-K by rank counting (keys are distinct: ids are)
     for (int i = tid; i < n; i += 128) {
-        const uint64_t key = cand[i];
-        if (key == 0ull) continue;
-        int rank = 0;
-        for (int j = 0; j < n; ++j) rank += cand[j] > key ? 1 : 0;
+        const uint64_t key = merge_cand[i];
+        int rank = i % kMaxK;
+        if (key == 0ull || rank >= p.K) continue;
+        for (int l = 0; l < n; l += kMaxK) {
+            if (l == i - i % kMaxK) continue;
+            int pos = 0;
+#pragma unroll
+            for (int step = kMaxK / 2; step >= 1; step >>= 1)
+                if (merge_cand[l + pos + step - 1] > key) pos += step;
+            rank += pos + (merge_cand[l + pos] > key ? 1 : 0);
+        }
         if (rank < p.K) outk[rank] = key;
     }
     __syncthreads();
     if (tid >= 32) return;
-    int have = 0;
-    bool internal = false;
-    for (int sidx = 0; sidx < p.n_shards; ++sidx) {
-        have += (int)(sN[sidx] & 0x7FFFFFFFu);
-        internal = internal || (sN[sidx] >> 31) != 0u;
+    double Cm = fmax(c2[0], c2[1]), S = 0.0;
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) Cm = fmax(Cm, __shfl_xor_sync(0xFFFFFFFFu, Cm, d));
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        if (c2[h] != -INFINITY)
+            S += s2[h] * exp2(c2[h] - Cm);
+        else if (s2[h] != s2[h])
+            S += s2[h];
     }
-    const int nk = have < p.K ? have : p.K;
-    double Cm = -INFINITY;
-    uint32_t vm = 0u;
-    for (int sidx = 0; sidx < p.n_shards; ++sidx) {
-        Cm = fmax(Cm, sC[sidx]);
-        vm = vm > sV[sidx] ? vm : sV[sidx];
-    }
-    double S = 0.0;
-    for (int sidx = 0; sidx < p.n_shards; ++sidx) {
-        if (sC[sidx] != -INFINITY)
-            S += sS[sidx] * exp2(sC[sidx] - Cm);
-        else if (sS[sidx] != sS[sidx])
-            S += sS[sidx];
-    }
-    vp_finalize(Cm, S, vm, nk, p.K, outk, lane, p.topk_id + (size_t)row * p.K, p.topk_lp + (size_t)row * p.K,
-                p.lse + row, p.row_status + row, internal);
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) S += __shfl_xor_sync(0xFFFFFFFFu, S, d);
+    vm = __reduce_max_sync(0xFFFFFFFFu, vm);
+    have = __reduce_add_sync(0xFFFFFFFFu, have);
+    internal = __any_sync(0xFFFFFFFFu, internal);
+    vp_finalize(Cm, S, vm, have < p.K ? have : p.K, p.K, outk, lane, p.topk_id + (size_t)row * p.K,
+                p.topk_lp + (size_t)row * p.K, p.lse + row, p.row_status + row, internal != 0);
 }
 
 }  // namespace
@@ -1454,9 +1500,9 @@ cudaError_t vp_merge_launch(graft_ctx* ctx, int batch, int n_shards, const graft
     p.topk_lp = d_topk_lp;
     p.lse = d_lse;
     p.row_status = d_row_status;
-    vocab_merge_kernel<<<p.rows, 128, 0, st>>>(p);
+    const cudaError_t e = launch_pdl(vocab_merge_kernel, dim3(p.rows), dim3(128), (size_t)n_shards * kMaxK * sizeof(uint64_t), st, p);
     ctx->launches += 1;
-    return cudaGetLastError();
+    return e != cudaSuccess ? e : cudaGetLastError();
 }
 int vp_merge_max_shards() { return kMergeMaxShards; }
 
