@@ -84,8 +84,8 @@ graft_status graft_create(const graft_config* cfg, graft_ctx** out) {
         cudaGetLastError();
         return GRAFT_ERR_CUDA;
     }
-    cudaDeviceProp prop;
-    if (cudaGetDeviceProperties(&prop, dev) != cudaSuccess) {
+    int num_sms = 0;  // (one attribute: cudaGetDeviceProperties takes milliseconds)
+    if (cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
         cudaGetLastError();
         return GRAFT_ERR_CUDA;
     }
@@ -94,7 +94,7 @@ graft_status graft_create(const graft_config* cfg, graft_ctx** out) {
     memset(ctx, 0, sizeof(*ctx));
     ctx->cfg = *cfg;
     ctx->device = dev;
-    ctx->num_sms = prop.multiProcessorCount;
+    ctx->num_sms = num_sms;
     ctx->nmax = cfg->budget_max + 1;
     ctx->mask_words = (ctx->nmax + 31) / 32;
     ctx->grid_pts = (cfg->budget_max - cfg->budget_min) / cfg->budget_step + 1;

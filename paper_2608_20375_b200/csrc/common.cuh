@@ -144,6 +144,12 @@ __device__ __forceinline__ float4 ldg_f4_keep(const float4* p, uint64_t policy) 
                  : "l"(p), "l"(policy));
     return v;
 }
+// releases what this thread (and, after a barrier, its CTA) wrote, acquires what earlier arrivals released
+__device__ __forceinline__ int atom_add_acq_rel(int* p, int v) {
+    int old;
+    asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(v) : "memory");
+    return old;
+}
 // named barrier among a subset of the CTA's warps
 __device__ __forceinline__ void named_bar_sync(int id, int nthreads) {
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");

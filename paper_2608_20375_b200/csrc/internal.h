@@ -14,11 +14,9 @@ constexpr int kMaxCostPts = 16;
 // ---- vocab pass -----------------------------------------------------------------------------
 constexpr int kVpConsumerWarps = 16;                 // streaming warps (one CTA per SM)
 constexpr int kVpConsumers = kVpConsumerWarps * 32;  // 512
-constexpr int kVpEpiThreads = 128;                   // four warps per epilogue group
-constexpr int kVpEpiGroups = 2;                      // the groups take alternate segments
-constexpr int kVpBufs = 4;                           // hand-over buffers between streaming and epilogue warps
+constexpr int kVpEpiWarps = 8;                       // epilogue warps: two groups of four or four groups of two
 constexpr int kVpGroups = 64;   // groups of streaming threads whose maxima bound the K-th largest element (>= kMaxK)
-constexpr int kVpThreads = kVpConsumers + kVpEpiGroups * kVpEpiThreads + 64;  // + one producer warp + one cosine warp
+constexpr int kVpThreads = kVpConsumers + kVpEpiWarps * 32 + 64;  // + one producer warp + one cosine warp
 constexpr int kVpTileBytes = 32768;                  // one ring stage (2 KiB per streaming warp)
 constexpr int kVpQuantum = 2048;                     // elements; granularity of the work partition
 constexpr int kVpCandCap = 1280;                     // candidate keys held in shared memory (K chunks of 32 elements and their ties)
@@ -36,6 +34,8 @@ struct VpRecord {
 
 struct VpPlan {
     int grid;            // CTAs launched
+    int whole;           // every CTA gets whole rows
+    int groups;          // epilogue groups (2 or 4)
     int stages;          // ring depth
     int max_seg_tiles;   // tiles in the longest segment a CTA can get
     size_t smem_bytes;

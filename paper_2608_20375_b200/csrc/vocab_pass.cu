@@ -3,12 +3,13 @@
 // (Preliminaries, "DFlash one-pass marginals": q_{t,d} and c^{(r)}_{t,d}; Eq. 3's log q).
 //
 // Shape of the kernel (sm_100a):
-//   * persistent grid, one CTA per SM; the rows*V element stream is cut into equal contiguous shares,
-//     one per CTA, so a CTA sees at most two partial rows plus whole rows in between ("segments");
+//   * persistent grid, one CTA per SM at most; a CTA gets whole rows where that comes out even enough, else the
+//     rows*V element stream is cut into equal contiguous shares, so a CTA sees at most two partial rows plus whole
+//     rows in between ("segments"; vp_make_plan has the rule);
 //   * warp roles: one producer warp feeds a four-stage shared-memory ring with 32 KiB TMA bulk copies
 //     (cp.async.bulk + mbarrier complete_tx); sixteen streaming warps read the ring with 16-byte shared loads;
-//     two epilogue groups of four warps finish alternate segments while the streaming warps are already in
-//     later ones; one warp computes the adjacent-position cosines of the SABA state (Eq. 15) beside the stream;
+//     two epilogue groups of four warps (four of two for many short rows) finish segments in turn while the
+//     streaming warps are already in later ones; one warp computes the adjacent-position cosines of the SABA state (Eq. 15) beside the stream;
 //   * per 32-element chunk a streaming lane takes a packed max (stored for the second stage, 2 bytes per
 //     chunk), keeps a lazily rescaled reference exponent and adds 2^(z log2e - ref) with ex2.approx;
 //   * top-K needs no per-element work in the stream: after the segment, the K-th largest of 64 group maxima
@@ -42,7 +43,7 @@ namespace {
 
 constexpr int NW = kVpConsumerWarps;          // streaming warps
 constexpr int NT = kVpConsumers;              // streaming threads
-constexpr int PROD_WARP = NW + kVpEpiGroups * kVpEpiThreads / 32;  // warp index of the producer warp
+constexpr int PROD_WARP = NW + kVpEpiWarps;  // warp index of the producer warp
 constexpr int TILE = kVpTileBytes;
 constexpr int WBLK = TILE / NW;               // bytes of a tile owned by one warp (2048)
 static_assert(WBLK == 2048, "one warp owns 2 KiB of every tile");
@@ -52,8 +53,18 @@ static_assert(WBLK == 32 * 4 * 16, "the exact fall-back selection reads one warp
 constexpr uint32_t kOrdNegInf = 0x007FFFFFu;  // ord_from_bits of -inf: every finite value maps above it
 constexpr uint32_t kVpIdleHintNs = 10000;  // suspend hint of the waits of the producer and epilogue warps
 constexpr int COS_WARP = PROD_WARP + 1;  // warp that computes the SABA cosines beside the stream
-static_assert(kVpThreads == NT + kVpEpiGroups * kVpEpiThreads + 64,
+static_assert(kVpThreads == NT + kVpEpiWarps * 32 + 64,
               "thread count = streaming warps + epilogue warps + producer warp + cosine warp");
+
+// The eight epilogue warps work as GROUPS groups, each on a segment of its own (segments in turn).  An epilogue is a chain
+// of latencies (8k cycles alone, 10k beside the stream; 20 % more with two warps instead of four), so a CTA whose
+// segments stream faster than two groups finish them is served better by four.
+template <int GROUPS>
+struct Epi {
+    static constexpr int THREADS = kVpEpiWarps * 32 / GROUPS;
+    static constexpr int BUFS = 2 * GROUPS;  // hand-over buffers between streaming and epilogue warps
+};
+constexpr int kVpMaxBufs = 8;
 
 template <bool BF16>
 struct VT;
@@ -400,15 +411,17 @@ struct __align__(16) EpiShared {  // private to one epilogue group
                     // plus the first elements equal to T
     uint32_t Tv;
 };
+template <int GROUPS>
 struct __align__(16) VpShared {
-    EpiShared epi[kVpEpiGroups];
-    uint32_t tmax[kVpBufs][NT];  // per-thread maxima of a finished segment, one buffer per segment in flight
-    uint32_t gmax[kVpBufs][kVpGroups];  // the same maxima folded into 64 groups (lane, warp parity); zero when idle
-    float wc[kVpBufs][NW], ws[kVpBufs][NW];
+    EpiShared epi[GROUPS];
+    uint32_t tmax[Epi<GROUPS>::BUFS][NT];  // per-thread maxima of a finished segment, one buffer per segment in flight
+    uint32_t gmax[Epi<GROUPS>::BUFS][kVpGroups];  // the same maxima folded into 64 groups (lane, warp parity); zero when idle
+    float wc[Epi<GROUPS>::BUFS][NW], ws[Epi<GROUPS>::BUFS][NW];
     volatile int abort_flag;
 };
 
-__device__ __forceinline__ void epi_bar(int group) { named_bar_sync(2 + group, kVpEpiThreads); }
+template <int ET>  // threads of a group
+__device__ __forceinline__ void epi_bar(int group) { named_bar_sync(2 + group, ET); }
 
 // ---- epilogue-warp helpers (32 threads, warp-synchronous) ----------------------------------------------
 // Append `key` for the lanes with pred set; returns the new count.  Entries beyond the capacity are dropped
@@ -445,8 +458,9 @@ __device__ void warp_select_topk(EpiShared* sh, int n, int K, int lane) {
 }
 
 // The K-th largest chunk maximum of a segment (every streaming thread leaves one 16-bit maximum per tile), as a 16-bit
-// order-preserving pattern; 0 when the segment has fewer than K chunks.  All 128 threads of an epilogue group; two
+// order-preserving pattern; 0 when the segment has fewer than K chunks.  All threads of an epilogue group; two
 // histogram passes of eight bits each over the idle hit list.  Out of line: rows that need it are rare.
+template <int ET>
 __device__ __noinline__ uint32_t epi_kth_chunk_max(EpiShared* es, const uint16_t* cmx, int max_tiles, int ntiles, int K,
                                                    int etid, int grp) {
     uint32_t* hist = es->hits;  // [0, 256) counts, [256] the bin found, [257] the count above it
@@ -454,10 +468,10 @@ __device__ __noinline__ uint32_t epi_kth_chunk_max(EpiShared* es, const uint16_t
     int want = K;
 #pragma unroll 1
     for (int pass = 0; pass < 2; ++pass) {
-        for (int i = etid; i < 258; i += kVpEpiThreads) hist[i] = 0u;
-        epi_bar(grp);
+        for (int i = etid; i < 258; i += ET) hist[i] = 0u;
+        epi_bar<ET>(grp);
 #pragma unroll 1
-        for (int t = etid; t < NT; t += kVpEpiThreads) {
+        for (int t = etid; t < NT; t += ET) {
             const uint16_t* row = cmx + (size_t)t * max_tiles;
 #pragma unroll 1
             for (int tile = 0; tile < ntiles; ++tile) {
@@ -468,7 +482,7 @@ __device__ __noinline__ uint32_t epi_kth_chunk_max(EpiShared* es, const uint16_t
                     atomicAdd(&hist[v & 255u], 1u);
             }
         }
-        epi_bar(grp);
+        epi_bar<ET>(grp);
         if (etid < 32) {  // the bin in which the count from the top reaches `want`: eight bins a lane
             uint32_t own = 0u;
 #pragma unroll
@@ -492,7 +506,7 @@ __device__ __noinline__ uint32_t epi_kth_chunk_max(EpiShared* es, const uint16_t
                 }
             }
         }
-        epi_bar(grp);
+        epi_bar<ET>(grp);
         const uint32_t bin = hist[256];
         if (bin == 0u) {  // fewer than K chunks (uniform)
             prefix = 0u;
@@ -501,7 +515,7 @@ __device__ __noinline__ uint32_t epi_kth_chunk_max(EpiShared* es, const uint16_t
             prefix = (prefix << 8) | (bin & 255u);
             want -= (int)hist[257];
         }
-        epi_bar(grp);  // (read before the next pass clears it)
+        epi_bar<ET>(grp);  // (read before the next pass clears it)
     }
     return prefix;
 }
@@ -510,14 +524,15 @@ __device__ __noinline__ uint32_t epi_kth_chunk_max(EpiShared* es, const uint16_t
 // K-th largest key is found by a search over its bits, two at a time with three counts each -- over the value word
 // first; over the id word, among the keys of that value, only if more keys share the K-th largest value than are
 // wanted -- and the K keys that reach it (keys are distinct: exactly K) are ranked into outk.  Whatever the keys'
-// order or values.  All 128 threads of an epilogue group; the counts of its warps meet in the idle hit list.  Out of
+// order or values.  All threads of an epilogue group; the counts of its warps meet in the idle hit list.  Out of
 // line: rows that need it are rare.
+template <int ET>
 __device__ __noinline__ void epi_select_many(EpiShared* es, int n, int K, int etid, int grp) {
     uint32_t* cnt = es->hits;                       // [2 * 16 * 3] counts of the steps, [96], [97] above / at the value, [98] kept
     uint64_t* kept = (uint64_t*)(es->hits + 128);   // [K] the keys that reach the K-th largest
     const uint32_t* word = (const uint32_t*)es->cand;  // key i: id word at 2 i, value word at 2 i + 1
-    for (int i = etid; i < 99; i += kVpEpiThreads) cnt[i] = 0u;
-    epi_bar(grp);
+    for (int i = etid; i < 99; i += ET) cnt[i] = 0u;
+    epi_bar<ET>(grp);
     uint32_t vk = 0u, ik = 0u;  // the K-th largest key's value word and id word
     int want = K;
 #pragma unroll 1
@@ -529,7 +544,7 @@ __device__ __noinline__ void epi_select_many(EpiShared* es, int n, int K, int et
             const uint32_t t1 = kth | (1u << bit), t2 = kth | (2u << bit), t3 = kth | (3u << bit);
             int c1 = 0, c2 = 0, c3 = 0;
 #pragma unroll 2
-            for (int i = etid; i < n; i += kVpEpiThreads) {
+            for (int i = etid; i < n; i += ET) {
                 const uint32_t hi = word[2 * i + 1];
                 const uint32_t x = phase == 0 ? hi : (hi == vk ? word[2 * i] : 0u);  // (an id word is never 0)
                 c1 += (x >= t1) ? 1 : 0;
@@ -545,7 +560,7 @@ __device__ __noinline__ void epi_select_many(EpiShared* es, int n, int K, int et
                 atomicAdd(&slot[1], (uint32_t)c2);
                 atomicAdd(&slot[2], (uint32_t)c3);
             }
-            epi_bar(grp);
+            epi_bar<ET>(grp);
             const int n1 = (int)slot[0], n2 = (int)slot[1], n3 = (int)slot[2];
             kth = n3 >= want ? t3 : (n2 >= want ? t2 : (n1 >= want ? t1 : kth));
         }
@@ -555,7 +570,7 @@ __device__ __noinline__ void epi_select_many(EpiShared* es, int n, int K, int et
         }
         vk = kth;
         int above = 0, at = 0;
-        for (int i = etid; i < n; i += kVpEpiThreads) {
+        for (int i = etid; i < n; i += ET) {
             const uint32_t hi = word[2 * i + 1];
             above += (hi > vk) ? 1 : 0;
             at += (hi == vk) ? 1 : 0;
@@ -566,19 +581,19 @@ __device__ __noinline__ void epi_select_many(EpiShared* es, int n, int K, int et
             atomicAdd(&cnt[96], (uint32_t)above);
             atomicAdd(&cnt[97], (uint32_t)at);
         }
-        epi_bar(grp);
+        epi_bar<ET>(grp);
         want = K - (int)cnt[96];
         if ((int)cnt[97] == want) break;  // (uniform) every key of that value is wanted: ik = 0 lets them all through
     }
     const uint64_t kth_key = ((uint64_t)vk << 32) | ik;
-    for (int i = etid; i < n; i += kVpEpiThreads) {
+    for (int i = etid; i < n; i += ET) {
         const uint64_t k = es->cand[i];
         if (k >= kth_key) {
             const uint32_t pos = atomicAdd(&cnt[98], 1u);
             if (pos < (uint32_t)kMaxK) kept[pos] = k;
         }
     }
-    epi_bar(grp);
+    epi_bar<ET>(grp);
     const int m = (int)cnt[98] < K ? (int)cnt[98] : K;
     if (etid < m) {
         const uint64_t k = kept[etid];
@@ -703,36 +718,37 @@ __device__ __forceinline__ void vp_finalize(double Cd, double Sd, uint32_t Vm, i
     }
 }
 
-template <bool BF16>
+template <bool BF16, int GROUPS>
 __global__ void __launch_bounds__(kVpThreads, 1) vocab_pass_kernel(const VpParams p) {
     using T = VT<BF16>;
     using cm_t = typename T::cm_t;
+    constexpr int ET = Epi<GROUPS>::THREADS, BUFS = Epi<GROUPS>::BUFS;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     pdl_launch_dependents();  // the edge-score kernel's CTAs may move in as this grid's CTAs leave; they wait for it
     unsigned char* ring = smem_raw;
-    uint64_t* bars = (uint64_t*)(ring + (size_t)p.stages * TILE);  // full[8], empty[8], ready[4], done[4]
-    VpShared* sh = (VpShared*)(bars + 24);
-    cm_t* cmax = (cm_t*)(sh + 1);  // [kVpBufs][n_cmax]
+    uint64_t* bars = (uint64_t*)(ring + (size_t)p.stages * TILE);  // full[8], empty[8], ready[8], done[8]
+    VpShared<GROUPS>* sh = (VpShared<GROUPS>*)(bars + 16 + 2 * kVpMaxBufs);
+    cm_t* cmax = (cm_t*)(sh + 1);  // [BUFS][n_cmax]
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const long long G = gridDim.x;
     const long long q0 = cta_start(blockIdx.x, p.Q, G), q1 = cta_start(blockIdx.x + 1, p.Q, G);
     const uint32_t full0 = smem_u32(bars), empty0 = smem_u32(bars + 8);
-    const uint32_t ready0 = smem_u32(bars + 16), done0 = smem_u32(bars + 20);
+    const uint32_t ready0 = smem_u32(bars + 16), done0 = smem_u32(bars + 16 + kVpMaxBufs);
 
     if (tid == 0) {
         for (int s = 0; s < p.stages; ++s) {
             mbar_init(full0 + 8 * s, 1);
             mbar_init(empty0 + 8 * s, NW);
         }
-        for (int s = 0; s < kVpBufs; ++s) {
+        for (int s = 0; s < BUFS; ++s) {
             mbar_init(ready0 + 8 * s, NW);
             mbar_init(done0 + 8 * s, 1);
         }
         mbar_fence_init();
         sh->abort_flag = 0;
     }
-    if (tid < kVpBufs * kVpGroups) (&sh->gmax[0][0])[tid] = 0u;
+    if (tid < BUFS * kVpGroups) (&sh->gmax[0][0])[tid] = 0u;
     __syncthreads();
     // Launched with programmatic stream serialization inside a round: the CTA is set up while the kernel ahead of it in
     // the stream (the previous round's walk or tree kernel) drains; nothing is read or written before that kernel has
@@ -794,15 +810,15 @@ __global__ void __launch_bounds__(kVpThreads, 1) vocab_pass_kernel(const VpParam
         // ------------------------------ streaming warps ------------------------------------------
         uint32_t st = 0, ph = 0;  // ring position and parity of the "full" phase to wait for
         const uint32_t nst = (uint32_t)p.stages;
-        uint32_t k = 0;           // segment counter: hand-over buffers are indexed by k % kVpBufs
+        uint32_t k = 0;           // segment counter: hand-over buffers are indexed by k % BUFS
         SegIter it = seg_iter_begin<BF16>(p, q0, q1);
         Seg sg;
         for (; seg_iter_next<BF16>(p, it, sg); ++k) {
-            const uint32_t pb = k % kVpBufs;
+            const uint32_t pb = k % BUFS;
             Acc a;
             acc_init<BF16>(a);
-            // buffer pb is free once the epilogue of segment k - kVpBufs is done
-            if (k >= kVpBufs) mbar_wait_bounded(done0 + 8 * pb, ((k / kVpBufs) - 1u) & 1u, &sh->abort_flag);
+            // buffer pb is free once the epilogue of segment k - BUFS is done
+            if (k >= BUFS) mbar_wait_bounded(done0 + 8 * pb, ((k / BUFS) - 1u) & 1u, &sh->abort_flag);
             {
                 const int nfull = (int)(sg.body_bytes / TILE);
                 cm_t* slot = cmax + (size_t)pb * p.n_cmax + (size_t)tid * p.max_tiles;  // this thread's slots, by tile
@@ -860,22 +876,23 @@ __global__ void __launch_bounds__(kVpThreads, 1) vocab_pass_kernel(const VpParam
             }
         }
     } else {
-        // ------------------------------ epilogue groups (four warps each) ------------------------
-        // Group g finishes the segments with k % 2 == g, so a group has two segment times for one epilogue.
+        // ------------------------------ epilogue groups ----------------------------------------
+        // Group g finishes the segments with k % GROUPS == g, so a group has GROUPS segment times for one epilogue.
         // Warp 0 of a group owns the hand-over barriers and the sequential parts; the data-parallel parts (which
-        // chunks reach T, re-reading them, ranking the candidates) are shared by the group's 128 threads.
-        const int grp = (warp - NW) / (kVpEpiThreads / 32), ew = (warp - NW) % (kVpEpiThreads / 32);
-        const int etid = (tid - NT) % kVpEpiThreads;
+        // chunks reach T, re-reading them, ranking the candidates) are shared by the group's threads.
+        const int grp = (warp - NW) / (ET / 32), ew = (warp - NW) % (ET / 32);
+        const int etid = (tid - NT) % ET;
         EpiShared* const es = &sh->epi[grp];
         uint32_t k = 0;
         SegIter it = seg_iter_begin<BF16>(p, q0, q1);
+        const int my_first_row = it.r_first;
         Seg sg;
         for (; seg_iter_next<BF16>(p, it, sg); ++k) {
-            if ((int)(k % kVpEpiGroups) != grp) continue;
-            const uint32_t pb = k % kVpBufs;
+            if ((int)(k % GROUPS) != grp) continue;
+            const uint32_t pb = k % BUFS;
             const char* rowp = p.logits + (size_t)sg.row * p.V * T::ESZ;
             const cm_t* cmx = cmax + (size_t)pb * p.n_cmax;
-            if (ew == 0) mbar_wait_bounded_hint(ready0 + 8 * pb, (k / kVpBufs) & 1u, &sh->abort_flag, kVpIdleHintNs);
+            if (ew == 0) mbar_wait_bounded_hint(ready0 + 8 * pb, (k / BUFS) & 1u, &sh->abort_flag, kVpIdleHintNs);
             float c = -INFINITY, s = 0.f;
             uint32_t vmo = 0;
             if (ew == 0) {
@@ -974,16 +991,16 @@ __global__ void __launch_bounds__(kVpThreads, 1) vocab_pass_kernel(const VpParam
                     es->tie_groups = tie_groups;
                 }
             }
-            epi_bar(grp);
+            epi_bar<ET>(grp);
             uint32_t Tv = es->Tv;
             // (d) chunks whose stored maximum reaches T: only threads whose own maximum reaches T can have one.
             //     List positions come from shared-memory atomics (the order does not matter: the final selection
             //     ranks exact keys).  A hit is recorded as the byte offset of the chunk's first vector.
-            for (int t = etid; t < NT; t += kVpEpiThreads) {
+            for (int t = etid; t < NT; t += ET) {
                 const uint32_t x = sh->tmax[pb][t];
                 if (x >= Tv && x != 0u) es->hthreads[atomicAdd(&es->nht, 1)] = (uint16_t)t;
             }
-            epi_bar(grp);
+            epi_bar<ET>(grp);
             // Te: what a chunk's maximum (and, below, an element) must reach.  T itself at first.  If more chunks reach T
             // than the list holds, either thousands of elements tie with T (a flat rest under a few winners: most of the
             // 64 group maxima are T itself) or T is a poor bound (the groups of threads are a partition that a pattern in
@@ -1001,11 +1018,11 @@ __global__ void __launch_bounds__(kVpThreads, 1) vocab_pass_kernel(const VpParam
                 const uint32_t magic = sg.ntiles > 1 ? 0xFFFFFFFFu / (uint32_t)sg.ntiles + 1u : 0u;  // ceil(2^32 / ntiles)
                 constexpr int PU = 4;
                 bool stop = false;
-                for (int base = 0; base < npairs && !stop; base += kVpEpiThreads * PU) {
+                for (int base = 0; base < npairs && !stop; base += ET * PU) {
                     uint32_t raw[PU], off[PU];
 #pragma unroll
                     for (int u = 0; u < PU; ++u) {
-                        const int idx = base + u * kVpEpiThreads + etid;
+                        const int idx = base + u * ET + etid;
                         raw[u] = 0u;
                         off[u] = 0u;
                         if (idx < npairs) {
@@ -1017,7 +1034,7 @@ __global__ void __launch_bounds__(kVpThreads, 1) vocab_pass_kernel(const VpParam
                     }
 #pragma unroll
                     for (int u = 0; u < PU; ++u) {
-                        if (ord_from_bits(raw[u] << 16) >= Te && base + u * kVpEpiThreads + etid < npairs && !stop) {
+                        if (ord_from_bits(raw[u] << 16) >= Te && base + u * ET + etid < npairs && !stop) {
                             const int pos = atomicAdd(&es->nhits, 1);
                             if (pos >= kVpHitCap)
                                 stop = true;  // too many: the exact selection over the segment takes over
@@ -1026,15 +1043,15 @@ __global__ void __launch_bounds__(kVpThreads, 1) vocab_pass_kernel(const VpParam
                         }
                     }
                 }
-                epi_bar(grp);
+                epi_bar<ET>(grp);
                 // (a list several times as long as a good bound leaves it -- about K chunks -- also says that T is poor:
                 // its chunks would overflow the key buffer)
                 const bool over = es->nhits > kVpHitCap;
                 if (es->fill_ninf || (refined && tied)) break;  // (uniform)
                 if (!over && !(pass == 0 && es->nhits > 5 * p.K && es->tie_groups < 16)) break;  // (uniform)
-                epi_bar(grp);  // (everybody has read the count)
+                epi_bar<ET>(grp);  // (everybody has read the count)
                 if (!refined && (tied || !BF16 || es->tie_groups < 16)) {
-                    uint32_t kth = epi_kth_chunk_max(es, cmx, p.max_tiles, sg.ntiles, p.K, etid, grp);
+                    uint32_t kth = epi_kth_chunk_max<ET>(es, cmx, p.max_tiles, sg.ntiles, p.K, etid, grp);
                     // (fp32 logits: the stored maxima are rounded up to bf16, the pattern below is a bound)
                     if (!BF16 && kth > 0u) kth -= 1u;
                     refined = true;
@@ -1047,7 +1064,7 @@ __global__ void __launch_bounds__(kVpThreads, 1) vocab_pass_kernel(const VpParam
                             es->fill_tie = 0;
                             es->Tv = Tv;
                         }
-                        epi_bar(grp);
+                        epi_bar<ET>(grp);
                         continue;
                     }
                     if (tied) break;  // (no better bound and what lies above T overflows the list: the exact selection)
@@ -1059,7 +1076,7 @@ __global__ void __launch_bounds__(kVpThreads, 1) vocab_pass_kernel(const VpParam
                     es->fill_tie = 1;
                 }
                 Te = Tv + 0x10000u;  // (the next bf16 value up, whatever the sign: T holds the value's upper 16 bits)
-                epi_bar(grp);
+                epi_bar<ET>(grp);
             }
             // (e) the 16-byte vectors of the hit chunks, re-read from global memory; elements >= T become keys.
             //     A thread issues its loads of a round before it uses any: under a saturated memory system one
@@ -1070,15 +1087,15 @@ __global__ void __launch_bounds__(kVpThreads, 1) vocab_pass_kernel(const VpParam
                 const bool hit_ovf = es->nhits > kVpHitCap;
                 const int nhits = hit_ovf ? 0 : es->nhits;
                 if (etid == 0 && hit_ovf) es->ovf = 1;
-                constexpr int RU = 2;
+                constexpr int RU = 256 / ET;
                 const int nvec = nhits * VEC_PER_LANE;
                 bool full = false;
-                for (int base = 0; base < nvec && !full; base += kVpEpiThreads * RU) {
+                for (int base = 0; base < nvec && !full; base += ET * RU) {
                     uint4 vv[RU];
                     uint32_t offs[RU];
 #pragma unroll
                     for (int u = 0; u < RU; ++u) {
-                        const int i = base + u * kVpEpiThreads + etid;
+                        const int i = base + u * ET + etid;
                         vv[u] = make_uint4(T::NEG_INF_WORD, T::NEG_INF_WORD, T::NEG_INF_WORD, T::NEG_INF_WORD);
                         offs[u] = 0xFFFFFFFFu;
                         if (i < nvec) {
@@ -1113,7 +1130,7 @@ __global__ void __launch_bounds__(kVpThreads, 1) vocab_pass_kernel(const VpParam
                     }
                 }
             }
-            epi_bar(grp);
+            epi_bar<ET>(grp);
             if (es->fill_ninf || es->fill_tie) {  // (uniform)
                 if (ew == 0) {
                     // The first K elements equal to -inf (or, for bulk ties, to T) of the segment's body in id order (the
@@ -1158,7 +1175,7 @@ __global__ void __launch_bounds__(kVpThreads, 1) vocab_pass_kernel(const VpParam
                     }
                     if (gave_up && lane == 0) es->ovf = 1;
                 }
-                epi_bar(grp);
+                epi_bar<ET>(grp);
             }
             // (f) exact top-K of the candidates by rank counting (keys are distinct, so ranks are a permutation)
             // (ranking n candidates costs n^2 compares shared by 128 threads: beyond 256 -- rows whose large elements sit
@@ -1169,7 +1186,7 @@ __global__ void __launch_bounds__(kVpThreads, 1) vocab_pass_kernel(const VpParam
             int nk = ncand < p.K ? ncand : p.K;
             if (!overflow) {
                 // two neighbouring lanes per candidate, each over every other key, two running counts each
-                for (int i0 = 0; i0 < ncand; i0 += kVpEpiThreads / 2) {
+                for (int i0 = 0; i0 < ncand; i0 += ET / 2) {
                     const int i = i0 + (etid >> 1);
                     const uint64_t key = i < ncand ? es->cand[i] : ~0ull;
                     int r0 = 0, r1 = 0;
@@ -1182,14 +1199,14 @@ __global__ void __launch_bounds__(kVpThreads, 1) vocab_pass_kernel(const VpParam
                     if (i < ncand && (etid & 1) == 0 && rank < p.K) es->outk[rank] = key;
                 }
             } else if (es->ovf == 0 && es->ncand <= kVpCandCap) {  // (uniform; every candidate is in the buffer)
-                epi_select_many(es, ncand, p.K, etid, grp);
+                epi_select_many<ET>(es, ncand, p.K, etid, grp);
             } else if (ew == 0) {
                 // (T is a lower bound of the K-th largest element: the filter starts there, not at nothing -- a row sorted
                 // in ascending order would otherwise send every element through the buffer; with the threshold moved up
                 // from -inf, elements equal to -inf may be among the K best and nothing is ruled out)
                 nk = warp_fallback_select<BF16>(es, p, sg, cmx, lane, es->fill_ninf ? 0ull : ((uint64_t)Tv << 32) - 1ull);
             }
-            epi_bar(grp);
+            epi_bar<ET>(grp);
             // the double-buffered arrays of parity pb may be reused from here on
             if (ew == 0) {
                 __syncwarp();
@@ -1205,7 +1222,6 @@ __global__ void __launch_bounds__(kVpThreads, 1) vocab_pass_kernel(const VpParam
             if (!whole_row) {
                 const long long x0 = (long long)sg.row * p.nq;
                 const int c_first = cta_of(x0, p.Q, G), nseg = cta_of(x0 + p.nq - 1, p.Q, G) - c_first + 1;
-                const int my_first_row = (int)(q0 / p.nq);
                 if (ew == 0) {
                     VpRecord* rec = p.records + (size_t)blockIdx.x * 2 + (sg.row == my_first_row ? 0 : 1);
                     if (lane < kMaxK) rec->keys[lane] = lane < nk ? es->outk[lane] : 0ull;
@@ -1215,17 +1231,13 @@ __global__ void __launch_bounds__(kVpThreads, 1) vocab_pass_kernel(const VpParam
                         rec->vmax = __uint_as_float(vmo);
                         rec->nkeys = (uint32_t)nk | (sh->abort_flag ? 0x80000000u : 0u);
                     }
-                    __threadfence();
                     __syncwarp();
-                    if (lane == 0) {
-                        es->arrived = nseg == 1 ? 0 : atomicAdd(p.row_counter + sg.row, 1);
-                        __threadfence();
-                    }
+                    if (lane == 0) es->arrived = atom_add_acq_rel(p.row_counter + sg.row, 1);  // (the lanes' stores included)
                 }
-                epi_bar(grp);
+                epi_bar<ET>(grp);
                 if (es->arrived == nseg - 1) {  // (uniform)
                     finish = true;
-                    // Merge the records of the row's CTAs, the group's 128 threads together.  Every CTA after the first
+                    // Merge the records of the row's CTAs, the group's threads together.  Every CTA after the first
                     // starts inside the row, so the row is its first and its record the first of its two; every record's
                     // keys are in descending order (empty ones, 0, last): a key's rank is its place in its own record plus
                     // the places that a binary search finds for it in the others.  (One warp that ranked all keys against
@@ -1249,11 +1261,11 @@ __global__ void __launch_bounds__(kVpThreads, 1) vocab_pass_kernel(const VpParam
                     int have = 0;                                   // lists of kMaxK keys carried over: 0 or 1
                     for (int r0 = 0; r0 < nseg; r0 += kRound) {
                         const int cnt = nseg - r0 < kRound ? nseg - r0 : kRound, n = (have + cnt) * kMaxK;
-                        for (int i = etid; i < cnt * kMaxK; i += kVpEpiThreads)
+                        for (int i = etid; i < cnt * kMaxK; i += ET)
                             es->cand[have * kMaxK + i] = __ldcg((const unsigned long long*)&record(r0 + i / kMaxK)->keys[i % kMaxK]);
                         if (etid < kMaxK) es->outk[etid] = 0ull;
-                        epi_bar(grp);
-                        for (int i = etid; i < n; i += kVpEpiThreads) {
+                        epi_bar<ET>(grp);
+                        for (int i = etid; i < n; i += ET) {
                             const uint64_t key = es->cand[i];
                             int rank = i % kMaxK;
                             for (int l = 0; l < n; l += kMaxK) {
@@ -1266,11 +1278,11 @@ __global__ void __launch_bounds__(kVpThreads, 1) vocab_pass_kernel(const VpParam
                             }
                             if (key != 0ull && rank < p.K) es->outk[rank] = key;
                         }
-                        epi_bar(grp);
+                        epi_bar<ET>(grp);
                         if (r0 + kRound < nseg) {  // (uniform)
                             if (etid < kMaxK) es->cand[etid] = es->outk[etid];
                             have = 1;
-                            epi_bar(grp);
+                            epi_bar<ET>(grp);
                         }
                     }
                     if (ew == 0) {
@@ -1420,34 +1432,57 @@ __global__ void __launch_bounds__(128) vocab_merge_kernel(const __grid_constant_
 }  // namespace
 
 // ---- host side ----------------------------------------------------------------------------------
-static size_t vp_smem_bytes(int stages, int n_cmax) {
-    return (size_t)stages * TILE + 24 * sizeof(uint64_t) + sizeof(VpShared) + (size_t)kVpBufs * n_cmax * 2 + 16;
+static void (*vp_kernel(bool bf16, int groups))(const VpParams) {
+    if (groups == 4) return bf16 ? vocab_pass_kernel<true, 4> : vocab_pass_kernel<false, 4>;
+    return bf16 ? vocab_pass_kernel<true, 2> : vocab_pass_kernel<false, 2>;
+}
+static size_t vp_smem_bytes(int groups, int stages, int n_cmax) {
+    const size_t sh = groups == 4 ? sizeof(VpShared<4>) : sizeof(VpShared<2>);
+    return (size_t)stages * TILE + (16 + 2 * kVpMaxBufs) * sizeof(uint64_t) + sh + (size_t)2 * groups * n_cmax * 2 + 16;
 }
 
 VpPlan vp_make_plan(const graft_config& cfg, int num_sms, int batch) {
     VpPlan pl;
     const bool bf16 = cfg.logits_dtype == GRAFT_BF16;
-    const int esz = bf16 ? 2 : 4;
+    const long long esz = bf16 ? 2 : 4, rows = (long long)batch * cfg.L, row_bytes = (long long)cfg.V * esz;
     const long long nq = cfg.V / kVpQuantum > 0 ? cfg.V / kVpQuantum : 1;
-    const long long Q = nq * (long long)batch * cfg.L;
-    long long G = (long long)num_sms;  // one CTA per SM
-    // small inputs: a CTA's share is at least 64 KiB, so that a row is not cut into more pieces than its merge is
-    // worth (at batch 1 a 128 KB row over nine CTAs spent 14 us merging nine records per row)
-    const long long min_share_q = (64 * 1024) / ((long long)kVpQuantum * esz);
-    if (G > Q / min_share_q) G = Q / min_share_q;
-    if (G > Q) G = Q;
-    if (G < 1) G = 1;
+    long long G, share_q, per = 0;  // CTAs (one per SM at most), a CTA's share at most, whole rows of a CTA at most
+    // A row that no other CTA has a piece of needs no merge, which is what a small input waits for (a record and a merge
+    // take 5 to 6 us, the stream of a 64 KB row 1.4 us): whole rows wherever the CTAs' shares come out even enough.  Measured
+    // on 148 SMs, one launch after the other, bf16, L = 16.
+    if (rows < num_sms) {
+        // n pieces of each row, n = 1 unless the stream gets shorter by more than the merge costs (190 KB): V = 151,936
+        // batch 1: n = 1 18.5 us, n = 2 18.6, n = 4 17.1, n = 9 20.9; batch 4: n = 1 18.9, n = 2 19.7
+        long long n = row_bytes / (76 * 1024);
+        if (n > num_sms / rows) n = num_sms / rows;
+        if (n > nq) n = nq;
+        if (n < 1 || row_bytes - row_bytes / n < 190 * 1024) n = 1;
+        G = rows * n;
+        pl.whole = n == 1;
+        share_q = (nq + n - 1) / n;
+        per = 1;
+    } else {
+        // whole rows, unless that gives some CTA over 90 KB more than the average (V = 151,936: batch 16 28.5 -> 27.0 us with
+        // whole rows, batch 24 the same, batch 20 30.3 -> 33.3, batch 256 204 -> 207); rows up to 132 KB always (V = 50,021:
+        // batch 16 23.7 -> 19.9 us, batch 28 27.2 -> 26.9; V = 32,000, batch 16: 23.0 -> 16.8)
+        per = (rows + num_sms - 1) / num_sms;
+        pl.whole = row_bytes <= 132 * 1024 || per * row_bytes - rows * row_bytes / num_sms <= 90 * 1024;
+        G = pl.whole ? (rows + per - 1) / per : num_sms;
+        share_q = pl.whole ? per * nq : (nq * rows + G - 1) / G;
+    }
+    if (pl.whole == 0 && G > nq * rows) G = nq * rows;
     pl.grid = (int)G;
-    long long share_q = (Q + G - 1) / G;
-    long long seg_elems = share_q * kVpQuantum;
-    seg_elems += kVpQuantum;  // a row's last quantum also takes the remainder
-    if (seg_elems > cfg.V) seg_elems = cfg.V;
+    long long seg_elems = share_q * kVpQuantum + kVpQuantum;  // a row's last quantum also takes the remainder
+    if (pl.whole || seg_elems > cfg.V) seg_elems = cfg.V;
     pl.max_seg_tiles = (int)((seg_elems * esz + TILE - 1) / TILE) + 1;
+    // four epilogue groups where three short rows or more queue for them (V = 32,000: batch 192 74.4 -> 67.3 us, batch 40
+    // 27.2 -> 25.7; a group alone is slower, batch 8 13.7 -> 14.9; rows of 100 KB: batch 64 39.3 -> 40.5)
+    pl.groups = seg_elems * esz <= 68 * 1024 && per >= 3 ? 4 : 2;
     const size_t budget = 224 * 1024;  // one CTA per SM
     int stages = 6;
-    while (stages > 2 && vp_smem_bytes(stages, pl.max_seg_tiles * NT) > budget) --stages;
+    while (stages > 2 && vp_smem_bytes(pl.groups, stages, pl.max_seg_tiles * NT) > budget) --stages;
     pl.stages = stages;
-    pl.smem_bytes = vp_smem_bytes(stages, pl.max_seg_tiles * NT);
+    pl.smem_bytes = vp_smem_bytes(pl.groups, stages, pl.max_seg_tiles * NT);
     return pl;
 }
 
@@ -1462,7 +1497,7 @@ cudaError_t vp_launch(graft_ctx* ctx, int batch, const void* d_logits, int32_t* 
     p.rows = batch * cfg.L;
     p.V = cfg.V;
     p.K = cfg.K;
-    p.nq = cfg.V / kVpQuantum > 0 ? cfg.V / kVpQuantum : 1;
+    p.nq = pl.whole || cfg.V < kVpQuantum ? 1 : cfg.V / kVpQuantum;
     p.Q = p.nq * p.rows;
     p.stages = pl.stages;
     p.n_cmax = pl.max_seg_tiles * NT;
@@ -1481,8 +1516,7 @@ cudaError_t vp_launch(graft_ctx* ctx, int batch, const void* d_logits, int32_t* 
     p.L = cfg.L;
     p.cos_out = (d_hidden != nullptr && cfg.L > 1) ? d_cos : nullptr;
     p.use_hint = 1;
-    const cudaError_t e = launch_pdl(bf16 ? vocab_pass_kernel<true> : vocab_pass_kernel<false>, dim3(pl.grid),
-                                     dim3(kVpThreads), pl.smem_bytes, st, p);
+    const cudaError_t e = launch_pdl(vp_kernel(bf16, pl.groups), dim3(pl.grid), dim3(kVpThreads), pl.smem_bytes, st, p);
     ctx->launches += 1;
     return e != cudaSuccess ? e : cudaGetLastError();
 }
@@ -1511,11 +1545,9 @@ cudaError_t vp_configure(const graft_config& cfg, int num_sms, size_t* max_smem)
     VpPlan pl = vp_make_plan(cfg, num_sms, cfg.max_batch > 4096 ? cfg.max_batch : 4096);
     *max_smem = pl.smem_bytes;
     if (pl.smem_bytes > 225 * 1024) return cudaErrorInvalidValue;
-    cudaError_t e;
-    if (cfg.logits_dtype == GRAFT_BF16)
-        e = cudaFuncSetAttribute(vocab_pass_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 225 * 1024);
-    else
-        e = cudaFuncSetAttribute(vocab_pass_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 225 * 1024);
+    cudaError_t e = cudaSuccess;
+    for (int groups = 2; groups <= 4 && e == cudaSuccess; groups += 2)
+        e = cudaFuncSetAttribute(vp_kernel(cfg.logits_dtype == GRAFT_BF16, groups), cudaFuncAttributeMaxDynamicSharedMemorySize, 225 * 1024);
     return e;
 }
 
@@ -1591,13 +1623,12 @@ extern "C" graft_status graft_vocab_pass_static(int32_t batch, int32_t L, int32_
                 cudaGetLastError();
                 return GRAFT_ERR_CUDA;
             }
-            if (cudaFuncSetAttribute(vocab_pass_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 225 * 1024) !=
-                    cudaSuccess ||
-                cudaFuncSetAttribute(vocab_pass_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 225 * 1024) !=
-                    cudaSuccess) {
-                cudaGetLastError();
-                return GRAFT_ERR_CUDA;
-            }
+            for (int i = 0; i < 4; ++i)
+                if (cudaFuncSetAttribute(vp_kernel((i & 1) != 0, i < 2 ? 2 : 4), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         225 * 1024) != cudaSuccess) {
+                    cudaGetLastError();
+                    return GRAFT_ERR_CUDA;
+                }
             sd->scratch = (VpStaticScratch*)ptr;
             sd->num_sms = sms;
             sd->ready = true;
@@ -1617,7 +1648,7 @@ extern "C" graft_status graft_vocab_pass_static(int32_t batch, int32_t L, int32_
     p.rows = batch * L;
     p.V = V;
     p.K = K;
-    p.nq = V / kVpQuantum > 0 ? V / kVpQuantum : 1;
+    p.nq = pl.whole || V < kVpQuantum ? 1 : V / kVpQuantum;
     p.Q = p.nq * p.rows;
     p.stages = pl.stages;
     p.n_cmax = pl.max_seg_tiles * NT;
@@ -1636,9 +1667,6 @@ extern "C" graft_status graft_vocab_pass_static(int32_t batch, int32_t L, int32_
     p.L = L;
     p.cos_out = nullptr;
     p.use_hint = 1;
-    if (logits_dtype == GRAFT_BF16)
-        vocab_pass_kernel<true><<<pl.grid, kVpThreads, pl.smem_bytes, st>>>(p);
-    else
-        vocab_pass_kernel<false><<<pl.grid, kVpThreads, pl.smem_bytes, st>>>(p);
+    vp_kernel(logits_dtype == GRAFT_BF16, pl.groups)<<<pl.grid, kVpThreads, pl.smem_bytes, st>>>(p);
     return cudaGetLastError() == cudaSuccess ? GRAFT_OK : GRAFT_ERR_CUDA;
 }

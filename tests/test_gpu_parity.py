@@ -83,6 +83,28 @@ def test_vocab_pass_shapes(V, K, L, Bt, dtype):
     _vocab_case(z, K, dtype)
 
 
+@pytest.mark.parametrize("V,K,L,Bt,dtype", [
+    (151937, 32, 16, 1, "bf16"),   # fewer rows than SMs, every row in four pieces with ragged ends
+    (151936, 16, 11, 4, "bf16"),   # three pieces
+    (300011, 32, 1, 1, "bf16"),    # one row in seven pieces
+    (90001, 8, 16, 2, "f32"),      # pieces of fp32 rows
+    (151937, 32, 15, 10, "bf16"),  # more rows than SMs, shares cut across rows
+    (70001, 16, 16, 10, "f32"),    # the same in fp32
+    (20011, 32, 16, 28, "bf16"),   # short whole rows, four epilogue groups
+    (9001, 8, 16, 40, "f32"),      # the same in fp32
+    (34001, 8, 16, 19, "bf16"),    # three whole rows a CTA or two
+    (2047, 16, 16, 10, "bf16"),    # rows shorter than a quantum of the partition
+])
+def test_vocab_pass_partitions_of_the_rows(V, K, L, Bt, dtype):
+    g = torch.Generator().manual_seed(V + Bt)
+    z = 2.0 * torch.randn((Bt, L, V), generator=g)
+    z[:, :, :: max(1, V // 7)] += 5.0
+    z = z.to(torch.bfloat16) if dtype == "bf16" else z
+    z[0, 0, V // 2:] = float("-inf")      # a piece without a finite element
+    z[Bt - 1, L - 1, ::5] = z[Bt - 1, L - 1, 3]  # ties in every piece
+    _vocab_case(z, K, dtype)
+
+
 def test_vocab_pass_ties_uniform_masked_and_bad_rows():
     V, K = 9000, 32
     g = torch.Generator().manual_seed(1)
