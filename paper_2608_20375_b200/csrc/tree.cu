@@ -42,7 +42,6 @@ struct TreeParams {
     const SabaResult* saba_pre;  // [batch] budget, status and state worked out by the edge-score kernel, or NULL
 };
 
-constexpr int TREE_THREADS = 1024;  // one CTA per SM (shared memory bound): all warps serve the parallel phases
 
 struct TreeSmem {
     float* es;           // [L*K*K]  sorted edge rows
@@ -192,6 +191,7 @@ __device__ __forceinline__ bool entry_before(const TreeSmem& sm, uint64_t e1, in
 // where this one stopped (pass0 = the earlier pass1, prefix and remaining as returned).  The 256 bins exist in four
 // copies (neighbouring warps use different ones) and in two generations, so that the next pass's bins are cleared
 // while this pass's are scanned.
+template <int NT>
 __device__ uint32_t cta_kth_largest(const TreeSmem& sm, const uint32_t* keys, int lo, int hi, int kth, int pass0,
                                     int pass1, uint32_t prefix, int& remaining, int tid) {
     const int warp = tid >> 5, lane = tid & 31;
@@ -200,16 +200,16 @@ __device__ uint32_t cta_kth_largest(const TreeSmem& sm, const uint32_t* keys, in
         prefix = 0u;
         remaining = kth;
     }
-    sm.hist[(pass0 & 1) * 1024 + tid] = 0u;
+    for (int i = tid; i < 1024; i += NT) sm.hist[(pass0 & 1) * 1024 + i] = 0u;
     __syncthreads();
     for (int pass = pass0; pass < pass1; ++pass) {
         const int shift = 24 - 8 * pass;
         uint32_t* h = sm.hist + (pass & 1) * 1024 + (warp & 3) * 256;
-        for (int i = lo + tid; i < hi; i += TREE_THREADS) {
+        for (int i = lo + tid; i < hi; i += NT) {
             const uint32_t k = keys[i];
             if ((k & mask) == prefix) atomicAdd(&h[(k >> shift) & 255u], 1u);
         }
-        sm.hist[((pass + 1) & 1) * 1024 + tid] = 0u;  // the other generation, for the next pass
+        for (int i = tid; i < 1024; i += NT) sm.hist[((pass + 1) & 1) * 1024 + i] = 0u;  // the other generation, for the next pass
         __syncthreads();
         if (warp == 0) {  // lane l owns bins 255-8l .. 248-8l, from the top down
             const uint32_t* hh = sm.hist + (pass & 1) * 1024;
@@ -256,12 +256,13 @@ __device__ uint32_t cta_kth_largest(const TreeSmem& sm, const uint32_t* keys, in
 // a level from flooding the node table while few keys are known (sharply peaked rows: every deviation from the
 // best chain costs tens of units, and the B-th largest key of the table stays far down for several levels).
 // Every thread of the CTA calls it; the children number at least kth in all.
+template <int NT>
 __device__ uint32_t cta_kth_largest_of_children_radix(const TreeSmem& sm, int cnt, uint32_t kx, float sx, int row,
                                                       int cx, int K, int kth, int tid) {
     const int warp = tid >> 5, lane = tid & 31;
     uint32_t prefix = 0u, mask = 0u;
     int remaining = kth;
-    sm.hist[tid] = 0u;
+    for (int i = tid; i < 1024; i += NT) sm.hist[i] = 0u;
     __syncthreads();
     for (int pass = 0; pass < 2; ++pass) {
         const int shift = 24 - 8 * pass;
@@ -271,7 +272,7 @@ __device__ uint32_t cta_kth_largest_of_children_radix(const TreeSmem& sm, int cn
             const uint32_t k = oc < kx ? oc : kx;
             if ((k & mask) == prefix) atomicAdd(&h[(k >> shift) & 255u], 1u);
         }
-        sm.hist[((pass + 1) & 1) * 1024 + tid] = 0u;  // the other generation, for the next pass
+        for (int i = tid; i < 1024; i += NT) sm.hist[((pass + 1) & 1) * 1024 + i] = 0u;  // the other generation, for the next pass
         __syncthreads();
         if (warp == 0) {  // lane l owns bins 255-8l .. 248-8l, from the top down
             const uint32_t* hh = sm.hist + (pass & 1) * 1024;
@@ -327,12 +328,12 @@ __device__ __forceinline__ int select_bin(uint32_t key, float top) {
 // (every child counted reaches it) and the best child, whose lower edge is the bound; the radix passes only if that
 // range is not finite (their top bits crowd into a few counters, which thousands of atomics then queue on; bins in
 // score spread them).
+template <int NT>
 __device__ uint32_t cta_kth_largest_of_children(const TreeSmem& sm, int cnt, uint32_t kx, float sx, int row, int cx,
                                                 int K, int kth, uint32_t theta, int tid) {
     const int warp = tid >> 5, lane = tid & 31;
     uint32_t* h = sm.hist;  // [1024 + 32], then [1] the best child key
-    h[tid] = 0u;
-    if (tid < 33) h[1024 + tid] = 0u;
+    for (int i = tid; i < 1024 + 33; i += NT) h[i] = 0u;
     __syncthreads();
     {
         uint32_t best = 0u;  // a node's first child has its largest key
@@ -348,7 +349,7 @@ __device__ uint32_t cta_kth_largest_of_children(const TreeSmem& sm, int cnt, uin
     const float scale = 1023.0f / (top - low);
     if (!(scale > 0.0f) || !(scale < 1e30f)) {  // (uniform) no finite range: -inf scores, or all children equal
         __syncthreads();
-        return cta_kth_largest_of_children_radix(sm, cnt, kx, sx, row, cx, K, kth, tid);
+        return cta_kth_largest_of_children_radix<NT>(sm, cnt, kx, sx, row, cx, K, kth, tid);
     }
     for (int r = 0; r < cnt; ++r) {
         const uint32_t oc = ord_from_float(sx + sm.es[row + es_col(r, cx, K)]);
@@ -405,23 +406,26 @@ __device__ __forceinline__ bool select_in_bucket(const SelBucket& st, uint32_t k
 // radix passes would, for one pass.  If the B-th largest falls into the shared last bin, two radix passes find its
 // 16-bit bucket instead.  Bins are padded by one word per 32 (the flood search's lanes own 32 consecutive bins each
 // and read them without bank conflicts).  Every thread of the CTA calls this; hi_i - lo_i >= kth >= 1.
+template <int NT>
 __device__ uint32_t cta_select_bucket(const TreeSmem& sm, const uint32_t* keys, int lo_i, int hi_i, int kth, float top,
                                       SelBucket& st, int tid) {
     const int warp = tid >> 5, lane = tid & 31;
     uint32_t* h = sm.hist;  // [1024 + 32] bins, [1060 + 32] sums of 32 bins
-    h[tid] = 0u;
-    if (tid < 32) h[1024 + tid] = 0u;
+    for (int i = tid; i < 1024 + 32; i += NT) h[i] = 0u;
     __syncthreads();
-    for (int i = lo_i + tid; i < hi_i; i += TREE_THREADS) {
+    for (int i = lo_i + tid; i < hi_i; i += NT) {
         const int d = select_bin(keys[i], top);
         atomicAdd(&h[d + (d >> 5)], 1u);
     }
     __syncthreads();
-    // warp w adds up bins 32 w .. 32 w + 31 (bin 0 holds the largest keys); warp 0 then finds the group of 32 bins that
+    // a warp adds up 32 bins at a time (bin 0 holds the largest keys); warp 0 then finds the group of 32 bins that
     // holds the kth largest key in a scan of the 32 sums, and the bin in a scan of that group: two short steps
     {
-        const uint32_t wsum = __reduce_add_sync(0xFFFFFFFFu, h[33 * warp + lane]);
-        if (lane == 0) h[1060 + warp] = wsum;
+#pragma unroll
+        for (int g = 0; g < 32; g += NT / 32) {
+            const uint32_t wsum = __reduce_add_sync(0xFFFFFFFFu, h[33 * (g + warp) + lane]);
+            if (lane == 0) h[1060 + g + warp] = wsum;
+        }
     }
     __syncthreads();
     if (warp == 0) {
@@ -454,7 +458,7 @@ __device__ uint32_t cta_select_bucket(const TreeSmem& sm, const uint32_t* keys, 
     if (bin >= 1023) {  // (uniform) below the range the bins resolve
         __syncthreads();
         int rem = 0;
-        const uint32_t prefix = cta_kth_largest(sm, keys, lo_i, hi_i, kth, 0, 2, 0u, rem, tid);
+        const uint32_t prefix = cta_kth_largest<NT>(sm, keys, lo_i, hi_i, kth, 0, 2, 0u, rem, tid);
         st.bin = -1;
         st.lo = prefix;
         st.hi = prefix | 0xFFFFu;
@@ -470,6 +474,7 @@ __device__ uint32_t cta_select_bucket(const TreeSmem& sm, const uint32_t* keys, 
 // many more values than there are buckets), so they are collected and ranked against each other directly; if there
 // are more than the list holds (heavy ties), a full radix select runs instead.
 // *n_reach: how many of all the keys reach the value returned (kth if no other key ties with it), or -1 if unknown.
+template <int NT>
 __device__ uint32_t cta_finish_select(const TreeSmem& sm, const uint32_t* keys, int lo_i, int hi_i, int kth, float top,
                                       const SelBucket& st, int tid, int* n_reach) {
     constexpr int kCap = 512;
@@ -477,7 +482,7 @@ __device__ uint32_t cta_finish_select(const TreeSmem& sm, const uint32_t* keys, 
     int* cnt = (int*)(sm.hist + 1100);  // [1]
     if (tid == 0) *cnt = 0;
     __syncthreads();
-    for (int i = lo_i + tid; i < hi_i; i += TREE_THREADS) {
+    for (int i = lo_i + tid; i < hi_i; i += NT) {
         const uint32_t k = keys[i];
         if (select_in_bucket(st, k, top)) {
             const int pos = atomicAdd(cnt, 1);
@@ -490,10 +495,10 @@ __device__ uint32_t cta_finish_select(const TreeSmem& sm, const uint32_t* keys, 
         __syncthreads();
         int rem = 0;
         *n_reach = -1;
-        return cta_kth_largest(sm, keys, lo_i, hi_i, kth, 0, 4, 0u, rem, tid);
+        return cta_kth_largest<NT>(sm, keys, lo_i, hi_i, kth, 0, 4, 0u, rem, tid);
     }
     const int remaining = st.rem;
-    for (int i = tid; i < n; i += TREE_THREADS) {
+    for (int i = tid; i < n; i += NT) {
         const uint32_t k = list[i];
         int gt = 0, ge = 0;
         for (int j = 0; j < n; ++j) {
@@ -516,12 +521,13 @@ __device__ uint32_t cta_finish_select(const TreeSmem& sm, const uint32_t* keys, 
 // The smallest of keys[lo_i..hi_i) that reaches the bound `theta` of the B-th largest key: a bound of it as well (the
 // B-th largest is one of those keys), reached by the same keys, and an actual key -- where hundreds of keys tie just
 // above a bucket's edge, their value.  The whole CTA; word: one word of scratch.
+template <int NT>
 __device__ __forceinline__ uint32_t cta_snap_to_key(const uint32_t* keys, int lo_i, int hi_i, uint32_t theta, uint32_t* word,
                                                     int tid) {
     if (tid == 0) *word = 0xFFFFFFFFu;
     __syncthreads();
     uint32_t mn = 0xFFFFFFFFu;
-    for (int i = lo_i + tid; i < hi_i; i += TREE_THREADS) {
+    for (int i = lo_i + tid; i < hi_i; i += NT) {
         const uint32_t k = keys[i];
         mn = (k >= theta && k < mn) ? k : mn;
     }
@@ -558,12 +564,13 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // Every thread calls this; the copies of one row form one group per thread.
+template <int NT>
 __device__ __forceinline__ void lazy_issue_gather(const TreeParams& p, const TreeSmem& sm, int j, int root_token, int tid,
                                                   const int K, const int m) {
     if (j >= p.L || lazy_neutral(p, j)) return;
     const int ld = m + 4, q4 = m / 4, n_par = j == 0 ? 1 : K;
     const int warp = tid >> 5, lane = tid & 31;
-    for (int r = warp; r <= n_par + K; r += TREE_THREADS / 32) {  // a warp per table row, a lane per 16 bytes
+    for (int r = warp; r <= n_par + K; r += NT / 32) {  // a warp per table row, a lane per 16 bytes
         const float* src;
         float* dst;
         if (r == n_par + K) {
@@ -581,6 +588,7 @@ __device__ __forceinline__ void lazy_issue_gather(const TreeParams& p, const Tre
 }
 // Every thread of the CTA calls this.
 // `inflight` is the depth whose table rows are on their way (or -1).
+template <int NT>
 __device__ __forceinline__ void lazy_score_row(const TreeParams& p, const TreeSmem& sm, int j, int root_token, int tid,
                                                int& inflight, const int K, const int m) {
     const int n_par = j == 0 ? 1 : K;
@@ -590,24 +598,24 @@ __device__ __forceinline__ void lazy_score_row(const TreeParams& p, const TreeSm
     const float* lps = sm.lpv + j * K;
     if (lazy_neutral(p, j)) {
         // edge = log q exactly (the DDTree score of Eq. 3); log q is already ordered by rank
-        for (int i = tid; i < K * K; i += TREE_THREADS) {
+        for (int i = tid; i < K * K; i += NT) {
             es[(i / K) * K + es_col(i % K, i / K, K)] = (i / K) < n_par ? lps[i % K] : 0.f;
             ei[i] = (uint8_t)(i % K);
         }
         __syncthreads();
         return;
     }
-    if (inflight != j) lazy_issue_gather(p, sm, j, root_token, tid, K, m);
+    if (inflight != j) lazy_issue_gather<NT>(p, sm, j, root_token, tid, K, m);
     cp_async_wait_all();
     __syncthreads();
     float* part = (float*)sm.hist;                // [K][K] dot products (the histogram space is idle here)
     uint32_t* wsc = sm.hist + 1024 + warp * 32;   // [32] per warp
     if (warp < 8) edge_dots<true>(sm.gP, sm.gC, sm.gU, m, K, n_par, part, warp, lane);
     __syncthreads();
-    lazy_issue_gather(p, sm, j + 1, root_token, tid, K, m);  // the table rows of this depth are no longer read
+    lazy_issue_gather<NT>(p, sm, j + 1, root_token, tid, K, m);  // the table rows of this depth are no longer read
     inflight = j + 1;
     const float inv_K = 1.0f / (float)K;
-    for (int par = warp; par < K; par += TREE_THREADS / 32) {  // one warp per parent
+    for (int par = warp; par < K; par += NT / 32) {  // one warp per parent
         float val;
         int rank;
         edge_row_finish(par < n_par ? part + (size_t)par * K : nullptr, lps, p.scale, p.beta, K, inv_K, wsc, lane, val,
@@ -620,6 +628,7 @@ __device__ __forceinline__ void lazy_score_row(const TreeParams& p, const TreeSm
     __syncthreads();
 }
 
+// NT: threads of the CTA (tree_pick)
 // KC, MC: the number of candidates per position and the width of the TDES tables as compile-time constants (the
 // configured workloads' K = 32, m = 128: every index computation with K becomes a shift), or 0: taken from the parameters
 // FAST: the usual round is known at compile time as well -- the budget comes from the edge-score kernel (no SABA
@@ -628,8 +637,8 @@ __device__ __forceinline__ void lazy_score_row(const TreeParams& p, const TreeSm
 // prefixes tie with the B-th largest key: it resolves them in parallel (the other instances leave more than 32 tied
 // keys to the sequential expansion; with edge scores in the keys such ties do not occur in tens, and the code's mere
 // presence costs this register-bound kernel 0.4 us a round)
-template <int KC, int MC, bool FAST, int NMAXC = 0, bool TIES = false>
-__global__ void __launch_bounds__(TREE_THREADS) tree_kernel(const TreeParams p) {
+template <int NT, int KC, int MC, bool FAST, int NMAXC = 0, bool TIES = false>
+__global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int K = KC ? KC : p.K, p_m = MC ? MC : p.m;
     const bool p_lazy = FAST ? true : p.lazy != 0;
@@ -660,11 +669,16 @@ __global__ void __launch_bounds__(TREE_THREADS) tree_kernel(const TreeParams p) 
     pre_r.status = 0;
     pre_r.state[0] = pre_r.state[1] = pre_r.state[2] = pre_r.state[3] = 0.f;
     if ((FAST || p.saba_pre) && tid == 0) pre_r = p.saba_pre[b];
-    int32_t lz_tok = 0;
-    float lz_lp = 0.f;
-    if (p_lazy && tid < L * K) {  // (L K <= 1024: a thread per candidate)
-        lz_tok = p.topk_id[(size_t)b * L * K + tid];
-        lz_lp = p.topk_lp[(size_t)b * L * K + tid];
+    constexpr int LZ = 1024 / NT;  // (L K <= 1024)
+    int32_t lz_tok[LZ] = {};
+    float lz_lp[LZ] = {};
+#pragma unroll
+    for (int q = 0; q < LZ; ++q) {
+        const int i = tid + q * NT;
+        if (p_lazy && i < L * K) {
+            lz_tok[q] = p.topk_id[(size_t)b * L * K + i];
+            lz_lp[q] = p.topk_lp[(size_t)b * L * K + i];
+        }
     }
     int rows_done = rows_pre;  // rows [0, rows_done) are in shared memory
     int inflight = -1;           // on-demand scoring: depth whose table rows are being fetched
@@ -689,26 +703,30 @@ __global__ void __launch_bounds__(TREE_THREADS) tree_kernel(const TreeParams p) 
             }
         }
     } else {
-        for (int i = tid; i < ne; i += TREE_THREADS) {
+        for (int i = tid; i < ne; i += NT) {
             sm.es[i] = p.esort[seq_e + i];
             sm.ei[i] = p.eidx[seq_e + i];
         }
     }
     if (p_lazy) {  // the candidates of every depth, for the rows that may have to be scored here
-        if (tid < L * K) {
-            sm.tokid[tid] = lz_tok;
-            sm.lpv[tid] = lz_lp;
+#pragma unroll
+        for (int q = 0; q < LZ; ++q) {
+            const int i = tid + q * NT;
+            if (i < L * K) {
+                sm.tokid[i] = lz_tok[q];
+                sm.lpv[i] = lz_lp[q];
+            }
         }
         if (rows_pre == 0) {  // the table rows of depth 0 arrive while the budget is worked out
             __syncthreads();
-            lazy_issue_gather(p, sm, 0, root, tid, K, p_m);
+            lazy_issue_gather<NT>(p, sm, 0, root, tid, K, p_m);
             inflight = 0;
         }
     }
     // a sequence whose tree will run deep had its deeper rows scored by the edge-score kernel as well (they are needed
     // several levels from here: plain loads, consumed after many barriers)
     if (p.rows_adaptive && deep_tree_decide(lp_top, L)) {  // (uniform)
-        for (int i = ne + tid; i < L * K * K; i += TREE_THREADS) {
+        for (int i = ne + tid; i < L * K * K; i += NT) {
             sm.es[i] = p.esort[seq_e + i];
             sm.ei[i] = p.eidx[seq_e + i];
         }
@@ -723,7 +741,7 @@ __global__ void __launch_bounds__(TREE_THREADS) tree_kernel(const TreeParams p) 
     const bool spec = bulk && rows_pre >= 2 && L >= 2 && 1 + K + K * K <= ncap;
     if (spec && warp >= 1) {
         mbar_wait_bounded(smem_u32(&rows_bar), 0, &rows_abort);
-        const int t1 = tid - 32, nth = TREE_THREADS - 32;
+        const int t1 = tid - 32, nth = NT - 32;
         if (t1 == 0) {
             sm.nkey[0] = 0xFFFFFFFFu;
             sm.nS[0] = 0.0f;
@@ -821,7 +839,7 @@ __global__ void __launch_bounds__(TREE_THREADS) tree_kernel(const TreeParams p) 
                 // level 2 that appends a third of what it would.
                 int nsel = ntot;
                 if (L > 2 && rows_done > 2 && ntot + K * K <= ncap) {  // (uniform)
-                    for (int j = tid; j < K * K; j += TREE_THREADS) {
+                    for (int j = tid; j < K * K; j += NT) {
                         const int x = 1 + K + j;
                         const uint32_t kx = sm.nkey[x];
                         const int cx = (int)((sm.ninfo[x] >> 13) & 31u);
@@ -831,10 +849,10 @@ __global__ void __launch_bounds__(TREE_THREADS) tree_kernel(const TreeParams p) 
                     nsel = ntot + K * K;
                     __syncthreads();
                 }
-                theta = cta_select_bucket(sm, sm.nkey, 1, nsel, budget, sel_top, sel, tid);
+                theta = cta_select_bucket<NT>(sm, sm.nkey, 1, nsel, budget, sel_top, sel, tid);
                 if (TIES) {
                     __syncthreads();
-                    theta = cta_snap_to_key(sm.nkey, 1, nsel, theta, sm.hist + 1100, tid);
+                    theta = cta_snap_to_key<NT>(sm.nkey, 1, nsel, theta, sm.hist + 1100, tid);
                     th_depth = nsel != ntot ? 3 : 2;
                 }
                 if (nsel != ntot) sel.valid = false;  // (the bucket counts keys that are not in the table)
@@ -852,9 +870,9 @@ __global__ void __launch_bounds__(TREE_THREADS) tree_kernel(const TreeParams p) 
             bool over = false;  // the node table is full
             if (d >= rows_done) {  // the edge rows of this depth: scored now, never if the expansion stops above it
                 int alive = 0;  // (nor if no node of the level can still have a selected child)
-                for (int x = b0 + tid; x < b1; x += TREE_THREADS) alive |= sm.nkey[x] >= theta ? 1 : 0;
+                for (int x = b0 + tid; x < b1; x += NT) alive |= sm.nkey[x] >= theta ? 1 : 0;
                 if (!__syncthreads_or(alive)) break;
-                lazy_score_row(p, sm, d, root, tid, inflight, K, p_m);
+                lazy_score_row<NT>(p, sm, d, root, tid, inflight, K, p_m);
                 rows_done = d + 1;
             }
             // grow: can a node appended here have a child that reaches theta?  (Its best child stands first in its sorted
@@ -869,7 +887,7 @@ __global__ void __launch_bounds__(TREE_THREADS) tree_kernel(const TreeParams p) 
                 if (ntot + total > ncap) {
                     over = true;
                 } else {
-                    for (int j = tid; j < total; j += TREE_THREADS) {
+                    for (int j = tid; j < total; j += NT) {
                         const int xi = j / K, r = j - xi * K, x = b0 + xi;
                         const uint32_t kx = sm.nkey[x];
                         const int cx = (int)((sm.ninfo[x] >> 13) & 31u), row = (d * K + cx) * K;
@@ -884,20 +902,20 @@ __global__ void __launch_bounds__(TREE_THREADS) tree_kernel(const TreeParams p) 
                 }
             } else {
                 // The children that can still matter are a prefix of a node's sorted row (scores only fall along the
-                // row); its length comes from a binary search.  The level is taken in chunks of 1024 nodes: one thread
+                // row); its length comes from a binary search.  The level is taken in chunks of NT nodes: one thread
                 // per node finds the length and the set of candidate ranks in that prefix, a scan of the lengths places
                 // the chunk's children in the table in the order of the nodes, then one thread per child (its node found
                 // in the scan by binary search) writes it, behind its siblings of lower rank.  No shared counter, a node
                 // with many children holds nobody up, and the table stays in level order.
                 int cur = ntot;
-                int* pre = (int*)sm.hist;            // [1024] inclusive scan of the chunk, then [32] warp totals
-                uint32_t* cmask = sm.hist + 1100;    // [1024] candidate ranks of the children a node appends
+                int* pre = (int*)sm.hist;            // [NT] inclusive scan of the chunk, then [32] warp totals
+                uint32_t* cmask = sm.hist + 1100;    // [NT] candidate ranks of the children a node appends
                 // At most B nodes of a level end up in the tree: a chunk that would append many times more children than
                 // that (or more than the table has room for) first raises theta to (a lower bound of) the B-th largest
                 // key among those children.  (The search costs about as much as two ordinary levels: ordinary rounds,
                 // whose levels stay within a few times B, never run it.)
                 const int flood = 8 * budget > 1024 ? 8 * budget : 1024;
-                for (int c0 = b0; c0 < b1; c0 += TREE_THREADS) {  // (uniform)
+                for (int c0 = b0; c0 < b1; c0 += NT) {  // (uniform)
                   const int x = c0 + tid;
                   int total = 0;
                   for (int attempt = 0;; ++attempt) {  // (uniform: at most two rounds)
@@ -948,9 +966,9 @@ __global__ void __launch_bounds__(TREE_THREADS) tree_kernel(const TreeParams p) 
                         const int t = __shfl_up_sync(0xFFFFFFFFu, incl, o2);
                         if (lane >= o2) incl += t;
                     }
-                    if (lane == 31) pre[TREE_THREADS + warp] = incl;
+                    if (lane == 31) pre[NT + warp] = incl;
                     __syncthreads();
-                    const int wt = pre[TREE_THREADS + lane];
+                    const int wt = lane < NT / 32 ? pre[NT + lane] : 0;
                     int wincl = wt;
 #pragma unroll
                     for (int o2 = 1; o2 < 32; o2 <<= 1) {
@@ -961,7 +979,7 @@ __global__ void __launch_bounds__(TREE_THREADS) tree_kernel(const TreeParams p) 
                     pre[tid] = __shfl_sync(0xFFFFFFFFu, wincl - wt, warp) + incl;
                     __syncthreads();
                     if (attempt == 0 && total >= budget && (total > flood || cur + total > ncap)) {  // (uniform) the search below uses the scan's space: count again
-                        const uint32_t tl = cta_kth_largest_of_children(sm, cnt, kx, sx, row, cx, K, budget, theta, tid);
+                        const uint32_t tl = cta_kth_largest_of_children<NT>(sm, cnt, kx, sx, row, cx, K, budget, theta, tid);
                         theta = tl > theta ? tl : theta;
                         if (TIES) th_depth = d + 1;
                         continue;
@@ -972,8 +990,8 @@ __global__ void __launch_bounds__(TREE_THREADS) tree_kernel(const TreeParams p) 
                         over = true;
                         break;
                     }
-                    for (int i = tid; i < total; i += TREE_THREADS) {
-                        int lo_t = 0, hi_t = TREE_THREADS - 1;  // owner: the first thread whose scan exceeds i
+                    for (int i = tid; i < total; i += NT) {
+                        int lo_t = 0, hi_t = NT - 1;  // owner: the first thread whose scan exceeds i
                         while (lo_t < hi_t) {
                             const int mid = (lo_t + hi_t) >> 1;
                             if (pre[mid] > i)
@@ -1002,7 +1020,7 @@ __global__ void __launch_bounds__(TREE_THREADS) tree_kernel(const TreeParams p) 
                         sm.ninfo[at] = (uint32_t)xo | ((uint32_t)c << 13) | ((uint32_t)(d + 1) << 18) | ((uint32_t)r << 24);
                     }
                     cur += total;
-                    if (c0 + TREE_THREADS < b1) __syncthreads();  // the scan space is reused by the next chunk
+                    if (c0 + NT < b1) __syncthreads();  // the scan space is reused by the next chunk
                 }
                 lvl_end = cur;
             }
@@ -1021,10 +1039,10 @@ __global__ void __launch_bounds__(TREE_THREADS) tree_kernel(const TreeParams p) 
             // the exact B-th largest key is recomputed only when the table has grown noticeably
             if (ntot - 1 >= budget && (theta == 0u || ntot - n_at_select >= ntot / 8)) {
                 sel_top = 0.0f + sm.es[0];  // the root's best child
-                theta = cta_select_bucket(sm, sm.nkey, 1, ntot, budget, sel_top, sel, tid);  // a lower bound
+                theta = cta_select_bucket<NT>(sm, sm.nkey, 1, ntot, budget, sel_top, sel, tid);  // a lower bound
                 if (TIES) {
                     __syncthreads();
-                    theta = cta_snap_to_key(sm.nkey, 1, ntot, theta, sm.hist + 1100, tid);
+                    theta = cta_snap_to_key<NT>(sm.nkey, 1, ntot, theta, sm.hist + 1100, tid);
                     th_depth = d + 1;
                 }
                 n_at_select = ntot;
@@ -1036,13 +1054,13 @@ __global__ void __launch_bounds__(TREE_THREADS) tree_kernel(const TreeParams p) 
             // the exact value: the last 16-bit search still holds if nothing was appended after it
             if (!(n_at_select == ntot && sel.valid)) {
                 sel_top = 0.0f + sm.es[0];  // the root's best child
-                cta_select_bucket(sm, sm.nkey, 1, ntot, budget, sel_top, sel, tid);
+                cta_select_bucket<NT>(sm, sm.nkey, 1, ntot, budget, sel_top, sel, tid);
             }
-            theta = cta_finish_select(sm, sm.nkey, 1, ntot, budget, sel_top, sel, tid, &n_reach);
+            theta = cta_finish_select<NT>(sm, sm.nkey, 1, ntot, budget, sel_top, sel, tid, &n_reach);
         }
         __syncthreads();
         if (table_ok) {
-            const int per = (ntot + TREE_THREADS - 1) / TREE_THREADS;
+            const int per = (ntot + NT - 1) / NT;
             const int i0 = tid * per < ntot ? tid * per : ntot, i1 = i0 + per < ntot ? i0 + per : ntot;
             // The tree is {key > theta} plus some of the keys equal to theta.  If exactly B keys reach theta (no other
             // key ties with the B-th largest: the usual case), {key >= theta} is the whole tree; so is the table itself
@@ -1172,7 +1190,7 @@ __global__ void __launch_bounds__(TREE_THREADS) tree_kernel(const TreeParams p) 
             }
             if (lane == 31) sm.hist[warp] = (uint32_t)incl;
             __syncthreads();
-            const int wt = (int)sm.hist[lane];  // (32 warps: a lane per warp total)
+            const int wt = lane < NT / 32 ? (int)sm.hist[lane] : 0;  // (a lane per warp total)
             int wincl = wt;
 #pragma unroll
             for (int o2 = 1; o2 < 32; o2 <<= 1) {
@@ -1202,7 +1220,7 @@ __global__ void __launch_bounds__(TREE_THREADS) tree_kernel(const TreeParams p) 
             __syncthreads();
             // (for the sequential tail only) frontier entries of the selected nodes: the first child of the sorted row
             // that is not selected, i.e. the first with ord(score) <= theta
-            for (int n = tid; n <= n_gt && !ordered; n += TREE_THREADS) {
+            for (int n = tid; n <= n_gt && !ordered; n += NT) {
                 const int d = sm.depth[n];
                 uint64_t e = 0ull;
                 if (d < L) {
@@ -1223,7 +1241,7 @@ __global__ void __launch_bounds__(TREE_THREADS) tree_kernel(const TreeParams p) 
         }
     }
     if (p_lazy && !table_ok && budget > 0) {  // the sequential fall-back may reach any depth
-        for (; rows_done < L; ++rows_done) lazy_score_row(p, sm, rows_done, root, tid, inflight, K, p_m);
+        for (; rows_done < L; ++rows_done) lazy_score_row<NT>(p, sm, rows_done, root, tid, inflight, K, p_m);
     }
     if (!table_ok && tid == 0) sm.ent[0] = budget > 0 ? pack_entry(0.0f + sm.es[0], 1, 0, 0, sm.ei[0]) : 0ull;
     if (ordered) {  // (uniform) the tree is complete and in level order
@@ -1238,11 +1256,11 @@ __global__ void __launch_bounds__(TREE_THREADS) tree_kernel(const TreeParams p) 
         sm.lvl_count[tid] = 0;
         sm.lvl_fill[tid] = 0;
     }
-    for (int n = tid; n < nmax; n += TREE_THREADS) sm.chmask[n] = 0u;
+    for (int n = tid; n < nmax; n += NT) sm.chmask[n] = 0u;
     __syncthreads();
     const int n_pre = table_ok ? n_gt : 0;  // nodes 0..n_pre are final before the tail starts
     if (warp >= 1) {
-        for (int n = tid - 32; n <= n_pre; n += TREE_THREADS - 32) {
+        for (int n = tid - 32; n <= n_pre; n += NT - 32) {
             if (n > 0) atomicOr(&sm.chmask[sm.parent[n]], 1u << sm.cand[n]);
             atomicAdd(&sm.lvl_count[sm.depth[n]], 1);
         }
@@ -1383,7 +1401,7 @@ __global__ void __launch_bounds__(TREE_THREADS) tree_kernel(const TreeParams p) 
             __syncwarp();
         }
     } else if (warp != 0) {
-        for (int i = n_nodes + tid - 32; i < nmax; i += TREE_THREADS - 32) {
+        for (int i = n_nodes + tid - 32; i < nmax; i += NT - 32) {
             o.d_token[ob + i] = -1;
             o.d_parent[ob + i] = -1;
             o.d_depth[ob + i] = -1;
@@ -1392,10 +1410,10 @@ __global__ void __launch_bounds__(TREE_THREADS) tree_kernel(const TreeParams p) 
         }
         // mask rows from the first multiple of 32 at or above n_nodes on are all padding
         const int z0 = ((n_nodes + 31) / 32) * 32;
-        for (size_t k = (size_t)z0 * W + tid - 32; k < (size_t)nmax * W; k += TREE_THREADS - 32) o.d_mask[ob * W + k] = 0u;
+        for (size_t k = (size_t)z0 * W + tid - 32; k < (size_t)nmax * W; k += NT - 32) o.d_mask[ob * W + k] = 0u;
     }
     if (!ordered) __syncthreads();  // (the placement above; the padding is nobody's input)
-    for (int n = tid; n < n_nodes; n += TREE_THREADS) {
+    for (int n = tid; n < n_nodes; n += NT) {
         const int i = ordered ? n : sm.canon[n], d = sm.depth[n];
         const int par = n == 0 ? -1 : (ordered ? sm.parent[n] : sm.canon[sm.parent[n]]);
         sm.cparent[i] = (int16_t)par;
@@ -1415,7 +1433,7 @@ __global__ void __launch_bounds__(TREE_THREADS) tree_kernel(const TreeParams p) 
         const size_t region = (size_t)ncap * 12 > stage_off + (size_t)8 * 32 * W * 4 ? (size_t)ncap * 12
                                                                                          : stage_off + (size_t)8 * 32 * W * 4;
         int mw = (int)((region - stage_off) / ((size_t)32 * W * 4));
-        mw = mw > TREE_THREADS / 32 ? TREE_THREADS / 32 : mw;
+        mw = mw > NT / 32 ? NT / 32 : mw;
         uint32_t* tile = sm.stage + (size_t)warp * 32 * W;
         for (int i0 = warp * 32; i0 < n_nodes && warp < mw; i0 += mw * 32) {
             const int i = i0 + lane;
@@ -1564,15 +1582,42 @@ size_t tree_smem_bytes(const graft_config& cfg) {
     return tree_smem_layout(cfg.L, cfg.K, nmax, tree_node_cap(cfg.L, cfg.K, nmax, lazy_m), lazy_m, nullptr, nullptr);
 }
 
+struct TreeInstance {
+    void (*kernel)(const TreeParams);
+    int threads;
+};
+// Threads of a CTA: a phase costs its instructions times the warps that run it, and the levels' sizes go with K (1 + K +
+// K^2 nodes to begin with): 256 threads for K <= 8 (round at batch 1, V = 32,000, K = 8: 34.0 us with 1024 threads, 32.2
+// with 512, 31.8 with 256), 512 for K <= 20 (batch 16, K = 16: 50.6, 48.5, 50.5; batch 37, K = 11, beta = 0: 52.5, 51.8,
+// 55.2), else 1024 (batch 64, K = 32: 97.3, 99.9, 108.9).
+// usual: the budget from the edge-score kernel, deeper rows on demand; neutral: beta = 0
+template <bool NEUTRAL>
+static TreeInstance tree_pick_general(int K) {
+    if (K <= 8) return {tree_kernel<256, 0, 0, false, 0, NEUTRAL>, 256};
+    if (K <= 20) return {tree_kernel<512, 0, 0, false, 0, NEUTRAL>, 512};
+    return {tree_kernel<1024, 0, 0, false, 0, NEUTRAL>, 1024};
+}
+static TreeInstance tree_pick(const graft_config& cfg, bool usual, bool neutral) {
+    const int nmax = cfg.budget_max + 1;
+    usual = usual && cfg.m == 128;
+    if (neutral) {
+        if (usual && cfg.K == 32) return {tree_kernel<1024, 32, 128, true, 0, true>, 1024};
+        return tree_pick_general<true>(cfg.K);
+    }
+    if (usual && cfg.K == 32) {
+        if (nmax == 513 && tree_node_cap(cfg.L, cfg.K, nmax, cfg.m) == 6144) return {tree_kernel<1024, 32, 128, true, 513>, 1024};
+        return {tree_kernel<1024, 32, 128, true>, 1024};
+    }
+    if (usual && cfg.K == 16) return {tree_kernel<512, 16, 128, true>, 512};
+    if (usual && cfg.K == 8) return {tree_kernel<256, 8, 128, true>, 256};
+    return tree_pick_general<false>(cfg.K);
+}
+
 cudaError_t tree_configure(const graft_config& cfg) {
     const int bytes = (int)tree_smem_bytes(cfg);
-    cudaError_t e = cudaFuncSetAttribute(tree_kernel<0, 0, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(tree_kernel<32, 128, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(tree_kernel<32, 128, true, 513>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(tree_kernel<16, 128, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(tree_kernel<8, 128, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(tree_kernel<0, 0, false, 0, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(tree_kernel<32, 128, true, 0, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    cudaError_t e = cudaSuccess;
+    for (int i = 0; i < 4 && e == cudaSuccess; ++i)
+        e = cudaFuncSetAttribute(tree_pick(cfg, (i & 1) != 0, (i & 2) != 0).kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     return e;
 }
 
@@ -1621,13 +1666,9 @@ cudaError_t tree_launch(graft_ctx* ctx, int batch, const int32_t* d_topk_id, con
     p.saba_pre = d_saba_pre;
     // the instances with K and m known at compile time serve the usual round (the budget from the edge-score kernel,
     // deeper rows on demand)
-    const bool usual = cfg.m == 128 && p.lazy && p.saba_pre != nullptr;
-    void (*kern)(const TreeParams) = tree_kernel<0, 0, false>;
-    if (usual && cfg.K == 32) kern = (ctx->nmax == 513 && p.ncap == 6144) ? tree_kernel<32, 128, true, 513> : tree_kernel<32, 128, true>;
-    if (usual && cfg.K == 16) kern = tree_kernel<16, 128, true>;
-    if (usual && cfg.K == 8) kern = tree_kernel<8, 128, true>;
-    if (p.beta == 0.0f) kern = (usual && cfg.K == 32) ? tree_kernel<32, 128, true, 0, true> : tree_kernel<0, 0, false, 0, true>;
-    const cudaError_t e = launch_pdl(kern, dim3(batch), dim3(TREE_THREADS), tree_smem_bytes(cfg), st, p);
+    const bool usual = p.lazy && p.saba_pre != nullptr;
+    const TreeInstance kern = tree_pick(cfg, usual, p.beta == 0.0f);
+    const cudaError_t e = launch_pdl(kern.kernel, dim3(batch), dim3(kern.threads), tree_smem_bytes(cfg), st, p);
     ctx->launches += 1;
     return e != cudaSuccess ? e : cudaGetLastError();
 }
