@@ -16,6 +16,7 @@ namespace graft {
 __device__ __forceinline__ double saba_cost(const SabaDev& sp, double B, double prefix) {
     if (sp.cost_mode == 0) return sp.c0 + sp.c1 * B + sp.c2 * B * prefix;
     if (B <= sp.pts_n[0]) return sp.pts_t[0];
+#pragma unroll 1
     for (int i = 1; i < sp.n_pts; ++i)
         if (B <= sp.pts_n[i]) {
             double w = (B - sp.pts_n[i - 1]) / (sp.pts_n[i] - sp.pts_n[i - 1]);
@@ -34,6 +35,7 @@ __device__ __forceinline__ SabaResult saba_warp(const SabaDev& saba, int bmin, i
     SabaResult r;
     // everything that comes from global memory is asked for first
     int st = 0;
+#pragma unroll 1
     for (int j = lane; j < L; j += 32) st |= row_status[j];
     const int err = vp_err[0];
     const bool use_saba = fixed_budget == nullptr;
@@ -41,7 +43,9 @@ __device__ __forceinline__ SabaResult saba_warp(const SabaDev& saba, int bmin, i
     float hist_f = 0.f;
     int prefix_i = 0, fixed = 0;
     if (use_saba) {
+#pragma unroll 1
         for (int j = lane; j < L; j += 32) conf += exp((double)topk_lp[(size_t)j * K]);
+#pragma unroll 1
         for (int j = lane; j < L - 1; j += 32) rs += cosv[j];
         if (L >= 2) {
             c_first = cosv[0];
@@ -77,6 +81,7 @@ __device__ __forceinline__ SabaResult saba_warp(const SabaDev& saba, int bmin, i
             const double prefix = (double)prefix_i;
             double ubest = -INFINITY;
             int bbest = bmin;
+#pragma unroll 1
             for (int B = bmin + lane * bstep; B <= bmax; B += 32 * bstep) {
                 const double G = 1.0 - exp(-(double)B / tau);
                 const double u = G / saba_cost(saba, (double)B, prefix);

@@ -165,6 +165,7 @@ __device__ __forceinline__ uint64_t pack_entry(float score, int child_depth, int
 // Does the prefix of node n1 come before the prefix of node n2 in lexicographic order of candidate ranks?
 // Both at the same depth, n1 != n2.
 __device__ __forceinline__ bool path_less(const TreeSmem& sm, int n1, int n2) {
+#pragma unroll 1
     for (int step = 0; step < kMaxL && sm.parent[n1] != sm.parent[n2]; ++step) {  // (depth <= L: the bound is never hit)
         n1 = sm.parent[n1];
         n2 = sm.parent[n2];
@@ -200,15 +201,19 @@ __device__ uint32_t cta_kth_largest(const TreeSmem& sm, const uint32_t* keys, in
         prefix = 0u;
         remaining = kth;
     }
+#pragma unroll 1
     for (int i = tid; i < 1024; i += NT) sm.hist[(pass0 & 1) * 1024 + i] = 0u;
     __syncthreads();
+#pragma unroll 1
     for (int pass = pass0; pass < pass1; ++pass) {
         const int shift = 24 - 8 * pass;
         uint32_t* h = sm.hist + (pass & 1) * 1024 + (warp & 3) * 256;
+#pragma unroll 1
         for (int i = lo + tid; i < hi; i += NT) {
             const uint32_t k = keys[i];
             if ((k & mask) == prefix) atomicAdd(&h[(k >> shift) & 255u], 1u);
         }
+#pragma unroll 1
         for (int i = tid; i < 1024; i += NT) sm.hist[((pass + 1) & 1) * 1024 + i] = 0u;  // the other generation, for the next pass
         __syncthreads();
         if (warp == 0) {  // lane l owns bins 255-8l .. 248-8l, from the top down
@@ -262,16 +267,20 @@ __device__ uint32_t cta_kth_largest_of_children_radix(const TreeSmem& sm, int cn
     const int warp = tid >> 5, lane = tid & 31;
     uint32_t prefix = 0u, mask = 0u;
     int remaining = kth;
+#pragma unroll 1
     for (int i = tid; i < 1024; i += NT) sm.hist[i] = 0u;
     __syncthreads();
+#pragma unroll 1
     for (int pass = 0; pass < 2; ++pass) {
         const int shift = 24 - 8 * pass;
         uint32_t* h = sm.hist + (pass & 1) * 1024 + (warp & 3) * 256;
+#pragma unroll 1
         for (int r = 0; r < cnt; ++r) {
             const uint32_t oc = ord_from_float(sx + sm.es[row + es_col(r, cx, K)]);
             const uint32_t k = oc < kx ? oc : kx;
             if ((k & mask) == prefix) atomicAdd(&h[(k >> shift) & 255u], 1u);
         }
+#pragma unroll 1
         for (int i = tid; i < 1024; i += NT) sm.hist[((pass + 1) & 1) * 1024 + i] = 0u;  // the other generation, for the next pass
         __syncthreads();
         if (warp == 0) {  // lane l owns bins 255-8l .. 248-8l, from the top down
@@ -333,6 +342,7 @@ __device__ uint32_t cta_kth_largest_of_children(const TreeSmem& sm, int cnt, uin
                                                 int K, int kth, uint32_t theta, int tid) {
     const int warp = tid >> 5, lane = tid & 31;
     uint32_t* h = sm.hist;  // [1024 + 32], then [1] the best child key
+#pragma unroll 1
     for (int i = tid; i < 1024 + 33; i += NT) h[i] = 0u;
     __syncthreads();
     {
@@ -351,6 +361,7 @@ __device__ uint32_t cta_kth_largest_of_children(const TreeSmem& sm, int cnt, uin
         __syncthreads();
         return cta_kth_largest_of_children_radix<NT>(sm, cnt, kx, sx, row, cx, K, kth, tid);
     }
+#pragma unroll 1
     for (int r = 0; r < cnt; ++r) {
         const uint32_t oc = ord_from_float(sx + sm.es[row + es_col(r, cx, K)]);
         const float sc = __uint_as_float(bits_from_ord(oc < kx ? oc : kx));
@@ -373,6 +384,7 @@ __device__ uint32_t cta_kth_largest_of_children(const TreeSmem& sm, int cnt, uin
         const int excl = incl - sum;
         if (excl < kth && kth <= incl) {
             int acc = excl, bin = 32 * lane;
+#pragma unroll 1
             for (int q = 0; q < 32; ++q) {
                 const int c = (int)mine[q];
                 if (acc < kth && kth <= acc + c) bin = 32 * lane + q;
@@ -411,8 +423,10 @@ __device__ uint32_t cta_select_bucket(const TreeSmem& sm, const uint32_t* keys, 
                                       SelBucket& st, int tid) {
     const int warp = tid >> 5, lane = tid & 31;
     uint32_t* h = sm.hist;  // [1024 + 32] bins, [1060 + 32] sums of 32 bins
+#pragma unroll 1
     for (int i = tid; i < 1024 + 32; i += NT) h[i] = 0u;
     __syncthreads();
+#pragma unroll (NT == 1024 ? 4 : 1)
     for (int i = lo_i + tid; i < hi_i; i += NT) {
         const int d = select_bin(keys[i], top);
         atomicAdd(&h[d + (d >> 5)], 1u);
@@ -482,6 +496,7 @@ __device__ uint32_t cta_finish_select(const TreeSmem& sm, const uint32_t* keys, 
     int* cnt = (int*)(sm.hist + 1100);  // [1]
     if (tid == 0) *cnt = 0;
     __syncthreads();
+#pragma unroll (NT == 1024 ? 4 : 1)
     for (int i = lo_i + tid; i < hi_i; i += NT) {
         const uint32_t k = keys[i];
         if (select_in_bucket(st, k, top)) {
@@ -498,9 +513,11 @@ __device__ uint32_t cta_finish_select(const TreeSmem& sm, const uint32_t* keys, 
         return cta_kth_largest<NT>(sm, keys, lo_i, hi_i, kth, 0, 4, 0u, rem, tid);
     }
     const int remaining = st.rem;
+#pragma unroll 1
     for (int i = tid; i < n; i += NT) {
         const uint32_t k = list[i];
         int gt = 0, ge = 0;
+#pragma unroll 1
         for (int j = 0; j < n; ++j) {
             const uint32_t o = list[j];
             gt += o > k ? 1 : 0;
@@ -527,6 +544,7 @@ __device__ __forceinline__ uint32_t cta_snap_to_key(const uint32_t* keys, int lo
     if (tid == 0) *word = 0xFFFFFFFFu;
     __syncthreads();
     uint32_t mn = 0xFFFFFFFFu;
+#pragma unroll (NT == 1024 ? 4 : 1)
     for (int i = lo_i + tid; i < hi_i; i += NT) {
         const uint32_t k = keys[i];
         mn = (k >= theta && k < mn) ? k : mn;
@@ -570,6 +588,7 @@ __device__ __forceinline__ void lazy_issue_gather(const TreeParams& p, const Tre
     if (j >= p.L || lazy_neutral(p, j)) return;
     const int ld = m + 4, q4 = m / 4, n_par = j == 0 ? 1 : K;
     const int warp = tid >> 5, lane = tid & 31;
+#pragma unroll 1
     for (int r = warp; r <= n_par + K; r += NT / 32) {  // a warp per table row, a lane per 16 bytes
         const float* src;
         float* dst;
@@ -582,6 +601,7 @@ __device__ __forceinline__ void lazy_issue_gather(const TreeParams& p, const Tre
             src = (r < n_par ? p.P : p.C) + (size_t)tok * m;
             dst = r < n_par ? sm.gP + (size_t)r * ld : sm.gC + (size_t)(r - n_par) * ld;
         }
+#pragma unroll 1
         for (int k4 = lane; k4 < q4; k4 += 32) cp_async16(smem_u32(dst + 4 * k4), src + 4 * k4);
     }
     cp_async_commit();
@@ -598,6 +618,7 @@ __device__ __forceinline__ void lazy_score_row(const TreeParams& p, const TreeSm
     const float* lps = sm.lpv + j * K;
     if (lazy_neutral(p, j)) {
         // edge = log q exactly (the DDTree score of Eq. 3); log q is already ordered by rank
+#pragma unroll 1
         for (int i = tid; i < K * K; i += NT) {
             es[(i / K) * K + es_col(i % K, i / K, K)] = (i / K) < n_par ? lps[i % K] : 0.f;
             ei[i] = (uint8_t)(i % K);
@@ -615,6 +636,7 @@ __device__ __forceinline__ void lazy_score_row(const TreeParams& p, const TreeSm
     lazy_issue_gather<NT>(p, sm, j + 1, root_token, tid, K, m);  // the table rows of this depth are no longer read
     inflight = j + 1;
     const float inv_K = 1.0f / (float)K;
+#pragma unroll 1
     for (int par = warp; par < K; par += NT / 32) {  // one warp per parent
         float val;
         int rank;
@@ -629,6 +651,11 @@ __device__ __forceinline__ void lazy_score_row(const TreeParams& p, const TreeSm
 }
 
 // NT: threads of the CTA (tree_pick)
+// Code size: a round's kernels run most of their phases once, so a phase costs its instructions' way from L2 as well as
+// their issue.  Loops are not unrolled unless that measured faster (207 -> 126 KB of code for the K = 32 instance, 215 -> 106
+// for K = 8; batch 1, V = 32,000, K = 8: 32.4 -> 29.5 us a round; batch 37, K = 11, beta = 0: 52.0 -> 49.0; batch 256: 298.3
+// -> 296.8; batch 64 with wide levels 97.1 -> 98.2).  Searches that are rare or have several sites as calls: smaller still,
+// but a call costs this register-bound kernel 3 us.
 // KC, MC: the number of candidates per position and the width of the TDES tables as compile-time constants (the
 // configured workloads' K = 32, m = 128: every index computation with K becomes a shift), or 0: taken from the parameters
 // FAST: the usual round is known at compile time as well -- the budget comes from the edge-score kernel (no SABA
@@ -693,16 +720,19 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
             mbar_arrive_expect_tx(smem_u32(&rows_bar), (uint32_t)ne * 5u);
             const char* g_es = (const char*)(p.esort + seq_e);
             const char* g_ei = (const char*)(p.eidx + seq_e);
+#pragma unroll 1
             for (uint32_t off = 0; off < (uint32_t)ne * 4u; off += 16384u) {
                 const uint32_t bytes = (uint32_t)ne * 4u - off < 16384u ? (uint32_t)ne * 4u - off : 16384u;
                 tma_load_1d(smem_u32((char*)sm.es + off), g_es + off, bytes, smem_u32(&rows_bar));
             }
+#pragma unroll 1
             for (uint32_t off = 0; off < (uint32_t)ne; off += 16384u) {
                 const uint32_t bytes = (uint32_t)ne - off < 16384u ? (uint32_t)ne - off : 16384u;
                 tma_load_1d(smem_u32((char*)sm.ei + off), g_ei + off, bytes, smem_u32(&rows_bar));
             }
         }
     } else {
+#pragma unroll 1
         for (int i = tid; i < ne; i += NT) {
             sm.es[i] = p.esort[seq_e + i];
             sm.ei[i] = p.eidx[seq_e + i];
@@ -726,6 +756,7 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
     // a sequence whose tree will run deep had its deeper rows scored by the edge-score kernel as well (they are needed
     // several levels from here: plain loads, consumed after many barriers)
     if (p.rows_adaptive && deep_tree_decide(lp_top, L)) {  // (uniform)
+#pragma unroll 1
         for (int i = ne + tid; i < L * K * K; i += NT) {
             sm.es[i] = p.esort[seq_e + i];
             sm.ei[i] = p.eidx[seq_e + i];
@@ -755,6 +786,7 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
             sm.ninfo[1 + c] = 0u | ((uint32_t)c << 13) | (1u << 18) | ((uint32_t)t1 << 24);
         }
         named_bar_sync(1, nth);
+#pragma unroll 1
         for (int j = t1; j < K * K; j += nth) {  // level 1
             const int xi = j / K, r = j - xi * K, x = 1 + xi;
             const uint32_t kx = sm.nkey[x];
@@ -779,6 +811,7 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
             sm.scal[0] = r.budget;
             sm.scal[2] = r.status;
             if (o.d_state) {
+#pragma unroll 1
                 for (int i = 0; i < 4; ++i) o.d_state[(size_t)b * 4 + i] = r.state[i];
             }
         }
@@ -839,6 +872,7 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
                 // level 2 that appends a third of what it would.
                 int nsel = ntot;
                 if (L > 2 && rows_done > 2 && ntot + K * K <= ncap) {  // (uniform)
+#pragma unroll (NT == 1024 ? 4 : 1)
                     for (int j = tid; j < K * K; j += NT) {
                         const int x = 1 + K + j;
                         const uint32_t kx = sm.nkey[x];
@@ -863,6 +897,7 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
         // (the bounds of the level being expanded and the end of the table are the same in every thread: no thread has to
         // publish them, and a level costs three barriers -- two in the scan, one at its end)
         int lv0 = spec ? 1 + K : 0, lv1 = spec ? 1 + K + K * K : 1;
+#pragma unroll 1
         for (int d = spec ? 2 : 0; d < L; ++d) {
             const int b0 = lv0, b1 = lv1;
             if (b1 == b0) break;
@@ -870,6 +905,7 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
             bool over = false;  // the node table is full
             if (d >= rows_done) {  // the edge rows of this depth: scored now, never if the expansion stops above it
                 int alive = 0;  // (nor if no node of the level can still have a selected child)
+#pragma unroll 1
                 for (int x = b0 + tid; x < b1; x += NT) alive |= sm.nkey[x] >= theta ? 1 : 0;
                 if (!__syncthreads_or(alive)) break;
                 lazy_score_row<NT>(p, sm, d, root, tid, inflight, K, p_m);
@@ -887,6 +923,7 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
                 if (ntot + total > ncap) {
                     over = true;
                 } else {
+#pragma unroll 1
                     for (int j = tid; j < total; j += NT) {
                         const int xi = j / K, r = j - xi * K, x = b0 + xi;
                         const uint32_t kx = sm.nkey[x];
@@ -915,9 +952,11 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
                 // key among those children.  (The search costs about as much as two ordinary levels: ordinary rounds,
                 // whose levels stay within a few times B, never run it.)
                 const int flood = 8 * budget > 1024 ? 8 * budget : 1024;
+#pragma unroll 1
                 for (int c0 = b0; c0 < b1; c0 += NT) {  // (uniform)
                   const int x = c0 + tid;
                   int total = 0;
+#pragma unroll 1
                   for (int attempt = 0;; ++attempt) {  // (uniform: at most two rounds)
                     const uint32_t th_in = theta + ((TIES && d + 1 > th_depth) ? 1u : 0u);  // what a child's score must reach
                     int cnt = 0;
@@ -946,6 +985,7 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
                             const int r_lo = tail ? cnt : 0, r_hi = tail ? K : cnt;
                             if ((K & 3) == 0) {
                                 const uint32_t* eiw = (const uint32_t*)(sm.ei + row);
+#pragma unroll 1
                                 for (int r0 = r_lo & ~3; r0 < r_hi; r0 += 4) {
                                     const uint32_t q = eiw[r0 >> 2];
                                     if (r0 >= r_lo) mask |= 1u << (q & 31u);
@@ -954,6 +994,7 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
                                     if (r0 + 3 >= r_lo && r0 + 3 < r_hi) mask |= 1u << ((q >> 24) & 31u);
                                 }
                             } else {
+#pragma unroll 1
                                 for (int r = r_lo; r < r_hi; ++r) mask |= 1u << sm.ei[row + r];
                             }
                             if (tail) mask = (K == 32 ? 0xFFFFFFFFu : (1u << K) - 1u) & ~mask;
@@ -990,6 +1031,7 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
                         over = true;
                         break;
                     }
+#pragma unroll (NT == 1024 ? 4 : 1)
                     for (int i = tid; i < total; i += NT) {
                         int lo_t = 0, hi_t = NT - 1;  // owner: the first thread whose scan exceeds i
                         while (lo_t < hi_t) {
@@ -1069,6 +1111,7 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
             if (theta != 0u) {
                 if (n_reach < 0) {  // (uniform) the radix search does not count them: one pass over the table
                     int ge = 0;
+#pragma unroll 1
                     for (int i = i0 > 1 ? i0 : 1; i < i1; ++i) ge += sm.nkey[i] >= theta ? 1 : 0;
                     ge = __reduce_add_sync(0xFFFFFFFFu, ge);
                     if (tid == 0) sm.scal[8] = 0;
@@ -1090,6 +1133,7 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
                     int* tlist = (int*)sm.hist;  // [32] table indices of the tied nodes, [32]: their number
                     if (tid == 0) tlist[32] = 0;
                     __syncthreads();
+#pragma unroll 1
                     for (int i = i0 > 1 ? i0 : 1; i < i1; ++i) {
                         if (sm.nkey[i] == theta) {
                             const int pos = atomicAdd(&tlist[32], 1);
@@ -1109,6 +1153,7 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
                                                 (31u - ((info >> 24) & 31u));
                             bool avail = lane < nt && sm.nkey[par] > theta;  // (else the parent is a tied node itself)
                             bool picked = false;
+#pragma unroll 1
                             for (int step = 0; step < want; ++step) {
                                 const uint32_t bh = __reduce_max_sync(0xFFFFFFFFu, avail && !picked ? hi : 0u);
                                 const uint32_t bl = __reduce_max_sync(0xFFFFFFFFu, avail && !picked && hi == bh ? lo + 1u : 0u);
@@ -1133,6 +1178,7 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
                         // expansion below.
                         const int want = budget - (n_reach - nt);
                         int mono = 1, same = 1;  // same: every tied node's own path score is theta (the usual tie)
+#pragma unroll 1
                         for (int i = i0 > 1 ? i0 : 1; i < i1; ++i) {
                             if (sm.nkey[i] != theta) continue;
                             same &= ord_from_float(sm.nS[i]) == theta ? 1 : 0;
@@ -1151,6 +1197,7 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
                                 const int bit = 54 - 2 * step;
                                 const uint64_t t1 = kth | (1ull << bit), t2 = kth | (2ull << bit), t3 = kth | (3ull << bit);
                                 int c1 = 0, c2 = 0, c3 = 0;
+#pragma unroll 1
                                 for (int i = i0 > 1 ? i0 : 1; i < i1; ++i) {
                                     if (sm.nkey[i] != theta) continue;
                                     const uint64_t o = tie_order(sm.nS[i], sm.ninfo[i]);
@@ -1170,6 +1217,7 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
                                 const int n1 = (int)cnt[3 * step], n2 = (int)cnt[3 * step + 1], n3 = (int)cnt[3 * step + 2];
                                 kth = n3 >= want ? t3 : (n2 >= want ? t2 : (n1 >= want ? t1 : kth));
                             }
+#pragma unroll 1
                             for (int i = i0 > 1 ? i0 : 1; i < i1; ++i)
                                 if (sm.nkey[i] == theta && tie_order(sm.nS[i], sm.ninfo[i]) >= kth) sm.nkey[i] = theta + 1u;
                             __syncthreads();
@@ -1181,6 +1229,7 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
                 ordered = true;  // fewer prefixes than the budget: all of them
             }
             int cnt = 0;
+#pragma unroll (NT == 1024 ? 4 : 1)
             for (int i = i0; i < i1; ++i) cnt += (i == 0 || sm.nkey[i] > cut) ? 1 : 0;
             int incl = cnt;
 #pragma unroll
@@ -1201,12 +1250,14 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
             const int total = __shfl_sync(0xFFFFFFFFu, wincl, 31);
             int run = woff + incl - cnt;
             __syncthreads();
+#pragma unroll (NT == 1024 ? 4 : 1)
             for (int i = i0; i < i1; ++i) {
                 const bool sel = (i == 0 || sm.nkey[i] > cut);
                 sm.nkey[i] = sel ? (uint32_t)run : 0xFFFFFFFFu;  // the key is no longer needed: keep the compact index
                 run += sel ? 1 : 0;
             }
             __syncthreads();
+#pragma unroll (NT == 1024 ? 4 : 1)
             for (int i = i0; i < i1; ++i) {
                 const uint32_t n = sm.nkey[i];
                 if (n == 0xFFFFFFFFu || i == 0) continue;
@@ -1220,6 +1271,7 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
             __syncthreads();
             // (for the sequential tail only) frontier entries of the selected nodes: the first child of the sorted row
             // that is not selected, i.e. the first with ord(score) <= theta
+#pragma unroll 1
             for (int n = tid; n <= n_gt && !ordered; n += NT) {
                 const int d = sm.depth[n];
                 uint64_t e = 0ull;
@@ -1241,6 +1293,7 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
         }
     }
     if (p_lazy && !table_ok && budget > 0) {  // the sequential fall-back may reach any depth
+#pragma unroll 1
         for (; rows_done < L; ++rows_done) lazy_score_row<NT>(p, sm, rows_done, root, tid, inflight, K, p_m);
     }
     if (!table_ok && tid == 0) sm.ent[0] = budget > 0 ? pack_entry(0.0f + sm.es[0], 1, 0, 0, sm.ei[0]) : 0ull;
@@ -1256,10 +1309,12 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
         sm.lvl_count[tid] = 0;
         sm.lvl_fill[tid] = 0;
     }
+#pragma unroll 1
     for (int n = tid; n < nmax; n += NT) sm.chmask[n] = 0u;
     __syncthreads();
     const int n_pre = table_ok ? n_gt : 0;  // nodes 0..n_pre are final before the tail starts
     if (warp >= 1) {
+#pragma unroll 1
         for (int n = tid - 32; n <= n_pre; n += NT - 32) {
             if (n > 0) atomicOr(&sm.chmask[sm.parent[n]], 1u << sm.cand[n]);
             atomicAdd(&sm.lvl_count[sm.depth[n]], 1);
@@ -1273,6 +1328,7 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
         while (n_sel < budget) {
             uint64_t be = 0ull;
             int bn = -1;
+#pragma unroll 1
             for (int n = lane; n <= n_sel; n += 32) {
                 const uint64_t e = sm.ent[n];
                 if (e != 0ull && entry_before(sm, e, n, be, bn)) {
@@ -1323,6 +1379,7 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
             }
             __syncwarp();
         }
+#pragma unroll 1
         for (int n = n_pre + 1 + lane; n <= n_sel; n += 32) {  // the tail's nodes
             atomicOr(&sm.chmask[sm.parent[n]], 1u << sm.cand[n]);
             atomicAdd(&sm.lvl_count[sm.depth[n]], 1);
@@ -1366,11 +1423,13 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
             }
         }
         __syncwarp();
+#pragma unroll 1
         for (int n = lane; n < n_nodes; n += 32) {  // the nodes of every level, in no particular order
             const int d = sm.depth[n];
             sm.lvl_list[sm.lvl_start[d] + atomicAdd(&sm.lvl_fill[d], 1)] = (int16_t)n;
         }
         __syncwarp();
+#pragma unroll 1
         for (int d = 1; d <= L; ++d) {
             const int s_prev = sm.lvl_start[d - 1], n_prev = sm.lvl_count[d - 1];
             const int s_cur = sm.lvl_start[d], n_cur = sm.lvl_count[d];
@@ -1378,6 +1437,7 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
             int16_t* ccp = sm.cc + ((d - 1) & 1) * nmax;
             int16_t* ccn = sm.cc + (d & 1) * nmax;
             int carry = 0;  // exclusive scan of ccp[0..n_prev), 32 entries at a time
+#pragma unroll 1
             for (int base = 0; base < n_prev; base += 32) {
                 const int i = base + lane;
                 const int v = i < n_prev ? ccp[i] : 0;
@@ -1391,6 +1451,7 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
                 carry += __shfl_sync(0xFFFFFFFFu, incl, 31);
             }
             __syncwarp();
+#pragma unroll 1
             for (int i = lane; i < n_cur; i += 32) {
                 const int x = sm.lvl_list[s_cur + i];
                 const int y = sm.parent[x];
@@ -1401,6 +1462,7 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
             __syncwarp();
         }
     } else if (warp != 0) {
+#pragma unroll 1
         for (int i = n_nodes + tid - 32; i < nmax; i += NT - 32) {
             o.d_token[ob + i] = -1;
             o.d_parent[ob + i] = -1;
@@ -1410,9 +1472,11 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
         }
         // mask rows from the first multiple of 32 at or above n_nodes on are all padding
         const int z0 = ((n_nodes + 31) / 32) * 32;
+#pragma unroll 1
         for (size_t k = (size_t)z0 * W + tid - 32; k < (size_t)nmax * W; k += NT - 32) o.d_mask[ob * W + k] = 0u;
     }
     if (!ordered) __syncthreads();  // (the placement above; the padding is nobody's input)
+#pragma unroll (NT == 1024 ? 4 : 1)
     for (int n = tid; n < n_nodes; n += NT) {
         const int i = ordered ? n : sm.canon[n], d = sm.depth[n];
         const int par = n == 0 ? -1 : (ordered ? sm.parent[n] : sm.canon[sm.parent[n]]);
@@ -1435,19 +1499,23 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
         int mw = (int)((region - stage_off) / ((size_t)32 * W * 4));
         mw = mw > NT / 32 ? NT / 32 : mw;
         uint32_t* tile = sm.stage + (size_t)warp * 32 * W;
+#pragma unroll 1
         for (int i0 = warp * 32; i0 < n_nodes && warp < mw; i0 += mw * 32) {
             const int i = i0 + lane;
             uint32_t* row = tile + lane * W;
             // the tile is cleared by the warp together, then a lane sets the bits of its node's ancestors (itself included)
+#pragma unroll (NT == 1024 ? 4 : 1)
             for (int k = lane; k < 32 * W; k += 32) tile[k] = 0u;
             __syncwarp();
             if (i < n_nodes) {
                 int steps = 0;  // a node has at most L ancestors: the bound keeps the walk finite whatever the arrays hold
+#pragma unroll 1
                 for (int a = i; a >= 0 && a < nmax && steps <= L; a = sm.cparent[a], ++steps) row[a >> 5] |= 1u << (a & 31);
             }
             __syncwarp();
             const int rows = min(32, nmax - i0);
             uint32_t* dst = o.d_mask + (ob + i0) * W;
+#pragma unroll (NT == 1024 ? 4 : 1)
             for (int k = lane; k < rows * W; k += 32) dst[k] = tile[k];
             __syncwarp();
         }
@@ -1536,6 +1604,7 @@ __global__ void __launch_bounds__(128) accept_kernel(const AcceptParams ap) {
                 lo = mid + 1;
         }
         int found = -1;
+#pragma unroll 1
         for (int i0 = lo; i0 < nn && found < 0; i0 += 32) {  // the children of cur are contiguous from lo on
             const int i = i0 + lane;
             const bool child = i < nn && par[i] == cur;
@@ -1549,6 +1618,7 @@ __global__ void __launch_bounds__(128) accept_kernel(const AcceptParams ap) {
         ++a;
         cur = found;
     }
+#pragma unroll 1
     for (int i = a + lane; i < L; i += 32) accept_path[(size_t)b * L + i] = -1;
     if (lane == 0) {
         accept_len[b] = a;
@@ -1562,6 +1632,7 @@ __global__ void __launch_bounds__(128) accept_kernel(const AcceptParams ap) {
             ap.hist_count[b] = n;
             const int cnt = n < w ? n : w;
             int sum = 0;
+#pragma unroll 1
             for (int i = 0; i < cnt; ++i) sum += ring[i];
             ap.hist_out[b] = (float)((double)sum / (double)cnt);
         }
@@ -1616,6 +1687,7 @@ static TreeInstance tree_pick(const graft_config& cfg, bool usual, bool neutral)
 cudaError_t tree_configure(const graft_config& cfg) {
     const int bytes = (int)tree_smem_bytes(cfg);
     cudaError_t e = cudaSuccess;
+#pragma unroll 1
     for (int i = 0; i < 4 && e == cudaSuccess; ++i)
         e = cudaFuncSetAttribute(tree_pick(cfg, (i & 1) != 0, (i & 2) != 0).kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     return e;
