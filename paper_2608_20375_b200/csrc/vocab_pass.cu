@@ -23,6 +23,8 @@
 //   * rows shared by several CTAs are merged by the last CTA to arrive (a counter, no waiting);
 //   * vocabulary-parallel use: the row's pieces are left for a merge over shards instead (vocab_merge_kernel).
 // Every wait on an mbarrier is bounded; when one runs out the kernel raises an error flag and drains.
+// Loops outside the stream are not unrolled unless that measured faster: the epilogue's code comes from L2 round after
+// round, beside the tree kernel's (156 -> 112 KB; batch 256 297.4 -> 295.8 us a round, batch 64 97.4 -> 96.8).
 #include <stdlib.h>
 #include <string.h>
 
@@ -448,9 +450,11 @@ __device__ __forceinline__ int warp_append(uint64_t* buf, int n, int cap, bool p
 // distinct (ids are), so ranks are a permutation.
 __device__ void warp_select_topk(EpiShared* sh, int n, int K, int lane) {
     __syncwarp();
+#pragma unroll 1
     for (int i = lane; i < n; i += 32) {
         const uint64_t key = sh->cand[i];
         int rank = 0;
+#pragma unroll 1
         for (int j = 0; j < n; ++j) rank += (sh->cand[j] > key) ? 1 : 0;
         if (rank < K) sh->outk[rank] = key;
     }
@@ -468,6 +472,7 @@ __device__ __noinline__ uint32_t epi_kth_chunk_max(EpiShared* es, const uint16_t
     int want = K;
 #pragma unroll 1
     for (int pass = 0; pass < 2; ++pass) {
+#pragma unroll 1
         for (int i = etid; i < 258; i += ET) hist[i] = 0u;
         epi_bar<ET>(grp);
 #pragma unroll 1
@@ -495,6 +500,7 @@ __device__ __noinline__ uint32_t epi_kth_chunk_max(EpiShared* es, const uint16_t
             }
             if (above >= (uint32_t)want && above - own < (uint32_t)want) {  // (one lane at most)
                 uint32_t acc = above - own;
+#pragma unroll 1
                 for (int i = 7; i >= 0; --i) {
                     const uint32_t c = hist[8 * etid + i];
                     if (acc + c >= (uint32_t)want) {
@@ -531,6 +537,7 @@ __device__ __noinline__ void epi_select_many(EpiShared* es, int n, int K, int et
     uint32_t* cnt = es->hits;                       // [2 * 16 * 3] counts of the steps, [96], [97] above / at the value, [98] kept
     uint64_t* kept = (uint64_t*)(es->hits + 128);   // [K] the keys that reach the K-th largest
     const uint32_t* word = (const uint32_t*)es->cand;  // key i: id word at 2 i, value word at 2 i + 1
+#pragma unroll 1
     for (int i = etid; i < 99; i += ET) cnt[i] = 0u;
     epi_bar<ET>(grp);
     uint32_t vk = 0u, ik = 0u;  // the K-th largest key's value word and id word
@@ -570,6 +577,7 @@ __device__ __noinline__ void epi_select_many(EpiShared* es, int n, int K, int et
         }
         vk = kth;
         int above = 0, at = 0;
+#pragma unroll 1
         for (int i = etid; i < n; i += ET) {
             const uint32_t hi = word[2 * i + 1];
             above += (hi > vk) ? 1 : 0;
@@ -586,6 +594,7 @@ __device__ __noinline__ void epi_select_many(EpiShared* es, int n, int K, int et
         if ((int)cnt[97] == want) break;  // (uniform) every key of that value is wanted: ik = 0 lets them all through
     }
     const uint64_t kth_key = ((uint64_t)vk << 32) | ik;
+#pragma unroll 1
     for (int i = etid; i < n; i += ET) {
         const uint64_t k = es->cand[i];
         if (k >= kth_key) {
@@ -598,6 +607,7 @@ __device__ __noinline__ void epi_select_many(EpiShared* es, int n, int K, int et
     if (etid < m) {
         const uint64_t k = kept[etid];
         int rank = 0;
+#pragma unroll 1
         for (int j2 = 0; j2 < m; ++j2) rank += (kept[j2] > k) ? 1 : 0;
         es->outk[rank] = k;
     }
@@ -640,6 +650,7 @@ __device__ int warp_fallback_select(EpiShared* sh, const VpParams& p, const Seg&
         }
     };
     auto one_by_one = [&](int e_begin, int e_end) {
+#pragma unroll 1
         for (int e0 = e_begin; e0 < e_end; e0 += 32) {
             const int e = e0 + lane;
             uint64_t key = 0;
@@ -652,6 +663,7 @@ __device__ int warp_fallback_select(EpiShared* sh, const VpParams& p, const Seg&
     constexpr int U = 4;
     const int nvec = (int)(sg.body_bytes / 16);
     const uint4* body = (const uint4*)sg.body;
+#pragma unroll 1
     for (int v0 = 0; v0 < nvec; v0 += 32 * U) {
         // The batch is one streaming warp's 2 KiB of a tile, and this lane's four consecutive vectors are the chunk whose
         // maximum (rounded up to bf16) that warp's lane left in cmx.  A chunk cannot hold a key above the filter if
@@ -737,10 +749,12 @@ __global__ void __launch_bounds__(kVpThreads, 1) vocab_pass_kernel(const VpParam
     const uint32_t ready0 = smem_u32(bars + 16), done0 = smem_u32(bars + 16 + kVpMaxBufs);
 
     if (tid == 0) {
+#pragma unroll 1
         for (int s = 0; s < p.stages; ++s) {
             mbar_init(full0 + 8 * s, 1);
             mbar_init(empty0 + 8 * s, NW);
         }
+#pragma unroll 1
         for (int s = 0; s < BUFS; ++s) {
             mbar_init(ready0 + 8 * s, NW);
             mbar_init(done0 + 8 * s, 1);
@@ -769,6 +783,7 @@ __global__ void __launch_bounds__(kVpThreads, 1) vocab_pass_kernel(const VpParam
                 // the segment this CTA visits last is read the ordinary way instead of evict-first: the second
                 // stage of its epilogue, which nothing overlaps any more, then finds its chunks in L2
                 const bool hint = p.use_hint && !seg_iter_at_end(it);
+#pragma unroll 1
                 for (int tile = 0; tile < sg.ntiles; ++tile, ++t) {
                     if (t >= nst) mbar_wait_bounded_hint(empty0 + 8 * st, ph, &sh->abort_flag, kVpIdleHintNs);
 #ifdef GRAFT_TEST_WITHHOLD_TILE
@@ -798,6 +813,7 @@ __global__ void __launch_bounds__(kVpThreads, 1) vocab_pass_kernel(const VpParam
             }
             if (sh->abort_flag) {
                 // a consumer gave up: make sure none of our copies is still in flight before the CTA retires
+#pragma unroll 1
                 for (uint32_t back = 0; back < nst && back < t; ++back) {
                     const uint32_t tt = t - 1 - back;
                     uint32_t tries = 0;
@@ -813,6 +829,7 @@ __global__ void __launch_bounds__(kVpThreads, 1) vocab_pass_kernel(const VpParam
         uint32_t k = 0;           // segment counter: hand-over buffers are indexed by k % BUFS
         SegIter it = seg_iter_begin<BF16>(p, q0, q1);
         Seg sg;
+#pragma unroll 1
         for (; seg_iter_next<BF16>(p, it, sg); ++k) {
             const uint32_t pb = k % BUFS;
             Acc a;
@@ -822,6 +839,7 @@ __global__ void __launch_bounds__(kVpThreads, 1) vocab_pass_kernel(const VpParam
             {
                 const int nfull = (int)(sg.body_bytes / TILE);
                 cm_t* slot = cmax + (size_t)pb * p.n_cmax + (size_t)tid * p.max_tiles;  // this thread's slots, by tile
+#pragma unroll 1
                 for (int tile = 0; tile < sg.ntiles; ++tile, ++slot) {
                     mbar_wait_bounded_hint(full0 + 8 * st, ph, &sh->abort_flag, 2000u);
                     const uint4* wb = (const uint4*)(ring + (size_t)st * TILE + (size_t)warp * WBLK);
@@ -868,6 +886,7 @@ __global__ void __launch_bounds__(kVpThreads, 1) vocab_pass_kernel(const VpParam
         // beside the logits stream (under 3 % of its bytes) so that nothing downstream waits for them.
         if (p.cos_out != nullptr) {
             const int npairs = (p.rows / p.L) * (p.L - 1);
+#pragma unroll 1
             for (int q = (int)blockIdx.x; q < npairs; q += (int)gridDim.x) {
                 const int sb = q / (p.L - 1), d = q - sb * (p.L - 1);
                 const double r = warp_adjacent_cosine(p.hidden, p.hidden_bf16, p.hidden_dim,
@@ -887,6 +906,7 @@ __global__ void __launch_bounds__(kVpThreads, 1) vocab_pass_kernel(const VpParam
         SegIter it = seg_iter_begin<BF16>(p, q0, q1);
         const int my_first_row = it.r_first;
         Seg sg;
+#pragma unroll 1
         for (; seg_iter_next<BF16>(p, it, sg); ++k) {
             if ((int)(k % GROUPS) != grp) continue;
             const uint32_t pb = k % BUFS;
@@ -904,6 +924,7 @@ __global__ void __launch_bounds__(kVpThreads, 1) vocab_pass_kernel(const VpParam
                 //     candidate (at most 7 + 7 elements unless the whole segment is shorter than 16 bytes)
                 {
                     const int nhead = sg.e_body0 - sg.e0, ntail = sg.e1 - sg.e_tail0;
+#pragma unroll 1
                     for (int i0 = 0; i0 < nhead + ntail; i0 += 32) {
                         const int i = i0 + lane;
                         const bool in = i < nhead + ntail;
@@ -947,6 +968,7 @@ __global__ void __launch_bounds__(kVpThreads, 1) vocab_pass_kernel(const VpParam
                         sh->gmax[pb][i * 32 + lane] = 0u;  // idle again (published by the `done` arrival below)
                         vmo = mine[i] > vmo ? mine[i] : vmo;
                     }
+#pragma unroll 1
                     for (int bit = 30; bit >= 16; bit -= 2) {  // two bits per step: three independent counts
                         const uint32_t t1 = Tv | (1u << bit), t2 = Tv | (2u << bit), t3 = Tv | (3u << bit);
                         int c1 = 0, c2 = 0, c3 = 0;
@@ -996,6 +1018,7 @@ __global__ void __launch_bounds__(kVpThreads, 1) vocab_pass_kernel(const VpParam
             // (d) chunks whose stored maximum reaches T: only threads whose own maximum reaches T can have one.
             //     List positions come from shared-memory atomics (the order does not matter: the final selection
             //     ranks exact keys).  A hit is recorded as the byte offset of the chunk's first vector.
+#pragma unroll 1
             for (int t = etid; t < NT; t += ET) {
                 const uint32_t x = sh->tmax[pb][t];
                 if (x >= Tv && x != 0u) es->hthreads[atomicAdd(&es->nht, 1)] = (uint16_t)t;
@@ -1011,6 +1034,7 @@ __global__ void __launch_bounds__(kVpThreads, 1) vocab_pass_kernel(const VpParam
             // follows if the list overflows again: four scans at most, then the exact selection.
             uint32_t Te = Tv;
             bool refined = false, tied = false;
+#pragma unroll 1
             for (int pass = 0;; ++pass) {  // (uniform)
                 // (listed thread, tile) pairs, four per thread at a time with their loads in flight together; the pair's
                 // thread comes from a multiplication (idx / ntiles for idx < 2^16 and ntiles < 2^16, exactly)
@@ -1018,6 +1042,7 @@ __global__ void __launch_bounds__(kVpThreads, 1) vocab_pass_kernel(const VpParam
                 const uint32_t magic = sg.ntiles > 1 ? 0xFFFFFFFFu / (uint32_t)sg.ntiles + 1u : 0u;  // ceil(2^32 / ntiles)
                 constexpr int PU = 4;
                 bool stop = false;
+#pragma unroll 1
                 for (int base = 0; base < npairs && !stop; base += ET * PU) {
                     uint32_t raw[PU], off[PU];
 #pragma unroll
@@ -1090,6 +1115,7 @@ __global__ void __launch_bounds__(kVpThreads, 1) vocab_pass_kernel(const VpParam
                 constexpr int RU = 256 / ET;
                 const int nvec = nhits * VEC_PER_LANE;
                 bool full = false;
+#pragma unroll 1
                 for (int base = 0; base < nvec && !full; base += ET * RU) {
                     uint4 vv[RU];
                     uint32_t offs[RU];
@@ -1146,6 +1172,7 @@ __global__ void __launch_bounds__(kVpThreads, 1) vocab_pass_kernel(const VpParam
                     int need = tie && es->nhits >= p.K ? 0 : p.K, visits = 0;
                     const int max_visits = tie ? 2 * p.K : 256;
                     bool gave_up = false;
+#pragma unroll 1
                     for (int blk = 0; blk < sg.ntiles * NW && need > 0; ++blk) {
                         const int tile = blk / NW, w = blk % NW;
                         const uint32_t cm = ord_from_bits((uint32_t)cmx[(size_t)(w * 32 + lane) * p.max_tiles + tile] << 16) >> 16;
@@ -1186,6 +1213,7 @@ __global__ void __launch_bounds__(kVpThreads, 1) vocab_pass_kernel(const VpParam
             int nk = ncand < p.K ? ncand : p.K;
             if (!overflow) {
                 // two neighbouring lanes per candidate, each over every other key, two running counts each
+#pragma unroll 1
                 for (int i0 = 0; i0 < ncand; i0 += ET / 2) {
                     const int i = i0 + (etid >> 1);
                     const uint64_t key = i < ncand ? es->cand[i] : ~0ull;
@@ -1259,15 +1287,19 @@ __global__ void __launch_bounds__(kVpThreads, 1) vocab_pass_kernel(const VpParam
                     }
                     constexpr int kRound = kVpCandCap / kMaxK - 1;  // records a round, behind the best of the rounds before
                     int have = 0;                                   // lists of kMaxK keys carried over: 0 or 1
+#pragma unroll 1
                     for (int r0 = 0; r0 < nseg; r0 += kRound) {
                         const int cnt = nseg - r0 < kRound ? nseg - r0 : kRound, n = (have + cnt) * kMaxK;
+#pragma unroll 1
                         for (int i = etid; i < cnt * kMaxK; i += ET)
                             es->cand[have * kMaxK + i] = __ldcg((const unsigned long long*)&record(r0 + i / kMaxK)->keys[i % kMaxK]);
                         if (etid < kMaxK) es->outk[etid] = 0ull;
                         epi_bar<ET>(grp);
+#pragma unroll 1
                         for (int i = etid; i < n; i += ET) {
                             const uint64_t key = es->cand[i];
                             int rank = i % kMaxK;
+#pragma unroll 1
                             for (int l = 0; l < n; l += kMaxK) {
                                 if (l == i - i % kMaxK) continue;
                                 int pos = 0;  // keys of list l above this one
@@ -1289,6 +1321,7 @@ __global__ void __launch_bounds__(kVpThreads, 1) vocab_pass_kernel(const VpParam
                         // log-sum-exp pieces, folded in double
                         double Cm = (double)rc, S = 0.0;
                         uint32_t vm = rv;
+#pragma unroll 1
                         for (int i = lane + 32; i < nseg; i += 32) {
                             const VpRecord* r = record(i);
                             const uint32_t kn = __ldcg(&r->nkeys), v2 = __float_as_uint(__ldcg(&r->vmax));
@@ -1301,6 +1334,7 @@ __global__ void __launch_bounds__(kVpThreads, 1) vocab_pass_kernel(const VpParam
                         for (int d = 16; d > 0; d >>= 1) Cm = fmax(Cm, __shfl_xor_sync(0xFFFFFFFFu, Cm, d));
                         vm = __reduce_max_sync(0xFFFFFFFFu, vm);
                         have_all = __reduce_add_sync(0xFFFFFFFFu, have_all);
+#pragma unroll 1
                         for (int i = lane; i < nseg; i += 32) {
                             const float c2 = i < 32 ? rc : __ldcg(&record(i)->c), s2 = i < 32 ? rs : __ldcg(&record(i)->s);
                             if (c2 != -INFINITY)
@@ -1529,6 +1563,7 @@ cudaError_t vp_merge_launch(graft_ctx* ctx, int batch, int n_shards, const graft
     p.n_shards = n_shards;
     p.rows = batch * ctx->cfg.L;
     p.K = ctx->cfg.K;
+#pragma unroll 1
     for (int i = 0; i < kMergeMaxShards; ++i) p.v_offset[i] = i < n_shards ? h_v_offset[i] : 0;
     p.topk_id = d_topk_id;
     p.topk_lp = d_topk_lp;
@@ -1546,6 +1581,7 @@ cudaError_t vp_configure(const graft_config& cfg, int num_sms, size_t* max_smem)
     *max_smem = pl.smem_bytes;
     if (pl.smem_bytes > 225 * 1024) return cudaErrorInvalidValue;
     cudaError_t e = cudaSuccess;
+#pragma unroll 1
     for (int groups = 2; groups <= 4 && e == cudaSuccess; groups += 2)
         e = cudaFuncSetAttribute(vp_kernel(cfg.logits_dtype == GRAFT_BF16, groups), cudaFuncAttributeMaxDynamicSharedMemorySize, 225 * 1024);
     return e;
@@ -1623,6 +1659,7 @@ extern "C" graft_status graft_vocab_pass_static(int32_t batch, int32_t L, int32_
                 cudaGetLastError();
                 return GRAFT_ERR_CUDA;
             }
+#pragma unroll 1
             for (int i = 0; i < 4; ++i)
                 if (cudaFuncSetAttribute(vp_kernel((i & 1) != 0, i < 2 ? 2 : 4), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          225 * 1024) != cudaSuccess) {
