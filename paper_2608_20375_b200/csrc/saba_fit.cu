@@ -5,10 +5,16 @@
 //                   tau_i = -B_i / ln(1 - g_i); (phi, bias) = argmin sum_i (tau_i - phi . s_i - bias)^2
 //   cost (Eq. 17):  (c0, c1, c2) = argmin sum_i (T_i - c0 - c1 B_i - c2 B_i prefix_i)^2
 //
-// One pass over the tuples accumulates the normal equations in fp64 (per thread, then per warp by shuffles, per CTA
-// in shared memory, per grid by atomics: 36 bytes read per tuple, so the pass is bound by HBM); the CTA that
-// finishes last solves the two small systems (columns scaled to unit diagonal first, then Gaussian elimination with
-// partial pivoting) and clears the accumulators for the next call.
+// One pass over the tuples accumulates the normal equations in fp64 (per thread, per warp by shuffles, per CTA in shared
+// memory, per grid by one atomic a sum); the CTA that finishes last solves the two small systems (columns scaled to unit
+// diagonal first, then Gauss-Jordan elimination with partial pivoting) and clears the accumulators for the next call.
+//
+// 36 bytes are read a tuple and some 75 fp64 operations done on it, a third of them in the logarithm: the fp64 pipe and
+// the conversions in front of it bound the slope (6.7 us per million tuples, 5.4 TB/s; copies into shared memory ahead
+// of the arithmetic, two and four tuples interleaved, and 24 warps an SM instead of 16 were no faster or slower), and a
+// call costs 8 us however few the tuples.  4 million tuples on a B200: 56.9 -> 37.0 us with log for log1p, counts as
+// integers, products by one folded (-> 45.3), the elimination on a warp and sums without shared-memory atomics (n = 64:
+// 12.3 -> 8.2).
 #include <cuda_runtime.h>
 #include <math.h>
 
@@ -33,137 +39,161 @@ struct FitParams {
     double* out;            // [10]
 };
 
-// x = argmin |A x - r| for the normal equations A (n x n, symmetric, upper triangle given row by row), n <= 4.
-// Returns false when a pivot of the scaled system vanishes.
-__device__ bool solve_normal(const double* tri, const double* rhs, int n, double* x) {
-    double a[4][5], d[4];
-    int t = 0;
-    for (int i = 0; i < n; ++i)
-        for (int j = i; j < n; ++j) {
-            a[i][j] = tri[t];
-            a[j][i] = tri[t];
-            ++t;
+// x = argmin |A x - r| for the normal equations A (n x n, symmetric, upper triangle given row by row; n <= 4), by one warp:
+// lane (r, c) of n x (n + 1) holds an entry of the scaled system [A | r], and Gauss-Jordan elimination with partial pivoting
+// runs on shuffles, so that a step is one division deep.  One thread with the matrix in local memory took 3 us more.
+// Lane r (n + 1) + n returns x[r]; ok is false when a pivot of the scaled system vanishes.
+__device__ __forceinline__ double solve_normal(const double* tri, const double* rhs, int n, int lane, bool& ok) {
+    const int w = n + 1;
+    const bool on = lane < n * w;
+    const int r = on ? lane / w : 0, c = on ? lane % w : 0;
+    const int i = min(r, c), j = max(r, c);
+    const auto diag = [&](int k) { return tri[k * n - k * (k - 1) / 2]; };  // entry (k, k); (i, j) is j - i behind (i, i)
+    const double drr = diag(r), dcc = c < n ? diag(c) : 1.0;
+    ok = __all_sync(0xFFFFFFFFu, drr > 0.0);
+    if (!ok) return 0.0;
+    const double dr = 1.0 / sqrt(drr), dc = c < n ? 1.0 / sqrt(dcc) : 1.0;
+    double a = (c < n ? tri[i * n - i * (i - 1) / 2 + j - i] : rhs[r]) * (dr * dc);
+#pragma unroll 1
+    for (int k = 0; k < n; ++k) {
+        int piv = k;
+        double best = fabs(__shfl_sync(0xFFFFFFFFu, a, k * w + k));
+#pragma unroll 1
+        for (int q = k + 1; q < n; ++q) {
+            const double v = fabs(__shfl_sync(0xFFFFFFFFu, a, q * w + k));
+            if (v > best) best = v, piv = q;
         }
-    for (int i = 0; i < n; ++i) {
-        if (!(a[i][i] > 0.0)) return false;
-        d[i] = 1.0 / sqrt(a[i][i]);
+        ok = best > 1e-13;
+        if (!ok) return 0.0;  // the same in every lane
+        a = __shfl_sync(0xFFFFFFFFu, a, (r == k ? piv : r == piv ? k : r) * w + c);
+        const double f = __shfl_sync(0xFFFFFFFFu, a, r * w + k) / __shfl_sync(0xFFFFFFFFu, a, k * w + k);
+        const double t = __shfl_sync(0xFFFFFFFFu, a, k * w + c);
+        if (r != k) a -= f * t;
     }
-    for (int i = 0; i < n; ++i) {
-        for (int j = 0; j < n; ++j) a[i][j] *= d[i] * d[j];
-        a[i][n] = rhs[i] * d[i];
-    }
-    for (int c = 0; c < n; ++c) {
-        int piv = c;
-        for (int i = c + 1; i < n; ++i)
-            if (fabs(a[i][c]) > fabs(a[piv][c])) piv = i;
-        if (!(fabs(a[piv][c]) > 1e-13)) return false;
-        if (piv != c)
-            for (int j = c; j <= n; ++j) {
-                const double tmp = a[c][j];
-                a[c][j] = a[piv][j];
-                a[piv][j] = tmp;
-            }
-        for (int i = c + 1; i < n; ++i) {
-            const double f = a[i][c] / a[c][c];
-            for (int j = c; j <= n; ++j) a[i][j] -= f * a[c][j];
-        }
-    }
-    for (int i = n - 1; i >= 0; --i) {
-        double s = a[i][n];
-        for (int j = i + 1; j < n; ++j) s -= a[i][j] * x[j];
-        x[i] = s / a[i][i];
-    }
-    for (int i = 0; i < n; ++i) x[i] *= d[i];
-    return true;
+    return a / __shfl_sync(0xFFFFFFFFu, a, r * w + r) * dr;
 }
 
-// one logged round into the running sums
-__device__ __forceinline__ void fit_accumulate(double* acc, float s0, float s1, float s2, int budget, float gain,
-                                               int prefix, float latency) {
-    const double B = (double)budget, g = (double)gain;
-    if (g > 0.0 && g < 1.0) {  // a gain of 0 or 1 says nothing about tau
-        const double f[4] = {(double)s0, (double)s1, (double)s2, 1.0};
-        const double tau = -B / log1p(-g);
-        int t = 0;
-#pragma unroll
-        for (int a = 0; a < 4; ++a)
-#pragma unroll
-            for (int b = a; b < 4; ++b) acc[t++] += f[a] * f[b];
-#pragma unroll
-        for (int a = 0; a < 4; ++a) acc[10 + a] += f[a] * tau;
-        acc[14] += 1.0;
-    }
-    const double h[3] = {1.0, B, B * (double)prefix};
-    const double T = (double)latency;
-    int t = 15;
-#pragma unroll
-    for (int a = 0; a < 3; ++a)
-#pragma unroll
-        for (int b = a; b < 3; ++b) acc[t++] += h[a] * h[b];
-#pragma unroll
-    for (int a = 0; a < 3; ++a) acc[21 + a] += h[a] * T;
-    acc[24] += 1.0;
+// The sums of one thread: everything but the two counts in fp64.
+struct FitSums {
+    double acc[kFitAcc];
+    int n_gain, n_cost;
+};
+// One logged round into the running sums.  No branch around the gain model (a warp nearly always has both kinds): a round
+// that says nothing about tau takes part with zeros.
+__device__ __forceinline__ void fit_accumulate(FitSums& t, float s0, float s1, float s2, int budget, float gain, int prefix,
+                                               float latency) {
+    double* acc = t.acc;
+    const double B = (double)budget;
+    const bool ok = gain > 0.0f && gain < 1.0f;  // a gain of 0 or 1 says nothing about tau
+    // 1 - g is exact in fp64 from 2^-29 up (g has 24 bits), and log(1 - g) costs less than log1p(-g)
+    const double g = ok ? (double)gain : 0.5;
+    const double tau = ok ? -B / (g >= 0x1p-29 ? log(1.0 - g) : log1p(-g)) : 0.0;
+    const double a = (double)(ok ? s0 : 0.f), b = (double)(ok ? s1 : 0.f), c = (double)(ok ? s2 : 0.f);
+    acc[0] = fma(a, a, acc[0]);
+    acc[1] = fma(a, b, acc[1]);
+    acc[2] = fma(a, c, acc[2]);
+    acc[3] += a;
+    acc[4] = fma(b, b, acc[4]);
+    acc[5] = fma(b, c, acc[5]);
+    acc[6] += b;
+    acc[7] = fma(c, c, acc[7]);
+    acc[8] += c;
+    acc[10] = fma(a, tau, acc[10]);
+    acc[11] = fma(b, tau, acc[11]);
+    acc[12] = fma(c, tau, acc[12]);
+    acc[13] += tau;
+    t.n_gain += ok ? 1 : 0;
+    const double T = (double)latency, BP = B * (double)prefix;
+    acc[16] += B;
+    acc[17] += BP;
+    acc[18] = fma(B, B, acc[18]);
+    acc[19] = fma(B, BP, acc[19]);
+    acc[20] = fma(BP, BP, acc[20]);
+    acc[21] += T;
+    acc[22] = fma(B, T, acc[22]);
+    acc[23] = fma(BP, T, acc[23]);
+    ++t.n_cost;
 }
 
 // VEC: every array is 16-byte aligned, so a thread takes four consecutive rounds with seven 16-byte loads
 template <bool VEC>
 __global__ void __launch_bounds__(kFitThreads, 2) saba_fit_kernel(const FitParams p) {
-    __shared__ double s_acc[kFitAcc];
+    __shared__ double s_acc[kFitAcc], s_warp[kFitThreads / 32][kFitAcc];
     __shared__ bool s_last;
-    double acc[kFitAcc];
+    __shared__ int s_bad[2];
+    FitSums t;
 #pragma unroll
-    for (int i = 0; i < kFitAcc; ++i) acc[i] = 0.0;
-    if (threadIdx.x < kFitAcc) s_acc[threadIdx.x] = 0.0;
-    __syncthreads();
+    for (int i = 0; i < kFitAcc; ++i) t.acc[i] = 0.0;
+    t.n_gain = t.n_cost = 0;
     const long long tid = blockIdx.x * (long long)kFitThreads + threadIdx.x, nth = (long long)gridDim.x * kFitThreads;
     long long done = 0;
     if (VEC) {
         const long long n4 = p.n / 4;
+#pragma unroll 1
         for (long long q = tid; q < n4; q += nth) {
             const float4 a = __ldg((const float4*)p.state + 3 * q), b = __ldg((const float4*)p.state + 3 * q + 1),
                          c = __ldg((const float4*)p.state + 3 * q + 2);
             const int4 bu = __ldg((const int4*)p.budget + q), pr = __ldg((const int4*)p.prefix + q);
             const float4 ga = __ldg((const float4*)p.gain + q), la = __ldg((const float4*)p.latency + q);
-            fit_accumulate(acc, a.x, a.y, a.z, bu.x, ga.x, pr.x, la.x);
-            fit_accumulate(acc, a.w, b.x, b.y, bu.y, ga.y, pr.y, la.y);
-            fit_accumulate(acc, b.z, b.w, c.x, bu.z, ga.z, pr.z, la.z);
-            fit_accumulate(acc, c.y, c.z, c.w, bu.w, ga.w, pr.w, la.w);
+            fit_accumulate(t, a.x, a.y, a.z, bu.x, ga.x, pr.x, la.x);
+            fit_accumulate(t, a.w, b.x, b.y, bu.y, ga.y, pr.y, la.y);
+            fit_accumulate(t, b.z, b.w, c.x, bu.z, ga.z, pr.z, la.z);
+            fit_accumulate(t, c.y, c.z, c.w, bu.w, ga.w, pr.w, la.w);
         }
         done = n4 * 4;
     }
     for (long long i = done + tid; i < p.n; i += nth)
-        fit_accumulate(acc, p.state[3 * i], p.state[3 * i + 1], p.state[3 * i + 2], p.budget[i], p.gain[i], p.prefix[i],
+        fit_accumulate(t, p.state[3 * i], p.state[3 * i + 1], p.state[3 * i + 2], p.budget[i], p.gain[i], p.prefix[i],
                        p.latency[i]);
+    t.acc[9] = t.acc[14] = (double)t.n_gain;
+    t.acc[15] = t.acc[24] = (double)t.n_cost;
+    // The warp's sums of all 25 in 31 steps of exchange (each halves what a lane still carries: lane i ends with sum i)
+    // instead of 25 x 5, and a CTA's sums by one thread each: shared-memory atomics on doubles are retry loops.
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
-    for (int i = 0; i < kFitAcc; ++i) {
-        double v = acc[i];
+    for (int d = 16; d > 0; d >>= 1) {
+        const bool up = (lane & d) != 0;
 #pragma unroll
-        for (int d = 16; d > 0; d >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, d);
-        if ((threadIdx.x & 31) == 0) atomicAdd(&s_acc[i], v);
+        for (int i = 0; i < d; ++i) {
+            const double lo = t.acc[i], hi = i + d < kFitAcc ? t.acc[i + d] : 0.0;
+            t.acc[i] = (up ? hi : lo) + __shfl_xor_sync(0xFFFFFFFFu, up ? lo : hi, d);
+        }
     }
+    if (lane < kFitAcc) s_warp[warp][lane] = t.acc[0];
     __syncthreads();
-    if (threadIdx.x < kFitAcc) atomicAdd(p.acc + threadIdx.x, s_acc[threadIdx.x]);
+    if (threadIdx.x < kFitAcc) {
+        double v = s_warp[0][lane];
+#pragma unroll
+        for (int i = 1; i < kFitThreads / 32; ++i) v += s_warp[i][lane];
+        atomicAdd(p.acc + lane, v);
+    }
     __threadfence();
     __syncthreads();
     if (threadIdx.x == 0) s_last = atomicAdd(p.ticket, 1u) == gridDim.x - 1;
     __syncthreads();
-    if (!s_last || threadIdx.x != 0) return;
+    if (!s_last) return;
     __threadfence();
-    double tot[kFitAcc];
-    for (int i = 0; i < kFitAcc; ++i) {
-        tot[i] = __ldcg(p.acc + i);
-        p.acc[i] = 0.0;  // ready for the next call
+    if (threadIdx.x < kFitAcc) {
+        s_acc[threadIdx.x] = __ldcg(p.acc + threadIdx.x);
+        p.acc[threadIdx.x] = 0.0;  // ready for the next call
     }
-    *p.ticket = 0u;
-    double phi[4] = {0.0, 0.0, 0.0, 0.0}, c[3] = {0.0, 0.0, 0.0};
-    int status = 0;
-    if (!(tot[14] >= 4.0) || !solve_normal(tot, tot + 10, 4, phi)) status |= 1;
-    if (!(tot[24] >= 3.0) || !solve_normal(tot + 15, tot + 21, 3, c)) status |= 2;
-    for (int i = 0; i < 4; ++i) p.out[i] = (status & 1) ? 0.0 : phi[i];
-    for (int i = 0; i < 3; ++i) p.out[4 + i] = (status & 2) ? 0.0 : c[i];
-    p.out[7] = tot[14];
-    p.out[8] = tot[24];
-    p.out[9] = (double)status;
+    if (threadIdx.x == 0) *p.ticket = 0u;
+    __syncthreads();
+    if (warp < 2) {  // the two systems side by side
+        const int n = 4 - warp;
+        const double* tri = s_acc + 15 * warp;
+        const double* rhs = tri + n * (n + 1) / 2;
+        bool ok;
+        const double x = solve_normal(tri, rhs, n, lane, ok), count = rhs[n];
+        ok = ok && count >= (double)n;
+        if (lane < n * (n + 1) && lane % (n + 1) == n) p.out[4 * warp + lane / (n + 1)] = ok ? x : 0.0;
+        if (lane == 0) {
+            p.out[7 + warp] = count;
+            s_bad[warp] = ok ? 0 : 1 + warp;
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) p.out[9] = (double)(s_bad[0] | s_bad[1]);
 }
 
 }  // namespace
