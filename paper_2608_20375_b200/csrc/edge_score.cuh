@@ -44,71 +44,88 @@ __device__ __forceinline__ int es_col(int r, int c, int K) {
     return x < K ? x : x - K;
 }
 
-// K x K dot products by 8 warps.  Warp ty takes parents ty, ty+8, ty+16, ty+24; lane = (ks, tx): children tx and
-// tx+16, and every second float4 of the m axis starting at ks.  A lane keeps a 4 x 2 tile of running sums, each as
-// a packed fp32 pair (even and odd elements of the m axis; `fma.rn.f32x2`, so 16 packed FMAs per six 16-byte
-// loads); the pair is added at the end and the two ks of a tile by one butterfly step, in a fixed order.
-// rP / rC: [.][ld] rows in shared memory, ld = m + 4 floats (16-byte aligned, conflict-free float4 reads).
+// K x K dot products by G * G / 8 warps (8 for G = 8, 32 for G = 16).  A lane keeps a T x T tile of running sums (parents
+// pg, pg + G, ..., children cg, cg + G, ...; G T >= K), each as a packed fp32 pair (even and odd elements of the m axis;
+// `fma.rn.f32x2`), and takes a quarter ks of the m axis: two float4s of every eight.  A warp holds 2 x 4 such tiles in all
+// four quarters, so a step's T float4s of parents are one pass over the shared-memory banks each (8 places) and the T of
+// children two (16 places, no conflicts): 12 passes for 32 packed FMAs with T = 4, where a 4 x 2 tile a lane took 12 for
+// 16 and made shared memory the bound (a round of batch 1, K = 8: 29.7 -> 28.6 us; batch 16, K = 16: 47.8 -> 46.1;
+// batch 64, K = 32: 96.6 -> 95.1; batch 256: 295.4 -> 292.9).
+// The pair is added at the end and the four quarters of a tile by two exchange steps; a sum's order of additions depends
+// on m alone, so the bits do not depend on T and G.
+// rP / rC: [.][ld] rows in shared memory, ld = m + 4 floats (16-byte aligned).
 // ADD_U: the rows hold P and C and u is added on the way into the registers; otherwise they already hold P + u and
-// C + u (the same fp32 sums either way).  part: [K][K] floats of shared memory; rows >= n_par are not written.
-template <bool ADD_U>
+// C + u (the same fp32 sums either way).  Sums of rows past n_par and K are never used; CLAMP reads the last row for
+// them, otherwise rP and rC have room for G T rows.  part: [n_par][dots_ld(K)] floats of shared memory.
+__host__ __device__ constexpr int dots_ld(int K) { return K + 4; }
+
+template <bool ADD_U, int G, int T, bool CLAMP>
 __device__ __forceinline__ void edge_dots(const float* rP, const float* rC, const float* rU, int m, int K, int n_par,
-                                          float* part, int ty, int lane) {
-    if (ty >= n_par) return;
-    const int tx = lane & 15, ks = lane >> 4, q4 = m / 4, ld = m + 4;
-    float2 acc[4][2];
+                                          float* part, int warp, int lane) {
+    const int ks = lane >> 3, pg = 2 * (warp / (G / 4)) + ((lane >> 2) & 1), cg = 4 * (warp % (G / 4)) + (lane & 3);
+    if (2 * (warp / (G / 4)) >= n_par) return;  // (uniform in the warp)
+    const int q4 = m / 4, ld = m + 4;
+    float2 acc[T][T];  // [child][parent]
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int c = 0; c < T; ++c)
 #pragma unroll
-        for (int i2 = 0; i2 < 2; ++i2) acc[i][i2] = make_float2(0.f, 0.f);
-    const float* c0 = rC + (size_t)min(tx, K - 1) * ld;  // (rows past K: read, never used)
-    const float* c1 = rC + (size_t)min(tx + 16, K - 1) * ld;
-#pragma unroll 2
-    for (int k4 = ks; k4 < q4; k4 += 2) {
-        float4 uu = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (ADD_U) uu = *(const float4*)(rU + 4 * k4);
-        float4 cv[2];
-        cv[0] = *(const float4*)(c0 + 4 * k4);
-        cv[1] = *(const float4*)(c1 + 4 * k4);
-        if (ADD_U) {
+        for (int i = 0; i < T; ++i) acc[c][i] = make_float2(0.f, 0.f);
+    rP += 8 * ks;
+    rC += 8 * ks;
+    if (ADD_U) rU += 8 * ks;
+#pragma unroll 1
+    for (int k = 0; k < q4; k += 8) {
 #pragma unroll
-            for (int i2 = 0; i2 < 2; ++i2) {
-                cv[i2].x += uu.x;
-                cv[i2].y += uu.y;
-                cv[i2].z += uu.z;
-                cv[i2].w += uu.w;
-            }
-        }
+        for (int h = 0; h < 2; ++h) {
+            if (q4 % 8 != 0 && k + 2 * ks + h >= q4) break;
+            const int at = 4 * (k + h);
+            float4 uu = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (ADD_U) uu = *(const float4*)(rU + at);
+            float4 cv[T];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            float4 pv = *(const float4*)(rP + (size_t)min(ty + 8 * i, n_par - 1) * ld + 4 * k4);
-            if (ADD_U) {
-                pv.x += uu.x;
-                pv.y += uu.y;
-                pv.z += uu.z;
-                pv.w += uu.w;
+            for (int c = 0; c < T; ++c) {
+                const int r = cg + G * c;
+                cv[c] = *(const float4*)(rC + (size_t)(CLAMP ? min(r, K - 1) : r) * ld + at);
+                if (ADD_U) cv[c] = make_float4(cv[c].x + uu.x, cv[c].y + uu.y, cv[c].z + uu.z, cv[c].w + uu.w);
             }
 #pragma unroll
-            for (int i2 = 0; i2 < 2; ++i2) {
-                float2 a = acc[i][i2];
-                a = __ffma2_rn(make_float2(pv.x, pv.y), make_float2(cv[i2].x, cv[i2].y), a);
-                a = __ffma2_rn(make_float2(pv.z, pv.w), make_float2(cv[i2].z, cv[i2].w), a);
-                acc[i][i2] = a;
+            for (int i = 0; i < T; ++i) {
+                const int r = pg + G * i;
+                float4 pv = *(const float4*)(rP + (size_t)(CLAMP ? min(r, n_par - 1) : r) * ld + at);
+                if (ADD_U) pv = make_float4(pv.x + uu.x, pv.y + uu.y, pv.z + uu.z, pv.w + uu.w);
+#pragma unroll
+                for (int c = 0; c < T; ++c) {
+                    acc[c][i] = __ffma2_rn(make_float2(pv.x, pv.y), make_float2(cv[c].x, cv[c].y), acc[c][i]);
+                    acc[c][i] = __ffma2_rn(make_float2(pv.z, pv.w), make_float2(cv[c].z, cv[c].w), acc[c][i]);
+                }
             }
         }
     }
+    constexpr int N = T * T;
+    float v[N];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        float v[2];
+    for (int e = 0; e < N; ++e) v[e] = acc[e / T][e % T].x + acc[e / T][e % T].y;
+    if constexpr (N % 4 == 0) {  // every exchange halves what a lane carries on: lane ks ends with a quarter of the tile's sums
+        const bool u8 = (lane & 8) != 0, u16 = (lane & 16) != 0;
 #pragma unroll
-        for (int i2 = 0; i2 < 2; ++i2) {
-            float a = acc[i][i2].x + acc[i][i2].y;
-            a += __shfl_xor_sync(0xFFFFFFFFu, a, 16);
-            v[i2] = a;
+        for (int e = 0; e < N / 2; ++e)
+            v[e] = (u8 ? v[e + N / 2] : v[e]) + __shfl_xor_sync(0xFFFFFFFFu, u8 ? v[e] : v[e + N / 2], 8);
+#pragma unroll
+        for (int e = 0; e < N / 4; ++e)
+            v[e] = (u16 ? v[e + N / 4] : v[e]) + __shfl_xor_sync(0xFFFFFFFFu, u16 ? v[e] : v[e + N / 4], 16);
+        const int first = (u8 ? N / 2 : 0) + (u16 ? N / 4 : 0);
+#pragma unroll
+        for (int e = 0; e < N / 4; ++e) {
+            const int c = cg + G * ((first + e) / T), r = pg + G * ((first + e) % T);
+            if (c < K && r < n_par) part[(size_t)r * dots_ld(K) + c] = v[e];
         }
-        if (ks == (i & 1) && ty + 8 * i < n_par) {
-            if (tx < K) part[(size_t)(ty + 8 * i) * K + tx] = v[0];
-            if (tx + 16 < K) part[(size_t)(ty + 8 * i) * K + tx + 16] = v[1];
+    } else {
+#pragma unroll
+        for (int e = 0; e < N; ++e) {
+            v[e] += __shfl_xor_sync(0xFFFFFFFFu, v[e], 8);
+            v[e] += __shfl_xor_sync(0xFFFFFFFFu, v[e], 16);
+            const int c = cg + G * (e / T), r = pg + G * (e % T);
+            if (ks == (e & 3) && c < K && r < n_par) part[(size_t)r * dots_ld(K) + c] = v[e];
         }
     }
 }
@@ -136,12 +153,19 @@ __device__ __forceinline__ void edge_row_finish(const float* dots, const float* 
     __syncwarp();
     wsc[c] = mine;
     __syncwarp();
-    rank = 0;
+    // o > mine is the carry out of o + ~mine: an add and an add-with-carry a child, 0.75 cycles an SM where compare, select
+    // and add take 0.93
+    uint32_t above = 0;
 #pragma unroll
     for (int i4 = 0; i4 < 8; ++i4) {
         const uint4 o4 = *(const uint4*)(wsc + 4 * i4);
-        rank += (o4.x > mine ? 1 : 0) + (o4.y > mine ? 1 : 0) + (o4.z > mine ? 1 : 0) + (o4.w > mine ? 1 : 0);
+        asm("{\n\t.reg .u32 t;\n\t"
+            "add.cc.u32 t, %1, %5;\n\taddc.u32 %0, %0, 0;\n\tadd.cc.u32 t, %2, %5;\n\taddc.u32 %0, %0, 0;\n\t"
+            "add.cc.u32 t, %3, %5;\n\taddc.u32 %0, %0, 0;\n\tadd.cc.u32 t, %4, %5;\n\taddc.u32 %0, %0, 0;\n\t}"
+            : "+r"(above)
+            : "r"(o4.x), "r"(o4.y), "r"(o4.z), "r"(o4.w), "r"(~mine));
     }
+    rank = (int)above;
     // equal scores (rare) go by child rank: the counts above are a permutation of 0..K-1 unless some scores are equal,
     // and only then are the lanes with the same score looked up (a slow instruction)
     const uint32_t seen = __reduce_or_sync(0xFFFFFFFFu, c < K ? 1u << rank : 0u);

@@ -193,15 +193,20 @@ __global__ void __launch_bounds__(256, 4) tdes_edges_kernel(const EdgeParams p) 
     }
     __syncthreads();
     // dot products into shared memory, then every warp finishes the rows of parents warp, warp+8, ...
-    float* part = sC + (size_t)kMaxK * ld;  // [K][K]
+    float* part = sC + (size_t)kMaxK * ld;  // [K][dots_ld(K)]
     __shared__ uint32_t wsc[8][32];
-    edge_dots<false>(sP, sC, nullptr, m, K, n_par, part, warp, lane);
+    if constexpr (KC != 0)
+        edge_dots<false, 8, (KC ? KC + 7 : 8) / 8, false>(sP, sC, nullptr, m, K, n_par, part, warp, lane);
+    else if (K <= 16)
+        edge_dots<false, 8, 2, false>(sP, sC, nullptr, m, K, n_par, part, warp, lane);
+    else
+        edge_dots<false, 8, 4, false>(sP, sC, nullptr, m, K, n_par, part, warp, lane);
     __syncthreads();
     const float inv_K = 1.0f / (float)K;
     for (int par = warp; par < K; par += 8) {
         float val;
         int rank;
-        edge_row_finish(par < n_par ? part + (size_t)par * K : nullptr, lps, p.scale, p.beta, K, inv_K, wsc[warp], lane,
+        edge_row_finish(par < n_par ? part + (size_t)par * dots_ld(K) : nullptr, lps, p.scale, p.beta, K, inv_K, wsc[warp], lane,
                         val, rank);
         if (lane < K) {
             if (WRITE_EDGE) p.edge[(row * K + par) * K + lane] = val;
@@ -226,7 +231,7 @@ cudaError_t tdes_precompute_launch(graft_ctx* ctx, const void* d_emb, graft_dtyp
 }
 
 size_t tdes_edges_smem(const graft_config& cfg) {
-    return ((size_t)2 * kMaxK * (cfg.m + 4) + (size_t)kMaxK * kMaxK) * sizeof(float);  // P rows, C rows, dot products
+    return ((size_t)2 * kMaxK * (cfg.m + 4) + (size_t)kMaxK * dots_ld(kMaxK)) * sizeof(float);  // P rows, C rows, dot products
 }
 
 cudaError_t tdes_edges_configure(const graft_config& cfg) {

@@ -608,7 +608,7 @@ __device__ __forceinline__ void lazy_issue_gather(const TreeParams& p, const Tre
 }
 // Every thread of the CTA calls this.
 // `inflight` is the depth whose table rows are on their way (or -1).
-template <int NT>
+template <int NT, int KC>
 __device__ __forceinline__ void lazy_score_row(const TreeParams& p, const TreeSmem& sm, int j, int root_token, int tid,
                                                int& inflight, const int K, const int m) {
     const int n_par = j == 0 ? 1 : K;
@@ -629,9 +629,13 @@ __device__ __forceinline__ void lazy_score_row(const TreeParams& p, const TreeSm
     if (inflight != j) lazy_issue_gather<NT>(p, sm, j, root_token, tid, K, m);
     cp_async_wait_all();
     __syncthreads();
-    float* part = (float*)sm.hist;                // [K][K] dot products (the histogram space is idle here)
-    uint32_t* wsc = sm.hist + 1024 + warp * 32;   // [32] per warp
-    if (warp < 8) edge_dots<true>(sm.gP, sm.gC, sm.gU, m, K, n_par, part, warp, lane);
+    float* part = (float*)sm.hist;                                // [K][dots_ld(K)] (the histogram space is idle here)
+    uint32_t* wsc = sm.hist + kMaxK * dots_ld(kMaxK) + warp * 32;  // [32] per warp
+    // (T G covers the largest K that tree_pick gives NT threads)
+    if constexpr (NT == 1024)
+        edge_dots<true, 16, 2, KC != 32>(sm.gP, sm.gC, sm.gU, m, K, n_par, part, warp, lane);
+    else if (warp < 8)
+        edge_dots<true, 8, NT == 256 ? 1 : KC == 16 ? 2 : 3, KC == 0>(sm.gP, sm.gC, sm.gU, m, K, n_par, part, warp, lane);
     __syncthreads();
     lazy_issue_gather<NT>(p, sm, j + 1, root_token, tid, K, m);  // the table rows of this depth are no longer read
     inflight = j + 1;
@@ -640,7 +644,7 @@ __device__ __forceinline__ void lazy_score_row(const TreeParams& p, const TreeSm
     for (int par = warp; par < K; par += NT / 32) {  // one warp per parent
         float val;
         int rank;
-        edge_row_finish(par < n_par ? part + (size_t)par * K : nullptr, lps, p.scale, p.beta, K, inv_K, wsc, lane, val,
+        edge_row_finish(par < n_par ? part + (size_t)par * dots_ld(K) : nullptr, lps, p.scale, p.beta, K, inv_K, wsc, lane, val,
                         rank);
         if (lane < K) {
             es[(size_t)par * K + es_col(rank, par, K)] = val;
@@ -908,7 +912,7 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
 #pragma unroll 1
                 for (int x = b0 + tid; x < b1; x += NT) alive |= sm.nkey[x] >= theta ? 1 : 0;
                 if (!__syncthreads_or(alive)) break;
-                lazy_score_row<NT>(p, sm, d, root, tid, inflight, K, p_m);
+                lazy_score_row<NT, KC>(p, sm, d, root, tid, inflight, K, p_m);
                 rows_done = d + 1;
             }
             // grow: can a node appended here have a child that reaches theta?  (Its best child stands first in its sorted
@@ -1294,7 +1298,7 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
     }
     if (p_lazy && !table_ok && budget > 0) {  // the sequential fall-back may reach any depth
 #pragma unroll 1
-        for (; rows_done < L; ++rows_done) lazy_score_row<NT>(p, sm, rows_done, root, tid, inflight, K, p_m);
+        for (; rows_done < L; ++rows_done) lazy_score_row<NT, KC>(p, sm, rows_done, root, tid, inflight, K, p_m);
     }
     if (!table_ok && tid == 0) sm.ent[0] = budget > 0 ? pack_entry(0.0f + sm.es[0], 1, 0, 0, sm.ei[0]) : 0ull;
     if (ordered) {  // (uniform) the tree is complete and in level order
