@@ -514,14 +514,14 @@ __device__ uint32_t cta_finish_select(const TreeSmem& sm, const uint32_t* keys, 
     }
     const int remaining = st.rem;
 #pragma unroll 1
-    for (int i = tid; i < n; i += NT) {
+    for (int i = tid >> 5; i < n; i += NT / 32) {  // a warp per key, a lane per key it is compared with
         const uint32_t k = list[i];
         int gt = 0, ge = 0;
 #pragma unroll 1
-        for (int j = 0; j < n; ++j) {
-            const uint32_t o = list[j];
-            gt += o > k ? 1 : 0;
-            ge += o >= k ? 1 : 0;
+        for (int j = tid & 31; j - (tid & 31) < n; j += 32) {
+            const uint32_t o = j < n ? list[j] : 0u;  // (0 is below every key)
+            gt += __popc(__ballot_sync(0xFFFFFFFFu, o > k));
+            ge += __popc(__ballot_sync(0xFFFFFFFFu, o >= k));
         }
         if (gt < remaining && remaining <= ge) {  // (every writer writes the same values)
             sm.scal[6] = (int)k;
@@ -901,6 +901,10 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
         // (the bounds of the level being expanded and the end of the table are the same in every thread: no thread has to
         // publish them, and a level costs three barriers -- two in the scan, one at its end)
         int lv0 = spec ? 1 + K : 0, lv1 = spec ? 1 + K + K * K : 1;
+        // Where few nodes of a level can have children, `grp` lanes take one node's sorted row together, NT / grp nodes (32
+        // at most) at once; n_grow bounds the number of such nodes of the level being expanded (> NT: unknown).
+        const int grp = NT == 256 ? 8 : (NT == 512 && K <= 16) ? 16 : 32;
+        int n_grow = NT + 1;
 #pragma unroll 1
         for (int d = spec ? 2 : 0; d < L; ++d) {
             const int b0 = lv0, b1 = lv1;
@@ -940,6 +944,69 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
                         sm.ninfo[at] = (uint32_t)x | ((uint32_t)c << 13) | ((uint32_t)(d + 1) << 18) | ((uint32_t)r << 24);
                     }
                     lvl_end = ntot + total;
+                }
+            } else if (n_grow <= NT / grp) {
+                // The last levels of nearly every tree: a thread per node finds the nodes that can have children by the best
+                // entry of their rows, then a group of lanes takes one of them each, a lane per entry.  No search along a
+                // row and none for a child's node: FAST_BEFORE_AFTER
+                int* wcnt = (int*)sm.hist;       // [32] such nodes per warp
+                int* list = (int*)sm.hist + 32;  // [32] those nodes in the order of the level, -1: none
+                int* ccnt = (int*)sm.hist + 64;  // [32] their children that reach theta
+                const uint32_t th_in = theta + ((TIES && d + 1 > th_depth) ? 1u : 0u);
+                const int x = b0 + tid;  // (a level of at most NT nodes)
+                bool alive = false;
+                if (x < b1 && sm.nkey[x] >= theta) {
+                    const int cx = (int)((sm.ninfo[x] >> 13) & 31u);
+                    alive = ord_from_float(sm.nS[x] + sm.es[(d * K + cx) * K + cx]) >= th_in;  // (entry 0: column cx)
+                }
+                const uint32_t am = __ballot_sync(0xFFFFFFFFu, alive);
+                if (lane == 0) wcnt[warp] = __popc(am);
+                if (tid < 32) list[tid] = -1;
+                __syncthreads();
+                const int at_list = (int)__reduce_add_sync(0xFFFFFFFFu, lane < warp ? (uint32_t)wcnt[lane] : 0u) +
+                                    __popc(am & ((1u << lane) - 1u));
+                if (alive && at_list < 32) list[at_list] = x;
+                __syncthreads();
+                const int nd = tid / grp, r = tid % grp, xo = list[nd];
+                int c = 0;
+                uint32_t kx = 0u, oc = 0u;
+                float sc = 0.0f;
+                bool take = false;
+                if (xo >= 0 && r < K) {
+                    kx = sm.nkey[xo];
+                    const int co = (int)((sm.ninfo[xo] >> 13) & 31u), row = (d * K + co) * K;
+                    sc = sm.nS[xo] + sm.es[row + es_col(r, co, K)];
+                    oc = ord_from_float(sc);
+                    c = sm.ei[row + r];
+                    take = oc >= th_in;
+                }
+                uint32_t mask = take ? 1u << c : 0u;  // the candidate ranks of the node's children
+                if (grp == 32) {
+                    mask = __reduce_or_sync(0xFFFFFFFFu, mask);
+                } else {
+#pragma unroll 1
+                    for (int o2 = grp / 2; o2 > 0; o2 >>= 1) mask |= __shfl_xor_sync(0xFFFFFFFFu, mask, o2);
+                }
+                if (r == 0) ccnt[nd] = __popc(mask);
+                __syncthreads();
+                const int v = lane < NT / grp ? ccnt[lane] : 0;
+                int incl = v;
+#pragma unroll
+                for (int o2 = 1; o2 < 32; o2 <<= 1) {
+                    const int t = __shfl_up_sync(0xFFFFFFFFu, incl, o2);
+                    if (lane >= o2) incl += t;
+                }
+                const int first = __shfl_sync(0xFFFFFFFFu, incl - v, nd);
+                lvl_end = ntot + __shfl_sync(0xFFFFFFFFu, incl, 31);
+                if (lvl_end > ncap) {  // (uniform)
+                    over = true;
+                } else if (take) {
+                    if (d + 1 < L)  // (a row that is not scored yet: grow)
+                        grow = d + 1 >= rows_done || ord_from_float(sc + sm.es[((d + 1) * K + c) * K + c]) >= theta ? 1 : 0;
+                    const int at = ntot + first + __popc(mask & ((1u << c) - 1u));
+                    sm.nkey[at] = oc < kx ? oc : kx;
+                    sm.nS[at] = sc;
+                    sm.ninfo[at] = (uint32_t)xo | ((uint32_t)c << 13) | ((uint32_t)(d + 1) << 18) | ((uint32_t)r << 24);
                 }
             } else {
                 // The children that can still matter are a prefix of a node's sorted row (scores only fall along the
@@ -1070,7 +1137,7 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
                 }
                 lvl_end = cur;
             }
-            const int any_grow = __syncthreads_or(grow);  // (the level's nodes are in the table for every thread)
+            const int grown = __syncthreads_count(grow);  // (the level's nodes are in the table for every thread)
             const int nt = lvl_end;
             if (over) {
                 table_ok = false;
@@ -1080,10 +1147,11 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
             lv0 = ntot;
             lv1 = nt;
             ntot = nt;
-            if (!any_grow) break;  // no node of the new level can have a child in the tree
+            if (!grown) break;  // no node of the new level can have a child in the tree
+            n_grow = b1 - b0 <= NT && lv1 - lv0 <= NT ? grown : NT + 1;  // (a thread appended one node of the level at most)
             // theta only has to be a lower bound of its final value while the levels are built (it prunes), so
             // the exact B-th largest key is recomputed only when the table has grown noticeably
-            if (ntot - 1 >= budget && (theta == 0u || ntot - n_at_select >= ntot / 8)) {
+            if (ntot - 1 >= budget && (theta == 0u || ntot - n_at_select >= ntot / 4)) {
                 sel_top = 0.0f + sm.es[0];  // the root's best child
                 theta = cta_select_bucket<NT>(sm, sm.nkey, 1, ntot, budget, sel_top, sel, tid);  // a lower bound
                 if (TIES) {
