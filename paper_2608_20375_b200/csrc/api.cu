@@ -398,7 +398,9 @@ graft_status graft_build_trees(graft_ctx* ctx, int32_t batch, const void* d_logi
     // caller asks for the score array); the tree kernel scores deeper rows itself if an expansion gets that far.
     // The depth-0 CTA of each sequence in that kernel also works out the sequence's budget (Sec. 3.3), which the tree
     // kernel then only reads; without an edge-score kernel the tree kernel does it itself.
-    const int rows = out->d_edge ? ctx->cfg.L : ctx->edge_rows;
+    // Without edge scores (beta = 0) nothing needs that kernel: the tree kernel lays the rows out from log q.
+    const bool neutral = ctx->cfg.beta == 0.0f || !ctx->tdes_set;
+    const int rows = out->d_edge ? ctx->cfg.L : neutral ? 0 : ctx->edge_rows;
     if (rows > 0 && tdes_edges_launch(ctx, batch, ids, lps, d_root_token, ctx->w_row_status, edge, ctx->w_esort,
                                       ctx->w_eidx, rows, ctx->w_saba, d_hist, d_prefix_len, d_fixed_budget,
                                       st) != cudaSuccess)

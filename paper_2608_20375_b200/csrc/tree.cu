@@ -69,7 +69,6 @@ struct TreeSmem {
     int* lvl_count;      // [kMaxL + 2]
     int* lvl_start;      // [kMaxL + 2]
     int* lvl_fill;       // [kMaxL + 2]
-    double* cosv;        // [kMaxL]  adjacent-position cosines r_d (Eq. 15)
     // on-demand edge scoring only:
     float* gP;           // [K][m+4]  gathered parent rows P[token]
     float* gC;           // [K][m+4]  gathered child rows C[token]
@@ -95,7 +94,7 @@ __host__ __device__ inline size_t tree_smem_layout(int L, int K, int nmax, int n
     size_t o_ent = take((size_t)nmax * 8), o_S = take((size_t)nmax * 4), o_chm = take((size_t)nmax * 4),
            o_par = take((size_t)nmax * 2), o_can = take((size_t)nmax * 2), o_cp = take((size_t)nmax * 2),
            o_cand = take(nmax), o_dep = take(nmax), o_hist = take(2208 * 4), o_lc = take((kMaxL + 2) * 4),
-           o_ls = take((kMaxL + 2) * 4), o_lf = take((kMaxL + 2) * 4), o_sc = take(16 * 4), o_cos = take(kMaxL * 8);
+           o_ls = take((kMaxL + 2) * 4), o_lf = take((kMaxL + 2) * 4), o_sc = take(16 * 4);
     size_t o_gp = 0, o_gc = 0, o_gu = 0, o_tk = 0, o_lp = 0;
     if (lazy_m > 0) {
         o_gp = take((size_t)K * (lazy_m + 4) * 4);
@@ -126,7 +125,6 @@ __host__ __device__ inline size_t tree_smem_layout(int L, int K, int nmax, int n
         s->lvl_start = (int*)(base + o_ls);
         s->lvl_fill = (int*)(base + o_lf);
         s->scal = (int*)(base + o_sc);
-        s->cosv = (double*)(base + o_cos);
         s->gP = (float*)(base + o_gp);
         s->gC = (float*)(base + o_gc);
         s->gU = (float*)(base + o_gu);
@@ -664,7 +662,9 @@ __device__ __forceinline__ void lazy_score_row(const TreeParams& p, const TreeSm
 // configured workloads' K = 32, m = 128: every index computation with K becomes a shift), or 0: taken from the parameters
 // FAST: the usual round is known at compile time as well -- the budget comes from the edge-score kernel (no SABA
 // arithmetic in this instance) and deeper rows are scored on demand
-// TIES: the instance for rounds without edge scores (beta = 0), where exactly equal probabilities make hundreds of
+// TIES: the instance for rounds without edge scores (beta = 0).  It lays the rows out itself (no edge-score kernel ran, and
+// the budget is worked out here as well: two launches a round less its gap; batch 37, K = 11: 48.0 -> 41.0 us a round) and
+// expects that exactly equal probabilities make hundreds of
 // prefixes tie with the B-th largest key: it resolves them in parallel (the other instances leave more than 32 tied
 // keys to the sequential expansion; with edge scores in the keys such ties do not occur in tens, and the code's mere
 // presence costs this register-bound kernel 0.4 us a round)
@@ -687,14 +687,14 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
     // (they land while warp 0 works out the budget), plain loads otherwise
     __shared__ __align__(8) uint64_t rows_bar;
     __shared__ int rows_abort;
-    const int rows_pre = p.rows_pre;
+    const int rows_pre = TIES ? L : p.rows_pre;
     const int ne = rows_pre * K * K;  // entries that come from the edge-score kernel for every sequence
     // (a bulk copy's source and size are multiples of 16 bytes: the child ranks are bytes, so the entries copied and the
     // entries between two sequences both have to be multiples of 16 -- L = 11, K = 10 with 8 rows ahead has 800 and 1100)
-    const bool bulk = ne > 0 && (ne % 16) == 0 && (L * K * K) % 16 == 0;
+    const bool bulk = !TIES && ne > 0 && (ne % 16) == 0 && (L * K * K) % 16 == 0;
     // the prologue's loads from global memory are all issued before the first of them is used: one round trip
     const int root = p.root_token[b];
-    const float lp_top = p.rows_adaptive ? deep_tree_load(p.topk_lp + (size_t)b * L * K, L, K) : 0.f;
+    const float lp_top = !TIES && p.rows_adaptive ? deep_tree_load(p.topk_lp + (size_t)b * L * K, L, K) : 0.f;
     SabaResult pre_r;
     pre_r.budget = 0;
     pre_r.status = 0;
@@ -706,7 +706,7 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
 #pragma unroll
     for (int q = 0; q < LZ; ++q) {
         const int i = tid + q * NT;
-        if (p_lazy && i < L * K) {
+        if (!TIES && p_lazy && i < L * K) {
             lz_tok[q] = p.topk_id[(size_t)b * L * K + i];
             lz_lp[q] = p.topk_lp[(size_t)b * L * K + i];
         }
@@ -735,14 +735,14 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
                 tma_load_1d(smem_u32((char*)sm.ei + off), g_ei + off, bytes, smem_u32(&rows_bar));
             }
         }
-    } else {
+    } else if (!TIES) {
 #pragma unroll 1
         for (int i = tid; i < ne; i += NT) {
             sm.es[i] = p.esort[seq_e + i];
             sm.ei[i] = p.eidx[seq_e + i];
         }
     }
-    if (p_lazy) {  // the candidates of every depth, for the rows that may have to be scored here
+    if (!TIES && p_lazy) {  // the candidates of every depth, for the rows that may have to be scored here
 #pragma unroll
         for (int q = 0; q < LZ; ++q) {
             const int i = tid + q * NT;
@@ -759,7 +759,7 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
     }
     // a sequence whose tree will run deep had its deeper rows scored by the edge-score kernel as well (they are needed
     // several levels from here: plain loads, consumed after many barriers)
-    if (p.rows_adaptive && deep_tree_decide(lp_top, L)) {  // (uniform)
+    if (!TIES && p.rows_adaptive && deep_tree_decide(lp_top, L)) {  // (uniform)
 #pragma unroll 1
         for (int i = ne + tid; i < L * K * K; i += NT) {
             sm.es[i] = p.esort[seq_e + i];
@@ -767,15 +767,37 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
         }
         rows_done = L;
     }
-    // adjacent-position cosines r_d = cos(h_d, h_{d+1}) (Eq. 15): written by the vocab pass
-    if (!FAST && p.use_saba && !p.saba_pre && tid < L - 1) sm.cosv[tid] = p.cos_pre[(size_t)b * L + tid];
-    __syncthreads();
+    if (!TIES) __syncthreads();
+    if (TIES && warp >= 1) {  // (warp 0 is at the budget from the start)
+        // no edge scores: every row of a position is its log q, which is ordered by rank already
+        const float* lps = p.topk_lp + (size_t)b * L * K;
+        if (p_lazy) {
+#pragma unroll 1
+            for (int i = tid - 32; i < L * K; i += NT - 32) {
+                const int32_t tok = p.topk_id[(size_t)b * L * K + i];
+                const float lp = lps[i];
+                sm.tokid[i] = tok;
+                sm.lpv[i] = lp;
+            }
+            named_bar_sync(1, NT - 32);
+            lps = sm.lpv;
+        }
+#pragma unroll 1
+        for (int rw = warp - 1; rw < L * K; rw += NT / 32 - 1) {  // (position, parent)
+            const int j = rw / K, par = rw - j * K;
+            if (lane < K) {
+                sm.es[rw * K + es_col(lane, par, K)] = lps[j * K + lane];
+                sm.ei[rw * K + lane] = (uint8_t)lane;
+            }
+        }
+        named_bar_sync(1, NT - 32);
+    }
     // While warp 0 works out the budget, the other warps expand levels 0 and 1 in full (1 + K + K^2 nodes), which
     // needs no budget: with fewer than B nodes in the table every child is appended anyway, and if B is smaller
     // than that the extra nodes only fall below the threshold found afterwards.
-    const bool spec = bulk && rows_pre >= 2 && L >= 2 && 1 + K + K * K <= ncap;
+    const bool spec = rows_pre >= 2 && L >= 2 && 1 + K + K * K <= ncap;
     if (spec && warp >= 1) {
-        mbar_wait_bounded(smem_u32(&rows_bar), 0, &rows_abort);
+        if (bulk) mbar_wait_bounded(smem_u32(&rows_bar), 0, &rows_abort);
         const int t1 = tid - 32, nth = NT - 32;
         if (t1 == 0) {
             sm.nkey[0] = 0xFFFFFFFFu;
@@ -809,7 +831,7 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
             r = pre_r;  // (lane 0's copy is the one used below)
         else
             r = saba_warp(p.saba, p.bmin, p.bmax, p.bstep, L, K, p.row_status + (size_t)b * L, p.vp_err,
-                          p.topk_lp + (size_t)b * L * K, sm.cosv, p.hist + b, p.prefix_len + b,
+                          p.topk_lp + (size_t)b * L * K, p.cos_pre + (size_t)b * L, p.hist + b, p.prefix_len + b,
                           p.use_saba ? nullptr : p.fixed_budget + b, lane);
         if (lane == 0) {
             sm.scal[0] = r.budget;
@@ -868,14 +890,15 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
         float sel_top = 0.0f;  // the best score (the root's best child): where the bins of the threshold searches start
         if (spec) {  // levels 0 and 1 are in the table already: the threshold they give, then on from level 2
             ntot = 1 + K + K * K;
-            if (ntot - 1 >= budget) {
+            const bool look = L > 2 && rows_done > 2 && ntot + K * K <= ncap;
+            if (ntot - 1 + (look ? K * K : 0) >= budget) {
                 sel_top = 0.0f + sm.es[0];  // the root's best child
                 // The threshold of levels 0 and 1 alone is loose: the best child of every level-1 node is a prefix too, and
                 // its key costs one look at the node's sorted row.  Those K^2 keys stand behind the table for the search
                 // (the level's real children overwrite them), which then gives a bound closer to the final one and a
-                // level 2 that appends a third of what it would.
+                // level 2 that appends a third of what it would (and a bound at all where levels 0 and 1 hold fewer than B).
                 int nsel = ntot;
-                if (L > 2 && rows_done > 2 && ntot + K * K <= ncap) {  // (uniform)
+                if (look) {  // (uniform)
 #pragma unroll (NT == 1024 ? 4 : 1)
                     for (int j = tid; j < K * K; j += NT) {
                         const int x = 1 + K + j;
@@ -911,7 +934,7 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
             if (b1 == b0) break;
             int lvl_end = ntot;
             bool over = false;  // the node table is full
-            if (d >= rows_done) {  // the edge rows of this depth: scored now, never if the expansion stops above it
+            if (!TIES && d >= rows_done) {  // the edge rows of this depth: scored now, never if the expansion stops above it
                 int alive = 0;  // (nor if no node of the level can still have a selected child)
 #pragma unroll 1
                 for (int x = b0 + tid; x < b1; x += NT) alive |= sm.nkey[x] >= theta ? 1 : 0;
@@ -948,7 +971,7 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
             } else if (n_grow <= NT / grp) {
                 // The last levels of nearly every tree: a thread per node finds the nodes that can have children by the best
                 // entry of their rows, then a group of lanes takes one of them each, a lane per entry.  No search along a
-                // row and none for a child's node: FAST_BEFORE_AFTER
+                // row and none for a child's node: 1.8k cycles a level, the path below takes 3.1k.
                 int* wcnt = (int*)sm.hist;       // [32] such nodes per warp
                 int* list = (int*)sm.hist + 32;  // [32] those nodes in the order of the level, -1: none
                 int* ccnt = (int*)sm.hist + 64;  // [32] their children that reach theta
@@ -1364,7 +1387,7 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
             }
         }
     }
-    if (p_lazy && !table_ok && budget > 0) {  // the sequential fall-back may reach any depth
+    if (!TIES && p_lazy && !table_ok && budget > 0) {  // the sequential fall-back may reach any depth
 #pragma unroll 1
         for (; rows_done < L; ++rows_done) lazy_score_row<NT, KC>(p, sm, rows_done, root, tid, inflight, K, p_m);
     }
@@ -1592,7 +1615,7 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
             __syncwarp();
         }
     }
-    if (p_lazy) cp_async_wait_all();  // table rows fetched ahead for a depth that was never scored
+    if (!TIES && p_lazy) cp_async_wait_all();  // table rows fetched ahead for a depth that was never scored
     if (tid == 0) {
         o.d_n_nodes[b] = n_nodes;
         o.d_budget[b] = sm.scal[0];
@@ -1744,7 +1767,7 @@ static TreeInstance tree_pick(const graft_config& cfg, bool usual, bool neutral)
     const int nmax = cfg.budget_max + 1;
     usual = usual && cfg.m == 128;
     if (neutral) {
-        if (usual && cfg.K == 32) return {tree_kernel<1024, 32, 128, true, 0, true>, 1024};
+        if (cfg.K == 32) return {tree_kernel<1024, 32, 0, false, 0, true>, 1024};
         return tree_pick_general<true>(cfg.K);
     }
     if (usual && cfg.K == 32) {
@@ -1790,7 +1813,9 @@ cudaError_t tree_launch(graft_ctx* ctx, int batch, const int32_t* d_topk_id, con
     p.nmax = ctx->nmax;
     p.W = ctx->mask_words;
     p.rows_pre = ctx->edge_rows;
-    p.lazy = p.rows_pre < cfg.L ? 1 : 0;  // (only possible when tree_lazy_fits)
+    p.beta = ctx->tdes_set ? cfg.beta : 0.0f;
+    const bool neutral = p.beta == 0.0f;  // (the candidates are staged whenever there is room; no row is scored)
+    p.lazy = neutral ? tree_lazy_fits(cfg) : p.rows_pre < cfg.L ? 1 : 0;  // (only possible when tree_lazy_fits)
     p.rows_adaptive = (p.lazy && p.rows_pre > 0 && d_saba_pre != nullptr) ? 1 : 0;
     p.lazy_m = tree_lazy_fits(cfg) ? cfg.m : 0;
     p.ncap = tree_node_cap(cfg.L, cfg.K, ctx->nmax, p.lazy_m);
@@ -1798,7 +1823,6 @@ cudaError_t tree_launch(graft_ctx* ctx, int batch, const int32_t* d_topk_id, con
     p.C = ctx->d_C;
     p.u = ctx->d_u;
     p.scale = ctx->tdes_s / sqrtf((float)cfg.m);
-    p.beta = ctx->tdes_set ? cfg.beta : 0.0f;
     p.root_edge = cfg.root_edge;
     p.m = cfg.m;
     p.V = cfg.V;
@@ -1811,7 +1835,7 @@ cudaError_t tree_launch(graft_ctx* ctx, int batch, const int32_t* d_topk_id, con
     // the instances with K and m known at compile time serve the usual round (the budget from the edge-score kernel,
     // deeper rows on demand)
     const bool usual = p.lazy && p.saba_pre != nullptr;
-    const TreeInstance kern = tree_pick(cfg, usual, p.beta == 0.0f);
+    const TreeInstance kern = tree_pick(cfg, usual, neutral);
     const cudaError_t e = launch_pdl(kern.kernel, dim3(batch), dim3(kern.threads), tree_smem_bytes(cfg), st, p);
     ctx->launches += 1;
     return e != cudaSuccess ? e : cudaGetLastError();

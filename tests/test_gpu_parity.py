@@ -596,6 +596,26 @@ def test_round_rows_of_a_sequence_off_the_16_byte_grid(L, K, beta):
     g.destroy()
 
 
+@pytest.mark.parametrize("L,K,m", [(1, 4, 36), (2, 8, 36), (5, 9, 64), (6, 20, 64), (7, 21, 64), (4, 32, 40), (6, 32, 512)])
+@pytest.mark.parametrize("beta", [0.3, 0.0])
+@pytest.mark.parametrize("fixed", [None, 61])
+def test_round_at_the_edges_of_the_tree_kernel_instances(L, K, m, beta, fixed):
+    """Trees on either side of the candidate counts at which the tree kernel's thread count changes, of one and two
+    levels, with rows scored ahead, on demand or not at all (beta = 0: no edge-score kernel runs unless its array is asked
+    for), with room for the on-demand buffers and without (m = 512); the call with and without debug outputs agree."""
+    w = gi.small(batch=3, L=L, V=4099, K=K, budget_min=16, budget_max=160, budget_step=16, logits_dtype="bf16", m=m,
+                 hidden_dim=40, beta=beta, fixed_budget=fixed)
+    g = _graft(w)
+    tb, saba_kw, keep = _setup(w, g)
+    x = gi.batch_inputs(w)
+    out, gpu = gpu_round(g, w, x)
+    compare_round(oracle, w, x, tb, saba_kw, gpu, oracle_round(oracle, w, x, tb, saba_kw))
+    _, gpu2 = gpu_round(g, w, x, debug=False)
+    for k in ("n_nodes", "budget", "status", "token", "parent", "depth", "position", "path_score", "mask"):
+        assert np.array_equal(gpu[k], gpu2[k]), k
+    g.destroy()
+
+
 @pytest.mark.parametrize("kw", _SPLIT_CASES[:3] + [
     dict(batch=3, L=16, V=6000, K=32, budget_min=32, budget_max=512, budget_step=16, m=512, hidden_dim=64)])
 @pytest.mark.parametrize("rows", [0, None])
