@@ -125,22 +125,28 @@ def _check(lib, rc, what):
         raise GraftError(f"{what}: {lib.graft_status_str(rc).decode()} (status {rc})")
 
 
+# A round at batch 1 takes the GPU 27 us and passes some thirty tensors, so a tensor's checks are one test when all is well
+# (0.35 us instead of 0.5, pointers as plain integers, which ctypes takes for void pointers) and the reason is looked for
+# afterwards.
 def _ptr(t, dtype=None, cuda=True):
     if t is None:
         return None
+    if t.is_cuda is cuda and (dtype is None or t.dtype is dtype) and t.is_contiguous():
+        return t.data_ptr()
     if cuda and not t.is_cuda:
         raise GraftError("expected a CUDA tensor")
     if not cuda and t.is_cuda:
         raise GraftError("expected a CPU tensor")
     if not t.is_contiguous():
         raise GraftError("tensor must be contiguous")
-    if dtype is not None and t.dtype != dtype:
-        raise GraftError(f"expected dtype {dtype}, got {t.dtype}")
-    return C.c_void_p(t.data_ptr())
+    raise GraftError(f"expected dtype {dtype}, got {t.dtype}")
 
 
 def _stream():
-    return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+    """The current stream of the current device (as torch.cuda.current_stream(), without its Stream object)."""
+    if torch.cuda.is_initialized():
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    return torch.cuda.current_stream().cuda_stream
 
 
 def vocab_pass_static(logits, K, topk_id, topk_lp, lse, row_status):
@@ -180,23 +186,13 @@ class TreeOut:
     state: torch.Tensor | None = None
 
     def _c(self, cuda=True):
-        o = _TreeOut()
         i32, f32 = torch.int32, torch.float32
-        o.d_n_nodes = _ptr(self.n_nodes, i32, cuda)
-        o.d_budget = _ptr(self.budget, i32, cuda)
-        o.d_token = _ptr(self.token, i32, cuda)
-        o.d_parent = _ptr(self.parent, i32, cuda)
-        o.d_depth = _ptr(self.depth, i32, cuda)
-        o.d_position = _ptr(self.position, i32, cuda)
-        o.d_path_score = _ptr(self.path_score, f32, cuda)
-        o.d_mask = _ptr(self.mask, i32, cuda)  # uint32 bit patterns held in an int32 tensor
-        o.d_status = _ptr(self.status, i32, cuda)
-        o.d_topk_id = _ptr(self.topk_id, i32, cuda)
-        o.d_topk_lp = _ptr(self.topk_lp, f32, cuda)
-        o.d_lse = _ptr(self.lse, f32, cuda)
-        o.d_edge = _ptr(self.edge, f32, cuda)
-        o.d_state = _ptr(self.state, f32, cuda)
-        return o
+        return _TreeOut(  # (in the order of the structure; mask: uint32 bit patterns held in an int32 tensor)
+            _ptr(self.n_nodes, i32, cuda), _ptr(self.budget, i32, cuda), _ptr(self.token, i32, cuda),
+            _ptr(self.parent, i32, cuda), _ptr(self.depth, i32, cuda), _ptr(self.position, i32, cuda),
+            _ptr(self.path_score, f32, cuda), _ptr(self.mask, i32, cuda), _ptr(self.status, i32, cuda),
+            _ptr(self.topk_id, i32, cuda), _ptr(self.topk_lp, f32, cuda), _ptr(self.lse, f32, cuda),
+            _ptr(self.edge, f32, cuda), _ptr(self.state, f32, cuda))
 
     def cpu(self) -> dict:
         out = {}
@@ -346,7 +342,7 @@ class Graft:
     def accept(self, trees: TreeOut, target_next, accept_len, accept_path, bonus_token):
         batch = target_next.shape[0]
         i32 = torch.int32
-        oc = trees._c()
+        oc = _TreeOut(d_n_nodes=_ptr(trees.n_nodes, i32), d_token=_ptr(trees.token, i32), d_parent=_ptr(trees.parent, i32))
         _check(self.lib, self.lib.graft_accept(self._ctx, batch, C.byref(oc), _ptr(target_next, i32),
                                                _ptr(accept_len, i32), _ptr(accept_path, i32),
                                                _ptr(bonus_token, i32), _stream()), "graft_accept")
