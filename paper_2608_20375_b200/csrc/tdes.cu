@@ -130,13 +130,24 @@ __global__ void __launch_bounds__(256, 4) tdes_edges_kernel(const EdgeParams p) 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int n_par = (j == 0) ? 1 : K;
     const size_t row = (size_t)b * p.L + j;
-    if (j == 0 && p.saba_out != nullptr && warp == 7) {
-        // the depth-0 unit has one parent, so this CTA has time to spare: its last warp works out the sequence's budget,
-        // which the tree kernel would otherwise do in front of everything else
+    // The depth-0 unit has one parent, so this CTA has time to spare: its last warp works out the sequence's budget, which
+    // the tree kernel would otherwise do in front of everything else.  That takes longer than the scores of a unit (a
+    // chain of fp64 operations, 3 us), so the warp does nothing else and the other seven do not wait for it (batch 16,
+    // K = 16: 44.7 -> 44.4 us a round; batch 1, K = 32: 41.7 -> 40.3; batch 256: 293.5 -> 292.3).
+    const bool with_saba = j == 0 && p.saba_out != nullptr;
+    const int nw = with_saba ? 7 : 8;  // warps on the scores
+    const auto sync = [&] {
+        if (with_saba)
+            named_bar_sync(1, 7 * 32);
+        else
+            __syncthreads();
+    };
+    if (with_saba && warp == 7) {
         const SabaResult r = saba_warp(p.saba, p.bmin, p.bmax, p.bstep, p.L, K, p.row_status + (size_t)b * p.L, p.vp_err,
                                        p.topk_lp + (size_t)b * p.L * K, p.cos_pre + (size_t)b * p.L, p.hist + b,
                                        p.prefix_len + b, p.fixed_budget ? p.fixed_budget + b : nullptr, lane);
         if (lane == 0) p.saba_out[b] = r;
+        return;
     }
     float* outs = p.esort + row * K * K;
     uint8_t* outi = p.eidx + row * K * K;
@@ -148,7 +159,7 @@ __global__ void __launch_bounds__(256, 4) tdes_edges_kernel(const EdgeParams p) 
     if (neutral) {
         // edge = log q exactly (the DDTree score of Eq. 3); bad rows get zeros
         // (log q is already ordered by rank, so the sorted rows are the rows themselves)
-        for (int i = threadIdx.x; i < K * K; i += 256) {
+        for (int i = threadIdx.x; i < K * K; i += nw * 32) {
             int par = i / K, c = i % K;
             const float v = (bad || par >= n_par) ? 0.f : lps[c];
             if (WRITE_EDGE) p.edge[row * K * K + i] = v;
@@ -165,7 +176,7 @@ __global__ void __launch_bounds__(256, 4) tdes_edges_kernel(const EdgeParams p) 
         int32_t tok = r < n_par ? (j == 0 ? p.root_token[b] : p.topk_id[(row - 1) * K + r]) : ids[r - n_par];
         toks[r] = tok < 0 ? 0 : (tok >= p.V ? p.V - 1 : tok);
     }
-    __syncthreads();
+    sync();
     const float* urow = p.u + (size_t)j * m;
     constexpr int RPW = 2 * kMaxK / 8;  // rows per warp at most
     const uint64_t keep = l2_policy_evict_last();
@@ -174,7 +185,7 @@ __global__ void __launch_bounds__(256, 4) tdes_edges_kernel(const EdgeParams p) 
         float4 t[RPW];
 #pragma unroll
         for (int q = 0; q < RPW; ++q) {
-            const int r = warp + 8 * q;
+            const int r = warp + nw * q;
             t[q] = make_float4(0.f, 0.f, 0.f, 0.f);
             if (r < n_par + K && k4 < m / 4)
                 t[q] = ldg_f4_keep((const float4*)((r < n_par ? p.P : p.C) + (size_t)toks[r] * m) + k4, keep);
@@ -183,7 +194,7 @@ __global__ void __launch_bounds__(256, 4) tdes_edges_kernel(const EdgeParams p) 
             const float4 uu = *(const float4*)(urow + k4 * 4);
 #pragma unroll
             for (int q = 0; q < RPW; ++q) {
-                const int r = warp + 8 * q;
+                const int r = warp + nw * q;
                 if (r < n_par + K) {
                     float* dst = (r < n_par ? sP + (size_t)r * ld : sC + (size_t)(r - n_par) * ld) + k4 * 4;
                     *(float4*)dst = make_float4(t[q].x + uu.x, t[q].y + uu.y, t[q].z + uu.z, t[q].w + uu.w);
@@ -191,7 +202,7 @@ __global__ void __launch_bounds__(256, 4) tdes_edges_kernel(const EdgeParams p) 
             }
         }
     }
-    __syncthreads();
+    sync();
     // dot products into shared memory, then every warp finishes the rows of parents warp, warp+8, ...
     float* part = sC + (size_t)kMaxK * ld;  // [K][dots_ld(K)]
     __shared__ uint32_t wsc[8][32];
@@ -201,9 +212,9 @@ __global__ void __launch_bounds__(256, 4) tdes_edges_kernel(const EdgeParams p) 
         edge_dots<false, 8, 2, false>(sP, sC, nullptr, m, K, n_par, part, warp, lane);
     else
         edge_dots<false, 8, 4, false>(sP, sC, nullptr, m, K, n_par, part, warp, lane);
-    __syncthreads();
+    sync();
     const float inv_K = 1.0f / (float)K;
-    for (int par = warp; par < K; par += 8) {
+    for (int par = warp; par < K; par += nw) {
         float val;
         int rank;
         edge_row_finish(par < n_par ? part + (size_t)par * dots_ld(K) : nullptr, lps, p.scale, p.beta, K, inv_K, wsc[warp], lane,
