@@ -88,8 +88,8 @@ struct EdgeParams {
     float* esort;     // same rows, each sorted by (edge descending, child rank ascending), stored rotated (es_col)
     uint8_t* eidx;    // child rank of every sorted entry
     int L, K, m, V;
-    int rows;     // depths [0, rows) are scored for every sequence: one CTA each
-    int rows_all; // CTAs per sequence: depths [rows, rows_all) are scored only for sequences whose trees will run deep
+    int rows;     // depths [0, rows) are scored for every sequence: one CTA each; deeper ones
+                  // only for sequences whose trees will run deep
     float scale;  // s / sqrt(m)
     float beta;
     int root_edge;
@@ -111,18 +111,11 @@ __global__ void __launch_bounds__(256, 4) tdes_edges_kernel(const EdgeParams p) 
     extern __shared__ __align__(16) float smem[];
     pdl_launch_dependents();  // the tree kernel may move in as SMs free up; it waits for this grid before it reads
     pdl_wait();               // the candidates come from the vocab pass
-    // the depths scored for every sequence come first in the grid, the depths that only deep trees need behind them: the
-    // CTAs of the latter mostly exit at once and should not take the places of CTAs with work
-    const int n_all = (int)gridDim.x / p.rows_all * p.rows;  // units that every sequence needs
-    int b, j;
-    if ((int)blockIdx.x < n_all) {
-        b = (int)blockIdx.x / p.rows;
-        j = (int)blockIdx.x - b * p.rows;
-    } else {
-        const int r = (int)blockIdx.x - n_all, nd = p.rows_all - p.rows;
-        b = r / nd;
-        j = p.rows + (r - b * nd);
-    }
+    // Sequences run fastest in the grid: the depth-0 units, whose budgets take longest, come first, and the depths that
+    // only deep trees need behind those scored for every sequence (their CTAs mostly exit at once and should not take the
+    // places of CTAs with work).  No division stands in front of the first loads (batch 16: 44.4 -> 43.7 us a round; batch 64:
+    // 95.1 -> 94.8).
+    const int b = blockIdx.x, j = blockIdx.y;
     if (j >= p.rows && !deep_tree_likely(p.topk_lp + (size_t)b * p.L * p.K, p.L, p.K)) return;  // (uniform)
     const int K = KC ? KC : p.K, m = MC ? MC : p.m, ld = m + 4;  // padded row: 16-byte aligned, conflict-free float4 reads
     float* sP = smem;                        // [K][ld]  parent rows + u_d
@@ -283,7 +276,7 @@ cudaError_t tdes_edges_launch(graft_ctx* ctx, int batch, const int32_t* d_topk_i
     p.beta = ctx->tdes_set ? cfg.beta : 0.0f;
     p.root_edge = cfg.root_edge;
     p.rows = rows;
-    p.rows_all = d_edge || rows == cfg.L ? rows : cfg.L;  // (rows < L only when the tree kernel can score on demand)
+    const int rows_all = d_edge || rows == cfg.L ? rows : cfg.L;  // (rows < L only when the tree kernel can score on demand)
     p.saba_out = d_row_status ? d_saba_out : nullptr;
     p.cos_pre = ctx->w_cos;
     p.vp_err = ctx->w_errflag;
@@ -300,7 +293,7 @@ cudaError_t tdes_edges_launch(graft_ctx* ctx, int batch, const int32_t* d_topk_i
         if (cfg.K == 16) kern = tdes_edges_kernel<false, 16, 128>;
         if (cfg.K == 8) kern = tdes_edges_kernel<false, 8, 128>;
     }
-    const cudaError_t e = launch_pdl(kern, dim3(batch * p.rows_all), dim3(256), tdes_edges_smem(cfg), st, p);
+    const cudaError_t e = launch_pdl(kern, dim3(batch, rows_all), dim3(256), tdes_edges_smem(cfg), st, p);
     ctx->launches += 1;
     return e != cudaSuccess ? e : cudaGetLastError();
 }
