@@ -282,7 +282,7 @@ graft_status graft_vocab_pass(graft_ctx* ctx, int32_t batch, const void* d_logit
     const int esz = ctx->cfg.logits_dtype == GRAFT_BF16 ? 2 : 4;
     if ((uintptr_t)d_logits % esz) return GRAFT_ERR_INVALID_ARG;
     if (vp_launch(ctx, batch, d_logits, d_topk_id, d_topk_lp, d_lse, d_row_status ? d_row_status : ctx->w_row_status,
-                  nullptr, nullptr, nullptr, (cudaStream_t)stream) != cudaSuccess)
+                  nullptr, nullptr, nullptr, false, (cudaStream_t)stream) != cudaSuccess)
         return GRAFT_ERR_CUDA;
     return GRAFT_OK;
 }
@@ -389,9 +389,10 @@ graft_status graft_build_trees(graft_ctx* ctx, int32_t batch, const void* d_logi
     float* lse = out->d_lse ? out->d_lse : ctx->w_lse;
     float* edge = out->d_edge;  // NULL: the edge kernel writes only the sorted rows the tree kernel reads
 
+    const bool neutral = ctx->cfg.beta == 0.0f || !ctx->tdes_set;  // a round without edge scores
     if (ev) cudaEventRecord(ev[0], st);
     if (vp_launch(ctx, batch, d_logits, ids, lps, lse, ctx->w_row_status, use_saba ? d_hidden : nullptr, ctx->w_cos,
-                  nullptr, st) != cudaSuccess)
+                  nullptr, neutral, st) != cudaSuccess)
         return GRAFT_ERR_CUDA;
     if (ev) cudaEventRecord(ev[1], st);
     // Edge scores of Eq. 4-6: the kernel scores the depths [0, edge_rows) for every sequence (all depths when the
@@ -399,7 +400,6 @@ graft_status graft_build_trees(graft_ctx* ctx, int32_t batch, const void* d_logi
     // The depth-0 CTA of each sequence in that kernel also works out the sequence's budget (Sec. 3.3), which the tree
     // kernel then only reads; without an edge-score kernel the tree kernel does it itself.
     // Without edge scores (beta = 0) nothing needs that kernel: the tree kernel lays the rows out from log q.
-    const bool neutral = ctx->cfg.beta == 0.0f || !ctx->tdes_set;
     const int rows = out->d_edge ? ctx->cfg.L : neutral ? 0 : ctx->edge_rows;
     if (rows > 0 && tdes_edges_launch(ctx, batch, ids, lps, d_root_token, ctx->w_row_status, edge, ctx->w_esort,
                                       ctx->w_eidx, rows, ctx->w_saba, d_hist, d_prefix_len, d_fixed_budget,
@@ -437,7 +437,7 @@ graft_status graft_vocab_pass_partial(graft_ctx* ctx, int32_t batch, const void*
     const int esz = ctx->cfg.logits_dtype == GRAFT_BF16 ? 2 : 4;
     if ((uintptr_t)d_logits_shard % esz || (uintptr_t)d_out % 8) return GRAFT_ERR_INVALID_ARG;
     if (vp_launch(ctx, batch, d_logits_shard, ctx->w_topk_id, ctx->w_topk_lp, ctx->w_lse, ctx->w_row_status, nullptr,
-                  nullptr, d_out, (cudaStream_t)stream) != cudaSuccess)
+                  nullptr, d_out, false, (cudaStream_t)stream) != cudaSuccess)
         return GRAFT_ERR_CUDA;
     return GRAFT_OK;
 }

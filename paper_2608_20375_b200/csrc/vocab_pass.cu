@@ -1475,7 +1475,7 @@ static size_t vp_smem_bytes(int groups, int stages, int n_cmax) {
     return (size_t)stages * TILE + (16 + 2 * kVpMaxBufs) * sizeof(uint64_t) + sh + (size_t)2 * groups * n_cmax * 2 + 16;
 }
 
-VpPlan vp_make_plan(const graft_config& cfg, int num_sms, int batch) {
+VpPlan vp_make_plan(const graft_config& cfg, int num_sms, int batch, bool equal_shares) {
     VpPlan pl;
     const bool bf16 = cfg.logits_dtype == GRAFT_BF16;
     const long long esz = bf16 ? 2 : 4, rows = (long long)batch * cfg.L, row_bytes = (long long)cfg.V * esz;
@@ -1484,7 +1484,18 @@ VpPlan vp_make_plan(const graft_config& cfg, int num_sms, int batch) {
     // A row that no other CTA has a piece of needs no merge, which is what a small input waits for (a record and a merge
     // take 5 to 6 us, the stream of a 64 KB row 1.4 us): whole rows wherever the CTAs' shares come out even enough.  Measured
     // on 148 SMs, one launch after the other, bf16, L = 16.
-    if (rows < num_sms) {
+    if (equal_shares) {
+        // Rounds without edge scores.  Their path scores are sums of log-probabilities alone, and of logits with few digits
+        // hundreds of such sums are equal but for the rounding of the rows' log-sum-exp: its last bit, which hangs on how a
+        // row's sum is cut into pieces, decides which prefix stands first.  These rounds keep one partition (equal shares of
+        // at least 64 KB of the whole stream), and with it their trees, whatever suits the others best; batch 37, L = 11,
+        // V = 50,021: 42.6 us a round, 39.8 with whole rows.
+        G = nq * rows / (64 * 1024 / (kVpQuantum * esz));
+        if (G > num_sms) G = num_sms;
+        if (G < 1) G = 1;
+        pl.whole = 0;
+        share_q = (nq * rows + G - 1) / G;
+    } else if (rows < num_sms) {
         // n pieces of each row, n = 1 unless the stream gets shorter by more than the merge costs (190 KB): V = 151,936
         // batch 1: n = 1 18.5 us, n = 2 18.6, n = 4 17.1, n = 9 20.9; batch 4: n = 1 18.9, n = 2 19.7
         long long n = row_bytes / (76 * 1024);
@@ -1504,7 +1515,7 @@ VpPlan vp_make_plan(const graft_config& cfg, int num_sms, int batch) {
         G = pl.whole ? (rows + per - 1) / per : num_sms;
         share_q = pl.whole ? per * nq : (nq * rows + G - 1) / G;
     }
-    if (pl.whole == 0 && G > nq * rows) G = nq * rows;
+    if (!equal_shares && pl.whole == 0 && G > nq * rows) G = nq * rows;
     pl.grid = (int)G;
     long long seg_elems = share_q * kVpQuantum + kVpQuantum;  // a row's last quantum also takes the remainder
     if (pl.whole || seg_elems > cfg.V) seg_elems = cfg.V;
@@ -1522,10 +1533,10 @@ VpPlan vp_make_plan(const graft_config& cfg, int num_sms, int batch) {
 
 cudaError_t vp_launch(graft_ctx* ctx, int batch, const void* d_logits, int32_t* d_topk_id, float* d_topk_lp,
                       float* d_lse, int32_t* d_row_status, const void* d_hidden, double* d_cos,
-                      graft_vocab_partial* d_partial, cudaStream_t st) {
+                      graft_vocab_partial* d_partial, bool equal_shares, cudaStream_t st) {
     const graft_config& cfg = ctx->cfg;
     const bool bf16 = cfg.logits_dtype == GRAFT_BF16;
-    VpPlan pl = vp_make_plan(cfg, ctx->num_sms, batch);
+    VpPlan pl = vp_make_plan(cfg, ctx->num_sms, batch, equal_shares);
     VpParams p;
     p.logits = (const char*)d_logits;
     p.rows = batch * cfg.L;
@@ -1577,7 +1588,7 @@ int vp_merge_max_shards() { return kMergeMaxShards; }
 
 cudaError_t vp_configure(const graft_config& cfg, int num_sms, size_t* max_smem) {
     // the largest dynamic shared-memory request any batch can produce (segment = a whole row)
-    VpPlan pl = vp_make_plan(cfg, num_sms, cfg.max_batch > 4096 ? cfg.max_batch : 4096);
+    VpPlan pl = vp_make_plan(cfg, num_sms, cfg.max_batch > 4096 ? cfg.max_batch : 4096, false);
     *max_smem = pl.smem_bytes;
     if (pl.smem_bytes > 225 * 1024) return cudaErrorInvalidValue;
     cudaError_t e = cudaSuccess;
@@ -1671,7 +1682,7 @@ extern "C" graft_status graft_vocab_pass_static(int32_t batch, int32_t L, int32_
             sd->ready = true;
         }
     }
-    const VpPlan pl = vp_make_plan(cfg, sd->num_sms, batch);
+    const VpPlan pl = vp_make_plan(cfg, sd->num_sms, batch, false);
     if (pl.grid > kStaticMaxGrid || pl.smem_bytes > 225 * 1024) return GRAFT_ERR_UNSUPPORTED;
     cudaStream_t st = (cudaStream_t)stream;
     // the array keeps whatever the previous call left: the arrival counters and the error word must start at 0
