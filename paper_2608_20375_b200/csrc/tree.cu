@@ -663,7 +663,7 @@ __device__ __forceinline__ void lazy_score_row(const TreeParams& p, const TreeSm
 // FAST: the usual round is known at compile time as well -- the budget comes from the edge-score kernel (no SABA
 // arithmetic in this instance) and deeper rows are scored on demand
 // TIES: the instance for rounds without edge scores (beta = 0).  It lays the rows out itself (no edge-score kernel ran, and
-// the budget is worked out here as well: two launches a round less its gap; batch 37, K = 11: 7 us a round less) and
+// the budget is worked out here as well: a launch and its gap less; batch 37, K = 11: 7 us a round) and
 // expects that exactly equal probabilities make hundreds of
 // prefixes tie with the B-th largest key: it resolves them in parallel (the other instances leave more than 32 tied
 // keys to the sequential expansion; with edge scores in the keys such ties do not occur in tens, and the code's mere
