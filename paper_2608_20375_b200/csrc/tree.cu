@@ -685,7 +685,7 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
     // ---- status and budget ---------------------------------------------------------------------------
     // the sorted edge rows of this sequence: bulk copies through the TMA unit when the 16-byte rules allow it
     // (they land while warp 0 works out the budget), plain loads otherwise
-    __shared__ __align__(8) uint64_t rows_bar;
+    __shared__ __align__(8) uint64_t rows_bar, deep_bar;  // (deep_bar: 1024 threads only)
     __shared__ int rows_abort;
     const int rows_pre = TIES ? L : p.rows_pre;
     const int ne = rows_pre * K * K;  // entries that come from the edge-score kernel for every sequence
@@ -716,25 +716,22 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
     if (tid == 0) {
         rows_abort = 0;
         mbar_init(smem_u32(&rows_bar), 1);
+        if (NT == 1024) mbar_init(smem_u32(&deep_bar), 1);
         mbar_fence_init();
     }
     const size_t seq_e = (size_t)b * L * K * K;  // this sequence's rows in esort / eidx
-    if (bulk) {
-        if (tid == 0) {
-            mbar_arrive_expect_tx(smem_u32(&rows_bar), (uint32_t)ne * 5u);
-            const char* g_es = (const char*)(p.esort + seq_e);
-            const char* g_ei = (const char*)(p.eidx + seq_e);
+    // entries [lo, hi) of this sequence's rows as bulk copies behind a barrier: one thread
+    const auto copy_rows = [&](uint32_t lo, uint32_t hi, uint32_t bar) {
+        mbar_arrive_expect_tx(bar, (hi - lo) * 5u);
 #pragma unroll 1
-            for (uint32_t off = 0; off < (uint32_t)ne * 4u; off += 16384u) {
-                const uint32_t bytes = (uint32_t)ne * 4u - off < 16384u ? (uint32_t)ne * 4u - off : 16384u;
-                tma_load_1d(smem_u32((char*)sm.es + off), g_es + off, bytes, smem_u32(&rows_bar));
-            }
-#pragma unroll 1
-            for (uint32_t off = 0; off < (uint32_t)ne; off += 16384u) {
-                const uint32_t bytes = (uint32_t)ne - off < 16384u ? (uint32_t)ne - off : 16384u;
-                tma_load_1d(smem_u32((char*)sm.ei + off), g_ei + off, bytes, smem_u32(&rows_bar));
-            }
+        for (uint32_t at = lo; at < hi; at += 4096u) {
+            const uint32_t n = hi - at < 4096u ? hi - at : 4096u;
+            tma_load_1d(smem_u32(sm.es + at), p.esort + seq_e + at, n * 4u, bar);
+            tma_load_1d(smem_u32(sm.ei + at), p.eidx + seq_e + at, n, bar);
         }
+    };
+    if (bulk) {
+        if (tid == 0) copy_rows(0u, (uint32_t)ne, smem_u32(&rows_bar));
     } else if (!TIES) {
 #pragma unroll 1
         for (int i = tid; i < ne; i += NT) {
@@ -757,13 +754,19 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
             inflight = 0;
         }
     }
-    // a sequence whose tree will run deep had its deeper rows scored by the edge-score kernel as well (they are needed
-    // several levels from here: plain loads, consumed after many barriers)
-    if (!TIES && p.rows_adaptive && deep_tree_decide(lp_top, L)) {  // (uniform)
+    // a sequence whose tree will run deep had its deeper rows scored by the edge-score kernel as well: bulk copies again for
+    // large K (plain loads, eight round trips with K = 32, kept such a sequence 2 us: batch 64 with mixed confidence 99.6 ->
+    // 98.4 us a round), plain loads for K <= 20, which are fewer (batch 16, K = 16: 49.0 us, 49.5 with bulk copies)
+    const bool deep = !TIES && p.rows_adaptive && deep_tree_decide(lp_top, L);  // (uniform)
+    if (deep) {
+        if (NT == 1024 && bulk) {
+            if (tid == 0) copy_rows((uint32_t)ne, (uint32_t)(L * K * K), smem_u32(&deep_bar));
+        } else {
 #pragma unroll 1
-        for (int i = ne + tid; i < L * K * K; i += NT) {
-            sm.es[i] = p.esort[seq_e + i];
-            sm.ei[i] = p.eidx[seq_e + i];
+            for (int i = ne + tid; i < L * K * K; i += NT) {
+                sm.es[i] = p.esort[seq_e + i];
+                sm.ei[i] = p.eidx[seq_e + i];
+            }
         }
         rows_done = L;
     }
@@ -846,6 +849,8 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
     if (bulk) {
         // bounded wait for the bulk copies; on a timeout the sequence is reported through its status word
         if (!mbar_wait_bounded(smem_u32(&rows_bar), 0, &rows_abort) && tid == 0) sm.scal[2] |= GRAFT_ST_INTERNAL;
+        if (NT == 1024 && deep && !mbar_wait_bounded(smem_u32(&deep_bar), 0, &rows_abort) && tid == 0)
+            sm.scal[2] |= GRAFT_ST_INTERNAL;
         __syncthreads();
     }
 
