@@ -1181,7 +1181,10 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
             // the exact B-th largest key is recomputed only when the table has grown noticeably
             if (ntot - 1 >= budget && (theta == 0u || ntot - n_at_select >= ntot / 4)) {
                 sel_top = 0.0f + sm.es[0];  // the root's best child
-                theta = cta_select_bucket<NT>(sm, sm.nkey, 1, ntot, budget, sel_top, sel, tid);  // a lower bound
+                // a lower bound; never below the one in use, which a search over a level's children may have put higher (the
+                // count of the nodes that can have children holds for a threshold that rises only)
+                const uint32_t bound = cta_select_bucket<NT>(sm, sm.nkey, 1, ntot, budget, sel_top, sel, tid);
+                theta = bound > theta ? bound : theta;
                 if (TIES) {
                     __syncthreads();
                     theta = cta_snap_to_key<NT>(sm.nkey, 1, ntot, theta, sm.hist + 1100, tid);
