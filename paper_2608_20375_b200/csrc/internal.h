@@ -123,6 +123,21 @@ inline cudaError_t launch_pdl(void (*kernel)(P), dim3 grid, dim3 block, size_t s
     return cudaLaunchKernelEx(&lc, kernel, params);
 }
 
+// Let launches of `kernel` ask for `need` bytes of dynamic shared memory; an error if the device has less.  The limit
+// belongs to the kernel on the device and not to a context: it is raised to all there is, so that a context of smaller
+// sizes created later does not take room from an older one.
+inline cudaError_t allow_smem(const void* kernel, size_t need) {
+    int dev = 0, most = 0;
+    cudaFuncAttributes a;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, kernel);
+    if (e != cudaSuccess) return e;
+    most -= (int)a.sharedSizeBytes;
+    if (most < 0 || need > (size_t)most) return cudaErrorInvalidValue;
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+}
+
 VpPlan vp_make_plan(const graft_config& cfg, int num_sms, int batch, bool equal_shares);
 cudaError_t vp_configure(const graft_config& cfg, int num_sms, size_t* max_smem);
 cudaError_t vp_launch(graft_ctx* ctx, int batch, const void* d_logits, int32_t* d_topk_id, float* d_topk_lp,

@@ -239,16 +239,11 @@ size_t tdes_edges_smem(const graft_config& cfg) {
 }
 
 cudaError_t tdes_edges_configure(const graft_config& cfg) {
-    const int bytes = (int)tdes_edges_smem(cfg);
-    cudaError_t e = cudaFuncSetAttribute(tdes_edges_kernel<true, 0, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(tdes_edges_kernel<false, 0, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(tdes_edges_kernel<false, 32, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(tdes_edges_kernel<false, 16, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(tdes_edges_kernel<false, 8, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    const size_t bytes = tdes_edges_smem(cfg);
+    cudaError_t e = cudaSuccess;
+    for (void (*kern)(const EdgeParams) : {tdes_edges_kernel<true, 0, 0>, tdes_edges_kernel<false, 0, 0>, tdes_edges_kernel<false, 32, 128>,
+                                           tdes_edges_kernel<false, 16, 128>, tdes_edges_kernel<false, 8, 128>})
+        if (e == cudaSuccess) e = allow_smem((const void*)kern, bytes);
     return e;
 }
 

@@ -853,13 +853,9 @@ cudaError_t tdes_loss_launch(graft_ctx* ctx, const graft_tdes_traces* tr, const 
 }
 
 cudaError_t tdes_loss_configure(const graft_config& cfg) {
-    const int smem = (int)tdes_loss_smem(cfg);
-    if (smem <= 48 * 1024) return cudaSuccess;
-    if (cfg.m <= 128) return cudaFuncSetAttribute(rows_kernel(cfg), cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    cudaError_t e = cudaFuncSetAttribute(tdes_loss_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(tdes_loss_kernel<kTrMaxChunks>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    return e;
+    const size_t smem = tdes_loss_smem(cfg);
+    if (cfg.m <= 128) return allow_smem((const void*)rows_kernel(cfg), smem);
+    return allow_smem((const void*)(cfg.m <= 256 ? tdes_loss_kernel<2> : tdes_loss_kernel<kTrMaxChunks>), smem);
 }
 bool tdes_loss_supported(const graft_config& cfg) { return cfg.m % 4 == 0 && cfg.m <= 128 * kTrMaxChunks; }
 

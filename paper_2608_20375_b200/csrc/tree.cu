@@ -1767,11 +1767,10 @@ static TreeInstance tree_pick(const graft_config& cfg, bool usual, bool neutral)
 }
 
 cudaError_t tree_configure(const graft_config& cfg) {
-    const int bytes = (int)tree_smem_bytes(cfg);
+    const size_t bytes = tree_smem_bytes(cfg);
     cudaError_t e = cudaSuccess;
-#pragma unroll 1
     for (int i = 0; i < 4 && e == cudaSuccess; ++i)
-        e = cudaFuncSetAttribute(tree_pick(cfg, (i & 1) != 0, (i & 2) != 0).kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+        e = allow_smem((const void*)tree_pick(cfg, (i & 1) != 0, (i & 2) != 0).kernel, bytes);
     return e;
 }
 

@@ -213,3 +213,35 @@ def test_micro_batches_on_streams_of_their_own():
     for g, *_ in ctxs:
         g.set_hist_window(0)
         g.destroy()
+
+
+@pytest.mark.parametrize("K,m,beta", [(32, 128, 0.2), (32, 128, 0.0), (8, 124, 0.2), (11, 64, 0.2)])
+def test_a_later_smaller_context_takes_no_shared_memory_from_an_older_one(K, m, beta):
+    """The limit on a kernel's dynamic shared memory is the kernel's on the device: a context of smaller sizes that runs
+    the same instances, created while a larger one lives, must leave the larger one's rounds and training steps alone."""
+    w = gi.small(batch=2, L=16, V=2003, K=K, budget_min=16, budget_max=400, budget_step=16, m=m, hidden_dim=32, beta=beta)
+    g, _, _, keep = _graft(w)
+    x = gi.batch_inputs(w)
+    tr = gi.tdes_traces(w.V, w.L, K, 20, 30, 40, seed=3)
+    groups = {k: torch.from_numpy(np.ascontiguousarray(v)).cuda() for k, v in tr["groups"].items()}
+    pairs, edges = torch.from_numpy(tr["pairs"]).cuda(), torch.from_numpy(tr["edges"]).cuda()
+    loss = torch.empty((2, 4), dtype=torch.float64, device="cuda")
+
+    def work(i):
+        _, gpu = gpu_round(g, w, x)          # every depth scored ahead, the score array asked for
+        _, plain = gpu_round(g, w, x, debug=False)
+        g.tdes_loss(groups, pairs, edges, gamma=0.5, w1=4.0, lambda_kl=1.0, lambda_pair=1.0, lambda_bce=0.25, loss=loss[i])
+        torch.cuda.synchronize()
+        return gpu, plain
+
+    before = work(0)
+    small = gi.small(batch=2, L=4, V=2003, K=K, budget_min=16, budget_max=64, budget_step=16, m=16 if m == 64 else m,
+                     hidden_dim=32, beta=beta)
+    g2, _, _, keep2 = _graft(small)
+    after = work(1)
+    for a, b in zip(before, after):
+        for k in a:
+            assert np.array_equal(a[k], b[k], equal_nan=True), k
+    assert torch.allclose(loss[0], loss[1], rtol=1e-12)  # (64-bit sums in no fixed order)
+    g2.destroy()
+    g.destroy()
