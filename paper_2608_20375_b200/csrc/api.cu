@@ -18,6 +18,7 @@ using namespace graft;
 namespace {
 
 constexpr int kTimingRing = 64;
+constexpr int kMaxOldTables = 16;  // (each at least twice the one before)
 
 struct Timing {
     cudaEvent_t ev[kTimingRing][4];
@@ -50,9 +51,39 @@ struct CtxExtra {
     char* d_in = nullptr;
     char* d_out = nullptr;
     size_t in_bytes = 0, out_bytes = 0;
+    // scratch of the table precompute that became too small
+    void* old_tables[kMaxOldTables];
+    int n_old_tables = 0;
 };
 
 CtxExtra* extra_of(graft_ctx* ctx) { return (CtxExtra*)ctx->stage; }
+
+// Scratch of the tensor-core table precompute, `need` bytes at least, or NULL if there is no memory for it.  It comes with
+// the first call that needs it, be it under stream capture: the allocation is made outside of any capture.  A captured call
+// keeps the address, so scratch that has become too small lives on until the context goes; a new piece is at least twice
+// the size of the last, so that all the old ones together are smaller than the one in use.
+void* tables_scratch(graft_ctx* ctx, size_t need) {
+    if (ctx->tables_scratch_bytes >= need) return ctx->tables_scratch;
+    CtxExtra* ex = extra_of(ctx);
+    if (ctx->tables_scratch && ex->n_old_tables == kMaxOldTables) return nullptr;
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    const size_t bytes = need > 2 * ctx->tables_scratch_bytes ? need : 2 * ctx->tables_scratch_bytes;
+    void* buf = nullptr;
+    if (cudaMalloc(&buf, bytes) != cudaSuccess) {
+        cudaGetLastError();
+        buf = nullptr;
+    }
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    if (buf == nullptr) return nullptr;
+    if (ctx->tables_scratch) ex->old_tables[ex->n_old_tables++] = ctx->tables_scratch;
+    ctx->tables_scratch = buf;
+    ctx->tables_scratch_bytes = bytes;
+    return buf;
+}
 
 }  // namespace
 
@@ -178,6 +209,7 @@ graft_status graft_destroy(graft_ctx* ctx) {
                 for (int j = 0; j < 4; ++j) cudaEventDestroy(ex->timing.ev[i][j]);
         if (ex->d_in) cudaFree(ex->d_in);
         if (ex->d_out) cudaFree(ex->d_out);
+        for (int i = 0; i < ex->n_old_tables; ++i) cudaFree(ex->old_tables[i]);
         delete ex;
     }
     if (ctx->tables_scratch) cudaFree(ctx->tables_scratch);
@@ -249,26 +281,15 @@ graft_status graft_tdes_precompute(graft_ctx* ctx, const void* d_emb, graft_dtyp
                                    const float* d_W, const float* d_b, float* d_out, void* stream) {
     if (!ctx || !d_emb || !d_W || !d_out || E < 1) return GRAFT_ERR_INVALID_ARG;
     if (emb_dtype != GRAFT_F32 && emb_dtype != GRAFT_BF16) return GRAFT_ERR_INVALID_ARG;
-    // the tensor cores (bf16 parts of the inputs, exact products); their scratch is allocated on the first call (this is
-    // the once-per-model setup step, not the round)
+    // the tensor cores (bf16 parts of the inputs, exact products), where the rows fit and their scratch is to be had
     if (tables_mma_fits(d_emb, emb_dtype, E, d_out)) {
-        const size_t need = tables_mma_scratch_bytes(ctx->num_sms, E, ctx->cfg.m, emb_dtype);
-        if (ctx->tables_scratch_bytes < need) {
-            if (ctx->tables_scratch) cudaFree(ctx->tables_scratch);
-            ctx->tables_scratch = nullptr;
-            ctx->tables_scratch_bytes = 0;
-            if (cudaMalloc(&ctx->tables_scratch, need) != cudaSuccess) {
-                cudaGetLastError();
-                return GRAFT_ERR_WORKSPACE;
-            }
-            ctx->tables_scratch_bytes = need;
-        }
-        if (tables_mma_launch(ctx, d_emb, emb_dtype, E, d_W, d_b, d_out, ctx->tables_scratch, (cudaStream_t)stream) !=
-            cudaSuccess) {
+        void* scratch = tables_scratch(ctx, tables_mma_scratch_bytes(ctx->num_sms, E, ctx->cfg.m, emb_dtype));
+        if (scratch != nullptr) {
+            if (tables_mma_launch(ctx, d_emb, emb_dtype, E, d_W, d_b, d_out, scratch, (cudaStream_t)stream) == cudaSuccess)
+                return GRAFT_OK;
             cudaGetLastError();
             return GRAFT_ERR_CUDA;
         }
-        return GRAFT_OK;
     }
     if (tdes_precompute_launch(ctx, d_emb, emb_dtype, E, d_W, d_b, d_out, (cudaStream_t)stream) != cudaSuccess)
         return GRAFT_ERR_CUDA;
