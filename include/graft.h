@@ -136,7 +136,8 @@ int32_t graft_edge_rows(const graft_ctx* ctx);
  * d_W [m, E] fp32, d_b [m] fp32 or NULL, d_out [V, m] fp32.  fp32 accumulation.  Call once per tower.
  * With d_emb and d_out 16-byte aligned and E a multiple of 8 (bf16) or 4 (fp32) the products run on the tensor cores:
  * fp32 numbers enter as three bf16 parts, whose products are exact, so the result differs from a fp32 FMA one only by
- * the order of the additions (an infinite entry gives NaN).
+ * the order of the additions.  With fp32 embeddings, infinities and values up to the largest fp32 give what fp32 arithmetic
+ * gives; a bf16 embedding or a W beside bf16 embeddings that is infinite, or a W that rounds past the largest bf16, gives NaN.
  * Such calls use scratch of the context (3 m E bf16 values and up to 40 MB of partial sums, m rounded up to 128), which the
  * first of them allocates and one that needs more replaces -- under stream capture too; a captured call keeps the scratch it
  * was captured with until the context is destroyed.  Without memory for it, and for other pointers and E, an FMA kernel

@@ -91,11 +91,13 @@ struct TablesRing {
 struct __align__(64) TablesParams {
     CUtensorMap map_w;  // [3 * m_pad, E_pad] bf16
     CUtensorMap map_e;  // [V, E] embeddings
+    const void* emb;    // [V, E]
+    const float* W;     // [m, E]
     const float* bias;  // [m] or NULL
     float* out;         // [V, m]
     float* pieces;      // [pairs][2 pieces][ROWS][128]
     int32_t* errflag;
-    int V, m, m_pad, n_mb, n_kb;
+    int V, E, m, m_pad, n_mb, n_kb;
     int pairs, full_rounds;
     int left, share_pairs;  // left-over tiles, pairs that share them
     int box_n;              // fp32 embeddings: rows of W's boxes
@@ -191,6 +193,19 @@ __device__ __forceinline__ float4 ld_shared_f4(uint32_t at) {
     return v;
 }
 
+// fp32 embeddings: an entry whose bf16 parts are not all finite -- an infinity, a value that rounds past the largest bf16 --
+// turns every result it has a part in into a NaN or an infinity.  Results that are not finite are worked out again as one
+// chain of fp32 multiply-adds, which gives what fp32 arithmetic gives; such entries are rare, so the time does not matter.
+__device__ __forceinline__ bool tables_finite(float x) { return fabsf(x) <= 3.402823466e38f; }
+__device__ __noinline__ float tables_fp32(const TablesParams& p, int v, int c) {
+    const float* e = (const float*)p.emb + (size_t)v * p.E;
+    const float* w = p.W + (size_t)c * p.E;
+    float a = 0.f;
+#pragma unroll 8
+    for (int k = 0; k < p.E; ++k) a = fmaf(__ldg(e + k), __ldg(w + k), a);
+    return a + (p.bias ? p.bias[c] : 0.f);
+}
+
 template <bool F32>
 __global__ void __cluster_dims__(F32 ? 1 : 2, 1, 1) __launch_bounds__(TablesCfg<F32>::THREADS, 1)
     tables_mma_kernel(const __grid_constant__ TablesParams p) {
@@ -200,6 +215,7 @@ __global__ void __cluster_dims__(F32 ? 1 : 2, 1, 1) __launch_bounds__(TablesCfg<
     __shared__ __align__(8) uint64_t bars[2 * (NA + NW + NR) + 4];
     __shared__ uint32_t s_tmem;
     __shared__ volatile int s_abort;
+    __shared__ bool s_mend;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const uint32_t rank = C::PAIR ? cluster_ctarank() : 0u;
     const int pair = C::PAIR ? (int)blockIdx.x >> 1 : (int)blockIdx.x;
@@ -235,6 +251,7 @@ __global__ void __cluster_dims__(F32 ? 1 : 2, 1, 1) __launch_bounds__(TablesCfg<
         }
         mbar_fence_init();
         s_abort = 0;
+        s_mend = false;
     }
     pdl_launch_dependents();  // (the kernel that adds up the pieces; it waits for this grid)
     if (warp == 9) tmem_alloc<C::PAIR>(smem_u32(&s_tmem), 512);
@@ -252,6 +269,7 @@ __global__ void __cluster_dims__(F32 ? 1 : 2, 1, 1) __launch_bounds__(TablesCfg<
         const int half = warp >> 2, quarter = warp & 3;
         const uint32_t accempty_even = mapa_u32(accempty0, 0);
         uint32_t cc = 0;  // chunks emptied so far
+        float check = 0.f;  // fp32 embeddings: NaN once a result of this thread was not finite
         for (int i = 0; tables_item(p, pair, i, it); ++i) {
             const int rt = it.tile / p.n_mb, mb = it.tile - rt * p.n_mb;
             const uint32_t n = (uint32_t)tables_n<F32>(p, mb);
@@ -309,6 +327,11 @@ __global__ void __cluster_dims__(F32 ? 1 : 2, 1, 1) __launch_bounds__(TablesCfg<
                             for (int k = 0; k < 8; ++k)
                                 if (k < 4 || both) acc[h][c + k] += __ldg(bias + c + k);
                         }
+                        if (F32 && !piece) {
+#pragma unroll
+                            for (int k = 0; k < 8; ++k)
+                                if (k < 4 || both) check = fmaf(0.f, acc[h][c + k], check);
+                        }
                         if (wide) {  // (both: m is a multiple of 8)
                             st_global_v8(dst + c, &acc[h][c]);
                         } else {
@@ -317,6 +340,22 @@ __global__ void __cluster_dims__(F32 ? 1 : 2, 1, 1) __launch_bounds__(TablesCfg<
                                 *(float4*)(dst + c + 4) = make_float4(acc[h][c + 4], acc[h][c + 5], acc[h][c + 6], acc[h][c + 7]);
                         }
                     }
+                }
+            }
+        }
+        if (F32) {  // (nothing waits for these warps any more)
+            if (check != 0.f) s_mend = true;
+            __syncwarp();
+            named_bar_sync(1, kTmEpiWarps * 32);  // (the tiles are written for every thread of these warps)
+            if (s_mend && !s_abort) {
+                for (int i = 0; tables_item(p, pair, i, it); ++i) {
+                    if (it.q0 != it.q1) continue;  // (pieces: the kernel that adds them up)
+                    const int rt = it.tile / p.n_mb, c0 = (it.tile - rt * p.n_mb) * 128;
+                    for (int v = rt * C::ROWS + warp; v < p.V && v < (rt + 1) * C::ROWS; v += kTmEpiWarps)
+                        for (int c = c0 + lane; c < p.m && c < c0 + 128; c += 32) {
+                            float* o = p.out + (size_t)v * p.m + c;
+                            if (!tables_finite(*o)) *o = tables_fp32(p, v, c);
+                        }
                 }
             }
         }
@@ -526,7 +565,14 @@ __global__ void __launch_bounds__(256) tables_pieces_kernel(const __grid_constan
         const float* b = p.bias + mb * 128 + c;
         s.x += b[0], s.y += b[1], s.z += b[2], s.w += b[3];
     }
-    *(float4*)(p.out + (size_t)(rt * C::ROWS + v) * p.m + mb * 128 + c) = s;
+    const int row = rt * C::ROWS + v, col = mb * 128 + c;
+    if (F32) {
+        if (!tables_finite(s.x)) s.x = tables_fp32(p, row, col);
+        if (!tables_finite(s.y)) s.y = tables_fp32(p, row, col + 1);
+        if (!tables_finite(s.z)) s.z = tables_fp32(p, row, col + 2);
+        if (!tables_finite(s.w)) s.w = tables_fp32(p, row, col + 3);
+    }
+    *(float4*)(p.out + (size_t)row * p.m + col) = s;
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
@@ -606,11 +652,14 @@ cudaError_t tables_mma_launch(graft_ctx* ctx, const void* d_emb, graft_dtype dt,
     if (!encode_map(&p.map_w, w, false, (uint64_t)3 * s.m_pad, s.E_pad, f32 ? p.box_n : 64, 2 * blk) ||
         !encode_map(&p.map_e, d_emb, f32, V, E, 128, 128))
         return cudaErrorUnknown;
+    p.emb = d_emb;
+    p.W = d_W;
     p.bias = d_b;
     p.out = d_out;
     p.pieces = (float*)scratch;
     p.errflag = ctx->w_errflag;
     p.V = V;
+    p.E = E;
     p.m = m;
     p.m_pad = s.m_pad;
     p.n_mb = s.n_mb;

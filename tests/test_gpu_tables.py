@@ -82,3 +82,27 @@ def test_no_memory_for_the_scratch(dtype):
     assert (out - want).abs().max() < 2e-5
     assert (odd - _exact(emb[:, :E - 1], W[:, :E - 1], b)).abs().max() < 2e-5
     assert (_call(g, emb, W, b, m) - want).abs().max() < 2e-5  # and with memory again
+
+
+@pytest.mark.parametrize("V,E,m", [(300, 64, 128), (19300, 1092, 40), (40003, 132, 256)])  # whole tiles, pieces, both
+def test_fp32_entries_that_bf16_parts_cannot_hold(V, E, m):
+    """Infinities, NaN and finite values that round past the largest bf16, in the embeddings and in W: what fp32 arithmetic
+    gives, and nothing else is touched."""
+    emb, W, b = _inputs(V, E, m, "f32", 5)
+    inf, huge = float("inf"), 3.4e38
+    emb[:, 0] *= 0.1  # (times -huge, below: finite, on the way too)
+    for v, x in ((0, inf), (1, -inf), (2, huge), (3, -huge), (4, float("nan")), (V // 2, inf), (V - 1, huge)):
+        emb[v, (7 * v) % E] = x
+    emb[5, 3], emb[5, 9] = inf, -inf
+    emb[6] = 0.0
+    W[0, 5], W[m - 1, 0] = inf, -huge
+    W[:, 1] = 0.0
+    emb[7, 1] = inf       # (infinity times zero)
+    got = _call(_graft(V, m), emb, W, b, m).double()
+    want = _exact(emb, W, b)
+    over = want.abs() > 3.4028234e38  # past fp32 (with the sums' rounding to either side of the limit, none is near it)
+    want[over] = want[over].sign() * inf
+    assert torch.equal(got.isnan(), want.isnan())
+    assert torch.equal(got.isinf(), want.isinf()) and torch.equal(got[got.isinf()], want[want.isinf()])
+    fin = want.isfinite()
+    assert ((got - want)[fin].abs() <= 2e-5 + 2e-6 * want[fin].abs()).all()
