@@ -342,7 +342,7 @@ class Graft:
     def accept(self, trees: TreeOut, target_next, accept_len, accept_path, bonus_token):
         batch = target_next.shape[0]
         i32 = torch.int32
-        oc = _TreeOut(d_n_nodes=_ptr(trees.n_nodes, i32), d_token=_ptr(trees.token, i32), d_parent=_ptr(trees.parent, i32))
+        oc = trees._c()  # (accept reads three of the arrays; a wrong one among the others is still the caller's mistake)
         _check(self.lib, self.lib.graft_accept(self._ctx, batch, C.byref(oc), _ptr(target_next, i32),
                                                _ptr(accept_len, i32), _ptr(accept_path, i32),
                                                _ptr(bonus_token, i32), _stream()), "graft_accept")

@@ -245,3 +245,23 @@ def test_a_later_smaller_context_takes_no_shared_memory_from_an_older_one(K, m, 
     assert torch.allclose(loss[0], loss[1], rtol=1e-12)  # (64-bit sums in no fixed order)
     g2.destroy()
     g.destroy()
+
+
+@pytest.mark.parametrize("field", ["mask", "budget", "depth", "position", "path_score", "status"])
+@pytest.mark.parametrize("wrong", ["cpu", "dtype", "strides"])
+def test_accept_refuses_a_wrong_tree(field, wrong):
+    """Every array of the tree is looked at, whether the walk reads it or not."""
+    from paper_2608_20375_b200 import GraftError
+    w = gi.small(batch=2, L=4, V=300, K=4, budget_min=8, budget_max=16, budget_step=8, m=16, hidden_dim=8)
+    g, _, _, keep = _graft(w)
+    out, _ = gpu_round(g, w, gi.batch_inputs(w))
+    tn = torch.zeros((2, g.nmax), dtype=torch.int32, device="cuda")
+    a, path, bonus = (torch.empty(s, dtype=torch.int32, device="cuda") for s in ((2,), (2, w.L), (2,)))
+    g.accept(out, tn, a, path, bonus)
+    t = getattr(out, field)
+    setattr(out, field, t.cpu() if wrong == "cpu" else t.to(torch.int64) if wrong == "dtype" else
+            torch.stack([t, t], -1)[..., 0])
+    with pytest.raises(GraftError):
+        g.accept(out, tn, a, path, bonus)
+    torch.cuda.synchronize()
+    g.destroy()
