@@ -315,8 +315,8 @@ __global__ void __launch_bounds__(kTrThreads) tdes_loss_kernel(const TrainParams
 //   * every warp adds into a copy of gu of its own (a plain load, add and store);
 //   * the few hottest tokens' gradient rows (additions to one row serialise in L2) are picked once per CTA from a sample of
 //     the tokens, and every warp keeps its sums of them in shared memory; everything else is a 16-byte vector atomic.
-// Measured (B200, V = 151,936, m = 128, L = 16, 32,768 groups of 32, 131,072 pairs, 262,144 edges): 337 us (434 us by the
-// one-item-a-warp kernel with replaced cached rows).  What bounds it now: the vector atomics -- a million rows spread
+// Measured (B200, V = 151,936, m = 128, L = 16, 32,768 groups of 32, 131,072 pairs, 262,144 edges): 323 us (420 us by the
+// one-item-a-warp kernel with replaced cached rows; 500 of 8, 2000 and 4000: 16.6 and 19.6 us).  What bounds it now: the vector atomics -- a million rows spread
 // evenly take 96 us whether from 8 or from 32 warps an SM or as bulk reductions from shared memory, a million with the
 // Zipf(1.1) tokens of these traces 790 us, without their eight hottest 152 us -- and, in front of them in the same
 // queue, 1.6 million row loads (138 us for the losses alone).  One copy of gu with atomics instead of one a warp leaves
@@ -324,7 +324,10 @@ __global__ void __launch_bounds__(kTrThreads) tdes_loss_kernel(const TrainParams
 constexpr int kTsThreads = 384;
 constexpr int kTsWarps = kTsThreads / 32;
 constexpr int kTsSample = 256;
-constexpr int kTsSampleMin = 16384;  // references to rows from which looking for hot ones (about 2 us) is worth it
+// References to rows from which looking for hot ones is worth its time (10 us: two rounds of loads, 256 x 256 compares).
+// With and without: 41 thousand references 26.8 and 22.8 us, 65 thousand 34.0 and 26.7, 74 thousand 33.0 and 35.0, 164
+// thousand 47.4 and 61.0.
+constexpr int kTsSampleMin = 65536;
 
 constexpr int kTsSlots = 8;  // hot rows per table
 struct __align__(16) TrainHot {
@@ -441,6 +444,14 @@ __device__ __forceinline__ int train_sample(const TrainParams& p, int t, int i) 
     return tok >= 0 && tok < p.V ? tok : -1;
 }
 
+// The work is one list -- groups, blocks of eight pairs, blocks of eight edges -- dealt to the warps in turn: the first of a
+// kind, with `ahead` entries of other kinds ahead of it, that warp wid of nw gets.  (Dealt kind by kind, the first warps got
+// one of each, one after the other, while the rest had nothing: half of a small call's time.)
+__device__ __forceinline__ int first_block(int wid, long long ahead, int nw) {
+    const int r = wid - (int)(ahead % nw);
+    return r < 0 ? r + nw : r;
+}
+
 // KC: children held in registers, a multiple of 8 (K <= KC)
 template <int KC, bool FULL>
 __global__ void __launch_bounds__(kTsThreads, 1) tdes_loss_rows_kernel(const TrainParams p) {
@@ -466,8 +477,9 @@ __global__ void __launch_bounds__(kTsThreads, 1) tdes_loss_rows_kernel(const Tra
     c.m = p.m;
     for (int i = tid; i < Lm; i += kTsThreads) smem_f[i] = p.u[i];
     if (grad) {
-        for (int i = tid; i < Lm * p.gu_copies; i += kTsThreads) s_gu[i] = 0.f;
-        for (int i = tid; i < kTsWarps * 2 * kTsSlots * 128; i += kTsThreads) s_rows[i] = 0.f;
+        for (int i = tid; i < Lm / 4 * p.gu_copies; i += kTsThreads) ((float4*)s_gu)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (p.sample)
+            for (int i = tid; i < kTsWarps * 2 * kTsSlots * 32; i += kTsThreads) ((float4*)s_rows)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
     if (tid < 3) s_loss[tid] = 0.0;
     if (tid == 0) {
@@ -579,7 +591,7 @@ __global__ void __launch_bounds__(kTsThreads, 1) tdes_loss_rows_kernel(const Tra
         ctx_add_u<FULL>(c, d, acc);
     }
     // ---- pairwise level (Eq. 10): blocks of eight pairs, four at a time; lanes 0-7 hold the block's ids
-    for (int b0 = wid * 8; b0 < p.n_pairs; b0 += nw * 8) {
+    for (int b0 = first_block(wid, p.n_groups, nw) * 8; b0 < p.n_pairs; b0 += nw * 8) {
         int id[6] = {0, 0, 1, 0, 0, 1};
         bool ok = false;
         if (lane < 8 && b0 + lane < p.n_pairs) {
@@ -664,7 +676,7 @@ __global__ void __launch_bounds__(kTsThreads, 1) tdes_loss_rows_kernel(const Tra
         }
     }
     // ---- edge level (Eq. 11): eight edges at a time; lanes 0-7 hold their ids
-    for (int b0 = wid * 8; b0 < p.n_edges; b0 += nw * 8) {
+    for (int b0 = first_block(wid, p.n_groups + (p.n_pairs + 7ll) / 8, nw) * 8; b0 < p.n_edges; b0 += nw * 8) {
         int tp = 0, tc = 0, d = 1, y = 0;
         bool ok = false;
         if (lane < 8 && b0 + lane < p.n_edges) {
@@ -736,7 +748,7 @@ __global__ void __launch_bounds__(kTsThreads, 1) tdes_loss_rows_kernel(const Tra
             for (int w = 1; w < p.gu_copies; ++w) v += s_gu[(size_t)w * Lm + i];
             if (v != 0.f) atomicAdd(p.gu + i, v);
         }
-        for (int i = tid; i < 2 * kTsSlots * 32; i += kTsThreads) {
+        for (int i = tid; p.sample && i < 2 * kTsSlots * 32; i += kTsThreads) {
             const int r = i >> 5, l = i & 31, tok = s_hot.tok[r / kTsSlots][r % kTsSlots];
             if (tok < 0 || l >= p.m / 4) continue;
             float4 v = zero4;
@@ -825,9 +837,8 @@ cudaError_t tdes_loss_launch(graft_ctx* ctx, const graft_tdes_traces* tr, const 
         p.acc = ctx->w_loss;
         p.gu_copies = rows_gu_copies(cfg);
         p.sample = (long long)tr->n_groups * (cfg.K + 1) + 4ll * tr->n_pairs + 2ll * tr->n_edges >= kTsSampleMin;
-        long long work = tr->n_groups;  // a warp takes a group, eight pairs or eight edges at a time
-        if (work < (tr->n_pairs + 7) / 8) work = (tr->n_pairs + 7) / 8;
-        if (work < (tr->n_edges + 7) / 8) work = (tr->n_edges + 7) / 8;
+        // a warp takes a group, eight pairs or eight edges at a time
+        const long long work = (long long)tr->n_groups + (tr->n_pairs + 7ll) / 8 + (tr->n_edges + 7ll) / 8;
         long long grid = (work + kTsWarps - 1) / kTsWarps;
         if (grid > ctx->num_sms) grid = ctx->num_sms;
         rows_kernel(cfg)<<<(int)grid, kTsThreads, smem, st>>>(p);

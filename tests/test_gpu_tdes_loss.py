@@ -66,11 +66,19 @@ def _compare(got, ref, grad=True):
     (1500, 4, 8, 256, 200, 300, 0),         # two 128-float chunks per row, no edges
     (1200, 3, 7, 384, 150, 150, 150),       # three chunks
     (900, 32, 1, 8, 100, 100, 100),         # K = 1: pi = 1, the distribution term vanishes
-    (5000, 16, 8, 128, 1801, 3001, 4007),   # children held eight at a time, enough rows to look for hot ones
+    (5000, 16, 8, 128, 1801, 3001, 4007),   # children held eight at a time
     (5000, 16, 9, 128, 1500, 2500, 3003),   # sixteen
     (5000, 32, 16, 128, 1500, 2500, 3003),  # one copy of gu (L m > 2048)
     (5000, 16, 17, 124, 1000, 2500, 3003),  # thirty-two, lanes without a part of a row
     (400, 16, 4, 64, 7, 9, 17),             # less than a block of items
+    (5000, 16, 8, 128, 3601, 5001, 7007),   # enough references to look for hot rows: every instance
+    (5000, 16, 9, 128, 3300, 5000, 7003),
+    (5000, 32, 16, 128, 2100, 5000, 7003),
+    (5000, 16, 17, 124, 2000, 5000, 5003),
+    (5000, 16, 8, 124, 3601, 5001, 7007),
+    (5000, 16, 32, 128, 1301, 3001, 7007),
+    (700, 16, 8, 128, 1, 0, 3000),          # blocks of edges behind one group, and behind pairs alone: where a warp's first is
+    (700, 16, 8, 128, 0, 3001, 9),
 ])
 def test_loss_and_gradients(V, L, K, m, ng, npair, ne):
     g, P, Ct, u, s, keep = _ctx(V, L, K, m, seed=V + m)
