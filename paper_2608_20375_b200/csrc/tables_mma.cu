@@ -21,7 +21,7 @@
 // rows halve the passes over W, which comes from L2 every time.  The fp32 kernel works on single CTAs because its rows
 // go through threads: telling the other CTA of a pair about every block cost more (136 - 160 us at V = 32,000, E = 2048)
 // than the second CTA's half of W saves (120 us).  The embeddings are read from memory once; nothing but the tables is
-// written.  What is left when the tiles do not divide by the workers is dealt out along E in equal shares, whose sums a
+// written.  What is left when the tiles do not divide by the workers is dealt out along E in shares, whose sums a
 // small kernel adds up in order (summing them inside, by the warp that came last, stalled its tile: 462 against 370 us).
 //
 // Measured (one tower, back to back, B200): V = 151,936, E = 4096, m = 128, bf16: 373 us (798 us with the library
@@ -673,6 +673,17 @@ cudaError_t tables_mma_launch(graft_ctx* ctx, const void* d_emb, graft_dtype dt,
     long long sp = s.pairs;
     if (sp > (long long)p.left * kTmMaxSplit) sp = (long long)p.left * kTmMaxSplit;
     if (sp > (long long)p.left * p.n_kb * blk / 256) sp = (long long)p.left * p.n_kb * blk / 256;
+    if (sp > p.left) {
+        // Shares of equal length that cut tiles anywhere, or a whole number q of shares a tile on fewer workers?  A share that
+        // lies in two tiles empties its accumulators and writes a piece twice, and with q = 1 nothing has to be added up:
+        // the whole number saves 6 us on pairs and 3 us on single CTAs, 22 and 10 us for q = 1, and costs 0.02 and 0.03 us
+        // for every column of E by which a share gets longer.  (Measured over 26 to 73 and 52 to 147 tiles left, E = 1024 to
+        // 4096, with and without a round of whole tiles ahead.  V = 16,000, bf16: E = 1024 35.0 -> 29.2 us, E = 4096 61.5 ->
+        // 57.9; V = 32,000, E = 1024: bf16 47.5 -> 32.7, fp32 71.9 -> 68.4; fp32, E = 2048 stays: 118.7 against 121.2.)
+        const long long q = sp / p.left;
+        const double longer = (1.0 / (double)q - (double)p.left / (double)sp) * E;
+        if (longer <= (f32 ? (q == 1 ? 380 : 130) : (q == 1 ? 850 : 350))) sp = q * p.left;
+    }
     p.share_pairs = (int)(sp < p.left ? p.left : sp);
     p.wide = m % 8 == 0 && ((uintptr_t)d_out & 31) == 0;
     weight_split_kernel<<<dim3((s.E_pad + 511) / 512, s.m_pad), 256, 0, st>>>(d_W, m, E, s.m_pad, s.E_pad, w);

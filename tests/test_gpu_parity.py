@@ -394,15 +394,19 @@ def test_vocab_pass_is_reproducible_and_counters_reset():
     (500, 100, 16, "bf16"),     # E not a multiple of 8: the FMA kernel
     (777, 200, 24, "f32"),
     (70001, 2048, 8, "bf16"),   # tensor-core path at the sizes it runs at: several tiles a pair of CTAs
-    (66000, 1096, 24, "bf16"),  # left-over tiles cut in two along E, a last block of 8 columns
-    (19200, 2048, 8, "bf16"),   # one left-over tile, cut into the most pieces
+    (66000, 1096, 24, "bf16"),  # left-over tiles whole, one a pair, a last block of 8 columns
+    (19200, 2048, 8, "bf16"),   # shares of the left-over tiles that lie in two of them
+    (13000, 1096, 24, "bf16"),  # two shares a left-over tile
+    (38300, 2048, 8, "bf16"),   # one left-over tile, cut into the most pieces
+    (9700, 1024, 24, "f32"),    # single CTAs: shares that lie in two tiles
+    (16000, 1024, 24, "f32"),   # left-over tiles whole
     (4, 8, 4, "bf16"),          # the smallest
     (385, 72, 512, "bf16"),     # four blocks of m, the second CTA's rows of the last tile outside
     (500, 101, 16, "f32"),      # E not a multiple of 4: the FMA kernel
     (4, 4, 4, "f32"),
     (5003, 516, 300, "f32"),    # three blocks of m, the last ragged; a last block of 4 columns
-    (19300, 1092, 40, "f32"),   # left-over tiles in pieces
-    (40003, 640, 128, "f32"),   # several tiles a pair
+    (19300, 1092, 40, "f32"),   # four shares a left-over tile
+    (40003, 640, 128, "f32"),   # several tiles a CTA, two shares a left-over tile
 ])
 def test_tdes_precompute_against_oracle(V, E, m, emb_dtype):
     L = 4
