@@ -447,16 +447,24 @@ __device__ __forceinline__ int warp_append(uint64_t* buf, int n, int cap, bool p
 }
 
 // Exact top-K of cand[0..n) by rank counting; result sorted descending in outk[0..min(n,K)).  Keys are
-// distinct (ids are), so ranks are a permutation.
-__device__ void warp_select_topk(EpiShared* sh, int n, int K, int lane) {
+// distinct (ids are), so ranks are a permutation.  One warp's n^2 compares are most of the exact selection's time: two keys a
+// lane, unrolled, unlike the loops around it (one key, not unrolled: sorted rows 140 us a launch at batch 64 against 104, ramps
+// with ties 308 against 204).  Out of line: inlined, the longer code costs every ordinary launch half a per cent.
+__device__ __noinline__ void warp_select_topk(EpiShared* sh, int n, int K, int lane) {
     __syncwarp();
 #pragma unroll 1
-    for (int i = lane; i < n; i += 32) {
-        const uint64_t key = sh->cand[i];
-        int rank = 0;
-#pragma unroll 1
-        for (int j = 0; j < n; ++j) rank += (sh->cand[j] > key) ? 1 : 0;
-        if (rank < K) sh->outk[rank] = key;
+    for (int i = lane; i < n; i += 64) {
+        const bool two = i + 32 < n;
+        const uint64_t k0 = sh->cand[i], k1 = two ? sh->cand[i + 32] : ~0ull;
+        int r0 = 0, r1 = 0;
+#pragma unroll 8
+        for (int j = 0; j < n; ++j) {
+            const uint64_t c = sh->cand[j];
+            r0 += c > k0 ? 1 : 0;
+            r1 += c > k1 ? 1 : 0;
+        }
+        if (r0 < K) sh->outk[r0] = k0;
+        if (two && r1 < K) sh->outk[r1] = k1;
     }
     __syncwarp();
 }
