@@ -973,15 +973,17 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
                     }
                     lvl_end = ntot + total;
                 }
-            } else if (n_grow <= NT / grp) {
-                // The last levels of nearly every tree: a thread per node finds the nodes that can have children by the best
-                // entry of their rows, then a group of lanes takes one of them each, a lane per entry.  No search along a
-                // row and none for a child's node: 1.8k cycles a level, the path below takes 3.1k.
-                int* wcnt = (int*)sm.hist;       // [32] such nodes per warp
-                int* list = (int*)sm.hist + 32;  // [32] those nodes in the order of the level, -1: none
-                int* ccnt = (int*)sm.hist + 64;  // [32] their children that reach theta
-                const uint32_t th_in = theta + ((TIES && d + 1 > th_depth) ? 1u : 0u);
-                const int x = b0 + tid;  // (a level of at most NT nodes)
+            } else {
+              // The last levels of nearly every tree: a thread per node finds the nodes that can have children by the best
+              // entry of their rows, then a group of lanes takes one of them each, a lane per entry.  No search along a
+              // row and none for a child's node: 1.8k cycles a level, the path below takes 3.1k.  The nodes are counted: if
+              // they were more than the groups take, or the table might not hold their children, that path has the level.
+              const uint32_t th_in = theta + ((TIES && d + 1 > th_depth) ? 1u : 0u);  // what a child's score must reach
+              int* list = (int*)sm.hist + 32;  // [32] those nodes in the order of the level, -1: none
+              bool few = n_grow <= NT / grp;
+              if (few) {
+                int* wcnt = (int*)sm.hist;  // [32] such nodes per warp
+                const int x = b0 + tid;     // (a level of at most NT nodes)
                 bool alive = false;
                 if (x < b1 && sm.nkey[x] >= theta) {
                     const int cx = (int)((sm.ninfo[x] >> 13) & 31u);
@@ -991,9 +993,14 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
                 if (lane == 0) wcnt[warp] = __popc(am);
                 if (tid < 32) list[tid] = -1;
                 __syncthreads();
-                const int at_list = (int)__reduce_add_sync(0xFFFFFFFFu, lane < warp ? (uint32_t)wcnt[lane] : 0u) +
-                                    __popc(am & ((1u << lane) - 1u));
-                if (alive && at_list < 32) list[at_list] = x;
+                const uint32_t wn = lane < NT / 32 ? (uint32_t)wcnt[lane] : 0u;
+                const int at_list = (int)__reduce_add_sync(0xFFFFFFFFu, lane < warp ? wn : 0u) + __popc(am & ((1u << lane) - 1u));
+                const int n_alive = (int)__reduce_add_sync(0xFFFFFFFFu, wn);
+                few = n_alive <= NT / grp && ntot + n_alive * K <= ncap;  // (uniform)
+                if (few && alive) list[at_list] = x;
+              }
+              if (few) {
+                int* ccnt = (int*)sm.hist + 64;  // [32] their children that reach theta
                 __syncthreads();
                 const int nd = tid / grp, r = tid % grp, xo = list[nd];
                 int c = 0;
@@ -1026,9 +1033,7 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
                 }
                 const int first = __shfl_sync(0xFFFFFFFFu, incl - v, nd);
                 lvl_end = ntot + __shfl_sync(0xFFFFFFFFu, incl, 31);
-                if (lvl_end > ncap) {  // (uniform)
-                    over = true;
-                } else if (take) {
+                if (take) {
                     if (d + 1 < L)  // (a row that is not scored yet: grow)
                         grow = d + 1 >= rows_done || ord_from_float(sc + sm.es[((d + 1) * K + c) * K + c]) >= theta ? 1 : 0;
                     const int at = ntot + first + __popc(mask & ((1u << c) - 1u));
@@ -1036,7 +1041,7 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
                     sm.nS[at] = sc;
                     sm.ninfo[at] = (uint32_t)xo | ((uint32_t)c << 13) | ((uint32_t)(d + 1) << 18) | ((uint32_t)r << 24);
                 }
-            } else {
+              } else {
                 // The children that can still matter are a prefix of a node's sorted row (scores only fall along the
                 // row); its length comes from a binary search.  The level is taken in chunks of NT nodes: one thread
                 // per node finds the length and the set of candidate ranks in that prefix, a scan of the lengths places
@@ -1057,7 +1062,7 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
                   int total = 0;
 #pragma unroll 1
                   for (int attempt = 0;; ++attempt) {  // (uniform: at most two rounds)
-                    const uint32_t th_in = theta + ((TIES && d + 1 > th_depth) ? 1u : 0u);  // what a child's score must reach
+                    const uint32_t th_in = theta + ((TIES && d + 1 > th_depth) ? 1u : 0u);  // (theta may have risen)
                     int cnt = 0;
                     uint32_t mask = 0u, kx = 0u;
                     float sx = 0.0f;
@@ -1164,6 +1169,7 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
                     if (c0 + NT < b1) __syncthreads();  // the scan space is reused by the next chunk
                 }
                 lvl_end = cur;
+              }
             }
             const int grown = __syncthreads_count(grow);  // (the level's nodes are in the table for every thread)
             const int nt = lvl_end;
