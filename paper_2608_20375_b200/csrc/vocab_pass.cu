@@ -1268,6 +1268,11 @@ __global__ void __launch_bounds__(kVpThreads, 1) vocab_pass_kernel(const VpParam
                         rec->nkeys = (uint32_t)nk | (sh->abort_flag ? 0x80000000u : 0u);
                     }
                     __syncwarp();
+#ifdef GRAFT_TEST_LATE_RECORDS
+                    // Test builds only: every CTA but the first waits some milliseconds here, so that a row of which CTA 0 has
+                    // a piece is merged by another.
+                    for (int i = 0; blockIdx.x != 0 && i < GRAFT_TEST_LATE_RECORDS; ++i) __nanosleep(1000000u);
+#endif
                     if (lane == 0) es->arrived = atom_add_acq_rel(p.row_counter + sg.row, 1);  // (the lanes' stores included)
                 }
                 epi_bar<ET>(grp);
