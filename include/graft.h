@@ -135,9 +135,11 @@ int32_t graft_edge_rows(const graft_ctx* ctx);
 /* Table precompute (same passage): d_out[v] = W e_v + b for one tower.  d_emb [V, E] (dtype as given),
  * d_W [m, E] fp32, d_b [m] fp32 or NULL, d_out [V, m] fp32.  fp32 accumulation.  Call once per tower.
  * With d_emb and d_out 16-byte aligned and E a multiple of 8 (bf16) or 4 (fp32) the products run on the tensor cores:
- * fp32 numbers enter as three bf16 parts, whose products are exact, so the result differs from a fp32 FMA one only by
- * the order of the additions.  With fp32 embeddings, infinities and values up to the largest fp32 give what fp32 arithmetic
- * gives; a bf16 embedding or a W beside bf16 embeddings that is infinite, or a W that rounds past the largest bf16, gives NaN.
+ * fp32 numbers enter as three bf16 parts, whose products are exact.  Against a chain of fp32 multiply-adds the result
+ * differs by the order and the rounding of the additions and, for fp32 embeddings, by the products left out, below 2^-26 of
+ * a term (largest error against fp64 products of N(0, 1) results 3.2e-6 at E = 4096, 3.0e-6 at E = 2048 in fp32; the chain:
+ * 1.2e-5).  With fp32 embeddings, infinities and values up to the largest fp32 give what fp32 arithmetic gives; a bf16
+ * embedding or a W beside bf16 embeddings that is infinite, or a W that rounds past the largest bf16, gives NaN.
  * Such calls use scratch of the context (3 m E bf16 values and up to 40 MB of partial sums, m rounded up to 128), which the
  * first of them allocates and one that needs more replaces -- under stream capture too; a captured call keeps the scratch it
  * was captured with until the context is destroyed.  Without memory for it, and for other pointers and E, an FMA kernel
@@ -153,7 +155,10 @@ graft_status graft_tdes_precompute(graft_ctx* ctx, const void* d_emb, graft_dtyp
  *   d_hist         [batch] hist_t = mean of the last w accepted lengths (Eq. 15); may be NULL iff fixed budget
  *   d_prefix_len   [batch] tokens in the prefix x^(t), the root included
  *   d_fixed_budget [batch] or NULL.  NULL: B_t from SABA.  Else B_t = clamp(value, 0, budget_max).
- * Requires graft_set_tdes_tables unless beta == 0 (then edge = log q and no table is read). */
+ * Requires graft_set_tdes_tables unless beta == 0 (then edge = log q and no table is read).
+ * Path scores that are equal but for the rounding of the rows' log-sum-exp -- with beta == 0 there can be hundreds -- are
+ * ordered by that rounding, whose last bit depends on how the rows are cut: on the batch, the sequence's place in it and the
+ * GPU.  The same call on the same GPU repeats bit for bit; graft_vocab_pass may cut the rows of such a round otherwise. */
 graft_status graft_build_trees(graft_ctx* ctx, int32_t batch, const void* d_logits, const void* d_hidden,
                                const int32_t* d_root_token, const float* d_hist, const int32_t* d_prefix_len,
                                const int32_t* d_fixed_budget, const graft_tree_out* out, void* stream);

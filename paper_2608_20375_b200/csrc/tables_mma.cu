@@ -4,9 +4,9 @@
 // Operands are bf16 parts of the inputs: an fp32 number is the sum of three bf16 ones (8 + 8 + 8 mantissa bits), and a
 // product of two bf16 numbers is exact in the fp32 accumulator.
 //   bf16 embeddings: out = e W1 + e W2 + e W3               (three products a step, all exact)
-//   fp32 embeddings: out = e1 W1 + (e1 W2 + e1 W3 + e2 W1 + e2 W2 + e3 W1)   (what is dropped is below 2^-23 of a term)
-// so the result differs from an fp32 GEMM only by the order of the additions.  The accumulators of the tensor cores
-// round less carefully than an FMA chain: they are emptied into fp32 registers after 32 (bf16) or 24 (fp32
+//   fp32 embeddings: out = (e1 + e2 + e3) W1 + ((e1 + e2 + e3) W2 + e1 W3)   (what is dropped is below 2^-26 of a term)
+// so the result differs from an fp32 GEMM by the order and the rounding of the additions.  The accumulators of the tensor
+// cores round less carefully than an FMA chain: they are emptied into fp32 registers after 32 (bf16) or 24 (fp32
 // embeddings) additions to the large products' accumulators, which W2's and W3's do not share.
 //
 // One persistent kernel.  A worker -- a pair of CTAs (cluster of two, tcgen05 cta_group::2) for bf16 embeddings, one CTA

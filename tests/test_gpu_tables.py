@@ -106,3 +106,47 @@ def test_fp32_entries_that_bf16_parts_cannot_hold(V, E, m):
     assert torch.equal(got.isinf(), want.isinf()) and torch.equal(got[got.isinf()], want[want.isinf()])
     fin = want.isfinite()
     assert ((got - want)[fin].abs() <= 2e-5 + 2e-6 * want[fin].abs()).all()
+
+
+@pytest.mark.parametrize("part", ["embedding", "W", "both"])
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_parts_of_every_order_count(part, dtype):
+    """Terms +-(1 + 2^-10 + t 2^-19) whose first and second parts cancel: the third parts are the whole result, exactly (all
+    sums are short multiples of powers of two)."""
+    if dtype == "bf16" and part != "W":
+        pytest.skip("bf16 embeddings have one part")
+    V, E, m = 1000, 2048, 128
+    g = torch.Generator(device="cuda").manual_seed(6)
+    sign = torch.where(torch.arange(E, device="cuda") % 2 == 0, 1.0, -1.0)
+    third = lambda n: 1.0 + 2.0 ** -10 + 2.0 ** -19 * torch.randint(0, 3, (n, E), generator=g, device="cuda")  # noqa: E731
+    emb = (third(V) if part != "W" else torch.ones((V, E), device="cuda")) * sign
+    W = third(m) if part != "embedding" else torch.ones((m, E), device="cuda")
+    got, want = _call(_graft(V, m), emb.to(DTYPES[dtype]), W, None, m).double(), _exact(emb, W)
+    assert want.abs().max() > 1e-5
+    # 2^-29 a term is left out where both numbers have three parts (second times third)
+    assert (got - want).abs().max() <= (2.0 ** -27 * E if part == "both" else 0.0)
+
+
+@pytest.mark.parametrize("V,E,m,dtype", [(8192, 4096, 128, "bf16"), (8192, 2048, 128, "f32")])
+def test_error_against_64_bit_products(V, E, m, dtype):
+    """N(0, 1) embeddings, results of N(0, 1): twice the largest error seen over a million results (3.2e-6 and 3.0e-6; a chain
+    of fp32 multiply-adds 1.2e-5)."""
+    emb, W, _ = _inputs(V, E, m, dtype, 8)
+    assert (_call(_graft(V, m), emb, W, None, m) - _exact(emb, W)).abs().max() <= 6e-6
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("off", ["embedding", "out", "neither"])
+def test_rows_off_the_16_byte_grid(dtype, off):
+    """Pointers that the tensor cores' copies cannot take go to the FMA kernel."""
+    V, E, m = 333, 72, 20
+    emb, W, b = _inputs(V, E, m, dtype, 9)
+    pad = torch.empty(V * E + 8, dtype=DTYPES[dtype], device="cuda")
+    o_pad = torch.full((V * m + 8,), 7.0, device="cuda")
+    i, j = (1 if off == "embedding" else 0), (1 if off == "out" else 0)
+    e2, out = pad[i:i + V * E].view(V, E), o_pad[j:j + V * m].view(V, m)
+    e2.copy_(emb)
+    _graft(V, m).tdes_precompute(e2, W, b, out)
+    torch.cuda.synchronize()
+    assert (out - _exact(emb, W, b)).abs().max() < 1e-5
+    assert (o_pad[:j] == 7.0).all() and (o_pad[j + V * m:] == 7.0).all()
