@@ -49,8 +49,7 @@ __device__ __forceinline__ int es_col(int r, int c, int K) {
 // `fma.rn.f32x2`), and takes a quarter ks of the m axis: two float4s of every eight.  A warp holds 2 x 4 such tiles in all
 // four quarters, so a step's T float4s of parents are one pass over the shared-memory banks each (8 places) and the T of
 // children two (16 places, no conflicts): 12 passes for 32 packed FMAs with T = 4, where a 4 x 2 tile a lane took 12 for
-// 16 and made shared memory the bound (a round of batch 1, K = 8: 29.7 -> 28.6 us; batch 16, K = 16: 47.8 -> 46.1;
-// batch 64, K = 32: 96.6 -> 95.1; batch 256: 295.4 -> 292.9).
+// 16 and made shared memory the bound (1 us of a round at batch 1, K = 8, 1.5 to 2.5 us at batch 16 to 256).
 // The pair is added at the end and the four quarters of a tile by two exchange steps; a sum's order of additions depends
 // on m alone, so the bits do not depend on T and G.
 // rP / rC: [.][ld] rows in shared memory, ld = m + 4 floats (16-byte aligned).

@@ -113,8 +113,7 @@ __global__ void __launch_bounds__(256, 4) tdes_edges_kernel(const EdgeParams p) 
     pdl_wait();               // the candidates come from the vocab pass
     // Sequences run fastest in the grid: the depth-0 units, whose budgets take longest, come first, and the depths that
     // only deep trees need behind those scored for every sequence (their CTAs mostly exit at once and should not take the
-    // places of CTAs with work).  No division stands in front of the first loads (batch 16: 44.4 -> 43.7 us a round; batch 64:
-    // 95.1 -> 94.8).
+    // places of CTAs with work).  No division stands in front of the first loads (0.7 us of a round at batch 16).
     const int b = blockIdx.x, j = blockIdx.y;
     if (j >= p.rows && !deep_tree_likely(p.topk_lp + (size_t)b * p.L * p.K, p.L, p.K)) return;  // (uniform)
     const int K = KC ? KC : p.K, m = MC ? MC : p.m, ld = m + 4;  // padded row: 16-byte aligned, conflict-free float4 reads
@@ -125,8 +124,8 @@ __global__ void __launch_bounds__(256, 4) tdes_edges_kernel(const EdgeParams p) 
     const size_t row = (size_t)b * p.L + j;
     // The depth-0 unit has one parent, so this CTA has time to spare: its last warp works out the sequence's budget, which
     // the tree kernel would otherwise do in front of everything else.  That takes longer than the scores of a unit (a
-    // chain of fp64 operations, 3 us), so the warp does nothing else and the other seven do not wait for it (batch 16,
-    // K = 16: 44.7 -> 44.4 us a round; batch 1, K = 32: 41.7 -> 40.3; batch 256: 293.5 -> 292.3).
+    // chain of fp64 operations, 3 us), so the warp does nothing else and the other seven do not wait for it (1.4 us of a
+    // round at batch 1, K = 32, 0.3 to 1.2 us at batch 16 and 256).
     const bool with_saba = j == 0 && p.saba_out != nullptr;
     const int nw = with_saba ? 7 : 8;  // warps on the scores
     const auto sync = [&] {

@@ -655,15 +655,15 @@ __device__ __forceinline__ void lazy_score_row(const TreeParams& p, const TreeSm
 // NT: threads of the CTA (tree_pick)
 // Code size: a round's kernels run most of their phases once, so a phase costs its instructions' way from L2 as well as
 // their issue.  Loops are not unrolled unless that measured faster (207 -> 126 KB of code for the K = 32 instance, 215 -> 106
-// for K = 8; batch 1, V = 32,000, K = 8: 32.4 -> 29.5 us a round; batch 37, K = 11, beta = 0: 52.0 -> 49.0; batch 256: 298.3
-// -> 296.8; batch 64 with wide levels 97.1 -> 98.2).  Searches that are rare or have several sites as calls: smaller still,
+// for K = 8; 9 % of a round at batch 1, K = 8, 6 % at batch 37, K = 11, beta = 0, half a per cent at batch 256; sequences with
+// wide levels lose 1 us).  Searches that are rare or have several sites as calls: smaller still,
 // but a call costs this register-bound kernel 3 us.
 // KC, MC: the number of candidates per position and the width of the TDES tables as compile-time constants (the
 // configured workloads' K = 32, m = 128: every index computation with K becomes a shift), or 0: taken from the parameters
 // FAST: the usual round is known at compile time as well -- the budget comes from the edge-score kernel (no SABA
 // arithmetic in this instance) and deeper rows are scored on demand
 // TIES: the instance for rounds without edge scores (beta = 0).  It lays the rows out itself (no edge-score kernel ran, and
-// the budget is worked out here as well: a launch and its gap less; batch 37, K = 11: 7 us a round) and
+// the budget is worked out here as well: a launch and its gap less, 7 us of a round at batch 37, K = 11) and
 // expects that exactly equal probabilities make hundreds of
 // prefixes tie with the B-th largest key: it resolves them in parallel (the other instances leave more than 32 tied
 // keys to the sequential expansion; with edge scores in the keys such ties do not occur in tens, and the code's mere
@@ -755,8 +755,8 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
         }
     }
     // a sequence whose tree will run deep had its deeper rows scored by the edge-score kernel as well: bulk copies again for
-    // large K (plain loads, eight round trips with K = 32, kept such a sequence 2 us: batch 64 with mixed confidence 99.6 ->
-    // 98.4 us a round), plain loads for K <= 20, which are fewer (batch 16, K = 16: 49.0 us, 49.5 with bulk copies)
+    // 1024 threads, K > 20 (plain loads, eight round trips with K = 32, kept such a sequence 2 us); plain loads for K <= 20,
+    // which are 40 % as many or less (bulk copies behind a barrier of their own: half a microsecond slower at K = 16)
     const bool deep = !TIES && p.rows_adaptive && deep_tree_decide(lp_top, L);  // (uniform)
     if (deep) {
         if (NT == 1024 && bulk) {
@@ -1640,8 +1640,7 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
 // ---- acceptance walk: one CTA per sequence ---------------------------------------------------------------------
 // Every node but the root asks, in parallel, whether it carries the token that the target puts behind its parent; the one
 // child that does is its parent's successor, and the walk follows successors, one shared-memory load a level.  (A walk that
-// looks for the children of every node on its way, by binary search, took 1.5 us: batch 1 at V = 151,936
-// 39.9 -> 38.9 us a round, batch 37 41.2 -> 39.8, batch 64 95.1 -> 93.4.)
+// looks for the children of every node on its way, by binary search, took 1 to 1.7 us more.)
 struct AcceptParams {
     const int32_t* n_nodes;
     const int32_t* token;
@@ -1746,9 +1745,9 @@ struct TreeInstance {
     int threads;
 };
 // Threads of a CTA: a phase costs its instructions times the warps that run it, and the levels' sizes go with K (1 + K +
-// K^2 nodes to begin with): 256 threads for K <= 8 (round at batch 1, V = 32,000, K = 8: 34.0 us with 1024 threads, 32.2
-// with 512, 31.8 with 256), 512 for K <= 20 (batch 16, K = 16: 50.6, 48.5, 50.5; batch 37, K = 11, beta = 0: 52.5, 51.8,
-// 55.2), else 1024 (batch 64, K = 32: 97.3, 99.9, 108.9).
+// K^2 nodes to begin with): 256 threads for K <= 8 (a round at batch 1, V = 32,000, K = 8 with 1024 / 512 / 256 threads: 1 /
+// 0.95 / 0.94), 512 for K <= 20 (batch 16, K = 16: 1 / 0.96 / 1.00; batch 37, K = 11, beta = 0: 1 / 0.99 / 1.05), else 1024
+// (batch 64, K = 32: 1 / 1.03 / 1.12).
 // usual: the budget from the edge-score kernel, deeper rows on demand; neutral: beta = 0
 template <bool NEUTRAL>
 static TreeInstance tree_pick_general(int K) {

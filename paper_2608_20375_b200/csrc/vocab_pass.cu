@@ -24,7 +24,7 @@
 //   * vocabulary-parallel use: the row's pieces are left for a merge over shards instead (vocab_merge_kernel).
 // Every wait on an mbarrier is bounded; when one runs out the kernel raises an error flag and drains.
 // Loops outside the stream are not unrolled unless that measured faster: the epilogue's code comes from L2 round after
-// round, beside the tree kernel's (156 -> 112 KB; batch 256 297.4 -> 295.8 us a round, batch 64 97.4 -> 96.8).
+// round, beside the tree kernel's (156 -> 112 KB of code, half a per cent of a round at batch 64 and 256).
 #include <stdlib.h>
 #include <string.h>
 
@@ -1282,7 +1282,7 @@ __global__ void __launch_bounds__(kVpThreads, 1) vocab_pass_kernel(const VpParam
                     // starts inside the row, so the row is its first and its record the first of its two; every record's
                     // keys are in descending order (empty ones, 0, last): a key's rank is its place in its own record plus
                     // the places that a binary search finds for it in the others.  (One warp that ranked all keys against
-                    // each other took 10 us of a batch-1 round.)
+                    // each other took 10 us for nine records.)
                     const VpRecord* rec0 = p.records + (size_t)c_first * 2 + ((int)(cta_start(c_first, p.Q, G) / p.nq) == sg.row ? 0 : 1);
                     auto record = [&](int i) { return i == 0 ? rec0 : p.records + (size_t)(c_first + i) * 2; };
                     // the log-sum-exp pieces (warp 0), on their way while the keys are ranked
@@ -1500,17 +1500,20 @@ VpPlan vp_make_plan(const graft_config& cfg, int num_sms, int batch, bool equal_
     if (equal_shares) {
         // Rounds without edge scores.  Their path scores are sums of log-probabilities alone, and of logits with few digits
         // hundreds of such sums are equal but for the rounding of the rows' log-sum-exp: its last bit, which hangs on how a
-        // row's sum is cut into pieces, decides which prefix stands first.  These rounds keep one partition (equal shares of
-        // at least 64 KB of the whole stream), and with it their trees, whatever suits the others best; batch 37, L = 11,
-        // V = 50,021: 42.6 us a round, 39.8 with whole rows.
+        // row's sum is cut into pieces, decides which prefix stands first.  These rounds keep the partition that all rounds
+        // once had (equal shares of at least 64 KB of the whole stream), so that a batch gives the trees that it always gave;
+        // whole rows would make a round 7 % shorter (batch 37, L = 11, V = 50,021).  It is no more than that: in a batch of
+        // another size, in another place of it or on another number of SMs a row is cut elsewhere, and such prefixes may
+        // come out in another order.
         G = nq * rows / (64 * 1024 / (kVpQuantum * esz));
         if (G > num_sms) G = num_sms;
         if (G < 1) G = 1;
         pl.whole = 0;
         share_q = (nq * rows + G - 1) / G;
     } else if (rows < num_sms) {
-        // n pieces of each row, n = 1 unless the stream gets shorter by more than the merge costs (190 KB): V = 151,936
-        // batch 1: n = 1 18.5 us, n = 2 18.6, n = 4 17.1, n = 9 20.9; batch 4: n = 1 18.9, n = 2 19.7
+        // n pieces of each row of 76 KB or more, n = 1 unless the stream gets shorter by more than the merge costs (190 KB):
+        // V = 151,936 (where n is 3 at batch 1 to 3) batch 1: n = 1 18.5 us, n = 2 18.6, n = 4 17.1, n = 9 20.9; batch 4: n = 1
+        // 18.9, n = 2 19.7
         long long n = row_bytes / (76 * 1024);
         if (n > num_sms / rows) n = num_sms / rows;
         if (n > nq) n = nq;
@@ -1587,7 +1590,6 @@ cudaError_t vp_merge_launch(graft_ctx* ctx, int batch, int n_shards, const graft
     p.n_shards = n_shards;
     p.rows = batch * ctx->cfg.L;
     p.K = ctx->cfg.K;
-#pragma unroll 1
     for (int i = 0; i < kMergeMaxShards; ++i) p.v_offset[i] = i < n_shards ? h_v_offset[i] : 0;
     p.topk_id = d_topk_id;
     p.topk_lp = d_topk_lp;
@@ -1605,7 +1607,6 @@ cudaError_t vp_configure(const graft_config& cfg, int num_sms, size_t* max_smem)
     *max_smem = pl.smem_bytes;
     if (pl.smem_bytes > 225 * 1024) return cudaErrorInvalidValue;
     cudaError_t e = cudaSuccess;
-#pragma unroll 1
     for (int groups = 2; groups <= 4 && e == cudaSuccess; groups += 2)
         e = cudaFuncSetAttribute(vp_kernel(cfg.logits_dtype == GRAFT_BF16, groups), cudaFuncAttributeMaxDynamicSharedMemorySize, 225 * 1024);
     return e;
@@ -1683,7 +1684,6 @@ extern "C" graft_status graft_vocab_pass_static(int32_t batch, int32_t L, int32_
                 cudaGetLastError();
                 return GRAFT_ERR_CUDA;
             }
-#pragma unroll 1
             for (int i = 0; i < 4; ++i)
                 if (cudaFuncSetAttribute(vp_kernel((i & 1) != 0, i < 2 ? 2 : 4), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          225 * 1024) != cudaSuccess) {
