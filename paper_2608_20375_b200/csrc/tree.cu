@@ -511,19 +511,39 @@ __device__ uint32_t cta_finish_select(const TreeSmem& sm, const uint32_t* keys, 
         return cta_kth_largest<NT>(sm, keys, lo_i, hi_i, kth, 0, 4, 0u, rem, tid);
     }
     const int remaining = st.rem;
-#pragma unroll 1
-    for (int i = tid >> 5; i < n; i += NT / 32) {  // a warp per key, a lane per key it is compared with
-        const uint32_t k = list[i];
-        int gt = 0, ge = 0;
-#pragma unroll 1
-        for (int j = tid & 31; j - (tid & 31) < n; j += 32) {
-            const uint32_t o = j < n ? list[j] : 0u;  // (0 is below every key)
-            gt += __popc(__ballot_sync(0xFFFFFFFFu, o > k));
-            ge += __popc(__ballot_sync(0xFFFFFFFFu, o >= k));
-        }
+    const auto note = [&](uint32_t k, int gt, int ge) {
         if (gt < remaining && remaining <= ge) {  // (every writer writes the same values)
             sm.scal[6] = (int)k;
             sm.scal[7] = kth - remaining + ge;  // the keys above the bucket, and those of the bucket that reach k
+        }
+    };
+    // A few keys: a warp per key, a lane per key it is compared with.  Hundreds of them (tables of near-equal scores): a
+    // thread per key; by warps they took 10k cycles more.
+    if (n <= NT / 8) {  // (uniform)
+#pragma unroll 1
+        for (int i = tid >> 5; i < n; i += NT / 32) {
+            const uint32_t k = list[i];
+            int gt = 0, ge = 0;
+#pragma unroll 1
+            for (int j = tid & 31; j - (tid & 31) < n; j += 32) {
+                const uint32_t o = j < n ? list[j] : 0u;  // (0 is below every key)
+                gt += __popc(__ballot_sync(0xFFFFFFFFu, o > k));
+                ge += __popc(__ballot_sync(0xFFFFFFFFu, o >= k));
+            }
+            note(k, gt, ge);
+        }
+    } else {
+#pragma unroll 1
+        for (int i = tid; i < n; i += NT) {
+            const uint32_t k = list[i];
+            int gt = 0, ge = 0;
+#pragma unroll 4
+            for (int j = 0; j < n; ++j) {
+                const uint32_t o = list[j];
+                gt += o > k ? 1 : 0;
+                ge += o >= k ? 1 : 0;
+            }
+            note(k, gt, ge);
         }
     }
     __syncthreads();
@@ -1184,8 +1204,10 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
             if (!grown) break;  // no node of the new level can have a child in the tree
             n_grow = b1 - b0 <= NT && lv1 - lv0 <= NT ? grown : NT + 1;  // (a thread appended one node of the level at most)
             // theta only has to be a lower bound of its final value while the levels are built (it prunes), so
-            // the exact B-th largest key is recomputed only when the table has grown noticeably
-            if (ntot - 1 >= budget && (theta == 0u || ntot - n_at_select >= ntot / 4)) {
+            // the exact B-th largest key is recomputed only when the table has grown noticeably -- and in front of the first
+            // row that is not scored ahead: scoring it costs four searches, and a tighter threshold often ends the tree
+            // there (a batch of 64 with mixed confidence: 6 % of the round)
+            if (ntot - 1 >= budget && (theta == 0u || ntot - n_at_select >= ntot / 4 || (!TIES && d + 1 == rows_pre))) {
                 sel_top = 0.0f + sm.es[0];  // the root's best child
                 // a lower bound; never below the one in use, which a search over a level's children may have put higher (the
                 // count of the nodes that can have children holds for a threshold that rises only)

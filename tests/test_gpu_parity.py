@@ -620,6 +620,27 @@ def test_round_at_the_edges_of_the_tree_kernel_instances(L, K, m, beta, fixed):
     g.destroy()
 
 
+@pytest.mark.parametrize("K", [5, 6, 8, 11, 16, 20, 22, 32])
+@pytest.mark.parametrize("beta", [0.0, 1e-3])
+def test_round_with_many_keys_in_the_last_bucket(K, beta):
+    """K^2 prefixes whose scores lie within 1/32 of one another and a budget in their midst: 25 to 1024 keys in the bucket in
+    which the B-th largest is looked for, on either side of what a warp per key ranks (32, 64 and 128 keys for 256, 512 and
+    1024 threads) and of what its list holds (512)."""
+    w = gi.small(batch=4, L=5, V=2003, K=K, budget_min=1, budget_max=min(1023, K + K * K), budget_step=1, logits_dtype="f32",
+                 m=64, hidden_dim=8, beta=beta, fixed_budget=K + K * K // 2)
+    g = _graft(w)
+    tb, saba_kw, keep = _setup(w, g)
+    x = gi.batch_inputs(w)
+    gen = torch.Generator().manual_seed(K)
+    z = torch.full((4, 5, w.V), -30.0)
+    z[:, :, 100:100 + K] = 10.0 + 0.012 * torch.rand((4, 5, K), generator=gen)
+    x["logits"] = z
+    _, gpu = gpu_round(g, w, x)
+    compare_round(oracle, w, x, tb, saba_kw, gpu, oracle_round(oracle, w, x, tb, saba_kw))
+    assert (gpu["n_nodes"] == 1 + K + K * K // 2).all()
+    g.destroy()
+
+
 @pytest.mark.parametrize("kw", _SPLIT_CASES[:3] + [
     dict(batch=3, L=16, V=6000, K=32, budget_min=32, budget_max=512, budget_step=16, m=512, hidden_dim=64)])
 @pytest.mark.parametrize("rows", [0, None])
