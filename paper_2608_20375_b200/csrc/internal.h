@@ -135,6 +135,7 @@ inline cudaError_t allow_smem(const void* kernel, size_t need) {
     if (e != cudaSuccess) return e;
     most -= (int)a.sharedSizeBytes;
     if (most < 0 || need > (size_t)most) return cudaErrorInvalidValue;
+    if ((size_t)a.maxDynamicSharedSizeBytes >= need) return cudaSuccess;
     return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
 }
 
