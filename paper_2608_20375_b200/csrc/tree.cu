@@ -1204,10 +1204,11 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
             if (!grown) break;  // no node of the new level can have a child in the tree
             n_grow = b1 - b0 <= NT && lv1 - lv0 <= NT ? grown : NT + 1;  // (a thread appended one node of the level at most)
             // theta only has to be a lower bound of its final value while the levels are built (it prunes), so
-            // the exact B-th largest key is recomputed only when the table has grown noticeably -- and in front of the first
-            // row that is not scored ahead: scoring it costs four searches, and a tighter threshold often ends the tree
-            // there (a batch of 64 with mixed confidence: 6 % of the round)
-            if (ntot - 1 >= budget && (theta == 0u || ntot - n_at_select >= ntot / 4 || (!TIES && d + 1 == rows_pre))) {
+            // the exact B-th largest key is recomputed only when the table has grown noticeably, by a quarter -- by a sixteenth
+            // in front of the first row that is not scored ahead: scoring it costs four searches, and a tighter threshold
+            // often ends the tree there (a batch of 64 with mixed confidence: 6 % of the round)
+            if (ntot - 1 >= budget &&
+                (theta == 0u || ntot - n_at_select >= (!TIES && d + 1 == rows_pre ? ntot / 16 : ntot / 4))) {
                 sel_top = 0.0f + sm.es[0];  // the root's best child
                 // a lower bound; never below the one in use, which a search over a level's children may have put higher (the
                 // count of the nodes that can have children holds for a threshold that rises only)
