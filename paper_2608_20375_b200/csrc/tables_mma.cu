@@ -269,7 +269,7 @@ __global__ void __cluster_dims__(F32 ? 1 : 2, 1, 1) __launch_bounds__(TablesCfg<
         const int half = warp >> 2, quarter = warp & 3;
         const uint32_t accempty_even = mapa_u32(accempty0, 0);
         uint32_t cc = 0;  // chunks emptied so far
-        float check = 0.f;  // fp32 embeddings: NaN once a result of this thread was not finite
+        float2 check = make_float2(0.f, 0.f);  // fp32 embeddings: NaN once a result of this thread was not finite
         for (int i = 0; tables_item(p, pair, i, it); ++i) {
             const int rt = it.tile / p.n_mb, mb = it.tile - rt * p.n_mb;
             const uint32_t n = (uint32_t)tables_n<F32>(p, mb);
@@ -329,8 +329,9 @@ __global__ void __cluster_dims__(F32 ? 1 : 2, 1, 1) __launch_bounds__(TablesCfg<
                         }
                         if (F32 && !piece) {
 #pragma unroll
-                            for (int k = 0; k < 8; ++k)
-                                if (k < 4 || both) check = fmaf(0.f, acc[h][c + k], check);
+                            for (int k = 0; k < 8; k += 2)
+                                if (k < 4 || both)
+                                    check = __ffma2_rn(make_float2(0.f, 0.f), make_float2(acc[h][c + k], acc[h][c + k + 1]), check);
                         }
                         if (wide) {  // (both: m is a multiple of 8)
                             st_global_v8(dst + c, &acc[h][c]);
@@ -344,7 +345,7 @@ __global__ void __cluster_dims__(F32 ? 1 : 2, 1, 1) __launch_bounds__(TablesCfg<
             }
         }
         if (F32) {  // (nothing waits for these warps any more)
-            if (check != 0.f) s_mend = true;
+            if (check.x + check.y != 0.f) s_mend = true;
             __syncwarp();
             named_bar_sync(1, kTmEpiWarps * 32);  // (the tiles are written for every thread of these warps)
             if (s_mend && !s_abort) {
@@ -566,7 +567,7 @@ __global__ void __launch_bounds__(256) tables_pieces_kernel(const __grid_constan
         s.x += b[0], s.y += b[1], s.z += b[2], s.w += b[3];
     }
     const int row = rt * C::ROWS + v, col = mb * 128 + c;
-    if (F32) {
+    if (F32 && fmaf(0.f, s.x, fmaf(0.f, s.y, fmaf(0.f, s.z, 0.f * s.w))) != 0.f) {
         if (!tables_finite(s.x)) s.x = tables_fp32(p, row, col);
         if (!tables_finite(s.y)) s.y = tables_fp32(p, row, col + 1);
         if (!tables_finite(s.z)) s.z = tables_fp32(p, row, col + 2);
