@@ -612,7 +612,7 @@ def run_saba_fit(args):
     from paper_2608_20375_b200 import Graft
     import oracle  # CPU-baseline leg only
 
-    n = 16_000_000  # 36 bytes a round: 576 MB, well over L2
+    n = 16_000_000  # 28 bytes a round: 448 MB, well over L2
     dev = torch.device("cuda", 0)
     torch.cuda.set_device(dev)
     g = Graft(1000, 4, 4, 16, 8, 1, 8, 8, 8, 0.0, 1, 0, 0)
@@ -639,7 +639,7 @@ def run_saba_fit(args):
     ref = oracle.saba_fit(**{k: v[:n_s] for k, v in lg.items()})
     t_cpu = time.perf_counter() - t0
     hbm_peak, peak_kind = _peaks()
-    alg = n * 36
+    alg = n * 28
     print(json.dumps({
         "kind": "least-squares fit of the SABA gain and cost models (graft_saba_fit)", "rounds_logged": n,
         "ms_per_fit": round(ms, 4), "algorithmic_bytes": alg, "achieved_gbs": round(alg / (ms * 1e-3) / 1e9, 1),

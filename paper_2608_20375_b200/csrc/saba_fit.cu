@@ -9,8 +9,8 @@
 // memory, per grid by one atomic a sum); the CTA that finishes last solves the two small systems (columns scaled to unit
 // diagonal first, then Gauss-Jordan elimination with partial pivoting) and clears the accumulators for the next call.
 //
-// 36 bytes are read a tuple and some 75 fp64 operations done on it, a third of them in the logarithm: the fp64 pipe and
-// the conversions in front of it bound the slope (6.7 us per million tuples, 5.4 TB/s; copies into shared memory ahead
+// 28 bytes are read a tuple and some 75 fp64 operations done on it, a third of them in the logarithm: the fp64 pipe and
+// the conversions in front of it bound the slope (6.7 us per million tuples, 4.2 TB/s; copies into shared memory ahead
 // of the arithmetic, two and four tuples interleaved, and 24 warps an SM instead of 16 were no faster or slower), and a
 // call costs 8 us however few the tuples.  4 million tuples on a B200: 56.9 -> 37.0 us with log for log1p, counts as
 // integers, products by one folded (-> 45.3), the elimination on a warp and sums without shared-memory atomics (n = 64:
