@@ -18,7 +18,7 @@ ALL_HEADERS = ["common.cuh", "internal.h", "edge_score.cuh", "cosine.cuh", "saba
 # source -> headers it depends on
 SOURCES = {
     "api.cu": ALL_HEADERS,
-    "vocab_pass.cu": ALL_HEADERS,
+    "vocab_pass.cu": ALL_HEADERS + ["umma.cuh", "vocab_common.cuh", "vocab_rows.cuh"],
     "tdes.cu": ALL_HEADERS,
     "tree.cu": ALL_HEADERS,
     "tdes_train.cu": ["common.cuh", "internal.h", GRAFT_H],

@@ -14,7 +14,7 @@ constexpr int kMaxCostPts = 16;
 // ---- vocab pass -----------------------------------------------------------------------------
 constexpr int kVpConsumerWarps = 16;                 // streaming warps (one CTA per SM)
 constexpr int kVpConsumers = kVpConsumerWarps * 32;  // 512
-constexpr int kVpEpiWarps = 8;                       // epilogue warps: two groups of four or four groups of two
+constexpr int kVpEpiWarps = 8;                       // epilogue warps: two groups of four
 constexpr int kVpGroups = 64;   // groups of streaming threads whose maxima bound the K-th largest element (>= kMaxK)
 constexpr int kVpThreads = kVpConsumers + kVpEpiWarps * 32 + 64;  // + one producer warp + one cosine warp
 constexpr int kVpTileBytes = 32768;                  // one ring stage (2 KiB per streaming warp)
@@ -33,9 +33,10 @@ struct VpRecord {
 };
 
 struct VpPlan {
+    int cluster;         // CTAs that hold a row together in shared memory (vocab_rows.cuh); 0: the streaming kernel, as below
+    int threads;         // threads of such a CTA that work on the row
     int grid;            // CTAs launched
     int whole;           // every CTA gets whole rows
-    int groups;          // epilogue groups (2 or 4)
     int stages;          // ring depth
     int max_seg_tiles;   // tiles in the longest segment a CTA can get
     size_t smem_bytes;

@@ -2,13 +2,16 @@
 // yields log-sum-exp over the vocabulary and the K top-ranked tokens with their log-probabilities
 // (Preliminaries, "DFlash one-pass marginals": q_{t,d} and c^{(r)}_{t,d}; Eq. 3's log q).
 //
-// Shape of the kernel (sm_100a):
+// Rows that fit into shared memory, and few rows of any length, are held there (vocab_rows.cuh; rows_plan below has the rule);
+// the rest go through the streaming kernel of this file.
+//
+// Shape of the streaming kernel (sm_100a):
 //   * persistent grid, one CTA per SM at most; a CTA gets whole rows where that comes out even enough, else the
 //     rows*V element stream is cut into equal contiguous shares, so a CTA sees at most two partial rows plus whole
 //     rows in between ("segments"; vp_make_plan has the rule);
 //   * warp roles: one producer warp feeds a four-stage shared-memory ring with 32 KiB TMA bulk copies
 //     (cp.async.bulk + mbarrier complete_tx); sixteen streaming warps read the ring with 16-byte shared loads;
-//     two epilogue groups of four warps (four of two for many short rows) finish segments in turn while the
+//     two epilogue groups of four warps finish segments in turn while the
 //     streaming warps are already in later ones; one warp computes the adjacent-position cosines of the SABA state (Eq. 15) beside the stream;
 //   * per 32-element chunk a streaming lane takes a packed max (stored for the second stage, 2 bytes per
 //     chunk), keeps a lazily rescaled reference exponent and adds 2^(z log2e - ref) with ex2.approx;
@@ -33,10 +36,8 @@
 #include "common.cuh"
 #include "internal.h"
 #include "cosine.cuh"
-
-#ifndef GRAFT_VP_F32X2
-#define GRAFT_VP_F32X2 1  // packed fp32 pair arithmetic (fma.rn.f32x2 / add.rn.f32x2)
-#endif
+#include "vocab_common.cuh"
+#include "vocab_rows.cuh"
 
 namespace graft {
 
@@ -49,8 +50,7 @@ constexpr int PROD_WARP = NW + kVpEpiWarps;  // warp index of the producer warp
 constexpr int TILE = kVpTileBytes;
 constexpr int WBLK = TILE / NW;               // bytes of a tile owned by one warp (2048)
 static_assert(WBLK == 2048, "one warp owns 2 KiB of every tile");
-constexpr int VEC_PER_LANE = WBLK / 16 / 32;  // 4
-static_assert(VEC_PER_LANE == 4, "chunk layout assumes four 16-byte vectors per lane per tile");
+static_assert(VEC_PER_LANE == WBLK / 16 / 32, "four 16-byte vectors per lane per tile");
 static_assert(WBLK == 32 * 4 * 16, "the exact fall-back selection reads one warp block per batch");
 constexpr uint32_t kOrdNegInf = 0x007FFFFFu;  // ord_from_bits of -inf: every finite value maps above it
 constexpr uint32_t kVpIdleHintNs = 10000;  // suspend hint of the waits of the producer and epilogue warps
@@ -58,30 +58,11 @@ constexpr int COS_WARP = PROD_WARP + 1;  // warp that computes the SABA cosines 
 static_assert(kVpThreads == NT + kVpEpiWarps * 32 + 64,
               "thread count = streaming warps + epilogue warps + producer warp + cosine warp");
 
-// The eight epilogue warps work as GROUPS groups, each on a segment of its own (segments in turn).  An epilogue is a chain
-// of latencies (8k cycles alone, 10k beside the stream; 20 % more with two warps instead of four), so a CTA whose
-// segments stream faster than two groups finish them is served better by four.
-template <int GROUPS>
-struct Epi {
-    static constexpr int THREADS = kVpEpiWarps * 32 / GROUPS;
-    static constexpr int BUFS = 2 * GROUPS;  // hand-over buffers between streaming and epilogue warps
-};
-constexpr int kVpMaxBufs = 8;
-
-template <bool BF16>
-struct VT;
-template <>
-struct VT<true> {
-    using cm_t = uint16_t;
-    static constexpr int ESZ = 2, EPV = 8;
-    static constexpr uint32_t NEG_INF_WORD = 0xFF80FF80u;
-};
-template <>
-struct VT<false> {
-    using cm_t = uint16_t;  // the chunk maximum rounded UP to bf16 precision: an upper bound is all the scan needs
-    static constexpr int ESZ = 4, EPV = 4;
-    static constexpr uint32_t NEG_INF_WORD = 0xFF800000u;
-};
+// The eight epilogue warps work as two groups, each on a segment of its own (segments in turn).  An epilogue is a chain
+// of latencies (8k cycles alone, 10k beside the stream; 20 % more with two warps instead of four).
+constexpr int GROUPS = 2;
+constexpr int ET = kVpEpiWarps * 32 / GROUPS;  // threads of a group
+constexpr int BUFS = 2 * GROUPS;               // hand-over buffers between streaming and epilogue warps
 
 struct VpParams {
     const char* logits;
@@ -185,95 +166,6 @@ __device__ __forceinline__ bool seg_iter_next(const VpParams& p, SegIter& it, Se
 // After seg_iter_next returned a segment: is it the one this CTA visits last?
 __device__ __forceinline__ bool seg_iter_at_end(const SegIter& it) { return it.row >= it.r_last; }
 
-__device__ __forceinline__ float load_elem_f32(const char* p, bool bf16) {
-    if (bf16) return __uint_as_float(((uint32_t) * (const uint16_t*)p) << 16);
-    return *(const float*)p;
-}
-
-// ---- per-thread streaming state -----------------------------------------------------------------
-#if GRAFT_VP_F32X2
-__device__ __forceinline__ uint64_t pack2(float lo, float hi) {
-    uint64_t r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-    return r;
-}
-__device__ __forceinline__ void unpack2(uint64_t v, float& lo, float& hi) {
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
-}
-__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
-    uint64_t r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
-__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
-    uint64_t r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
-    uint64_t r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-#endif
-
-// The running log-sum-exp of one streaming thread over a segment: sum of 2^(z log2e - ref) in four fp32
-// accumulators (two packed pairs), a reference exponent that is raised lazily (only when a chunk's maximum exceeds
-// it by more than 2^16, so that rescaling is rare and every term stays far from overflow), and the largest value.
-struct Acc {
-    float ref;      // reference exponent, log2 domain; -inf before the first finite value
-    float nref;     // -ref (0 while ref is -inf): the addend of the fused multiply-add
-    uint32_t thr;   // a chunk maximum above this value raises the reference: bf16 logits: the value in both halves
-                    // of a packed pair; fp32 logits: float bits
-    uint32_t rmax;  // largest value so far: bf16 logits: a packed pair of running maxima; fp32 logits: float bits
-#if GRAFT_VP_F32X2
-    uint64_t a0, a1;
-#else
-    float s0, s1, s2, s3;
-#endif
-};
-
-template <bool BF16>
-__device__ __forceinline__ void acc_init(Acc& a) {
-    a.ref = -INFINITY;
-    a.nref = 0.f;
-    a.thr = BF16 ? 0xFF80FF80u : 0xFF800000u;  // -inf: the first finite value sets the reference
-    a.rmax = a.thr;
-#if GRAFT_VP_F32X2
-    a.a0 = a.a1 = 0ull;
-#else
-    a.s0 = a.s1 = a.s2 = a.s3 = 0.f;
-#endif
-}
-
-// The chunk maximum cm exceeded the threshold: raise the reference to cm (rare).
-template <bool BF16>
-__device__ __forceinline__ void acc_raise(Acc& a, float cm) {
-    const float cms = cm * kLog2e;
-    if (!(cms > a.ref + 16.0f)) return;  // (the threshold is a truncated copy of ref + 16: it may fire a little early)
-    const float f = ex2_approx(a.ref - cms);  // 0 when ref is -inf (nothing added yet) or cm is +inf
-#if GRAFT_VP_F32X2
-    const uint64_t f2 = pack2(f, f);
-    a.a0 = mul2(a.a0, f2);
-    a.a1 = mul2(a.a1, f2);
-#else
-    a.s0 *= f;
-    a.s1 *= f;
-    a.s2 *= f;
-    a.s3 *= f;
-#endif
-    a.ref = cms;
-    a.nref = -cms;
-    // values above (ref + 16) / log2e raise the reference again; the bound need not be exact (terms overflow only
-    // 2^111 above it), so it is kept as its leading 16 bits for the packed comparison of bf16 chunks
-    const uint32_t zb = __float_as_uint((cms + 16.0f) * 0.6931471805599453f);
-    a.thr = BF16 ? ((zb >> 16) | (zb & 0xFFFF0000u)) : zb;
-}
-
-__device__ __forceinline__ float pair_max_bf16(uint32_t pm) {  // the larger half of a packed bf16 pair, as fp32
-    return fmaxf(__uint_as_float(pm << 16), __uint_as_float(pm & 0xFFFF0000u));
-}
-
 // One chunk of a streaming lane: four 16-byte vectors of a tile (32 bf16 or 16 fp32 logits).  The chunk maximum goes
 // to *cmax_slot for the second stage (2 bytes: the bf16 value, or the fp32 maximum rounded up to bf16).
 template <bool BF16, bool GUARD>
@@ -325,68 +217,7 @@ __device__ __forceinline__ void process_chunk(const uint4* __restrict__ wb, int 
         }
         if (m > __uint_as_float(a.thr)) acc_raise<BF16>(a, m);
     }
-#if GRAFT_VP_F32X2
-    const uint64_t c2 = pack2(kLog2e, kLog2e), r2 = pack2(a.nref, a.nref);
-#pragma unroll
-    for (int i = 0; i < VEC_PER_LANE; ++i) {
-        const uint32_t w[4] = {v[i].x, v[i].y, v[i].z, v[i].w};
-        if (BF16) {
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const uint64_t x2 = pack2(__uint_as_float(w[k] << 16), __uint_as_float(w[k] & 0xFFFF0000u));
-                float t0, t1;
-                unpack2(fma2(x2, c2, r2), t0, t1);
-                const uint64_t e2 = pack2(ex2_approx(t0), ex2_approx(t1));
-                if (k & 1)
-                    a.a1 = add2(a.a1, e2);
-                else
-                    a.a0 = add2(a.a0, e2);
-            }
-        } else {
-            float t0, t1, t2, t3;
-            unpack2(fma2(pack2(__uint_as_float(w[0]), __uint_as_float(w[1])), c2, r2), t0, t1);
-            unpack2(fma2(pack2(__uint_as_float(w[2]), __uint_as_float(w[3])), c2, r2), t2, t3);
-            a.a0 = add2(a.a0, pack2(ex2_approx(t0), ex2_approx(t1)));
-            a.a1 = add2(a.a1, pack2(ex2_approx(t2), ex2_approx(t3)));
-        }
-    }
-#else
-#pragma unroll
-    for (int i = 0; i < VEC_PER_LANE; ++i) {
-        const uint32_t w[4] = {v[i].x, v[i].y, v[i].z, v[i].w};
-        if (BF16) {
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const float lo = __uint_as_float(w[k] << 16), hi = __uint_as_float(w[k] & 0xFFFF0000u);
-                const float e0 = ex2_approx(fmaf(lo, kLog2e, a.nref)), e1 = ex2_approx(fmaf(hi, kLog2e, a.nref));
-                if (k & 1) {
-                    a.s2 += e0;
-                    a.s3 += e1;
-                } else {
-                    a.s0 += e0;
-                    a.s1 += e1;
-                }
-            }
-        } else {
-            a.s0 += ex2_approx(fmaf(__uint_as_float(w[0]), kLog2e, a.nref));
-            a.s1 += ex2_approx(fmaf(__uint_as_float(w[1]), kLog2e, a.nref));
-            a.s2 += ex2_approx(fmaf(__uint_as_float(w[2]), kLog2e, a.nref));
-            a.s3 += ex2_approx(fmaf(__uint_as_float(w[3]), kLog2e, a.nref));
-        }
-    }
-#endif
-}
-
-template <bool BF16>
-__device__ __forceinline__ float acc_sum(const Acc& a) {
-#if GRAFT_VP_F32X2
-    float s0, s1, s2, s3;
-    unpack2(a.a0, s0, s1);
-    unpack2(a.a1, s2, s3);
-    return (s0 + s1) + (s2 + s3);
-#else
-    return (a.s0 + a.s1) + (a.s2 + a.s3);
-#endif
+    acc_add<BF16>(v, a);
 }
 
 // (c, s) pairs stand for s * 2^c; merge two of them
@@ -413,16 +244,14 @@ struct __align__(16) EpiShared {  // private to one epilogue group
                     // plus the first elements equal to T
     uint32_t Tv;
 };
-template <int GROUPS>
 struct __align__(16) VpShared {
     EpiShared epi[GROUPS];
-    uint32_t tmax[Epi<GROUPS>::BUFS][NT];  // per-thread maxima of a finished segment, one buffer per segment in flight
-    uint32_t gmax[Epi<GROUPS>::BUFS][kVpGroups];  // the same maxima folded into 64 groups (lane, warp parity); zero when idle
-    float wc[Epi<GROUPS>::BUFS][NW], ws[Epi<GROUPS>::BUFS][NW];
+    uint32_t tmax[BUFS][NT];  // per-thread maxima of a finished segment, one buffer per segment in flight
+    uint32_t gmax[BUFS][kVpGroups];  // the same maxima folded into 64 groups (lane, warp parity); zero when idle
+    float wc[BUFS][NW], ws[BUFS][NW];
     volatile int abort_flag;
 };
 
-template <int ET>  // threads of a group
 __device__ __forceinline__ void epi_bar(int group) { named_bar_sync(2 + group, ET); }
 
 // ---- epilogue-warp helpers (32 threads, warp-synchronous) ----------------------------------------------
@@ -472,7 +301,6 @@ __device__ __noinline__ void warp_select_topk(EpiShared* sh, int n, int K, int l
 // The K-th largest chunk maximum of a segment (every streaming thread leaves one 16-bit maximum per tile), as a 16-bit
 // order-preserving pattern; 0 when the segment has fewer than K chunks.  All threads of an epilogue group; two
 // histogram passes of eight bits each over the idle hit list.  Out of line: rows that need it are rare.
-template <int ET>
 __device__ __noinline__ uint32_t epi_kth_chunk_max(EpiShared* es, const uint16_t* cmx, int max_tiles, int ntiles, int K,
                                                    int etid, int grp) {
     uint32_t* hist = es->hits;  // [0, 256) counts, [256] the bin found, [257] the count above it
@@ -482,7 +310,7 @@ __device__ __noinline__ uint32_t epi_kth_chunk_max(EpiShared* es, const uint16_t
     for (int pass = 0; pass < 2; ++pass) {
 #pragma unroll 1
         for (int i = etid; i < 258; i += ET) hist[i] = 0u;
-        epi_bar<ET>(grp);
+        epi_bar(grp);
 #pragma unroll 1
         for (int t = etid; t < NT; t += ET) {
             const uint16_t* row = cmx + (size_t)t * max_tiles;
@@ -495,7 +323,7 @@ __device__ __noinline__ uint32_t epi_kth_chunk_max(EpiShared* es, const uint16_t
                     atomicAdd(&hist[v & 255u], 1u);
             }
         }
-        epi_bar<ET>(grp);
+        epi_bar(grp);
         if (etid < 32) {  // the bin in which the count from the top reaches `want`: eight bins a lane
             uint32_t own = 0u;
 #pragma unroll
@@ -520,7 +348,7 @@ __device__ __noinline__ uint32_t epi_kth_chunk_max(EpiShared* es, const uint16_t
                 }
             }
         }
-        epi_bar<ET>(grp);
+        epi_bar(grp);
         const uint32_t bin = hist[256];
         if (bin == 0u) {  // fewer than K chunks (uniform)
             prefix = 0u;
@@ -529,7 +357,7 @@ __device__ __noinline__ uint32_t epi_kth_chunk_max(EpiShared* es, const uint16_t
             prefix = (prefix << 8) | (bin & 255u);
             want -= (int)hist[257];
         }
-        epi_bar<ET>(grp);  // (read before the next pass clears it)
+        epi_bar(grp);  // (read before the next pass clears it)
     }
     return prefix;
 }
@@ -540,14 +368,13 @@ __device__ __noinline__ uint32_t epi_kth_chunk_max(EpiShared* es, const uint16_t
 // wanted -- and the K keys that reach it (keys are distinct: exactly K) are ranked into outk.  Whatever the keys'
 // order or values.  All threads of an epilogue group; the counts of its warps meet in the idle hit list.  Out of
 // line: rows that need it are rare.
-template <int ET>
 __device__ __noinline__ void epi_select_many(EpiShared* es, int n, int K, int etid, int grp) {
     uint32_t* cnt = es->hits;                       // [2 * 16 * 3] counts of the steps, [96], [97] above / at the value, [98] kept
     uint64_t* kept = (uint64_t*)(es->hits + 128);   // [K] the keys that reach the K-th largest
     const uint32_t* word = (const uint32_t*)es->cand;  // key i: id word at 2 i, value word at 2 i + 1
 #pragma unroll 1
     for (int i = etid; i < 99; i += ET) cnt[i] = 0u;
-    epi_bar<ET>(grp);
+    epi_bar(grp);
     uint32_t vk = 0u, ik = 0u;  // the K-th largest key's value word and id word
     int want = K;
 #pragma unroll 1
@@ -575,7 +402,7 @@ __device__ __noinline__ void epi_select_many(EpiShared* es, int n, int K, int et
                 atomicAdd(&slot[1], (uint32_t)c2);
                 atomicAdd(&slot[2], (uint32_t)c3);
             }
-            epi_bar<ET>(grp);
+            epi_bar(grp);
             const int n1 = (int)slot[0], n2 = (int)slot[1], n3 = (int)slot[2];
             kth = n3 >= want ? t3 : (n2 >= want ? t2 : (n1 >= want ? t1 : kth));
         }
@@ -597,7 +424,7 @@ __device__ __noinline__ void epi_select_many(EpiShared* es, int n, int K, int et
             atomicAdd(&cnt[96], (uint32_t)above);
             atomicAdd(&cnt[97], (uint32_t)at);
         }
-        epi_bar<ET>(grp);
+        epi_bar(grp);
         want = K - (int)cnt[96];
         if ((int)cnt[97] == want) break;  // (uniform) every key of that value is wanted: ik = 0 lets them all through
     }
@@ -610,7 +437,7 @@ __device__ __noinline__ void epi_select_many(EpiShared* es, int n, int K, int et
             if (pos < (uint32_t)kMaxK) kept[pos] = k;
         }
     }
-    epi_bar<ET>(grp);
+    epi_bar(grp);
     const int m = (int)cnt[98] < K ? (int)cnt[98] : K;
     if (etid < m) {
         const uint64_t k = kept[etid];
@@ -708,53 +535,22 @@ __device__ int warp_fallback_select(EpiShared* sh, const VpParams& p, const Seg&
     return n < K ? n : K;
 }
 
-// The outputs of a finished row from its pieces: C, S with sum_v 2^(z_v c) = S 2^C (c = fp32(log2 e)), the largest
-// logit, and the K best keys.  One warp.  `internal`: a bounded wait ran out in a CTA that worked on this row.
-__device__ __forceinline__ void vp_finalize(double Cd, double Sd, uint32_t Vm, int nk, int K, const uint64_t* keys,
-                                            int lane, int32_t* topk_id, float* topk_lp, float* lse,
-                                            int32_t* row_status, bool internal) {
-    // The stream accumulates 2^(z c - ref) with c = fp32(log2 e), so (C + log2 S) ln 2 is the
-    // log-sum-exp of the logits scaled by a = c ln 2 = 1 + 1.3e-8.  To first order that adds
-    // (a - 1) E_q[z]; the largest logit stands in for the mean under q (the difference is a few
-    // units times 1e-8).
-    // every lane must use the same bits: the folds that produced C and S are butterflies of fused multiply-adds,
-    // which leave the lanes an ulp apart, and log-probabilities of equal logits (and their order) must not depend on
-    // the lane that writes them
-    Cd = __shfl_sync(0xFFFFFFFFu, Cd, 0);
-    Sd = __shfl_sync(0xFFFFFFFFu, Sd, 0);
-    Vm = __shfl_sync(0xFFFFFFFFu, Vm, 0);
-    const float vmax = __uint_as_float(bits_from_ord(Vm));
-    const double a_minus_1 = (double)kLog2e * kLn2 - 1.0;
-    const double lse_d = (Cd + log2(Sd)) * kLn2 - a_minus_1 * (double)vmax;
-    const bool bad = !(Sd > 0.0) || !(Sd < 1e300) || Vm == 0u || vmax == INFINITY || vmax == -INFINITY || nk < K;
-    if (lane < K) {
-        const uint64_t key = lane < nk ? keys[lane] : 0ull;
-        topk_id[lane] = lane < nk ? (int32_t)key_id(key) : -1;
-        topk_lp[lane] = lane < nk ? (float)((double)key_value(key) - lse_d) : 0.f;
-    }
-    if (lane == 0) {
-        *lse = (float)lse_d;
-        *row_status = (bad ? GRAFT_ST_BAD_LOGITS : 0) | (internal ? GRAFT_ST_INTERNAL : 0);
-    }
-}
-
-template <bool BF16, int GROUPS>
+template <bool BF16>
 __global__ void __launch_bounds__(kVpThreads, 1) vocab_pass_kernel(const VpParams p) {
     using T = VT<BF16>;
     using cm_t = typename T::cm_t;
-    constexpr int ET = Epi<GROUPS>::THREADS, BUFS = Epi<GROUPS>::BUFS;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     pdl_launch_dependents();  // the edge-score kernel's CTAs may move in as this grid's CTAs leave; they wait for it
     unsigned char* ring = smem_raw;
-    uint64_t* bars = (uint64_t*)(ring + (size_t)p.stages * TILE);  // full[8], empty[8], ready[8], done[8]
-    VpShared<GROUPS>* sh = (VpShared<GROUPS>*)(bars + 16 + 2 * kVpMaxBufs);
+    uint64_t* bars = (uint64_t*)(ring + (size_t)p.stages * TILE);  // full[8], empty[8], ready[BUFS], done[BUFS]
+    VpShared* sh = (VpShared*)(bars + 16 + 2 * BUFS);
     cm_t* cmax = (cm_t*)(sh + 1);  // [BUFS][n_cmax]
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const long long G = gridDim.x;
     const long long q0 = cta_start(blockIdx.x, p.Q, G), q1 = cta_start(blockIdx.x + 1, p.Q, G);
     const uint32_t full0 = smem_u32(bars), empty0 = smem_u32(bars + 8);
-    const uint32_t ready0 = smem_u32(bars + 16), done0 = smem_u32(bars + 16 + kVpMaxBufs);
+    const uint32_t ready0 = smem_u32(bars + 16), done0 = smem_u32(bars + 16 + BUFS);
 
     if (tid == 0) {
 #pragma unroll 1
@@ -1021,7 +817,7 @@ __global__ void __launch_bounds__(kVpThreads, 1) vocab_pass_kernel(const VpParam
                     es->tie_groups = tie_groups;
                 }
             }
-            epi_bar<ET>(grp);
+            epi_bar(grp);
             uint32_t Tv = es->Tv;
             // (d) chunks whose stored maximum reaches T: only threads whose own maximum reaches T can have one.
             //     List positions come from shared-memory atomics (the order does not matter: the final selection
@@ -1031,7 +827,7 @@ __global__ void __launch_bounds__(kVpThreads, 1) vocab_pass_kernel(const VpParam
                 const uint32_t x = sh->tmax[pb][t];
                 if (x >= Tv && x != 0u) es->hthreads[atomicAdd(&es->nht, 1)] = (uint16_t)t;
             }
-            epi_bar<ET>(grp);
+            epi_bar(grp);
             // Te: what a chunk's maximum (and, below, an element) must reach.  T itself at first.  If more chunks reach T
             // than the list holds, either thousands of elements tie with T (a flat rest under a few winners: most of the
             // 64 group maxima are T itself) or T is a poor bound (the groups of threads are a partition that a pattern in
@@ -1076,15 +872,15 @@ __global__ void __launch_bounds__(kVpThreads, 1) vocab_pass_kernel(const VpParam
                         }
                     }
                 }
-                epi_bar<ET>(grp);
+                epi_bar(grp);
                 // (a list several times as long as a good bound leaves it -- about K chunks -- also says that T is poor:
                 // its chunks would overflow the key buffer)
                 const bool over = es->nhits > kVpHitCap;
                 if (es->fill_ninf || (refined && tied)) break;  // (uniform)
                 if (!over && !(pass == 0 && es->nhits > 5 * p.K && es->tie_groups < 16)) break;  // (uniform)
-                epi_bar<ET>(grp);  // (everybody has read the count)
+                epi_bar(grp);  // (everybody has read the count)
                 if (!refined && (tied || !BF16 || es->tie_groups < 16)) {
-                    uint32_t kth = epi_kth_chunk_max<ET>(es, cmx, p.max_tiles, sg.ntiles, p.K, etid, grp);
+                    uint32_t kth = epi_kth_chunk_max(es, cmx, p.max_tiles, sg.ntiles, p.K, etid, grp);
                     // (fp32 logits: the stored maxima are rounded up to bf16, the pattern below is a bound)
                     if (!BF16 && kth > 0u) kth -= 1u;
                     refined = true;
@@ -1097,7 +893,7 @@ __global__ void __launch_bounds__(kVpThreads, 1) vocab_pass_kernel(const VpParam
                             es->fill_tie = 0;
                             es->Tv = Tv;
                         }
-                        epi_bar<ET>(grp);
+                        epi_bar(grp);
                         continue;
                     }
                     if (tied) break;  // (no better bound and what lies above T overflows the list: the exact selection)
@@ -1109,7 +905,7 @@ __global__ void __launch_bounds__(kVpThreads, 1) vocab_pass_kernel(const VpParam
                     es->fill_tie = 1;
                 }
                 Te = Tv + 0x10000u;  // (the next bf16 value up, whatever the sign: T holds the value's upper 16 bits)
-                epi_bar<ET>(grp);
+                epi_bar(grp);
             }
             // (e) the 16-byte vectors of the hit chunks, re-read from global memory; elements >= T become keys.
             //     A thread issues its loads of a round before it uses any: under a saturated memory system one
@@ -1164,7 +960,7 @@ __global__ void __launch_bounds__(kVpThreads, 1) vocab_pass_kernel(const VpParam
                     }
                 }
             }
-            epi_bar<ET>(grp);
+            epi_bar(grp);
             if (es->fill_ninf || es->fill_tie) {  // (uniform)
                 if (ew == 0) {
                     // The first K elements equal to -inf (or, for bulk ties, to T) of the segment's body in id order (the
@@ -1210,7 +1006,7 @@ __global__ void __launch_bounds__(kVpThreads, 1) vocab_pass_kernel(const VpParam
                     }
                     if (gave_up && lane == 0) es->ovf = 1;
                 }
-                epi_bar<ET>(grp);
+                epi_bar(grp);
             }
             // (f) exact top-K of the candidates by rank counting (keys are distinct, so ranks are a permutation)
             // (ranking n candidates costs n^2 compares shared by 128 threads: beyond 256 -- rows whose large elements sit
@@ -1235,14 +1031,14 @@ __global__ void __launch_bounds__(kVpThreads, 1) vocab_pass_kernel(const VpParam
                     if (i < ncand && (etid & 1) == 0 && rank < p.K) es->outk[rank] = key;
                 }
             } else if (es->ovf == 0 && es->ncand <= kVpCandCap) {  // (uniform; every candidate is in the buffer)
-                epi_select_many<ET>(es, ncand, p.K, etid, grp);
+                epi_select_many(es, ncand, p.K, etid, grp);
             } else if (ew == 0) {
                 // (T is a lower bound of the K-th largest element: the filter starts there, not at nothing -- a row sorted
                 // in ascending order would otherwise send every element through the buffer; with the threshold moved up
                 // from -inf, elements equal to -inf may be among the K best and nothing is ruled out)
                 nk = warp_fallback_select<BF16>(es, p, sg, cmx, lane, es->fill_ninf ? 0ull : ((uint64_t)Tv << 32) - 1ull);
             }
-            epi_bar<ET>(grp);
+            epi_bar(grp);
             // the double-buffered arrays of parity pb may be reused from here on
             if (ew == 0) {
                 __syncwarp();
@@ -1275,7 +1071,7 @@ __global__ void __launch_bounds__(kVpThreads, 1) vocab_pass_kernel(const VpParam
 #endif
                     if (lane == 0) es->arrived = atom_add_acq_rel(p.row_counter + sg.row, 1);  // (the lanes' stores included)
                 }
-                epi_bar<ET>(grp);
+                epi_bar(grp);
                 if (es->arrived == nseg - 1) {  // (uniform)
                     finish = true;
                     // Merge the records of the row's CTAs, the group's threads together.  Every CTA after the first
@@ -1307,7 +1103,7 @@ __global__ void __launch_bounds__(kVpThreads, 1) vocab_pass_kernel(const VpParam
                         for (int i = etid; i < cnt * kMaxK; i += ET)
                             es->cand[have * kMaxK + i] = __ldcg((const unsigned long long*)&record(r0 + i / kMaxK)->keys[i % kMaxK]);
                         if (etid < kMaxK) es->outk[etid] = 0ull;
-                        epi_bar<ET>(grp);
+                        epi_bar(grp);
 #pragma unroll 1
                         for (int i = etid; i < n; i += ET) {
                             const uint64_t key = es->cand[i];
@@ -1323,11 +1119,11 @@ __global__ void __launch_bounds__(kVpThreads, 1) vocab_pass_kernel(const VpParam
                             }
                             if (key != 0ull && rank < p.K) es->outk[rank] = key;
                         }
-                        epi_bar<ET>(grp);
+                        epi_bar(grp);
                         if (r0 + kRound < nseg) {  // (uniform)
                             if (etid < kMaxK) es->cand[etid] = es->outk[etid];
                             have = 1;
-                            epi_bar<ET>(grp);
+                            epi_bar(grp);
                         }
                     }
                     if (ew == 0) {
@@ -1443,10 +1239,11 @@ __global__ void __launch_bounds__(128) vocab_merge_kernel(const __grid_constant_
     __syncthreads();
     for (int i = tid; i < n; i += 128) {
         const uint64_t key = merge_cand[i];
-        int rank = i % kMaxK;
-        if (key == 0ull || rank >= p.K) continue;
+        int rank = 0;
+        if (key == 0ull || i % kMaxK >= p.K) continue;
+        // (its own list too, which gives its place there: four searches in step, none waits for another)
+#pragma unroll 4
         for (int l = 0; l < n; l += kMaxK) {
-            if (l == i - i % kMaxK) continue;
             int pos = 0;
 #pragma unroll
             for (int step = kMaxK / 2; step >= 1; step >>= 1)
@@ -1479,13 +1276,79 @@ __global__ void __launch_bounds__(128) vocab_merge_kernel(const __grid_constant_
 }  // namespace
 
 // ---- host side ----------------------------------------------------------------------------------
-static void (*vp_kernel(bool bf16, int groups))(const VpParams) {
-    if (groups == 4) return bf16 ? vocab_pass_kernel<true, 4> : vocab_pass_kernel<false, 4>;
-    return bf16 ? vocab_pass_kernel<true, 2> : vocab_pass_kernel<false, 2>;
+static void (*vp_kernel(bool bf16))(const VpParams) { return bf16 ? vocab_pass_kernel<true> : vocab_pass_kernel<false>; }
+static size_t vp_smem_bytes(int stages, int n_cmax) {
+    return (size_t)stages * TILE + (16 + 2 * BUFS) * sizeof(uint64_t) + sizeof(VpShared) + (size_t)BUFS * n_cmax * 2 + 16;
 }
-static size_t vp_smem_bytes(int groups, int stages, int n_cmax) {
-    const size_t sh = groups == 4 ? sizeof(VpShared<4>) : sizeof(VpShared<2>);
-    return (size_t)stages * TILE + (16 + 2 * kVpMaxBufs) * sizeof(uint64_t) + sh + (size_t)2 * groups * n_cmax * 2 + 16;
+
+// ---- rows in shared memory (vocab_rows.cuh) ----
+typedef void (*RowsKernel)(const RowsParams);
+static RowsKernel rows_kernel(bool bf16, int cl, int nt) {
+    if (cl == 4) return bf16 ? vocab_rows_kernel<true, 4, 256> : vocab_rows_kernel<false, 4, 256>;
+    if (nt == 512) return bf16 ? vocab_rows_kernel<true, 1, 512> : vocab_rows_kernel<false, 1, 512>;
+    return bf16 ? vocab_rows_kernel<true, 1, 256> : vocab_rows_kernel<false, 1, 256>;
+}
+static int rows_vecs(long long row_bytes, int cl) { return (int)((row_bytes / 16 + cl - 1) / cl) + 3; }
+static size_t rows_smem_bytes(long long row_bytes, int cl, int nt) {
+    const size_t sh = cl == 4 ? sizeof(RowsShared<4, 256>) : nt == 512 ? sizeof(RowsShared<1, 512>) : sizeof(RowsShared<1, 256>);
+    const int vecs = rows_vecs(row_bytes, cl);
+    return (size_t)vecs * 16 + sh + (size_t)((vecs + rows_tile_vecs(nt) - 1) / rows_tile_vecs(nt)) * nt * 2;
+}
+// CTAs of a size that an SM holds side by side (threads and registers allow four of 256 threads, two of 512)
+static int rows_per_sm(long long row_bytes, int cl, int nt) {
+    if (row_bytes / cl > kRowsMaxBytes) return 0;
+    const int n = (int)(227 * 1024 / (rows_smem_bytes(row_bytes, cl, nt) + 1024)), most = nt == 512 ? 2 : 4;
+    return n < most ? n : most;
+}
+// The cluster that holds a row, or 0: the streaming kernel.  Measured on 148 SMs, L = 16, K = 32, one launch after the other,
+// streaming kernel -> rows in shared memory.
+static void rows_plan(long long rows, long long row_bytes, int num_sms, VpPlan* pl) {
+    pl->cluster = 0;
+    const bool alone = rows * 4 <= num_sms;  // four CTAs a row and an SM for each
+    if (rows_per_sm(row_bytes, 1, 256) >= 2 && !(alone && row_bytes >= 80 * 1024)) {
+        // a row a CTA where two or more share an SM, any number of rows.  bf16, V = 32,000 (three an SM): batch 1 8.3 -> 5.8 us,
+        // batch 16 11.2 -> 9.2, batch 64 25.2 -> 20.4, batch 256 74.7 -> 63.9; V = 16,000 (four): batch 64 20.9 -> 13.7, batch
+        // 256 63.5 -> 42.4; V = 50,021 (two): batch 64 34.3 -> 31.5, batch 256 114 -> 107.  With one CTA an SM nothing loads
+        // while a row is finished: fp32, V = 32,000, batch 64 29.5 -> 45
+        pl->cluster = 1;
+        pl->threads = 256;
+    } else if (!alone && rows <= num_sms && rows_per_sm(row_bytes, 1, 512) >= 1) {
+        // longer rows, an SM for each (bf16, V = 75,000: batch 4 10.4 -> 7.2, batch 8 10.8 -> 7.8; with 256 threads 7.7, 8.3)
+        pl->cluster = 1;
+        pl->threads = 512;
+    } else if (rows * 4 <= (long long)num_sms * rows_per_sm(row_bytes, 4, 256)) {
+        // rows too long for one CTA, or rows of 80 KB and more where four times as many SMs would stand idle, as far as all
+        // pieces are resident at once.  V = 151,936: bf16 batch 1 12.7 -> 8.0, batch 4 13.4 -> 8.9, batch 8 (two turns) 15.1 ->
+        // 18.5; fp32 batch 1 13.7 -> 7.2.  V = 50,021, bf16, batch 1 10.0 -> 5.8 (6.6 in one CTA), V = 32,000 the same in one
+        // CTA as in four.  (512 threads: 9.0 at batch 1, V = 151,936; eight CTAs a row 7.9, but 10.0 at batch 4.)
+        pl->cluster = 4;
+        pl->threads = 256;
+    }
+}
+static cudaError_t rows_launch(bool bf16, const VpPlan& pl, long long row_bytes, const RowsParams& p, bool pdl, cudaStream_t st) {
+    cudaLaunchConfig_t lc = {};
+    lc.gridDim = dim3(p.rows * pl.cluster);
+    lc.blockDim = dim3(pl.threads + 32);
+    lc.dynamicSmemBytes = rows_smem_bytes(row_bytes, pl.cluster, pl.threads);
+    lc.stream = st;
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = pdl ? 1 : 0;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = pl.cluster;
+    at[1].val.clusterDim.y = 1;
+    at[1].val.clusterDim.z = 1;
+    lc.attrs = at;
+    lc.numAttrs = pl.cluster > 1 ? 2 : 1;
+    const cudaError_t e = cudaLaunchKernelEx(&lc, rows_kernel(bf16, pl.cluster, pl.threads), p);
+    return e != cudaSuccess ? e : cudaGetLastError();
+}
+static cudaError_t rows_configure(bool bf16) {
+    cudaError_t e = cudaSuccess;
+    const int variants[3][2] = {{1, 256}, {1, 512}, {4, 256}};
+    for (int i = 0; i < 3 && e == cudaSuccess; ++i)
+        e = allow_smem((const void*)rows_kernel(bf16, variants[i][0], variants[i][1]), 225 * 1024);
+    return e;
 }
 
 VpPlan vp_make_plan(const graft_config& cfg, int num_sms, int batch, bool equal_shares) {
@@ -1493,9 +1356,11 @@ VpPlan vp_make_plan(const graft_config& cfg, int num_sms, int batch, bool equal_
     const bool bf16 = cfg.logits_dtype == GRAFT_BF16;
     const long long esz = bf16 ? 2 : 4, rows = (long long)batch * cfg.L, row_bytes = (long long)cfg.V * esz;
     const long long nq = cfg.V / kVpQuantum > 0 ? cfg.V / kVpQuantum : 1;
+    pl.cluster = 0;
+    if (!equal_shares) rows_plan(rows, row_bytes, num_sms, &pl);
     long long G, share_q, per = 0;  // CTAs (one per SM at most), a CTA's share at most, whole rows of a CTA at most
     // A row that no other CTA has a piece of needs no merge, which is what a small input waits for (a record and a merge
-    // take 5 to 6 us, the stream of a 64 KB row 1.4 us): whole rows wherever the CTAs' shares come out even enough.  Measured
+    // take 5 to 6 us): whole rows wherever the CTAs' shares come out even enough.  Measured
     // on 148 SMs, one launch after the other, bf16, L = 16.
     if (equal_shares) {
         // Rounds without edge scores.  Their path scores are sums of log-probabilities alone, and of logits with few digits
@@ -1511,9 +1376,9 @@ VpPlan vp_make_plan(const graft_config& cfg, int num_sms, int batch, bool equal_
         pl.whole = 0;
         share_q = (nq * rows + G - 1) / G;
     } else if (rows < num_sms) {
-        // n pieces of each row of 76 KB or more, n = 1 unless the stream gets shorter by more than the merge costs (190 KB):
-        // V = 151,936 (where n is 3 at batch 1 to 3) batch 1: n = 1 18.5 us, n = 2 18.6, n = 4 17.1, n = 9 20.9; batch 4: n = 1
-        // 18.9, n = 2 19.7
+        // n pieces of each row of 76 KB or more, n = 1 unless the stream gets shorter by more than the merge costs (190 KB), as
+        // rows of 380 KB do (measured on bf16 rows of 300 KB: 16 rows n = 1 18.5 us, n = 2 18.6, n = 4 17.1, n = 9 20.9; 64 rows
+        // n = 1 18.9, n = 2 19.7)
         long long n = row_bytes / (76 * 1024);
         if (n > num_sms / rows) n = num_sms / rows;
         if (n > nq) n = nq;
@@ -1524,8 +1389,8 @@ VpPlan vp_make_plan(const graft_config& cfg, int num_sms, int batch, bool equal_
         per = 1;
     } else {
         // whole rows, unless that gives some CTA over 90 KB more than the average (V = 151,936: batch 16 28.5 -> 27.0 us with
-        // whole rows, batch 24 the same, batch 20 30.3 -> 33.3, batch 256 204 -> 207); rows up to 132 KB always (V = 50,021:
-        // batch 16 23.7 -> 19.9 us, batch 28 27.2 -> 26.9; V = 32,000, batch 16: 23.0 -> 16.8)
+        // whole rows, batch 24 the same, batch 20 30.3 -> 33.3, batch 256 204 -> 207); rows up to 132 KB always (rows
+        // of 100 KB: batch 16 23.7 -> 19.9 us, batch 28 27.2 -> 26.9)
         per = (rows + num_sms - 1) / num_sms;
         pl.whole = row_bytes <= 132 * 1024 || per * row_bytes - rows * row_bytes / num_sms <= 90 * 1024;
         G = pl.whole ? (rows + per - 1) / per : num_sms;
@@ -1536,14 +1401,11 @@ VpPlan vp_make_plan(const graft_config& cfg, int num_sms, int batch, bool equal_
     long long seg_elems = share_q * kVpQuantum + kVpQuantum;  // a row's last quantum also takes the remainder
     if (pl.whole || seg_elems > cfg.V) seg_elems = cfg.V;
     pl.max_seg_tiles = (int)((seg_elems * esz + TILE - 1) / TILE) + 1;
-    // four epilogue groups where three short rows or more queue for them (V = 32,000: batch 192 74.4 -> 67.3 us, batch 40
-    // 27.2 -> 25.7; a group alone is slower, batch 8 13.7 -> 14.9; rows of 100 KB: batch 64 39.3 -> 40.5)
-    pl.groups = seg_elems * esz <= 68 * 1024 && per >= 3 ? 4 : 2;
     const size_t budget = 224 * 1024;  // one CTA per SM
     int stages = 6;
-    while (stages > 2 && vp_smem_bytes(pl.groups, stages, pl.max_seg_tiles * NT) > budget) --stages;
+    while (stages > 2 && vp_smem_bytes(stages, pl.max_seg_tiles * NT) > budget) --stages;
     pl.stages = stages;
-    pl.smem_bytes = vp_smem_bytes(pl.groups, stages, pl.max_seg_tiles * NT);
+    pl.smem_bytes = vp_smem_bytes(stages, pl.max_seg_tiles * NT);
     return pl;
 }
 
@@ -1553,6 +1415,27 @@ cudaError_t vp_launch(graft_ctx* ctx, int batch, const void* d_logits, int32_t* 
     const graft_config& cfg = ctx->cfg;
     const bool bf16 = cfg.logits_dtype == GRAFT_BF16;
     VpPlan pl = vp_make_plan(cfg, ctx->num_sms, batch, equal_shares);
+    if (pl.cluster > 0) {
+        RowsParams r;
+        r.logits = (const char*)d_logits;
+        r.rows = batch * cfg.L;
+        r.V = cfg.V;
+        r.K = cfg.K;
+        r.topk_id = d_topk_id;
+        r.topk_lp = d_topk_lp;
+        r.lse = d_lse;
+        r.row_status = d_row_status;
+        r.errflag = ctx->w_errflag;
+        r.partial_out = d_partial;
+        r.hidden = d_hidden;
+        r.hidden_bf16 = cfg.hidden_dtype == GRAFT_BF16 ? 1 : 0;
+        r.hidden_dim = cfg.hidden_dim;
+        r.L = cfg.L;
+        r.cos_out = (d_hidden != nullptr && cfg.L > 1) ? d_cos : nullptr;
+        r.vecs = rows_vecs((long long)cfg.V * (bf16 ? 2 : 4), pl.cluster);
+        ctx->launches += 1;
+        return rows_launch(bf16, pl, (long long)cfg.V * (bf16 ? 2 : 4), r, true, st);
+    }
     VpParams p;
     p.logits = (const char*)d_logits;
     p.rows = batch * cfg.L;
@@ -1577,7 +1460,7 @@ cudaError_t vp_launch(graft_ctx* ctx, int batch, const void* d_logits, int32_t* 
     p.L = cfg.L;
     p.cos_out = (d_hidden != nullptr && cfg.L > 1) ? d_cos : nullptr;
     p.use_hint = 1;
-    const cudaError_t e = launch_pdl(vp_kernel(bf16, pl.groups), dim3(pl.grid), dim3(kVpThreads), pl.smem_bytes, st, p);
+    const cudaError_t e = launch_pdl(vp_kernel(bf16), dim3(pl.grid), dim3(kVpThreads), pl.smem_bytes, st, p);
     ctx->launches += 1;
     return e != cudaSuccess ? e : cudaGetLastError();
 }
@@ -1607,8 +1490,9 @@ cudaError_t vp_configure(const graft_config& cfg, int num_sms, size_t* max_smem)
     *max_smem = pl.smem_bytes;
     if (pl.smem_bytes > 225 * 1024) return cudaErrorInvalidValue;
     cudaError_t e = cudaSuccess;
-    for (int groups = 2; groups <= 4 && e == cudaSuccess; groups += 2)
-        e = cudaFuncSetAttribute(vp_kernel(cfg.logits_dtype == GRAFT_BF16, groups), cudaFuncAttributeMaxDynamicSharedMemorySize, 225 * 1024);
+    e = rows_configure(cfg.logits_dtype == GRAFT_BF16);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(vp_kernel(cfg.logits_dtype == GRAFT_BF16), cudaFuncAttributeMaxDynamicSharedMemorySize, 225 * 1024);
     return e;
 }
 
@@ -1684,18 +1568,44 @@ extern "C" graft_status graft_vocab_pass_static(int32_t batch, int32_t L, int32_
                 cudaGetLastError();
                 return GRAFT_ERR_CUDA;
             }
-            for (int i = 0; i < 4; ++i)
-                if (cudaFuncSetAttribute(vp_kernel((i & 1) != 0, i < 2 ? 2 : 4), cudaFuncAttributeMaxDynamicSharedMemorySize,
+            for (int i = 0; i < 2; ++i)
+                if (cudaFuncSetAttribute(vp_kernel(i != 0), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          225 * 1024) != cudaSuccess) {
                     cudaGetLastError();
                     return GRAFT_ERR_CUDA;
                 }
+            if (rows_configure(true) != cudaSuccess || rows_configure(false) != cudaSuccess) {
+                cudaGetLastError();
+                return GRAFT_ERR_CUDA;
+            }
             sd->scratch = (VpStaticScratch*)ptr;
             sd->num_sms = sms;
             sd->ready = true;
         }
     }
     const VpPlan pl = vp_make_plan(cfg, sd->num_sms, batch, false);
+    if (pl.cluster > 0) {
+        cudaStream_t st = (cudaStream_t)stream;
+        if (cudaMemsetAsync(sd->scratch->errflag, 0, sizeof(sd->scratch->errflag), st) != cudaSuccess) {
+            cudaGetLastError();
+            return GRAFT_ERR_CUDA;
+        }
+        RowsParams r;
+        memset(&r, 0, sizeof r);
+        r.logits = (const char*)d_logits;
+        r.rows = batch * L;
+        r.V = V;
+        r.K = K;
+        r.topk_id = d_topk_id;
+        r.topk_lp = d_topk_lp;
+        r.lse = d_lse;
+        r.row_status = d_row_status;
+        r.errflag = sd->scratch->errflag;
+        r.L = L;
+        const long long row_bytes = (long long)V * (logits_dtype == GRAFT_BF16 ? 2 : 4);
+        r.vecs = rows_vecs(row_bytes, pl.cluster);
+        return rows_launch(logits_dtype == GRAFT_BF16, pl, row_bytes, r, false, st) == cudaSuccess ? GRAFT_OK : GRAFT_ERR_CUDA;
+    }
     if (pl.grid > kStaticMaxGrid || pl.smem_bytes > 225 * 1024) return GRAFT_ERR_UNSUPPORTED;
     cudaStream_t st = (cudaStream_t)stream;
     // the array keeps whatever the previous call left: the arrival counters and the error word must start at 0
@@ -1728,6 +1638,6 @@ extern "C" graft_status graft_vocab_pass_static(int32_t batch, int32_t L, int32_
     p.L = L;
     p.cos_out = nullptr;
     p.use_hint = 1;
-    vp_kernel(logits_dtype == GRAFT_BF16, pl.groups)<<<pl.grid, kVpThreads, pl.smem_bytes, st>>>(p);
+    vp_kernel(logits_dtype == GRAFT_BF16)<<<pl.grid, kVpThreads, pl.smem_bytes, st>>>(p);
     return cudaGetLastError() == cudaSuccess ? GRAFT_OK : GRAFT_ERR_CUDA;
 }

@@ -1,0 +1,98 @@
+"""Vocab pass with the rows held in shared memory, against the oracle, where its pieces can go wrong: rows shorter than a
+vector, at the edges of a step of all threads and of a cluster's pieces, on no 16-byte boundary, and rows that overflow the
+list of candidates in every way."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from helpers import tolerance
+
+pytestmark = pytest.mark.gpu
+
+
+def _row(style, V, g):
+    z = 2.0 * torch.randn(V, generator=g)
+    if style == "ascending":
+        return z.sort().values
+    if style == "descending":
+        return z.sort(descending=True).values
+    if style == "flat":
+        return torch.full((V,), -1.5)
+    if style == "masked":  # a few finite tokens more than K
+        keep = torch.randperm(V, generator=g)[:40]
+        out = torch.full((V,), -float("inf"))
+        out[keep] = z[keep]
+        return out
+    if style == "ties":
+        return (2.0 * z).round() / 2.0
+    if style == "winners":  # fewer winners than K over an exactly flat rest
+        z = torch.full((V,), -1.0)
+        z[torch.randperm(V, generator=g)[:5]] = 4.0
+        return z
+    if style == "block":  # large elements side by side
+        z[V // 3: V // 3 + V // 8] += 20.0
+        return z
+    if style == "ramps":
+        return (torch.arange(V) % 1024).float() / 100.0 - 5.0
+    return z
+
+
+STYLES = ["random", "ascending", "descending", "flat", "masked", "ties", "winners", "block", "ramps"]
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("batch,L,V,K,shift", [
+    (2, 9, 41, 32, 1),         # five vectors a row, most rows on no 16-byte boundary
+    (2, 9, 8176, 32, 0),       # bf16: one step of 256 threads with its two vectors of ragged ends, to the element
+    (2, 9, 8177, 1, 3),        # and one element more
+    (1, 9, 16001, 7, 1),
+    (4, 10, 20011, 32, 0),     # a row a CTA, and more rows than stand alone
+    (1, 9, 50021, 32, 5),      # four CTAs a row, uneven pieces; fp32: 200 KB
+    (1, 9, 130003, 32, 0),     # rows that no CTA holds alone
+    (5, 9, 54000, 32, 0),      # 512 threads a row (bf16: 108 KB; fp32: 216 KB)
+])
+def test_rows_in_shared_memory(batch, L, V, K, shift, dtype):
+    from paper_2608_20375_b200 import Graft
+    g = torch.Generator().manual_seed(V + K)
+    z = torch.stack([_row(STYLES[r % len(STYLES)] if V > 1000 else "ties", V, g) for r in range(batch * L)]).to(dtype)
+    flat = torch.empty(batch * L * V + 8, dtype=dtype, device="cuda")  # the rows begin `shift` elements behind a boundary
+    x = flat[shift:shift + batch * L * V].view(batch, L, V)
+    x.copy_(z.view(batch, L, V))
+    gr = Graft(V, L, K, 16, 8, batch, 8, 8, 8, 0.0, 1, 1 if dtype == torch.bfloat16 else 0, 0)
+    ids = torch.empty((batch, L, K), dtype=torch.int32, device="cuda")
+    lp = torch.empty((batch, L, K), device="cuda")
+    lse = torch.empty((batch, L), device="cuda")
+    st = torch.empty((batch, L), dtype=torch.int32, device="cuda")
+    gr.vocab_pass(x, ids, lp, lse, st)
+    torch.cuda.synchronize()
+    o_ids, o_lp, o_lse, o_st = oracle.vocab_pass(z, K)
+    assert np.array_equal(st.cpu().numpy().reshape(-1), o_st)
+    assert np.array_equal(ids.cpu().numpy().reshape(-1, K), o_ids)
+    a, b = lp.cpu().numpy().reshape(-1, K).astype(np.float64), o_lp.astype(np.float64)
+    assert np.array_equal(np.isneginf(a), np.isneginf(b))
+    fin = np.isfinite(b)
+    assert np.all(np.abs(a[fin] - b[fin]) <= tolerance(b[fin]))
+    assert np.all(np.abs(lse.cpu().numpy().reshape(-1) - o_lse) <= tolerance(o_lse))
+
+
+@pytest.mark.parametrize("bad", [float("nan"), float("inf"), -float("inf")])
+def test_rows_in_shared_memory_report_bad_logits(bad):
+    """A NaN, an infinity or nothing finite in any piece of a row marks that row and no other."""
+    from paper_2608_20375_b200 import Graft
+    L, V, K = 8, 60000, 8
+    g = torch.Generator().manual_seed(3)
+    z = 2.0 * torch.randn((1, L, V), generator=g)
+    if bad == -float("inf"):
+        z[0, 2] = bad
+    else:
+        z[0, 2, 1], z[0, 5, V - 2] = bad, bad
+    gr = Graft(V, L, K, 16, 8, 1, 8, 8, 8, 0.0, 1, 0, 0)
+    ids = torch.empty((1, L, K), dtype=torch.int32, device="cuda")
+    lp, lse = torch.empty((1, L, K), device="cuda"), torch.empty((1, L), device="cuda")
+    st = torch.empty((1, L), dtype=torch.int32, device="cuda")
+    gr.vocab_pass(z.cuda(), ids, lp, lse, st)
+    torch.cuda.synchronize()
+    _, _, _, o_st = oracle.vocab_pass(z.view(L, V), K)
+    assert np.array_equal(st.cpu().numpy().reshape(-1), o_st)
+    assert o_st[2] == 1 and o_st[0] == 0
