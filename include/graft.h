@@ -135,12 +135,15 @@ int32_t graft_edge_rows(const graft_ctx* ctx);
 /* Table precompute (same passage): d_out[v] = W e_v + b for one tower.  d_emb [V, E] (dtype as given),
  * d_W [m, E] fp32, d_b [m] fp32 or NULL, d_out [V, m] fp32.  fp32 accumulation.  Call once per tower.
  * With d_emb and d_out 16-byte aligned and E a multiple of 8 (bf16) or 4 (fp32) the products run on the tensor cores:
- * fp32 numbers enter as three bf16 parts, whose products are exact.  Against a chain of fp32 multiply-adds the result
- * differs by the order and the rounding of the additions and, for fp32 embeddings, by the products left out, below 2^-26 of
- * a term (largest error against fp64 products of N(0, 1) results 3.2e-6 at E = 4096, 3.0e-6 at E = 2048 in fp32; the chain:
- * 1.2e-5).  With fp32 embeddings, infinities and values up to the largest fp32 give what fp32 arithmetic gives; a bf16
- * embedding or a W beside bf16 embeddings that is infinite, or a W that rounds past the largest bf16, gives NaN.
- * Such calls use scratch of the context (3 m E bf16 values and up to 40 MB of partial sums, m rounded up to 128), which the
+ * W beside bf16 embeddings enters as three bf16 parts, fp32 embeddings and their W as two scaled fp16 parts each; products of
+ * parts are exact.  Against a chain of fp32 multiply-adds the result differs by the order and the rounding of the additions
+ * and, for fp32 embeddings, by the products left out, below 2^-24 of a term (largest error against fp64 products of N(0, 1)
+ * results 3.4e-6 at E = 4096, 2.2e-6 at E = 2048 in fp32; the chain: 1.2e-5).  With fp32 embeddings, rows whose largest entry is
+ * over 2^7 times larger or 2^18 times smaller than most rows' are worked out by such a chain, more slowly; other entries are held to
+ * 22 bits or 2^-26 of their row's largest, those of W to 22 bits or 2^-50; infinities and values up to the largest fp32 give what
+ * fp32 arithmetic gives.  A
+ * bf16 embedding or a W beside bf16 embeddings that is infinite, or a W that rounds past the largest bf16, gives NaN.
+ * Such calls use scratch of the context (3 m E 16-bit values, V bytes and up to 40 MB of partial sums, m rounded up to 128), which the
  * first of them allocates and one that needs more replaces -- under stream capture too; a captured call keeps the scratch it
  * was captured with until the context is destroyed.  Without memory for it, and for other pointers and E, an FMA kernel
  * takes the call.  This is the once-per-model setup step, not the round. */

@@ -283,7 +283,7 @@ graft_status graft_tdes_precompute(graft_ctx* ctx, const void* d_emb, graft_dtyp
     if (emb_dtype != GRAFT_F32 && emb_dtype != GRAFT_BF16) return GRAFT_ERR_INVALID_ARG;
     // the tensor cores (bf16 parts of the inputs, exact products), where the rows fit and their scratch is to be had
     if (tables_mma_fits(d_emb, emb_dtype, E, d_out)) {
-        void* scratch = tables_scratch(ctx, tables_mma_scratch_bytes(ctx->num_sms, E, ctx->cfg.m, emb_dtype));
+        void* scratch = tables_scratch(ctx, tables_mma_scratch_bytes(ctx->num_sms, ctx->cfg.V, E, ctx->cfg.m, emb_dtype));
         if (scratch != nullptr) {
             if (tables_mma_launch(ctx, d_emb, emb_dtype, E, d_W, d_b, d_out, scratch, (cudaStream_t)stream) == cudaSuccess)
                 return GRAFT_OK;

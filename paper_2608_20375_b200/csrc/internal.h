@@ -157,7 +157,7 @@ cudaError_t tdes_precompute_launch(graft_ctx* ctx, const void* d_emb, graft_dtyp
                                    const float* d_b, float* d_out, cudaStream_t st);
 // table precompute on the tensor cores (csrc/tables_mma.cu); inputs that do not fit go to tdes_precompute_launch
 bool tables_mma_fits(const void* d_emb, graft_dtype dt, int E, const void* d_out);
-size_t tables_mma_scratch_bytes(int num_sms, int E, int m, graft_dtype dt);
+size_t tables_mma_scratch_bytes(int num_sms, int V, int E, int m, graft_dtype dt);
 cudaError_t tables_mma_launch(graft_ctx* ctx, const void* d_emb, graft_dtype dt, int E, const float* d_W, const float* d_b,
                               float* d_out, void* scratch, cudaStream_t st);
 cudaError_t tdes_edges_launch(graft_ctx* ctx, int batch, const int32_t* d_topk_id, const float* d_topk_lp,

@@ -1,22 +1,27 @@
 // Table precompute on the tensor cores: out[v] = W e_v + b (text after Eq. 6: the projections depend only on the token
 // id and are computed once).  This is the one dense contraction of the method, [V, E] x [E, m].
 //
-// Operands are bf16 parts of the inputs: an fp32 number is the sum of three bf16 ones (8 + 8 + 8 mantissa bits), and a
-// product of two bf16 numbers is exact in the fp32 accumulator.
-//   bf16 embeddings: out = e W1 + e W2 + e W3               (three products a step, all exact)
-//   fp32 embeddings: out = (e1 + e2 + e3) W1 + ((e1 + e2 + e3) W2 + e1 W3)   (what is dropped is below 2^-26 of a term)
+// Operands are 16-bit parts of the inputs; products of parts are exact in the fp32 accumulator.
+//   bf16 embeddings: out = e W1 + e W2 + e W3, W as three bf16 parts (8 + 8 + 8 mantissa bits; three products a step)
+//   fp32 embeddings: out = e1 W1 + (e1 W2 + e2 W1), both as two fp16 parts (11 + 11 bits and the second part's sign; what is
+//     dropped, e2 W2, is below 2^-24 of a term and 2^-26 of it on average).  fp16 has few exponents, so a row of W is scaled by
+//     its largest entry and the embeddings by a power of two from a sample; second parts are kept times 2^11, and go to an
+//     accumulator of their own.  Rows of the embeddings that this does not suit are worked out in fp32.
 // so the result differs from an fp32 GEMM by the order and the rounding of the additions.  The accumulators of the tensor
-// cores round less carefully than an FMA chain: they are emptied into fp32 registers after 32 (bf16) or 24 (fp32
-// embeddings) additions to the large products' accumulators, which W2's and W3's do not share.
+// cores round less carefully than an FMA chain, the less so the more bits the products have: they are emptied into fp32
+// registers after 32 (bf16) or 16 (fp32 embeddings) additions to the large products' accumulators, which the small products do not
+// share.  (fp16 parts for bf16 embeddings too, two products instead of three: the conversion in shared memory and the shorter
+// chunks that the longer products need cost more than the third product, 398 against 375 us a tower, and at 32 additions the
+// error was a third larger.)
 //
 // One persistent kernel.  A worker -- a pair of CTAs (cluster of two, tcgen05 cta_group::2) for bf16 embeddings, one CTA
 // for fp32 -- owns a tile of 512 (fp32: 128) rows of V times up to 128 columns of m, and streams E in blocks of 64 (32)
 // columns through shared-memory rings.
 //   warps 0-7    empty the accumulators (TMEM, two sets of 2 x 128 columns), keep the running sums and write the tile
-//   warp 8       TMA loads: W's parts (split once per call into scratch by weight_split_kernel), bf16 embeddings
+//   warp 8       TMA loads: W's parts (split once per call into scratch by a small kernel), bf16 embeddings
 //   warp 9       issues the matrix instructions
-//   warp 10      fp32 only: TMA loads of the raw rows;  warps 11-18  raw rows -> bf16 parts in the operands' layout
-// W1 and W2 stand side by side as one operand of N = 256, W3 is an N = 128 of its own (three of N = 128 in a row on one
+//   warp 10      fp32 only: TMA loads of the raw rows;  warps 11-18  raw rows -> fp16 parts in the operands' layout
+// W1 and W2 stand side by side as one operand of N = 256, the third product is an N = 128 of its own (three of N = 128 in a row on one
 // accumulator took 122 cycles each: an instruction waits for the one ahead of it on the same columns).  Tiles of 512
 // rows halve the passes over W, which comes from L2 every time.  The fp32 kernel works on single CTAs because its rows
 // go through threads: telling the other CTA of a pair about every block cost more (136 - 160 us at V = 32,000, E = 2048)
@@ -24,12 +29,16 @@
 // written.  What is left when the tiles do not divide by the workers is dealt out along E in shares, whose sums a
 // small kernel adds up in order (summing them inside, by the warp that came last, stalled its tile: 462 against 370 us).
 //
-// Measured (one tower, back to back, B200): V = 151,936, E = 4096, m = 128, bf16: 373 us (798 us with the library
-// template's GEMMs, whose partial sums went through memory); its products take 287 us at the measured dense rate, the
-// loads alone 258 us.  V = 32,000, E = 2048, fp32: 120 us (1180 us by the FMA kernel; the loads and the splitting 82 us).
-// Largest error against fp64 products at those sizes: 3.2e-6 and 3.0e-6 (library template 6.3e-6, FMA kernel 1.2e-5).
+// Measured (one tower, back to back, B200): V = 151,936, E = 4096, m = 128, bf16: 358 us (375 before rows and W shared a barrier
+// and the first row block went two blocks ahead where accumulators are emptied; 798 us with the library template's GEMMs); its products
+// take 287 us at the measured dense rate, and the clock falls to 1.5 GHz on the way.  V = 32,000, E = 2048, fp32: 91 us (121 with
+// three bf16 parts, seven products; 1180 us by the FMA kernel).  What bounds the fp32 kernel: the one thread that issues, 0.6 k
+// cycles a block of 32 columns beside 0.4 k of products, and the eight warps that split.  Error against fp64 products at those
+// sizes, largest and root mean square over the results' size: bf16 2.7e-6 and 4.7e-7; fp32 2.2e-6 and 3.4e-7 (bf16 parts 2.7e-6 and 4.7e-7; FMA kernel
+// 1.2e-5 at most).
 #include <cuda.h>
 #include <cuda_bf16.h>
+#include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
 #include "internal.h"
@@ -49,17 +58,19 @@ struct TablesCfg {
     static constexpr int MT = F32 ? 1 : 2;     // row blocks of 128 a CTA works on at a time
     static constexpr int ROWS = F32 ? 128 : 512;  // rows of V per tile
     static constexpr int BLK = F32 ? 32 : 64;  // columns of E per block: rows of 64 or 128 bytes of bf16
-    static constexpr int CHUNK = F32 ? 4 : 8;  // blocks between two emptyings of an accumulator
-    static constexpr int PART = 128 * BLK * 2;                // bytes of 128 rows of bf16
-    static constexpr int A_BYTES = (F32 ? 3 : MT) * PART;     // a block's embeddings
-    static constexpr int W_BYTES = (F32 ? 384 : 192) * BLK * 2;  // a block's W; a pair: W1 (even CTA) or W2 (odd), half of W3
+    static constexpr int CHUNK = 8;            // blocks between two emptyings of an accumulator
+    static constexpr int PART = 128 * BLK * 2;                // bytes of 128 rows of 16-bit numbers
+    static constexpr int A_BYTES = 2 * PART;                  // a block's embeddings: two row blocks, or two parts
+    static constexpr int W_BYTES = (F32 ? 256 : 192) * BLK * 2;  // a block's W; a pair: W1 (even CTA) or W2 (odd), half of W3
     static constexpr int RAW = 128 * BLK * 4;                 // a block's fp32 embeddings
-    static constexpr int A_STAGES = F32 ? 3 : 4, W_STAGES = F32 ? 3 : 4, RAW_STAGES = F32 ? 4 : 1;
+    static constexpr int STAGES = 4, RAW_STAGES = F32 ? 5 : 1;  // (a stage: a block's embeddings and W)
     static constexpr int THREADS = (kTmEpiWarps + 2 + (F32 ? 1 + kTmConvWarps : 0)) * 32;
     // (the rings start on a 1024-byte boundary)
-    static constexpr size_t SMEM = (size_t)A_STAGES * A_BYTES + (size_t)W_STAGES * W_BYTES + (F32 ? (size_t)RAW_STAGES * RAW : 0) + 1024;
+    static constexpr size_t SMEM = (size_t)STAGES * (A_BYTES + W_BYTES) + (F32 ? (size_t)RAW_STAGES * RAW : 0) + 1024;
     static __device__ __forceinline__ uint64_t desc(uint32_t addr) { return F32 ? umma_desc_sw64(addr) : umma_desc_sw128(addr); }
 };
+
+constexpr float kTmLow = 2048.0f;  // fp16: second parts are kept times 2^11
 
 // A walk over the N stages of a ring: stages passed so far, the stage, the parity to wait for.
 template <uint32_t N>
@@ -89,13 +100,17 @@ struct TablesRing {
 };
 
 struct __align__(64) TablesParams {
-    CUtensorMap map_w;  // [3 * m_pad, E_pad] bf16
+    CUtensorMap map_w;  // [parts * m_pad, E_pad]: three bf16 parts, or two fp16 ones
     CUtensorMap map_e;  // [V, E] embeddings
     const void* emb;    // [V, E]
     const float* W;     // [m, E]
     const float* bias;  // [m] or NULL
     float* out;         // [V, m]
     float* pieces;      // [pairs][2 pieces][ROWS][128]
+    // fp32 embeddings only
+    const float2* unscale;  // [m_pad] what a column's sums are multiplied by, as two factors
+    const float* scale;     // [1] what the embeddings are multiplied by
+    uint8_t* bad_row;       // [tiles of V][ROWS] rows whose entries fp16 parts do not hold well enough
     int32_t* errflag;
     int V, E, m, m_pad, n_mb, n_kb;
     int pairs, full_rounds;
@@ -169,15 +184,119 @@ __global__ void __launch_bounds__(256) weight_split_kernel(const float* __restri
     }
 }
 
-// two fp32 numbers -> their three bf16 parts, packed
-__device__ __forceinline__ void split3(float x0, float x1, uint32_t& a, uint32_t& b, uint32_t& c) {
-    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(a) : "f"(x1), "f"(x0));
-    x0 -= __uint_as_float(a << 16);
-    x1 -= __uint_as_float(a & 0xFFFF0000u);
-    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(b) : "f"(x1), "f"(x0));
-    x0 -= __uint_as_float(b << 16);
-    x1 -= __uint_as_float(b & 0xFFFF0000u);
-    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(c) : "f"(x1), "f"(x0));
+// 2^x for a whole number x, as far as fp32 has it
+__device__ __forceinline__ float tables_exp2(int x) { return __uint_as_float((uint32_t)(127 + (x < -126 ? -126 : x > 127 ? 127 : x)) << 23); }
+
+// W (fp32, [m, E]) -> two fp16 parts [2][m_pad][E_pad], zero where padded: a row is multiplied by the power of two that takes
+// its largest entry to [2^13, 2^14), W1 is what fp16 holds of it and W2 what it holds of the rest, times 2^11.  Every block
+// (a row each) also looks at a sample of the embeddings, the same sample: the power of two that takes the median of 256 threads'
+// largest entries to [2^8, 2^9) is what they will be multiplied by, so that rows up to 2^8 times larger or smaller stay within fp16's
+// exponents.  And clears the flags of rows that do not.
+__global__ void __launch_bounds__(256) weight_split16_kernel(const float* __restrict__ W, const float* __restrict__ emb, int V, int m, int E,
+                                                           int m_pad, int E_pad, __half* __restrict__ w, float2* __restrict__ unscale,
+                                                           float* __restrict__ scale, uint32_t* __restrict__ flags, int n_flags) {
+    __shared__ float s_max[8];
+    __shared__ int s_hist[256];
+    __shared__ int s_mid;
+    pdl_launch_dependents();
+    const int r = blockIdx.x, tid = threadIdx.x;
+    s_hist[tid] = 0;
+    if (tid == 0) s_mid = 127 + 8;  // (nothing but zeros: scale 1)
+    for (int i = r * 256 + tid; i < n_flags; i += (int)gridDim.x * 256) flags[i] = 0u;
+    // the sample: four pieces of 16 bytes a thread, from a row of its own
+    float x = 0.f;
+    {
+        const size_t row = (size_t)((long long)tid * V / 256) * E;
+        const int n4 = E / 4;
+        float4 v[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            v[i] = __ldg((const float4*)(emb + row) + (int)((long long)(tid * 4 + i) * 37 % n4));
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const float q[4] = {fabsf(v[i].x), fabsf(v[i].y), fabsf(v[i].z), fabsf(v[i].w)};
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if (q[k] < INFINITY) x = fmaxf(x, q[k]);
+        }
+    }
+    // the row's largest finite entry
+    float top = 0.f;
+    if (r < m)
+        for (int e = tid; e < E; e += 256) {
+            const float a = fabsf(W[(size_t)r * E + e]);
+            if (a < INFINITY) top = fmaxf(top, a);
+        }
+    top = __uint_as_float(__reduce_max_sync(0xFFFFFFFFu, __float_as_uint(top)));
+    if ((tid & 31) == 0) s_max[tid >> 5] = top;
+    __syncthreads();
+    const int ex = (int)(__float_as_uint(x) >> 23);  // (biased; 0: zero or denormal)
+    if (ex > 0) atomicAdd(&s_hist[ex], 1);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) top = fmaxf(top, s_max[i]);
+    __syncthreads();
+    if (tid < 32) {
+        int own = 0;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) own += s_hist[8 * tid + i];
+        int upto = own;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const int o = __shfl_up_sync(0xFFFFFFFFu, upto, d);
+            if (tid >= d) upto += o;
+        }
+        const int half = (__shfl_sync(0xFFFFFFFFu, upto, 31) + 1) / 2;  // the median is where the count reaches this
+        if (half > 0 && upto >= half && upto - own < half) {
+            int c = upto - own;
+            for (int i = 0; i < 8; ++i) {
+                c += s_hist[8 * tid + i];
+                if (c >= half) {
+                    s_mid = 8 * tid + i;
+                    break;
+                }
+            }
+        }
+    }
+    __syncthreads();
+    int s = 127 + 8 - s_mid;
+    s = s < -120 ? -120 : s > 120 ? 120 : s;
+    int k = top > 0.f ? 13 + 127 - (int)(__float_as_uint(top) >> 23) : 0;
+    k = k > 126 ? 126 : k;
+    if (tid == 0) {
+        const int t = -(k + s), t1 = t / 2;
+        unscale[r] = make_float2(tables_exp2(t1), tables_exp2(t - t1));
+        if (r == 0) *scale = tables_exp2(s);
+    }
+    const float f = tables_exp2(k);
+    const size_t part = (size_t)m_pad * E_pad;
+    for (int e = tid * 2; e < E_pad; e += 512) {
+        const float x0 = (r < m && e < E) ? W[(size_t)r * E + e] * f : 0.f;
+        const float x1 = (r < m && e + 1 < E) ? W[(size_t)r * E + e + 1] * f : 0.f;
+        const __half2 a = __floats2half2_rn(x0, x1);
+        const __half2 b = __floats2half2_rn((x0 - __low2float(a)) * kTmLow, (x1 - __high2float(a)) * kTmLow);
+        __half* dst = w + (size_t)r * E_pad + e;
+        *(__half2*)dst = a;
+        *(__half2*)(dst + part) = b;
+    }
+}
+
+__device__ __forceinline__ uint32_t cvt_f16x2(float lo, float hi) {
+    uint32_t r;
+    asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
+    return r;
+}
+// two fp32 numbers, scaled -> their two fp16 parts, packed
+__device__ __forceinline__ void split2(float x0, float x1, float scale, uint32_t& a, uint32_t& b) {
+    const float2 x = __fmul2_rn(make_float2(x0, x1), make_float2(scale, scale));
+    a = cvt_f16x2(x.x, x.y);
+    const float2 y = __half22float2(*(const __half2*)&a);
+    const float2 z = __fmul2_rn(make_float2(x.x - y.x, x.y - y.y), make_float2(kTmLow, kTmLow));
+    b = cvt_f16x2(z.x, z.y);
+}
+// Is a row whose largest magnitude is m held well enough by the two parts, once scaled?  They are off by 2^-36 at most where fp16 has no
+// more bits below them: 2^-26 of the largest entry if that is 2^-10 or more.  Or the row is zero.
+__device__ __forceinline__ bool tables_row_ok(float m, float scale) {
+    return m == 0.f || (m * scale >= 0.0009765625f && m * scale <= 65504.f);
 }
 __device__ __forceinline__ void st_shared_v4(uint32_t at, const uint32_t (&v)[4]) {
     asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(at), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]) : "memory");
@@ -193,9 +312,9 @@ __device__ __forceinline__ float4 ld_shared_f4(uint32_t at) {
     return v;
 }
 
-// fp32 embeddings: an entry whose bf16 parts are not all finite -- an infinity, a value that rounds past the largest bf16 --
-// turns every result it has a part in into a NaN or an infinity.  Results that are not finite are worked out again as one
-// chain of fp32 multiply-adds, which gives what fp32 arithmetic gives; such entries are rare, so the time does not matter.
+// fp32 embeddings: results that are worked out again as one chain of fp32 multiply-adds, which gives what fp32 arithmetic gives:
+// rows whose entries fp16 parts do not hold well enough (over 2^7 times larger than most rows, or 2^18 times smaller), and whatever is
+// not finite (infinities).  They are rare, so the time does not matter.
 __device__ __forceinline__ bool tables_finite(float x) { return fabsf(x) <= 3.402823466e38f; }
 __device__ __noinline__ float tables_fp32(const TablesParams& p, int v, int c) {
     const float* e = (const float*)p.emb + (size_t)v * p.E;
@@ -210,9 +329,9 @@ template <bool F32>
 __global__ void __cluster_dims__(F32 ? 1 : 2, 1, 1) __launch_bounds__(TablesCfg<F32>::THREADS, 1)
     tables_mma_kernel(const __grid_constant__ TablesParams p) {
     using C = TablesCfg<F32>;
-    constexpr uint32_t NA = C::A_STAGES, NW = C::W_STAGES, NR = C::RAW_STAGES;
+    constexpr uint32_t NS = C::STAGES, NR = C::RAW_STAGES;
     extern __shared__ unsigned char smem_raw[];
-    __shared__ __align__(8) uint64_t bars[2 * (NA + NW + NR) + 4];
+    __shared__ __align__(8) uint64_t bars[2 * (NS + NR) + 4];
     __shared__ uint32_t s_tmem;
     __shared__ volatile int s_abort;
     __shared__ bool s_mend;
@@ -226,24 +345,20 @@ __global__ void __cluster_dims__(F32 ? 1 : 2, 1, 1) __launch_bounds__(TablesCfg<
             mbar_wait_bounded(bar, parity, &s_abort);
     };
     const uint32_t a_ring = (smem_u32(smem_raw) + 1023u) & ~1023u;
-    const uint32_t w_ring = a_ring + NA * C::A_BYTES, raw_ring = w_ring + NW * C::W_BYTES;
-    // afull / wfull: a block's rows, its W are there (a pair: in both CTAs; the even CTA's barriers), aempty / wempty: the
-    // instructions that read them are done, rfull / rempty: fp32 rows as loaded
-    const uint32_t afull0 = smem_u32(bars), aempty0 = afull0 + 8 * NA, wfull0 = aempty0 + 8 * NA, wempty0 = wfull0 + 8 * NW;
-    const uint32_t rfull0 = wempty0 + 8 * NW, rempty0 = rfull0 + 8 * NR;
+    const uint32_t w_ring = a_ring + NS * C::A_BYTES, raw_ring = w_ring + NS * C::W_BYTES;
+    // full: a block's rows and its W are there (a pair: in both CTAs; the even CTA's barriers), empty: the instructions that read
+    // them are done, rfull / rempty: fp32 rows as loaded.  (One barrier for rows and W: the thread that issues the instructions is
+    // the bottleneck of short blocks, every wait and every commit costs it a hundred cycles.)
+    const uint32_t full0 = smem_u32(bars), empty0 = full0 + 8 * NS, rfull0 = empty0 + 8 * NS, rempty0 = rfull0 + 8 * NR;
     const uint32_t accfull0 = rempty0 + 8 * NR, accempty0 = accfull0 + 16;
     if (tid == 0) {
-        for (uint32_t s = 0; s < NA; ++s) {
-            mbar_init(afull0 + 8 * s, F32 ? kTmConvWarps : 1);
-            mbar_init(aempty0 + 8 * s, 1);
-        }
-        for (uint32_t s = 0; s < NW; ++s) {
-            mbar_init(wfull0 + 8 * s, 1);
-            mbar_init(wempty0 + 8 * s, 1);
+        for (uint32_t s = 0; s < NS; ++s) {
+            mbar_init(full0 + 8 * s, F32 ? kTmConvWarps / 2 + 1 : 1);
+            mbar_init(empty0 + 8 * s, 1);
         }
         for (uint32_t s = 0; s < NR; ++s) {
             mbar_init(rfull0 + 8 * s, 1);
-            mbar_init(rempty0 + 8 * s, kTmConvWarps);
+            mbar_init(rempty0 + 8 * s, kTmConvWarps / 2);
         }
         for (int s = 0; s < 2; ++s) {
             mbar_init(accfull0 + 8 * s, 1);
@@ -293,7 +408,10 @@ __global__ void __cluster_dims__(F32 ? 1 : 2, 1, 1) __launch_bounds__(TablesCfg<
                             tmem_ld_32x16(t0 + n * lo + 16u * q, d);
                             tmem_wait_ld();
 #pragma unroll
-                            for (int c = 0; c < 16; ++c) acc[h][16 * q + c] += __uint_as_float(d[c]);
+                            for (int c = 0; c < 16; ++c) {
+                                const float x = __uint_as_float(d[c]);
+                                acc[h][16 * q + c] = F32 && lo ? fmaf(x, 1.0f / kTmLow, acc[h][16 * q + c]) : acc[h][16 * q + c] + x;
+                            }
                         }
                     }
                     tc_fence_before();
@@ -322,6 +440,13 @@ __global__ void __cluster_dims__(F32 ? 1 : 2, 1, 1) __launch_bounds__(TablesCfg<
                     for (int c = 0; c < 64; c += 8) {
                         if (c >= cols) break;
                         const bool both = c + 4 < cols;
+                        if (F32) {
+#pragma unroll
+                            for (int k = 0; k < 8; ++k) {
+                                const float2 f = __ldg(p.unscale + mb * 128 + half * 64 + c + k);
+                                acc[h][c + k] = acc[h][c + k] * f.x * f.y;
+                            }
+                        }
                         if (bias) {
 #pragma unroll
                             for (int k = 0; k < 8; ++k)
@@ -347,108 +472,110 @@ __global__ void __cluster_dims__(F32 ? 1 : 2, 1, 1) __launch_bounds__(TablesCfg<
         if (F32) {  // (nothing waits for these warps any more)
             if (check.x + check.y != 0.f) s_mend = true;
             __syncwarp();
-            named_bar_sync(1, kTmEpiWarps * 32);  // (the tiles are written for every thread of these warps)
+            named_bar_sync(1, (kTmEpiWarps + kTmConvWarps) * 32);  // (the tiles are written, their rows looked at)
             if (s_mend && !s_abort) {
                 for (int i = 0; tables_item(p, pair, i, it); ++i) {
                     if (it.q0 != it.q1) continue;  // (pieces: the kernel that adds them up)
                     const int rt = it.tile / p.n_mb, c0 = (it.tile - rt * p.n_mb) * 128;
-                    for (int v = rt * C::ROWS + warp; v < p.V && v < (rt + 1) * C::ROWS; v += kTmEpiWarps)
+                    for (int v = rt * C::ROWS + warp; v < p.V && v < (rt + 1) * C::ROWS; v += kTmEpiWarps) {
+                        const bool bad = p.bad_row[v] != 0;
                         for (int c = c0 + lane; c < p.m && c < c0 + 128; c += 32) {
                             float* o = p.out + (size_t)v * p.m + c;
-                            if (!tables_finite(*o)) *o = tables_fp32(p, v, c);
+                            if (bad || !tables_finite(*o)) *o = tables_fp32(p, v, c);
                         }
+                    }
                 }
             }
         }
     } else if (warp == 8) {
         // ------------------------------ TMA loads: W, bf16 embeddings ----------------------------
         if (lane == 0) {
-            const uint32_t afull_even = mapa_u32(afull0, 0), wfull_even = mapa_u32(wfull0, 0);
-            TablesRing<NA> a(1);
-            TablesRing<NW> w(1);
+            const uint32_t full_even = mapa_u32(full0, 0);
+            TablesRing<NS> w(1);
             for (int i = 0; tables_item(p, pair, i, it); ++i) {
                 const int rt = it.tile / p.n_mb, mb = it.tile - rt * p.n_mb;
                 const int n = tables_n<F32>(p, mb);
                 const int w12 = (int)rank * p.m_pad + mb * 128, w3 = 2 * p.m_pad + mb * 128 + (int)rank * (n >> 1);
                 for (int kb = it.kb0; kb < it.kb1; ++kb) {
                     const int x = kb * C::BLK;
-                    if (!F32) {
-                        if (a.t >= NA) wait(aempty0 + 8 * a.st, a.ph);
-                        if (s_abort) break;  // (no copy is started any more)
-                        if (rank == 0) mbar_arrive_expect_tx(afull0 + 8 * a.st, 2u * C::A_BYTES);
+                    if (w.t >= NS) wait(empty0 + 8 * w.st, w.ph);
+                    if (s_abort) break;  // (no copy is started any more)
+                    const uint32_t da = a_ring + w.st * C::A_BYTES, dw = w_ring + w.st * C::W_BYTES;
+                    if (C::PAIR) {
+                        const uint32_t fb = full_even + 8 * w.st;
+                        if (rank == 0) mbar_arrive_expect_tx(full0 + 8 * w.st, 2u * (C::A_BYTES + C::W_BYTES));
 #pragma unroll
                         for (int h = 0; h < C::MT; ++h)
-                            tma_load_2d_pair(a_ring + a.st * C::A_BYTES + h * C::PART, &p.map_e, x,
-                                             rt * C::ROWS + h * 256 + (int)rank * 128, afull_even + 8 * a.st);
-                        a.next();
-                    }
-                    if (w.t >= NW) wait(wempty0 + 8 * w.st, w.ph);
-                    if (s_abort) break;
-                    const uint32_t dw = w_ring + w.st * C::W_BYTES, fb = wfull_even + 8 * w.st;
-                    if (C::PAIR) {
-                        if (rank == 0) mbar_arrive_expect_tx(wfull0 + 8 * w.st, 2u * C::W_BYTES);
+                            tma_load_2d_pair(da + h * C::PART, &p.map_e, x, rt * C::ROWS + h * 256 + (int)rank * 128, fb);
                         tma_load_2d_pair(dw, &p.map_w, x, w12, fb);
                         tma_load_2d_pair(dw + C::W_BYTES / 3, &p.map_w, x, w12 + 64, fb);
                         tma_load_2d_pair(dw + 2 * (C::W_BYTES / 3), &p.map_w, x, w3, fb);
                     } else {
                         const uint32_t part = (uint32_t)n * C::BLK * 2;
-                        mbar_arrive_expect_tx(wfull0 + 8 * w.st, 3u * part);
+                        mbar_arrive_expect_tx(full0 + 8 * w.st, 2u * part);
 #pragma unroll
-                        for (int j = 0; j < 3; ++j)
-                            tma_load_2d(dw + j * part, &p.map_w, x, j * p.m_pad + mb * 128, wfull0 + 8 * w.st);
+                        for (int j = 0; j < 2; ++j)
+                            tma_load_2d(dw + j * part, &p.map_w, x, j * p.m_pad + mb * 128, full0 + 8 * w.st);
                     }
                     w.next();
                 }
             }
             // the last arrivals from the other CTA have come before this CTA retires; after an abort: no copy of the pair
             // is in flight any more
-            if (!F32) a.drain(aempty0, rank == 0 ? afull0 : 0u, &s_abort);
-            w.drain(wempty0, rank == 0 ? wfull0 : 0u, &s_abort);
+            w.drain(empty0, rank == 0 ? full0 : 0u, &s_abort);
         }
     } else if (warp == 9) {
         // ------------------------------ matrix instructions --------------------------------------
         if (rank == 0 && lane == 0) {
-            TablesRing<NA> a(0);
-            TablesRing<NW> w(0);
+            TablesRing<NS> w(0);
             uint32_t cc = 0;
             for (int i = 0; tables_item(p, pair, i, it); ++i) {
                 const int mb = it.tile % p.n_mb;
                 const int n = tables_n<F32>(p, mb);
                 constexpr int M = C::PAIR ? 256 : 128;
-                const uint32_t idesc2 = umma_idesc_bf16(M, 2 * n), idesc1 = umma_idesc_bf16(M, n);
-                const uint32_t o_w3 = C::PAIR ? 2 * (C::W_BYTES / 3) : (uint32_t)n * (2 * C::BLK * 2);
-                for (int kb = it.kb0; kb < it.kb1; ++kb) {
+                const uint32_t idesc2 = umma_idesc(M, 2 * n, !F32), idesc1 = umma_idesc(M, n, !F32);
+                constexpr uint32_t o_w3 = 2 * (C::W_BYTES / 3);  // (bf16)
+                // A pair takes two blocks at a time.  An instruction whose accumulator columns the one just ahead of it wrote waits
+                // for those, so with two row blocks their instructions alternate, except in the first and the last two blocks of a
+                // chunk, where the first row block goes ahead: its accumulators are emptied (or were) while the second's are filled.
+                constexpr int G = C::MT;
+                for (int kb = it.kb0; kb < it.kb1; kb += G) {
+                    const int g = kb + G <= it.kb1 ? G : it.kb1 - kb;
                     const bool first = (kb - it.kb0) % C::CHUNK == 0;
-                    const bool last = kb + 1 == it.kb1 || (kb + 1 - it.kb0) % C::CHUNK == 0;
-                    wait(wfull0 + 8 * w.st, w.ph);
-                    wait(afull0 + 8 * a.st, a.ph);
+                    const bool last = kb + g == it.kb1 || (kb + g - it.kb0) % C::CHUNK == 0;
+                    uint32_t a0[G], b0[G], done[G];
+#pragma unroll
+                    for (int k = 0; k < G; ++k) {
+                        if (k >= g) break;
+                        wait(full0 + 8 * w.st, w.ph);
+                        a0[k] = a_ring + w.st * C::A_BYTES;
+                        b0[k] = w_ring + w.st * C::W_BYTES;
+                        done[k] = empty0 + 8 * w.st;
+                        w.next();
+                    }
                     tc_fence_after();
-                    const uint32_t a0 = a_ring + a.st * C::A_BYTES, b0 = w_ring + w.st * C::W_BYTES;
-                    // An instruction whose accumulator columns the one just ahead of it wrote waits for those; with two row
-                    // blocks their instructions alternate, except in the first and the last block of a chunk, where the
-                    // first row block goes ahead (its accumulators are emptied, or were, while the second's are filled).
-                    auto mma = [&](int h, int ks, bool w3) {
+                    auto mma = [&](int k, int h, int ks, bool small) {
                         const uint32_t d = tmem + (C::MT == 1 ? (cc & 1u) : (uint32_t)h) * 256u;
-                        const uint64_t a1 = C::desc(a0 + h * C::PART + 32 * ks);
-                        if (w3) {
-                            umma<C::PAIR>(d + (uint32_t)n, a1, C::desc(b0 + o_w3 + 32 * ks), idesc1, true);
-                        } else {
-                            const uint64_t w12 = C::desc(b0 + 32 * ks);
-                            umma<C::PAIR>(d, a1, w12, idesc2, !first || ks > 0);
-                            if (F32) {
-                                umma<C::PAIR>(d, C::desc(a0 + C::PART + 32 * ks), w12, idesc2, true);
-                                umma<C::PAIR>(d, C::desc(a0 + 2 * C::PART + 32 * ks), w12, idesc2, true);
-                            }
-                        }
+                        const uint64_t a1 = C::desc(a0[k] + h * C::PART + 32 * ks), w12 = C::desc(b0[k] + 32 * ks);
+                        if (!small)
+                            umma<C::PAIR>(d, a1, w12, idesc2, !first || k > 0 || ks > 0);
+                        else if (F32)  // (the second part of the embeddings times W1)
+                            umma<C::PAIR>(d + (uint32_t)n, C::desc(a0[k] + C::PART + 32 * ks), w12, idesc1, true);
+                        else
+                            umma<C::PAIR>(d + (uint32_t)n, a1, C::desc(b0[k] + o_w3 + 32 * ks), idesc1, true);
                     };
                     if (C::MT == 2 && !first && !last) {
                         if (!s_abort) {
 #pragma unroll
-                            for (int ks = 0; ks < C::BLK / 16; ++ks) {
-                                mma(0, ks, false);
-                                mma(1, ks, false);
-                                mma(0, ks, true);
-                                mma(1, ks, true);
+                            for (int k = 0; k < G; ++k) {
+                                if (k >= g) break;
+#pragma unroll
+                                for (int ks = 0; ks < C::BLK / 16; ++ks) {
+                                    mma(k, 0, ks, false);
+                                    mma(k, 1, ks, false);
+                                    mma(k, 0, ks, true);
+                                    mma(k, 1, ks, true);
+                                }
                             }
                         }
                     } else {
@@ -462,19 +589,24 @@ __global__ void __cluster_dims__(F32 ? 1 : 2, 1, 1) __launch_bounds__(TablesCfg<
                             }
                             if (!s_abort) {
 #pragma unroll
-                                for (int ks = 0; ks < C::BLK / 16; ++ks) {
-                                    mma(h, ks, false);
-                                    mma(h, ks, true);
+                                for (int k = 0; k < G; ++k) {
+                                    if (k >= g) break;
+#pragma unroll
+                                    for (int ks = 0; ks < C::BLK / 16; ++ks) {
+                                        mma(k, h, ks, false);
+                                        mma(k, h, ks, true);
+                                    }
                                 }
                             }
                             if (last) umma_commit<C::PAIR>(accfull0 + 8 * slot);
                         }
                     }
-                    umma_commit<C::PAIR>(aempty0 + 8 * a.st);
-                    umma_commit<C::PAIR>(wempty0 + 8 * w.st);
+#pragma unroll
+                    for (int k = 0; k < G; ++k) {
+                        if (k >= g) break;
+                        umma_commit<C::PAIR>(done[k]);
+                    }
                     if (last) ++cc;
-                    a.next();
-                    w.next();
                 }
             }
         }
@@ -495,48 +627,69 @@ __global__ void __cluster_dims__(F32 ? 1 : 2, 1, 1) __launch_bounds__(TablesCfg<
             r.drain(rempty0, rfull0, &s_abort);
         }
     } else if (F32) {
-        // ------------------------------ fp32 embeddings -> bf16 parts ----------------------------
-        const int ct = tid - (kTmEpiWarps + 3) * 32;
-        const int c8 = ct & 3, r0 = ct >> 2;  // columns 8 c8 .. 8 c8 + 7 of rows r0 and r0 + 64
-        TablesRing<NA> a(1);
+        // ------------------------------ fp32 embeddings -> fp16 parts ----------------------------
+        // four warps take the even blocks, four the odd ones: a block is a chain of waits and round trips
+        const int ct = (tid - (kTmEpiWarps + 3) * 32) & 127, half = (tid - (kTmEpiWarps + 3) * 32) >> 7;
+        const int c8 = ct & 3, r0 = ct >> 2;  // columns 8 c8 .. 8 c8 + 7 of rows r0, r0 + 32, r0 + 64 and r0 + 96
+        const float scale = *p.scale;
+        TablesRing<NS> a(1);
         TablesRing<NR> r(0);
         for (int i = 0; tables_item(p, pair, i, it); ++i) {
-            for (int kb = it.kb0; kb < it.kb1; ++kb) {
+            float most[4] = {0.f, 0.f, 0.f, 0.f};  // the largest magnitudes of the rows
+            for (int kb = it.kb0; kb < it.kb1; ++kb, a.next(), r.next()) {
+                if ((int)(a.t & 1u) != half) continue;
                 wait(rfull0 + 8 * r.st, r.ph);
                 const uint32_t src = raw_ring + r.st * C::RAW;
-                float4 x[2][2];
+                float4 x[4][2];
 #pragma unroll
-                for (int q = 0; q < 2; ++q) {
-                    const int row = r0 + 64 * q;
+                for (int q = 0; q < 4; ++q) {
+                    const int row = r0 + 32 * q;
 #pragma unroll
                     for (int h = 0; h < 2; ++h)  // (128-byte rows in the 128-byte swizzle)
                         x[q][h] = ld_shared_f4(src + (uint32_t)row * 128u + (uint32_t)(((2 * c8 + h) ^ (row & 7)) * 16));
                 }
                 __syncwarp();
                 if (lane == 0) mbar_arrive(rempty0 + 8 * r.st);
-                r.next();
-                if (a.t >= NA) wait(aempty0 + 8 * a.st, a.ph);
+                if (a.t >= NS) wait(empty0 + 8 * a.st, a.ph);
                 const uint32_t dst = a_ring + a.st * C::A_BYTES;
 #pragma unroll
-                for (int q = 0; q < 2; ++q) {
-                    const int row = r0 + 64 * q;  // (64-byte rows in the 64-byte swizzle)
+                for (int q = 0; q < 4; ++q) {
+                    const int row = r0 + 32 * q;  // (64-byte rows in the 64-byte swizzle)
                     const uint32_t at = dst + (uint32_t)row * 64u + (uint32_t)((c8 ^ ((row >> 1) & 3)) * 16);
-                    uint32_t b1[4], b2[4], b3[4];
-                    split3(x[q][0].x, x[q][0].y, b1[0], b2[0], b3[0]);
-                    split3(x[q][0].z, x[q][0].w, b1[1], b2[1], b3[1]);
-                    split3(x[q][1].x, x[q][1].y, b1[2], b2[2], b3[2]);
-                    split3(x[q][1].z, x[q][1].w, b1[3], b2[3], b3[3]);
+                    uint32_t b1[4], b2[4];
+                    split2(x[q][0].x, x[q][0].y, scale, b1[0], b2[0]);
+                    split2(x[q][0].z, x[q][0].w, scale, b1[1], b2[1]);
+                    split2(x[q][1].x, x[q][1].y, scale, b1[2], b2[2]);
+                    split2(x[q][1].z, x[q][1].w, scale, b1[3], b2[3]);
                     st_shared_v4(at, b1);
                     st_shared_v4(at + C::PART, b2);
-                    st_shared_v4(at + 2 * C::PART, b3);
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        most[q] = fmaxf(most[q], fmaxf(fabsf(x[q][h].x), fabsf(x[q][h].y)));
+                        most[q] = fmaxf(most[q], fmaxf(fabsf(x[q][h].z), fabsf(x[q][h].w)));
+                    }
                 }
                 fence_proxy_async();
                 __syncwarp();
-                if (lane == 0) mbar_arrive(afull0 + 8 * a.st);
-                a.next();
+                if (lane == 0) mbar_arrive(full0 + 8 * a.st);
+            }
+            // rows that fp16 does not hold well enough (in this thread's blocks)
+            const int rt = it.tile / p.n_mb;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                float mx = fmaxf(most[q], __shfl_xor_sync(0xFFFFFFFFu, most[q], 1));
+                mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, 2));
+                const int v = rt * C::ROWS + r0 + 32 * q;
+                if (c8 == 0 && v < p.V && !tables_row_ok(mx, scale)) {
+                    p.bad_row[v] = 1;
+                    if (it.q0 == it.q1) s_mend = true;
+                }
             }
         }
-        a.drain(aempty0, 0u, &s_abort);
+        a.drain(empty0, 0u, &s_abort);
+        __threadfence_block();  // (the flags, for the warps that write the tiles)
+        __syncwarp();
+        asm volatile("bar.arrive 1, %0;" ::"n"((kTmEpiWarps + kTmConvWarps) * 32) : "memory");
     }
     __syncwarp();
     tc_fence_before();
@@ -555,6 +708,7 @@ __global__ void __launch_bounds__(256) tables_pieces_kernel(const __grid_constan
     const int q0 = tables_owner(p, tile * p.n_kb), q1 = tables_owner(p, (tile + 1) * p.n_kb - 1);
     const int v = (int)blockIdx.x * 8 + (threadIdx.x >> 5), c = (threadIdx.x & 31) * 4;
     if (q0 == q1 || rt * C::ROWS + v >= p.V || mb * 128 + c >= p.m) return;  // (q0 == q1: written whole)
+    const bool bad = F32 && p.bad_row[rt * C::ROWS + v] != 0;
     float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll 4
     for (int q = q0; q <= q1; ++q) {
@@ -567,11 +721,11 @@ __global__ void __launch_bounds__(256) tables_pieces_kernel(const __grid_constan
         s.x += b[0], s.y += b[1], s.z += b[2], s.w += b[3];
     }
     const int row = rt * C::ROWS + v, col = mb * 128 + c;
-    if (F32 && fmaf(0.f, s.x, fmaf(0.f, s.y, fmaf(0.f, s.z, 0.f * s.w))) != 0.f) {
-        if (!tables_finite(s.x)) s.x = tables_fp32(p, row, col);
-        if (!tables_finite(s.y)) s.y = tables_fp32(p, row, col + 1);
-        if (!tables_finite(s.z)) s.z = tables_fp32(p, row, col + 2);
-        if (!tables_finite(s.w)) s.w = tables_fp32(p, row, col + 3);
+    if (F32 && (bad || fmaf(0.f, s.x, fmaf(0.f, s.y, fmaf(0.f, s.z, 0.f * s.w))) != 0.f)) {
+        if (bad || !tables_finite(s.x)) s.x = tables_fp32(p, row, col);
+        if (bad || !tables_finite(s.y)) s.y = tables_fp32(p, row, col + 1);
+        if (bad || !tables_finite(s.z)) s.z = tables_fp32(p, row, col + 2);
+        if (bad || !tables_finite(s.w)) s.w = tables_fp32(p, row, col + 3);
     }
     *(float4*)(p.out + (size_t)row * p.m + col) = s;
 }
@@ -593,11 +747,11 @@ EncodeTiledFn encode_tiled() {
     return fn;
 }
 // [rows, cols], boxes of box_rows rows of box_bytes, in the swizzle of that width, zeros outside
-bool encode_map(CUtensorMap* map, const void* base, bool f32, uint64_t rows, uint64_t cols, uint32_t box_rows, uint32_t box_bytes) {
-    const uint32_t esz = f32 ? 4 : 2;
+bool encode_map(CUtensorMap* map, const void* base, CUtensorMapDataType type, uint64_t rows, uint64_t cols, uint32_t box_rows, uint32_t box_bytes) {
+    const uint32_t esz = type == CU_TENSOR_MAP_DATA_TYPE_FLOAT32 ? 4 : 2;
     const cuuint64_t dims[2] = {cols, rows}, strides[1] = {cols * esz};
     const cuuint32_t box[2] = {box_bytes / esz, box_rows}, step[2] = {1, 1};
-    return encode_tiled()(map, f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2,
+    return encode_tiled()(map, type, 2,
                           const_cast<void*>(base), dims, strides, box, step, CU_TENSOR_MAP_INTERLEAVE_NONE,
                           box_bytes == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
                           CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
@@ -605,16 +759,20 @@ bool encode_map(CUtensorMap* map, const void* base, bool f32, uint64_t rows, uin
 
 struct TablesSizes {
     int n_mb, m_pad, E_pad, pairs;
-    size_t o_w, total;
+    size_t o_w, o_unscale, o_scale, o_bad, n_bad, total;  // (fp32 only: from o_unscale on)
 };
-TablesSizes tables_sizes(int num_sms, int E, int m, bool f32) {
+TablesSizes tables_sizes(int num_sms, int V, int E, int m, bool f32) {
     TablesSizes s;
     s.n_mb = (m + 127) / 128;
     s.m_pad = 128 * s.n_mb;
     s.E_pad = (E + 63) / 64 * 64;
     s.pairs = f32 ? num_sms : num_sms / 2;
     s.o_w = (size_t)s.pairs * 2 * (f32 ? TablesCfg<true>::ROWS : TablesCfg<false>::ROWS) * 128 * sizeof(float);
-    s.total = s.o_w + (size_t)3 * s.m_pad * s.E_pad * 2;
+    s.o_unscale = s.o_w + (size_t)(f32 ? 2 : 3) * s.m_pad * s.E_pad * 2;
+    s.o_scale = s.o_unscale + (f32 ? (size_t)s.m_pad * sizeof(float2) : 0);
+    s.o_bad = s.o_scale + (f32 ? 256 : 0);
+    s.n_bad = f32 ? (size_t)(V + TablesCfg<true>::ROWS - 1) / TablesCfg<true>::ROWS * TablesCfg<true>::ROWS : 0;
+    s.total = s.o_bad + s.n_bad;
     return s;
 }
 template <bool F32>
@@ -636,8 +794,8 @@ cudaError_t tables_run(const TablesParams& p, cudaStream_t st, int* launches) {
 bool tables_mma_fits(const void* d_emb, graft_dtype dt, int E, const void* d_out) {
     return E % (dt == GRAFT_BF16 ? 8 : 4) == 0 && (((uintptr_t)d_emb | (uintptr_t)d_out) & 15) == 0 && encode_tiled() != nullptr;
 }
-size_t tables_mma_scratch_bytes(int num_sms, int E, int m, graft_dtype dt) {
-    return tables_sizes(num_sms, E, m, dt == GRAFT_F32).total;
+size_t tables_mma_scratch_bytes(int num_sms, int V, int E, int m, graft_dtype dt) {
+    return tables_sizes(num_sms, V, E, m, dt == GRAFT_F32).total;
 }
 
 // out [V, m] = emb [V, E] . W^T + bias.  scratch: tables_mma_scratch_bytes, 256-byte aligned.
@@ -645,19 +803,23 @@ cudaError_t tables_mma_launch(graft_ctx* ctx, const void* d_emb, graft_dtype dt,
                               float* d_out, void* scratch, cudaStream_t st) {
     const int V = ctx->cfg.V, m = ctx->cfg.m;
     const bool f32 = dt == GRAFT_F32;
-    const TablesSizes s = tables_sizes(ctx->num_sms, E, m, f32);
-    __nv_bfloat16* w = (__nv_bfloat16*)((char*)scratch + s.o_w);
+    const TablesSizes s = tables_sizes(ctx->num_sms, V, E, m, f32);
+    void* w = (char*)scratch + s.o_w;
     TablesParams p;
     const int blk = f32 ? TablesCfg<true>::BLK : TablesCfg<false>::BLK;
     p.box_n = s.n_mb > 1 ? 128 : (m + 31) / 32 * 32;
-    if (!encode_map(&p.map_w, w, false, (uint64_t)3 * s.m_pad, s.E_pad, f32 ? p.box_n : 64, 2 * blk) ||
-        !encode_map(&p.map_e, d_emb, f32, V, E, 128, 128))
+    if (!encode_map(&p.map_w, w, f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16,
+                    (uint64_t)(f32 ? 2 : 3) * s.m_pad, s.E_pad, f32 ? p.box_n : 64, 2 * blk) ||
+        !encode_map(&p.map_e, d_emb, f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, V, E, 128, 128))
         return cudaErrorUnknown;
     p.emb = d_emb;
     p.W = d_W;
     p.bias = d_b;
     p.out = d_out;
     p.pieces = (float*)scratch;
+    p.unscale = (const float2*)((char*)scratch + s.o_unscale);
+    p.scale = (const float*)((char*)scratch + s.o_scale);
+    p.bad_row = (uint8_t*)scratch + s.o_bad;
     p.errflag = ctx->w_errflag;
     p.V = V;
     p.E = E;
@@ -687,7 +849,12 @@ cudaError_t tables_mma_launch(graft_ctx* ctx, const void* d_emb, graft_dtype dt,
     }
     p.share_pairs = (int)(sp < p.left ? p.left : sp);
     p.wide = m % 8 == 0 && ((uintptr_t)d_out & 31) == 0;
-    weight_split_kernel<<<dim3((s.E_pad + 511) / 512, s.m_pad), 256, 0, st>>>(d_W, m, E, s.m_pad, s.E_pad, w);
+    if (f32)
+        weight_split16_kernel<<<s.m_pad, 256, 0, st>>>(d_W, (const float*)d_emb, V, m, E, s.m_pad, s.E_pad, (__half*)w,
+                                                       (float2*)((char*)scratch + s.o_unscale), (float*)((char*)scratch + s.o_scale),
+                                                       (uint32_t*)p.bad_row, (int)(s.n_bad / 4));
+    else
+        weight_split_kernel<<<dim3((s.E_pad + 511) / 512, s.m_pad), 256, 0, st>>>(d_W, m, E, s.m_pad, s.E_pad, (__nv_bfloat16*)w);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     int launches = 1;

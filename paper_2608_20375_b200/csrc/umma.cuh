@@ -98,7 +98,7 @@ __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.
 
 // ---- matrix instruction ----------------------------------------------------------------------------------------
 // Shared-memory operand: K-major rows of 128 bytes in the 128-byte swizzle, groups of eight rows 1024 bytes apart; tiles
-// start on 1024-byte boundaries and a K step of 16 bf16 advances the start address by 32 bytes.
+// start on 1024-byte boundaries and a K step of 16 numbers advances the start address by 32 bytes.
 __device__ __forceinline__ uint64_t umma_desc_sw128(uint32_t smem_addr) {
     return (uint64_t)((smem_addr & 0x3FFFFu) >> 4) | ((uint64_t)1 << 16) | ((uint64_t)(1024 >> 4) << 32) | ((uint64_t)1 << 46) |
            ((uint64_t)2 << 61);
@@ -108,9 +108,9 @@ __device__ __forceinline__ uint64_t umma_desc_sw64(uint32_t smem_addr) {
     return (uint64_t)((smem_addr & 0x3FFFFu) >> 4) | ((uint64_t)1 << 16) | ((uint64_t)(512 >> 4) << 32) | ((uint64_t)1 << 46) |
            ((uint64_t)4 << 61);
 }
-// bf16 x bf16 -> fp32, both operands K-major
-__host__ __device__ constexpr uint32_t umma_idesc_bf16(int M, int N) {
-    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
+// bf16 x bf16 or fp16 x fp16 -> fp32, both operands K-major
+__host__ __device__ constexpr uint32_t umma_idesc(int M, int N, bool bf16) {
+    return (1u << 4) | (bf16 ? (1u << 7) | (1u << 10) : 0u) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 // One thread (of the pair's even CTA): D (+)= A B.  PAIR: D in both CTAs' TMEM, A and B from both CTAs' shared memory.
 template <bool PAIR>

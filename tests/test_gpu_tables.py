@@ -150,3 +150,24 @@ def test_rows_off_the_16_byte_grid(dtype, off):
     torch.cuda.synchronize()
     assert (out - _exact(emb, W, b)).abs().max() < 1e-5
     assert (o_pad[:j] == 7.0).all() and (o_pad[j + V * m:] == 7.0).all()
+
+
+@pytest.mark.parametrize("V,E,m", [(300, 64, 128), (19300, 1092, 40), (40003, 132, 256)])  # whole tiles, pieces, both
+def test_fp32_rows_of_other_sizes(V, E, m):
+    """Rows far larger or smaller than the others, rows of zeros, rows with one large entry, and columns of W of every size: an error
+    of 2e-5 (the chain of fp32 multiply-adds: 1.2e-5) of a result's size, row by row."""
+    emb, W, _ = _inputs(V, E, m, "f32", 11)
+    size = torch.ones(V, device="cuda")
+    for i, e in enumerate((-100, -40, -25, -19, -17, -12, -9, 5, 8, 9, 16, 40, 60)):
+        size[(7919 * i) % V], size[V - 1 - i] = 2.0 ** e, 2.0 ** e
+    emb *= size[:, None]
+    emb[V // 3] = 0.0
+    emb[V // 4, E // 2], emb[V // 5, 0] = 200.0, 3e4  # (beside entries of N(0, 1))
+    size[V // 4], size[V // 5] = 4.0, 3e4 * E ** -0.5 + 1.0
+    wide = 2.0 ** (torch.arange(m, device="cuda") % 50 - 30)
+    W = W * wide[:, None]
+    got = _call(_graft(V, m), emb, W, None, m).double()
+    # (sums in fp32's denormals, the smallest rows and columns: half a spacing of 1.4e-45 an addition)
+    bound = 2e-5 * size[:, None].double() * wide[None].double() + 0.7e-45 * E
+    over = (got - _exact(emb, W)).abs() / bound
+    assert over.max() <= 1.0, (over.max(), over.argmax() // m, size[over.argmax() // m], over.argmax() % m)
