@@ -9,12 +9,12 @@
 // memory, per grid by one atomic a sum); the CTA that finishes last solves the two small systems (columns scaled to unit
 // diagonal first, then Gauss-Jordan elimination with partial pivoting) and clears the accumulators for the next call.
 //
-// 28 bytes are read a tuple and some 75 fp64 operations done on it, a third of them in the logarithm: the fp64 pipe and
-// the conversions in front of it bound the slope (6.7 us per million tuples, 4.2 TB/s; copies into shared memory ahead
-// of the arithmetic, two and four tuples interleaved, and 24 warps an SM instead of 16 were no faster or slower), and a
-// call costs 8 us however few the tuples.  4 million tuples on a B200: 56.9 -> 37.0 us with log for log1p, counts as
-// integers, products by one folded (-> 45.3), the elimination on a warp and sums without shared-memory atomics (n = 64:
-// 12.3 -> 8.2).
+// 28 bytes are read a tuple and some 55 fp64 operations done on it: the fp64 pipe and the conversions of five floats in front
+// of it bound the slope (5 us per million tuples, 5.6 TB/s), and a call costs 8 us however few the tuples.  4 million tuples on a
+// B200: 37.3 -> 28.9 us with logarithms from a table and a short series instead of log, one division for four quotients and whole
+// numbers converted on the fp64 pipe (earlier steps, from 56.9: log for log1p, counts as integers, products by one folded, the
+// elimination on a warp and sums without shared-memory atomics; copies into shared memory ahead of the arithmetic, two and four
+// tuples interleaved, and 24 warps an SM instead of 16 were no faster or slower).
 #include <cuda_runtime.h>
 #include <math.h>
 
@@ -24,7 +24,7 @@
 namespace graft {
 namespace {
 
-constexpr int kFitThreads = 256;
+constexpr int kFitThreads = 256;  // (and entries of the table of logarithms)
 constexpr int kFitAcc = 25;  // gain: 10 (upper triangle of 4 x 4) + 4 + 1 count; cost: 6 + 3 + 1 count
 
 struct FitParams {
@@ -78,16 +78,35 @@ struct FitSums {
     double acc[kFitAcc];
     int n_gain, n_cost;
 };
+// a whole number as fp64, on the fp64 pipe (conversions run at a quarter of its rate)
+__device__ __forceinline__ double fit_double(int x) {
+    return __hiloint2double(0x43300000, x ^ (int)0x80000000) - 4503601774854144.0;  // 2^52 + 2^31
+}
+// log(1 - g) for 0 < g < 1 (24 bits, so 1 - g is exact from 2^-29 up), by a table of logarithms and a short series (P. T. P. Tang,
+// "Table-driven implementation of the logarithm function in IEEE floating-point arithmetic", 1990): 1 - g = 2^e f, c the
+// multiple of 1/512 nearest to f in [1/2, 1), r = f / c - 1, log(1 - g) = e ln 2 + log c + log(1 + r), |r| <= 2^-9; the series' first term
+// left out is 2^-57 of r.  With c = 1 for g below 2^-10, where r is -g itself, small results keep their relative precision.
+// tab[k]: 1 / c rounded, and minus the logarithm of that, c = 1/2 + k / 512.  Largest relative error 3e-16.
+__device__ __forceinline__ double fit_log(const double2* tab, double g) {
+    const double x = 1.0 - g;
+    const int hi = __double2hiint(x);
+    const bool near1 = g < 0x1p-10;
+    const double2 t = tab[near1 ? 256 : ((hi & 0xFFFFF) + 0x800) >> 12];
+    const double f = __hiloint2double((hi & 0xFFFFF) | 0x3FE00000, __double2loint(x));
+    const double e = fit_double(near1 ? 0 : (hi >> 20) - 1022);
+    const double r = near1 ? -g : fma(f, t.x, -1.0);
+    double q = fma(r, -1.0 / 6.0, 0.2);
+    q = fma(r, q, -0.25);
+    q = fma(r, q, 1.0 / 3.0);
+    q = fma(r, q, -0.5);
+    return fma(e, 0.69314718055994530942, t.y) + fma(r * r, q, r);
+}
 // One logged round into the running sums.  No branch around the gain model (a warp nearly always has both kinds): a round
 // that says nothing about tau takes part with zeros.
-__device__ __forceinline__ void fit_accumulate(FitSums& t, float s0, float s1, float s2, int budget, float gain, int prefix,
+__device__ __forceinline__ bool fit_ok(float gain) { return gain > 0.0f && gain < 1.0f; }  // a gain of 0 or 1 says nothing about tau
+__device__ __forceinline__ void fit_accumulate(FitSums& t, float s0, float s1, float s2, double B, bool ok, double tau, int prefix,
                                                float latency) {
     double* acc = t.acc;
-    const double B = (double)budget;
-    const bool ok = gain > 0.0f && gain < 1.0f;  // a gain of 0 or 1 says nothing about tau
-    // 1 - g is exact in fp64 from 2^-29 up (g has 24 bits), and log(1 - g) costs less than log1p(-g)
-    const double g = ok ? (double)gain : 0.5;
-    const double tau = ok ? -B / (g >= 0x1p-29 ? log(1.0 - g) : log1p(-g)) : 0.0;
     const double a = (double)(ok ? s0 : 0.f), b = (double)(ok ? s1 : 0.f), c = (double)(ok ? s2 : 0.f);
     acc[0] = fma(a, a, acc[0]);
     acc[1] = fma(a, b, acc[1]);
@@ -103,7 +122,7 @@ __device__ __forceinline__ void fit_accumulate(FitSums& t, float s0, float s1, f
     acc[12] = fma(c, tau, acc[12]);
     acc[13] += tau;
     t.n_gain += ok ? 1 : 0;
-    const double T = (double)latency, BP = B * (double)prefix;
+    const double T = (double)latency, BP = B * fit_double(prefix);
     acc[16] += B;
     acc[17] += BP;
     acc[18] = fma(B, B, acc[18]);
@@ -118,9 +137,16 @@ __device__ __forceinline__ void fit_accumulate(FitSums& t, float s0, float s1, f
 // VEC: every array is 16-byte aligned, so a thread takes four consecutive rounds with seven 16-byte loads
 template <bool VEC>
 __global__ void __launch_bounds__(kFitThreads, 2) saba_fit_kernel(const FitParams p) {
+    __shared__ double2 s_log[257];
     __shared__ double s_acc[kFitAcc], s_warp[kFitThreads / 32][kFitAcc];
     __shared__ bool s_last;
     __shared__ int s_bad[2];
+    {
+        const double inv = 1.0 / (0.5 + threadIdx.x * (1.0 / 512.0));
+        s_log[threadIdx.x] = make_double2(inv, -log(inv));
+        if (threadIdx.x == 0) s_log[kFitThreads] = make_double2(1.0, 0.0);
+    }
+    __syncthreads();
     FitSums t;
 #pragma unroll
     for (int i = 0; i < kFitAcc; ++i) t.acc[i] = 0.0;
@@ -135,16 +161,29 @@ __global__ void __launch_bounds__(kFitThreads, 2) saba_fit_kernel(const FitParam
                          c = __ldg((const float4*)p.state + 3 * q + 2);
             const int4 bu = __ldg((const int4*)p.budget + q), pr = __ldg((const int4*)p.prefix + q);
             const float4 ga = __ldg((const float4*)p.gain + q), la = __ldg((const float4*)p.latency + q);
-            fit_accumulate(t, a.x, a.y, a.z, bu.x, ga.x, pr.x, la.x);
-            fit_accumulate(t, a.w, b.x, b.y, bu.y, ga.y, pr.y, la.y);
-            fit_accumulate(t, b.z, b.w, c.x, bu.z, ga.z, pr.z, la.z);
-            fit_accumulate(t, c.y, c.z, c.w, bu.w, ga.w, pr.w, la.w);
+            // tau = -B / log(1 - g), the four quotients by one division: 1 / l0 = (l2 l3 / (l0 l1 l2 l3)) l1 and so on (P. L.
+            // Montgomery's simultaneous inversion, 1987); the product of four logarithms is between 1e-180 and 1e5
+            const bool ok[4] = {fit_ok(ga.x), fit_ok(ga.y), fit_ok(ga.z), fit_ok(ga.w)};
+            const float g4[4] = {ga.x, ga.y, ga.z, ga.w};
+            double l[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) l[i] = ok[i] ? fit_log(s_log, (double)g4[i]) : 1.0;
+            const double l01 = l[0] * l[1], l23 = l[2] * l[3], inv = 1.0 / (l01 * l23), i01 = inv * l23, i23 = inv * l01;
+            const double B[4] = {fit_double(bu.x), fit_double(bu.y), fit_double(bu.z), fit_double(bu.w)};
+            fit_accumulate(t, a.x, a.y, a.z, B[0], ok[0], ok[0] ? -B[0] * (i01 * l[1]) : 0.0, pr.x, la.x);
+            fit_accumulate(t, a.w, b.x, b.y, B[1], ok[1], ok[1] ? -B[1] * (i01 * l[0]) : 0.0, pr.y, la.y);
+            fit_accumulate(t, b.z, b.w, c.x, B[2], ok[2], ok[2] ? -B[2] * (i23 * l[3]) : 0.0, pr.z, la.z);
+            fit_accumulate(t, c.y, c.z, c.w, B[3], ok[3], ok[3] ? -B[3] * (i23 * l[2]) : 0.0, pr.w, la.w);
         }
         done = n4 * 4;
     }
-    for (long long i = done + tid; i < p.n; i += nth)
-        fit_accumulate(t, p.state[3 * i], p.state[3 * i + 1], p.state[3 * i + 2], p.budget[i], p.gain[i], p.prefix[i],
-                       p.latency[i]);
+    for (long long i = done + tid; i < p.n; i += nth) {
+        const float gain = p.gain[i];
+        const bool ok = fit_ok(gain);
+        const double B = fit_double(p.budget[i]);
+        const double tau = ok ? -B / fit_log(s_log, (double)gain) : 0.0;
+        fit_accumulate(t, p.state[3 * i], p.state[3 * i + 1], p.state[3 * i + 2], B, ok, tau, p.prefix[i], p.latency[i]);
+    }
     t.acc[9] = t.acc[14] = (double)t.n_gain;
     t.acc[15] = t.acc[24] = (double)t.n_cost;
     // The warp's sums of all 25 in 31 steps of exchange (each halves what a lane still carries: lane i ends with sum i)

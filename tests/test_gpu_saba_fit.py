@@ -72,3 +72,21 @@ def test_unaligned_arrays_take_the_scalar_path():
     assert got[9] == 0.0 and got[8] == 3000
     assert np.allclose(got[:4], ref["phi"], rtol=1e-7) and np.allclose(got[4:7], ref["c"], rtol=1e-7)
     g.destroy()
+
+
+@pytest.mark.parametrize("g0", [1e-42, 2.0 ** -60, 2.0 ** -29, 2.0 ** -10, 2.0 ** -9, 0.25, 0.5, 0.625, 1 - 2.0 ** -9, 1 - 2.0 ** -22])
+def test_logarithms_of_gains(g0):
+    """Gains around one value, on both sides of where the logarithm's table changes its entry or its way: the gain model is a
+    regression of -B / ln(1 - g), so an error there shows in it."""
+    rng = np.random.default_rng(13)
+    n = 4003
+    gain = (np.float64(g0) * (1.0 + rng.integers(-4, 5, n) * (2.0 ** -4 if g0 < 0.5 else 2.0 ** -24))).astype(np.float32)
+    lg = dict(state=rng.random((n, 3), dtype=np.float32), budget=rng.integers(16, 513, n).astype(np.int32),
+              gain=np.minimum(gain, np.float32(1 - 2.0 ** -24)), prefix_len=rng.integers(1, 4096, n).astype(np.int32),
+              latency=rng.random(n, dtype=np.float32) + 1)
+    ref = oracle.saba_fit(**lg)
+    g = _ctx()
+    got = _fit(g, lg)
+    assert got[9] == 0.0 and got[7] == ref["n_gain"] == n
+    assert np.all(np.abs(got[:4] - ref["phi"]) <= RTOL * np.abs(ref["phi"]).max()), (got[:4], ref["phi"])
+    g.destroy()
