@@ -1184,11 +1184,12 @@ __global__ void __launch_bounds__(kVpThreads, 1) vocab_pass_kernel(const VpParam
     if (tid == 0 && sh->abort_flag) atomicOr(p.errflag, 1);
 }
 
-// ---- vocabulary-parallel merge: one CTA of 128 threads per row ---------------------------------------------------
+// ---- vocabulary-parallel merge: one CTA per row ------------------------------------------------------------------
 // A latency chain (1024 rows of 8 shards are 2.3 MB): every load is issued at once, a key's rank is its place in its own
 // shard's descending list plus the places a binary search finds for it in the others (ranking all keys against each
-// other, 256 x 256 compares a row, and folding the log-sum-exp pieces one after the other took 19 us of 49), and the
-// pieces are folded by a lane each.
+// other, 256 x 256 compares a row, and folding the log-sum-exp pieces one after the other took 19 us of 49), a key a
+// thread for eight shards; one warp more folds the pieces, by a lane each, meanwhile.
+constexpr int kMergeThreads = 256;
 constexpr int kMergeMaxShards = 64;
 struct MergeParams {
     const graft_vocab_partial* parts;  // [n_shards, rows]
@@ -1199,18 +1200,20 @@ struct MergeParams {
     float* lse;
     int32_t* row_status;
 };
-__global__ void __launch_bounds__(128) vocab_merge_kernel(const __grid_constant__ MergeParams p) {
+__global__ void __launch_bounds__(kMergeThreads + 32) vocab_merge_kernel(const __grid_constant__ MergeParams p) {
     extern __shared__ uint64_t merge_cand[];  // [n_shards][kMaxK]
     __shared__ uint64_t outk[kMaxK];
+    __shared__ double s_lse;
+    __shared__ int s_status, s_nk;
     const int row = blockIdx.x, tid = threadIdx.x, lane = tid & 31;
     const int n = p.n_shards * kMaxK;
     pdl_launch_dependents();
     pdl_wait();
-    // warp 0: the shards' pieces (two a lane: up to 64 shards)
-    double c2[2] = {-INFINITY, -INFINITY}, s2[2] = {0.0, 0.0};
-    uint32_t vm = 0u;
-    int have = 0, internal = 0;
-    if (tid < 32) {
+    if (tid >= kMergeThreads) {
+        // the shards' pieces (two a lane: up to 64 shards)
+        double c2[2] = {-INFINITY, -INFINITY}, s2[2] = {0.0, 0.0};
+        uint32_t vm = 0u;
+        int have = 0, internal = 0;
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const int i = lane + 32 * h;
@@ -1224,9 +1227,33 @@ __global__ void __launch_bounds__(128) vocab_merge_kernel(const __grid_constant_
                 internal |= (int)(kn >> 31);
             }
         }
+        double Cm = fmax(c2[0], c2[1]), S = 0.0;
+#pragma unroll
+        for (int d = 16; d > 0; d >>= 1) Cm = fmax(Cm, __shfl_xor_sync(0xFFFFFFFFu, Cm, d));
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            if (c2[h] != -INFINITY)
+                S += s2[h] * exp2(c2[h] - Cm);
+            else if (s2[h] != s2[h])
+                S += s2[h];
+        }
+#pragma unroll
+        for (int d = 16; d > 0; d >>= 1) S += __shfl_xor_sync(0xFFFFFFFFu, S, d);
+        vm = __reduce_max_sync(0xFFFFFFFFu, vm);
+        have = __reduce_add_sync(0xFFFFFFFFu, have);
+        internal = __any_sync(0xFFFFFFFFu, internal);
+        if (lane == 0) {
+            const int nk = have < p.K ? have : p.K;
+            s_lse = vp_lse(Cm, S, __uint_as_float(bits_from_ord(vm)));
+            s_status = (vp_bad_row(S, vm, nk, p.K) ? GRAFT_ST_BAD_LOGITS : 0) | (internal ? GRAFT_ST_INTERNAL : 0);
+            s_nk = nk;
+        }
+        __syncthreads();
+        __syncthreads();
+        return;
     }
     // the shards' keys with global token ids (an empty slot stays 0 and ranks below every key)
-    for (int i = tid; i < n; i += 128) {
+    for (int i = tid; i < n; i += kMergeThreads) {
         const int sidx = i / kMaxK, kk = i % kMaxK;
         const graft_vocab_partial* r = p.parts + (size_t)sidx * p.rows + row;
         const uint32_t kn = r->nkeys;
@@ -1237,7 +1264,7 @@ __global__ void __launch_bounds__(128) vocab_merge_kernel(const __grid_constant_
     }
     if (tid < kMaxK) outk[tid] = 0ull;
     __syncthreads();
-    for (int i = tid; i < n; i += 128) {
+    for (int i = tid; i < n; i += kMergeThreads) {
         const uint64_t key = merge_cand[i];
         int rank = 0;
         if (key == 0ull || i % kMaxK >= p.K) continue;
@@ -1253,24 +1280,9 @@ __global__ void __launch_bounds__(128) vocab_merge_kernel(const __grid_constant_
         if (rank < p.K) outk[rank] = key;
     }
     __syncthreads();
-    if (tid >= 32) return;
-    double Cm = fmax(c2[0], c2[1]), S = 0.0;
-#pragma unroll
-    for (int d = 16; d > 0; d >>= 1) Cm = fmax(Cm, __shfl_xor_sync(0xFFFFFFFFu, Cm, d));
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        if (c2[h] != -INFINITY)
-            S += s2[h] * exp2(c2[h] - Cm);
-        else if (s2[h] != s2[h])
-            S += s2[h];
-    }
-#pragma unroll
-    for (int d = 16; d > 0; d >>= 1) S += __shfl_xor_sync(0xFFFFFFFFu, S, d);
-    vm = __reduce_max_sync(0xFFFFFFFFu, vm);
-    have = __reduce_add_sync(0xFFFFFFFFu, have);
-    internal = __any_sync(0xFFFFFFFFu, internal);
-    vp_finalize(Cm, S, vm, have < p.K ? have : p.K, p.K, outk, lane, p.topk_id + (size_t)row * p.K,
-                p.topk_lp + (size_t)row * p.K, p.lse + row, p.row_status + row, internal != 0);
+    if (tid < 32)
+        vp_write_row(s_lse, s_status, s_nk, p.K, outk, lane, p.topk_id + (size_t)row * p.K, p.topk_lp + (size_t)row * p.K,
+                     p.lse + row, p.row_status + row);
 }
 
 }  // namespace
@@ -1478,7 +1490,7 @@ cudaError_t vp_merge_launch(graft_ctx* ctx, int batch, int n_shards, const graft
     p.topk_lp = d_topk_lp;
     p.lse = d_lse;
     p.row_status = d_row_status;
-    const cudaError_t e = launch_pdl(vocab_merge_kernel, dim3(p.rows), dim3(128), (size_t)n_shards * kMaxK * sizeof(uint64_t), st, p);
+    const cudaError_t e = launch_pdl(vocab_merge_kernel, dim3(p.rows), dim3(kMergeThreads + 32), (size_t)n_shards * kMaxK * sizeof(uint64_t), st, p);
     ctx->launches += 1;
     return e != cudaSuccess ? e : cudaGetLastError();
 }
