@@ -1328,9 +1328,10 @@ static void rows_plan(long long rows, long long row_bytes, int num_sms, VpPlan* 
         // longer rows, an SM for each (bf16, V = 75,000: batch 4 10.4 -> 7.2, batch 8 10.8 -> 7.8; with 256 threads 7.7, 8.3)
         pl->cluster = 1;
         pl->threads = 512;
-    } else if (rows * 4 <= (long long)num_sms * rows_per_sm(row_bytes, 4, 256)) {
+    } else if (rows * 4 <= (long long)num_sms * rows_per_sm(row_bytes, 4, 256) * (row_bytes >= 380 * 1024 ? 2 : 1)) {
         // rows too long for one CTA, or rows of 80 KB and more where four times as many SMs would stand idle, as far as all
-        // pieces are resident at once.  V = 151,936: bf16 batch 1 12.7 -> 8.0, batch 4 13.4 -> 8.9, batch 8 (two turns) 15.1 ->
+        // pieces are resident at once; twice as far with rows of 380 KB, which the streaming kernel would cut and merge (rounds,
+        // fp32, V = 151,936: batch 3 46.8 -> 42.1 us, batch 4 52.8 -> 47.4, batch 6 53.4 -> 58.5).  V = 151,936: bf16 batch 1 12.7 -> 8.0, batch 4 13.4 -> 8.9, batch 8 (two turns) 15.1 ->
         // 18.5; fp32 batch 1 13.7 -> 7.2.  V = 50,021, bf16, batch 1 10.0 -> 5.8 (6.6 in one CTA), V = 32,000 the same in one
         // CTA as in four.  (512 threads: 9.0 at batch 1, V = 151,936; eight CTAs a row 7.9, but 10.0 at batch 4.)
         pl->cluster = 4;
