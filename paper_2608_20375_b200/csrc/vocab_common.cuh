@@ -120,14 +120,14 @@ __device__ __forceinline__ float pair_max_bf16(uint32_t pm) {  // the larger hal
     return fmaxf(__uint_as_float(pm << 16), __uint_as_float(pm & 0xFFFF0000u));
 }
 
-// Four 16-byte vectors of logits into the running sum.
+// 16-byte vectors of logits into the running sum (four a step).
 constexpr int VEC_PER_LANE = 4;
-template <bool BF16>
-__device__ __forceinline__ void acc_add(const uint4 (&v)[VEC_PER_LANE], Acc& a) {
+template <bool BF16, int N>
+__device__ __forceinline__ void acc_add(const uint4 (&v)[N], Acc& a) {
 #if GRAFT_VP_F32X2
     const uint64_t c2 = pack2(kLog2e, kLog2e), r2 = pack2(a.nref, a.nref);
 #pragma unroll
-    for (int i = 0; i < VEC_PER_LANE; ++i) {
+    for (int i = 0; i < N; ++i) {
         const uint32_t w[4] = {v[i].x, v[i].y, v[i].z, v[i].w};
         if (BF16) {
 #pragma unroll
@@ -151,7 +151,7 @@ __device__ __forceinline__ void acc_add(const uint4 (&v)[VEC_PER_LANE], Acc& a) 
     }
 #else
 #pragma unroll
-    for (int i = 0; i < VEC_PER_LANE; ++i) {
+    for (int i = 0; i < N; ++i) {
         const uint32_t w[4] = {v[i].x, v[i].y, v[i].z, v[i].w};
         if (BF16) {
 #pragma unroll
