@@ -1319,8 +1319,8 @@ static void rows_plan(long long rows, long long row_bytes, int num_sms, VpPlan* 
     const bool alone = rows * 4 <= num_sms;  // four CTAs a row and an SM for each
     if (rows_per_sm(row_bytes, 1, 256) >= 2 && !(alone && row_bytes >= 80 * 1024)) {
         // a row a CTA where two or more share an SM, any number of rows.  bf16, V = 32,000 (three an SM): batch 1 8.3 -> 5.8 us,
-        // batch 16 11.2 -> 9.2, batch 64 25.2 -> 20.4, batch 256 74.7 -> 63.9; V = 16,000 (four): batch 64 20.9 -> 13.7, batch
-        // 256 63.5 -> 42.4; V = 50,021 (two): batch 64 34.3 -> 31.5, batch 256 114 -> 107.  With one CTA an SM nothing loads
+        // batch 16 11.2 -> 9.5, batch 64 25.2 -> 20.7, batch 256 74.7 -> 62.5; V = 16,000 (four): batch 64 20.9 -> 13.5, batch
+        // 256 63.5 -> 41.2; V = 50,021 (two): batch 64 34.3 -> 30.8, batch 256 114 -> 102.5.  With one CTA an SM nothing loads
         // while a row is finished: fp32, V = 32,000, batch 64 29.5 -> 45
         pl->cluster = 1;
         pl->threads = 256;

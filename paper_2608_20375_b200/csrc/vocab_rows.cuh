@@ -13,9 +13,9 @@
 //     row's and about K + 12 candidates in all go to the first CTA, which ranks them: two exchanges of 1.3 k cycles, no global
 //     memory, no counters;
 //   * rows whose candidates overflow the list (ties in bulk, sorted rows) are bisected on the logits' bits in shared memory.
-// What bounds it: batch 1 at V = 151,936 is a chain -- load 3.9 k cycles (arithmetic of 19 k logits a quarter SM), sums and T 1.7 k,
-// candidates 1.6 k, second exchange 1.3 k, ranks and outputs 1.4 k -- 8.0 us a launch (12.7 by the streaming kernel).  Many
-// short rows: the issue slots and latencies of the four CTAs on an SM, 42.4 us for 131 MB at V = 16,000 (63.5).
+// What bounds it: batch 1 at V = 151,936 is a chain -- load 3.9 k cycles (the arithmetic of 38 k logits an SM among them), sums and
+// T 1.7 k, candidates 1.6 k, second exchange 1.3 k, ranks and outputs 1.4 k -- 8.0 us a launch (12.7 by the streaming kernel).
+// Many short rows: the issue slots (72 % taken by the four CTAs of an SM), 41.2 us for 131 MB at V = 16,000 (63.5).
 // References of the sums are whole numbers, so that sums are brought together exactly.
 #pragma once
 #include "umma.cuh"
