@@ -47,11 +47,16 @@ def test_a_wait_that_runs_out_is_reported_by_the_block_that_merges_the_row(tmp_p
     _case(_build_test_library(tmp_path, "-DGRAFT_TEST_LATE_RECORDS=20"), 1, 16, [0])
 
 
-def _case(so, Bt, L, flagged_rows):
+def test_a_wait_that_runs_out_is_reported_by_the_block_that_merges_a_long_row(tmp_path):
+    # the same where rows are too long for a cluster's shared memory: nine pieces a row, through records in global memory
+    _case(_build_test_library(tmp_path, "-DGRAFT_TEST_LATE_RECORDS=20"), 1, 16, [0], V=480000)
+
+
+def _case(so, Bt, L, flagged_rows, V=151936):
     lib = C.CDLL(so)
     vp = C.c_void_p
     lib.graft_vocab_pass_static.argtypes = [C.c_int32, C.c_int32, C.c_int32, C.c_int32, C.c_int, vp, vp, vp, vp, vp, vp]
-    V, K = 151936, 16
+    K = 16
     g = torch.Generator().manual_seed(5)
     z = (2.0 * torch.randn((Bt, L, V), generator=g)).to(torch.bfloat16)
     zc = z.cuda()
