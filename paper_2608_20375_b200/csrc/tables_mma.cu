@@ -63,7 +63,7 @@ struct TablesCfg {
     static constexpr int A_BYTES = 2 * PART;                  // a block's embeddings: two row blocks, or two parts
     static constexpr int W_BYTES = (F32 ? 256 : 192) * BLK * 2;  // a block's W; a pair: W1 (even CTA) or W2 (odd), half of W3
     static constexpr int RAW = 128 * BLK * 4;                 // a block's fp32 embeddings
-    static constexpr int STAGES = 4, RAW_STAGES = F32 ? 5 : 1;  // (a stage: a block's embeddings and W)
+    static constexpr int STAGES = 4, RAW_STAGES = F32 ? 4 : 1;  // (a stage: a block's embeddings and W)
     static constexpr int THREADS = (kTmEpiWarps + 2 + (F32 ? 1 + kTmConvWarps : 0)) * 32;
     // (the rings start on a 1024-byte boundary)
     static constexpr size_t SMEM = (size_t)STAGES * (A_BYTES + W_BYTES) + (F32 ? (size_t)RAW_STAGES * RAW : 0) + 1024;
@@ -628,7 +628,11 @@ __global__ void __cluster_dims__(F32 ? 1 : 2, 1, 1) __launch_bounds__(TablesCfg<
         }
     } else if (F32) {
         // ------------------------------ fp32 embeddings -> fp16 parts ----------------------------
-        // four warps take the even blocks, four the odd ones: a block is a chain of waits and round trips
+        // four warps take the even blocks, four the odd ones: a block is a chain of waits and round trips.  A wait on a barrier's parity
+        // tells a phase from the ones beside it and not from the one two before, so a half has to wait for every phase of the
+        // barriers that it waits on: with an even number of stages every stage is always the same half's.  (Four raw stages or six: V =
+        // 32,000, E = 2048, two towers 208.4 and 209.3 us.)
+        static_assert(!F32 || (NR % 2 == 0 && NS % 2 == 0), "a stage of either ring belongs to one half of the converting warps");
         const int ct = (tid - (kTmEpiWarps + 3) * 32) & 127, half = (tid - (kTmEpiWarps + 3) * 32) >> 7;
         const int c8 = ct & 3, r0 = ct >> 2;  // columns 8 c8 .. 8 c8 + 7 of rows r0, r0 + 32, r0 + 64 and r0 + 96
         const float scale = *p.scale;
