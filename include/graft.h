@@ -143,7 +143,7 @@ int32_t graft_edge_rows(const graft_ctx* ctx);
  * 22 bits or 2^-26 of their row's largest, those of W to 22 bits or 2^-50; infinities and values up to the largest fp32 give what
  * fp32 arithmetic gives.  A
  * bf16 embedding or a W beside bf16 embeddings that is infinite, or a W that rounds past the largest bf16, gives NaN.
- * Such calls use scratch of the context (3 m E 16-bit values, V bytes and up to 40 MB of partial sums, m rounded up to 128), which the
+ * Such calls use scratch of the context (3 m E 16-bit values, V m / 128 bytes and up to 40 MB of partial sums, m rounded up to 128), which the
  * first of them allocates and one that needs more replaces -- under stream capture too; a captured call keeps the scratch it
  * was captured with until the context is destroyed.  Without memory for it, and for other pointers and E, an FMA kernel
  * takes the call.  This is the once-per-model setup step, not the round. */

@@ -110,7 +110,7 @@ struct __align__(64) TablesParams {
     // fp32 embeddings only
     const float2* unscale;  // [m_pad] what a column's sums are multiplied by, as two factors
     const float* scale;     // [1] what the embeddings are multiplied by
-    uint8_t* bad_row;       // [tiles of V][ROWS] rows whose entries fp16 parts do not hold well enough
+    uint8_t* bad_row;       // [tiles][ROWS] rows whose entries fp16 parts do not hold well enough, as the tile's workers saw them
     int32_t* errflag;
     int V, E, m, m_pad, n_mb, n_kb;
     int pairs, full_rounds;
@@ -478,7 +478,7 @@ __global__ void __cluster_dims__(F32 ? 1 : 2, 1, 1) __launch_bounds__(TablesCfg<
                     if (it.q0 != it.q1) continue;  // (pieces: the kernel that adds them up)
                     const int rt = it.tile / p.n_mb, c0 = (it.tile - rt * p.n_mb) * 128;
                     for (int v = rt * C::ROWS + warp; v < p.V && v < (rt + 1) * C::ROWS; v += kTmEpiWarps) {
-                        const bool bad = p.bad_row[v] != 0;
+                        const bool bad = p.bad_row[(size_t)it.tile * C::ROWS + (v - rt * C::ROWS)] != 0;
                         for (int c = c0 + lane; c < p.m && c < c0 + 128; c += 32) {
                             float* o = p.out + (size_t)v * p.m + c;
                             if (bad || !tables_finite(*o)) *o = tables_fp32(p, v, c);
@@ -685,7 +685,7 @@ __global__ void __cluster_dims__(F32 ? 1 : 2, 1, 1) __launch_bounds__(TablesCfg<
                 mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, 2));
                 const int v = rt * C::ROWS + r0 + 32 * q;
                 if (c8 == 0 && v < p.V && !tables_row_ok(mx, scale)) {
-                    p.bad_row[v] = 1;
+                    p.bad_row[(size_t)it.tile * C::ROWS + r0 + 32 * q] = 1;
                     if (it.q0 == it.q1) s_mend = true;
                 }
             }
@@ -712,7 +712,7 @@ __global__ void __launch_bounds__(256) tables_pieces_kernel(const __grid_constan
     const int q0 = tables_owner(p, tile * p.n_kb), q1 = tables_owner(p, (tile + 1) * p.n_kb - 1);
     const int v = (int)blockIdx.x * 8 + (threadIdx.x >> 5), c = (threadIdx.x & 31) * 4;
     if (q0 == q1 || rt * C::ROWS + v >= p.V || mb * 128 + c >= p.m) return;  // (q0 == q1: written whole)
-    const bool bad = F32 && p.bad_row[rt * C::ROWS + v] != 0;
+    const bool bad = F32 && p.bad_row[(size_t)tile * C::ROWS + v] != 0;
     float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll 4
     for (int q = q0; q <= q1; ++q) {
@@ -775,7 +775,7 @@ TablesSizes tables_sizes(int num_sms, int V, int E, int m, bool f32) {
     s.o_unscale = s.o_w + (size_t)(f32 ? 2 : 3) * s.m_pad * s.E_pad * 2;
     s.o_scale = s.o_unscale + (f32 ? (size_t)s.m_pad * sizeof(float2) : 0);
     s.o_bad = s.o_scale + (f32 ? 256 : 0);
-    s.n_bad = f32 ? (size_t)(V + TablesCfg<true>::ROWS - 1) / TablesCfg<true>::ROWS * TablesCfg<true>::ROWS : 0;
+    s.n_bad = f32 ? (size_t)(V + TablesCfg<true>::ROWS - 1) / TablesCfg<true>::ROWS * s.n_mb * TablesCfg<true>::ROWS : 0;
     s.total = s.o_bad + s.n_bad;
     return s;
 }

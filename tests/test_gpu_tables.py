@@ -171,3 +171,26 @@ def test_fp32_rows_of_other_sizes(V, E, m):
     bound = 2e-5 * size[:, None].double() * wide[None].double() + 0.7e-45 * E
     over = (got - _exact(emb, W)).abs() / bound
     assert over.max() <= 1.0, (over.max(), over.argmax() // m, size[over.argmax() // m], over.argmax() % m)
+
+
+@pytest.mark.parametrize("row", ["a small piece", "a piece of two sizes"])
+def test_fp32_rows_are_judged_tile_by_tile(row):
+    """Three blocks of columns of the table, of which two are left over and cut along E while the third is worked out whole: a row that only
+    the pieces' workers find unfit for fp16 parts keeps its results in the third block, whatever else is worked out again there."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    m, E = 384, 2048
+    tiles = next(t for t in range(sms + 1, sms + 10) if t % 3 == 0 and (t - sms) % 3 != 0)
+    V = tiles // 3 * 128
+    emb, W, _ = _inputs(V, E, m, "f32", 12)
+    if row == "a small piece":
+        emb[10, 256:512] *= 2.0 ** -25
+    else:
+        emb[10, 256:288] *= 2.0 ** -9
+        emb[10, 320:352] *= 2.0 ** 6
+    g = _graft(V, m)
+    want = _call(g, emb, W, None, m)
+    emb[20, 0] = float("inf")  # (its results are not finite: the third block's tile of these rows is looked through)
+    got = _call(g, emb, W, None, m)
+    rest = torch.arange(V, device="cuda") != 20
+    assert torch.equal(got[rest], want[rest])
+    assert not got[20].isfinite().any()
