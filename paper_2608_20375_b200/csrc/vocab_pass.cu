@@ -670,10 +670,11 @@ __global__ void __launch_bounds__(kVpThreads, 1) vocab_pass_kernel(const VpParam
             {
                 // the warp's piece of the log-sum-exp: the largest reference of its lanes (one integer reduction over
                 // the order-preserving images), every lane's sum rescaled to it once, then a butterfly of plain adds
-                // (a fixed order: the result does not depend on timing)
+                // (a fixed order: the result does not depend on timing).  A lane without a reference has added up zeros, or a
+                // NaN, which marks the row.
                 const uint32_t co = __reduce_max_sync(0xFFFFFFFFu, ord_from_float(a.ref));
                 const float c = __uint_as_float(bits_from_ord(co));
-                float s = (a.ref == -INFINITY) ? 0.f : acc_sum<BF16>(a) * ex2_approx(a.ref - c);
+                float s = acc_sum<BF16>(a) * (a.ref == -INFINITY ? 1.f : ex2_approx(a.ref - c));
 #pragma unroll
                 for (int d = 16; d > 0; d >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, d);
                 if (lane == 0) {

@@ -408,9 +408,10 @@ __global__ void __launch_bounds__(NT + 32, NT == 256 ? 4 : 2) vocab_rows_kernel(
     const uint32_t tmax = ord_from_float(BF16 ? pair_max_bf16(a.rmax) : __uint_as_float(a.rmax));
     atomicMax(&sh->gmax[tid & (kVpGroups - 1)], tmax);
     {
-        // the warp's sum, at the largest reference of its lanes (references are whole numbers: exact)
+        // the warp's sum, at the largest reference of its lanes (references are whole numbers: exact; a thread without one has
+        // added up zeros, or a NaN, which marks the row)
         const float c = __uint_as_float(bits_from_ord(__reduce_max_sync(0xFFFFFFFFu, ord_from_float(a.ref))));
-        float s = a.ref == -INFINITY ? 0.f : acc_sum<BF16>(a) * ex2_whole(a.ref - c);
+        float s = acc_sum<BF16>(a) * (a.ref == -INFINITY ? 1.f : ex2_whole(a.ref - c));
 #pragma unroll
         for (int d = 16; d > 0; d >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, d);
         if (lane == 0) sh->lse[CL > 1 ? rank : 0][warp] = make_float2(c, s);

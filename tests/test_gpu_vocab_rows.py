@@ -96,3 +96,36 @@ def test_rows_in_shared_memory_report_bad_logits(bad):
     _, _, _, o_st = oracle.vocab_pass(z.view(L, V), K)
     assert np.array_equal(st.cpu().numpy().reshape(-1), o_st)
     assert o_st[2] == 1 and o_st[0] == 0
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("batch,V", [
+    (2, 20011),    # a row a CTA
+    (2, 75011),    # bf16: a row a CTA of 512 threads; fp32: clusters of four
+    (1, 130003),   # clusters of four
+    (20, 150001),  # the streaming kernel, whole rows and rows in pieces
+])
+def test_a_nan_among_masked_tokens_is_reported(batch, V, dtype):
+    """Rows masked to -inf but for 40 tokens, and one NaN: at either ragged end, in the body, where no finite token is near it."""
+    from paper_2608_20375_b200 import Graft
+    L, K = 8, 32
+    g = torch.Generator().manual_seed(7)
+    z = torch.full((batch * L, V), -float("inf"))
+    for r in range(batch * L):
+        keep = torch.randint(V // 3, V // 2, (64,), generator=g).unique()[:40]
+        z[r, keep] = torch.randn(len(keep), generator=g)
+    places = [None, 0, V - 1, V // 4 + 13, 3 * V // 4 + 5, 9000, None, V - 2]
+    for r in range(batch * L):
+        if places[r % 8] is not None:
+            z[r, places[r % 8]] = float("nan")
+    z = z.to(dtype)
+    gr = Graft(V, L, K, 16, 8, batch, 8, 8, 8, 0.0, 1, 1 if dtype == torch.bfloat16 else 0, 0)
+    out = (torch.empty((batch, L, K), dtype=torch.int32, device="cuda"), torch.empty((batch, L, K), device="cuda"),
+           torch.empty((batch, L), device="cuda"), torch.empty((batch, L), dtype=torch.int32, device="cuda"))
+    gr.vocab_pass(z.view(batch, L, V).cuda(), *out)
+    torch.cuda.synchronize()
+    bad = np.array([places[r % 8] is not None for r in range(batch * L)]).astype(np.int32)
+    assert np.array_equal(out[3].cpu().numpy().reshape(-1), bad)
+    o_ids, _, _, o_st = oracle.vocab_pass(z[:8], K)
+    assert np.array_equal(o_st, bad[:8])
+    assert np.array_equal(out[0].cpu().numpy().reshape(-1, K)[:8][bad[:8] == 0], o_ids[bad[:8] == 0])
