@@ -558,7 +558,10 @@ __global__ void __launch_bounds__(NT + 32, NT == 256 ? 4 : 2) vocab_rows_kernel(
             st_async_v2(to + 8 * lane, (uint32_t)key, (uint32_t)(key >> 32), bar);
             if (lane == 0) {
                 st_async_v2(mapa_u32(smem_u32(&sh->cnt[rank]), 0), (uint32_t)n, sh->abort_flag ? 1u : 0u, bar);
-                mbar_arrive_cluster(mapa_u32(x3, 0));
+#ifdef GRAFT_TEST_WITHHOLD_LISTS
+                if (rank != 1)  // (test builds only: the rest of a long list is never said to be there)
+#endif
+                    mbar_arrive_cluster(mapa_u32(x3, 0));
             }
         }
         __syncwarp();
@@ -569,7 +572,7 @@ __global__ void __launch_bounds__(NT + 32, NT == 256 ? 4 : 2) vocab_rows_kernel(
     // ------------------------------ ranks, outputs (the first CTA) ---------------------------------
     if (rank == 0) {
         int total = n;
-        bool internal = sh->abort_flag != 0;
+        bool internal = false;
         uint64_t* const all = sh->cand;
         if (CL > 1) {
             // the lists one behind the other; a warp moves a list (CL = 2 and 4: some do nothing)
@@ -607,6 +610,7 @@ __global__ void __launch_bounds__(NT + 32, NT == 256 ? 4 : 2) vocab_rows_kernel(
         }
         rows_bar<NT>();
         const int nk = total < p.K ? total : p.K;
+        internal |= sh->abort_flag != 0;  // (behind the barrier: no warp of this CTA waits for anything any more)
         if (warp == 0) {
             if (p.partial_out != nullptr) {
                 graft_vocab_partial* po = p.partial_out + row;

@@ -24,11 +24,11 @@ pytestmark = pytest.mark.gpu
 ST_INTERNAL = 8
 
 
-def _build_test_library(tmp_path, *flags):
+def _build_test_library(tmp_path, *flags, withheld="-DGRAFT_TEST_WITHHOLD_TILE=2"):
     from paper_2608_20375_b200 import build as b
     out = os.path.join(str(tmp_path), "libgraft_waittest.so")
     cmd = [os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc"), *b.NVCC_FLAGS, "-DGRAFT_SPIN_LIMIT=512u",
-           "-DGRAFT_TEST_WITHHOLD_TILE=2", *flags, "-I", os.path.join(b.HERE, "..", "include"), "-shared",
+           withheld, *flags, "-I", os.path.join(b.HERE, "..", "include"), "-shared",
            os.path.join(b.CSRC, "vocab_pass.cu"), "-o", out, "-lcudart"]
     subprocess.check_call(cmd, stderr=subprocess.DEVNULL)
     return out
@@ -52,13 +52,21 @@ def test_a_wait_that_runs_out_is_reported_by_the_block_that_merges_a_long_row(tm
     _case(_build_test_library(tmp_path, "-DGRAFT_TEST_LATE_RECORDS=20"), 1, 16, [0], V=480000)
 
 
-def _case(so, Bt, L, flagged_rows, V=151936):
+def test_a_wait_that_runs_out_after_the_lists_were_sent_is_reported(tmp_path):
+    # clusters of four; one row has over 32 candidates in every piece and the arrival behind a piece's list never comes: the first
+    # block of that cluster gives up when all counts are there.  Other rows' lists are short and nothing waits for that arrival.
+    _case(_build_test_library(tmp_path, withheld="-DGRAFT_TEST_WITHHOLD_LISTS"), 1, 16, [3], ties=3)
+
+
+def _case(so, Bt, L, flagged_rows, V=151936, ties=None):
     lib = C.CDLL(so)
     vp = C.c_void_p
     lib.graft_vocab_pass_static.argtypes = [C.c_int32, C.c_int32, C.c_int32, C.c_int32, C.c_int, vp, vp, vp, vp, vp, vp]
     K = 16
     g = torch.Generator().manual_seed(5)
     z = (2.0 * torch.randn((Bt, L, V), generator=g)).to(torch.bfloat16)
+    if ties is not None:
+        z.view(-1, V)[ties, ::620] = 20.0  # (61 in every quarter of the row)
     zc = z.cuda()
     ids = torch.full((Bt, L, K), -7, dtype=torch.int32, device="cuda")
     lp = torch.zeros((Bt, L, K), dtype=torch.float32, device="cuda")
