@@ -22,6 +22,10 @@
 #include "vocab_common.cuh"
 #include "cosine.cuh"
 
+#ifndef GRAFT_TEST_WITHHOLD_CTA
+#define GRAFT_TEST_WITHHOLD_CTA 0  // (test builds: the thread block one of whose copies is never issued)
+#endif
+
 namespace graft {
 
 namespace {
@@ -325,7 +329,7 @@ __global__ void __launch_bounds__(NT + 32, NT == 256 ? 4 : 2) vocab_rows_kernel(
                 const uint32_t bytes = s1 > s0 ? (uint32_t)(s1 - s0) * 16u : 0u;
                 mbar_arrive_expect_tx(full0 + 8 * t, bytes);
 #ifdef GRAFT_TEST_WITHHOLD_TILE
-                if (blockIdx.x == 0 && t == GRAFT_TEST_WITHHOLD_TILE) continue;  // (as in the streaming kernel: test builds only)
+                if (blockIdx.x == GRAFT_TEST_WITHHOLD_CTA && t == GRAFT_TEST_WITHHOLD_TILE) continue;  // (as in the streaming kernel: test builds only)
 #endif
                 if (bytes) tma_load_1d_hint(smem_u32(vec + s0), body + (size_t)(s0 - 1) * 16, bytes, full0 + 8 * t, policy);
             }

@@ -5,9 +5,10 @@ The vocab pass waits on shared-memory barriers with an iteration limit; when a w
 raises a flag, stops waiting, drains its copies in flight and finishes, and every row it finishes or leaves a piece of
 carries GRAFT_ST_INTERNAL.  To make a wait run out without faulting, trapping or hanging anything, this test compiles
 a SECOND copy of the vocab pass (one source file, into a temporary folder) with a tiny iteration limit and a build flag
-under which thread block 0 never issues the copy of its third tile.  The shipped library is not touched.  A second flag
+under which one thread block never issues the copy of its third tile.  The shipped library is not touched.  A second flag
 lets the other thread blocks leave their records of shared rows some milliseconds late, after block 0 has given up: the
-block that merges block 0's row has seen no time-out itself and knows of it from block 0's record alone.
+block that merges block 0's row has seen no time-out itself and knows of it from block 0's record alone.  A third keeps
+one block of every cluster from saying that the rest of its list of candidates is there.
 """
 import ctypes as C
 import os
@@ -42,13 +43,18 @@ def test_a_wait_that_runs_out_is_reported_and_the_device_stays_usable(tmp_path, 
     _case(_build_test_library(tmp_path), Bt, L, flagged_rows)
 
 
+@pytest.mark.parametrize("Bt,V,block,flagged_rows", [
+    (4, 50021, 5, [5]),     # a row a thread block of 256 threads, six tiles
+    (4, 75000, 0, [0]),     # of 512 threads, four tiles
+    (1, 151936, 4, [1]),    # a row a cluster of four, four tiles each: the block that ranks the row's candidates
+    (1, 151936, 6, [1]),    # and another, which tells the first with its number of candidates
+])
+def test_a_wait_that_runs_out_on_a_row_in_shared_memory_is_reported(tmp_path, Bt, V, block, flagged_rows):
+    _case(_build_test_library(tmp_path, f"-DGRAFT_TEST_WITHHOLD_CTA={block}"), Bt, 16, flagged_rows, V=V)
+
+
 def test_a_wait_that_runs_out_is_reported_by_the_block_that_merges_the_row(tmp_path):
-    # one sequence: every row in three pieces of four tiles, a thread block each
-    _case(_build_test_library(tmp_path, "-DGRAFT_TEST_LATE_RECORDS=20"), 1, 16, [0])
-
-
-def test_a_wait_that_runs_out_is_reported_by_the_block_that_merges_a_long_row(tmp_path):
-    # the same where rows are too long for a cluster's shared memory: nine pieces a row, through records in global memory
+    # rows too long for a cluster's shared memory: nine pieces a row, a thread block each, which meet through records in global memory
     _case(_build_test_library(tmp_path, "-DGRAFT_TEST_LATE_RECORDS=20"), 1, 16, [0], V=480000)
 
 
