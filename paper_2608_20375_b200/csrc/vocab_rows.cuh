@@ -71,6 +71,7 @@ struct __align__(16) RowsShared {
     uint32_t vmax;
     uint32_t T;
     uint32_t gmost;            // the largest group maximum, its low bits set
+    uint32_t gleast;           // the least, its low bits cut off
     uint2 cnt[CL];             // the first CTA's: candidates of every CTA; has a bounded wait run out there?
     int ncand, nhits;
     uint16_t hits[kRowsHits];  // (step, thread) whose maximum reaches T
@@ -153,18 +154,115 @@ __device__ __forceinline__ float rows_step(const uint4 (&v)[N], Acc& a, uint16_t
 }
 __device__ __forceinline__ uint64_t rows_key(uint32_t o, int e) { return ((uint64_t)o << 32) | (uint64_t)(0xFFFFFFFFu - (uint32_t)e); }
 
+// The elements of the listed steps that reach T (ABOVE: that exceed it), to the list of candidates, a vector a thread.
+template <bool BF16, bool ABOVE, int CL, int NT>
+__device__ __forceinline__ void rows_take_hits(RowsShared<CL, NT>* sh, const uint4* vec, const RowsPiece& pc, int nhits, float Tf, int tid) {
+    using T = VT<BF16>;
+    using Sh = RowsShared<CL, NT>;
+#pragma unroll 1
+    for (int i = tid; i < nhits * VEC_PER_LANE; i += NT) {
+        const uint32_t at = sh->hits[i / VEC_PER_LANE];
+        const int s = (int)(at / NT) * Sh::TILE + (i % VEC_PER_LANE) * NT + (int)(at % NT);
+        if (s >= pc.nvec) continue;
+        const uint4 x = vec[s];
+        const uint32_t w[4] = {x.x, x.y, x.z, x.w};
+        const int e = pc.e_vec0 + s * T::EPV;
+        uint32_t in = 0u;
+#pragma unroll
+        for (int j = 0; j < T::EPV; ++j) {
+            const uint32_t xb = !BF16 ? w[j] : (j & 1) ? (w[j >> 1] & 0xFFFF0000u) : (w[j >> 1] << 16);
+            in |= (ABOVE ? __uint_as_float(xb) > Tf : __uint_as_float(xb) >= Tf) ? 1u << j : 0u;
+        }
+        if (!ABOVE && in != 0u && (s == 0 || s == pc.nvec - 1)) {  // (places that are nobody's, which only a T of -inf lets in)
+#pragma unroll
+            for (int j = 0; j < T::EPV; ++j)
+                if (e + j < pc.e0 || e + j >= pc.e1) in &= ~(1u << j);
+        }
+        if (in != 0u) {
+            int pos = atomicAdd(&sh->ncand, __popc(in));
+#pragma unroll 1
+            for (; in != 0u; in &= in - 1u, ++pos) {
+                const int j = __ffs(in) - 1;
+                if (pos < Sh::CAP)
+                    sh->cand[pos] = rows_key(ord_from_float(load_elem_f32((const char*)(vec + s) + j * T::ESZ, BF16)), e + j);
+            }
+        }
+    }
+}
+
 // A piece in which more elements reach T than its list holds: leaves the list (in this CTA's memory) with the best K of the
-// piece, in no order, and returns their number (K, or all elements of a shorter piece).  First what lies above T and then
-// elements equal to T in the order of their ids (bulk ties, a vocabulary masked to -inf); if what lies above T overflows too
-// (T is a poor bound: sorted rows), a bound that keeps between K and CAP elements is bisected for, and where one value alone
-// spans that gap its elements are taken in the order of their ids.  All threads of the row; rare, hence out of line.
-// vmax: an image that no element exceeds.
+// piece, in no order, and returns their number (K or more, or all elements of a shorter piece).  First what lies above the bound
+// and then elements equal to it in the order of their ids (bulk ties, a vocabulary masked to -inf or to a low value); if what lies
+// above it overflows too (a poor bound: sorted rows), a bound that keeps between K and CAP elements is bisected for, and where
+// one value alone spans that gap its elements are taken in the order of their ids.  All threads of the row; out of line.
+// cmax: the steps' maxima; vmax: an image that no element exceeds; fresh: nothing has been listed yet.
+//
+// Masked rows are ordinary work, so what lies above the bound is found as in other rows, by the steps' maxima.  (All elements by every
+// thread and, in fp32, a bisection whenever the value of the masked has one of the six bits that T is cut by, took 288 us at V = 151,936,
+// fp32, batch 4, where the streaming kernel takes 14.7.)
 template <bool BF16, int CL, int NT>
-__device__ __noinline__ int rows_select_exact(RowsShared<CL, NT>* sh, const uint4* vec, const RowsPiece pc, uint32_t T, uint32_t vmax,
-                                              uint32_t tmax, int K, uint64_t* list, int tid) {
+__device__ __noinline__ int rows_select_exact(RowsShared<CL, NT>* sh, const uint4* vec, const uint16_t* cmax, const RowsPiece pc, uint32_t T,
+                                              uint32_t vmax, uint32_t tmax, int K, bool fresh, uint64_t* list, int tid) {
     constexpr int CAP = RowsShared<CL, NT>::CAP;
     constexpr int SH = BF16 ? 16 : 0;  // (bf16: images that differ differ in their upper halves)
     const int warp = tid >> 5, lane = tid & 31;
+    // T with the bits that it was cut by: the least of the group maxima that reach it, K or more
+    {
+        uint32_t least = 0xFFFFFFFFu;
+#pragma unroll
+        for (int h = 0; h < kVpGroups / 32; ++h) {
+            uint32_t m = CL > 1 ? 0u : sh->gmax[lane + 32 * h];
+#pragma unroll
+            for (int i = 0; i < (CL > 1 ? CL : 0); ++i) m = max(m, sh->gall[i][lane + 32 * h]);
+            if (m >= T) least = min(least, m);
+        }
+        T = __reduce_min_sync(0xFFFFFFFFu, least);
+    }
+    int n;
+    {
+        // the steps of threads that hold more than T, and their elements
+        if (!fresh) {
+            rows_bar<NT>();
+            if (tid == 0) sh->ncand = sh->nhits = 0;
+            rows_bar<NT>();
+        }
+        const float Tf = __uint_as_float(bits_from_ord(T));
+        const uint32_t tb = __float_as_uint(Tf);
+        // (fp32: a step's maximum is rounded up, so that one whose rounded maximum is T's has to be looked at, unless T itself is that)
+        const uint32_t up = BF16 ? T : ord_from_bits((tb >> 31 ? tb >> 16 : (tb + 0xFFFFu) >> 16) << 16);
+        const bool look = !BF16 && (tb & 0xFFFFu) != 0u;
+        if (tmax > T) {
+            uint32_t steps = 0u;
+            const int ntiles = (pc.nvec + RowsShared<CL, NT>::TILE - 1) / RowsShared<CL, NT>::TILE;
+#pragma unroll 1
+            for (int t = 0; t < ntiles; ++t) {
+                const uint32_t m = ord_from_bits((uint32_t)cmax[t * NT + tid] << 16);
+                bool hit = m > up;
+                if (look && m == up) {
+#pragma unroll
+                    for (int i = 0; i < VEC_PER_LANE; ++i) {
+                        const int s = t * RowsShared<CL, NT>::TILE + i * NT + tid;
+                        if (s < pc.nvec) {
+                            const uint4 x = vec[s];
+                            hit |= __uint_as_float(x.x) > Tf || __uint_as_float(x.y) > Tf || __uint_as_float(x.z) > Tf || __uint_as_float(x.w) > Tf;
+                        }
+                    }
+                }
+                steps |= hit ? 1u << t : 0u;
+            }
+            int pos = atomicAdd(&sh->nhits, __popc(steps));
+#pragma unroll 1
+            for (; steps != 0u; steps &= steps - 1u, ++pos)
+                if (pos < kRowsHits) sh->hits[pos] = (uint16_t)((__ffs(steps) - 1) * NT + tid);
+        }
+        __syncwarp();
+        rows_bar<NT>();
+        const int nhits = sh->nhits;
+        if (nhits <= kRowsHits) rows_take_hits<BF16, true>(sh, vec, pc, nhits, Tf, tid);
+        __syncwarp();
+        rows_bar<NT>();
+        n = nhits <= kRowsHits ? sh->ncand : CAP + 1;
+    }
     // the elements whose image reaches `least`, to the list; their number
     auto collect = [&](uint32_t least) {
         rows_bar<NT>();
@@ -181,7 +279,10 @@ __device__ __noinline__ int rows_select_exact(RowsShared<CL, NT>* sh, const uint
         return sh->ncand;
     };
     uint32_t lo = T >> SH, hi = 0u;  // more than CAP elements reach lo, fewer than K reach hi (0: not looked for yet)
-    int n = collect(((lo + 1u) << SH));
+    if (n > CAP) {
+        n = collect((lo + 1u) << SH);
+        if (n <= CAP && n >= K) return n;
+    }
     if (n > CAP) {
         if (tid == 0) sh->count[0] = sh->count[1] = 0;
         rows_bar<NT>();
@@ -218,7 +319,7 @@ __device__ __noinline__ int rows_select_exact(RowsShared<CL, NT>* sh, const uint
     }
     if (n >= K) return n;
     // the first K - n elements equal to the value of lo, by id
-    const uint32_t tie = lo;
+    const uint32_t tie = lo, tie_ord = SH == 0 ? lo : lo >> 15 ? lo << 16 : (lo << 16) | 0xFFFFu;
 #pragma unroll 1
     for (int s0 = 0; s0 < pc.nvec && n < K; s0 += NT) {  // (uniform)
         const int s = s0 + tid;
@@ -250,8 +351,7 @@ __device__ __noinline__ int rows_select_exact(RowsShared<CL, NT>* sh, const uint
 #pragma unroll 1
         for (; eq != 0u && n + before < K; eq &= eq - 1u, ++before) {
             const int j = __ffs(eq) - 1;
-            const float z = load_elem_f32((const char*)(vec + s) + j * VT<BF16>::ESZ, BF16);
-            list[n + before] = rows_key(ord_from_float(z), pc.e_vec0 + s * VT<BF16>::EPV + j);
+            list[n + before] = rows_key(tie_ord, pc.e_vec0 + s * VT<BF16>::EPV + j);
         }
         n = n + total < K ? n + total : K;
         rows_bar<NT>();
@@ -459,13 +559,17 @@ __global__ void __launch_bounds__(NT + 32, NT == 256 ? 4 : 2) vocab_rows_kernel(
         if ((tid & 3) == 0) {
             if (r == p.K - 1) sh->T = mine & ~low;
             if (r == 0) sh->gmost = mine | low;
+            if (r == kVpGroups - 1) sh->gleast = mine & ~low;
         }
     }
     rows_bar<NT>();
     // ------------------------------ candidates -----------------------------------------------------
     const uint32_t Tv = sh->T;
+    // Where the least of the groups holds T too, the rest of the row is one value (masked tokens) or nearly so: such rows go to
+    // rows_select_exact at once.
+    const bool tied = sh->gleast == Tv;
     // A list of the steps of threads that reach T, about K + 12 in the row, ...
-    {
+    if (!tied) {
         uint32_t steps = 0u;
         if (tmax >= Tv) {
 #pragma unroll 4
@@ -476,41 +580,13 @@ __global__ void __launch_bounds__(NT + 32, NT == 256 ? 4 : 2) vocab_rows_kernel(
             for (; steps != 0u; steps &= steps - 1u, ++pos)
                 if (pos < kRowsHits) sh->hits[pos] = (uint16_t)((__ffs(steps) - 1) * NT + tid);
         }
+        rows_bar<NT>();
     }
-    rows_bar<NT>();
-    const int nhits = sh->nhits;
+    const int nhits = tied ? 0 : sh->nhits;
     // (the same order but for NaN, which makes a row bad anyway; cut off below -inf the image is not a number's)
     const float Tf = Tv <= 0x007FFFFFu ? -INFINITY : __uint_as_float(bits_from_ord(Tv));
     // ... and their elements, a vector a thread.
-#pragma unroll 1
-    for (int i = tid; i < (nhits <= kRowsHits ? nhits * VEC_PER_LANE : 0); i += NT) {
-        const uint32_t at = sh->hits[i / VEC_PER_LANE];
-        const int s = (int)(at / NT) * Sh::TILE + (i % VEC_PER_LANE) * NT + (int)(at % NT);
-        if (s >= pc.nvec) continue;
-        const uint4 x = vec[s];
-        const uint32_t w[4] = {x.x, x.y, x.z, x.w};
-        const int e = pc.e_vec0 + s * T::EPV;
-        uint32_t in = 0u;
-#pragma unroll
-        for (int j = 0; j < T::EPV; ++j) {
-            const uint32_t xb = !BF16 ? w[j] : (j & 1) ? (w[j >> 1] & 0xFFFF0000u) : (w[j >> 1] << 16);
-            in |= __uint_as_float(xb) >= Tf ? 1u << j : 0u;
-        }
-        if (in != 0u && (s == 0 || s == pc.nvec - 1)) {  // (places that are nobody's, which only a T of -inf lets in)
-#pragma unroll
-            for (int j = 0; j < T::EPV; ++j)
-                if (e + j < pc.e0 || e + j >= pc.e1) in &= ~(1u << j);
-        }
-        if (in != 0u) {
-            int pos = atomicAdd(&sh->ncand, __popc(in));
-#pragma unroll 1
-            for (; in != 0u; in &= in - 1u, ++pos) {
-                const int j = __ffs(in) - 1;
-                if (pos < Sh::CAP)
-                    sh->cand[pos] = rows_key(ord_from_float(load_elem_f32((const char*)(vec + s) + j * T::ESZ, BF16)), e + j);
-            }
-        }
-    }
+    rows_take_hits<BF16, false>(sh, vec, pc, nhits <= kRowsHits ? nhits : 0, Tf, tid);
     if (warp == Sh::WARPS - 1 && rank == 0) {
         // meanwhile, one warp: the log-sum-exp
         constexpr int N = CL * Sh::WARPS, H = (N + 31) / 32;
@@ -541,10 +617,10 @@ __global__ void __launch_bounds__(NT + 32, NT == 256 ? 4 : 2) vocab_rows_kernel(
             sh->lse_d = vp_lse((double)cm, S, __uint_as_float(bits_from_ord(vm)));
         }
     }
-    rows_bar<NT>();
-    int n = sh->ncand;
-    if (n > Sh::CAP || nhits > kRowsHits) {  // (uniform)
-        n = rows_select_exact<BF16, CL, NT>(sh, vec, pc, Tv, sh->gmost, tmax, p.K, sh->cand, tid);
+    if (!tied) rows_bar<NT>();
+    int n = tied ? 0 : sh->ncand;
+    if (tied || n > Sh::CAP || nhits > kRowsHits) {  // (uniform)
+        n = rows_select_exact<BF16, CL, NT>(sh, vec, cmax, pc, Tv, sh->gmost, tmax, p.K, tied, sh->cand, tid);
         rows_bar<NT>();
     }
     if (CL > 1) {

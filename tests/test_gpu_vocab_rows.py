@@ -129,3 +129,68 @@ def test_a_nan_among_masked_tokens_is_reported(batch, V, dtype):
     o_ids, _, _, o_st = oracle.vocab_pass(z[:8], K)
     assert np.array_equal(o_st, bad[:8])
     assert np.array_equal(out[0].cpu().numpy().reshape(-1, K)[:8][bad[:8] == 0], o_ids[bad[:8] == 0])
+
+
+def _masked(batch, L, V, dtype, value, keep, g):
+    z = torch.full((batch * L, V), value)
+    for r in range(batch * L):
+        at = torch.randperm(V, generator=g)[:keep]
+        z[r, at] = torch.randn(keep, generator=g)
+    if value > -float("inf"):  # elements just above and just below the value of the masked
+        up = torch.tensor(value, dtype=dtype)
+        z[0, V // 2] = torch.nextafter(up, torch.tensor(0.0, dtype=dtype)).float()
+        z[1, ::7] = torch.nextafter(up, torch.tensor(-float("inf"), dtype=dtype)).float()
+    return z.to(dtype).view(batch, L, V)
+
+
+def _outputs(batch, L, K):
+    return (torch.empty((batch, L, K), dtype=torch.int32, device="cuda"), torch.empty((batch, L, K), device="cuda"),
+            torch.empty((batch, L), device="cuda"), torch.empty((batch, L), dtype=torch.int32, device="cuda"))
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("value", [-float("inf"), -1e4, -17.3])
+@pytest.mark.parametrize("V,keep", [(20011, 5), (20011, 40), (75000, 40), (130003, 5), (130003, 300)])
+def test_masked_rows(V, keep, value, dtype):
+    """Rows in which all but a few tokens hold one low value: fewer of them than K, a few more, more than the list takes."""
+    from paper_2608_20375_b200 import Graft
+    batch, L, K = 2, 4, 32
+    z = _masked(batch, L, V, dtype, value, keep, torch.Generator().manual_seed(keep))
+    gr = Graft(V, L, K, 16, 8, batch, 8, 8, 8, 0.0, 1, 1 if dtype == torch.bfloat16 else 0, 0)
+    out = _outputs(batch, L, K)
+    gr.vocab_pass(z.cuda(), *out)
+    torch.cuda.synchronize()
+    o_ids, o_lp, o_lse, o_st = oracle.vocab_pass(z.view(batch * L, V), K)
+    assert np.array_equal(out[3].cpu().numpy().reshape(-1), o_st)
+    assert np.array_equal(out[0].cpu().numpy().reshape(-1, K), o_ids)
+    a, b = out[1].cpu().numpy().reshape(-1, K).astype(np.float64), o_lp.astype(np.float64)
+    fin = np.isfinite(b)
+    assert np.array_equal(np.isneginf(a), np.isneginf(b)) and np.all(np.abs(a[fin] - b[fin]) <= tolerance(b[fin]))
+    assert np.all(np.abs(out[2].cpu().numpy().reshape(-1) - o_lse) <= tolerance(o_lse))
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("batch,V", [(2, 151936), (16, 16000)])
+@pytest.mark.parametrize("value", [-float("inf"), -1e4])
+def test_masked_rows_take_no_longer_than_others(batch, V, value, dtype):
+    """... or not much; by bisection 2 to 20 times as long."""
+    from paper_2608_20375_b200 import Graft
+    L, K = 16, 32
+    gr = Graft(V, L, K, 16, 8, batch, 8, 8, 8, 0.0, 1, 1 if dtype == torch.bfloat16 else 0, 0)
+    out = _outputs(batch, L, K)
+    z = (2.0 * torch.randn((batch, L, V), device="cuda")).to(dtype)
+    keep = torch.zeros((batch, L, V), dtype=torch.bool, device="cuda")
+    keep.scatter_(2, torch.randint(0, V, (batch, L, 40), device="cuda"), True)
+    times = []
+    for x in (z, z.masked_fill(~keep, value)):
+        a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+        best = float("inf")
+        for _ in range(5):
+            a.record()
+            for _ in range(20):
+                gr.vocab_pass(x, *out)
+            b.record()
+            b.synchronize()
+            best = min(best, a.elapsed_time(b))
+        times.append(best)
+    assert times[1] < 2.0 * times[0], times
