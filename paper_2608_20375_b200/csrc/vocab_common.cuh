@@ -96,7 +96,10 @@ __device__ __forceinline__ float ex2_whole(float d) { return d < -126.f ? 0.f : 
 template <bool BF16, bool WHOLE = false>
 __device__ __forceinline__ void acc_raise(Acc& a, float cm) {
     const float cms = WHOLE ? ceilf(cm * kLog2e) : cm * kLog2e;
-    if (!(cms > a.ref + 16.0f)) return;  // (the threshold is a truncated copy of ref + 16: it may fire a little early)
+    if (!(cms > a.ref + 16.0f)) return;  // (the threshold is a copy of ref + 16 rounded down: it may fire a little early)
+    // Masked tokens may hold any low value.  Below -1e9 the product with log2(e) is rounded by hundreds and more, by which the terms
+    // of a sum at that reference would overflow; they add nothing to a row that has any other value and are left out.
+    if (cms < 0.f && fmaf(cm, kLog2e, -cms) > 100.0f) return;
     const float f = WHOLE ? ex2_whole(a.ref - cms) : ex2_approx(a.ref - cms);  // 0 when ref is -inf (nothing added yet) or cm is +inf
 #if GRAFT_VP_F32X2
     const uint64_t f2 = pack2(f, f);
@@ -110,10 +113,13 @@ __device__ __forceinline__ void acc_raise(Acc& a, float cm) {
 #endif
     a.ref = cms;
     a.nref = -cms;
-    // values above (ref + 16) / log2e raise the reference again; the bound need not be exact (terms overflow only
-    // 2^111 above it), so it is kept as its leading 16 bits for the packed comparison of bf16 chunks
-    const uint32_t zb = __float_as_uint((cms + 16.0f) * 0.6931471805599453f);
-    a.thr = BF16 ? ((zb >> 16) | (zb & 0xFFFF0000u)) : zb;
+    // values above (ref + 16) / log2e raise the reference again; the bound need not be exact (terms overflow only 2^111 above it), so
+    // it is kept as its leading 16 bits for the packed comparison of bf16 chunks, always rounded down: neighbours among values
+    // below -8192 (bf16) or -1e9 are further apart than that
+    const float z = (cms + 16.0f) * 0.6931471805599453f;
+    const uint32_t zb = __float_as_uint(fmaf(fabsf(z), -0x1p-22f, z));
+    const uint32_t z16 = (zb + (zb >> 31 ? 0xFFFFu : 0u)) >> 16;
+    a.thr = BF16 ? (z16 | (z16 << 16)) : zb;
 }
 
 __device__ __forceinline__ float pair_max_bf16(uint32_t pm) {  // the larger half of a packed bf16 pair, as fp32

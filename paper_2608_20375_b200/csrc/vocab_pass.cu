@@ -744,8 +744,7 @@ __global__ void __launch_bounds__(kVpThreads, 1) vocab_pass_kernel(const VpParam
                             // |x| = 30, which is the whole error of the row when its largest logit sits here)
                             float c1 = __fmul_rn(x, kLog2e);
                             float s1 = fmaf(fmaf(x, kLog2e, -c1), 0.69314718f, 1.0f);
-                            if (x == -INFINITY) {
-                                c1 = -INFINITY;
+                            if (c1 == -INFINITY) {  // (-inf, or a finite value whose term is 0 and whose remainder is infinite)
                                 s1 = 0.f;
                             } else if (!(x < INFINITY)) {
                                 s1 = NAN;  // +inf or NaN poisons the sum and marks the row

@@ -194,3 +194,37 @@ def test_masked_rows_take_no_longer_than_others(batch, V, value, dtype):
             best = min(best, a.elapsed_time(b))
         times.append(best)
     assert times[1] < 2.0 * times[0], times
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("value", ["lowest", -1e30, -1e10, -1e9, -3e4])
+@pytest.mark.parametrize("batch,V,shift", [(2, 20011, 1), (2, 75011, 3), (1, 130003, 1), (20, 150001, 1)])
+def test_rows_masked_far_below(batch, V, shift, value, dtype):
+    """Low values whose product with log2(e) is infinite or rounded by more than an exponent holds, with neighbours a spacing or
+    a few apart, at the ragged ends of rows too: nothing is wrong with such rows."""
+    from paper_2608_20375_b200 import Graft
+    L, K, n = 8, 32, 8
+    low = torch.tensor(torch.finfo(dtype).min if value == "lowest" else value, dtype=dtype)
+    z = _masked(1, n, V, dtype, low.item(), 40, torch.Generator().manual_seed(9)).view(n, V)
+    if value == "lowest":
+        z[1] = z[0]  # (_masked puts infinities beside its second row's values)
+    for r in range(2, 5):  # the masked of the row's second half a spacing up, two, three
+        up = low
+        for _ in range(r - 1):
+            up = torch.nextafter(up, torch.tensor(0.0, dtype=dtype))
+        half = z[r, V // 2:]
+        half[half == low] = up
+    flat = torch.empty(batch * L * V + 8, dtype=dtype, device="cuda")
+    x = flat[shift:shift + batch * L * V].view(batch, L, V)
+    x.copy_(z.cuda().expand(batch, L, V))
+    gr = Graft(V, L, K, 16, 8, batch, 8, 8, 8, 0.0, 1, 1 if dtype == torch.bfloat16 else 0, 0)
+    out = _outputs(batch, L, K)
+    gr.vocab_pass(x, *out)
+    torch.cuda.synchronize()
+    o_ids, o_lp, o_lse, o_st = oracle.vocab_pass(z, K)
+    assert not o_st.any()
+    for b in range(batch):
+        assert np.array_equal(out[3][b].cpu().numpy(), o_st)
+        assert np.array_equal(out[0][b].cpu().numpy(), o_ids)
+        assert np.all(np.abs(out[1][b].cpu().numpy().astype(np.float64) - o_lp) <= tolerance(o_lp))
+        assert np.all(np.abs(out[2][b].cpu().numpy() - o_lse) <= tolerance(o_lse))
