@@ -1308,7 +1308,7 @@ static size_t rows_smem_bytes(long long row_bytes, int cl, int nt) {
 }
 // CTAs of a size that an SM holds side by side (threads and registers allow four of 256 threads, two of 512)
 static int rows_per_sm(long long row_bytes, int cl, int nt) {
-    if (row_bytes / cl > kRowsMaxBytes) return 0;
+    if (rows_vecs(row_bytes, cl) > kRowsMaxBytes / 16) return 0;  // (barriers for so many tiles)
     const int n = (int)(227 * 1024 / (rows_smem_bytes(row_bytes, cl, nt) + 1024)), most = nt == 512 ? 2 : 4;
     return n < most ? n : most;
 }

@@ -32,7 +32,7 @@ namespace {
 
 // NT threads work on a row (or a piece of it), four 16-byte vectors each a step; one warp more: copies, cosines.
 constexpr int rows_tile_vecs(int nt) { return nt * VEC_PER_LANE; }
-constexpr int kRowsMaxBytes = 224 * 1024;       // the longest piece
+constexpr int kRowsMaxBytes = 224 * 1024;       // the longest piece, the vectors of its ragged ends among it
 
 constexpr int kRowsHits = 512;                  // steps of threads that can reach T before the exact selection takes over
 
@@ -58,6 +58,7 @@ template <int CL, int NT>
 struct __align__(16) RowsShared {
     static constexpr int CAP = rows_cap(CL);
     static constexpr int WARPS = NT / 32, TILE = rows_tile_vecs(NT), MAX_TILES = kRowsMaxBytes / (16 * TILE);
+    static_assert(kRowsMaxBytes % (16 * TILE) == 0 && MAX_TILES <= 32, "a barrier a tile, a bit a tile");
     uint64_t cand[CL * CAP];   // this CTA's candidates; in the end, in the first CTA, the row's
     uint64_t in[CL > 1 ? CL : 1][CL > 1 ? CAP : 1];  // the first CTA's: every CTA's candidates
     uint64_t outk[kMaxK];
