@@ -137,11 +137,15 @@ int32_t graft_edge_rows(const graft_ctx* ctx);
  * With d_emb and d_out 16-byte aligned and E a multiple of 8 (bf16) or 4 (fp32) the products run on the tensor cores:
  * W beside bf16 embeddings enters as three bf16 parts, fp32 embeddings and their W as two scaled fp16 parts each; products of
  * parts are exact.  Against a chain of fp32 multiply-adds the result differs by the order and the rounding of the additions
- * and, for fp32 embeddings, by the products left out, below 2^-24 of a term (largest error against fp64 products of N(0, 1)
- * results 3.4e-6 at E = 4096, 2.2e-6 at E = 2048 in fp32; the chain: 1.2e-5).  With fp32 embeddings, rows whose largest entry is
- * over 2^7 times larger or 2^18 times smaller than most rows' are worked out by such a chain, more slowly; other entries are held to
- * 22 bits or 2^-26 of their row's largest, those of W to 22 bits or 2^-50; infinities and values up to the largest fp32 give what
- * fp32 arithmetic gives.  A
+ * and, for fp32 embeddings, by what two parts do not hold of a number (below 2^-23 of it) and by the products of second parts, which
+ * are left out (below 2^-22 of a term, 2^-24.6 root mean square).  Errors against fp64 products, largest and root mean square, over
+ * the size of the results, and a chain's at the same inputs: N(0, 1) bf16 embeddings at E = 4096 3.4e-6 and 4.8e-7 (1.7e-5 and 1.1e-6),
+ * fp32 at E = 2048 2.2e-6 and 3.5e-7 (9.2e-6 and 8.1e-7), the latter with all terms of one sign 1.5e-6 and 1.1e-6 (3.6e-6 and 6.5e-7).
+ * fp32 embeddings are scaled row by row, by the largest entry of a row's first 32 columns (of a worker's first 32, where workers
+ * share a row).  Rows with an entry over 2^11 times larger than that, or with eight entries side by side that are not zero and all over
+ * 2^16 times smaller, are worked out by fp32 multiply-adds, more slowly (V = 32,000, E = 2048: 0.84 ms a tower if all are, 0.09
+ * if none is).  Other rows' entries are held to 2^-23 of themselves or 2^-24 of the largest of the eight beside them, those of W to 2^-23
+ * or 2^-50 of their row's largest; infinities and values up to the largest fp32 give what fp32 arithmetic gives.  A
  * bf16 embedding or a W beside bf16 embeddings that is infinite, or a W that rounds past the largest bf16, gives NaN.
  * Such calls use scratch of the context (3 m E 16-bit values, V m / 128 bytes and up to 40 MB of partial sums, m rounded up to 128), which the
  * first of them allocates and one that needs more replaces -- under stream capture too; a captured call keeps the scratch it

@@ -4,9 +4,10 @@
 // Operands are 16-bit parts of the inputs; products of parts are exact in the fp32 accumulator.
 //   bf16 embeddings: out = e W1 + e W2 + e W3, W as three bf16 parts (8 + 8 + 8 mantissa bits; three products a step)
 //   fp32 embeddings: out = e1 W1 + (e1 W2 + e2 W1), both as two fp16 parts (11 + 11 bits and the second part's sign; what is
-//     dropped, e2 W2, is below 2^-24 of a term and 2^-26 of it on average).  fp16 has few exponents, so a row of W is scaled by
-//     its largest entry and the embeddings by a power of two from a sample; second parts are kept times 2^11, and go to an
-//     accumulator of their own.  Rows of the embeddings that this does not suit are worked out in fp32.
+//     dropped, e2 W2, is below 2^-22 of a term, 2^-24.6 root mean square).  fp16 has few exponents, so a row of W is scaled by
+//     its largest entry and a row of the embeddings by the largest of its first block; second parts are kept times 2^11, and go to
+//     an accumulator of their own (H. Ootomo and R. Yokota, "Recovering single precision accuracy from Tensor Cores while surpassing
+//     the FP32 theoretical peak performance", 2022).  Rows of the embeddings that this does not suit are worked out in fp32.
 // so the result differs from an fp32 GEMM by the order and the rounding of the additions.  The accumulators of the tensor
 // cores round less carefully than an FMA chain, the less so the more bits the products have: they are emptied into fp32
 // registers after 32 (bf16) or 16 (fp32 embeddings) additions to the large products' accumulators, which the small products do not
@@ -29,13 +30,15 @@
 // written.  What is left when the tiles do not divide by the workers is dealt out along E in shares, whose sums a
 // small kernel adds up in order (summing them inside, by the warp that came last, stalled its tile: 462 against 370 us).
 //
-// Measured (one tower, back to back, B200): V = 151,936, E = 4096, m = 128, bf16: 358 us (375 before rows and W shared a barrier
+// Measured (one tower, back to back, B200): V = 151,936, E = 4096, m = 128, bf16: 355 us (376 before rows and W shared a barrier
 // and the first row block went two blocks ahead where accumulators are emptied; 798 us with the library template's GEMMs); its products
-// take 287 us at the measured dense rate, and the clock falls to 1.5 GHz on the way.  V = 32,000, E = 2048, fp32: 91 us (121 with
-// three bf16 parts, seven products; 1180 us by the FMA kernel).  What bounds the fp32 kernel: the one thread that issues, 0.6 k
+// take 287 us at the measured dense rate, and the clock falls to 1.5 GHz on the way.  V = 32,000, E = 2048, fp32: 88 us (120 with
+// three bf16 parts, seven products; 1135 us by the FMA kernel).  What bounds the fp32 kernel: the one thread that issues, 0.6 k
 // cycles a block of 32 columns beside 0.4 k of products, and the eight warps that split.  Error against fp64 products at those
-// sizes, largest and root mean square over the results' size: bf16 2.7e-6 and 4.7e-7; fp32 2.2e-6 and 3.4e-7 (bf16 parts 2.7e-6 and 4.7e-7; FMA kernel
-// 1.2e-5 at most).
+// sizes, largest and root mean square over the results' size: bf16 3.4e-6 and 4.8e-7 (FMA kernel 1.7e-5, 1.1e-6); fp32 2.2e-6 and
+// 3.5e-7 (three bf16 parts 3.3e-6, 4.7e-7; FMA kernel 9.2e-6, 8.1e-7).  The accumulators round towards zero, so terms of one sign
+// are off by more: fp32 1.5e-6 and 1.1e-6 (8.0e-7 and 3.9e-7; 3.6e-6 and 6.5e-7), emptied every 8 additions 8.5e-7 and 4.7e-7 in 93
+// us instead of 89.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
@@ -71,6 +74,14 @@ struct TablesCfg {
 };
 
 constexpr float kTmLow = 2048.0f;  // fp16: second parts are kept times 2^11
+// fp32 embeddings: a row is multiplied by the power of two that takes the largest entry of its first block (in a piece of a tile: of the
+// piece's first block) to [16, 32).  Two parts hold a number up to 65504 to 2^-23 of it or to 2^-36, whichever is more; where the
+// largest of eight entries side by side is 2^-12 or more, that is 2^-23 of themselves or 2^-24 of that largest.  So the rest of a row may
+// be 2^11 times larger than its first block, and any eight entries 2^16 times smaller.  (With one scale for the table, one column 300
+// times larger than the others left 40 % of the rows to tables_mend's forerunner.)
+constexpr int kTmTarget = 4;
+constexpr float kTmLeast = 0x1p-12f, kTmMost = 65504.f;
+constexpr uint32_t kTmScales = 4;  // tiles whose rows' scales are kept
 
 // A walk over the N stages of a ring: stages passed so far, the stage, the parity to wait for.
 template <uint32_t N>
@@ -109,7 +120,6 @@ struct __align__(64) TablesParams {
     float* pieces;      // [pairs][2 pieces][ROWS][128]
     // fp32 embeddings only
     const float2* unscale;  // [m_pad] what a column's sums are multiplied by, as two factors
-    const float* scale;     // [1] what the embeddings are multiplied by
     uint8_t* bad_row;       // [tiles][ROWS] rows whose entries fp16 parts do not hold well enough, as the tile's workers saw them
     int32_t* errflag;
     int V, E, m, m_pad, n_mb, n_kb;
@@ -186,98 +196,55 @@ __global__ void __launch_bounds__(256) weight_split_kernel(const float* __restri
 
 // 2^x for a whole number x, as far as fp32 has it
 __device__ __forceinline__ float tables_exp2(int x) { return __uint_as_float((uint32_t)(127 + (x < -126 ? -126 : x > 127 ? 127 : x)) << 23); }
+// What a row is multiplied by whose first block's largest magnitude is m (zero: 1)
+__device__ __forceinline__ float tables_row_scale(float m) {
+    const int s = m > 0.f ? 127 + kTmTarget - (int)(__float_as_uint(m) >> 23) : 0;
+    return tables_exp2(s < -120 ? -120 : s > 120 ? 120 : s);
+}
+// 2^-s as a product of two factors: results are multiplied by a row's and a column's, and none of the steps leaves fp32 before the result does
+__device__ __forceinline__ float2 tables_unscale(int s) { return make_float2(tables_exp2(-s / 2), tables_exp2(-s - -s / 2)); }
 
 // W (fp32, [m, E]) -> two fp16 parts [2][m_pad][E_pad], zero where padded: a row is multiplied by the power of two that takes
-// its largest entry to [2^13, 2^14), W1 is what fp16 holds of it and W2 what it holds of the rest, times 2^11.  Every block
-// (a row each) also looks at a sample of the embeddings, the same sample: the power of two that takes the median of 256 threads'
-// largest entries to [2^8, 2^9) is what they will be multiplied by, so that rows up to 2^8 times larger or smaller stay within fp16's
-// exponents.  And clears the flags of rows that do not.
-__global__ void __launch_bounds__(256) weight_split16_kernel(const float* __restrict__ W, const float* __restrict__ emb, int V, int m, int E,
-                                                           int m_pad, int E_pad, __half* __restrict__ w, float2* __restrict__ unscale,
-                                                           float* __restrict__ scale, uint32_t* __restrict__ flags, int n_flags) {
+// its largest entry to [2^13, 2^14), W1 is what fp16 holds of it and W2 what it holds of the rest, times 2^11.  A block a row.  And
+// clears the flags of the embeddings' rows.
+__global__ void __launch_bounds__(256) weight_split16_kernel(const float* __restrict__ W, int m, int E, int m_pad, int E_pad,
+                                                           __half* __restrict__ w, float2* __restrict__ unscale,
+                                                           uint32_t* __restrict__ flags, int n_flags) {
     __shared__ float s_max[8];
-    __shared__ int s_hist[256];
-    __shared__ int s_mid;
     pdl_launch_dependents();
     const int r = blockIdx.x, tid = threadIdx.x;
-    s_hist[tid] = 0;
-    if (tid == 0) s_mid = 127 + 8;  // (nothing but zeros: scale 1)
+    // the row's largest finite entry; up to E = 4096 the row stays in registers
+    constexpr int N = 16;
+    const float* const src = W + (size_t)(r < m ? r : 0) * E;
+    const bool kept = E <= N * 256;
+    float x[N], top = 0.f;
+#pragma unroll
+    for (int i = 0; i < N; ++i) x[i] = r < m && tid + 256 * i < E ? src[tid + 256 * i] : 0.f;
+#pragma unroll
+    for (int i = 0; i < N; ++i) top = fmaxf(top, fabsf(x[i]) < INFINITY ? fabsf(x[i]) : 0.f);
+    if (r < m && !kept)
+        for (int e = N * 256 + tid; e < E; e += 256) top = fmaxf(top, fabsf(src[e]) < INFINITY ? fabsf(src[e]) : 0.f);
     for (int i = r * 256 + tid; i < n_flags; i += (int)gridDim.x * 256) flags[i] = 0u;
-    // the sample: four pieces of 16 bytes a thread, from a row of its own
-    float x = 0.f;
-    {
-        const size_t row = (size_t)((long long)tid * V / 256) * E;
-        const int n4 = E / 4;
-        float4 v[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-            v[i] = __ldg((const float4*)(emb + row) + (int)((long long)(tid * 4 + i) * 37 % n4));
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const float q[4] = {fabsf(v[i].x), fabsf(v[i].y), fabsf(v[i].z), fabsf(v[i].w)};
-#pragma unroll
-            for (int k = 0; k < 4; ++k)
-                if (q[k] < INFINITY) x = fmaxf(x, q[k]);
-        }
-    }
-    // the row's largest finite entry
-    float top = 0.f;
-    if (r < m)
-        for (int e = tid; e < E; e += 256) {
-            const float a = fabsf(W[(size_t)r * E + e]);
-            if (a < INFINITY) top = fmaxf(top, a);
-        }
     top = __uint_as_float(__reduce_max_sync(0xFFFFFFFFu, __float_as_uint(top)));
     if ((tid & 31) == 0) s_max[tid >> 5] = top;
     __syncthreads();
-    const int ex = (int)(__float_as_uint(x) >> 23);  // (biased; 0: zero or denormal)
-    if (ex > 0) atomicAdd(&s_hist[ex], 1);
 #pragma unroll
     for (int i = 0; i < 8; ++i) top = fmaxf(top, s_max[i]);
-    __syncthreads();
-    if (tid < 32) {
-        int own = 0;
-#pragma unroll
-        for (int i = 0; i < 8; ++i) own += s_hist[8 * tid + i];
-        int upto = own;
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const int o = __shfl_up_sync(0xFFFFFFFFu, upto, d);
-            if (tid >= d) upto += o;
-        }
-        const int half = (__shfl_sync(0xFFFFFFFFu, upto, 31) + 1) / 2;  // the median is where the count reaches this
-        if (half > 0 && upto >= half && upto - own < half) {
-            int c = upto - own;
-            for (int i = 0; i < 8; ++i) {
-                c += s_hist[8 * tid + i];
-                if (c >= half) {
-                    s_mid = 8 * tid + i;
-                    break;
-                }
-            }
-        }
-    }
-    __syncthreads();
-    int s = 127 + 8 - s_mid;
-    s = s < -120 ? -120 : s > 120 ? 120 : s;
     int k = top > 0.f ? 13 + 127 - (int)(__float_as_uint(top) >> 23) : 0;
     k = k > 126 ? 126 : k;
-    if (tid == 0) {
-        const int t = -(k + s), t1 = t / 2;
-        unscale[r] = make_float2(tables_exp2(t1), tables_exp2(t - t1));
-        if (r == 0) *scale = tables_exp2(s);
-    }
+    if (tid == 0) unscale[r] = tables_unscale(k);
     const float f = tables_exp2(k);
     const size_t part = (size_t)m_pad * E_pad;
-    for (int e = tid * 2; e < E_pad; e += 512) {
-        const float x0 = (r < m && e < E) ? W[(size_t)r * E + e] * f : 0.f;
-        const float x1 = (r < m && e + 1 < E) ? W[(size_t)r * E + e + 1] * f : 0.f;
-        const __half2 a = __floats2half2_rn(x0, x1);
-        const __half2 b = __floats2half2_rn((x0 - __low2float(a)) * kTmLow, (x1 - __high2float(a)) * kTmLow);
-        __half* dst = w + (size_t)r * E_pad + e;
-        *(__half2*)dst = a;
-        *(__half2*)(dst + part) = b;
-    }
+    __half* const dst = w + (size_t)r * E_pad;
+    auto put = [&](int e, float v) {
+        const __half a = __float2half_rn(v * f);
+        dst[e] = a;
+        dst[part + e] = __float2half_rn((v * f - __half2float(a)) * kTmLow);
+    };
+#pragma unroll
+    for (int i = 0; i < N; ++i)
+        if (tid + 256 * i < E_pad) put(tid + 256 * i, x[i]);
+    for (int e = N * 256 + tid; e < E_pad; e += 256) put(e, r < m && e < E ? src[e] : 0.f);
 }
 
 __device__ __forceinline__ uint32_t cvt_f16x2(float lo, float hi) {
@@ -293,11 +260,6 @@ __device__ __forceinline__ void split2(float x0, float x1, float scale, uint32_t
     const float2 z = __fmul2_rn(make_float2(x.x - y.x, x.y - y.y), make_float2(kTmLow, kTmLow));
     b = cvt_f16x2(z.x, z.y);
 }
-// Is a row whose largest magnitude is m held well enough by the two parts, once scaled?  They are off by 2^-36 at most where fp16 has no
-// more bits below them: 2^-26 of the largest entry if that is 2^-10 or more.  Or the row is zero.
-__device__ __forceinline__ bool tables_row_ok(float m, float scale) {
-    return m == 0.f || (m * scale >= 0.0009765625f && m * scale <= 65504.f);
-}
 __device__ __forceinline__ void st_shared_v4(uint32_t at, const uint32_t (&v)[4]) {
     asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(at), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]) : "memory");
 }
@@ -312,17 +274,70 @@ __device__ __forceinline__ float4 ld_shared_f4(uint32_t at) {
     return v;
 }
 
-// fp32 embeddings: results that are worked out again as one chain of fp32 multiply-adds, which gives what fp32 arithmetic gives:
-// rows whose entries fp16 parts do not hold well enough (over 2^7 times larger than most rows, or 2^18 times smaller), and whatever is
-// not finite (infinities).  They are rare, so the time does not matter.
-__device__ __forceinline__ bool tables_finite(float x) { return fabsf(x) <= 3.402823466e38f; }
-__device__ __noinline__ float tables_fp32(const TablesParams& p, int v, int c) {
-    const float* e = (const float*)p.emb + (size_t)v * p.E;
-    const float* w = p.W + (size_t)c * p.E;
-    float a = 0.f;
-#pragma unroll 8
-    for (int k = 0; k < p.E; ++k) a = fmaf(__ldg(e + k), __ldg(w + k), a);
-    return a + (p.bias ? p.bias[c] : 0.f);
+// fp32 embeddings: rows that are worked out again by fp32 multiply-adds, which give what fp32 arithmetic gives: rows whose entries fp16
+// parts do not hold well enough, and whatever has results that are not finite (infinities).  32 rows (-1: none) of 128 columns from
+// c0, 256 threads, four rows and four columns each, blocks of 32 columns of E through shared memory, the next on its way meanwhile.  Sums
+// of 256 terms are added up apart, so that the error is no larger than that of the other rows.
+constexpr int kTmMendRows = 32;
+struct __align__(16) TablesMend {
+    float w[32][132], e[32][kTmMendRows + 4];
+    int rows[kTmMendRows];
+};
+__device__ __noinline__ void tables_mend(const TablesParams& p, TablesMend* sm, int c0, int tid) {
+    const int c = c0 + (tid & 31) * 4, r0 = (tid >> 5) * 4;
+    // a warp fetches eight columns of E of four rows of W, four times side by side, then of the next four rows (rows past m: the last)
+    const int wk = tid & 7, wc = (tid >> 5) * 16 + ((tid & 31) >> 3), ek = (tid & 7) * 4, er = tid >> 3;
+    const int e_row = sm->rows[er];
+    const float* const e_src = (const float*)p.emb + (size_t)(e_row < 0 ? 0 : e_row) * p.E;
+    const float* w_src[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) w_src[i] = p.W + (size_t)(c0 + wc + 4 * i < p.m ? c0 + wc + 4 * i : p.m - 1) * p.E + wk;
+    if (e_row >= 0)  // (the rows come from memory, a line a step: all of them on their way at once)
+        for (int k = (tid & 7) * 32; k < p.E; k += 256) asm volatile("prefetch.global.L2 [%0];" ::"l"(e_src + k));
+    float sum[4][4] = {}, part[4][4] = {}, w[16];
+    float4 x;
+    auto fetch = [&](int k0) {
+#pragma unroll
+        for (int i = 0; i < 16; ++i) w[i] = k0 + wk + 8 * (i & 3) < p.E ? __ldg(w_src[i >> 2] + k0 + 8 * (i & 3)) : 0.f;
+        x = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (e_row >= 0 && k0 + ek < p.E) x = __ldg((const float4*)(e_src + k0 + ek));
+    };
+    const bool busy = sm->rows[r0] >= 0;  // (a warp's rows: none without the first)
+    fetch(0);
+    for (int k0 = 0, turn = 1; k0 < p.E; k0 += 32, ++turn) {
+        named_bar_sync(3, 256);  // (what was there before has been read)
+#pragma unroll
+        for (int i = 0; i < 16; ++i) sm->w[wk + 8 * (i & 3)][wc + 4 * (i >> 2)] = w[i];
+        sm->e[ek][er] = x.x, sm->e[ek + 1][er] = x.y, sm->e[ek + 2][er] = x.z, sm->e[ek + 3][er] = x.w;
+        named_bar_sync(3, 256);
+        if (k0 + 32 < p.E) fetch(k0 + 32);
+        if (!busy) continue;
+#pragma unroll 4
+        for (int k = 0; k < 32; ++k) {
+            const float4 wv = *(const float4*)&sm->w[k][(tid & 31) * 4], ev = *(const float4*)&sm->e[k][r0];
+            const float ee[4] = {ev.x, ev.y, ev.z, ev.w}, ww[4] = {wv.x, wv.y, wv.z, wv.w};
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) part[i][j] = fmaf(ee[i], ww[j], part[i][j]);
+        }
+        if (turn % 8 == 0 || k0 + 32 >= p.E) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) sum[i][j] += part[i][j], part[i][j] = 0.f;
+        }
+    }
+    if (c < p.m) {
+        float4 b = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (p.bias) b = make_float4(p.bias[c], p.bias[c + 1], p.bias[c + 2], p.bias[c + 3]);
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            if (sm->rows[r0 + i] >= 0)
+                *(float4*)(p.out + (size_t)sm->rows[r0 + i] * p.m + c) =
+                    make_float4(sum[i][0] + b.x, sum[i][1] + b.y, sum[i][2] + b.z, sum[i][3] + b.w);
+    }
+    named_bar_sync(3, 256);
 }
 
 template <bool F32>
@@ -331,7 +346,9 @@ __global__ void __cluster_dims__(F32 ? 1 : 2, 1, 1) __launch_bounds__(TablesCfg<
     using C = TablesCfg<F32>;
     constexpr uint32_t NS = C::STAGES, NR = C::RAW_STAGES;
     extern __shared__ unsigned char smem_raw[];
-    __shared__ __align__(8) uint64_t bars[2 * (NS + NR) + 4];
+    __shared__ __align__(8) uint64_t bars[2 * (NS + NR) + 4 + 2 * kTmScales];
+    __shared__ uint8_t s_scale[F32 ? kTmScales : 1][128];  // the exponents (biased) of what the rows of the last tiles are multiplied by
+    __shared__ float2 s_unscale[F32 ? 512 : 1];  // what columns are multiplied by (from memory at a tile's end: V = 30,000, E = 32 22.0 us, so 18.5)
     __shared__ uint32_t s_tmem;
     __shared__ volatile int s_abort;
     __shared__ bool s_mend;
@@ -350,7 +367,7 @@ __global__ void __cluster_dims__(F32 ? 1 : 2, 1, 1) __launch_bounds__(TablesCfg<
     // them are done, rfull / rempty: fp32 rows as loaded.  (One barrier for rows and W: the thread that issues the instructions is
     // the bottleneck of short blocks, every wait and every commit costs it a hundred cycles.)
     const uint32_t full0 = smem_u32(bars), empty0 = full0 + 8 * NS, rfull0 = empty0 + 8 * NS, rempty0 = rfull0 + 8 * NR;
-    const uint32_t accfull0 = rempty0 + 8 * NR, accempty0 = accfull0 + 16;
+    const uint32_t accfull0 = rempty0 + 8 * NR, accempty0 = accfull0 + 16, sfull0 = accempty0 + 16, sempty0 = sfull0 + 8 * kTmScales;
     if (tid == 0) {
         for (uint32_t s = 0; s < NS; ++s) {
             mbar_init(full0 + 8 * s, F32 ? kTmConvWarps / 2 + 1 : 1);
@@ -363,6 +380,10 @@ __global__ void __cluster_dims__(F32 ? 1 : 2, 1, 1) __launch_bounds__(TablesCfg<
         for (int s = 0; s < 2; ++s) {
             mbar_init(accfull0 + 8 * s, 1);
             mbar_init(accempty0 + 8 * s, (C::PAIR ? 2 : 1) * kTmEpiWarps);  // (the even CTA's)
+        }
+        for (uint32_t s = 0; s < kTmScales; ++s) {
+            mbar_init(sfull0 + 8 * s, kTmConvWarps / 2);
+            mbar_init(sempty0 + 8 * s, kTmEpiWarps + kTmConvWarps);
         }
         mbar_fence_init();
         s_abort = 0;
@@ -384,10 +405,21 @@ __global__ void __cluster_dims__(F32 ? 1 : 2, 1, 1) __launch_bounds__(TablesCfg<
         const int half = warp >> 2, quarter = warp & 3;
         const uint32_t accempty_even = mapa_u32(accempty0, 0);
         uint32_t cc = 0;  // chunks emptied so far
-        float2 check = make_float2(0.f, 0.f);  // fp32 embeddings: NaN once a result of this thread was not finite
+        if (F32) {
+            for (int c = tid; c < p.m_pad; c += kTmEpiWarps * 32) s_unscale[c] = __ldg(p.unscale + c);
+            named_bar_sync(3, kTmEpiWarps * 32);
+        }
         for (int i = 0; tables_item(p, pair, i, it); ++i) {
             const int rt = it.tile / p.n_mb, mb = it.tile - rt * p.n_mb;
             const uint32_t n = (uint32_t)tables_n<F32>(p, mb);
+            int row_exp = 127;  // (fp32) the exponent of what this thread's row is multiplied by
+            if (F32) {
+                const uint32_t slot = (uint32_t)i % kTmScales;
+                wait(sfull0 + 8 * slot, ((uint32_t)i / kTmScales) & 1u);
+                row_exp = s_scale[slot][quarter * 32 + lane];
+                __syncwarp();
+                if (lane == 0) mbar_arrive(sempty0 + 8 * slot);
+            }
             float acc[C::MT][64];
 #pragma unroll
             for (int h = 0; h < C::MT; ++h)
@@ -434,8 +466,10 @@ __global__ void __cluster_dims__(F32 ? 1 : 2, 1, 1) __launch_bounds__(TablesCfg<
 #pragma unroll
             for (int h = 0; h < C::MT; ++h) {
                 const int v = h * 256 + (int)rank * 128 + quarter * 32 + lane;
+                float2 check = make_float2(0.f, 0.f);  // fp32 embeddings: NaN once a result is not finite
                 if (v < rows) {
                     float* dst = base + (size_t)v * ld + half * 64;
+                    const float2 row_unscale = tables_unscale(row_exp - 127);
 #pragma unroll
                     for (int c = 0; c < 64; c += 8) {
                         if (c >= cols) break;
@@ -443,8 +477,8 @@ __global__ void __cluster_dims__(F32 ? 1 : 2, 1, 1) __launch_bounds__(TablesCfg<
                         if (F32) {
 #pragma unroll
                             for (int k = 0; k < 8; ++k) {
-                                const float2 f = __ldg(p.unscale + mb * 128 + half * 64 + c + k);
-                                acc[h][c + k] = acc[h][c + k] * f.x * f.y;
+                                const float2 f = s_unscale[mb * 128 + half * 64 + c + k];
+                                acc[h][c + k] = acc[h][c + k] * (f.x * row_unscale.x) * (f.y * row_unscale.y);
                             }
                         }
                         if (bias) {
@@ -467,22 +501,42 @@ __global__ void __cluster_dims__(F32 ? 1 : 2, 1, 1) __launch_bounds__(TablesCfg<
                         }
                     }
                 }
+                if (F32 && check.x + check.y != 0.f) {
+                    p.bad_row[(size_t)it.tile * C::ROWS + v] = 1;
+                    s_mend = true;
+                }
             }
         }
         if (F32) {  // (nothing waits for these warps any more)
-            if (check.x + check.y != 0.f) s_mend = true;
             __syncwarp();
-            named_bar_sync(1, (kTmEpiWarps + kTmConvWarps) * 32);  // (the tiles are written, their rows looked at)
+            named_bar_sync(1, (kTmEpiWarps + kTmConvWarps) * 32);  // (the tiles are written, their rows looked at; the rings are done with)
             if (s_mend && !s_abort) {
+                TablesMend* const sm = (TablesMend*)(smem_raw + (a_ring - smem_u32(smem_raw)));
                 for (int i = 0; tables_item(p, pair, i, it); ++i) {
                     if (it.q0 != it.q1) continue;  // (pieces: the kernel that adds them up)
-                    const int rt = it.tile / p.n_mb, c0 = (it.tile - rt * p.n_mb) * 128;
-                    for (int v = rt * C::ROWS + warp; v < p.V && v < (rt + 1) * C::ROWS; v += kTmEpiWarps) {
-                        const bool bad = p.bad_row[(size_t)it.tile * C::ROWS + (v - rt * C::ROWS)] != 0;
-                        for (int c = c0 + lane; c < p.m && c < c0 + 128; c += 32) {
-                            float* o = p.out + (size_t)v * p.m + c;
-                            if (bad || !tables_finite(*o)) *o = tables_fp32(p, v, c);
+                    // the tile's flagged rows, 32 at a time; every warp looks at all flags
+                    uint32_t again[C::ROWS / 32];
+                    int n = 0;
+#pragma unroll
+                    for (int j = 0; j < C::ROWS / 32; ++j) {
+                        again[j] = __ballot_sync(0xFFFFFFFFu, p.bad_row[(size_t)it.tile * C::ROWS + j * 32 + lane] != 0);
+                        n += __popc(again[j]);
+                    }
+                    for (int first = 0; first < n; first += kTmMendRows) {
+                        if (warp == 0) {
+                            sm->rows[lane] = -1;
+                            __syncwarp();
+                            int before = -first;
+#pragma unroll
+                            for (int j = 0; j < C::ROWS / 32; ++j) {
+                                const int at = before + __popc(again[j] & ((1u << lane) - 1u));
+                                if ((again[j] >> lane & 1u) != 0u && at >= 0 && at < kTmMendRows)
+                                    sm->rows[at] = it.tile / p.n_mb * C::ROWS + j * 32 + lane;
+                                before += __popc(again[j]);
+                            }
                         }
+                        named_bar_sync(3, kTmEpiWarps * 32);
+                        tables_mend(p, sm, it.tile % p.n_mb * 128, tid);
                     }
                 }
             }
@@ -635,25 +689,58 @@ __global__ void __cluster_dims__(F32 ? 1 : 2, 1, 1) __launch_bounds__(TablesCfg<
         static_assert(!F32 || (NR % 2 == 0 && NS % 2 == 0), "a stage of either ring belongs to one half of the converting warps");
         const int ct = (tid - (kTmEpiWarps + 3) * 32) & 127, half = (tid - (kTmEpiWarps + 3) * 32) >> 7;
         const int c8 = ct & 3, r0 = ct >> 2;  // columns 8 c8 .. 8 c8 + 7 of rows r0, r0 + 32, r0 + 64 and r0 + 96
-        const float scale = *p.scale;
         TablesRing<NS> a(1);
         TablesRing<NR> r(0);
+        float4 x[4][2];
+        auto load = [&]() {
+            wait(rfull0 + 8 * r.st, r.ph);
+            const uint32_t src = raw_ring + r.st * C::RAW;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int row = r0 + 32 * q;
+#pragma unroll
+                for (int h = 0; h < 2; ++h)  // (128-byte rows in the 128-byte swizzle)
+                    x[q][h] = ld_shared_f4(src + (uint32_t)row * 128u + (uint32_t)(((2 * c8 + h) ^ (row & 7)) * 16));
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(rempty0 + 8 * r.st);
+        };
+        auto largest = [&](int q) {
+            const float m0 = fmaxf(fmaxf(fabsf(x[q][0].x), fabsf(x[q][0].y)), fmaxf(fabsf(x[q][0].z), fabsf(x[q][0].w)));
+            const float m1 = fmaxf(fmaxf(fabsf(x[q][1].x), fabsf(x[q][1].y)), fmaxf(fabsf(x[q][1].z), fabsf(x[q][1].w)));
+            return fmaxf(m0, m1);
+        };
         for (int i = 0; tables_item(p, pair, i, it); ++i) {
-            float most[4] = {0.f, 0.f, 0.f, 0.f};  // the largest magnitudes of the rows
-            for (int kb = it.kb0; kb < it.kb1; ++kb, a.next(), r.next()) {
-                if ((int)(a.t & 1u) != half) continue;
-                wait(rfull0 + 8 * r.st, r.ph);
-                const uint32_t src = raw_ring + r.st * C::RAW;
-                float4 x[4][2];
+            // the rows' scales, from the half that has the tile's first block, for both halves and for the warps that empty the
+            // accumulators (everybody waits for every phase of these barriers, the half that sets the scales too)
+            const uint32_t slot = (uint32_t)i % kTmScales, turn = (uint32_t)i / kTmScales;
+            const bool lead = (int)(a.t & 1u) == half;
+            if (turn > 0) wait(sempty0 + 8 * slot, (turn - 1u) & 1u);
+            if (lead) {
+                load();
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
-                    const int row = r0 + 32 * q;
-#pragma unroll
-                    for (int h = 0; h < 2; ++h)  // (128-byte rows in the 128-byte swizzle)
-                        x[q][h] = ld_shared_f4(src + (uint32_t)row * 128u + (uint32_t)(((2 * c8 + h) ^ (row & 7)) * 16));
+                    float m = largest(q);
+                    m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, 1));
+                    m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, 2));
+                    if (c8 == 0) s_scale[slot][r0 + 32 * q] = (uint8_t)(__float_as_uint(tables_row_scale(m)) >> 23);
                 }
                 __syncwarp();
-                if (lane == 0) mbar_arrive(rempty0 + 8 * r.st);
+                if (lane == 0) mbar_arrive(sfull0 + 8 * slot);
+            }
+            wait(sfull0 + 8 * slot, turn & 1u);
+            float scale[4], most[4], least[4];  // largest and smallest, but for zero, of eight entries' largest magnitudes
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                scale[q] = __uint_as_float((uint32_t)s_scale[slot][r0 + 32 * q] << 23);
+                most[q] = 0.f;
+                least[q] = INFINITY;
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(sempty0 + 8 * slot);
+            for (int kb = it.kb0; kb < it.kb1; ++kb, a.next(), r.next()) {
+                if ((int)(a.t & 1u) != half) continue;
+                if (kb != it.kb0) load();
                 if (a.t >= NS) wait(empty0 + 8 * a.st, a.ph);
                 const uint32_t dst = a_ring + a.st * C::A_BYTES;
 #pragma unroll
@@ -661,31 +748,27 @@ __global__ void __cluster_dims__(F32 ? 1 : 2, 1, 1) __launch_bounds__(TablesCfg<
                     const int row = r0 + 32 * q;  // (64-byte rows in the 64-byte swizzle)
                     const uint32_t at = dst + (uint32_t)row * 64u + (uint32_t)((c8 ^ ((row >> 1) & 3)) * 16);
                     uint32_t b1[4], b2[4];
-                    split2(x[q][0].x, x[q][0].y, scale, b1[0], b2[0]);
-                    split2(x[q][0].z, x[q][0].w, scale, b1[1], b2[1]);
-                    split2(x[q][1].x, x[q][1].y, scale, b1[2], b2[2]);
-                    split2(x[q][1].z, x[q][1].w, scale, b1[3], b2[3]);
+                    split2(x[q][0].x, x[q][0].y, scale[q], b1[0], b2[0]);
+                    split2(x[q][0].z, x[q][0].w, scale[q], b1[1], b2[1]);
+                    split2(x[q][1].x, x[q][1].y, scale[q], b1[2], b2[2]);
+                    split2(x[q][1].z, x[q][1].w, scale[q], b1[3], b2[3]);
                     st_shared_v4(at, b1);
                     st_shared_v4(at + C::PART, b2);
-#pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        most[q] = fmaxf(most[q], fmaxf(fabsf(x[q][h].x), fabsf(x[q][h].y)));
-                        most[q] = fmaxf(most[q], fmaxf(fabsf(x[q][h].z), fabsf(x[q][h].w)));
-                    }
+                    const float m = largest(q);
+                    most[q] = fmaxf(most[q], m);
+                    if (m != 0.f) least[q] = fminf(least[q], m);
                 }
                 fence_proxy_async();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(full0 + 8 * a.st);
             }
-            // rows that fp16 does not hold well enough (in this thread's blocks)
+            // rows that the parts do not hold well enough (in this thread's entries)
             const int rt = it.tile / p.n_mb;
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-                float mx = fmaxf(most[q], __shfl_xor_sync(0xFFFFFFFFu, most[q], 1));
-                mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, 2));
-                const int v = rt * C::ROWS + r0 + 32 * q;
-                if (c8 == 0 && v < p.V && !tables_row_ok(mx, scale)) {
-                    p.bad_row[(size_t)it.tile * C::ROWS + r0 + 32 * q] = 1;
+                const int v = r0 + 32 * q;
+                if ((most[q] * scale[q] > kTmMost || least[q] * scale[q] < kTmLeast) && rt * C::ROWS + v < p.V) {
+                    p.bad_row[(size_t)it.tile * C::ROWS + v] = 1;
                     if (it.q0 == it.q1) s_mend = true;
                 }
             }
@@ -703,35 +786,57 @@ __global__ void __cluster_dims__(F32 ? 1 : 2, 1, 1) __launch_bounds__(TablesCfg<
     if (tid == 0 && s_abort) atomicOr(p.errflag, 1);
 }
 
-// The left-over tiles' pieces, added up in order: one thread per four columns of a row.
-template <bool F32>
-__global__ void __launch_bounds__(256) tables_pieces_kernel(const __grid_constant__ TablesParams p) {
+// The left-over tiles' pieces, added up in order: four columns of N rows a thread, a warp a row, 8 N rows a block.
+template <bool F32, int N>
+__global__ void __launch_bounds__(256, F32 ? 3 : 8) tables_pieces_kernel(const __grid_constant__ TablesParams p) {
     using C = TablesCfg<F32>;
+    static_assert(8 * N <= kTmMendRows, "rows that may have to be worked out again");
+    __shared__ TablesMend sm;
     pdl_wait();
     const int tile = (int)blockIdx.y, rt = tile / p.n_mb, mb = tile - rt * p.n_mb;
     const int q0 = tables_owner(p, tile * p.n_kb), q1 = tables_owner(p, (tile + 1) * p.n_kb - 1);
-    const int v = (int)blockIdx.x * 8 + (threadIdx.x >> 5), c = (threadIdx.x & 31) * 4;
-    if (q0 == q1 || rt * C::ROWS + v >= p.V || mb * 128 + c >= p.m) return;  // (q0 == q1: written whole)
-    const bool bad = F32 && p.bad_row[(size_t)tile * C::ROWS + v] != 0;
-    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+    const int v0 = (int)blockIdx.x * 8 * N, warp = threadIdx.x >> 5, c = (threadIdx.x & 31) * 4, col = mb * 128 + c;
+    if (q0 == q1 || rt * C::ROWS + v0 >= p.V) return;  // (q0 == q1: written whole; uniform)
+    float4 s[N];
+#pragma unroll
+    for (int i = 0; i < N; ++i) s[i] = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll 4
     for (int q = q0; q <= q1; ++q) {
         const int seg = tables_share(p, q) < tile * p.n_kb ? 1 : 0;
-        const float4 x = __ldcs((const float4*)(p.pieces + ((size_t)(q * 2 + seg) * C::ROWS + v) * 128 + c));
-        s.x += x.x, s.y += x.y, s.z += x.z, s.w += x.w;
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            const float4 x = __ldcs((const float4*)(p.pieces + ((size_t)(q * 2 + seg) * C::ROWS + v0 + 8 * i + warp) * 128 + c));
+            s[i].x += x.x, s[i].y += x.y, s[i].z += x.z, s[i].w += x.w;
+        }
     }
-    if (p.bias) {
-        const float* b = p.bias + mb * 128 + c;
-        s.x += b[0], s.y += b[1], s.z += b[2], s.w += b[3];
+    float4 b = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (p.bias && col < p.m) b = make_float4(p.bias[col], p.bias[col + 1], p.bias[col + 2], p.bias[col + 3]);
+    bool any = false;
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        const int v = v0 + 8 * i + warp, row = rt * C::ROWS + v;
+        bool off = false;
+        if (row < p.V && col < p.m) {
+            s[i].x += b.x, s[i].y += b.y, s[i].z += b.z, s[i].w += b.w;
+            *(float4*)(p.out + (size_t)row * p.m + col) = s[i];
+            off = F32 && (p.bad_row[(size_t)tile * C::ROWS + v] != 0 || fmaf(0.f, s[i].x, fmaf(0.f, s[i].y, fmaf(0.f, s[i].z, 0.f * s[i].w))) != 0.f);
+        }
+        if (F32) {
+            off = __any_sync(0xFFFFFFFFu, off);
+            if (c == 0) sm.rows[8 * i + warp] = off ? row : -1;
+            any |= off;
+        }
     }
-    const int row = rt * C::ROWS + v, col = mb * 128 + c;
-    if (F32 && (bad || fmaf(0.f, s.x, fmaf(0.f, s.y, fmaf(0.f, s.z, 0.f * s.w))) != 0.f)) {
-        if (bad || !tables_finite(s.x)) s.x = tables_fp32(p, row, col);
-        if (bad || !tables_finite(s.y)) s.y = tables_fp32(p, row, col + 1);
-        if (bad || !tables_finite(s.z)) s.z = tables_fp32(p, row, col + 2);
-        if (bad || !tables_finite(s.w)) s.w = tables_fp32(p, row, col + 3);
+    if (F32 && __syncthreads_or(any)) {
+        if (warp == 0) {  // those that are wanted first
+            const int r = (c >> 2) < 8 * N ? sm.rows[c >> 2] : -1;
+            __syncwarp();
+            const uint32_t wanted = __ballot_sync(0xFFFFFFFFu, r >= 0), below = (1u << (c >> 2)) - 1u;
+            sm.rows[r >= 0 ? __popc(wanted & below) : __popc(wanted) + __popc(~wanted & below)] = r;
+        }
+        __syncthreads();
+        tables_mend(p, &sm, mb * 128, (int)threadIdx.x);
     }
-    *(float4*)(p.out + (size_t)row * p.m + col) = s;
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
@@ -763,7 +868,7 @@ bool encode_map(CUtensorMap* map, const void* base, CUtensorMapDataType type, ui
 
 struct TablesSizes {
     int n_mb, m_pad, E_pad, pairs;
-    size_t o_w, o_unscale, o_scale, o_bad, n_bad, total;  // (fp32 only: from o_unscale on)
+    size_t o_w, o_unscale, o_bad, n_bad, total;  // (fp32 only: from o_unscale on)
 };
 TablesSizes tables_sizes(int num_sms, int V, int E, int m, bool f32) {
     TablesSizes s;
@@ -773,8 +878,7 @@ TablesSizes tables_sizes(int num_sms, int V, int E, int m, bool f32) {
     s.pairs = f32 ? num_sms : num_sms / 2;
     s.o_w = (size_t)s.pairs * 2 * (f32 ? TablesCfg<true>::ROWS : TablesCfg<false>::ROWS) * 128 * sizeof(float);
     s.o_unscale = s.o_w + (size_t)(f32 ? 2 : 3) * s.m_pad * s.E_pad * 2;
-    s.o_scale = s.o_unscale + (f32 ? (size_t)s.m_pad * sizeof(float2) : 0);
-    s.o_bad = s.o_scale + (f32 ? 256 : 0);
+    s.o_bad = s.o_unscale + (f32 ? (size_t)s.m_pad * sizeof(float2) : 0);
     s.n_bad = f32 ? (size_t)(V + TablesCfg<true>::ROWS - 1) / TablesCfg<true>::ROWS * s.n_mb * TablesCfg<true>::ROWS : 0;
     s.total = s.o_bad + s.n_bad;
     return s;
@@ -786,7 +890,13 @@ cudaError_t tables_run(const TablesParams& p, cudaStream_t st, int* launches) {
     if (e == cudaSuccess) e = launch_pdl(tables_mma_kernel<F32>, dim3((C::PAIR ? 2 : 1) * p.pairs), dim3(C::THREADS), C::SMEM, st, p);
     *launches += 1;
     if (e == cudaSuccess && p.share_pairs > p.left) {
-        e = launch_pdl(tables_pieces_kernel<F32>, dim3(C::ROWS / 8, p.left), dim3(256), 0, st, p);
+        // fp32: 32 rows a block where that leaves a block an SM or more, else 8 (102 tiles left, V = 32,000, E =
+        // 2048: 87.2 and 92.8 us; 56, V = 64,000, E = 1536: 122.1 and 124.6; 9, V = 20,000, E = 2048: 69.1 and 65.1)
+        constexpr int N = F32 ? 4 : 1;
+        if (p.left * (C::ROWS / (8 * N)) >= p.pairs)
+            e = launch_pdl(tables_pieces_kernel<F32, N>, dim3(C::ROWS / (8 * N), p.left), dim3(256), 0, st, p);
+        else
+            e = launch_pdl(tables_pieces_kernel<F32, 1>, dim3(C::ROWS / 8, p.left), dim3(256), 0, st, p);
         *launches += 1;
     }
     return e;
@@ -822,7 +932,6 @@ cudaError_t tables_mma_launch(graft_ctx* ctx, const void* d_emb, graft_dtype dt,
     p.out = d_out;
     p.pieces = (float*)scratch;
     p.unscale = (const float2*)((char*)scratch + s.o_unscale);
-    p.scale = (const float*)((char*)scratch + s.o_scale);
     p.bad_row = (uint8_t*)scratch + s.o_bad;
     p.errflag = ctx->w_errflag;
     p.V = V;
@@ -854,8 +963,7 @@ cudaError_t tables_mma_launch(graft_ctx* ctx, const void* d_emb, graft_dtype dt,
     p.share_pairs = (int)(sp < p.left ? p.left : sp);
     p.wide = m % 8 == 0 && ((uintptr_t)d_out & 31) == 0;
     if (f32)
-        weight_split16_kernel<<<s.m_pad, 256, 0, st>>>(d_W, (const float*)d_emb, V, m, E, s.m_pad, s.E_pad, (__half*)w,
-                                                       (float2*)((char*)scratch + s.o_unscale), (float*)((char*)scratch + s.o_scale),
+        weight_split16_kernel<<<s.m_pad, 256, 0, st>>>(d_W, m, E, s.m_pad, s.E_pad, (__half*)w, (float2*)((char*)scratch + s.o_unscale),
                                                        (uint32_t*)p.bad_row, (int)(s.n_bad / 4));
     else
         weight_split_kernel<<<dim3((s.E_pad + 511) / 512, s.m_pad), 256, 0, st>>>(d_W, m, E, s.m_pad, s.E_pad, (__nv_bfloat16*)w);

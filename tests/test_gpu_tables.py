@@ -194,3 +194,61 @@ def test_fp32_rows_are_judged_tile_by_tile(row):
     rest = torch.arange(V, device="cuda") != 20
     assert torch.equal(got[rest], want[rest])
     assert not got[20].isfinite().any()
+
+
+def _row_error(got, emb, W):
+    """The largest error, of results of N(0, 1) for rows of N(0, 1), over the size of the row."""
+    size = emb.double().pow(2).mean(1, keepdim=True).sqrt().clamp(min=1e-300)
+    return ((got.double() - _exact(emb, W)).abs() / size).max().item()
+
+
+def _best_time(f):
+    best = float("inf")
+    for _ in range(4):
+        a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+        a.record()
+        f()
+        b.record()
+        b.synchronize()
+        best = min(best, a.elapsed_time(b))
+    return best
+
+
+@pytest.mark.parametrize("factor", [300.0, 1000.0, 1e-3, 1e7])
+@pytest.mark.parametrize("column", [5, 1000])  # in the block of columns by which a row is scaled, and not
+def test_fp32_column_of_another_size(column, factor):
+    """One column far larger or smaller than the others: no less precise than N(0, 1) alone (6e-6 of a row's size), and as fast as that
+    where fp16 parts hold it; where they do not (1e7 times), faster than the FMA kernel."""
+    V, E, m = 32000, 2048, 128
+    emb, W, _ = _inputs(V, E, m, "f32", 13)
+    out, g = torch.zeros((V, m), device="cuda"), _graft(V, m)
+    pad = torch.zeros(V * m + 4, device="cuda")
+    ordinary = _best_time(lambda: g.tdes_precompute(emb, W, None, out))
+    fma = _best_time(lambda: g.tdes_precompute(emb, W, None, pad[1:1 + V * m].view(V, m)))  # (off the 16-byte grid)
+    emb[:, column] *= factor
+    assert _row_error(_call(g, emb, W, None, m), emb, W) <= 6e-6
+    taken = _best_time(lambda: g.tdes_precompute(emb, W, None, out))
+    assert taken < (2.5 * ordinary if factor < 1e6 else fma), (ordinary, fma, taken)
+    # W made the other way round, so that all columns count as much
+    W[:, column] /= factor
+    like = emb.clone()
+    like[:, column] /= factor
+    got, want = _call(g, emb, W, None, m).double(), _exact(emb, W)
+    size = like.double().pow(2).mean(1, keepdim=True).sqrt()
+    assert ((got - want).abs() / size).max() <= 6e-6
+
+
+@pytest.mark.parametrize("V,E,m", [(300, 64, 128), (19300, 1092, 40), (40003, 132, 256)])  # whole tiles, pieces, both
+def test_fp32_rows_of_other_sizes_are_as_precise(V, E, m):
+    """Rows of every size, rows that begin with zeros, blocks of a row of other sizes than its first: twice the largest error of
+    N(0, 1) (6e-6 of a row's size; one chain of fp32 multiply-adds is off by 1.2e-5)."""
+    emb, W, _ = _inputs(V, E, m, "f32", 14)
+    W = W.clone()
+    for i, e in enumerate((-90, -60, -30, -19, -12, -7, 7, 8, 9, 16, 40, 60)):
+        emb[(7919 * i) % V] *= 2.0 ** e
+        emb[V - 1 - i, E // 2:] *= 2.0 ** e
+        emb[(4001 * i + 17) % V, :32] *= 2.0 ** e
+    emb[V // 2, :40], emb[V // 3, :32] = 0.0, 0.0
+    emb[V // 3] *= 2.0 ** 20
+    emb[V // 4, :33] = 1e-39
+    assert _row_error(_call(_graft(V, m), emb, W, None, m), emb, W) <= 6e-6
