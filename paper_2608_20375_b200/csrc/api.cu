@@ -303,7 +303,7 @@ graft_status graft_vocab_pass(graft_ctx* ctx, int32_t batch, const void* d_logit
     const int esz = ctx->cfg.logits_dtype == GRAFT_BF16 ? 2 : 4;
     if ((uintptr_t)d_logits % esz) return GRAFT_ERR_INVALID_ARG;
     if (vp_launch(ctx, batch, d_logits, d_topk_id, d_topk_lp, d_lse, d_row_status ? d_row_status : ctx->w_row_status,
-                  nullptr, nullptr, nullptr, false, (cudaStream_t)stream) != cudaSuccess)
+                  nullptr, nullptr, nullptr, VpUse::call, (cudaStream_t)stream) != cudaSuccess)
         return GRAFT_ERR_CUDA;
     return GRAFT_OK;
 }
@@ -413,7 +413,7 @@ graft_status graft_build_trees(graft_ctx* ctx, int32_t batch, const void* d_logi
     const bool neutral = ctx->cfg.beta == 0.0f || !ctx->tdes_set;  // a round without edge scores
     if (ev) cudaEventRecord(ev[0], st);
     if (vp_launch(ctx, batch, d_logits, ids, lps, lse, ctx->w_row_status, use_saba ? d_hidden : nullptr, ctx->w_cos,
-                  nullptr, neutral, st) != cudaSuccess)
+                  nullptr, neutral ? VpUse::neutral_round : VpUse::round, st) != cudaSuccess)
         return GRAFT_ERR_CUDA;
     if (ev) cudaEventRecord(ev[1], st);
     // Edge scores of Eq. 4-6: the kernel scores the depths [0, edge_rows) for every sequence (all depths when the
@@ -458,7 +458,7 @@ graft_status graft_vocab_pass_partial(graft_ctx* ctx, int32_t batch, const void*
     const int esz = ctx->cfg.logits_dtype == GRAFT_BF16 ? 2 : 4;
     if ((uintptr_t)d_logits_shard % esz || (uintptr_t)d_out % 8) return GRAFT_ERR_INVALID_ARG;
     if (vp_launch(ctx, batch, d_logits_shard, ctx->w_topk_id, ctx->w_topk_lp, ctx->w_lse, ctx->w_row_status, nullptr,
-                  nullptr, d_out, false, (cudaStream_t)stream) != cudaSuccess)
+                  nullptr, d_out, VpUse::call, (cudaStream_t)stream) != cudaSuccess)
         return GRAFT_ERR_CUDA;
     return GRAFT_OK;
 }

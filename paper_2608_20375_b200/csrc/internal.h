@@ -140,14 +140,15 @@ inline cudaError_t allow_smem(const void* kernel, size_t need) {
     return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
 }
 
-VpPlan vp_make_plan(const graft_config& cfg, int num_sms, int batch, bool equal_shares);
+// What a vocab pass is for: a call of its own (or one shard's), a round, a round without edge scores (equal shares, vp_make_plan).
+enum class VpUse { call, round, neutral_round };
+VpPlan vp_make_plan(const graft_config& cfg, int num_sms, int batch, VpUse use);
 cudaError_t vp_configure(const graft_config& cfg, int num_sms, size_t* max_smem);
 cudaError_t vp_launch(graft_ctx* ctx, int batch, const void* d_logits, int32_t* d_topk_id, float* d_topk_lp,
                       float* d_lse, int32_t* d_row_status, const void* d_hidden, double* d_cos,
-                      graft_vocab_partial* d_partial, bool equal_shares, cudaStream_t st);
+                      graft_vocab_partial* d_partial, VpUse use, cudaStream_t st);
 // d_hidden != NULL: one more warp per CTA also writes the adjacent-position cosines of the SABA state (Eq. 15)
-// to d_cos [batch, L]; d_partial != NULL: the rows' pieces go there instead of the outputs (vocabulary-parallel use);
-// equal_shares: the partition of the rounds without edge scores (vp_make_plan)
+// to d_cos [batch, L]; d_partial != NULL: the rows' pieces go there instead of the outputs (vocabulary-parallel use)
 cudaError_t vp_merge_launch(graft_ctx* ctx, int batch, int n_shards, const graft_vocab_partial* d_parts,
                             const int32_t* h_v_offset, int32_t* d_topk_id, float* d_topk_lp, float* d_lse,
                             int32_t* d_row_status, cudaStream_t st);

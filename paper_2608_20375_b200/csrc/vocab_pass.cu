@@ -1314,8 +1314,9 @@ static int rows_per_sm(long long row_bytes, int cl, int nt) {
 }
 // The cluster that holds a row, or 0: the streaming kernel.  Measured on 148 SMs, L = 16, K = 32, one launch after the other,
 // streaming kernel -> rows in shared memory.
-static void rows_plan(long long rows, long long row_bytes, int num_sms, VpPlan* pl) {
+static void rows_plan(long long rows, long long row_bytes, int num_sms, bool round, VpPlan* pl) {
     pl->cluster = 0;
+    const int per_sm = rows_per_sm(row_bytes, 4, 256);
     const bool alone = rows * 4 <= num_sms;  // four CTAs a row and an SM for each
     if (rows_per_sm(row_bytes, 1, 256) >= 2 && !(alone && row_bytes >= 80 * 1024)) {
         // a row a CTA where two or more share an SM, any number of rows.  bf16, V = 32,000 (three an SM): batch 1 8.3 -> 5.8 us,
@@ -1328,12 +1329,15 @@ static void rows_plan(long long rows, long long row_bytes, int num_sms, VpPlan* 
         // longer rows, an SM for each (bf16, V = 75,000: batch 4 10.4 -> 7.2, batch 8 10.8 -> 7.8; with 256 threads 7.7, 8.3)
         pl->cluster = 1;
         pl->threads = 512;
-    } else if (rows * 4 <= (long long)num_sms * rows_per_sm(row_bytes, 4, 256) * (row_bytes >= 380 * 1024 ? 2 : 1)) {
+    } else if (rows * 4 <= (long long)num_sms * per_sm * (round && per_sm == 1 ? 2 : 1)) {
         // rows too long for one CTA, or rows of 80 KB and more where four times as many SMs would stand idle, as far as all
-        // pieces are resident at once; twice as far with rows of 380 KB, which the streaming kernel would cut and merge (rounds,
-        // fp32, V = 151,936: batch 3 46.8 -> 42.1 us, batch 4 52.8 -> 47.4, batch 6 53.4 -> 58.5).  V = 151,936: bf16 batch 1 12.7 -> 8.0, batch 4 13.4 -> 8.9, batch 8 (two turns) 15.1 ->
+        // pieces are resident at once.  V = 151,936: bf16 batch 1 12.7 -> 8.0, batch 4 13.4 -> 8.9, batch 8 (two turns) 15.1 ->
         // 18.5; fp32 batch 1 13.7 -> 7.2.  V = 50,021, bf16, batch 1 10.0 -> 5.8 (6.6 in one CTA), V = 32,000 the same in one
         // CTA as in four.  (512 threads: 9.0 at batch 1, V = 151,936; eight CTAs a row 7.9, but 10.0 at batch 4.)
+        // Two turns in rounds on rows of which an SM holds one piece (over 390 KB), which the streaming kernel would cut and merge:
+        // fp32, batch 3 and 4, rounds V = 101,000 45.2 -> 39.9 and 46.7 -> 41.0 us, V = 151,936 45.2 -> 41.6 and 47.5 -> 44.8 (with a
+        // fixed budget 42.3 -> 37.7 and 44.3 -> 41.4); calls of their own 12.5 -> 12.2, 13.1 -> 12.9, 13.4 -> 14.2 and 14.3 -> 15.6.
+        // With two pieces an SM two turns are slower in rounds too (V = 97,600, batch 5: 41.6 -> 45.2).
         pl->cluster = 4;
         pl->threads = 256;
     }
@@ -1364,13 +1368,14 @@ static cudaError_t rows_configure(bool bf16) {
     return e;
 }
 
-VpPlan vp_make_plan(const graft_config& cfg, int num_sms, int batch, bool equal_shares) {
+VpPlan vp_make_plan(const graft_config& cfg, int num_sms, int batch, VpUse use) {
+    const bool equal_shares = use == VpUse::neutral_round;
     VpPlan pl;
     const bool bf16 = cfg.logits_dtype == GRAFT_BF16;
     const long long esz = bf16 ? 2 : 4, rows = (long long)batch * cfg.L, row_bytes = (long long)cfg.V * esz;
     const long long nq = cfg.V / kVpQuantum > 0 ? cfg.V / kVpQuantum : 1;
     pl.cluster = 0;
-    if (!equal_shares) rows_plan(rows, row_bytes, num_sms, &pl);
+    if (!equal_shares) rows_plan(rows, row_bytes, num_sms, use == VpUse::round, &pl);
     long long G, share_q, per = 0;  // CTAs (one per SM at most), a CTA's share at most, whole rows of a CTA at most
     // A row that no other CTA has a piece of needs no merge, which is what a small input waits for (a record and a merge
     // take 5 to 6 us): whole rows wherever the CTAs' shares come out even enough.  Measured
@@ -1424,10 +1429,10 @@ VpPlan vp_make_plan(const graft_config& cfg, int num_sms, int batch, bool equal_
 
 cudaError_t vp_launch(graft_ctx* ctx, int batch, const void* d_logits, int32_t* d_topk_id, float* d_topk_lp,
                       float* d_lse, int32_t* d_row_status, const void* d_hidden, double* d_cos,
-                      graft_vocab_partial* d_partial, bool equal_shares, cudaStream_t st) {
+                      graft_vocab_partial* d_partial, VpUse use, cudaStream_t st) {
     const graft_config& cfg = ctx->cfg;
     const bool bf16 = cfg.logits_dtype == GRAFT_BF16;
-    VpPlan pl = vp_make_plan(cfg, ctx->num_sms, batch, equal_shares);
+    VpPlan pl = vp_make_plan(cfg, ctx->num_sms, batch, use);
     if (pl.cluster > 0) {
         RowsParams r;
         r.logits = (const char*)d_logits;
@@ -1499,7 +1504,7 @@ int vp_merge_max_shards() { return kMergeMaxShards; }
 
 cudaError_t vp_configure(const graft_config& cfg, int num_sms, size_t* max_smem) {
     // the largest dynamic shared-memory request any batch can produce (segment = a whole row)
-    VpPlan pl = vp_make_plan(cfg, num_sms, cfg.max_batch > 4096 ? cfg.max_batch : 4096, false);
+    VpPlan pl = vp_make_plan(cfg, num_sms, cfg.max_batch > 4096 ? cfg.max_batch : 4096, VpUse::call);
     *max_smem = pl.smem_bytes;
     if (pl.smem_bytes > 225 * 1024) return cudaErrorInvalidValue;
     cudaError_t e = cudaSuccess;
@@ -1596,7 +1601,7 @@ extern "C" graft_status graft_vocab_pass_static(int32_t batch, int32_t L, int32_
             sd->ready = true;
         }
     }
-    const VpPlan pl = vp_make_plan(cfg, sd->num_sms, batch, false);
+    const VpPlan pl = vp_make_plan(cfg, sd->num_sms, batch, VpUse::call);
     if (pl.cluster > 0) {
         cudaStream_t st = (cudaStream_t)stream;
         if (cudaMemsetAsync(sd->scratch->errflag, 0, sizeof(sd->scratch->errflag), st) != cudaSuccess) {

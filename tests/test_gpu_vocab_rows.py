@@ -228,3 +228,27 @@ def test_rows_masked_far_below(batch, V, shift, value, dtype):
         assert np.array_equal(out[0][b].cpu().numpy(), o_ids)
         assert np.all(np.abs(out[1][b].cpu().numpy().astype(np.float64) - o_lp) <= tolerance(o_lp))
         assert np.all(np.abs(out[2][b].cpu().numpy() - o_lse) <= tolerance(o_lse))
+
+
+@pytest.mark.parametrize("batch,V", [(4, 99000), (3, 101003), (4, 151936), (5, 101003)])  # one turn of clusters, two in a round, streamed
+def test_rows_of_a_round_and_of_a_call_of_its_own(batch, V):
+    """fp32 rows near 390 KB, which rounds and calls of the vocab pass alone may cut in different ways: the same candidates."""
+    from paper_2608_20375_b200 import Graft
+    L, K = 16, 16
+    g = torch.Generator(device="cuda").manual_seed(V)
+    z = 2.0 * torch.randn((batch, L, V), generator=g, device="cuda")
+    z[:, :, 7::1000] = 6.5  # (ties that decide)
+    gr = Graft(V, L, K, 16, 64, batch, 16, 64, 16, 0.2, 1, 0, 0)
+    P, Ct = (torch.randn((V, 16), generator=g, device="cuda") for _ in range(2))
+    gr.set_tdes_tables(P, Ct, torch.randn((L, 16), generator=g, device="cuda"), 1.0)
+    o = gr.alloc_out(batch, debug=True)
+    ones = torch.ones(batch, dtype=torch.int32, device="cuda")
+    gr.build_trees(z, None, ones, None, 100 * ones, 32 * ones, o)
+    out = _outputs(batch, L, K)
+    gr.vocab_pass(z, *out)
+    torch.cuda.synchronize()
+    assert torch.equal(o.topk_id.view(batch, L, K), out[0]) and not out[3].any() and not o.status.any()
+    assert (o.topk_lp.view(batch, L, K) - out[1]).abs().max() <= 4e-6  # (two spacings at 10)
+    o_ids, _, o_lse, _ = oracle.vocab_pass(z[0].cpu(), K)
+    assert np.array_equal(out[0][0].cpu().numpy(), o_ids)
+    assert np.all(np.abs(o.lse.view(batch, L)[0].cpu().numpy() - o_lse) <= tolerance(o_lse))
