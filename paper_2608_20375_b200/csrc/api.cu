@@ -281,7 +281,7 @@ graft_status graft_tdes_precompute(graft_ctx* ctx, const void* d_emb, graft_dtyp
                                    const float* d_W, const float* d_b, float* d_out, void* stream) {
     if (!ctx || !d_emb || !d_W || !d_out || E < 1) return GRAFT_ERR_INVALID_ARG;
     if (emb_dtype != GRAFT_F32 && emb_dtype != GRAFT_BF16) return GRAFT_ERR_INVALID_ARG;
-    // the tensor cores (bf16 parts of the inputs, exact products), where the rows fit and their scratch is to be had
+    // the tensor cores (16-bit parts of the inputs, exact products), where the rows fit and their scratch is to be had
     if (tables_mma_fits(d_emb, emb_dtype, E, d_out)) {
         void* scratch = tables_scratch(ctx, tables_mma_scratch_bytes(ctx->num_sms, ctx->cfg.V, E, ctx->cfg.m, emb_dtype));
         if (scratch != nullptr) {

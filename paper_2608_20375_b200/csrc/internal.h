@@ -93,7 +93,8 @@ struct graft_ctx {
     double* w_loss;               // [8] sums of graft_tdes_loss and its arrival counter, zero between calls
     int32_t* w_errflag;           // [1] device-side internal error flag
     graft::VpPlan vp_plan;
-    // scratch of the tensor-core table precompute (allocated on its first use: pieces of split tiles, W's bf16 parts)
+    // scratch of the tensor-core table precompute (allocated on its first use: pieces of split tiles, W's parts,
+    // flags of rows)
     void* tables_scratch;
     size_t tables_scratch_bytes;
     // host-buffer staging (allocated on first use of graft_build_trees_host)

@@ -162,7 +162,8 @@ __global__ void __launch_bounds__(kFitThreads, 2) saba_fit_kernel(const FitParam
             const int4 bu = __ldg((const int4*)p.budget + q), pr = __ldg((const int4*)p.prefix + q);
             const float4 ga = __ldg((const float4*)p.gain + q), la = __ldg((const float4*)p.latency + q);
             // tau = -B / log(1 - g), the four quotients by one division: 1 / l0 = (l2 l3 / (l0 l1 l2 l3)) l1 and so on (P. L.
-            // Montgomery's simultaneous inversion, 1987); the product of four logarithms is between 1e-180 and 1e5
+            // Montgomery's simultaneous inversion, 1987); the product of four logarithms is between 1e-180 and 1e5.  A quotient goes
+            // through three products more than a division of its own: a few units in the last place of fp64, as does the series above.
             const bool ok[4] = {fit_ok(ga.x), fit_ok(ga.y), fit_ok(ga.z), fit_ok(ga.w)};
             const float g4[4] = {ga.x, ga.y, ga.z, ga.w};
             double l[4];
