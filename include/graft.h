@@ -49,7 +49,7 @@ typedef enum {
 typedef enum { GRAFT_F32 = 0, GRAFT_BF16 = 1 } graft_dtype;
 
 /* per-sequence bits written to d_status */
-#define GRAFT_ST_BAD_LOGITS 1     /* a logits row holds NaN or +inf, or no finite entry: root-only tree */
+#define GRAFT_ST_BAD_LOGITS 1     /* a logits row holds NaN or +inf, or no finite entry (entries below -1e9 may count as none): root-only tree */
 #define GRAFT_ST_TAU_CLAMPED 2    /* SABA: phi . s_t fell below tau_min and was clamped */
 #define GRAFT_ST_FRONTIER_EMPTY 4 /* fewer reachable prefixes than the budget */
 #define GRAFT_ST_INTERNAL 8       /* a bounded device-side wait ran out (should never happen) */
