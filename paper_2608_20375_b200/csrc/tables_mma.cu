@@ -78,7 +78,7 @@ constexpr float kTmLow = 2048.0f;  // fp16: second parts are kept times 2^11
 // piece's first block) to [16, 32).  Two parts hold a number up to 65504 to 2^-23 of it or to 2^-36, whichever is more; where the
 // largest of eight entries side by side is 2^-12 or more, that is 2^-23 of themselves or 2^-24 of that largest.  So the rest of a row may
 // be 2^11 times larger than its first block, and any eight entries 2^16 times smaller.  (With one scale for the table, one column 300
-// times larger than the others left 40 % of the rows to tables_mend's forerunner.)
+// times larger than the others left 40 % of the rows to be worked out again.)
 constexpr int kTmTarget = 4;
 constexpr float kTmLeast = 0x1p-12f, kTmMost = 65504.f;
 constexpr uint32_t kTmScales = 4;  // tiles whose rows' scales are kept

@@ -111,8 +111,8 @@ def test_fp32_entries_that_bf16_parts_cannot_hold(V, E, m):
 @pytest.mark.parametrize("part", ["embedding", "W", "both"])
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 def test_parts_of_every_order_count(part, dtype):
-    """Terms +-(1 + 2^-10 + t 2^-19) whose first and second parts cancel: the third parts are the whole result, exactly (all
-    sums are short multiples of powers of two)."""
+    """Terms +-(1 + 2^-10 + t 2^-19) whose leading parts cancel: what the last part holds (W beside bf16 embeddings: the third, fp32
+    embeddings and their W: the second) is the whole result, exactly (all sums are short multiples of powers of two)."""
     if dtype == "bf16" and part != "W":
         pytest.skip("bf16 embeddings have one part")
     V, E, m = 1000, 2048, 128
@@ -123,14 +123,14 @@ def test_parts_of_every_order_count(part, dtype):
     W = third(m) if part != "embedding" else torch.ones((m, E), device="cuda")
     got, want = _call(_graft(V, m), emb.to(DTYPES[dtype]), W, None, m).double(), _exact(emb, W)
     assert want.abs().max() > 1e-5
-    # 2^-29 a term is left out where both numbers have three parts (second times third)
+    # where both numbers have a part of some 2^-19, their product is left out: far below 2^-27 a term
     assert (got - want).abs().max() <= (2.0 ** -27 * E if part == "both" else 0.0)
 
 
 @pytest.mark.parametrize("V,E,m,dtype", [(8192, 4096, 128, "bf16"), (8192, 2048, 128, "f32")])
 def test_error_against_64_bit_products(V, E, m, dtype):
-    """N(0, 1) embeddings, results of N(0, 1): twice the largest error seen over a million results (3.2e-6 and 3.0e-6; a chain
-    of fp32 multiply-adds 1.2e-5)."""
+    """N(0, 1) embeddings, results of N(0, 1): twice the largest error seen over a million results (3.2e-6; in fp32 2.2e-6, with three
+    bf16 parts 3.0e-6; a chain of fp32 multiply-adds 1.2e-5)."""
     emb, W, _ = _inputs(V, E, m, dtype, 8)
     assert (_call(_graft(V, m), emb, W, None, m) - _exact(emb, W)).abs().max() <= 6e-6
 
