@@ -11,7 +11,8 @@
 // traffic out of L2, no tensor-core path.  One warp per item (a group of K children, a few pairs or edges): a lane holds
 // four consecutive floats of every 128-float chunk of a row, gradient rows go out as 16-byte vector atomics
 // (`red.global.add.v4.f32`), gu is accumulated in shared memory and flushed once, losses and the scale's gradient are
-// reduced per CTA.  Two kernels: tdes_loss_rows_kernel for m <= 128, tdes_loss_kernel for wider rows.
+// reduced per CTA.  tdes_loss_rows_kernel for m <= 128, tdes_groups_kernel and tdes_items_kernel for m <= 128 and many
+// traces, tdes_loss_kernel for wider rows.
 // The order of the atomic additions is not fixed, so the gradients are reproducible only up to fp32 rounding.
 #include <cuda_runtime.h>
 #include <math.h>
@@ -21,6 +22,12 @@
 
 namespace graft {
 namespace {
+
+// *q += v in global memory, nothing returned (an atomicAdd of a float4 brings the old values back, used or not: 1.6 million
+// rows in one step took 305 us so and 320 with it).
+__device__ __forceinline__ void red_add4(float4* q, const float4& v) {
+    asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(q), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w));
+}
 
 constexpr int kTrThreads = 256;
 constexpr int kTrWarps = kTrThreads / 32;
@@ -50,7 +57,8 @@ struct TrainParams {
     int32_t* skipped;  // [1] or NULL, zero at launch
     double* acc;       // m <= 128: [5] loss sums, skipped items, arrival counter; zero between calls
     int gu_copies;     // m <= 128: copies of gu in shared memory: one per warp, or one
-    int sample;        // m <= 128: look for hot tokens
+    int g_batch;       // m <= 128: groups of a batch
+    int ctas;          // m <= 128: CTAs of the call, that arrive at acc
     float* gP;
     float* gC;
     float* gu;
@@ -99,8 +107,8 @@ __device__ __forceinline__ void add_row_global(float* dst, int tok, int m, int l
     for (int ch = 0; ch < NCH; ++ch) {
         const int k4 = ch * 32 + lane;
         if (k4 < m / 4)
-            atomicAdd((float4*)(dst + (size_t)tok * m) + k4,
-                      make_float4(coef * r.v[ch].x, coef * r.v[ch].y, coef * r.v[ch].z, coef * r.v[ch].w));
+            red_add4((float4*)(dst + (size_t)tok * m) + k4,
+                     make_float4(coef * r.v[ch].x, coef * r.v[ch].y, coef * r.v[ch].z, coef * r.v[ch].w));
     }
 }
 // the CTA's copy of gu: row d-1 += coef * (a + b)
@@ -312,22 +320,14 @@ __global__ void __launch_bounds__(kTrThreads) tdes_loss_kernel(const TrainParams
 //     loads in flight together; pairs go four at a time and edges eight;
 //   * dot products are summed across the warp together (31 shuffles for 32 of them), which leaves dot i in the lanes
 //     that own item i: the transcendental functions are worked out once per item, not once per lane;
-//   * every warp adds into a copy of gu of its own (a plain load, add and store);
-//   * the few hottest tokens' gradient rows (additions to one row serialise in L2) are picked once per CTA from a sample of
-//     the tokens, and every warp keeps its sums of them in shared memory; everything else is a 16-byte vector atomic.
-// Measured (B200, V = 151,936, m = 128, L = 16, 32,768 groups of 32, 131,072 pairs, 262,144 edges): 323 us (420 us by the
-// one-item-a-warp kernel with replaced cached rows; 500 of 8, 2000 and 4000: 16.6 and 19.6 us).  What bounds it now: the vector atomics -- a million rows spread
-// evenly take 96 us whether from 8 or from 32 warps an SM or as bulk reductions from shared memory, a million with the
-// Zipf(1.1) tokens of these traces 790 us, without their eight hottest 152 us -- and, in front of them in the same
-// queue, 1.6 million row loads (138 us for the losses alone).  One copy of gu with atomics instead of one a warp leaves
-// more L1 for the rows but costs more than it saves (360 us).
+//   * every warp adds into a copy of gu of its own (a plain load, add and store).
+// Many traces have kernels of their own, further down.
 constexpr int kTsThreads = 384;
 constexpr int kTsWarps = kTsThreads / 32;
-constexpr int kTsSample = 256;
-// References to rows from which looking for hot ones is worth its time (10 us: two rounds of loads, 256 x 256 compares).
-// With and without: 41 thousand references 26.8 and 22.8 us, 65 thousand 34.0 and 26.7, 74 thousand 33.0 and 35.0, 164
-// thousand 47.4 and 61.0.
-constexpr int kTsSampleMin = 65536;
+// References to rows from which the two kernels for many traces are used: with gradients (K = 32: 98 thousand 35.5 us by the
+// kernel below and 37.5 by the two, 130 thousand 39.6 and 39.7, 195 thousand 57.7 and 47.4) and for the losses alone (260
+// thousand 21.0 and 29.2, 520 thousand 35.4 and 37.4, a million 63.7 and 56.5).
+constexpr long long kTsMany = 131072, kTsManyLoss = 655360;
 
 constexpr int kTsSlots = 8;  // hot rows per table
 struct __align__(16) TrainHot {
@@ -336,13 +336,17 @@ struct __align__(16) TrainHot {
 
 __device__ __forceinline__ float2 lo2(const float4& v) { return make_float2(v.x, v.y); }
 __device__ __forceinline__ float2 hi2(const float4& v) { return make_float2(v.z, v.w); }
-__device__ __forceinline__ float4 add4(const float4& a, const float4& b) { return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w); }
-__device__ __forceinline__ float4 sub4(const float4& a, const float4& b) { return make_float4(a.x - b.x, a.y - b.y, a.z - b.z, a.w - b.w); }
-__device__ __forceinline__ float4 mul4(float c, const float4& a) { return make_float4(c * a.x, c * a.y, c * a.z, c * a.w); }
+__device__ __forceinline__ float4 join4(const float2& l, const float2& h) { return make_float4(l.x, l.y, h.x, h.y); }
+__device__ __forceinline__ float4 add4(const float4& a, const float4& b) { return join4(__fadd2_rn(lo2(a), lo2(b)), __fadd2_rn(hi2(a), hi2(b))); }
+__device__ __forceinline__ float4 mul4(float c, const float4& a) {
+    const float2 cc = make_float2(c, c);
+    return join4(__fmul2_rn(cc, lo2(a)), __fmul2_rn(cc, hi2(a)));
+}
 __device__ __forceinline__ float4 fma4(float c, const float4& a, const float4& b) {
     const float2 cc = make_float2(c, c), l = __ffma2_rn(cc, lo2(a), lo2(b)), h = __ffma2_rn(cc, hi2(a), hi2(b));
-    return make_float4(l.x, l.y, h.x, h.y);
+    return join4(l, h);
 }
+__device__ __forceinline__ float4 sub4(const float4& a, const float4& b) { return fma4(-1.f, b, a); }
 __device__ __forceinline__ float dot4(const float4& a, const float4& b) {
     const float2 s = __ffma2_rn(lo2(a), lo2(b), __fmul2_rn(hi2(a), hi2(b)));
     return s.x + s.y;
@@ -352,6 +356,32 @@ __device__ __forceinline__ float dot4(const float4& a, const float4& b) {
 template <int N>
 __device__ __forceinline__ float warp_sums(float (&v)[N], int lane) {
     int mask = 16;
+#pragma unroll
+    for (int n = N / 2; n >= 1; n /= 2, mask >>= 1) {
+        const bool up = (lane & mask) != 0;
+#pragma unroll
+        for (int i = 0; i < n; ++i) {
+            const float give = up ? v[i] : v[i + n], keep = up ? v[i + n] : v[i];
+            v[i] = keep + __shfl_xor_sync(0xFFFFFFFFu, give, mask);
+        }
+    }
+    float s = v[0];
+#pragma unroll
+    for (; mask >= 1; mask >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, mask);
+    return s;
+}
+__device__ __forceinline__ float dot8(const float4 (&a)[2], const float4 (&b)[2]) {
+    float2 s = __fmul2_rn(hi2(a[0]), hi2(b[0]));
+    s = __ffma2_rn(lo2(a[0]), lo2(b[0]), s);
+    s = __ffma2_rn(lo2(a[1]), lo2(b[1]), s);
+    s = __ffma2_rn(hi2(a[1]), hi2(b[1]), s);
+    return s.x + s.y;
+}
+// Sums of N values over either half of the warp (N = 4, 8, 16): value i is returned to the half's lanes with
+// (l >> (4 - log2 N)) == i.
+template <int N>
+__device__ __forceinline__ float half_sums(float (&v)[N], int lane) {
+    int mask = 8;
 #pragma unroll
     for (int n = N / 2; n >= 1; n /= 2, mask >>= 1) {
         const bool up = (lane & mask) != 0;
@@ -402,7 +432,7 @@ __device__ __forceinline__ void ctx_add_row(const TrainParams& p, const TrainCtx
     if (slot >= 0)  // (uniform)
         smem_add4(c.hot + (t * kTsSlots + slot) * 32 + c.lane, v);
     else if (FULL || c.on)
-        atomicAdd(ctx_at<FULL>(c, t == 0 ? p.gP : p.gC, tok), v);
+        red_add4(ctx_at<FULL>(c, t == 0 ? p.gP : p.gC, tok), v);
 }
 template <bool FULL>
 __device__ __forceinline__ void ctx_add_u(const TrainCtx& c, int d, const float4& v) {
@@ -427,23 +457,6 @@ __device__ __forceinline__ float4 ctx_u(const TrainCtx& c, int d) {
     return FULL || c.on ? *ctx_at<FULL>(c, c.u, d - 1) : make_float4(0.f, 0.f, 0.f, 0.f);
 }
 
-// The i-th of kTsSample tokens spread evenly over the references to a table (0: P, 1: C), or -1.
-__device__ __forceinline__ int train_sample(const TrainParams& p, int t, int i) {
-    const long long ng = t == 0 ? p.n_groups : (long long)p.n_groups * p.K, np = 2ll * p.n_pairs;
-    const long long n = ng + np + p.n_edges;
-    long long at = n * i / kTsSample;
-    int tok;
-    if (at < ng) {
-        tok = t == 0 ? p.g_parent[at] : p.g_child[at];
-    } else if ((at -= ng) < np) {
-        tok = p.pairs[(at >> 1) * 6 + (at & 1) * 3 + t];
-    } else {
-        at -= np;
-        tok = at < p.n_edges ? p.edges[at * 4 + t] : -1;
-    }
-    return tok >= 0 && tok < p.V ? tok : -1;
-}
-
 // The work is one list -- groups, blocks of eight pairs, blocks of eight edges -- dealt to the warps in turn: the first of a
 // kind, with `ahead` entries of other kinds ahead of it, that warp wid of nw gets.  (Dealt kind by kind, the first warps got
 // one of each, one after the other, while the rest had nothing: half of a small call's time.)
@@ -452,66 +465,78 @@ __device__ __forceinline__ int first_block(int wid, long long ahead, int nw) {
     return r < 0 ? r + nw : r;
 }
 
+// The CTA's share of the losses: sums over its warps, one addition each; the CTA that arrives last (of p.ctas) writes the
+// losses and clears the sums for the next call.  Every thread calls this.
+struct TrainSums {
+    double loss[3];
+    float gs;
+    int skip;
+};
+__device__ __forceinline__ void train_finish(const TrainParams& p, TrainSums& s, double l_kl, double l_pair, double l_bce, float gs,
+                                             int skipped, int lane) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        l_kl += __shfl_xor_sync(0xFFFFFFFFu, l_kl, o);
+        l_pair += __shfl_xor_sync(0xFFFFFFFFu, l_pair, o);
+        l_bce += __shfl_xor_sync(0xFFFFFFFFu, l_bce, o);
+    }
+    gs = warp_sum(gs);
+    skipped = __reduce_add_sync(0xFFFFFFFFu, skipped);
+    if (lane == 0) {
+        atomicAdd(&s.loss[0], l_kl);
+        atomicAdd(&s.loss[1], l_pair);
+        atomicAdd(&s.loss[2], l_bce);
+        atomicAdd(&s.gs, gs);
+        if (skipped) atomicAdd(&s.skip, skipped);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        atomicAdd(p.acc + 0, s.loss[0]);
+        atomicAdd(p.acc + 1, s.loss[1]);
+        atomicAdd(p.acc + 2, s.loss[2]);
+        if (s.skip) atomicAdd((int*)(p.acc + 3), s.skip);
+        if (p.gP != nullptr && s.gs != 0.f) atomicAdd(p.gs, s.gs);
+        __threadfence();
+        if (atomicAdd((unsigned int*)(p.acc + 4), 1u) == (unsigned)p.ctas - 1) {
+            __threadfence();
+            const double kl = __ldcg(p.acc + 0) / (double)(p.n_groups > 0 ? p.n_groups : 1);
+            const double pr = __ldcg(p.acc + 1) / (double)(p.n_pairs > 0 ? p.n_pairs : 1);
+            const double bc = __ldcg(p.acc + 2) / (double)(p.n_edges > 0 ? p.n_edges : 1);
+            p.loss[0] = kl;
+            p.loss[1] = pr;
+            p.loss[2] = bc;
+            p.loss[3] = (double)p.lam_kl * kl + (double)p.lam_pair * pr + (double)p.lam_bce * bc;
+            if (p.skipped) *p.skipped = __ldcg((const int*)(p.acc + 3));
+            for (int i = 0; i < 5; ++i) p.acc[i] = 0.0;
+        }
+    }
+}
+
 // KC: children held in registers, a multiple of 8 (K <= KC)
 template <int KC, bool FULL>
 __global__ void __launch_bounds__(kTsThreads, 1) tdes_loss_rows_kernel(const TrainParams p) {
     extern __shared__ __align__(16) float smem_f[];
-    __shared__ TrainHot s_hot;
-    __shared__ int s_tok[2][kTsSample], s_cnt[2][kTsSample];
-    __shared__ double s_loss[3];
-    __shared__ float s_gs;
-    __shared__ int s_skip;
-    __shared__ bool s_last;
+    __shared__ TrainSums s_sum;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, Lm = p.L * p.m;
     const bool grad = p.gP != nullptr;
-    // [L][m] u, then the copies of gu, then the warps' hot rows
-    float* s_gu = smem_f + Lm;
-    float* s_rows = s_gu + (size_t)Lm * p.gu_copies;
+    float* s_gu = smem_f + Lm;  // [L][m] u, then the copies of gu
     TrainCtx c;
     c.u = smem_f;
     c.gu_shared = p.gu_copies == 1;
     c.gu = s_gu + (c.gu_shared ? 0 : (size_t)warp * Lm);
-    c.hot = (float4*)(s_rows + (size_t)warp * 2 * kTsSlots * 128);
+    c.hot = nullptr;
     c.on = lane < p.m / 4;
     c.lane = lane;
     c.m = p.m;
     for (int i = tid; i < Lm; i += kTsThreads) smem_f[i] = p.u[i];
-    if (grad) {
+    if (grad)
         for (int i = tid; i < Lm / 4 * p.gu_copies; i += kTsThreads) ((float4*)s_gu)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (p.sample)
-            for (int i = tid; i < kTsWarps * 2 * kTsSlots * 32; i += kTsThreads) ((float4*)s_rows)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-    if (tid < 3) s_loss[tid] = 0.0;
+    if (tid < 3) s_sum.loss[tid] = 0.0;
     if (tid == 0) {
-        s_gs = 0.f;
-        s_skip = 0;
-    }
-    if (tid < 2 * kTsSlots) s_hot.tok[tid / kTsSlots][tid % kTsSlots] = -1;
-    if (grad && p.sample) {  // (uniform) the tokens met most often in the sample get the slots
-        for (int i = tid; i < 2 * kTsSample; i += kTsThreads) s_tok[i / kTsSample][i % kTsSample] = train_sample(p, i / kTsSample, i % kTsSample);
-        __syncthreads();
-        for (int i = tid; i < 2 * kTsSample; i += kTsThreads) {
-            const int t = i / kTsSample, me = i % kTsSample, tok = s_tok[t][me];
-            int n = 0, first = me;
-            for (int j = kTsSample - 1; j >= 0; --j)
-                if (s_tok[t][j] == tok) {
-                    ++n;
-                    first = j;
-                }
-            s_cnt[t][me] = tok >= 0 && first == me && n >= 2 ? n * kTsSample + (kTsSample - 1 - me) : 0;  // (distinct, 0: none)
-        }
-        __syncthreads();
-        for (int i = tid; i < 2 * kTsSample; i += kTsThreads) {
-            const int t = i / kTsSample, me = i % kTsSample, mine = s_cnt[t][me];
-            if (mine > 0) {
-                int rank = 0;
-                for (int j = 0; j < kTsSample; ++j) rank += s_cnt[t][j] > mine ? 1 : 0;
-                if (rank < kTsSlots) s_hot.tok[t][rank] = s_tok[t][me];
-            }
-        }
+        s_sum.gs = 0.f;
+        s_sum.skip = 0;
     }
     __syncthreads();
-    const TrainHot& hot = s_hot;
     const int wid = blockIdx.x * kTsWarps + warp, nw = gridDim.x * kTsWarps;
     const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
     double l_kl = 0.0, l_pair = 0.0, l_bce = 0.0;  // per lane; summed at the end
@@ -570,8 +595,6 @@ __global__ void __launch_bounds__(kTsThreads, 1) tdes_loss_rows_kernel(const Tra
         const float gf = lane < p.K ? p.w_kl * (ph - pt) : 0.f;  // d L / d f
         if (lane < p.K) gs += gf * dot_c * p.inv_sqrt_m;
         const float coef = gf * p.k0;
-        const int slot = lane < p.K ? hot_slot(hot, 1, tc) : -1;
-        const uint32_t hots = __ballot_sync(0xFFFFFFFFu, slot >= 0);
         // sum_c coef_c (C_c + u) = sum_c coef_c C_c: the coefficients, differences of two distributions, add up to 0
         float4 acc = zero4;
 #pragma unroll
@@ -580,14 +603,10 @@ __global__ void __launch_bounds__(kTsThreads, 1) tdes_loss_rows_kernel(const Tra
                 const float cf = __shfl_sync(0xFFFFFFFFu, coef, i);
                 const int t = __shfl_sync(0xFFFFFFFFu, tc, i);
                 acc = fma4(cf, rows[i], acc);
-                if (!((hots >> i) & 1u) && (FULL || c.on)) atomicAdd(ctx_at<FULL>(c, p.gC, t), mul4(cf, a));
+                if (FULL || c.on) red_add4(ctx_at<FULL>(c, p.gC, t), mul4(cf, a));
             }
         }
-        for (uint32_t left = hots; left != 0u; left &= left - 1u) {  // (uniform)
-            const int i = __ffs(left) - 1;
-            smem_add4(c.hot + (kTsSlots + __shfl_sync(0xFFFFFFFFu, slot, i)) * 32 + lane, mul4(__shfl_sync(0xFFFFFFFFu, coef, i), a));
-        }
-        ctx_add_row<FULL>(p, c, 0, tp, hot_slot(hot, 0, tp), acc);
+        ctx_add_row<FULL>(p, c, 0, tp, -1, acc);
         ctx_add_u<FULL>(c, d, acc);
     }
     // ---- pairwise level (Eq. 10): blocks of eight pairs, four at a time; lanes 0-7 hold the block's ids
@@ -607,7 +626,6 @@ __global__ void __launch_bounds__(kTsThreads, 1) tdes_loss_rows_kernel(const Tra
             }
         }
         const uint32_t oks = __ballot_sync(0xFFFFFFFFu, ok);
-        const int sp1 = hot_slot(hot, 0, id[0]), sc1 = hot_slot(hot, 1, id[1]), sp2 = hot_slot(hot, 0, id[3]), sc2 = hot_slot(hot, 1, id[4]);
 #pragma unroll 1
         for (int h = 0; h < 2; ++h) {
             if (((oks >> (4 * h)) & 15u) == 0u) continue;  // (uniform)
@@ -652,18 +670,17 @@ __global__ void __launch_bounds__(kTsThreads, 1) tdes_loss_rows_kernel(const Tra
                 const float cf = __shfl_sync(0xFFFFFFFFu, coef, 8 * i);
                 const int p1 = __shfl_sync(0xFFFFFFFFu, id[0], s), c1 = __shfl_sync(0xFFFFFFFFu, id[1], s), d1 = __shfl_sync(0xFFFFFFFFu, id[2], s);
                 const int p2 = __shfl_sync(0xFFFFFFFFu, id[3], s), c2 = __shfl_sync(0xFFFFFFFFu, id[4], s), d2 = __shfl_sync(0xFFFFFFFFu, id[5], s);
-                const int h1 = __shfl_sync(0xFFFFFFFFu, sp1, s), h2 = __shfl_sync(0xFFFFFFFFu, sc1, s);
                 if (p1 == p2) {  // (uniform; an alternative keeps the pair's parent or its child: one addition for both)
-                    ctx_add_row<FULL>(p, c, 0, p1, h1, mul4(cf, sub4(b2[i], b1[i])));
+                    ctx_add_row<FULL>(p, c, 0, p1, -1, mul4(cf, sub4(b2[i], b1[i])));
                 } else {
-                    ctx_add_row<FULL>(p, c, 0, p1, h1, mul4(-cf, b1[i]));
-                    ctx_add_row<FULL>(p, c, 0, p2, __shfl_sync(0xFFFFFFFFu, sp2, s), mul4(cf, b2[i]));
+                    ctx_add_row<FULL>(p, c, 0, p1, -1, mul4(-cf, b1[i]));
+                    ctx_add_row<FULL>(p, c, 0, p2, -1, mul4(cf, b2[i]));
                 }
                 if (c1 == c2) {
-                    ctx_add_row<FULL>(p, c, 1, c1, h2, mul4(cf, sub4(a2[i], a1[i])));
+                    ctx_add_row<FULL>(p, c, 1, c1, -1, mul4(cf, sub4(a2[i], a1[i])));
                 } else {
-                    ctx_add_row<FULL>(p, c, 1, c1, h2, mul4(-cf, a1[i]));
-                    ctx_add_row<FULL>(p, c, 1, c2, __shfl_sync(0xFFFFFFFFu, sc2, s), mul4(cf, a2[i]));
+                    ctx_add_row<FULL>(p, c, 1, c1, -1, mul4(-cf, a1[i]));
+                    ctx_add_row<FULL>(p, c, 1, c2, -1, mul4(cf, a2[i]));
                 }
                 const float4 s1 = add4(a1[i], b1[i]), s2 = add4(a2[i], b2[i]);
                 if (d1 == d2) {
@@ -690,7 +707,6 @@ __global__ void __launch_bounds__(kTsThreads, 1) tdes_loss_rows_kernel(const Tra
             }
         }
         const uint32_t oks = __ballot_sync(0xFFFFFFFFu, ok);
-        const int sp = hot_slot(hot, 0, tp), sc = hot_slot(hot, 1, tc);
         float4 a[8], b[8];
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
@@ -720,64 +736,642 @@ __global__ void __launch_bounds__(kTsThreads, 1) tdes_loss_rows_kernel(const Tra
         for (int i = 0; i < 8; ++i) {
             if (!((oks >> i) & 1u)) continue;  // (uniform)
             const float cf = __shfl_sync(0xFFFFFFFFu, coef, 4 * i);
-            ctx_add_row<FULL>(p, c, 0, __shfl_sync(0xFFFFFFFFu, tp, i), __shfl_sync(0xFFFFFFFFu, sp, i), mul4(cf, b[i]));
-            ctx_add_row<FULL>(p, c, 1, __shfl_sync(0xFFFFFFFFu, tc, i), __shfl_sync(0xFFFFFFFFu, sc, i), mul4(cf, a[i]));
+            ctx_add_row<FULL>(p, c, 0, __shfl_sync(0xFFFFFFFFu, tp, i), -1, mul4(cf, b[i]));
+            ctx_add_row<FULL>(p, c, 1, __shfl_sync(0xFFFFFFFFu, tc, i), -1, mul4(cf, a[i]));
             ctx_add_u<FULL>(c, __shfl_sync(0xFFFFFFFFu, d, i), mul4(cf, add4(a[i], b[i])));
         }
     }
     // ---- per-CTA sums, then one round of global atomics
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        l_kl += __shfl_xor_sync(0xFFFFFFFFu, l_kl, o);
-        l_pair += __shfl_xor_sync(0xFFFFFFFFu, l_pair, o);
-        l_bce += __shfl_xor_sync(0xFFFFFFFFu, l_bce, o);
-    }
-    gs = warp_sum(gs);
-    skipped = __reduce_add_sync(0xFFFFFFFFu, skipped);
-    if (lane == 0) {
-        atomicAdd(&s_loss[0], l_kl);
-        atomicAdd(&s_loss[1], l_pair);
-        atomicAdd(&s_loss[2], l_bce);
-        atomicAdd(&s_gs, gs);
-        if (skipped) atomicAdd(&s_skip, skipped);
-    }
     __syncthreads();
-    if (grad) {
+    if (grad)
         for (int i = tid; i < Lm; i += kTsThreads) {
             float v = s_gu[i];
             for (int w = 1; w < p.gu_copies; ++w) v += s_gu[(size_t)w * Lm + i];
             if (v != 0.f) atomicAdd(p.gu + i, v);
         }
-        for (int i = tid; p.sample && i < 2 * kTsSlots * 32; i += kTsThreads) {
+    train_finish(p, s_sum, l_kl, l_pair, l_bce, gs, skipped, lane);
+}
+
+// ---- many traces: groups first, then pairs and edges ---------------------------------------------------------------------
+// What bounds a large step is the vector additions: an SM hands on one row (512 bytes) in 20 cycles, all of them a million
+// rows in 94 us however they are spread (row loads are three times faster and overlap them), and rows that meet take 4.6 ns
+// each.  So additions are saved where the operands are on chip already, and either half of the work has a kernel that keeps
+// what it needs there:
+//   * tdes_groups_kernel: a CTA's groups (up to 224) leave their parents' rows in shared memory, and the children are put in
+//     the order of their tokens (counting sort by a hash), so that what a token gets from all of them is summed up first: half
+//     of the children of 222 groups are met before in real traces (Zipf), 562 thousand additions instead of 965.  A batch goes
+//     through it in stages that hold eight rows a warp -- all products, then all distributions, then the additions with the
+//     children's rows read a second time -- because 24 warps of 80 registers beat 12 that keep the rows (150 us against 163);
+//   * tdes_items_kernel: a batch of pairs and edges is sorted by depth in shared memory, so that a warp keeps u_d and its sum
+//     of gu_d in registers; the most frequent tokens of the first batch are summed up per warp in shared memory.
+// Measured (B200, V = 151,936, m = 128, L = 16, 32,768 groups of 32, 131,072 pairs, 262,144 edges): 260 us, the two alone 150
+// and 99; 320 by the kernel above with the frequent tokens' rows per warp.  1.2 million additions are 115 us of it, the
+// rest chains of loads and exchanges.  Tried: the frequent tokens' rows as one dense block whose scores and coefficients are
+// single numbers (423 us: four numbers a reference cost what a row does, and the sums lost a digit); two warps a group with
+// the rows kept (150 - 190); both kernels on an SM at once, half the warps each (249 against 251).
+constexpr int kTgGroups = 224;  // groups of a batch at most
+constexpr int kTgThreads = 768;
+constexpr int kTgBinBits = 13, kTgBins = 1 << kTgBinBits;
+constexpr int kTeThreads = 512;
+constexpr int kTeWarps = kTeThreads / 32;
+constexpr int kTeEdges = 2 * kTeThreads;  // a batch: two edges a thread
+constexpr int kTePairs = kTeThreads;      // and a pair
+constexpr int kTeHash = 1024;   // counters for the frequent tokens
+
+__device__ __forceinline__ int tok_hash(int tok, int bits) { return (int)((uint32_t)tok * 2654435761u >> (32 - bits)); }
+
+// KC: children a group has room for, 8, 16 or 32 (K <= KC)
+template <int KC, bool FULL>
+__global__ void __launch_bounds__(kTgThreads, 1) tdes_groups_kernel(const TrainParams p) {
+    extern __shared__ __align__(16) float smem_f[];
+    __shared__ TrainSums s_sum;
+    __shared__ int s_scan[8];
+    __shared__ __align__(16) int s_parent[kTgGroups];
+    __shared__ uint8_t s_order[kTgGroups], s_depth[kTgGroups];  // (depth 0: a group that does not count)
+    constexpr int W = kTgThreads / 32, NB = kTgBins / 2;
+    __shared__ int s_run[W];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, h = lane >> 4, l = lane & 15, Lm = p.L * p.m;
+    const bool grad = p.gP != nullptr;
+    float4* s_a = (float4*)smem_f;                          // [g_batch][32] the groups' P + u
+    float* s_f = (float*)(s_a + p.g_batch * 32);            // [g_batch][KC] products, then coefficients
+    int* s_tok = (int*)(s_f + p.g_batch * KC);              // [g_batch][KC] the children
+    uint32_t* s_bin = (uint32_t*)(s_tok + p.g_batch * KC);  // [NB] two bins a word: where a bin's next child goes
+    float* s_u = (float*)(s_bin + NB);                      // [L][m]
+    float* s_gu = s_u + Lm;                                 // [L][m]
+    uint16_t* s_rec = (uint16_t*)(s_gu + Lm);               // [g_batch * KC + 32] the children in the order of their bins
+    pdl_launch_dependents();  // (the other kernel's work is independent of this one's; it waits for nothing here but the SMs)
+    for (int i = tid; i < Lm; i += kTgThreads) {
+        s_u[i] = p.u[i];
+        s_gu[i] = 0.f;
+    }
+    if (tid < 3) s_sum.loss[tid] = 0.0;
+    if (tid == 0) {
+        s_sum.gs = 0.f;
+        s_sum.skip = 0;
+    }
+    const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
+    const bool on = FULL || lane < p.m / 4, on0 = FULL || l < p.m / 4, on1 = FULL || 16 + l < p.m / 4;
+    const int mm = FULL ? 128 : p.m;
+    double l_kl = 0.0;
+    float gs = 0.f;
+    int skipped = 0;
+    // Half a warp a row, two float4s a lane (l and 16 + l): a sum over 16 lanes is one exchange shorter, and a lane handles
+    // half as many rows.
+    const auto half_row = [&](const float* table, int tok, float4 (&v)[2]) {
+        const float4* q = (const float4*)(table + (size_t)tok * mm) + l;
+        v[0] = on0 ? __ldg(q) : zero4;
+        v[1] = on1 ? __ldg(q + 16) : zero4;
+    };
+    const int g_lo = (int)((long long)p.n_groups * blockIdx.x / gridDim.x), g_hi = (int)((long long)p.n_groups * (blockIdx.x + 1) / gridDim.x);
+    const int n_batch = (g_hi - g_lo + p.g_batch - 1) / p.g_batch;
+    for (int bt = 0; bt < n_batch; ++bt) {
+        const int g0 = g_lo + (int)((long long)(g_hi - g_lo) * bt / n_batch), ng = g_lo + (int)((long long)(g_hi - g_lo) * (bt + 1) / n_batch) - g0;
+        __syncthreads();
+        // ---- the groups' ids; how many children fall into a bin
+        for (int i = tid; i < NB; i += kTgThreads) s_bin[i] = 0u;
+        for (int i = ng + tid; i < kTgGroups; i += kTgThreads) s_parent[i] = 0x7FFFFFFF;
+        __syncthreads();
+#pragma unroll 2
+        for (int gl = warp; gl < ng; gl += W) {
+            const int g = g0 + gl, tp = p.g_parent[g], d = p.g_depth[g];
+            const int tc = p.g_child[(size_t)g * p.K + min(lane, p.K - 1)];  // (places past K: the last child again)
+            const bool ok = __all_sync(0xFFFFFFFFu, tok_ok(tc, p.V)) && tok_ok(tp, p.V) && d >= 1 && d <= p.L;
+            if (lane < KC) s_tok[gl * KC + lane] = ok ? tc : 0;
+            if (ok && grad && lane < p.K) {
+                const int b = tok_hash(tc, kTgBinBits);
+                atomicAdd(&s_bin[b >> 1], b & 1 ? 0x10000u : 1u);
+            }
+            if (lane == 0) {
+                s_parent[gl] = tp;
+                s_depth[gl] = ok ? (uint8_t)d : 0;
+                skipped += ok ? 0 : 1;
+            }
+        }
+        __syncthreads();
+        // ---- the bins' places: an exclusive sum over them; beside it the order of the groups' parents
+        if (grad && warp < 8) {
+            uint32_t sum = 0;
+#pragma unroll 8
+            for (int i = 0; i < NB / 256; ++i) {
+                const uint32_t word = s_bin[warp * (NB / 8) + 32 * i + lane];
+                sum += (word & 0xFFFFu) + (word >> 16);
+            }
+            sum = __reduce_add_sync(0xFFFFFFFFu, sum);
+            if (lane == 0) s_scan[warp] = (int)sum;
+        }
+        if (grad && warp >= W - 7 && tid - 32 * (W - 7) < ng) {  // groups of one parent side by side: one addition to its row
+            const int i = tid - 32 * (W - 7), mine = s_parent[i];
+            int rank = 0;
+#pragma unroll 4
+            for (int j = 0; j < kTgGroups; j += 4) {
+                const int4 o = *(const int4*)(s_parent + j);
+                rank += (o.x < mine || (o.x == mine && j < i)) + (o.y < mine || (o.y == mine && j + 1 < i)) +
+                        (o.z < mine || (o.z == mine && j + 2 < i)) + (o.w < mine || (o.w == mine && j + 3 < i));
+            }
+            s_order[rank] = (uint8_t)i;
+        }
+        __syncthreads();
+        int n_rec = 0;
+        if (grad) {
+            uint32_t base = 0;
+            for (int w = 0; w < 8; ++w) {
+                base += w < warp ? s_scan[w] : 0;
+                n_rec += s_scan[w];
+            }
+            if (warp < 8) {
+#pragma unroll 4
+                for (int i = 0; i < NB / 256; ++i) {
+                    uint32_t* word = s_bin + warp * (NB / 8) + 32 * i + lane;
+                    const uint32_t lo = *word & 0xFFFFu, v = lo + (*word >> 16);
+                    uint32_t incl = v;
+#pragma unroll
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const uint32_t t = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+                        if (lane >= o) incl += t;
+                    }
+                    const uint32_t at = base + incl - v;
+                    *word = at | (at + lo) << 16;
+                    base += __shfl_sync(0xFFFFFFFFu, incl, 31);
+                }
+            }
+            if (tid < 32 && n_rec + tid < ((n_rec + 31) & ~31)) s_rec[n_rec + tid] = 0xFFFFu;
+        }
+        // ---- products with the parent: eight children at a time
+        for (int gl = warp; gl < ng; gl += W) {
+            const int d = s_depth[gl];
+            if (d == 0) continue;
+            float4 a[2];
+            half_row(p.P, s_parent[gl], a);
+            float au = 0.f;
+#pragma unroll 1
+            for (int c = 0; c < KC; c += 8) {
+                const int4 t = *(const int4*)(s_tok + gl * KC + c + 4 * h);
+                float4 rows[4][2];
+                half_row(p.C, t.x, rows[0]);
+                half_row(p.C, t.y, rows[1]);
+                half_row(p.C, t.z, rows[2]);
+                half_row(p.C, t.w, rows[3]);
+                if (c == 0) {  // f = k0 (a . C + a . u)
+                    const float4* q = (const float4*)(s_u + (d - 1) * p.m) + l;
+                    const float4 u0 = on0 ? q[0] : zero4, u1 = on1 ? q[16] : zero4;
+                    a[0] = add4(a[0], u0);
+                    a[1] = add4(a[1], u1);
+                    au = dot4(a[0], u0) + dot4(a[1], u1);
+#pragma unroll
+                    for (int o = 8; o > 0; o >>= 1) au += __shfl_xor_sync(0xFFFFFFFFu, au, o);
+                    s_a[gl * 32 + lane] = h ? a[1] : a[0];
+                }
+                float part[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) part[i] = dot8(a, rows[i]);
+                const float dot = half_sums<4>(part, lane);  // child i of the half in lanes 16 h + 4 i ..
+                if ((l & 3) == 0) s_f[gl * KC + c + 4 * h + (l >> 2)] = au + dot;
+            }
+        }
+        __syncthreads();
+        // ---- the two distributions, the loss, the coefficients (lane i: child i) and the children's places: two groups at a time
+        for (int gl = warp; gl < ng; gl += 2 * W) {
+            float z[2], al[2], dot[2], zmax[2], amax[2], ez[2], ea[2], zsum[2], asum[2];
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const int gq = gl + q * W;
+                const bool use = gq < ng && lane < p.K;
+                const size_t at = (size_t)(g0 + gq) * p.K + lane;
+                dot[q] = use ? s_f[gq * KC + lane] : 0.f;
+                z[q] = use ? p.g_ztgt[at] : -INFINITY;
+                al[q] = use ? p.g_logq[at] + p.k0 * dot[q] : -INFINITY;
+                zmax[q] = z[q];
+                amax[q] = al[q];
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+                for (int q = 0; q < 2; ++q) {
+                    zmax[q] = fmaxf(zmax[q], __shfl_xor_sync(0xFFFFFFFFu, zmax[q], o));
+                    amax[q] = fmaxf(amax[q], __shfl_xor_sync(0xFFFFFFFFu, amax[q], o));
+                }
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                zsum[q] = ez[q] = lane < p.K ? expf(z[q] - zmax[q]) : 0.f;
+                asum[q] = ea[q] = lane < p.K ? expf(al[q] - amax[q]) : 0.f;
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+                for (int q = 0; q < 2; ++q) {
+                    zsum[q] += __shfl_xor_sync(0xFFFFFFFFu, zsum[q], o);
+                    asum[q] += __shfl_xor_sync(0xFFFFFFFFu, asum[q], o);
+                }
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const int gq = gl + q * W;
+                if (gq >= ng || s_depth[gq] == 0) continue;  // (uniform)
+                const float pt = ez[q] / zsum[q], ph = ea[q] / asum[q];
+                if (lane < p.K && pt > 0.f) l_kl += (double)(pt * ((z[q] - zmax[q] - logf(zsum[q])) - (al[q] - amax[q] - logf(asum[q]))));
+                if (!grad) continue;
+                const float gf = lane < p.K ? p.w_kl * (ph - pt) : 0.f;  // d L / d f
+                gs += gf * dot[q] * p.inv_sqrt_m;
+                if (lane < KC) s_f[gq * KC + lane] = gf * p.k0;
+                if (lane < p.K) {
+                    const int b = tok_hash(s_tok[gq * KC + lane], kTgBinBits);
+                    const uint32_t old = atomicAdd(&s_bin[b >> 1], b & 1 ? 0x10000u : 1u);
+                    s_rec[b & 1 ? old >> 16 : old & 0xFFFFu] = (uint16_t)(gq * KC + lane);
+                }
+            }
+        }
+        if (!grad) continue;
+        __syncthreads();
+        // ---- the additions, turn by turn: a group's sum over its children (to its parent's row and its depth's), and 32 of the
+        // sorted children, of which a token's stand side by side (but for the few that share a bin), so that the vector
+        // additions to gC and the loads for gP overlap
+        const int at_lo = ng * warp / W, at_hi = ng * (warp + 1) / W;
+        int run_tp = -1;  // the parent whose groups are summed up in run
+        float4 run = zero4;
+        const auto flush = [&] {
+            if (run_tp >= 0 && on) red_add4((float4*)(p.gP + (size_t)run_tp * mm) + lane, run);
+            run = zero4;
+        };
+        for (int at = at_lo, r0 = warp * 32; at < at_hi || r0 < n_rec; ++at, r0 += kTgThreads) {
+            const int gl = at < at_hi ? s_order[at] : 0, d = at < at_hi ? s_depth[gl] : 0;
+            if (d != 0) {
+                // sum_c coef_c (C_c + u) = sum_c coef_c C_c: the coefficients, differences of two distributions, add up to 0
+                float4 acc[2] = {zero4, zero4};
+#pragma unroll 1
+                for (int c = 0; c < KC; c += 8) {
+                    const int4 t = *(const int4*)(s_tok + gl * KC + c + 4 * h);
+                    const float4 cf = *(const float4*)(s_f + gl * KC + c + 4 * h);
+                    float4 rows[4][2];
+                    half_row(p.C, t.x, rows[0]);
+                    half_row(p.C, t.y, rows[1]);
+                    half_row(p.C, t.z, rows[2]);
+                    half_row(p.C, t.w, rows[3]);
+#pragma unroll
+                    for (int k = 0; k < 2; ++k) {
+                        acc[k] = fma4(cf.x, rows[0][k], acc[k]);
+                        acc[k] = fma4(cf.y, rows[1][k], acc[k]);
+                        acc[k] = fma4(cf.z, rows[2][k], acc[k]);
+                        acc[k] = fma4(cf.w, rows[3][k], acc[k]);
+                    }
+                }
+                const float4 give = h ? acc[0] : acc[1], keep = h ? acc[1] : acc[0];
+                const float4 sum = make_float4(keep.x + __shfl_xor_sync(0xFFFFFFFFu, give.x, 16), keep.y + __shfl_xor_sync(0xFFFFFFFFu, give.y, 16),
+                                               keep.z + __shfl_xor_sync(0xFFFFFFFFu, give.z, 16), keep.w + __shfl_xor_sync(0xFFFFFFFFu, give.w, 16));
+                const int tp = s_parent[gl];
+                if (tp != run_tp) {  // (uniform)
+                    flush();
+                    run_tp = tp;
+                }
+                run = add4(run, sum);
+                if (on) {
+                    float* q = s_gu + (d - 1) * p.m + 4 * lane;
+                    atomicAdd(q + 0, sum.x);
+                    atomicAdd(q + 1, sum.y);
+                    atomicAdd(q + 2, sum.z);
+                    atomicAdd(q + 3, sum.w);
+                }
+            }
+            if (r0 < n_rec) {
+                const int me = s_rec[r0 + lane], tok = me != 0xFFFF ? s_tok[me] : -1, next = __shfl_down_sync(0xFFFFFFFFu, tok, 1);
+                const float my_cf = me != 0xFFFF ? s_f[me] : 0.f;
+                uint32_t ends = __ballot_sync(0xFFFFFFFFu, tok >= 0 && (lane == 31 || next != tok));  // the last of a token's
+                const int my_row = me != 0xFFFF ? me / KC * 32 : 0;
+                float4 acc = zero4;
+#pragma unroll 1
+                for (int i0 = 0; i0 < 32; i0 += 8, ends >>= 8) {
+                    float4 row[8];
+#pragma unroll
+                    for (int q = 0; q < 8; ++q) row[q] = s_a[__shfl_sync(0xFFFFFFFFu, my_row, i0 + q) + lane];
+#pragma unroll
+                    for (int q = 0; q < 8; ++q) {
+                        acc = fma4(__shfl_sync(0xFFFFFFFFu, my_cf, i0 + q), row[q], acc);
+                        if (ends & (1u << q)) {  // (uniform)
+                            const int t = __shfl_sync(0xFFFFFFFFu, tok, i0 + q);
+                            if (on) red_add4((float4*)(p.gC + (size_t)t * mm) + lane, acc);
+                            acc = zero4;
+                        }
+                    }
+                }
+            }
+        }
+        // the runs that the warps end with, neighbours' of one parent together
+        __syncthreads();
+        s_a[tid] = run;
+        if (lane == 0) s_run[warp] = run_tp;
+        __syncthreads();
+        if (run_tp >= 0 && (warp == 0 || s_run[warp - 1] != run_tp)) {
+            for (int w = warp + 1; w < W && s_run[w] == run_tp; ++w) run = add4(run, s_a[w * 32 + lane]);
+            flush();
+        }
+    }
+    if (grad) {
+        __syncthreads();
+        for (int i = tid; i < Lm / 4; i += kTgThreads) red_add4((float4*)p.gu + i, ((const float4*)s_gu)[i]);
+    }
+    __syncthreads();
+    train_finish(p, s_sum, l_kl, 0.0, 0.0, gs, skipped, lane);
+}
+
+// Pairs and edges.
+template <bool FULL>
+__global__ void __launch_bounds__(kTeThreads, 1) tdes_items_kernel(const TrainParams p) {
+    extern __shared__ __align__(16) float smem_f[];
+    __shared__ TrainSums s_sum;
+    __shared__ TrainHot s_hot;
+    __shared__ int s_nhot[2];
+    __shared__ int s_start[2][kMaxL + 1];  // edges, pairs: the first of a depth in the sorted batch
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, Lm = p.L * p.m;
+    const bool grad = p.gP != nullptr;
+    int4* s_edge = (int4*)smem_f;                   // [kTeEdges] parent, child, label | slots
+    int4* s_pair = s_edge + kTeEdges;               // [kTePairs] the four tokens
+    int* s_pinfo = (int*)(s_pair + kTePairs);       // [kTePairs] second depth | slots
+    float4* s_rows = (float4*)(s_pinfo + kTePairs); // [kTeWarps][2][kTsSlots][32] sums of the frequent tokens' rows
+    float* s_u = (float*)(s_rows + kTeWarps * 2 * kTsSlots * 32);  // [L][m]
+    float* s_gu = s_u + Lm;                                         // [L][m]
+    TrainCtx c;
+    c.u = s_u;
+    c.gu = nullptr;
+    c.hot = s_rows + warp * 2 * kTsSlots * 32;
+    c.gu_shared = false;
+    c.on = lane < p.m / 4;
+    c.lane = lane;
+    c.m = p.m;
+    const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
+    int* s_cnt = (int*)s_rows;               // [2][kTeHash] (before the rows)
+    int* s_tok = s_cnt + 2 * kTeHash;        // [2][kTeHash]
+    for (int i = tid; i < Lm; i += kTeThreads) {
+        s_u[i] = p.u[i];
+        s_gu[i] = 0.f;
+    }
+    const auto add_gu = [&](int d, const float4& v) {
+        if (d < 1 || !grad || !(FULL || c.on)) return;
+        float* q = s_gu + (d - 1) * p.m + 4 * lane;
+        atomicAdd(q + 0, v.x);
+        atomicAdd(q + 1, v.y);
+        atomicAdd(q + 2, v.z);
+        atomicAdd(q + 3, v.w);
+    };
+    for (int i = tid; i < 2 * kTeHash; i += kTeThreads) s_cnt[i] = 0;
+    if (tid < 3) s_sum.loss[tid] = 0.0;
+    if (tid == 0) {
+        s_sum.gs = 0.f;
+        s_sum.skip = 0;
+    }
+    if (tid < 2) s_nhot[tid] = 0;
+    if (tid < 2 * kTsSlots) s_hot.tok[tid / kTsSlots][tid % kTsSlots] = -1;
+    __syncthreads();
+    double l_pair = 0.0, l_bce = 0.0;
+    float gs = 0.f;
+    int skipped = 0;
+    const int e_lo = (int)((long long)p.n_edges * blockIdx.x / gridDim.x), e_hi = (int)((long long)p.n_edges * (blockIdx.x + 1) / gridDim.x);
+    const int q_lo = (int)((long long)p.n_pairs * blockIdx.x / gridDim.x), q_hi = (int)((long long)p.n_pairs * (blockIdx.x + 1) / gridDim.x);
+    const int n_batch = max((e_hi - e_lo + kTeEdges - 1) / kTeEdges, (q_hi - q_lo + kTePairs - 1) / kTePairs);
+    for (int bt = 0; bt < n_batch; ++bt) {
+        const auto part = [&](int lo, int hi, int i) { return lo + (int)((long long)(hi - lo) * i / n_batch); };
+        const int e0 = part(e_lo, e_hi, bt), ne = part(e_lo, e_hi, bt + 1) - e0, q0 = part(q_lo, q_hi, bt), nq = part(q_lo, q_hi, bt + 1) - q0;
+        // ---- the batch in registers, then sorted by depth into shared memory
+        int4 edge[2];
+        bool e_ok[2];
+        int id[6] = {0, 0, 1, 0, 0, 1};
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const int i = tid + k * kTeThreads;
+            edge[k] = make_int4(0, 0, 1, 0);
+            if (i < ne) {  // (the lists are aligned to their elements only)
+                const int32_t* e = p.edges + (size_t)(e0 + i) * 4;
+                edge[k] = make_int4(e[0], e[1], e[2], e[3]);
+            }
+        }
+        if (tid < nq) {
+            const int32_t* q = p.pairs + (size_t)(q0 + tid) * 6;
+#pragma unroll
+            for (int k = 0; k < 6; ++k) id[k] = q[k];
+        }
+        if (tid < 2 * kMaxL) s_start[tid / kMaxL][tid % kMaxL] = 0;
+        __syncthreads();
+        int e_rank[2] = {}, q_rank = 0;
+        const auto depth_ok = [&](int d) { return d >= 1 && d <= p.L; };
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            e_ok[k] = tid + k * kTeThreads < ne && tok_ok(edge[k].x, p.V) && tok_ok(edge[k].y, p.V) && depth_ok(edge[k].z);
+            skipped += tid + k * kTeThreads < ne && !e_ok[k] ? 1 : 0;
+            if (e_ok[k]) e_rank[k] = atomicAdd(&s_start[0][edge[k].z - 1], 1);
+        }
+        const bool q_ok = tid < nq && tok_ok(id[0], p.V) && tok_ok(id[1], p.V) && tok_ok(id[3], p.V) && tok_ok(id[4], p.V) && depth_ok(id[2]) && depth_ok(id[5]);
+        skipped += tid < nq && !q_ok ? 1 : 0;
+        if (q_ok) q_rank = atomicAdd(&s_start[1][id[2] - 1], 1);
+        if (grad && bt == 0) {  // the tokens met most often, by a hash
+            const auto count = [&](int t, int tok) {
+                const int h = t * kTeHash + tok_hash(tok, 10);
+                atomicAdd(&s_cnt[h], 1);
+                s_tok[h] = tok;
+            };
+#pragma unroll
+            for (int k = 0; k < 2; ++k)
+                if (e_ok[k]) {
+                    count(0, edge[k].x);
+                    count(1, edge[k].y);
+                }
+            if (q_ok) {
+                count(0, id[0]);
+                count(1, id[1]);
+                count(0, id[3]);
+                count(1, id[4]);
+            }
+        }
+        __syncthreads();
+        if (warp < 2) {  // a depth's count becomes the place of its first item, and behind the last depth stands their number
+            const int v = s_start[warp][lane];
+            int incl = v;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int t = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+                if (lane >= o) incl += t;
+            }
+            s_start[warp][lane] = incl - v;
+            if (lane == 31) s_start[warp][kMaxL] = incl;
+        }
+        if (grad && bt == 0) {
+            const int least = max(8, (ne + 2 * nq) / 64);
+            for (int i = tid; i < 2 * kTeHash; i += kTeThreads) {
+                const int t = i / kTeHash;
+                if (s_cnt[i] >= least) {
+                    const int slot = atomicAdd(&s_nhot[t], 1);
+                    if (slot < kTsSlots) s_hot.tok[t][slot] = s_tok[i];
+                }
+            }
+        }
+        __syncthreads();
+        if (grad && bt == 0)
+            for (int i = tid; i < kTeWarps * 2 * kTsSlots * 32; i += kTeThreads) s_rows[i] = zero4;
+        const auto slot_of = [&](int t, int tok) { return grad ? hot_slot(s_hot, t, tok) + 1 : 0; };  // 0: none
+#pragma unroll
+        for (int k = 0; k < 2; ++k)
+            if (e_ok[k])
+                s_edge[s_start[0][edge[k].z - 1] + e_rank[k]] = make_int4(edge[k].x, edge[k].y, edge[k].w ? 1 : 0, slot_of(0, edge[k].x) | slot_of(1, edge[k].y) << 4);
+        if (q_ok) {
+            const int at = s_start[1][id[2] - 1] + q_rank;
+            s_pair[at] = make_int4(id[0], id[1], id[3], id[4]);
+            s_pinfo[at] = id[5] | slot_of(0, id[0]) << 8 | slot_of(1, id[1]) << 12 | slot_of(0, id[3]) << 16 | slot_of(1, id[4]) << 20;
+        }
+        __syncthreads();
+        // ---- edge level (Eq. 11): a warp's stretch of the sorted edges, up to eight of one depth at a time
+        {
+            const int n = s_start[0][kMaxL];
+            int i = n * warp / kTeWarps;
+            const int hi = n * (warp + 1) / kTeWarps;
+            int d = 0, d_end = 0;
+            float4 u = zero4, gu = zero4;
+            while (i < hi) {
+                if (i >= d_end) {  // the next depth that has an edge
+                    add_gu(d, gu);
+                    do {
+                        ++d;
+                        d_end = s_start[0][d];
+                    } while (i >= d_end);
+                    u = ctx_u<FULL>(c, d);
+                    gu = zero4;
+                }
+                const int cnt = min(8, min(hi, d_end) - i);
+                float4 a[8], b[8];
+#pragma unroll
+                for (int q = 0; q < 8; ++q) {
+                    const int2 e = *(const int2*)(s_edge + i + min(q, cnt - 1));  // (past the last: it again, and no additions)
+                    a[q] = ctx_load<FULL>(c, p.P, e.x);
+                    b[q] = ctx_load<FULL>(c, p.C, e.y);
+                }
+                const bool mine = (lane >> 2) < cnt;
+                const bool good = s_edge[i + min(lane >> 2, cnt - 1)].z != 0;
+                float part[8];
+#pragma unroll
+                for (int q = 0; q < 8; ++q) {
+                    a[q] = add4(a[q], u);
+                    b[q] = add4(b[q], u);
+                    part[q] = dot4(a[q], b[q]);
+                }
+                const float dot = warp_sums<8>(part, lane);  // lanes 4 q .. 4 q + 3: edge q
+                const float f = p.k0 * dot;
+                const float fy = good ? -f : f, e = expf(-fabsf(fy)), w = good ? p.w1 : 1.f;  // softplus(fy), sigmoid(fy)
+                const float gf = mine && grad ? (good ? -p.w_bce : p.w_bce) * w * ((fy >= 0.f ? 1.f : e) / (1.f + e)) : 0.f;
+                if (mine && (lane & 3) == 0) {
+                    l_bce += (double)(w * (fmaxf(fy, 0.f) + log1pf(e)));
+                    gs += gf * dot * p.inv_sqrt_m;
+                }
+                if (grad) {
+                    const float coef = gf * p.k0;
+#pragma unroll
+                    for (int q = 0; q < 8; ++q) {
+                        if (q >= cnt) break;  // (uniform)
+                        const float cf = __shfl_sync(0xFFFFFFFFu, coef, 4 * q);
+                        const int4 e = s_edge[i + q];
+                        ctx_add_row<FULL>(p, c, 0, e.x, (e.w & 15) - 1, mul4(cf, b[q]));
+                        ctx_add_row<FULL>(p, c, 1, e.y, (e.w >> 4) - 1, mul4(cf, a[q]));
+                        gu = fma4(cf, add4(a[q], b[q]), gu);
+                    }
+                }
+                i += cnt;
+            }
+            add_gu(d, gu);
+        }
+        // ---- pairwise level (Eq. 10): four pairs at a time, sorted by the first one's depth
+        {
+            const int n = s_start[1][kMaxL];
+            int i = n * warp / kTeWarps;
+            const int hi = n * (warp + 1) / kTeWarps;
+            int d = 0, d_end = 0;
+            float4 u = zero4, gu = zero4;
+            while (i < hi) {
+                if (i >= d_end) {
+                    add_gu(d, gu);
+                    do {
+                        ++d;
+                        d_end = s_start[1][d];
+                    } while (i >= d_end);
+                    u = ctx_u<FULL>(c, d);
+                    gu = zero4;
+                }
+                const int cnt = min(4, min(hi, d_end) - i);
+                float4 a1[4], b1[4], a2[4], b2[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const int4 e = s_pair[i + min(q, cnt - 1)];
+                    a1[q] = ctx_load<FULL>(c, p.P, e.x);
+                    b1[q] = ctx_load<FULL>(c, p.C, e.y);
+                    a2[q] = ctx_load<FULL>(c, p.P, e.z);
+                    b2[q] = ctx_load<FULL>(c, p.C, e.w);
+                }
+                float part[8];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const int d2 = s_pinfo[i + min(q, cnt - 1)] & 255;
+                    const float4 u2 = d2 == d ? u : ctx_u<FULL>(c, d2);  // (uniform)
+                    a1[q] = add4(a1[q], u);
+                    b1[q] = add4(b1[q], u);
+                    a2[q] = add4(a2[q], u2);
+                    b2[q] = add4(b2[q], u2);
+                    part[2 * q] = dot4(a1[q], b1[q]);
+                    part[2 * q + 1] = dot4(a2[q], b2[q]);
+                }
+                const float dot = warp_sums<8>(part, lane);  // lanes 8 q .. 8 q + 3: v+ of pair q, the next four: v-
+                const float other = __shfl_xor_sync(0xFFFFFFFFu, dot, 4);
+                const float dp = (lane & 4) ? other : dot, dm = (lane & 4) ? dot : other;
+                const float x = p.gamma - p.k0 * dp + p.k0 * dm;
+                const bool mine = (lane >> 3) < cnt;
+                const float e = expf(-fabsf(x));
+                const float gx = mine && grad ? p.w_pair * ((x >= 0.f ? 1.f : e) / (1.f + e)) : 0.f;
+                if (mine && (lane & 7) == 0) {
+                    l_pair += (double)(fmaxf(x, 0.f) + log1pf(e));
+                    gs += gx * (dm - dp) * p.inv_sqrt_m;
+                }
+                if (grad) {
+                    const float coef = gx * p.k0;  // of v-; v+ gets its negative
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        if (q >= cnt) break;  // (uniform)
+                        const float cf = __shfl_sync(0xFFFFFFFFu, coef, 8 * q);
+                        const int4 e = s_pair[i + q];
+                        const int info = s_pinfo[i + q];
+                        const int h1 = (info >> 8 & 15) - 1, h2 = (info >> 12 & 15) - 1, h3 = (info >> 16 & 15) - 1, h4 = (info >> 20 & 15) - 1;
+                        if (e.x == e.z) {  // (uniform; an alternative keeps the pair's parent or its child: one addition for both)
+                            ctx_add_row<FULL>(p, c, 0, e.x, h1, mul4(cf, sub4(b2[q], b1[q])));
+                        } else {
+                            ctx_add_row<FULL>(p, c, 0, e.x, h1, mul4(-cf, b1[q]));
+                            ctx_add_row<FULL>(p, c, 0, e.z, h3, mul4(cf, b2[q]));
+                        }
+                        if (e.y == e.w) {
+                            ctx_add_row<FULL>(p, c, 1, e.y, h2, mul4(cf, sub4(a2[q], a1[q])));
+                        } else {
+                            ctx_add_row<FULL>(p, c, 1, e.y, h2, mul4(-cf, a1[q]));
+                            ctx_add_row<FULL>(p, c, 1, e.w, h4, mul4(cf, a2[q]));
+                        }
+                        const float4 s1 = add4(a1[q], b1[q]), s2 = add4(a2[q], b2[q]);
+                        if ((info & 255) == d) {
+                            gu = fma4(cf, sub4(s2, s1), gu);
+                        } else {
+                            gu = fma4(-cf, s1, gu);
+                            add_gu(info & 255, mul4(cf, s2));
+                        }
+                    }
+                }
+                i += cnt;
+            }
+            add_gu(d, gu);
+        }
+        __syncthreads();
+    }
+    if (grad && n_batch > 0) {
+        for (int i = tid; i < Lm / 4; i += kTeThreads) red_add4((float4*)p.gu + i, ((const float4*)s_gu)[i]);
+        for (int i = tid; i < 2 * kTsSlots * 32; i += kTeThreads) {
             const int r = i >> 5, l = i & 31, tok = s_hot.tok[r / kTsSlots][r % kTsSlots];
             if (tok < 0 || l >= p.m / 4) continue;
             float4 v = zero4;
-            for (int w = 0; w < kTsWarps; ++w) v = add4(v, ((const float4*)s_rows)[(size_t)w * 2 * kTsSlots * 32 + i]);
-            atomicAdd((float4*)((r < kTsSlots ? p.gP : p.gC) + (size_t)tok * p.m) + l, v);
+            for (int w = 0; w < kTeWarps; ++w) v = add4(v, s_rows[w * 2 * kTsSlots * 32 + i]);
+            red_add4((float4*)((r < kTsSlots ? p.gP : p.gC) + (size_t)tok * p.m) + l, v);
         }
     }
-    if (tid == 0) {
-        atomicAdd(p.acc + 0, s_loss[0]);
-        atomicAdd(p.acc + 1, s_loss[1]);
-        atomicAdd(p.acc + 2, s_loss[2]);
-        if (s_skip) atomicAdd((int*)(p.acc + 3), s_skip);
-        if (grad && s_gs != 0.f) atomicAdd(p.gs, s_gs);
-        __threadfence();
-        s_last = atomicAdd((unsigned int*)(p.acc + 4), 1u) == gridDim.x - 1;
-        if (s_last) {  // the CTA that finishes last writes the losses and clears the sums for the next call
-            __threadfence();
-            const double kl = __ldcg(p.acc + 0) / (double)(p.n_groups > 0 ? p.n_groups : 1);
-            const double pr = __ldcg(p.acc + 1) / (double)(p.n_pairs > 0 ? p.n_pairs : 1);
-            const double bc = __ldcg(p.acc + 2) / (double)(p.n_edges > 0 ? p.n_edges : 1);
-            p.loss[0] = kl;
-            p.loss[1] = pr;
-            p.loss[2] = bc;
-            p.loss[3] = (double)p.lam_kl * kl + (double)p.lam_pair * pr + (double)p.lam_bce * bc;
-            if (p.skipped) *p.skipped = __ldcg((const int*)(p.acc + 3));
-            for (int i = 0; i < 5; ++i) p.acc[i] = 0.0;
-        }
-    }
+    train_finish(p, s_sum, 0.0, l_pair, l_bce, gs, skipped, lane);
+    pdl_wait();  // (the end of this kernel stands for the end of both)
 }
+
 
 }  // namespace
 
@@ -786,11 +1380,28 @@ static int rows_gu_copies(const graft_config& cfg) { return cfg.L * cfg.m <= 204
 static size_t tdes_loss_smem(const graft_config& cfg) {
     const size_t lm = (size_t)((cfg.L * cfg.m + 3) & ~3);
     if (cfg.m > 128) return lm * sizeof(float);  // gu
-    return (lm * (1 + rows_gu_copies(cfg)) + (size_t)kTsWarps * 2 * kTsSlots * 128) * sizeof(float);
+    return lm * (1 + rows_gu_copies(cfg)) * sizeof(float);
 }
 static void (*rows_kernel(const graft_config& cfg))(const TrainParams) {
     if (cfg.m == 128) return cfg.K <= 8 ? tdes_loss_rows_kernel<8, true> : (cfg.K <= 16 ? tdes_loss_rows_kernel<16, true> : tdes_loss_rows_kernel<32, true>);
     return cfg.K <= 8 ? tdes_loss_rows_kernel<8, false> : (cfg.K <= 16 ? tdes_loss_rows_kernel<16, false> : tdes_loss_rows_kernel<32, false>);
+}
+
+static void (*groups_kernel(const graft_config& cfg))(const TrainParams) {
+    if (cfg.m == 128) return cfg.K <= 8 ? tdes_groups_kernel<8, true> : (cfg.K <= 16 ? tdes_groups_kernel<16, true> : tdes_groups_kernel<32, true>);
+    return cfg.K <= 8 ? tdes_groups_kernel<8, false> : (cfg.K <= 16 ? tdes_groups_kernel<16, false> : tdes_groups_kernel<32, false>);
+}
+static size_t groups_smem(const graft_config& cfg, int batch) {
+    const int kc = cfg.K <= 8 ? 8 : (cfg.K <= 16 ? 16 : 32);
+    return (size_t)batch * (512 + kc * (sizeof(float) + sizeof(int) + sizeof(uint16_t))) + 64 + kTgBins / 2 * sizeof(uint32_t) + 2 * (size_t)cfg.L * cfg.m * sizeof(float);
+}
+static int groups_batch(const graft_config& cfg) {  // (L m = 2048: all 224; 4096: 208)
+    int n = kTgGroups;
+    while (groups_smem(cfg, n) > (size_t)220 * 1024) n -= 8;
+    return n;
+}
+static size_t items_smem(const graft_config& cfg) {
+    return (size_t)(kTeEdges + kTePairs) * sizeof(int4) + kTePairs * sizeof(int) + (size_t)kTeWarps * 2 * kTsSlots * 512 + 2 * (size_t)cfg.L * cfg.m * sizeof(float);
 }
 
 cudaError_t tdes_loss_launch(graft_ctx* ctx, const graft_tdes_traces* tr, const graft_tdes_loss_config* lc,
@@ -836,14 +1447,36 @@ cudaError_t tdes_loss_launch(graft_ctx* ctx, const graft_tdes_traces* tr, const 
     if (cfg.m <= 128 && items > 0) {
         p.acc = ctx->w_loss;
         p.gu_copies = rows_gu_copies(cfg);
-        p.sample = (long long)tr->n_groups * (cfg.K + 1) + 4ll * tr->n_pairs + 2ll * tr->n_edges >= kTsSampleMin;
         // a warp takes a group, eight pairs or eight edges at a time
         const long long work = (long long)tr->n_groups + (tr->n_pairs + 7ll) / 8 + (tr->n_edges + 7ll) / 8;
         long long grid = (work + kTsWarps - 1) / kTsWarps;
         if (grid > ctx->num_sms) grid = ctx->num_sms;
-        rows_kernel(cfg)<<<(int)grid, kTsThreads, smem, st>>>(p);
-        ctx->launches += 1;
-        return cudaGetLastError();
+        const long long refs = (long long)tr->n_groups * (cfg.K + 1) + 4ll * tr->n_pairs + 2ll * tr->n_edges;
+        if (refs < (d_gP ? kTsMany : kTsManyLoss)) {
+            p.ctas = (int)grid;
+            rows_kernel(cfg)<<<(int)grid, kTsThreads, smem, st>>>(p);
+            ctx->launches += 1;
+            return cudaGetLastError();
+        }
+        const int n_g = tr->n_groups > 0 ? ctx->num_sms : 0, n_i = tr->n_pairs + tr->n_edges > 0 ? ctx->num_sms : 0;
+        p.ctas = n_g + n_i;
+        p.g_batch = groups_batch(cfg);
+        cudaError_t e = cudaSuccess;
+        if (n_g > 0) {
+            groups_kernel(cfg)<<<n_g, kTgThreads, groups_smem(cfg, p.g_batch), st>>>(p);
+            ctx->launches += 1;
+            e = cudaGetLastError();
+        }
+        if (n_i > 0 && e == cudaSuccess) {
+            void (*items)(const TrainParams) = cfg.m == 128 ? tdes_items_kernel<true> : tdes_items_kernel<false>;
+            if (n_g > 0)
+                e = launch_pdl(items, dim3(n_i), dim3(kTeThreads), items_smem(cfg), st, p);
+            else
+                items<<<n_i, kTeThreads, items_smem(cfg), st>>>(p);
+            ctx->launches += 1;
+            if (e == cudaSuccess) e = cudaGetLastError();
+        }
+        return e;
     }
     cudaError_t e = cudaMemsetAsync(d_loss, 0, 4 * sizeof(double), st);
     if (e != cudaSuccess) return e;
@@ -865,8 +1498,11 @@ cudaError_t tdes_loss_launch(graft_ctx* ctx, const graft_tdes_traces* tr, const 
 
 cudaError_t tdes_loss_configure(const graft_config& cfg) {
     const size_t smem = tdes_loss_smem(cfg);
-    if (cfg.m <= 128) return allow_smem((const void*)rows_kernel(cfg), smem);
-    return allow_smem((const void*)(cfg.m <= 256 ? tdes_loss_kernel<2> : tdes_loss_kernel<kTrMaxChunks>), smem);
+    if (cfg.m > 128) return allow_smem((const void*)(cfg.m <= 256 ? tdes_loss_kernel<2> : tdes_loss_kernel<kTrMaxChunks>), smem);
+    cudaError_t e = allow_smem((const void*)rows_kernel(cfg), smem);
+    if (e == cudaSuccess) e = allow_smem((const void*)groups_kernel(cfg), groups_smem(cfg, groups_batch(cfg)));
+    if (e == cudaSuccess) e = allow_smem((const void*)(cfg.m == 128 ? tdes_items_kernel<true> : tdes_items_kernel<false>), items_smem(cfg));
+    return e;
 }
 bool tdes_loss_supported(const graft_config& cfg) { return cfg.m % 4 == 0 && cfg.m <= 128 * kTrMaxChunks; }
 

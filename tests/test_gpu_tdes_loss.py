@@ -168,6 +168,65 @@ def test_empty_lists_and_argument_checks():
     g.destroy()
 
 
+@pytest.mark.parametrize("V,L,K,m,ng,npair,ne,grad", [
+    (3000, 16, 32, 128, 3000, 6000, 9000, True),      # every instance of the two kernels for many traces
+    (3000, 16, 17, 124, 4000, 9001, 16003, True),     # lanes without a part of a row, places without a child
+    (3000, 32, 16, 128, 5000, 7000, 13000, True),     # L m = 4096
+    (3000, 7, 9, 64, 7000, 9001, 13003, True),
+    (3000, 16, 8, 128, 8000, 9000, 13000, True),
+    (60000, 32, 32, 128, 4001, 3, 5, True),           # nearly every child is met once; CTAs without an item
+    (2000, 5, 3, 32, 34000, 0, 0, True),              # groups alone, two batches a CTA
+    (700, 16, 8, 128, 0, 40000, 0, True),             # pairs alone
+    (700, 16, 8, 128, 0, 0, 160000, True),            # edges alone, two batches a CTA
+    (20, 16, 8, 128, 13000, 9000, 13000, True),       # a bin holds most of a batch
+    (3000, 16, 32, 128, 19000, 6000, 9000, False),    # the losses alone
+])
+def test_many_traces(V, L, K, m, ng, npair, ne, grad):
+    g, P, Ct, u, s, keep = _ctx(V, L, K, m, seed=V + K)
+    tr = gi.tdes_traces(V, L, K, ng, npair, ne, seed=V + L)
+    tr["pairs"][::5, 5] = 1 + (tr["pairs"][::5, 5] + 2) % L  # an alternative of another depth
+    got = _run(g, V, L, m, tr, grad=grad)
+    _compare(got, oracle.tdes_loss(P, Ct, u, s, tr["groups"], tr["pairs"], tr["edges"], **CFG), grad=grad)
+    assert got["skipped"][0] == 0
+    g.destroy()
+
+
+def test_many_traces_bad_ids_and_lists_at_odd_addresses():
+    V, L, K, m, ng, npair, ne = 900, 6, 8, 128, 9000, 9000, 16000
+    g, P, Ct, u, s, keep = _ctx(V, L, K, m, seed=41)
+    tr = gi.tdes_traces(V, L, K, ng, npair, ne, seed=42)
+    gr = {k: v.copy() for k, v in tr["groups"].items()}
+    pairs, edges = tr["pairs"].copy(), tr["edges"].copy()
+    bad = np.arange(0, 9000, 10)
+    gr["parent"][bad[0::3]] = V
+    gr["child"][bad[1::3], 2] = -1
+    gr["depth"][bad[2::3]] = L + 1
+    pairs[bad[0::2], 4] = V + 7
+    pairs[bad[1::2], 5] = 0
+    edges[bad, 0] = -5
+    odd = torch.zeros(1 + pairs.size, dtype=torch.int32, device="cuda")[1:]  # four bytes behind a boundary
+    odd.copy_(torch.from_numpy(pairs.reshape(-1)))
+    odd_e = torch.zeros(1 + edges.size, dtype=torch.int32, device="cuda")[1:]
+    odd_e.copy_(torch.from_numpy(edges.reshape(-1)))
+    out = dict(loss=torch.zeros(4, dtype=torch.float64, device="cuda"), skipped=torch.zeros(1, dtype=torch.int32, device="cuda"),
+               gP=torch.zeros((V, m), device="cuda"), gC=torch.zeros((V, m), device="cuda"), gu=torch.zeros((L, m), device="cuda"),
+               gs=torch.zeros(1, device="cuda"))
+    groups = {k: torch.from_numpy(np.ascontiguousarray(v)).cuda() for k, v in gr.items()}
+    g.tdes_loss(groups, odd.view(npair, 6), odd_e.view(ne, 4), **out, **CFG)
+    torch.cuda.synchronize()
+    got = {k: v.cpu().numpy() for k, v in out.items()}
+    n = len(bad)
+    assert got["skipped"][0] == 3 * n
+    left = np.setdiff1d(np.arange(9000), bad)
+    sub = dict(groups={k: v[left] for k, v in gr.items()}, pairs=np.delete(pairs, bad, 0), edges=np.delete(edges, bad, 0))
+    share = np.array([1 - n / ng, 1 - n / npair, 1 - n / ne])
+    cfg = dict(CFG, **{k: CFG[k] * x for k, x in zip(("lambda_kl", "lambda_pair", "lambda_bce"), share)})
+    ref = oracle.tdes_loss(P, Ct, u, s, sub["groups"], sub["pairs"], sub["edges"], **cfg)
+    ref["loss"][:3] *= share
+    _compare(got, ref)
+    g.destroy()
+
+
 def test_full_size_tables():
     """The paper's shapes: V = 151,936, m = 128, L = 16, K = 32; tens of thousands of items."""
     V, L, K, m = 151936, 16, 32, 128
