@@ -18,10 +18,10 @@
 // One persistent kernel.  A worker -- a pair of CTAs (cluster of two, tcgen05 cta_group::2) for bf16 embeddings, one CTA
 // for fp32 -- owns a tile of 512 (fp32: 128) rows of V times up to 128 columns of m, and streams E in blocks of 64 (32)
 // columns through shared-memory rings.
-//   warps 0-7    empty the accumulators (TMEM, two sets of 2 x 128 columns), keep the running sums and write the tile
+//   warps 0-7    empty the accumulators (TMEM, two sets of 2 x 128 columns; fp32: kTmLo), keep the running sums and write the tile
 //   warp 8       TMA loads: W's parts (split once per call into scratch by a small kernel), bf16 embeddings
 //   warp 9       issues the matrix instructions
-//   warp 10      fp32 only: TMA loads of the raw rows;  warps 11-18  raw rows -> fp16 parts in the operands' layout
+//   warp 10      fp32 only: TMA loads of the raw rows;  warps 11-18  raw rows -> fp16 parts in TMEM, a thread a row
 // W1 and W2 stand side by side as one operand of N = 256, the third product is an N = 128 of its own (three of N = 128 in a row on one
 // accumulator took 122 cycles each: an instruction waits for the one ahead of it on the same columns).  Tiles of 512
 // rows halve the passes over W, which comes from L2 every time.  The fp32 kernel works on single CTAs because its rows
@@ -30,11 +30,14 @@
 // written.  What is left when the tiles do not divide by the workers is dealt out along E in shares, whose sums a
 // small kernel adds up in order (summing them inside, by the warp that came last, stalled its tile: 462 against 370 us).
 //
-// Measured (one tower, back to back, B200): V = 151,936, E = 4096, m = 128, bf16: 355 us (376 before rows and W shared a barrier
+// Measured (one tower, back to back, B200): V = 151,936, E = 4096, m = 128, bf16: 358 us (376 before rows and W shared a barrier
 // and the first row block went two blocks ahead where accumulators are emptied; 798 us with the library template's GEMMs); its products
-// take 287 us at the measured dense rate, and the clock falls to 1.5 GHz on the way.  V = 32,000, E = 2048, fp32: 88 us (120 with
-// three bf16 parts, seven products; 1135 us by the FMA kernel).  What bounds the fp32 kernel: the one thread that issues, 0.6 k
-// cycles a block of 32 columns beside 0.4 k of products, and the eight warps that split.  Error against fp64 products at those
+// take 287 us at the measured dense rate, and the clock falls to 1.5 GHz on the way.  V = 32,000, E = 2048, fp32: 76 us (89 with the
+// parts in shared memory and one thread in the issuing loop; 120 with three bf16 parts, seven products; 1135 us by the FMA
+// kernel).  What bounds the fp32 kernel: the issuing warp, 1.05 k cycles for two blocks of 32 columns beside 0.77 k of products (910
+// cycles a block by one thread, whose operands had to be moved for every instruction), and 0.5 k more where a chunk ends; then
+// the pieces, 7 us, and W's parts, 3 us.  The parts go through TMEM because in shared memory the copies, the conversion and the
+// products' reads together moved 104 KB a block, 0.8 k cycles of its bandwidth; now 72.  Error against fp64 products at those
 // sizes, largest and root mean square over the results' size: bf16 3.4e-6 and 4.8e-7 (FMA kernel 1.7e-5, 1.1e-6); fp32 2.2e-6 and
 // 3.5e-7 (three bf16 parts 3.3e-6, 4.7e-7; FMA kernel 9.2e-6, 8.1e-7).  The accumulators round towards zero, so terms of one sign
 // are off by more: fp32 1.5e-6 and 1.1e-6 (8.0e-7 and 3.9e-7; 3.6e-6 and 6.5e-7), emptied every 8 additions 8.5e-7 and 4.7e-7 in 93
@@ -63,14 +66,13 @@ struct TablesCfg {
     static constexpr int BLK = F32 ? 32 : 64;  // columns of E per block: rows of 64 or 128 bytes of bf16
     static constexpr int CHUNK = 8;            // blocks between two emptyings of an accumulator
     static constexpr int PART = 128 * BLK * 2;                // bytes of 128 rows of 16-bit numbers
-    static constexpr int A_BYTES = 2 * PART;                  // a block's embeddings: two row blocks, or two parts
+    static constexpr int A_BYTES = F32 ? 0 : 2 * PART;        // a block's embeddings: two row blocks (fp32: two parts, in TMEM)
     static constexpr int W_BYTES = (F32 ? 256 : 192) * BLK * 2;  // a block's W; a pair: W1 (even CTA) or W2 (odd), half of W3
     static constexpr int RAW = 128 * BLK * 4;                 // a block's fp32 embeddings
-    static constexpr int STAGES = 4, RAW_STAGES = F32 ? 4 : 1;  // (a stage: a block's embeddings and W)
+    static constexpr int STAGES = 4, RAW_STAGES = F32 ? 8 : 1;  // (a stage: a block's embeddings and W)
     static constexpr int THREADS = (kTmEpiWarps + 2 + (F32 ? 1 + kTmConvWarps : 0)) * 32;
     // (the rings start on a 1024-byte boundary)
     static constexpr size_t SMEM = (size_t)STAGES * (A_BYTES + W_BYTES) + (F32 ? (size_t)RAW_STAGES * RAW : 0) + 1024;
-    static __device__ __forceinline__ uint64_t desc(uint32_t addr) { return F32 ? umma_desc_sw64(addr) : umma_desc_sw128(addr); }
 };
 
 constexpr float kTmLow = 2048.0f;  // fp16: second parts are kept times 2^11
@@ -82,6 +84,12 @@ constexpr float kTmLow = 2048.0f;  // fp16: second parts are kept times 2^11
 constexpr int kTmTarget = 4;
 constexpr float kTmLeast = 0x1p-12f, kTmMost = 65504.f;
 constexpr uint32_t kTmScales = 4;  // tiles whose rows' scales are kept
+
+// fp32 embeddings, columns of TMEM: the small products' accumulator (emptied once a tile) with the large products' on either
+// side, which take turns from chunk to chunk, so that one instruction of twice the width fills both -- W1 before W2, or behind it --
+// and the stages of the embeddings' parts.
+constexpr uint32_t kTmLo = 128, kTmParts = 384;
+__device__ __forceinline__ uint32_t tables_hi(uint32_t slot, uint32_t n) { return slot ? kTmLo + n : kTmLo - n; }
 
 // A walk over the N stages of a ring: stages passed so far, the stage, the parity to wait for.
 template <uint32_t N>
@@ -136,33 +144,46 @@ struct TablesItem {
     int q0, q1;  // a piece: the first and the last worker that work on the tile (q0 == q1: the whole tile)
     int seg;     // 0: the pair's share begins in this tile, 1: it began in the tile before
 };
-__device__ __forceinline__ int tables_share(const TablesParams& p, int pair) {
-    return (int)((long long)pair * p.left * p.n_kb / p.share_pairs);
+__device__ __forceinline__ int tables_share(const TablesParams& p, int pair) {  // (32 bits: tables_mma_fits)
+    return (int)((uint32_t)pair * (uint32_t)(p.left * p.n_kb) / (uint32_t)p.share_pairs);
 }
 __device__ __forceinline__ int tables_owner(const TablesParams& p, int block) {
-    const long long T = (long long)p.left * p.n_kb;
-    return (int)(((long long)(block + 1) * p.share_pairs + T - 1) / T - 1);
+    const uint32_t T = (uint32_t)(p.left * p.n_kb);
+    return (int)(((uint32_t)(block + 1) * (uint32_t)p.share_pairs + T - 1) / T - 1);
 }
-__device__ __forceinline__ bool tables_item(const TablesParams& p, int pair, int i, TablesItem& it) {
-    if (pair < p.share_pairs) {
-        const int x0 = tables_share(p, pair), x1 = tables_share(p, pair + 1);
-        const int t = x0 / p.n_kb + i, b0 = t * p.n_kb, b1 = b0 + p.n_kb;
-        if (b0 < x1) {
-            it.tile = t;
-            it.kb0 = x0 > b0 ? x0 - b0 : 0;
-            it.kb1 = x1 < b1 ? x1 - b0 : p.n_kb;
-            it.seg = i;
-            it.q0 = tables_owner(p, b0);
-            it.q1 = tables_owner(p, b1 - 1);
-            return true;
-        }
-        i -= (x1 - 1) / p.n_kb - x0 / p.n_kb + 1;
+// A pair's share, worked out once (by one thread, while the kernel ahead runs): a dozen divisions took the start of every role
+// 5 k cycles.
+struct TablesShare {
+    int n;           // tiles that it lies in
+    TablesItem it[2];
+};
+__device__ __forceinline__ void tables_shares(const TablesParams& p, int pair, TablesShare& s) {
+    s.n = 0;
+    if (pair >= p.share_pairs) return;
+    const int x0 = tables_share(p, pair), x1 = tables_share(p, pair + 1);
+    for (int t = x0 / p.n_kb; t * p.n_kb < x1 && s.n < 2; ++t) {
+        const int b0 = t * p.n_kb, b1 = b0 + p.n_kb;
+        TablesItem& it = s.it[s.n];
+        it.tile = t;
+        it.kb0 = x0 > b0 ? x0 - b0 : 0;
+        it.kb1 = x1 < b1 ? x1 - b0 : p.n_kb;
+        it.seg = s.n++;
+        it.q0 = tables_owner(p, b0);
+        it.q1 = tables_owner(p, b1 - 1);
     }
+}
+__device__ __forceinline__ bool tables_item(const TablesParams& p, const TablesShare& s, int pair, int i, TablesItem& it) {
+    if (i < s.n) {
+        it = s.it[i];
+        return true;
+    }
+    i -= s.n;
     if (i >= p.full_rounds) return false;
     it.tile = p.left + pair + i * p.pairs;
     it.kb0 = 0;
     it.kb1 = p.n_kb;
     it.q0 = it.q1 = pair;
+    it.seg = 0;
     return true;
 }
 
@@ -175,9 +196,20 @@ __device__ __forceinline__ int tables_n(const TablesParams& p, int mb) {
 }
 
 // W (fp32, [m, E]) -> three bf16 parts [3][m_pad][E_pad], zero where padded
-__global__ void __launch_bounds__(256) weight_split_kernel(const float* __restrict__ W, int m, int E, int m_pad, int E_pad,
-                                                           __nv_bfloat16* __restrict__ w) {
+struct SplitParams {
+    const float* W;
+    int m, E, m_pad, E_pad;
+    void* w;
+    float2* unscale;  // fp32 embeddings only, as the rest
+    uint32_t* flags;
+    int n_flags;
+};
+__global__ void __launch_bounds__(256) weight_split_kernel(const SplitParams sp) {
+    const float* __restrict__ W = sp.W;
+    const int m = sp.m, E = sp.E, m_pad = sp.m_pad, E_pad = sp.E_pad;
+    __nv_bfloat16* __restrict__ w = (__nv_bfloat16*)sp.w;
     pdl_launch_dependents();
+    pdl_wait();  // (W may come from the kernel ahead, and a table before this one may still be read from the scratch)
     const size_t part = (size_t)m_pad * E_pad;
     const int r = blockIdx.y;
     for (int e = (blockIdx.x * 256 + threadIdx.x) * 2; e < E_pad; e += gridDim.x * 512) {
@@ -207,11 +239,15 @@ __device__ __forceinline__ float2 tables_unscale(int s) { return make_float2(tab
 // W (fp32, [m, E]) -> two fp16 parts [2][m_pad][E_pad], zero where padded: a row is multiplied by the power of two that takes
 // its largest entry to [2^13, 2^14), W1 is what fp16 holds of it and W2 what it holds of the rest, times 2^11.  A block a row.  And
 // clears the flags of the embeddings' rows.
-__global__ void __launch_bounds__(256) weight_split16_kernel(const float* __restrict__ W, int m, int E, int m_pad, int E_pad,
-                                                           __half* __restrict__ w, float2* __restrict__ unscale,
-                                                           uint32_t* __restrict__ flags, int n_flags) {
+__global__ void __launch_bounds__(256) weight_split16_kernel(const SplitParams sp) {
     __shared__ float s_max[8];
+    const float* __restrict__ W = sp.W;
+    const int m = sp.m, E = sp.E, m_pad = sp.m_pad, E_pad = sp.E_pad, n_flags = sp.n_flags;
+    __half* __restrict__ w = (__half*)sp.w;
+    float2* __restrict__ unscale = sp.unscale;
+    uint32_t* __restrict__ flags = sp.flags;
     pdl_launch_dependents();
+    pdl_wait();  // (as above)
     const int r = blockIdx.x, tid = threadIdx.x;
     // the row's largest finite entry; up to E = 4096 the row stays in registers
     constexpr int N = 16;
@@ -259,9 +295,6 @@ __device__ __forceinline__ void split2(float x0, float x1, float scale, uint32_t
     const float2 y = __half22float2(*(const __half2*)&a);
     const float2 z = __fmul2_rn(make_float2(x.x - y.x, x.y - y.y), make_float2(kTmLow, kTmLow));
     b = cvt_f16x2(z.x, z.y);
-}
-__device__ __forceinline__ void st_shared_v4(uint32_t at, const uint32_t (&v)[4]) {
-    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(at), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]) : "memory");
 }
 __device__ __forceinline__ void st_global_v8(float* dst, const float* v) {
     asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst), "f"(v[0]), "f"(v[1]), "f"(v[2]),
@@ -346,12 +379,13 @@ __global__ void __cluster_dims__(F32 ? 1 : 2, 1, 1) __launch_bounds__(TablesCfg<
     using C = TablesCfg<F32>;
     constexpr uint32_t NS = C::STAGES, NR = C::RAW_STAGES;
     extern __shared__ unsigned char smem_raw[];
-    __shared__ __align__(8) uint64_t bars[2 * (NS + NR) + 4 + 2 * kTmScales];
+    __shared__ __align__(8) uint64_t bars[2 * (NS + NR) + 5 + 2 * kTmScales];
     __shared__ uint8_t s_scale[F32 ? kTmScales : 1][128];  // the exponents (biased) of what the rows of the last tiles are multiplied by
     __shared__ float2 s_unscale[F32 ? 512 : 1];  // what columns are multiplied by (from memory at a tile's end: V = 30,000, E = 32 22.0 us, so 18.5)
     __shared__ uint32_t s_tmem;
     __shared__ volatile int s_abort;
     __shared__ bool s_mend;
+    __shared__ TablesShare s_share;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const uint32_t rank = C::PAIR ? cluster_ctarank() : 0u;
     const int pair = C::PAIR ? (int)blockIdx.x >> 1 : (int)blockIdx.x;
@@ -368,6 +402,7 @@ __global__ void __cluster_dims__(F32 ? 1 : 2, 1, 1) __launch_bounds__(TablesCfg<
     // the bottleneck of short blocks, every wait and every commit costs it a hundred cycles.)
     const uint32_t full0 = smem_u32(bars), empty0 = full0 + 8 * NS, rfull0 = empty0 + 8 * NS, rempty0 = rfull0 + 8 * NR;
     const uint32_t accfull0 = rempty0 + 8 * NR, accempty0 = accfull0 + 16, sfull0 = accempty0 + 16, sempty0 = sfull0 + 8 * kTmScales;
+    const uint32_t loempty = sempty0 + 8 * kTmScales;  // fp32: the small products' accumulator has been emptied
     if (tid == 0) {
         for (uint32_t s = 0; s < NS; ++s) {
             mbar_init(full0 + 8 * s, F32 ? kTmConvWarps / 2 + 1 : 1);
@@ -385,10 +420,12 @@ __global__ void __cluster_dims__(F32 ? 1 : 2, 1, 1) __launch_bounds__(TablesCfg<
             mbar_init(sfull0 + 8 * s, kTmConvWarps / 2);
             mbar_init(sempty0 + 8 * s, kTmEpiWarps + kTmConvWarps);
         }
+        mbar_init(loempty, kTmEpiWarps);
         mbar_fence_init();
         s_abort = 0;
         s_mend = false;
     }
+    if (tid == 32) tables_shares(p, pair, s_share);
     pdl_launch_dependents();  // (the kernel that adds up the pieces; it waits for this grid)
     if (warp == 9) tmem_alloc<C::PAIR>(smem_u32(&s_tmem), 512);
     tc_fence_before();
@@ -409,7 +446,7 @@ __global__ void __cluster_dims__(F32 ? 1 : 2, 1, 1) __launch_bounds__(TablesCfg<
             for (int c = tid; c < p.m_pad; c += kTmEpiWarps * 32) s_unscale[c] = __ldg(p.unscale + c);
             named_bar_sync(3, kTmEpiWarps * 32);
         }
-        for (int i = 0; tables_item(p, pair, i, it); ++i) {
+        for (int i = 0; tables_item(p, s_share, pair, i, it); ++i) {
             const int rt = it.tile / p.n_mb, mb = it.tile - rt * p.n_mb;
             const uint32_t n = (uint32_t)tables_n<F32>(p, mb);
             int row_exp = 127;  // (fp32) the exponent of what this thread's row is multiplied by
@@ -431,18 +468,21 @@ __global__ void __cluster_dims__(F32 ? 1 : 2, 1, 1) __launch_bounds__(TablesCfg<
                     const uint32_t slot = C::MT == 1 ? (cc & 1u) : (uint32_t)h;
                     wait(accfull0 + 8 * slot, (C::MT == 1 ? cc >> 1 : cc) & 1u);
                     tc_fence_after();
-                    const uint32_t t0 = tmem + ((uint32_t)(32 * quarter) << 16) + slot * 256u + (uint32_t)half * 64u;
+                    const uint32_t t0 = tmem + ((uint32_t)(32 * quarter) << 16) + (uint32_t)half * 64u;
+                    const uint32_t hi = F32 ? tables_hi(slot, n) : slot * 256u, lo = F32 ? kTmLo : slot * 256u + n;
+                    const bool both = !F32 || kb + C::CHUNK >= it.kb1;  // (fp32: the small products' sums at the tile's end)
 #pragma unroll
                     for (int q = 0; q < 4; ++q) {
 #pragma unroll
-                        for (int lo = 0; lo < 2; ++lo) {
+                        for (int j = 0; j < 2; ++j) {
+                            if (j == 1 && !both) break;
                             uint32_t d[16];
-                            tmem_ld_32x16(t0 + n * lo + 16u * q, d);
+                            tmem_ld_32x16(t0 + (j ? lo : hi) + 16u * q, d);
                             tmem_wait_ld();
 #pragma unroll
                             for (int c = 0; c < 16; ++c) {
                                 const float x = __uint_as_float(d[c]);
-                                acc[h][16 * q + c] = F32 && lo ? fmaf(x, 1.0f / kTmLow, acc[h][16 * q + c]) : acc[h][16 * q + c] + x;
+                                acc[h][16 * q + c] = F32 && j ? fmaf(x, 1.0f / kTmLow, acc[h][16 * q + c]) : acc[h][16 * q + c] + x;
                             }
                         }
                     }
@@ -453,6 +493,7 @@ __global__ void __cluster_dims__(F32 ? 1 : 2, 1, 1) __launch_bounds__(TablesCfg<
                             mbar_arrive_cluster(accempty_even + 8 * slot);
                         else
                             mbar_arrive(accempty0 + 8 * slot);
+                        if (F32 && both) mbar_arrive(loempty);
                     }
                 }
             }
@@ -512,7 +553,7 @@ __global__ void __cluster_dims__(F32 ? 1 : 2, 1, 1) __launch_bounds__(TablesCfg<
             named_bar_sync(1, (kTmEpiWarps + kTmConvWarps) * 32);  // (the tiles are written, their rows looked at; the rings are done with)
             if (s_mend && !s_abort) {
                 TablesMend* const sm = (TablesMend*)(smem_raw + (a_ring - smem_u32(smem_raw)));
-                for (int i = 0; tables_item(p, pair, i, it); ++i) {
+                for (int i = 0; tables_item(p, s_share, pair, i, it); ++i) {
                     if (it.q0 != it.q1) continue;  // (pieces: the kernel that adds them up)
                     // the tile's flagged rows, 32 at a time; every warp looks at all flags
                     uint32_t again[C::ROWS / 32];
@@ -546,7 +587,8 @@ __global__ void __cluster_dims__(F32 ? 1 : 2, 1, 1) __launch_bounds__(TablesCfg<
         if (lane == 0) {
             const uint32_t full_even = mapa_u32(full0, 0);
             TablesRing<NS> w(1);
-            for (int i = 0; tables_item(p, pair, i, it); ++i) {
+            uint32_t cc = 0;  // chunks ahead of this tile
+            for (int i = 0; tables_item(p, s_share, pair, i, it); cc += (uint32_t)(it.kb1 - it.kb0 + C::CHUNK - 1) / C::CHUNK, ++i) {
                 const int rt = it.tile / p.n_mb, mb = it.tile - rt * p.n_mb;
                 const int n = tables_n<F32>(p, mb);
                 const int w12 = (int)rank * p.m_pad + mb * 128, w3 = 2 * p.m_pad + mb * 128 + (int)rank * (n >> 1);
@@ -567,9 +609,10 @@ __global__ void __cluster_dims__(F32 ? 1 : 2, 1, 1) __launch_bounds__(TablesCfg<
                     } else {
                         const uint32_t part = (uint32_t)n * C::BLK * 2;
                         mbar_arrive_expect_tx(full0 + 8 * w.st, 2u * part);
+                        const int swap = (int)(cc + (uint32_t)(kb - it.kb0) / C::CHUNK) & 1;  // (tables_hi)
 #pragma unroll
                         for (int j = 0; j < 2; ++j)
-                            tma_load_2d(dw + j * part, &p.map_w, x, j * p.m_pad + mb * 128, full0 + 8 * w.st);
+                            tma_load_2d(dw + (j ^ swap) * part, &p.map_w, x, j * p.m_pad + mb * 128, full0 + 8 * w.st);
                     }
                     w.next();
                 }
@@ -580,85 +623,122 @@ __global__ void __cluster_dims__(F32 ? 1 : 2, 1, 1) __launch_bounds__(TablesCfg<
         }
     } else if (warp == 9) {
         // ------------------------------ matrix instructions --------------------------------------
-        if (rank == 0 && lane == 0) {
+        if constexpr (F32) {
+            // The tensor cores stand still while this warp does anything but issue (few instructions are queued), so a block is a
+            // wait, four instructions and a commit with next to nothing around them.  The whole warp goes through the loop, and one
+            // lane issues: the operands are the same in all lanes that way, and stay in the registers that the instructions want.
             TablesRing<NS> w(0);
+            const uint32_t tm = __shfl_sync(0xFFFFFFFFu, tmem, 0), lead = lane == 0 ? 1u : 0u;
             uint32_t cc = 0;
-            for (int i = 0; tables_item(p, pair, i, it); ++i) {
-                const int mb = it.tile % p.n_mb;
-                const int n = tables_n<F32>(p, mb);
-                constexpr int M = C::PAIR ? 256 : 128;
-                const uint32_t idesc2 = umma_idesc(M, 2 * n, !F32), idesc1 = umma_idesc(M, n, !F32);
-                constexpr uint32_t o_w3 = 2 * (C::W_BYTES / 3);  // (bf16)
-                // A pair takes two blocks at a time.  An instruction whose accumulator columns the one just ahead of it wrote waits
-                // for those, so with two row blocks their instructions alternate, except in the first and the last two blocks of a
-                // chunk, where the first row block goes ahead: its accumulators are emptied (or were) while the second's are filled.
-                constexpr int G = C::MT;
-                for (int kb = it.kb0; kb < it.kb1; kb += G) {
-                    const int g = kb + G <= it.kb1 ? G : it.kb1 - kb;
-                    const bool first = (kb - it.kb0) % C::CHUNK == 0;
-                    const bool last = kb + g == it.kb1 || (kb + g - it.kb0) % C::CHUNK == 0;
-                    uint32_t a0[G], b0[G], done[G];
-#pragma unroll
-                    for (int k = 0; k < G; ++k) {
-                        if (k >= g) break;
-                        wait(full0 + 8 * w.st, w.ph);
-                        a0[k] = a_ring + w.st * C::A_BYTES;
-                        b0[k] = w_ring + w.st * C::W_BYTES;
-                        done[k] = empty0 + 8 * w.st;
+            for (int i = 0; tables_item(p, s_share, pair, i, it); ++i) {
+                const uint32_t n = (uint32_t)p.box_n, idesc2 = umma_idesc(128, 2 * n, false), idesc1 = umma_idesc(128, n, false);
+                constexpr uint64_t kHi = umma_desc_sw64(0u);
+                const uint32_t wn = n * C::BLK * 2 / 16, lo = tm + kTmLo;
+                if (i > 0) wait(loempty, (uint32_t)(i - 1) & 1u);
+                for (int kb = it.kb0; kb < it.kb1; kb += C::CHUNK, ++cc) {
+                    const uint32_t slot = cc & 1u, hi = tm + tables_hi(slot, n), both = slot ? lo : hi, o_w1 = slot ? wn : 0u;
+                    if (cc >= 2) wait(accempty0 + 8 * slot, ((cc >> 1) - 1u) & 1u);
+                    const int left = it.kb1 - kb < C::CHUNK ? it.kb1 - kb : C::CHUNK;
+#pragma unroll 1
+                    for (int k = 0; k < left; k += 2) {  // two blocks at a time: their waits and commits side by side
+                        const bool two = k + 1 < left;
+                        const TablesRing<NS> w0 = w;
                         w.next();
+                        wait(full0 + 8 * w0.st, w0.ph);
+                        if (two) wait(full0 + 8 * w.st, w.ph);
+                        tc_fence_after();
+                        uint32_t e1 = tm + kTmParts + 32u * w0.st;
+                        uint64_t b = kHi | ((w_ring + w0.st * C::W_BYTES) >> 4);
+                        if (k == 0) {  // the large products' accumulator starts again, the small ones' with the tile
+                            umma_ts(hi, e1, b + o_w1, idesc1, false, lead);
+                            umma_ts(lo, e1, b + (wn - o_w1), idesc1, kb > it.kb0, lead);
+                        } else {
+                            umma_ts(both, e1, b, idesc2, true, lead);
+                        }
+                        umma_ts(lo, e1 + 16u, b + o_w1, idesc1, true, lead);
+                        umma_ts(both, e1 + 8u, b + 2, idesc2, true, lead);
+                        umma_ts(lo, e1 + 24u, b + o_w1 + 2, idesc1, true, lead);
+                        if (two) {
+                            e1 = tm + kTmParts + 32u * w.st;
+                            b = kHi | ((w_ring + w.st * C::W_BYTES) >> 4);
+                            umma_ts(both, e1, b, idesc2, true, lead);
+                            umma_ts(lo, e1 + 16u, b + o_w1, idesc1, true, lead);
+                            umma_ts(both, e1 + 8u, b + 2, idesc2, true, lead);
+                            umma_ts(lo, e1 + 24u, b + o_w1 + 2, idesc1, true, lead);
+                        }
+                        umma_commit_by(empty0 + 8 * w0.st, lead);
+                        if (two) {
+                            umma_commit_by(empty0 + 8 * w.st, lead);
+                            w.next();
+                        }
                     }
+                    umma_commit_by(accfull0 + 8 * slot, lead);
+                }
+            }
+        } else if (rank == 0) {
+            TablesRing<NS> w(0);
+            const uint32_t tm = __shfl_sync(0xFFFFFFFFu, tmem, 0), lead = lane == 0 ? 1u : 0u;
+            uint32_t cc = 0;
+            for (int i = 0; tables_item(p, s_share, pair, i, it); ++i) {
+                const int n = tables_n<F32>(p, it.tile % p.n_mb);
+                const uint32_t idesc2 = umma_idesc(256, 2 * n, true), idesc1 = umma_idesc(256, n, true);
+                constexpr uint64_t kHi = umma_desc_sw128(0u);
+                constexpr uint32_t o_w3 = 2 * (C::W_BYTES / 3) / 16;
+                // Two blocks at a time.  An instruction whose accumulator columns the one just ahead of it wrote waits for those, so
+                // the two row blocks' instructions alternate, except in the first and the last two blocks of a chunk, where the
+                // first row block goes ahead: its accumulators are emptied (or were) while the second's are filled.
+                for (int kb = it.kb0; kb < it.kb1; kb += 2) {
+                    const bool two = kb + 2 <= it.kb1;
+                    const bool first = (kb - it.kb0) % C::CHUNK == 0, last = kb + 2 >= it.kb1 || (kb + 2 - it.kb0) % C::CHUNK == 0;
+                    const TablesRing<NS> w0 = w;
+                    w.next();
+                    wait(full0 + 8 * w0.st, w0.ph);
+                    if (two) wait(full0 + 8 * w.st, w.ph);
                     tc_fence_after();
-                    auto mma = [&](int k, int h, int ks, bool small) {
-                        const uint32_t d = tmem + (C::MT == 1 ? (cc & 1u) : (uint32_t)h) * 256u;
-                        const uint64_t a1 = C::desc(a0[k] + h * C::PART + 32 * ks), w12 = C::desc(b0[k] + 32 * ks);
-                        if (!small)
-                            umma<C::PAIR>(d, a1, w12, idesc2, !first || k > 0 || ks > 0);
-                        else if (F32)  // (the second part of the embeddings times W1)
-                            umma<C::PAIR>(d + (uint32_t)n, C::desc(a0[k] + C::PART + 32 * ks), w12, idesc1, true);
-                        else
-                            umma<C::PAIR>(d + (uint32_t)n, a1, C::desc(b0[k] + o_w3 + 32 * ks), idesc1, true);
+                    const uint64_t a0 = kHi | ((a_ring + w0.st * C::A_BYTES) >> 4), b0 = kHi | ((w_ring + w0.st * C::W_BYTES) >> 4);
+                    const uint64_t a1 = kHi | ((a_ring + w.st * C::A_BYTES) >> 4), b1 = kHi | ((w_ring + w.st * C::W_BYTES) >> 4);
+                    const auto large = [&](uint64_t a, uint64_t b, int h, int ks, bool more) {
+                        umma_by(tm + h * 256u, a + h * (C::PART / 16) + 2 * ks, b + 2 * ks, idesc2, more, lead);
                     };
-                    if (C::MT == 2 && !first && !last) {
-                        if (!s_abort) {
+                    const auto small = [&](uint64_t a, uint64_t b, int h, int ks) {
+                        umma_by(tm + h * 256u + (uint32_t)n, a + h * (C::PART / 16) + 2 * ks, b + o_w3 + 2 * ks, idesc1, true, lead);
+                    };
+                    if (!first && !last) {  // (two blocks)
 #pragma unroll
-                            for (int k = 0; k < G; ++k) {
-                                if (k >= g) break;
-#pragma unroll
-                                for (int ks = 0; ks < C::BLK / 16; ++ks) {
-                                    mma(k, 0, ks, false);
-                                    mma(k, 1, ks, false);
-                                    mma(k, 0, ks, true);
-                                    mma(k, 1, ks, true);
-                                }
-                            }
+                        for (int ks = 0; ks < 2 * (C::BLK / 16); ++ks) {
+                            const int k = ks % (C::BLK / 16);
+                            const uint64_t a = ks < C::BLK / 16 ? a0 : a1, b = ks < C::BLK / 16 ? b0 : b1;
+                            large(a, b, 0, k, true);
+                            large(a, b, 1, k, true);
+                            small(a, b, 0, k);
+                            small(a, b, 1, k);
                         }
                     } else {
 #pragma unroll
-                        for (int h = 0; h < C::MT; ++h) {
-                            const uint32_t slot = C::MT == 1 ? (cc & 1u) : (uint32_t)h;
-                            const uint32_t turn = C::MT == 1 ? cc >> 1 : cc;  // how often the set has been filled before
-                            if (first && turn >= 1) {
-                                wait(accempty0 + 8 * slot, (turn - 1u) & 1u);
+                        for (int h = 0; h < 2; ++h) {
+                            if (first && cc >= 1) {
+                                wait(accempty0 + 8 * h, (cc - 1u) & 1u);
                                 tc_fence_after();
                             }
-                            if (!s_abort) {
 #pragma unroll
-                                for (int k = 0; k < G; ++k) {
-                                    if (k >= g) break;
+                            for (int ks = 0; ks < C::BLK / 16; ++ks) {
+                                large(a0, b0, h, ks, !first || ks > 0);
+                                small(a0, b0, h, ks);
+                            }
+                            if (two) {
 #pragma unroll
-                                    for (int ks = 0; ks < C::BLK / 16; ++ks) {
-                                        mma(k, h, ks, false);
-                                        mma(k, h, ks, true);
-                                    }
+                                for (int ks = 0; ks < C::BLK / 16; ++ks) {
+                                    large(a1, b1, h, ks, true);
+                                    small(a1, b1, h, ks);
                                 }
                             }
-                            if (last) umma_commit<C::PAIR>(accfull0 + 8 * slot);
+                            if (last) umma_commit_pair_by(accfull0 + 8 * h, lead);
                         }
                     }
-#pragma unroll
-                    for (int k = 0; k < G; ++k) {
-                        if (k >= g) break;
-                        umma_commit<C::PAIR>(done[k]);
+                    umma_commit_pair_by(empty0 + 8 * w0.st, lead);
+                    if (two) {
+                        umma_commit_pair_by(empty0 + 8 * w.st, lead);
+                        w.next();
                     }
                     if (last) ++cc;
                 }
@@ -668,7 +748,7 @@ __global__ void __cluster_dims__(F32 ? 1 : 2, 1, 1) __launch_bounds__(TablesCfg<
         // ------------------------------ TMA loads: fp32 embeddings -------------------------------
         if (lane == 0) {
             TablesRing<NR> r(1);
-            for (int i = 0; tables_item(p, pair, i, it); ++i) {
+            for (int i = 0; tables_item(p, s_share, pair, i, it); ++i) {
                 const int row = it.tile / p.n_mb * C::ROWS + (int)rank * 128;
                 for (int kb = it.kb0; kb < it.kb1; ++kb) {
                     if (r.t >= NR) wait(rempty0 + 8 * r.st, r.ph);
@@ -687,30 +767,26 @@ __global__ void __cluster_dims__(F32 ? 1 : 2, 1, 1) __launch_bounds__(TablesCfg<
         // barriers that it waits on: with an even number of stages every stage is always the same half's.  (Four raw stages or six: V =
         // 32,000, E = 2048, two towers 208.4 and 209.3 us.)
         static_assert(!F32 || (NR % 2 == 0 && NS % 2 == 0), "a stage of either ring belongs to one half of the converting warps");
-        const int ct = (tid - (kTmEpiWarps + 3) * 32) & 127, half = (tid - (kTmEpiWarps + 3) * 32) >> 7;
-        const int c8 = ct & 3, r0 = ct >> 2;  // columns 8 c8 .. 8 c8 + 7 of rows r0, r0 + 32, r0 + 64 and r0 + 96
+        // A thread has a row: a warp reaches its quarter of TMEM's lanes (its index modulo four), and a half has all four.
+        const int half = (warp - (kTmEpiWarps + 3)) >> 2, row = 32 * (warp & 3) + lane;
+        const uint32_t parts = tmem + kTmParts + ((uint32_t)(32 * (warp & 3)) << 16);
         TablesRing<NS> a(1);
         TablesRing<NR> r(0);
-        float4 x[4][2];
+        float4 x[8];
         auto load = [&]() {
             wait(rfull0 + 8 * r.st, r.ph);
-            const uint32_t src = raw_ring + r.st * C::RAW;
+            const uint32_t src = raw_ring + r.st * C::RAW + (uint32_t)row * 128u;
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int row = r0 + 32 * q;
-#pragma unroll
-                for (int h = 0; h < 2; ++h)  // (128-byte rows in the 128-byte swizzle)
-                    x[q][h] = ld_shared_f4(src + (uint32_t)row * 128u + (uint32_t)(((2 * c8 + h) ^ (row & 7)) * 16));
-            }
+            for (int j = 0; j < 8; ++j) x[j] = ld_shared_f4(src + (uint32_t)((j ^ (row & 7)) * 16));  // (128-byte rows in the 128-byte swizzle)
             __syncwarp();
             if (lane == 0) mbar_arrive(rempty0 + 8 * r.st);
         };
-        auto largest = [&](int q) {
-            const float m0 = fmaxf(fmaxf(fabsf(x[q][0].x), fabsf(x[q][0].y)), fmaxf(fabsf(x[q][0].z), fabsf(x[q][0].w)));
-            const float m1 = fmaxf(fmaxf(fabsf(x[q][1].x), fabsf(x[q][1].y)), fmaxf(fabsf(x[q][1].z), fabsf(x[q][1].w)));
+        auto largest = [&](int j) {  // of columns 8 j .. 8 j + 7
+            const float m0 = fmaxf(fmaxf(fabsf(x[2 * j].x), fabsf(x[2 * j].y)), fmaxf(fabsf(x[2 * j].z), fabsf(x[2 * j].w)));
+            const float m1 = fmaxf(fmaxf(fabsf(x[2 * j + 1].x), fabsf(x[2 * j + 1].y)), fmaxf(fabsf(x[2 * j + 1].z), fabsf(x[2 * j + 1].w)));
             return fmaxf(m0, m1);
         };
-        for (int i = 0; tables_item(p, pair, i, it); ++i) {
+        for (int i = 0; tables_item(p, s_share, pair, i, it); ++i) {
             // the rows' scales, from the half that has the tile's first block, for both halves and for the warps that empty the
             // accumulators (everybody waits for every phase of these barriers, the half that sets the scales too)
             const uint32_t slot = (uint32_t)i % kTmScales, turn = (uint32_t)i / kTmScales;
@@ -718,59 +794,45 @@ __global__ void __cluster_dims__(F32 ? 1 : 2, 1, 1) __launch_bounds__(TablesCfg<
             if (turn > 0) wait(sempty0 + 8 * slot, (turn - 1u) & 1u);
             if (lead) {
                 load();
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    float m = largest(q);
-                    m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, 1));
-                    m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, 2));
-                    if (c8 == 0) s_scale[slot][r0 + 32 * q] = (uint8_t)(__float_as_uint(tables_row_scale(m)) >> 23);
-                }
+                s_scale[slot][row] = (uint8_t)(__float_as_uint(tables_row_scale(fmaxf(fmaxf(largest(0), largest(1)), fmaxf(largest(2), largest(3))))) >> 23);
                 __syncwarp();
                 if (lane == 0) mbar_arrive(sfull0 + 8 * slot);
             }
             wait(sfull0 + 8 * slot, turn & 1u);
-            float scale[4], most[4], least[4];  // largest and smallest, but for zero, of eight entries' largest magnitudes
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                scale[q] = __uint_as_float((uint32_t)s_scale[slot][r0 + 32 * q] << 23);
-                most[q] = 0.f;
-                least[q] = INFINITY;
-            }
+            const float scale = __uint_as_float((uint32_t)s_scale[slot][row] << 23);
+            float most = 0.f, least = INFINITY;  // largest and smallest, but for zero, of eight entries' largest magnitudes
             __syncwarp();
             if (lane == 0) mbar_arrive(sempty0 + 8 * slot);
             for (int kb = it.kb0; kb < it.kb1; ++kb, a.next(), r.next()) {
                 if ((int)(a.t & 1u) != half) continue;
                 if (kb != it.kb0) load();
-                if (a.t >= NS) wait(empty0 + 8 * a.st, a.ph);
-                const uint32_t dst = a_ring + a.st * C::A_BYTES;
+                uint32_t b[32];  // columns of TMEM: the 32 numbers' first parts, then their second
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const int row = r0 + 32 * q;  // (64-byte rows in the 64-byte swizzle)
-                    const uint32_t at = dst + (uint32_t)row * 64u + (uint32_t)((c8 ^ ((row >> 1) & 3)) * 16);
-                    uint32_t b1[4], b2[4];
-                    split2(x[q][0].x, x[q][0].y, scale[q], b1[0], b2[0]);
-                    split2(x[q][0].z, x[q][0].w, scale[q], b1[1], b2[1]);
-                    split2(x[q][1].x, x[q][1].y, scale[q], b1[2], b2[2]);
-                    split2(x[q][1].z, x[q][1].w, scale[q], b1[3], b2[3]);
-                    st_shared_v4(at, b1);
-                    st_shared_v4(at + C::PART, b2);
-                    const float m = largest(q);
-                    most[q] = fmaxf(most[q], m);
-                    if (m != 0.f) least[q] = fminf(least[q], m);
+                for (int j = 0; j < 8; ++j) {
+                    split2(x[j].x, x[j].y, scale, b[2 * j], b[16 + 2 * j]);
+                    split2(x[j].z, x[j].w, scale, b[2 * j + 1], b[16 + 2 * j + 1]);
                 }
-                fence_proxy_async();
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const float m = largest(j);
+                    most = fmaxf(most, m);
+                    if (m != 0.f) least = fminf(least, m);
+                }
+                if (a.t >= NS) {
+                    wait(empty0 + 8 * a.st, a.ph);
+                    tc_fence_after();
+                }
+                tmem_st_32x32(parts + 32u * a.st, b);
+                tmem_wait_st();
+                tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(full0 + 8 * a.st);
             }
-            // rows that the parts do not hold well enough (in this thread's entries)
+            // rows that the parts do not hold well enough
             const int rt = it.tile / p.n_mb;
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int v = r0 + 32 * q;
-                if ((most[q] * scale[q] > kTmMost || least[q] * scale[q] < kTmLeast) && rt * C::ROWS + v < p.V) {
-                    p.bad_row[(size_t)it.tile * C::ROWS + v] = 1;
-                    if (it.q0 == it.q1) s_mend = true;
-                }
+            if ((most * scale > kTmMost || least * scale < kTmLeast) && rt * C::ROWS + row < p.V) {
+                p.bad_row[(size_t)it.tile * C::ROWS + row] = 1;
+                if (it.q0 == it.q1) s_mend = true;
             }
         }
         a.drain(empty0, 0u, &s_abort);
@@ -787,8 +849,8 @@ __global__ void __cluster_dims__(F32 ? 1 : 2, 1, 1) __launch_bounds__(TablesCfg<
 }
 
 // The left-over tiles' pieces, added up in order: four columns of N rows a thread, a warp a row, 8 N rows a block.
-template <bool F32, int N>
-__global__ void __launch_bounds__(256, F32 ? 3 : 8) tables_pieces_kernel(const __grid_constant__ TablesParams p) {
+template <bool F32, int N, int PER_SM>
+__global__ void __launch_bounds__(256, PER_SM) tables_pieces_kernel(const __grid_constant__ TablesParams p) {
     using C = TablesCfg<F32>;
     static_assert(8 * N <= kTmMendRows, "rows that may have to be worked out again");
     __shared__ TablesMend sm;
@@ -800,9 +862,10 @@ __global__ void __launch_bounds__(256, F32 ? 3 : 8) tables_pieces_kernel(const _
     float4 s[N];
 #pragma unroll
     for (int i = 0; i < N; ++i) s[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 4
+    const int seg0 = tables_share(p, q0) < tile * p.n_kb ? 1 : 0;  // (the others' shares begin in this tile)
+#pragma unroll(PER_SM == 4 ? 8 : 4)
     for (int q = q0; q <= q1; ++q) {
-        const int seg = tables_share(p, q) < tile * p.n_kb ? 1 : 0;
+        const int seg = q == q0 ? seg0 : 0;
 #pragma unroll
         for (int i = 0; i < N; ++i) {
             const float4 x = __ldcs((const float4*)(p.pieces + ((size_t)(q * 2 + seg) * C::ROWS + v0 + 8 * i + warp) * 128 + c));
@@ -893,10 +956,10 @@ cudaError_t tables_run(const TablesParams& p, cudaStream_t st, int* launches) {
         // fp32: 32 rows a block where that leaves a block an SM or more, else 8 (102 tiles left, V = 32,000, E =
         // 2048: 87.2 and 92.8 us; 56, V = 64,000, E = 1536: 122.1 and 124.6; 9, V = 20,000, E = 2048: 69.1 and 65.1)
         constexpr int N = F32 ? 4 : 1;
-        if (p.left * (C::ROWS / (8 * N)) >= p.pairs)
-            e = launch_pdl(tables_pieces_kernel<F32, N>, dim3(C::ROWS / (8 * N), p.left), dim3(256), 0, st, p);
-        else
-            e = launch_pdl(tables_pieces_kernel<F32, 1>, dim3(C::ROWS / 8, p.left), dim3(256), 0, st, p);
+        if (F32 ? p.left * (C::ROWS / (8 * N)) >= p.pairs : p.share_pairs < 6 * p.left)
+            e = launch_pdl(tables_pieces_kernel<F32, N, F32 ? 3 : 8>, dim3(C::ROWS / (8 * N), p.left), dim3(256), 0, st, p);
+        else  // (few tiles left, many pieces each: bf16 with registers for eight pieces' loads, V = 151,936: 14 -> 8 us)
+            e = launch_pdl(tables_pieces_kernel<F32, 1, F32 ? 3 : 4>, dim3(C::ROWS / 8, p.left), dim3(256), 0, st, p);
         *launches += 1;
     }
     return e;
@@ -906,7 +969,8 @@ cudaError_t tables_run(const TablesParams& p, cudaStream_t st, int* launches) {
 
 // Can the tensor cores take this table?  16-byte rows for the loads and stores; anything else goes to the FMA kernel.
 bool tables_mma_fits(const void* d_emb, graft_dtype dt, int E, const void* d_out) {
-    return E % (dt == GRAFT_BF16 ? 8 : 4) == 0 && (((uintptr_t)d_emb | (uintptr_t)d_out) & 15) == 0 && encode_tiled() != nullptr;
+    // (E: shares of the tiles that are left are worked out in 32 bits)
+    return E <= 1 << 22 && E % (dt == GRAFT_BF16 ? 8 : 4) == 0 && (((uintptr_t)d_emb | (uintptr_t)d_out) & 15) == 0 && encode_tiled() != nullptr;
 }
 size_t tables_mma_scratch_bytes(int num_sms, int V, int E, int m, graft_dtype dt) {
     return tables_sizes(num_sms, V, E, m, dt == GRAFT_F32).total;
@@ -962,12 +1026,19 @@ cudaError_t tables_mma_launch(graft_ctx* ctx, const void* d_emb, graft_dtype dt,
     }
     p.share_pairs = (int)(sp < p.left ? p.left : sp);
     p.wide = m % 8 == 0 && ((uintptr_t)d_out & 31) == 0;
-    if (f32)
-        weight_split16_kernel<<<s.m_pad, 256, 0, st>>>(d_W, m, E, s.m_pad, s.E_pad, (__half*)w, (float2*)((char*)scratch + s.o_unscale),
-                                                       (uint32_t*)p.bad_row, (int)(s.n_bad / 4));
-    else
-        weight_split_kernel<<<dim3((s.E_pad + 511) / 512, s.m_pad), 256, 0, st>>>(d_W, m, E, s.m_pad, s.E_pad, (__nv_bfloat16*)w);
-    cudaError_t e = cudaGetLastError();
+    SplitParams split;
+    split.W = d_W;
+    split.m = m;
+    split.E = E;
+    split.m_pad = s.m_pad;
+    split.E_pad = s.E_pad;
+    split.w = w;
+    split.unscale = (float2*)((char*)scratch + s.o_unscale);
+    split.flags = (uint32_t*)p.bad_row;
+    split.n_flags = (int)(s.n_bad / 4);
+    cudaError_t e = f32 ? launch_pdl(weight_split16_kernel, dim3(s.m_pad), dim3(256), 0, st, split)
+                        : launch_pdl(weight_split_kernel, dim3((s.E_pad + 511) / 512, s.m_pad), dim3(256), 0, st, split);
+    if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     int launches = 1;
     e = f32 ? tables_run<true>(p, st, &launches) : tables_run<false>(p, st, &launches);

@@ -108,6 +108,23 @@ def test_fp32_entries_that_bf16_parts_cannot_hold(V, E, m):
     assert ((got - want)[fin].abs() <= 2e-5 + 2e-6 * want[fin].abs()).all()
 
 
+@pytest.mark.parametrize("V,E,m", [
+    (130, 20, 32),       # less than a block of columns
+    (500, 288, 128),     # nine blocks: the second chunk, on the accumulators' other side, has one
+    (500, 544, 96),      # seventeen: three chunks, the last of one block
+    (129, 32, 200),      # two blocks of m, the second of 72 columns; a row in the second tile
+    (19000, 2080, 128),  # a whole tile and shares of the tiles left, which begin and end anywhere
+    (57000, 1056, 64),   # several whole tiles a worker, an odd number of chunks each
+])
+def test_fp32_chunks_and_tiles_of_odd_lengths(V, E, m):
+    """The large products' accumulators take turns on either side of the small ones', which last a tile: every chunk and every tile
+    counts once.  The sums are about 1; the parts of order 2^-11 of every chunk are 1e-4 of them and more."""
+    emb, W, b = _inputs(V, E, m, "f32", 11)
+    got = _call(_graft(V, m), emb, W, b, m).double()
+    want = _exact(emb, W, b)
+    assert ((got - want).abs() <= 1e-5 + 1e-6 * want.abs()).all()  # (a sum's rounding: 2e-6 at most, measured)
+
+
 @pytest.mark.parametrize("part", ["embedding", "W", "both"])
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 def test_parts_of_every_order_count(part, dtype):
