@@ -10,30 +10,43 @@
 
 namespace graft {
 
-// Will this sequence's tree run deep?  A confident drafter (high top-1 probabilities) gives a deep, narrow tree that
-// needs the edge scores of many depths; an uncertain one a shallow, wide tree that stops a few levels down.  The
-// edge-score kernel scores the deeper rows ahead of the tree kernel only for the sequences that pass this test (mean
-// top-1 probability of the block >= 0.2: on the configured workloads trees reach depth 8 from about there); the tree
-// kernel, which takes the same decision from the same numbers, scores what is missing on demand.  A matter of speed
-// only: a row has the same bits whoever scores it.
+// How many depths of this sequence will its tree look at?  A confident drafter (high top-1 probabilities) gives a deep, narrow
+// tree that needs the edge scores of many depths; an uncertain one a shallow, wide tree that stops a few levels down.  The
+// edge-score kernel scores that many depths ahead of the tree kernel, which takes the same decision from the same numbers
+// and scores what is missing on demand (3 - 4 us a depth in front of everything else, so the bounds err on the side of more).  A
+// matter of speed only: a row has the same bits whoever scores it.  By the mean top-1 probability of the block, of 2,500
+// sequences of the configured workloads (budgets 16 to 512, L = 12 and 16, K > 8): below 0.02 at most 4 depths, below 0.03 5,
+// below 0.06 6, below 0.1 7 (all but one in two hundred); below 0.2 8 (all but one in forty), above it up to 12.  With 8 or fewer
+// candidates trees are narrower and deeper (5 to 8 depths even at 0.01), and a depth's scores are cheap: 8.
 // (In two steps, so that a caller can have the load in flight beside its other loads: lane d's top-1 log-probability
 // of position d, 0 for d >= L; then the decision, taken by every lane of a warp together.)
-__device__ __forceinline__ float deep_tree_load(const float* __restrict__ topk_lp_seq, int L, int K) {
+// Fewer than `rows` of them only where the scores take more CTAs than the SMs hold at once (four each): in one wave nothing is gained,
+// and the decision stands in front of the work (batch 16, 64: 0.7 us of a round).
+inline int rows_ahead_least(int batch, int rows, int num_sms) { return rows > 4 && (long long)batch * rows > 4ll * num_sms ? 4 : rows; }
+__device__ __forceinline__ float rows_ahead_load(const float* __restrict__ topk_lp_seq, int L, int K) {
     const int lane = threadIdx.x & 31;
     return lane < L ? topk_lp_seq[(size_t)lane * K] : 0.f;
 }
-__device__ __forceinline__ bool deep_tree_decide(float lp_top, int L) {
+__device__ __forceinline__ float rows_ahead_sum(float lp_top, int L) {  // (of the block's top-1 probabilities)
     // lane d holds position d (L <= 32); a butterfly sum in a fixed order
     const int lane = threadIdx.x & 31;
     float s = lane < L ? ex2_approx(lp_top * kLog2e) : 0.f;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
-    return s >= 0.2f * (float)L;
+    return s;
 }
-__device__ __forceinline__ bool deep_tree_likely(const float* __restrict__ topk_lp_seq, int L, int K) {
-    return deep_tree_decide(deep_tree_load(topk_lp_seq, L, K), L);
+// rows: the depths scored ahead at most, unless the tree runs deeper than 8; least: and at least (rows: all of them)
+__device__ __forceinline__ int rows_ahead(float lp_top, int L, int K, int least, int rows) {
+    const float s = rows_ahead_sum(lp_top, L), one = (float)L;
+    if (s >= 0.2f * one) return L;
+    if (least == rows || K <= 8) return rows;
+    const int n = s < 0.02f * one ? 4 : s < 0.03f * one ? 5 : s < 0.06f * one ? 6 : s < 0.1f * one ? 7 : 8;
+    return n < rows ? n : rows;
 }
 
+// More sequences than SMs: the trees that take longest, those of confident drafters (from this mean on half of an ordinary
+// batch), are built first, so that those of the second wave are short.
+constexpr float kTreeLongMean = 0.06f;
 
 // Where the r-th entry of the sorted row of parent rank c stands inside the row (scores only; the child ranks stand
 // in order): rotated by the parent's rank.  The tree kernel's threads look at the same place r of different parents'

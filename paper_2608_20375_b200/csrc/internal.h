@@ -89,7 +89,10 @@ struct graft_ctx {
     uint8_t* w_eidx;              // [max_batch, L, K, K] child rank of each sorted entry
     double* w_cos;                // [max_batch, L] adjacent-position cosines (Eq. 15)
     graft::SabaResult* w_saba;    // [max_batch] budgets worked out by the edge-score kernel
+    int32_t* w_order;             // [max_batch] order in which the trees of more sequences than SMs are built
+    int* w_order_n;               // [2] sequences placed in it from either end, zero between rounds
     double* w_fit;                // [32] normal equations of graft_saba_fit and its arrival counter, zero between calls
+    bool loss_many;               // graft_tdes_loss's kernels for many traces are ready
     double* w_loss;               // [8] sums of graft_tdes_loss and its arrival counter, zero between calls
     int32_t* w_errflag;           // [1] device-side internal error flag
     graft::VpPlan vp_plan;
@@ -185,6 +188,7 @@ cudaError_t saba_fit_launch(graft_ctx* ctx, long long n, const float* d_state, c
                             const float* d_gain, const int32_t* d_prefix, const float* d_latency, double* d_out,
                             cudaStream_t st);
 size_t tree_smem_bytes(const graft_config& cfg);
+bool tree_ordered(const graft_ctx* ctx, int batch);  // the edge-score kernel gives the order of the trees
 bool tree_lazy_fits(const graft_config& cfg);  // edge scores are computed inside the tree kernel
 
 }  // namespace graft

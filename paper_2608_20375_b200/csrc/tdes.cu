@@ -88,13 +88,15 @@ struct EdgeParams {
     float* esort;     // same rows, each sorted by (edge descending, child rank ascending), stored rotated (es_col)
     uint8_t* eidx;    // child rank of every sorted entry
     int L, K, m, V;
-    int rows;     // depths [0, rows) are scored for every sequence: one CTA each; deeper ones
-                  // only for sequences whose trees will run deep
+    int rows, rows_least;  // depths [0, rows_least) are scored for every sequence, one CTA each; deeper ones for sequences whose
+                           // trees will look at them (rows_ahead)
     float scale;  // s / sqrt(m)
     float beta;
     int root_edge;
     // the budget of every sequence (Sec. 3.3), worked out by its depth-0 CTA when saba_out is not NULL
     SabaResult* saba_out;         // [batch]
+    int32_t* order;               // [batch] the sequences in the order in which their trees are built, or NULL
+    int* order_n;                 // [2] sequences placed from either end, zero between rounds
     const double* cos_pre;        // [batch, L] adjacent-position cosines from the vocab pass
     const int32_t* vp_err;
     const float* hist;            // [batch]
@@ -115,13 +117,19 @@ __global__ void __launch_bounds__(256, 4) tdes_edges_kernel(const EdgeParams p) 
     // only deep trees need behind those scored for every sequence (their CTAs mostly exit at once and should not take the
     // places of CTAs with work).  No division stands in front of the first loads (0.7 us of a round at batch 16).
     const int b = blockIdx.x, j = blockIdx.y;
-    if (j >= p.rows && !deep_tree_likely(p.topk_lp + (size_t)b * p.L * p.K, p.L, p.K)) return;  // (uniform)
     const int K = KC ? KC : p.K, m = MC ? MC : p.m, ld = m + 4;  // padded row: 16-byte aligned, conflict-free float4 reads
+    const size_t row = (size_t)b * p.L + j;
+    const int n_par = (j == 0) ? 1 : K;
+    if (j >= p.rows_least && j >= rows_ahead(rows_ahead_load(p.topk_lp + (size_t)b * p.L * K, p.L, K), p.L, K, p.rows_least, p.rows)) return;  // (uniform)
+    // the unit's tokens are on their way while the rows' states are looked at (0.3 us of a round at batch 1, K = 8)
+    int32_t tok = 0;
+    if (threadIdx.x < n_par + K) {
+        const int r = threadIdx.x;
+        tok = r < n_par ? (j == 0 ? p.root_token[b] : p.topk_id[(row - 1) * K + r]) : p.topk_id[row * K + r - n_par];
+    }
     float* sP = smem;                        // [K][ld]  parent rows + u_d
     float* sC = smem + (size_t)kMaxK * ld;   // [K][ld]  child rows + u_d
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int n_par = (j == 0) ? 1 : K;
-    const size_t row = (size_t)b * p.L + j;
     // The depth-0 unit has one parent, so this CTA has time to spare: its last warp works out the sequence's budget, which
     // the tree kernel would otherwise do in front of everything else.  That takes longer than the scores of a unit (a
     // chain of fp64 operations, 3 us), so the warp does nothing else and the other seven do not wait for it (1.4 us of a
@@ -139,11 +147,17 @@ __global__ void __launch_bounds__(256, 4) tdes_edges_kernel(const EdgeParams p) 
                                        p.topk_lp + (size_t)b * p.L * K, p.cos_pre + (size_t)b * p.L, p.hist + b,
                                        p.prefix_len + b, p.fixed_budget ? p.fixed_budget + b : nullptr, lane);
         if (lane == 0) p.saba_out[b] = r;
+        if (p.order != nullptr) {  // this sequence's place among the trees: from the front or from the back
+            const bool front = rows_ahead_sum(rows_ahead_load(p.topk_lp + (size_t)b * p.L * K, p.L, K), p.L) >= kTreeLongMean * (float)p.L;
+            if (lane == 0) {
+                const int at = atomicAdd(p.order_n + (front ? 0 : 1), 1);
+                p.order[front ? at : (int)gridDim.x - 1 - at] = b;
+            }
+        }
         return;
     }
     float* outs = p.esort + row * K * K;
     uint8_t* outi = p.eidx + row * K * K;
-    const int32_t* ids = p.topk_id + row * K;
     const float* lps = p.topk_lp + row * K;
 
     const bool bad = p.row_status != nullptr && (p.row_status[row] != 0 || (j > 0 && p.row_status[row - 1] != 0));
@@ -163,11 +177,7 @@ __global__ void __launch_bounds__(256, 4) tdes_edges_kernel(const EdgeParams p) 
     // gather: token ids first (one round trip), then every warp issues the loads of all its rows before it uses
     // any of them (a second round trip); one warp per table row, 16 bytes per lane
     __shared__ int toks[2 * kMaxK];
-    if (threadIdx.x < n_par + K) {
-        const int r = threadIdx.x;
-        int32_t tok = r < n_par ? (j == 0 ? p.root_token[b] : p.topk_id[(row - 1) * K + r]) : ids[r - n_par];
-        toks[r] = tok < 0 ? 0 : (tok >= p.V ? p.V - 1 : tok);
-    }
+    if (threadIdx.x < n_par + K) toks[threadIdx.x] = tok < 0 ? 0 : (tok >= p.V ? p.V - 1 : tok);
     sync();
     const float* urow = p.u + (size_t)j * m;
     constexpr int RPW = 2 * kMaxK / 8;  // rows per warp at most
@@ -270,8 +280,12 @@ cudaError_t tdes_edges_launch(graft_ctx* ctx, int batch, const int32_t* d_topk_i
     p.beta = ctx->tdes_set ? cfg.beta : 0.0f;
     p.root_edge = cfg.root_edge;
     p.rows = rows;
+    // (the tree kernel takes the same decision if it can score on demand and the budget comes from here)
+    p.rows_least = !d_edge && d_saba_out && d_row_status && rows < cfg.L ? rows_ahead_least(batch, rows, ctx->num_sms) : rows;
     const int rows_all = d_edge || rows == cfg.L ? rows : cfg.L;  // (rows < L only when the tree kernel can score on demand)
     p.saba_out = d_row_status ? d_saba_out : nullptr;
+    p.order = p.saba_out && tree_ordered(ctx, batch) ? ctx->w_order : nullptr;
+    p.order_n = ctx->w_order_n;
     p.cos_pre = ctx->w_cos;
     p.vp_err = ctx->w_errflag;
     p.hist = d_hist;

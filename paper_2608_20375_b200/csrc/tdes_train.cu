@@ -1452,7 +1452,15 @@ cudaError_t tdes_loss_launch(graft_ctx* ctx, const graft_tdes_traces* tr, const 
         long long grid = (work + kTsWarps - 1) / kTsWarps;
         if (grid > ctx->num_sms) grid = ctx->num_sms;
         const long long refs = (long long)tr->n_groups * (cfg.K + 1) + 4ll * tr->n_pairs + 2ll * tr->n_edges;
-        if (refs < (d_gP ? kTsMany : kTsManyLoss)) {
+        // (the two kernels are loaded with the first call that wants them: a millisecond each, which graft_create need not wait for)
+        bool many = refs >= (d_gP ? kTsMany : kTsManyLoss);
+        if (many && !ctx->loss_many) {
+            cudaError_t e = allow_smem((const void*)groups_kernel(cfg), groups_smem(cfg, groups_batch(cfg)));
+            if (e == cudaSuccess) e = allow_smem((const void*)(cfg.m == 128 ? tdes_items_kernel<true> : tdes_items_kernel<false>), items_smem(cfg));
+            if (e != cudaSuccess) cudaGetLastError();
+            many = ctx->loss_many = e == cudaSuccess;
+        }
+        if (!many) {
             p.ctas = (int)grid;
             rows_kernel(cfg)<<<(int)grid, kTsThreads, smem, st>>>(p);
             ctx->launches += 1;
@@ -1499,10 +1507,7 @@ cudaError_t tdes_loss_launch(graft_ctx* ctx, const graft_tdes_traces* tr, const 
 cudaError_t tdes_loss_configure(const graft_config& cfg) {
     const size_t smem = tdes_loss_smem(cfg);
     if (cfg.m > 128) return allow_smem((const void*)(cfg.m <= 256 ? tdes_loss_kernel<2> : tdes_loss_kernel<kTrMaxChunks>), smem);
-    cudaError_t e = allow_smem((const void*)rows_kernel(cfg), smem);
-    if (e == cudaSuccess) e = allow_smem((const void*)groups_kernel(cfg), groups_smem(cfg, groups_batch(cfg)));
-    if (e == cudaSuccess) e = allow_smem((const void*)(cfg.m == 128 ? tdes_items_kernel<true> : tdes_items_kernel<false>), items_smem(cfg));
-    return e;
+    return allow_smem((const void*)rows_kernel(cfg), smem);
 }
 bool tdes_loss_supported(const graft_config& cfg) { return cfg.m % 4 == 0 && cfg.m <= 128 * kTrMaxChunks; }
 

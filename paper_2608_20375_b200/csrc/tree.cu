@@ -29,7 +29,10 @@ struct TreeParams {
     // Edge scores (Eq. 4-6): the rows of depths [0, rows_pre) come from the edge-score kernel through esort / eidx;
     // deeper rows are scored inside this kernel (lazy = 1), level by level, only if the expansion gets there.
     int rows_pre;
-    int rows_adaptive;  // the edge-score kernel also scored the deeper rows of sequences whose trees will run deep
+    int rows_least;     // of those at least
+    const int32_t* order;  // [batch] which sequence's tree a CTA builds (more sequences than SMs), or NULL: its own number's
+    int* order_n;          // [2] cleared for the next round
+    int rows_adaptive;  // the edge-score kernel scored as many depths of a sequence as its tree will look at (rows_ahead)
     int lazy;
     int lazy_m;  // m when the shared-memory layout holds the buffers of the on-demand scorer, else 0
     const float* P;
@@ -688,7 +691,9 @@ __device__ __forceinline__ void lazy_score_row(const TreeParams& p, const TreeSm
 // prefixes tie with the B-th largest key: it resolves them in parallel (the other instances leave more than 32 tied
 // keys to the sequential expansion; with edge scores in the keys such ties do not occur in tens, and the code's mere
 // presence costs this register-bound kernel 0.4 us a round)
-template <int NT, int KC, int MC, bool FAST, int NMAXC = 0, bool TIES = false>
+// ORDER: more sequences than SMs, built in the order p.order (the sequence's number from memory instead of the CTA's costs the
+// others 0.3 to 0.8 us of a round)
+template <int NT, int KC, int MC, bool FAST, int NMAXC = 0, bool TIES = false, bool ORDER = false>
 __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int K = KC ? KC : p.K, p_m = MC ? MC : p.m;
@@ -696,11 +701,13 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
     TreeSmem sm;
     const int ncap = NMAXC ? 6144 : p.ncap;  // (the instance with the outputs' size known is used at full capacity only)
     tree_smem_layout(p.L, K, NMAXC ? NMAXC : p.nmax, ncap, p.lazy_m, &sm, smem_raw);
-    const int b = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int L = p.L, nmax = NMAXC ? NMAXC : p.nmax, W = NMAXC ? (NMAXC + 31) / 32 : p.W;
     const graft_tree_out& o = p.out;
     pdl_launch_dependents();  // an acceptance walk queued behind this kernel may move in; it waits for this grid
     pdl_wait();  // candidates, cosines and edge rows come from the kernels ahead in the stream
+    const int b = ORDER ? p.order[blockIdx.x] : (int)blockIdx.x;
+    if (ORDER && blockIdx.x == 0 && tid < 2) p.order_n[tid] = 0;
 
     // ---- status and budget ---------------------------------------------------------------------------
     // the sorted edge rows of this sequence: bulk copies through the TMA unit when the 16-byte rules allow it
@@ -714,7 +721,7 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
     const bool bulk = !TIES && ne > 0 && (ne % 16) == 0 && (L * K * K) % 16 == 0;
     // the prologue's loads from global memory are all issued before the first of them is used: one round trip
     const int root = p.root_token[b];
-    const float lp_top = !TIES && p.rows_adaptive ? deep_tree_load(p.topk_lp + (size_t)b * L * K, L, K) : 0.f;
+    const float lp_top = !TIES && p.rows_adaptive ? rows_ahead_load(p.topk_lp + (size_t)b * L * K, L, K) : 0.f;
     SabaResult pre_r;
     pre_r.budget = 0;
     pre_r.status = 0;
@@ -777,7 +784,9 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
     // a sequence whose tree will run deep had its deeper rows scored by the edge-score kernel as well: bulk copies again for
     // 1024 threads, K > 20 (plain loads, eight round trips with K = 32, kept such a sequence 2 us); plain loads for K <= 20,
     // which are 40 % as many or less (bulk copies behind a barrier of their own: half a microsecond slower at K = 16)
-    const bool deep = !TIES && p.rows_adaptive && deep_tree_decide(lp_top, L);  // (uniform)
+    const int ahead = !TIES && p.rows_adaptive ? rows_ahead(lp_top, L, K, p.rows_least, rows_pre) : rows_pre;  // (uniform)
+    const bool deep = ahead > rows_pre;
+    rows_done = ahead;
     if (deep) {
         if (NT == 1024 && bulk) {
             if (tid == 0) copy_rows((uint32_t)ne, (uint32_t)(L * K * K), smem_u32(&deep_bar));
@@ -788,7 +797,6 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
                 sm.ei[i] = p.eidx[seq_e + i];
             }
         }
-        rows_done = L;
     }
     if (!TIES) __syncthreads();
     if (TIES && warp >= 1) {  // (warp 0 is at the budget from the start)
@@ -1778,7 +1786,13 @@ static TreeInstance tree_pick_general(int K) {
     if (K <= 20) return {tree_kernel<512, 0, 0, false, 0, NEUTRAL>, 512};
     return {tree_kernel<1024, 0, 0, false, 0, NEUTRAL>, 1024};
 }
-static TreeInstance tree_pick(const graft_config& cfg, bool usual, bool neutral) {
+// Whether the trees of more sequences than SMs are built in an order of their own: the instances of the usual round.
+bool tree_ordered(const graft_ctx* ctx, int batch) {
+    const graft_config& cfg = ctx->cfg;
+    return batch > ctx->num_sms && ctx->tdes_set && cfg.beta != 0.0f && ctx->edge_rows > 0 && ctx->edge_rows < cfg.L && cfg.m == 128 &&
+           (cfg.K == 32 || cfg.K == 16 || cfg.K == 8);
+}
+static TreeInstance tree_pick(const graft_config& cfg, bool usual, bool neutral, bool order = false) {
     const int nmax = cfg.budget_max + 1;
     usual = usual && cfg.m == 128;
     if (neutral) {
@@ -1786,19 +1800,23 @@ static TreeInstance tree_pick(const graft_config& cfg, bool usual, bool neutral)
         return tree_pick_general<true>(cfg.K);
     }
     if (usual && cfg.K == 32) {
-        if (nmax == 513 && tree_node_cap(cfg.L, cfg.K, nmax, cfg.m) == 6144) return {tree_kernel<1024, 32, 128, true, 513>, 1024};
-        return {tree_kernel<1024, 32, 128, true>, 1024};
+        if (nmax == 513 && tree_node_cap(cfg.L, cfg.K, nmax, cfg.m) == 6144)
+            return {order ? tree_kernel<1024, 32, 128, true, 513, false, true> : tree_kernel<1024, 32, 128, true, 513>, 1024};
+        return {order ? tree_kernel<1024, 32, 128, true, 0, false, true> : tree_kernel<1024, 32, 128, true>, 1024};
     }
-    if (usual && cfg.K == 16) return {tree_kernel<512, 16, 128, true>, 512};
-    if (usual && cfg.K == 8) return {tree_kernel<256, 8, 128, true>, 256};
+    if (usual && cfg.K == 16) return {order ? tree_kernel<512, 16, 128, true, 0, false, true> : tree_kernel<512, 16, 128, true>, 512};
+    if (usual && cfg.K == 8) return {order ? tree_kernel<256, 8, 128, true, 0, false, true> : tree_kernel<256, 8, 128, true>, 256};
     return tree_pick_general<false>(cfg.K);
 }
 
 cudaError_t tree_configure(const graft_config& cfg) {
     const size_t bytes = tree_smem_bytes(cfg);
     cudaError_t e = cudaSuccess;
-    for (int i = 0; i < 4 && e == cudaSuccess; ++i)
-        e = allow_smem((const void*)tree_pick(cfg, (i & 1) != 0, (i & 2) != 0).kernel, bytes);
+    int dev = 0, num_sms = 0;
+    if (e == cudaSuccess) e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, dev);
+    for (int i = 0; i < (cfg.max_batch > num_sms ? 6 : 4) && e == cudaSuccess; ++i)
+        e = allow_smem((const void*)tree_pick(cfg, (i & 1) != 0, (i & 2) != 0, i >= 4).kernel, bytes);
     return e;
 }
 
@@ -1830,6 +1848,7 @@ cudaError_t tree_launch(graft_ctx* ctx, int batch, const int32_t* d_topk_id, con
     p.beta = ctx->tdes_set ? cfg.beta : 0.0f;
     const bool neutral = p.beta == 0.0f;  // (the candidates are staged whenever there is room; no row is scored)
     p.lazy = neutral ? tree_lazy_fits(cfg) : p.rows_pre < cfg.L ? 1 : 0;  // (only possible when tree_lazy_fits)
+    p.rows_least = rows_ahead_least(batch, p.rows_pre, ctx->num_sms);
     p.rows_adaptive = (p.lazy && p.rows_pre > 0 && d_saba_pre != nullptr) ? 1 : 0;
     p.lazy_m = tree_lazy_fits(cfg) ? cfg.m : 0;
     p.ncap = tree_node_cap(cfg.L, cfg.K, ctx->nmax, p.lazy_m);
@@ -1849,7 +1868,10 @@ cudaError_t tree_launch(graft_ctx* ctx, int batch, const int32_t* d_topk_id, con
     // the instances with K and m known at compile time serve the usual round (the budget from the edge-score kernel,
     // deeper rows on demand)
     const bool usual = p.lazy && p.saba_pre != nullptr;
-    const TreeInstance kern = tree_pick(cfg, usual, neutral);
+    const bool order = usual && tree_ordered(ctx, batch);
+    p.order = ctx->w_order;
+    p.order_n = ctx->w_order_n;
+    const TreeInstance kern = tree_pick(cfg, usual, neutral, order);
     const cudaError_t e = launch_pdl(kern.kernel, dim3(batch), dim3(kern.threads), tree_smem_bytes(cfg), st, p);
     ctx->launches += 1;
     return e != cudaSuccess ? e : cudaGetLastError();

@@ -265,3 +265,51 @@ def test_accept_refuses_a_wrong_tree(field, wrong):
         g.accept(out, tn, a, path, bonus)
     torch.cuda.synchronize()
     g.destroy()
+
+
+@pytest.mark.parametrize("K,m", [(32, 128), (16, 64), (8, 128)])
+@pytest.mark.parametrize("fixed", [False, True])
+def test_large_batches_build_the_trees_of_small_ones(K, m, fixed):
+    """From some batch on, how many depths are scored ahead depends on the sequence, and past one sequence an SM so does the order in
+    which the trees are built.  Neither shows: the same bits as in batches of forty, round after round."""
+    from paper_2608_20375_b200 import Graft
+    V, L, n, hd = 3000, 16, 330, 64
+    gen = torch.Generator(device="cuda").manual_seed(K + m)
+    rand = lambda *s: torch.randn(s, generator=gen, device="cuda")  # noqa: E731
+    height = 16.0 * torch.rand((n, 1, 1), generator=gen, device="cuda")  # mean top-1 probabilities from 0.01 to nearly 1
+    rank = torch.rand((n, L, V), generator=gen, device="cuda").argsort(2).float()
+    logits = (2.0 * rand(n, L, V) + height / (1.0 + rank)).to(torch.bfloat16)
+    logits[7, 3, 5] = float("nan")  # a bad row
+    P, Ct, u = rand(V, m), rand(V, m), 0.5 * rand(L, m)
+    root = torch.randint(0, V, (n,), generator=gen, device="cuda", dtype=torch.int32)
+    prefix = torch.randint(1, 4000, (n,), generator=gen, device="cuda", dtype=torch.int32)
+    hidden, hist = rand(n, L, hd).to(torch.bfloat16), 8.0 * torch.rand(n, generator=gen, device="cuda")
+    budget = torch.randint(1, 300, (n,), generator=gen, device="cuda", dtype=torch.int32)
+
+    def graft(batch):
+        g = Graft(V, L, K, m, hd, batch, 16, 304, 16, 0.2, 1)
+        g.set_tdes_tables(P, Ct, u, 1.0)
+        g.set_saba(phi_conf=-160.0, phi_degen=20.0, phi_hist=-5.0, phi_bias=200.0, tau_min=8.0, cost_mode=1,
+                   pts_n=[0.0, 64.0, 1024.0], pts_t=[18.0, 18.0, 37.2])
+        return g
+
+    def build(g, lo, hi):
+        o = g.alloc_out(hi - lo)
+        part = lambda t: t[lo:hi].contiguous()  # noqa: E731
+        g.build_trees(part(logits), None if fixed else part(hidden), part(root), None if fixed else part(hist), part(prefix),
+                      part(budget) if fixed else None, o)
+        torch.cuda.synchronize()
+        return o.cpu()
+
+    small = graft(40)
+    want = [build(small, lo, min(lo + 40, n)) for lo in range(0, n, 40)]
+    want = {k: np.concatenate([w[k] for w in want]) for k in want[0]}
+    depth = want["depth"].max(axis=1)
+    assert depth.min() <= 3 and depth.max() >= 9
+    big = graft(n)
+    for lo, hi in ((0, n), (0, n), (11, n), (30, 180), (0, 149), (0, 148), (5, 85), (0, n)):
+        got = build(big, lo, hi)
+        for k, w in want.items():
+            assert np.array_equal(got[k], w[lo:hi]), (k, lo, hi)
+    big.destroy()
+    small.destroy()
