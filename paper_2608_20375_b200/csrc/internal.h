@@ -91,7 +91,7 @@ struct graft_ctx {
     graft::SabaResult* w_saba;    // [max_batch] budgets worked out by the edge-score kernel
     int32_t* w_order;             // [max_batch] order in which the trees of more sequences than SMs are built
     int* w_order_n;               // [2] sequences placed in it from either end, zero between rounds
-    double* w_fit;                // [32] normal equations of graft_saba_fit and its arrival counter, zero between calls
+    double* w_fit;                // graft_saba_fit: table of logarithms, arrival counter and normal equations (both zero between calls)
     bool loss_many;               // graft_tdes_loss's kernels for many traces are ready
     double* w_loss;               // [8] sums of graft_tdes_loss and its arrival counter, zero between calls
     int32_t* w_errflag;           // [1] device-side internal error flag
@@ -184,6 +184,9 @@ cudaError_t tdes_loss_launch(graft_ctx* ctx, const graft_tdes_traces* tr, const 
                              cudaStream_t st);
 cudaError_t tdes_loss_configure(const graft_config& cfg);
 bool tdes_loss_supported(const graft_config& cfg);
+constexpr int kFitLog = 257;                        // entries of the fit's table of logarithms
+void saba_fit_table(double* table);                // [2 kFitLog], on the host
+size_t saba_fit_doubles();                         // graft_ctx::w_fit
 cudaError_t saba_fit_launch(graft_ctx* ctx, long long n, const float* d_state, const int32_t* d_budget,
                             const float* d_gain, const int32_t* d_prefix, const float* d_latency, double* d_out,
                             cudaStream_t st);

@@ -9,12 +9,14 @@
 // memory, per grid by one atomic a sum); the CTA that finishes last solves the two small systems (columns scaled to unit
 // diagonal first, then Gauss-Jordan elimination with partial pivoting) and clears the accumulators for the next call.
 //
-// 28 bytes are read a tuple and some 55 fp64 operations done on it: the fp64 pipe and the conversions of five floats in front
-// of it bound the slope (5 us per million tuples, 5.6 TB/s), and a call costs 8 us however few the tuples.  4 million tuples on a
-// B200: 37.3 -> 28.9 us with logarithms from a table and a short series instead of log, one division for four quotients and whole
-// numbers converted on the fp64 pipe (earlier steps, from 56.9: log for log1p, counts as integers, products by one folded, the
-// elimination on a warp and sums without shared-memory atomics; copies into shared memory ahead of the arithmetic, two and four
-// tuples interleaved, and 24 warps an SM instead of 16 were no faster or slower).
+// 28 bytes are read a tuple and some 55 fp64 operations done on it: with the next tuples' loads in flight and the table of logarithms
+// kept by the context a million tuples take 4.4 us (6.3 TB/s, the copy rate; 5.2 without), and a call costs 7 us however few:
+// launch, exchange, one round of atomics, the systems.  4 million tuples on a B200, one call after another: 30.0 -> 25.2 us, of
+// which 2.5 are the launch behind the call before (one CTA of 512 threads an SM and two of 256 are alike from 200,000 tuples on; the
+// CTAs' sums written out and added up in order by the last CTA instead of by atomics: 3 us slower at a million).  Before: 37.3 ->
+// 28.9 with logarithms from a table and a short series instead of log, one division for four quotients and whole numbers converted
+// on the fp64 pipe (earlier steps, from 56.9: log for log1p, counts as integers, products by one folded, the elimination on a warp
+// and sums without shared-memory atomics).
 #include <cuda_runtime.h>
 #include <math.h>
 
@@ -24,7 +26,7 @@
 namespace graft {
 namespace {
 
-constexpr int kFitThreads = 256;  // (and entries of the table of logarithms)
+constexpr int kFitThreads = 512;  // one CTA an SM
 constexpr int kFitAcc = 25;  // gain: 10 (upper triangle of 4 x 4) + 4 + 1 count; cost: 6 + 3 + 1 count
 
 struct FitParams {
@@ -34,6 +36,7 @@ struct FitParams {
     const float* gain;      // [n]
     const int32_t* prefix;  // [n]
     const float* latency;   // [n]
+    const double2* log;     // [kFitLog] table of logarithms (fit_log)
     double* acc;            // [kFitAcc] zero between calls
     unsigned int* ticket;   // zero between calls
     double* out;            // [10]
@@ -86,7 +89,7 @@ __device__ __forceinline__ double fit_double(int x) {
 // "Table-driven implementation of the logarithm function in IEEE floating-point arithmetic", 1990): 1 - g = 2^e f, c the
 // multiple of 1/512 nearest to f in [1/2, 1), r = f / c - 1, log(1 - g) = e ln 2 + log c + log(1 + r), |r| <= 2^-9; the series' first term
 // left out is 2^-57 of r.  With c = 1 for g below 2^-10, where r is -g itself, small results keep their relative precision.
-// tab[k]: 1 / c rounded, and minus the logarithm of that, c = 1/2 + k / 512.  Largest relative error 3e-16.
+// tab[k]: 1 / c rounded, and minus the logarithm of that, c = 1/2 + k / 512 (saba_fit_table).  Largest relative error 3e-16.
 __device__ __forceinline__ double fit_log(const double2* tab, double g) {
     const double x = 1.0 - g;
     const int hi = __double2hiint(x);
@@ -136,45 +139,53 @@ __device__ __forceinline__ void fit_accumulate(FitSums& t, float s0, float s1, f
 
 // VEC: every array is 16-byte aligned, so a thread takes four consecutive rounds with seven 16-byte loads
 template <bool VEC>
-__global__ void __launch_bounds__(kFitThreads, 2) saba_fit_kernel(const FitParams p) {
-    __shared__ double2 s_log[257];
-    __shared__ double s_acc[kFitAcc], s_warp[kFitThreads / 32][kFitAcc];
+__global__ void __launch_bounds__(kFitThreads, 1) saba_fit_kernel(const FitParams p) {
+    constexpr int W = kFitThreads / 32;
+    __shared__ double2 s_log[kFitLog];
+    __shared__ double s_acc[kFitAcc], s_warp[W][kFitAcc];
     __shared__ bool s_last;
     __shared__ int s_bad[2];
-    {
-        const double inv = 1.0 / (0.5 + threadIdx.x * (1.0 / 512.0));
-        s_log[threadIdx.x] = make_double2(inv, -log(inv));
-        if (threadIdx.x == 0) s_log[kFitThreads] = make_double2(1.0, 0.0);
-    }
+    pdl_launch_dependents();
+    pdl_wait();  // (the logs may come from the kernel ahead, and the one before this may still add up)
+    const long long tid = blockIdx.x * (long long)kFitThreads + threadIdx.x, nth = (long long)gridDim.x * kFitThreads;
+    const long long n4 = VEC ? p.n / 4 : 0;
+    // the next four rounds are on their way while four are worked on, the first beside the table
+    float4 a, b, c, ga, la;
+    int4 bu, pr;
+    const auto fetch = [&](long long q) {
+        if (q >= n4) return;
+        a = __ldg((const float4*)p.state + 3 * q), b = __ldg((const float4*)p.state + 3 * q + 1), c = __ldg((const float4*)p.state + 3 * q + 2);
+        bu = __ldg((const int4*)p.budget + q), pr = __ldg((const int4*)p.prefix + q);
+        ga = __ldg((const float4*)p.gain + q), la = __ldg((const float4*)p.latency + q);
+    };
+    if (VEC) fetch(tid);
+    if (threadIdx.x < kFitLog) s_log[threadIdx.x] = p.log[threadIdx.x];
     __syncthreads();
     FitSums t;
 #pragma unroll
     for (int i = 0; i < kFitAcc; ++i) t.acc[i] = 0.0;
     t.n_gain = t.n_cost = 0;
-    const long long tid = blockIdx.x * (long long)kFitThreads + threadIdx.x, nth = (long long)gridDim.x * kFitThreads;
     long long done = 0;
     if (VEC) {
-        const long long n4 = p.n / 4;
 #pragma unroll 1
         for (long long q = tid; q < n4; q += nth) {
-            const float4 a = __ldg((const float4*)p.state + 3 * q), b = __ldg((const float4*)p.state + 3 * q + 1),
-                         c = __ldg((const float4*)p.state + 3 * q + 2);
-            const int4 bu = __ldg((const int4*)p.budget + q), pr = __ldg((const int4*)p.prefix + q);
-            const float4 ga = __ldg((const float4*)p.gain + q), la = __ldg((const float4*)p.latency + q);
+            const float4 sa = a, sb = b, sc = c, gn = ga, lt = la;
+            const int4 bd = bu, pf = pr;
+            fetch(q + nth);
             // tau = -B / log(1 - g), the four quotients by one division: 1 / l0 = (l2 l3 / (l0 l1 l2 l3)) l1 and so on (P. L.
             // Montgomery's simultaneous inversion, 1987); the product of four logarithms is between 1e-180 and 1e5.  A quotient goes
             // through three products more than a division of its own: a few units in the last place of fp64, as does the series above.
-            const bool ok[4] = {fit_ok(ga.x), fit_ok(ga.y), fit_ok(ga.z), fit_ok(ga.w)};
-            const float g4[4] = {ga.x, ga.y, ga.z, ga.w};
+            const bool ok[4] = {fit_ok(gn.x), fit_ok(gn.y), fit_ok(gn.z), fit_ok(gn.w)};
+            const float g4[4] = {gn.x, gn.y, gn.z, gn.w};
             double l[4];
 #pragma unroll
             for (int i = 0; i < 4; ++i) l[i] = ok[i] ? fit_log(s_log, (double)g4[i]) : 1.0;
             const double l01 = l[0] * l[1], l23 = l[2] * l[3], inv = 1.0 / (l01 * l23), i01 = inv * l23, i23 = inv * l01;
-            const double B[4] = {fit_double(bu.x), fit_double(bu.y), fit_double(bu.z), fit_double(bu.w)};
-            fit_accumulate(t, a.x, a.y, a.z, B[0], ok[0], ok[0] ? -B[0] * (i01 * l[1]) : 0.0, pr.x, la.x);
-            fit_accumulate(t, a.w, b.x, b.y, B[1], ok[1], ok[1] ? -B[1] * (i01 * l[0]) : 0.0, pr.y, la.y);
-            fit_accumulate(t, b.z, b.w, c.x, B[2], ok[2], ok[2] ? -B[2] * (i23 * l[3]) : 0.0, pr.z, la.z);
-            fit_accumulate(t, c.y, c.z, c.w, B[3], ok[3], ok[3] ? -B[3] * (i23 * l[2]) : 0.0, pr.w, la.w);
+            const double B[4] = {fit_double(bd.x), fit_double(bd.y), fit_double(bd.z), fit_double(bd.w)};
+            fit_accumulate(t, sa.x, sa.y, sa.z, B[0], ok[0], ok[0] ? -B[0] * (i01 * l[1]) : 0.0, pf.x, lt.x);
+            fit_accumulate(t, sa.w, sb.x, sb.y, B[1], ok[1], ok[1] ? -B[1] * (i01 * l[0]) : 0.0, pf.y, lt.y);
+            fit_accumulate(t, sb.z, sb.w, sc.x, B[2], ok[2], ok[2] ? -B[2] * (i23 * l[3]) : 0.0, pf.z, lt.z);
+            fit_accumulate(t, sc.y, sc.z, sc.w, B[3], ok[3], ok[3] ? -B[3] * (i23 * l[2]) : 0.0, pf.w, lt.w);
         }
         done = n4 * 4;
     }
@@ -204,7 +215,7 @@ __global__ void __launch_bounds__(kFitThreads, 2) saba_fit_kernel(const FitParam
     if (threadIdx.x < kFitAcc) {
         double v = s_warp[0][lane];
 #pragma unroll
-        for (int i = 1; i < kFitThreads / 32; ++i) v += s_warp[i][lane];
+        for (int i = 1; i < W; ++i) v += s_warp[i][lane];
         atomicAdd(p.acc + lane, v);
     }
     __threadfence();
@@ -238,6 +249,17 @@ __global__ void __launch_bounds__(kFitThreads, 2) saba_fit_kernel(const FitParam
 
 }  // namespace
 
+size_t saba_fit_doubles() { return 2 * kFitLog + 2 + kFitAcc; }
+void saba_fit_table(double* table) {
+    for (int k = 0; k < kFitLog - 1; ++k) {
+        const double inv = 1.0 / (0.5 + k * (1.0 / 512.0));
+        table[2 * k] = inv;
+        table[2 * k + 1] = -log(inv);
+    }
+    table[2 * (kFitLog - 1)] = 1.0;
+    table[2 * (kFitLog - 1) + 1] = 0.0;
+}
+
 cudaError_t saba_fit_launch(graft_ctx* ctx, long long n, const float* d_state, const int32_t* d_budget,
                             const float* d_gain, const int32_t* d_prefix, const float* d_latency, double* d_out,
                             cudaStream_t st) {
@@ -248,21 +270,19 @@ cudaError_t saba_fit_launch(graft_ctx* ctx, long long n, const float* d_state, c
     p.gain = d_gain;
     p.prefix = d_prefix;
     p.latency = d_latency;
-    p.acc = ctx->w_fit;
-    p.ticket = (unsigned int*)(ctx->w_fit + kFitAcc + 1);
+    p.log = (const double2*)ctx->w_fit;
+    p.ticket = (unsigned int*)(ctx->w_fit + 2 * kFitLog);
+    p.acc = ctx->w_fit + 2 * kFitLog + 2;
     p.out = d_out;
     const bool vec = (((uintptr_t)d_state | (uintptr_t)d_budget | (uintptr_t)d_gain | (uintptr_t)d_prefix |
                        (uintptr_t)d_latency) & 15) == 0;
     long long grid = ((vec ? n / 4 + 3 : n) + kFitThreads - 1) / kFitThreads;
-    const long long cap = (long long)ctx->num_sms * 2;  // what the registers let an SM hold
+    const long long cap = ctx->num_sms;
     if (grid > cap) grid = cap;
     if (grid < 1) grid = 1;
-    if (vec)
-        saba_fit_kernel<true><<<(int)grid, kFitThreads, 0, st>>>(p);
-    else
-        saba_fit_kernel<false><<<(int)grid, kFitThreads, 0, st>>>(p);
+    const cudaError_t e = launch_pdl(vec ? saba_fit_kernel<true> : saba_fit_kernel<false>, dim3((int)grid), dim3(kFitThreads), 0, st, p);
     ctx->launches += 1;
-    return cudaGetLastError();
+    return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 }  // namespace graft

@@ -90,3 +90,23 @@ def test_logarithms_of_gains(g0):
     assert got[9] == 0.0 and got[7] == ref["n_gain"] == n
     assert np.all(np.abs(got[:4] - ref["phi"]) <= RTOL * np.abs(ref["phi"]).max()), (got[:4], ref["phi"])
     g.destroy()
+
+
+@pytest.mark.parametrize("n", [2047, 2049, 303103, 303109, 606211])  # rounds of a thread, of all CTAs once and twice: one less, some more
+def test_sizes_around_whole_turns_back_to_back(n):
+    """Calls that follow one another at once, on other logs: each has its own sums."""
+    g = _ctx()
+    logs = [gi.saba_replay_logs(n + 3 * k, seed=20 + k) for k in range(3)]
+    dev = [{k: torch.from_numpy(np.ascontiguousarray(v)).cuda() for k, v in lg.items()} for lg in logs]
+    outs = torch.zeros((6, 10), dtype=torch.float64, device="cuda")
+    torch.cuda.synchronize()
+    for i in range(6):
+        d = dev[i % 3]
+        g.saba_fit(d["state"], d["budget"], d["gain"], d["prefix_len"], d["latency"], outs[i])
+    got = outs.cpu().numpy()
+    for i in range(6):
+        ref = oracle.saba_fit(**logs[i % 3])
+        assert got[i, 9] == 0.0 and got[i, 7] == ref["n_gain"] and got[i, 8] == ref["n_cost"]
+        assert np.all(np.abs(got[i, :4] - ref["phi"]) <= RTOL * np.abs(ref["phi"]).max() * 10)
+        assert np.all(np.abs(got[i, 4:7] - ref["c"]) <= RTOL * np.maximum(np.abs(ref["c"]), 1e-9) * 100)
+    g.destroy()
