@@ -146,7 +146,7 @@ __device__ __forceinline__ void edge_dots(const float* rP, const float* rC, cons
 // place of every child in the order (edge descending, child rank ascending) by counting the children that come
 // before it.  dots: the parent's K dot products, or nullptr for a parent that does not exist (a row of zeros).
 // wsc: 32 words of shared memory of this warp.  Returns the score in `val` and the place in `rank` (lanes < K).
-__device__ __forceinline__ void edge_row_finish(const float* dots, const float* lps, float scale, float beta, int K,
+__device__ __forceinline__ void edge_row_finish(const float* dots, float lp, float scale, float beta, int K,
                                                 float inv_K, uint32_t* wsc, int lane, float& val, int& rank) {
     const int c = lane;
     val = 0.f;
@@ -159,7 +159,7 @@ __device__ __forceinline__ void edge_row_finish(const float* dots, const float* 
         // remainder, which gives the rounded quotient without the division's special-case code
         const float q0 = sum * inv_K;
         const float mean = fmaf(fmaf(-q0, (float)K, sum), inv_K, q0);
-        val = fmaf(beta, ft - mean, c < K ? lps[c] : 0.f);
+        val = fmaf(beta, ft - mean, lp);
     }
     const uint32_t mine = c < K ? ord_from_float(val) : 0u;  // 0 is below the image of every float
     __syncwarp();

@@ -33,24 +33,16 @@ __device__ __forceinline__ SabaResult saba_warp(const SabaDev& saba, int bmin, i
                                                 const float* topk_lp, const double* cosv, const float* hist_p,
                                                 const int32_t* prefix_p, const int32_t* fixed_budget, int lane) {
     SabaResult r;
-    // everything that comes from global memory is asked for first
-    int st = 0;
-#pragma unroll 1
-    for (int j = lane; j < L; j += 32) st |= row_status[j];
+    // everything that comes from global memory is asked for before any of it is looked at: a lane a position (L <= 32)
+    int st = lane < L ? row_status[lane] : 0;
     const int err = vp_err[0];
     const bool use_saba = fixed_budget == nullptr;
-    double conf = 0.0, rs = 0.0, c_first = 0.0, c_last = 0.0;
-    float hist_f = 0.f;
+    float lp = 0.f, hist_f = 0.f;
+    double rs = 0.0;
     int prefix_i = 0, fixed = 0;
     if (use_saba) {
-#pragma unroll 1
-        for (int j = lane; j < L; j += 32) conf += exp((double)topk_lp[(size_t)j * K]);
-#pragma unroll 1
-        for (int j = lane; j < L - 1; j += 32) rs += cosv[j];
-        if (L >= 2) {
-            c_first = cosv[0];
-            c_last = cosv[L - 2];
-        }
+        lp = lane < L ? topk_lp[(size_t)lane * K] : 0.f;
+        rs = lane < L - 1 ? cosv[lane] : 0.0;
         hist_f = hist_p[0];
         prefix_i = prefix_p[0];
     } else {
@@ -64,6 +56,8 @@ __device__ __forceinline__ SabaResult saba_warp(const SabaDev& saba, int bmin, i
         if (!use_saba) {
             r.budget = fixed < 0 ? 0 : (fixed > bmax ? bmax : fixed);
         } else {
+            double conf = lane < L ? exp((double)lp) : 0.0;
+            const double c_first = __shfl_sync(0xFFFFFFFFu, rs, 0), c_last = __shfl_sync(0xFFFFFFFFu, rs, L >= 2 ? L - 2 : 0);
 #pragma unroll
             for (int d = 16; d > 0; d >>= 1) {
                 conf += __shfl_xor_sync(0xFFFFFFFFu, conf, d);

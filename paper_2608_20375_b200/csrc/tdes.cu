@@ -127,6 +127,7 @@ __global__ void __launch_bounds__(256, 4) tdes_edges_kernel(const EdgeParams p) 
         const int r = threadIdx.x;
         tok = r < n_par ? (j == 0 ? p.root_token[b] : p.topk_id[(row - 1) * K + r]) : p.topk_id[row * K + r - n_par];
     }
+    const float lp_mine = (threadIdx.x & 31) < K ? p.topk_lp[row * K + (threadIdx.x & 31)] : 0.f;
     float* sP = smem;                        // [K][ld]  parent rows + u_d
     float* sC = smem + (size_t)kMaxK * ld;   // [K][ld]  child rows + u_d
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -219,7 +220,7 @@ __global__ void __launch_bounds__(256, 4) tdes_edges_kernel(const EdgeParams p) 
     for (int par = warp; par < K; par += nw) {
         float val;
         int rank;
-        edge_row_finish(par < n_par ? part + (size_t)par * dots_ld(K) : nullptr, lps, p.scale, p.beta, K, inv_K, wsc[warp], lane,
+        edge_row_finish(par < n_par ? part + (size_t)par * dots_ld(K) : nullptr, lp_mine, p.scale, p.beta, K, inv_K, wsc[warp], lane,
                         val, rank);
         if (lane < K) {
             if (WRITE_EDGE) p.edge[(row * K + par) * K + lane] = val;

@@ -665,7 +665,7 @@ __device__ __forceinline__ void lazy_score_row(const TreeParams& p, const TreeSm
     for (int par = warp; par < K; par += NT / 32) {  // one warp per parent
         float val;
         int rank;
-        edge_row_finish(par < n_par ? part + (size_t)par * dots_ld(K) : nullptr, lps, p.scale, p.beta, K, inv_K, wsc, lane, val,
+        edge_row_finish(par < n_par ? part + (size_t)par * dots_ld(K) : nullptr, lane < K ? lps[lane] : 0.f, p.scale, p.beta, K, inv_K, wsc, lane, val,
                         rank);
         if (lane < K) {
             es[(size_t)par * K + es_col(rank, par, K)] = val;
@@ -704,6 +704,14 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int L = p.L, nmax = NMAXC ? NMAXC : p.nmax, W = NMAXC ? (NMAXC + 31) / 32 : p.W;
     const graft_tree_out& o = p.out;
+    __shared__ __align__(8) uint64_t rows_bar, deep_bar;  // (deep_bar: 1024 threads only)
+    __shared__ int rows_abort;
+    if (tid == 0) {
+        rows_abort = 0;
+        mbar_init(smem_u32(&rows_bar), 1);
+        if (NT == 1024) mbar_init(smem_u32(&deep_bar), 1);
+        mbar_fence_init();
+    }
     pdl_launch_dependents();  // an acceptance walk queued behind this kernel may move in; it waits for this grid
     pdl_wait();  // candidates, cosines and edge rows come from the kernels ahead in the stream
     const int b = ORDER ? p.order[blockIdx.x] : (int)blockIdx.x;
@@ -712,8 +720,6 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
     // ---- status and budget ---------------------------------------------------------------------------
     // the sorted edge rows of this sequence: bulk copies through the TMA unit when the 16-byte rules allow it
     // (they land while warp 0 works out the budget), plain loads otherwise
-    __shared__ __align__(8) uint64_t rows_bar, deep_bar;  // (deep_bar: 1024 threads only)
-    __shared__ int rows_abort;
     const int rows_pre = TIES ? L : p.rows_pre;
     const int ne = rows_pre * K * K;  // entries that come from the edge-score kernel for every sequence
     // (a bulk copy's source and size are multiples of 16 bytes: the child ranks are bytes, so the entries copied and the
@@ -740,12 +746,6 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
     }
     int rows_done = rows_pre;  // rows [0, rows_done) are in shared memory
     int inflight = -1;           // on-demand scoring: depth whose table rows are being fetched
-    if (tid == 0) {
-        rows_abort = 0;
-        mbar_init(smem_u32(&rows_bar), 1);
-        if (NT == 1024) mbar_init(smem_u32(&deep_bar), 1);
-        mbar_fence_init();
-    }
     const size_t seq_e = (size_t)b * L * K * K;  // this sequence's rows in esort / eidx
     // entries [lo, hi) of this sequence's rows as bulk copies behind a barrier: one thread
     const auto copy_rows = [&](uint32_t lo, uint32_t hi, uint32_t bar) {
