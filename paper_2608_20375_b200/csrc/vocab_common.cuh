@@ -207,11 +207,10 @@ __device__ __forceinline__ bool vp_bad_row(double Sd, uint32_t Vm, int nk, int K
     const float vmax = __uint_as_float(bits_from_ord(Vm));
     return !(Sd > 0.0) || !(Sd < 1e300) || Vm == 0u || vmax == INFINITY || vmax == -INFINITY || nk < K;
 }
-// The outputs of a finished row: its log-sum-exp and the K best keys.  One warp.
-__device__ __forceinline__ void vp_write_row(double lse_d, int status, int nk, int K, const uint64_t* keys, int lane,
+// The outputs of a finished row: its log-sum-exp and the K best keys, a lane a key.  One warp.
+__device__ __forceinline__ void vp_write_row(double lse_d, int status, int nk, int K, uint64_t key, int lane,
                                              int32_t* topk_id, float* topk_lp, float* lse, int32_t* row_status) {
     if (lane < K) {
-        const uint64_t key = lane < nk ? keys[lane] : 0ull;
         topk_id[lane] = lane < nk ? (int32_t)key_id(key) : -1;
         topk_lp[lane] = lane < nk ? (float)((double)key_value(key) - lse_d) : 0.f;
     }
@@ -232,7 +231,7 @@ __device__ __forceinline__ void vp_finalize(double Cd, double Sd, uint32_t Vm, i
     Vm = __shfl_sync(0xFFFFFFFFu, Vm, 0);
     const double lse_d = vp_lse(Cd, Sd, __uint_as_float(bits_from_ord(Vm)));
     const int status = (vp_bad_row(Sd, Vm, nk, K) ? GRAFT_ST_BAD_LOGITS : 0) | (internal ? GRAFT_ST_INTERNAL : 0);
-    vp_write_row(lse_d, status, nk, K, keys, lane, topk_id, topk_lp, lse, row_status);
+    vp_write_row(lse_d, status, nk, K, lane < nk ? keys[lane] : 0ull, lane, topk_id, topk_lp, lse, row_status);
 }
 
 }  // namespace

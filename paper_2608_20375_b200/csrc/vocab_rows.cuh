@@ -706,7 +706,7 @@ __global__ void __launch_bounds__(NT + 32, NT == 256 ? 4 : 2) vocab_rows_kernel(
                 }
             } else {
                 const int status = (vp_bad_row(sh->S, sh->vmax, nk, p.K) ? GRAFT_ST_BAD_LOGITS : 0) | (internal ? GRAFT_ST_INTERNAL : 0);
-                vp_write_row(sh->lse_d, status, nk, p.K, sh->outk, lane, p.topk_id + (size_t)row * p.K,
+                vp_write_row(sh->lse_d, status, nk, p.K, lane < nk ? sh->outk[lane] : 0ull, lane, p.topk_id + (size_t)row * p.K,
                              p.topk_lp + (size_t)row * p.K, p.lse + row, p.row_status + row);
             }
         }

@@ -445,6 +445,41 @@ def test_tdes_edges_against_oracle(K, L, m, beta, root_edge):
 
 
 # --------------------------------------------------------------------------- vocabulary-parallel vocab pass
+@pytest.mark.parametrize("world", [1, 2, 3, 4, 5, 7, 8, 9, 16, 17, 33, 64])
+@pytest.mark.parametrize("K", [32, 5])
+def test_merge_over_any_number_of_shards(world, K):
+    """Lists merged two by two, eight at a time: the ids of the whole rows, masked and bad ones among them (five rows: the last CTA
+    of the merge has places without a row)."""
+    from paper_2608_20375_b200 import Graft
+    from paper_2608_20375_b200.binding import VOCAB_PARTIAL_BYTES
+    from paper_2608_20375_b200.vocab_parallel import vocab_range
+    V, L = 12800, 5
+    gen = torch.Generator(device="cuda").manual_seed(world)
+    z = 2.0 * torch.randn((1, L, V), generator=gen, device="cuda")
+    z[0, 1, 40:] = float("-inf")  # one shard has all that is left
+    z[0, 2] = torch.round(z[0, 2])  # ties across shards
+    z[0, 3, 77] = float("nan")
+    z[0, 4, 3:] = float("-inf")  # fewer than K tokens
+    whole = Graft(V, L, K, 16, 8, 1, 8, 8, 8, 0.0, 1, 0, 0)
+    e = lambda *s, t=torch.float32: torch.empty(s, dtype=t, device="cuda")  # noqa: E731
+    ids, lp, lse, rs = e(1, L, K, t=torch.int32), e(1, L, K), e(1, L), e(1, L, t=torch.int32)
+    whole.vocab_pass(z, ids, lp, lse, rs)
+    parts, offs = e(world, L, VOCAB_PARTIAL_BYTES, t=torch.uint8), []
+    for r in range(world):
+        lo, hi = vocab_range(V, r, world)
+        g = Graft(hi - lo, L, K, 16, 8, 1, 8, 8, 8, 0.0, 1, 0, 0)
+        g.vocab_pass_partial(z[:, :, lo:hi].contiguous(), parts[r])
+        offs.append(lo)
+    out = e(1, L, K, t=torch.int32), e(1, L, K), e(1, L), e(1, L, t=torch.int32)
+    g.vocab_merge(parts, offs, *out)
+    torch.cuda.synchronize()
+    assert torch.equal(out[3], rs) and rs[0].tolist()[:3] == [0, 0, 0] and rs[0, 3] != 0
+    good = rs[0] == 0
+    assert torch.equal(out[0][0, good], ids[0, good])
+    for got, want in ((out[1], lp), (out[2], lse)):  # (masked tokens: minus infinity on both sides)
+        assert torch.where(got == want, torch.zeros_like(got), got - want)[0, good].abs().max() <= 2e-6
+
+
 @pytest.mark.parametrize("V,K,L,Bt,dtype,world", [
     (50000, 16, 4, 3, "bf16", 2), (151936, 32, 2, 2, "bf16", 4), (32000, 8, 3, 2, "f32", 3), (9000, 32, 2, 2, "bf16", 8),
     (70, 16, 2, 2, "f32", 5),  # shards narrower than K
