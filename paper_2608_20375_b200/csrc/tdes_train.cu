@@ -741,13 +741,16 @@ __global__ void __launch_bounds__(kTsThreads, 1) tdes_loss_rows_kernel(const Tra
             ctx_add_u<FULL>(c, __shfl_sync(0xFFFFFFFFu, d, i), mul4(cf, add4(a[i], b[i])));
         }
     }
-    // ---- per-CTA sums, then one round of global atomics
+    // ---- per-CTA sums, then one round of global reductions, four values each: of few groups this end was a tenth of the
+    //      call (500 groups, K = 32: 15.6 us with one value each, 14.1 so; 2,000 groups: 40.4 and 38.6; 4,000: no change)
     __syncthreads();
     if (grad)
-        for (int i = tid; i < Lm; i += kTsThreads) {
-            float v = s_gu[i];
-            for (int w = 1; w < p.gu_copies; ++w) v += s_gu[(size_t)w * Lm + i];
-            if (v != 0.f) atomicAdd(p.gu + i, v);
+        for (int i = tid; i < Lm / 4; i += kTsThreads) {
+            const float4* q = (const float4*)s_gu + i;
+            float4 v = *q;
+#pragma unroll 4
+            for (int w = 1; w < p.gu_copies; ++w) v = add4(v, q[(size_t)w * (Lm / 4)]);
+            if (v.x != 0.f || v.y != 0.f || v.z != 0.f || v.w != 0.f) red_add4((float4*)p.gu + i, v);
         }
     train_finish(p, s_sum, l_kl, l_pair, l_bce, gs, skipped, lane);
 }
