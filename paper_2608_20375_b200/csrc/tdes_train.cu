@@ -767,11 +767,12 @@ __global__ void __launch_bounds__(kTsThreads, 1) tdes_loss_rows_kernel(const Tra
 //     children's rows read a second time -- because 24 warps of 80 registers beat 12 that keep the rows (150 us against 163);
 //   * tdes_items_kernel: a batch of pairs and edges is sorted by depth in shared memory, so that a warp keeps u_d and its sum
 //     of gu_d in registers; the most frequent tokens of the first batch are summed up per warp in shared memory.
-// Measured (B200, V = 151,936, m = 128, L = 16, 32,768 groups of 32, 131,072 pairs, 262,144 edges): 260 us, the two alone 150
+// Measured (B200, V = 151,936, m = 128, L = 16, 32,768 groups of 32, 131,072 pairs, 262,144 edges): 251 us, the two alone 150
 // and 99; 320 by the kernel above with the frequent tokens' rows per warp.  1.2 million additions are 115 us of it, the
 // rest chains of loads and exchanges.  Tried: the frequent tokens' rows as one dense block whose scores and coefficients are
 // single numbers (423 us: four numbers a reference cost what a row does, and the sums lost a digit); two warps a group with
-// the rows kept (150 - 190); both kernels on an SM at once, half the warps each (249 against 251).
+// the rows kept (150 - 190); both kernels on an SM at once, half the warps each (249 against 251); the children's rows read once, with
+// a running softmax (163 - 167 against 150: the longer chain of a group costs what the second read does).
 constexpr int kTgGroups = 224;  // groups of a batch at most
 constexpr int kTgThreads = 768;
 constexpr int kTgBinBits = 13, kTgBins = 1 << kTgBinBits;
