@@ -767,7 +767,7 @@ __global__ void __launch_bounds__(kTsThreads, 1) tdes_loss_rows_kernel(const Tra
 //     children's rows read a second time -- because 24 warps of 80 registers beat 12 that keep the rows (150 us against 163);
 //   * tdes_items_kernel: a batch of pairs and edges is sorted by depth in shared memory, so that a warp keeps u_d and its sum
 //     of gu_d in registers; the most frequent tokens of the first batch are summed up per warp in shared memory.
-// Measured (B200, V = 151,936, m = 128, L = 16, 32,768 groups of 32, 131,072 pairs, 262,144 edges): 251 us, the two alone 150
+// Measured (B200, V = 151,936, m = 128, L = 16, 32,768 groups of 32, 131,072 pairs, 262,144 edges): 250 us, the two alone 147
 // and 99; 320 by the kernel above with the frequent tokens' rows per warp.  1.2 million additions are 115 us of it, the
 // rest chains of loads and exchanges.  Tried: the frequent tokens' rows as one dense block whose scores and coefficients are
 // single numbers (423 us: four numbers a reference cost what a row does, and the sums lost a digit); two warps a group with
@@ -898,7 +898,7 @@ __global__ void __launch_bounds__(kTgThreads, 1) tdes_groups_kernel(const TrainP
                     base += __shfl_sync(0xFFFFFFFFu, incl, 31);
                 }
             }
-            if (tid < 32 && n_rec + tid < ((n_rec + 31) & ~31)) s_rec[n_rec + tid] = 0xFFFFu;
+            if (tid < 32 && n_rec + tid < ((n_rec + 31) & ~31)) s_rec[n_rec + tid] = 0u;
         }
         // ---- products with the parent: eight children at a time
         for (int gl = warp; gl < ng; gl += W) {
@@ -1035,19 +1035,25 @@ __global__ void __launch_bounds__(kTgThreads, 1) tdes_groups_kernel(const TrainP
                 }
             }
             if (r0 < n_rec) {
-                const int me = s_rec[r0 + lane], tok = me != 0xFFFF ? s_tok[me] : -1, next = __shfl_down_sync(0xFFFFFFFFu, tok, 1);
-                const float my_cf = me != 0xFFFF ? s_f[me] : 0.f;
+                const int me = s_rec[r0 + lane], tok = r0 + lane < n_rec ? s_tok[me] : -1, next = __shfl_down_sync(0xFFFFFFFFu, tok, 1);
                 uint32_t ends = __ballot_sync(0xFFFFFFFFu, tok >= 0 && (lane == 31 || next != tok));  // the last of a token's
-                const int my_row = me != 0xFFFF ? me / KC * 32 : 0;
                 float4 acc = zero4;
 #pragma unroll 1
                 for (int i0 = 0; i0 < 32; i0 += 8, ends >>= 8) {
+                    // (places and coefficients as broadcast loads: from lane to lane they cost two exchanges a row, 152 us against 147)
+                    const uint4 recs = *(const uint4*)(s_rec + r0 + i0);
+                    const uint32_t word[4] = {recs.x, recs.y, recs.z, recs.w};
                     float4 row[8];
-#pragma unroll
-                    for (int q = 0; q < 8; ++q) row[q] = s_a[__shfl_sync(0xFFFFFFFFu, my_row, i0 + q) + lane];
+                    float cf[8];
 #pragma unroll
                     for (int q = 0; q < 8; ++q) {
-                        acc = fma4(__shfl_sync(0xFFFFFFFFu, my_cf, i0 + q), row[q], acc);
+                        const uint32_t m = q & 1 ? word[q >> 1] >> 16 : word[q >> 1] & 0xFFFFu;
+                        cf[q] = s_f[m];
+                        row[q] = s_a[m / KC * 32 + lane];
+                    }
+#pragma unroll
+                    for (int q = 0; q < 8; ++q) {
+                        acc = fma4(cf[q], row[q], acc);
                         if (ends & (1u << q)) {  // (uniform)
                             const int t = __shfl_sync(0xFFFFFFFFu, tok, i0 + q);
                             if (on) red_add4((float4*)(p.gC + (size_t)t * mm) + lane, acc);
