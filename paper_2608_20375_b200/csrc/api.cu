@@ -427,14 +427,22 @@ graft_status graft_build_trees(graft_ctx* ctx, int32_t batch, const void* d_logi
     // kernel then only reads; without an edge-score kernel the tree kernel does it itself.
     // Without edge scores (beta = 0) nothing needs that kernel: the tree kernel lays the rows out from log q.
     const int rows = out->d_edge ? ctx->cfg.L : neutral ? 0 : ctx->edge_rows;
+    // the edge-score kernel counts sequences for the tree kernel, which clears the count: where either does not start, a clear
+    // in the stream takes its place
+    const auto failed = [&] {
+        cudaGetLastError();
+        cudaMemsetAsync(ctx->w_order_n, 0, 2 * sizeof(int), st);
+        cudaGetLastError();
+        return GRAFT_ERR_CUDA;
+    };
     if (rows > 0 && tdes_edges_launch(ctx, batch, ids, lps, d_root_token, ctx->w_row_status, edge, ctx->w_esort,
                                       ctx->w_eidx, rows, ctx->w_saba, d_hist, d_prefix_len, d_fixed_budget,
                                       st) != cudaSuccess)
-        return GRAFT_ERR_CUDA;
+        return failed();
     if (ev) cudaEventRecord(ev[2], st);
     if (tree_launch(ctx, batch, ids, lps, ctx->w_row_status, ctx->w_esort, ctx->w_eidx, d_hidden, d_root_token, d_hist,
                     d_prefix_len, d_fixed_budget, ctx->w_cos, rows > 0 ? ctx->w_saba : nullptr, out, st) != cudaSuccess)
-        return GRAFT_ERR_CUDA;
+        return failed();
     if (ev) {
         cudaEventRecord(ev[3], st);
         ex->timing.calls += 1;

@@ -152,7 +152,7 @@ __global__ void __launch_bounds__(256, 4) tdes_edges_kernel(const EdgeParams p) 
             const bool front = rows_ahead_sum(rows_ahead_load(p.topk_lp + (size_t)b * p.L * K, p.L, K), p.L) >= kTreeLongMean * (float)p.L;
             if (lane == 0) {
                 const int at = atomicAdd(p.order_n + (front ? 0 : 1), 1);
-                p.order[front ? at : (int)gridDim.x - 1 - at] = b;
+                if (at < (int)gridDim.x) p.order[front ? at : (int)gridDim.x - 1 - at] = b;  // (always, as long as order_n was zero)
             }
         }
         return;
