@@ -1494,6 +1494,11 @@ cudaError_t tdes_loss_launch(graft_ctx* ctx, const graft_tdes_traces* tr, const 
             ctx->launches += 1;
             if (e == cudaSuccess) e = cudaGetLastError();
         }
+        // (thread blocks of a kernel that did start have arrived at sums that the other's would have brought back to zero)
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            cudaMemsetAsync(ctx->w_loss, 0, kLossSums * sizeof(double), st);
+        }
         return e;
     }
     cudaError_t e = cudaMemsetAsync(d_loss, 0, 4 * sizeof(double), st);

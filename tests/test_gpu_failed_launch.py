@@ -28,7 +28,7 @@ int cudaLaunchKernelExC(const void* config, const void* func, void** args) {
 """
 
 
-@pytest.mark.parametrize("case", ["round"])
+@pytest.mark.parametrize("case", ["round", "loss"])
 def test_calls_after_a_launch_that_failed(tmp_path, case):
     src, so = os.path.join(str(tmp_path), "shim.c"), os.path.join(str(tmp_path), "shim.so")
     with open(src, "w") as f:
@@ -84,8 +84,49 @@ def _round(shim):
                 assert np.array_equal(got[k], w), k
 
 
+def _loss(shim):
+    """Many traces: two kernels whose thread blocks count themselves; the last of all of them writes the losses."""
+    import torch
+    from paper_2608_20375_b200 import Graft, GraftError
+    V, L, K, m, n = 3000, 16, 16, 128, 9000
+    gen = torch.Generator(device="cuda").manual_seed(5)
+    rand = lambda *s: torch.randn(s, generator=gen, device="cuda")  # noqa: E731
+    ints = lambda lo, hi, *s: torch.randint(lo, hi, s, generator=gen, device="cuda", dtype=torch.int32)  # noqa: E731
+    g = Graft(V, L, K, m, 32, 1, 8, 16)
+    P, Ct, u = rand(V, m), rand(V, m), 0.5 * rand(L, m)
+    g.set_tdes_tables(P, Ct, u, 1.0)
+    groups = dict(parent=ints(0, V, n), depth=ints(1, L + 1, n), child=ints(0, V, n, K), logq=rand(n, K), ztgt=rand(n, K))
+    pairs = torch.stack([ints(0, V, n), ints(0, V, n), ints(1, L + 1, n), ints(0, V, n), ints(0, V, n), ints(1, L + 1, n)], 1).contiguous()
+    edges = torch.stack([ints(0, V, n), ints(0, V, n), ints(1, L + 1, n), ints(0, 2, n)], 1).contiguous()
+
+    def step():
+        out = dict(loss=torch.zeros(4, dtype=torch.float64, device="cuda"), skipped=torch.zeros(1, dtype=torch.int32, device="cuda"),
+                   gP=torch.zeros((V, m), device="cuda"), gC=torch.zeros((V, m), device="cuda"),
+                   gu=torch.zeros((L, m), device="cuda"), gs=torch.zeros(1, device="cuda"))
+        g.tdes_loss(groups, pairs, edges, gamma=0.5, w1=4.0, lambda_kl=1.0, lambda_pair=1.0, lambda_bce=0.25, **out)
+        torch.cuda.synchronize()
+        return out
+
+    want = step()
+    for _ in range(3):
+        shim.shim_fail(1)  # (the second of the two kernels: the first is launched the ordinary way)
+        try:
+            step()
+            raise SystemExit("the call did not report the launch that failed")
+        except GraftError:
+            pass
+        torch.cuda.synchronize()
+    shim.shim_fail(0)
+    for _ in range(2):
+        got = step()
+        assert got["skipped"].item() == 0
+        assert torch.allclose(got["loss"], want["loss"], rtol=1e-12, atol=0.0), (got["loss"], want["loss"])
+        for k in ("gP", "gC", "gu"):
+            assert ((got[k] - want[k]).abs().max() <= 1e-4 * want[k].abs().max()).item(), k
+
+
 if __name__ == "__main__":
     import ctypes
     sys.path.insert(0, ROOT)
-    {"round": _round}[sys.argv[1]](ctypes.CDLL(sys.argv[2]))
+    {"round": _round, "loss": _loss}[sys.argv[1]](ctypes.CDLL(sys.argv[2]))
     print("fine")
