@@ -370,13 +370,6 @@ __device__ __forceinline__ float warp_sums(float (&v)[N], int lane) {
     for (; mask >= 1; mask >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, mask);
     return s;
 }
-__device__ __forceinline__ float dot8(const float4 (&a)[2], const float4 (&b)[2]) {
-    float2 s = __fmul2_rn(hi2(a[0]), hi2(b[0]));
-    s = __ffma2_rn(lo2(a[0]), lo2(b[0]), s);
-    s = __ffma2_rn(lo2(a[1]), lo2(b[1]), s);
-    s = __ffma2_rn(hi2(a[1]), hi2(b[1]), s);
-    return s.x + s.y;
-}
 // Sums of N values over either half of the warp (N = 4, 8, 16): value i is returned to the half's lanes with
 // (l >> (4 - log2 N)) == i.
 template <int N>
@@ -906,7 +899,7 @@ __global__ void __launch_bounds__(kTgThreads, 1) tdes_groups_kernel(const TrainP
             if (d == 0) continue;
             float4 a[2];
             half_row(p.P, s_parent[gl], a);
-            float au = 0.f;
+            float au[2] = {};
 #pragma unroll 1
             for (int c = 0; c < KC; c += 8) {
                 const int4 t = *(const int4*)(s_tok + gl * KC + c + 4 * h);
@@ -915,21 +908,20 @@ __global__ void __launch_bounds__(kTgThreads, 1) tdes_groups_kernel(const TrainP
                 half_row(p.C, t.y, rows[1]);
                 half_row(p.C, t.z, rows[2]);
                 half_row(p.C, t.w, rows[3]);
-                if (c == 0) {  // f = k0 (a . C + a . u)
+                if (c == 0) {  // f = k0 (a . C + a . u), summed up in the order of tdes_loss_rows_kernel: the same bits
                     const float4* q = (const float4*)(s_u + (d - 1) * p.m) + l;
                     const float4 u0 = on0 ? q[0] : zero4, u1 = on1 ? q[16] : zero4;
                     a[0] = add4(a[0], u0);
                     a[1] = add4(a[1], u1);
-                    au = dot4(a[0], u0) + dot4(a[1], u1);
-#pragma unroll
-                    for (int o = 8; o > 0; o >>= 1) au += __shfl_xor_sync(0xFFFFFFFFu, au, o);
+                    au[0] = dot4(a[0], u0);
+                    au[1] = dot4(a[1], u1);
                     s_a[gl * 32 + lane] = h ? a[1] : a[0];
                 }
                 float part[4];
 #pragma unroll
-                for (int i = 0; i < 4; ++i) part[i] = dot8(a, rows[i]);
+                for (int i = 0; i < 4; ++i) part[i] = (au[0] + dot4(a[0], rows[i][0])) + (au[1] + dot4(a[1], rows[i][1]));
                 const float dot = half_sums<4>(part, lane);  // child i of the half in lanes 16 h + 4 i ..
-                if ((l & 3) == 0) s_f[gl * KC + c + 4 * h + (l >> 2)] = au + dot;
+                if ((l & 3) == 0) s_f[gl * KC + c + 4 * h + (l >> 2)] = dot;
             }
         }
         __syncthreads();

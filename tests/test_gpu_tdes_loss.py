@@ -191,6 +191,21 @@ def test_many_traces(V, L, K, m, ng, npair, ne, grad):
     g.destroy()
 
 
+@pytest.mark.parametrize("V,L,K,m,ng,npair,ne", [
+    (3000, 16, 32, 128, 4000, 9000, 9000),
+    (3000, 16, 17, 64, 6000, 9000, 9000),
+    (3000, 7, 9, 124, 9000, 9000, 9000),
+    (3000, 32, 8, 128, 18000, 0, 0),
+])
+def test_losses_alone_of_many_traces(V, L, K, m, ng, npair, ne):
+    """With gradients these go to other kernels than without: the same scores, summed up in 64 bits in another order."""
+    g, P, Ct, u, s, keep = _ctx(V, L, K, m, seed=V + K)
+    tr = gi.tdes_traces(V, L, K, ng, npair, ne, seed=V + L)
+    both, alone = _run(g, V, L, m, tr), _run(g, V, L, m, tr, grad=False)
+    assert np.allclose(alone["loss"], both["loss"], rtol=1e-12, atol=0.0), (alone["loss"], both["loss"])
+    g.destroy()
+
+
 def test_many_traces_bad_ids_and_lists_at_odd_addresses():
     V, L, K, m, ng, npair, ne = 900, 6, 8, 128, 9000, 9000, 16000
     g, P, Ct, u, s, keep = _ctx(V, L, K, m, seed=41)
