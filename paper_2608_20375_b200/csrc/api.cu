@@ -287,7 +287,7 @@ graft_status graft_tdes_precompute(graft_ctx* ctx, const void* d_emb, graft_dtyp
     if (!ctx || !d_emb || !d_W || !d_out || E < 1) return GRAFT_ERR_INVALID_ARG;
     if (emb_dtype != GRAFT_F32 && emb_dtype != GRAFT_BF16) return GRAFT_ERR_INVALID_ARG;
     // the tensor cores (16-bit parts of the inputs, exact products), where the rows fit and their scratch is to be had
-    if (tables_mma_fits(d_emb, emb_dtype, E, d_out)) {
+    if (tables_mma_fits(ctx->num_sms, ctx->cfg.V, d_emb, emb_dtype, E, ctx->cfg.m, d_out)) {
         void* scratch = tables_scratch(ctx, tables_mma_scratch_bytes(ctx->num_sms, ctx->cfg.V, E, ctx->cfg.m, emb_dtype));
         if (scratch != nullptr) {
             if (tables_mma_launch(ctx, d_emb, emb_dtype, E, d_W, d_b, d_out, scratch, (cudaStream_t)stream) == cudaSuccess)

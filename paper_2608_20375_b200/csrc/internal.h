@@ -161,7 +161,7 @@ int vp_merge_max_shards();
 cudaError_t tdes_precompute_launch(graft_ctx* ctx, const void* d_emb, graft_dtype dt, int E, const float* d_W,
                                    const float* d_b, float* d_out, cudaStream_t st);
 // table precompute on the tensor cores (csrc/tables_mma.cu); inputs that do not fit go to tdes_precompute_launch
-bool tables_mma_fits(const void* d_emb, graft_dtype dt, int E, const void* d_out);
+bool tables_mma_fits(int num_sms, int V, const void* d_emb, graft_dtype dt, int E, int m, const void* d_out);
 size_t tables_mma_scratch_bytes(int num_sms, int V, int E, int m, graft_dtype dt);
 cudaError_t tables_mma_launch(graft_ctx* ctx, const void* d_emb, graft_dtype dt, int E, const float* d_W, const float* d_b,
                               float* d_out, void* scratch, cudaStream_t st);

@@ -968,9 +968,15 @@ cudaError_t tables_run(const TablesParams& p, cudaStream_t st, int* launches) {
 }  // namespace
 
 // Can the tensor cores take this table?  16-byte rows for the loads and stores; anything else goes to the FMA kernel.
-bool tables_mma_fits(const void* d_emb, graft_dtype dt, int E, const void* d_out) {
-    // (E: shares of the tiles that are left are worked out in 32 bits)
-    return E <= 1 << 22 && E % (dt == GRAFT_BF16 ? 8 : 4) == 0 && (((uintptr_t)d_emb | (uintptr_t)d_out) & 15) == 0 && encode_tiled() != nullptr;
+bool tables_mma_fits(int num_sms, int V, const void* d_emb, graft_dtype dt, int E, int m, const void* d_out) {
+    if (E % (dt == GRAFT_BF16 ? 8 : 4) != 0 || (((uintptr_t)d_emb | (uintptr_t)d_out) & 15) != 0 || encode_tiled() == nullptr) return false;
+    // Shares of the tiles that are left are worked out in 32 bits (tables_share, tables_owner), which holds for all that fits in
+    // memory: 148 workers share 28 million blocks and more, of 16 KB each, and a few narrow tiles are shared by fewer.
+    const int rows = dt == GRAFT_F32 ? TablesCfg<true>::ROWS : TablesCfg<false>::ROWS, blk = dt == GRAFT_F32 ? TablesCfg<true>::BLK : TablesCfg<false>::BLK;
+    const TablesSizes s = tables_sizes(num_sms, V, E, m, dt == GRAFT_F32);
+    const uint64_t left = (uint64_t)((V + (long long)rows - 1) / rows * s.n_mb % s.pairs);
+    const uint64_t share = left * kTmMaxSplit < (uint64_t)s.pairs ? left * kTmMaxSplit : (uint64_t)s.pairs;
+    return (share + 1) * left * ((uint64_t)(E + (long long)blk - 1) / blk) <= 0xFFFFFFFFull;
 }
 size_t tables_mma_scratch_bytes(int num_sms, int V, int E, int m, graft_dtype dt) {
     return tables_sizes(num_sms, V, E, m, dt == GRAFT_F32).total;

@@ -125,6 +125,19 @@ def test_fp32_chunks_and_tiles_of_odd_lengths(V, E, m):
     assert ((got - want).abs() <= 1e-5 + 1e-6 * want.abs()).all()  # (a sum's rounding: 2e-6 at most, measured)
 
 
+@pytest.mark.parametrize("V,E,m,dtype", [(5, (1 << 22) + 64, 8, "f32"), (5, (1 << 22) + 64, 8, "bf16"), (130, (1 << 23) + 4, 4, "f32")])
+def test_rows_of_many_million_columns(V, E, m, dtype):
+    """Tables of any length that fits in memory go to the tensor cores (more than one kernel a table)."""
+    emb, W, b = _inputs(V, E, m, dtype, 13)
+    g = _graft(V, m)
+    n = g.launch_count()
+    got = _call(g, emb, W, b, m).double()
+    assert g.launch_count() - n > 1
+    want = b.double() + sum(_exact(emb[:, i:i + (1 << 19)], W[:, i:i + (1 << 19)]) for i in range(0, E, 1 << 19))
+    assert ((got - want).abs() <= 2e-5 + 2e-6 * want.abs()).all()
+    g.destroy()
+
+
 @pytest.mark.parametrize("part", ["embedding", "W", "both"])
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 def test_parts_of_every_order_count(part, dtype):
