@@ -92,7 +92,7 @@ struct graft_ctx {
     int32_t* w_order;             // [max_batch] order in which the trees of more sequences than SMs are built
     int* w_order_n;               // [2] sequences placed in it from either end, zero between rounds
     double* w_fit;                // graft_saba_fit: table of logarithms, arrival counter and normal equations (both zero between calls)
-    bool loss_many;               // graft_tdes_loss's kernels for many traces are ready
+    bool loss_hot, loss_many;     // graft_tdes_loss's kernels for frequent tokens and for many traces are ready
     double* w_loss;               // [kLossSums] sums of graft_tdes_loss and its arrival counter, zero between calls
     int32_t* w_errflag;           // [1] device-side internal error flag
     graft::VpPlan vp_plan;

@@ -253,7 +253,44 @@ def test_full_size_tables():
     g.destroy()
 
 
-@pytest.mark.parametrize("n", [6000])
+@pytest.mark.parametrize("ng,npair,ne,V", [(2000, 4000, 8000, 40), (9000, 9000, 9000, 3000), (30, 40, 50, 300)])
+def test_first_call_under_capture(ng, npair, ne, V):
+    """Kernels that are loaded with the first call that wants them."""
+    L, K, m = 6, 32, 128
+    g, P, Ct, u, s, keep = _ctx(V, L, K, m, seed=51)
+    tr = gi.tdes_traces(V, L, K, ng, npair, ne, seed=52)
+    groups, pairs, edges = _dev(tr)
+    out = dict(loss=torch.zeros(4, dtype=torch.float64, device="cuda"), skipped=torch.zeros(1, dtype=torch.int32, device="cuda"),
+               gP=torch.zeros((V, m), device="cuda"), gC=torch.zeros((V, m), device="cuda"), gu=torch.zeros((L, m), device="cuda"),
+               gs=torch.zeros(1, device="cuda"))
+    graph = torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph):
+        g.tdes_loss(groups, pairs, edges, **out, **CFG)
+    ref = oracle.tdes_loss(P, Ct, u, s, tr["groups"], tr["pairs"], tr["edges"], **CFG)
+    for _ in range(2):
+        for k in ("gP", "gC", "gu", "gs"):
+            out[k].zero_()
+        graph.replay()
+        torch.cuda.synchronize()
+        _compare({k: v.cpu().numpy() for k, v in out.items()}, ref)
+        assert out["skipped"].item() == 0
+    del graph
+    g.destroy()
+
+
+def test_large_and_small_steps_by_turns():
+    """Every kernel of a step leaves the context's sums and counters as it found them."""
+    V, L, K, m = 700, 9, 16, 128
+    g, P, Ct, u, s, keep = _ctx(V, L, K, m, seed=61)
+    traces = [gi.tdes_traces(V, L, K, *n, seed=62 + i) for i, n in enumerate([(9000, 9000, 9000), (60, 70, 80), (3000, 5000, 5000), (9000, 0, 0), (0, 9000, 60000)])]
+    refs = [oracle.tdes_loss(P, Ct, u, s, t["groups"], t["pairs"], t["edges"], **CFG) for t in traces]
+    for i, grad in [(0, True), (0, True), (1, True), (0, False), (0, True), (2, True), (4, True), (3, True), (2, False), (1, False), (2, True), (0, True)]:
+        _compare(_run(g, V, L, m, traces[i], grad=grad), refs[i], grad=grad)
+    g.destroy()
+
+
+@pytest.mark.parametrize("n", [2000, 6000])
 def test_traces_of_few_tokens(n):
     """Additions to one row of a gradient follow one another, so frequent tokens' rows are summed up on chip first: with parents and items by
     a power of 1.6 of the tokens' rank, where ten tokens have three quarters of the references, a step takes as long as by 1.1
