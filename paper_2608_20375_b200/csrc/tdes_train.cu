@@ -333,7 +333,7 @@ constexpr long long kTsMany = 131072, kTsManyLoss = 655360;
 // sample is worth its 1.5 us: 65 thousand references 21.5 us).
 constexpr long long kTsHotMin = 65536;
 
-constexpr int kTsSlots = 8, kTsFew = 4;  // hot rows per table: of the kernel for pairs and edges, of the one for fewer traces
+constexpr int kTsSlots = 8;  // hot rows per table
 struct __align__(16) TrainHot {
     int tok[2][kTsSlots];
 };
@@ -398,15 +398,12 @@ __device__ __forceinline__ float warp_sum(float s) {
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
     return s;
 }
-template <int N>
 __device__ __forceinline__ int hot_slot(const TrainHot& h, int t, int tok) {
-    const int4 x = *(const int4*)h.tok[t];
+    const int4 x = *(const int4*)h.tok[t], y = *((const int4*)h.tok[t] + 1);
     int s = tok == x.x ? 0 : -1;
     s = tok == x.y ? 1 : s;
     s = tok == x.z ? 2 : s;
     s = tok == x.w ? 3 : s;
-    if (N == 4) return s;
-    const int4 y = *((const int4*)h.tok[t] + 1);
     s = tok == y.x ? 4 : s;
     s = tok == y.y ? 5 : s;
     s = tok == y.z ? 6 : s;
@@ -452,7 +449,7 @@ __device__ __forceinline__ void smem_add4(float4* q, const float4& v) { *q = add
 struct TrainCtx {
     const float* u;   // [L][m] shared copy of the depth embeddings
     float* gu;        // [L][m] this warp's sums (or the CTA's, with atomics)
-    float4* hot;      // [2][N][32] this warp's sums of the hot rows
+    float4* hot;      // [2][kTsSlots][32] this warp's sums of the hot rows
     bool gu_shared, on;  // on: this lane holds a part of a row
     int lane, m;
 };
@@ -461,10 +458,10 @@ template <bool FULL>
 __device__ __forceinline__ float4* ctx_at(const TrainCtx& c, const float* table, int tok) {
     return (float4*)(table + (size_t)tok * (FULL ? 128 : c.m)) + c.lane;
 }
-template <bool FULL, int N>
+template <bool FULL>
 __device__ __forceinline__ void ctx_add_row(const TrainParams& p, const TrainCtx& c, int t, int tok, int slot, const float4& v) {
     if (slot >= 0)  // (uniform)
-        smem_add4(c.hot + (t * N + slot) * 32 + c.lane, v);
+        smem_add4(c.hot + (t * kTsSlots + slot) * 32 + c.lane, v);
     else if (FULL || c.on)
         red_add4(ctx_at<FULL>(c, t == 0 ? p.gP : p.gC, tok), v);
 }
@@ -491,16 +488,15 @@ __device__ __forceinline__ float4 ctx_u(const TrainCtx& c, int d) {
     return FULL || c.on ? *ctx_at<FULL>(c, c.u, d - 1) : make_float4(0.f, 0.f, 0.f, 0.f);
 }
 
-// The sums of the frequent tokens' rows that the warps in the mask kept, [warp][2][N][32], go out: one addition a row and CTA.
-template <int N>
+// The sums of the frequent tokens' rows that the warps in the mask kept, [warp][2][kTsSlots][32], go out: one addition a row and CTA.
 __device__ __forceinline__ void flush_hot(const TrainParams& p, const TrainHot& h, const float4* rows, uint32_t warps, int tid, int threads) {
-    for (int i = tid; i < 2 * N * 32; i += threads) {
-        const int r = i >> 5, l = i & 31, tok = h.tok[r / N][r % N];
+    for (int i = tid; i < 2 * kTsSlots * 32; i += threads) {
+        const int r = i >> 5, l = i & 31, tok = h.tok[r / kTsSlots][r % kTsSlots];
         if (tok < 0 || l >= p.m / 4) continue;
         float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
         for (int w = 0; w < 32; ++w)
-            if (warps >> w & 1u) v = add4(v, rows[w * 2 * N * 32 + i]);
-        red_add4((float4*)((r < N ? p.gP : p.gC) + (size_t)tok * p.m) + l, v);
+            if (warps >> w & 1u) v = add4(v, rows[w * 2 * kTsSlots * 32 + i]);
+        red_add4((float4*)((r < kTsSlots ? p.gP : p.gC) + (size_t)tok * p.m) + l, v);
     }
 }
 // The i-th of kTsThreads tokens spread evenly over the references to a table (0: P, 1: C), or -1; every CTA has a sample of its own,
@@ -574,13 +570,14 @@ __device__ __forceinline__ void train_finish(const TrainParams& p, TrainSums& s,
     }
 }
 
-// HOT: additions to one row follow one another in L2, and what is behind them waits too, so that the most frequent tokens' rows are
-// summed up per warp in shared memory: those with a 24th of a sample of 384 references or more, four a table at most (a 16th:
-// 1,750 groups 36 us instead of 28.6 with tokens by a power of 1.1; eight slots: 1 us more, of L1).  Captured, K = 32, without and with,
-// us: 1,100 groups by a power of 1.1 23.6 and 23.0, 1.6 40.9 and 22.9; 2,000 by 1.1 39.6 and 31.6, 1.6 71.7 and 29.1, 2.5 103 and
-// 30.6, spread nearly evenly (0.5) 24.9 and 26.7.
+// HOT: additions to one row follow one another in L2, and what is behind them waits too; and each is rounded.  So the most frequent
+// tokens' rows are summed up per warp in shared memory: those with a 48th of a sample of 384 references or more, eight a table at most.
+// Captured, K = 32, without and with, us: 1,100 groups by a power of 1.1 of the tokens' rank 23.8 and 25.2, by 1.6 40.9 and 24.2; 2,000 by
+// 1.1 39.2 and 33.3, by 1.6 70.7 and 31.1, by 2.5 103 and 31.4, spread nearly evenly (0.5) 25.9 and 28.1.  Error against 64 bits, root mean
+// square, 2,000 by 1.1: gP 1.1e-6 and 2.3e-7, gC 7.0e-7 and 3.0e-7 (four slots and a 24th: 2.9e-7 and 4.1e-7, 1 to 3 us less).
 constexpr int kTsHashBits = 9, kTsHash = 1 << kTsHashBits;
-constexpr int kTsLeast = kTsThreads / 24;
+constexpr int kTsLeast = kTsThreads / 48;
+constexpr int kTsPicked = 256;  // s_ready: a picked table, and its slots
 constexpr int kTsTries = 4096;  // looks for the picked tokens before a warp does without
 
 // KC: children held in registers, a multiple of 8 (K <= KC).  HOT: frequent tokens, found in a sample of the references, have their
@@ -599,8 +596,8 @@ __global__ void __launch_bounds__(kTsThreads, 1) tdes_loss_rows_kernel(const Tra
     c.u = smem_f;
     c.gu_shared = p.gu_copies == 1;
     c.gu = s_gu + (c.gu_shared ? 0 : (size_t)warp * Lm);
-    float4* s_rows = (float4*)(s_gu + (size_t)Lm * p.gu_copies);  // HOT: [kTsWarps][2][kTsFew][32] sums of the frequent tokens' rows
-    c.hot = s_rows + (size_t)warp * 2 * kTsFew * 32;
+    float4* s_rows = (float4*)(s_gu + (size_t)Lm * p.gu_copies);  // HOT: [kTsWarps][2][kTsSlots][32] sums of the frequent tokens' rows
+    c.hot = s_rows + (size_t)warp * 2 * kTsSlots * 32;
     c.on = lane < p.m / 4;
     c.lane = lane;
     c.m = p.m;
@@ -615,14 +612,14 @@ __global__ void __launch_bounds__(kTsThreads, 1) tdes_loss_rows_kernel(const Tra
     }
     if (HOT) {
         for (int i = tid; i < 2 * kTsHash; i += kTsThreads) s_cnt[i] = 0;
-        if (tid < 2 * kTsFew) s_hot.tok[tid / kTsFew][tid % kTsFew] = -1;
+        if (tid < 2 * kTsSlots) s_hot.tok[tid / kTsSlots][tid % kTsSlots] = -1;
         if (tid == 0) {
             s_ready = 0;
             s_used = 0u;
         }
     }
     __syncthreads();
-    // One warp picks the tokens from the sample while the others are on their way to their first additions, in front of which they
+    // A warp a table picks the tokens from the sample while the others are on their way to their first additions, in front of which they
     // look for them (everybody waiting here: 2.5 us a call instead of 1.5).
     bool seen = false, any = false;  // (uniform)
     if constexpr (HOT) {
@@ -631,41 +628,38 @@ __global__ void __launch_bounds__(kTsThreads, 1) tdes_loss_rows_kernel(const Tra
             s_tok[t * kTsThreads + tid] = mine[t];
             if (mine[t] >= 0) atomicAdd(&s_cnt[t * kTsHash + tok_hash(mine[t], kTsHashBits)], 1);
         }
-        if (warp == 0) {
+        if (warp < 2) {
+            const int t = warp;
             named_bar_sync(1, kTsThreads);
-            int slots = 0;
-            for (int t = 0; t < 2; ++t)
-                for (int n = 0, slot = 0; n < 2 * kTsFew && slot < kTsFew; ++n) {  // the largest counter first
-                    int best = 0;
-                    for (int i = lane; i < kTsHash; i += 32) best = max(best, s_cnt[t * kTsHash + i] << kTsHashBits | i);
-                    best = __reduce_max_sync(0xFFFFFFFFu, best);
-                    if (best >> kTsHashBits < kTsLeast) break;
-                    best &= kTsHash - 1;
-                    // its token: what a lane meets most often, if that is enough by itself (the last one counted instead: a CTA in ten without
-                    // the most frequent child, 55 us instead of 30)
-                    int tok = -1, votes = 0, count = 0;
-                    for (int i = lane; i < kTsThreads; i += 32) {
-                        const int x = s_tok[t * kTsThreads + i];
-                        if (x < 0 || tok_hash(x, kTsHashBits) != best) continue;
-                        if (votes == 0) tok = x;
-                        votes += x == tok ? 1 : -1;
-                    }
-                    tok = __shfl_sync(0xFFFFFFFFu, tok, __reduce_max_sync(0xFFFFFFFFu, votes << 5 | lane) & 31);
-                    for (int i = lane; i < kTsThreads; i += 32) count += s_tok[t * kTsThreads + i] == tok ? 1 : 0;
-                    count = __reduce_add_sync(0xFFFFFFFFu, count);
-                    if (lane == 0) {
-                        s_cnt[t * kTsHash + best] = 0;
-                        if (count >= kTsLeast) s_hot.tok[t][slot] = tok;
-                    }
-                    if (count >= kTsLeast) {
-                        ++slot;
-                        ++slots;
-                    }
-                    __syncwarp();
+            int slot = 0;
+            for (int n = 0; n < 2 * kTsSlots && slot < kTsSlots; ++n) {  // the largest counter first
+                int best = 0;
+                for (int i = lane; i < kTsHash; i += 32) best = max(best, s_cnt[t * kTsHash + i] << kTsHashBits | i);
+                best = __reduce_max_sync(0xFFFFFFFFu, best);
+                if (best >> kTsHashBits < kTsLeast) break;
+                best &= kTsHash - 1;
+                // its token: what a lane meets most often, if that is enough by itself (the last one counted instead: a CTA in ten without
+                // the most frequent child, 55 us instead of 30)
+                int tok = -1, votes = 0, count = 0;
+                for (int i = lane; i < kTsThreads; i += 32) {
+                    const int x = s_tok[t * kTsThreads + i];
+                    if (x < 0 || tok_hash(x, kTsHashBits) != best) continue;
+                    if (votes == 0) tok = x;
+                    votes += x == tok ? 1 : -1;
                 }
+                tok = __shfl_sync(0xFFFFFFFFu, tok, __reduce_max_sync(0xFFFFFFFFu, votes << 5 | lane) & 31);
+                for (int i = lane; i < kTsThreads; i += 32) count += s_tok[t * kTsThreads + i] == tok ? 1 : 0;
+                count = __reduce_add_sync(0xFFFFFFFFu, count);
+                if (lane == 0) {
+                    s_cnt[t * kTsHash + best] = 0;
+                    if (count >= kTsLeast) s_hot.tok[t][slot] = tok;
+                }
+                slot += count >= kTsLeast ? 1 : 0;
+                __syncwarp();
+            }
             __threadfence_block();
             __syncwarp();
-            if (lane == 0) *(volatile int*)&s_ready = 1 + slots;
+            if (lane == 0) atomicAdd(&s_ready, kTsPicked + slot);
         } else {
             named_bar_arrive(1, kTsThreads);
         }
@@ -673,18 +667,18 @@ __global__ void __launch_bounds__(kTsThreads, 1) tdes_loss_rows_kernel(const Tra
     const auto look = [&] {
         if (!HOT || seen) return;
         int ready = 0;
-        for (int i = 0; i < kTsTries && ready == 0; ++i) ready = __shfl_sync(0xFFFFFFFFu, *(volatile int*)&s_ready, 0);
-        if (ready == 0) return;
+        for (int i = 0; i < kTsTries && ready < 2 * kTsPicked; ++i) ready = __shfl_sync(0xFFFFFFFFu, *(volatile int*)&s_ready, 0);
+        if (ready < 2 * kTsPicked) return;
         __threadfence_block();
         seen = true;
-        any = ready > 1;
+        any = ready > 2 * kTsPicked;
         if (!any) return;
-        for (int r = 0; r < 2 * kTsFew; ++r)
-            if (s_hot.tok[r / kTsFew][r % kTsFew] >= 0) c.hot[r * 32 + lane] = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int r = 0; r < 2 * kTsSlots; ++r)
+            if (s_hot.tok[r / kTsSlots][r % kTsSlots] >= 0) c.hot[r * 32 + lane] = make_float4(0.f, 0.f, 0.f, 0.f);
         if (lane == 0) atomicOr(&s_used, 1u << warp);
     };
     const auto slot_at = [&](int slot, int from) { return any ? __shfl_sync(0xFFFFFFFFu, slot, from) : -1; };
-    const auto slot_of = [&](int t, int tok) { return any ? hot_slot<kTsFew>(s_hot, t, tok) : -1; };
+    const auto slot_of = [&](int t, int tok) { return any ? hot_slot(s_hot, t, tok) : -1; };
     const int wid = blockIdx.x * kTsWarps + warp, nw = gridDim.x * kTsWarps;
     const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
     double l_kl = 0.0, l_pair = 0.0, l_bce = 0.0;  // per lane; summed at the end
@@ -759,9 +753,9 @@ __global__ void __launch_bounds__(kTsThreads, 1) tdes_loss_rows_kernel(const Tra
         }
         for (uint32_t left = hots; left != 0u; left &= left - 1u) {  // (uniform)
             const int i = __ffs(left) - 1;
-            smem_add4(c.hot + (kTsFew + __shfl_sync(0xFFFFFFFFu, slot, i)) * 32 + lane, mul4(__shfl_sync(0xFFFFFFFFu, coef, i), a));
+            smem_add4(c.hot + (kTsSlots + __shfl_sync(0xFFFFFFFFu, slot, i)) * 32 + lane, mul4(__shfl_sync(0xFFFFFFFFu, coef, i), a));
         }
-        ctx_add_row<FULL, kTsFew>(p, c, 0, tp, slot_of(0, tp), acc);
+        ctx_add_row<FULL>(p, c, 0, tp, slot_of(0, tp), acc);
         ctx_add_u<FULL>(c, d, acc);
     }
     // ---- pairwise level (Eq. 10): blocks of eight pairs, four at a time; lanes 0-7 hold the block's ids
@@ -829,16 +823,16 @@ __global__ void __launch_bounds__(kTsThreads, 1) tdes_loss_rows_kernel(const Tra
                 const int p2 = __shfl_sync(0xFFFFFFFFu, id[3], s), c2 = __shfl_sync(0xFFFFFFFFu, id[4], s), d2 = __shfl_sync(0xFFFFFFFFu, id[5], s);
                 const int h1 = slot_at(sp1, s), h2 = slot_at(sc1, s);
                 if (p1 == p2) {  // (uniform; an alternative keeps the pair's parent or its child: one addition for both)
-                    ctx_add_row<FULL, kTsFew>(p, c, 0, p1, h1, mul4(cf, sub4(b2[i], b1[i])));
+                    ctx_add_row<FULL>(p, c, 0, p1, h1, mul4(cf, sub4(b2[i], b1[i])));
                 } else {
-                    ctx_add_row<FULL, kTsFew>(p, c, 0, p1, h1, mul4(-cf, b1[i]));
-                    ctx_add_row<FULL, kTsFew>(p, c, 0, p2, slot_at(sp2, s), mul4(cf, b2[i]));
+                    ctx_add_row<FULL>(p, c, 0, p1, h1, mul4(-cf, b1[i]));
+                    ctx_add_row<FULL>(p, c, 0, p2, slot_at(sp2, s), mul4(cf, b2[i]));
                 }
                 if (c1 == c2) {
-                    ctx_add_row<FULL, kTsFew>(p, c, 1, c1, h2, mul4(cf, sub4(a2[i], a1[i])));
+                    ctx_add_row<FULL>(p, c, 1, c1, h2, mul4(cf, sub4(a2[i], a1[i])));
                 } else {
-                    ctx_add_row<FULL, kTsFew>(p, c, 1, c1, h2, mul4(-cf, a1[i]));
-                    ctx_add_row<FULL, kTsFew>(p, c, 1, c2, slot_at(sc2, s), mul4(cf, a2[i]));
+                    ctx_add_row<FULL>(p, c, 1, c1, h2, mul4(-cf, a1[i]));
+                    ctx_add_row<FULL>(p, c, 1, c2, slot_at(sc2, s), mul4(cf, a2[i]));
                 }
                 const float4 s1 = add4(a1[i], b1[i]), s2 = add4(a2[i], b2[i]);
                 if (d1 == d2) {
@@ -896,8 +890,8 @@ __global__ void __launch_bounds__(kTsThreads, 1) tdes_loss_rows_kernel(const Tra
         for (int i = 0; i < 8; ++i) {
             if (!((oks >> i) & 1u)) continue;  // (uniform)
             const float cf = __shfl_sync(0xFFFFFFFFu, coef, 4 * i);
-            ctx_add_row<FULL, kTsFew>(p, c, 0, __shfl_sync(0xFFFFFFFFu, tp, i), slot_at(sp, i), mul4(cf, b[i]));
-            ctx_add_row<FULL, kTsFew>(p, c, 1, __shfl_sync(0xFFFFFFFFu, tc, i), slot_at(sc, i), mul4(cf, a[i]));
+            ctx_add_row<FULL>(p, c, 0, __shfl_sync(0xFFFFFFFFu, tp, i), slot_at(sp, i), mul4(cf, b[i]));
+            ctx_add_row<FULL>(p, c, 1, __shfl_sync(0xFFFFFFFFu, tc, i), slot_at(sc, i), mul4(cf, a[i]));
             ctx_add_u<FULL>(c, __shfl_sync(0xFFFFFFFFu, d, i), mul4(cf, add4(a[i], b[i])));
         }
     }
@@ -912,7 +906,7 @@ __global__ void __launch_bounds__(kTsThreads, 1) tdes_loss_rows_kernel(const Tra
             for (int w = 1; w < p.gu_copies; ++w) v = add4(v, q[(size_t)w * (Lm / 4)]);
             if (v.x != 0.f || v.y != 0.f || v.z != 0.f || v.w != 0.f) red_add4((float4*)p.gu + i, v);
         }
-    if (HOT) flush_hot<kTsFew>(p, s_hot, s_rows, s_used, tid, kTsThreads);
+    if (HOT) flush_hot(p, s_hot, s_rows, s_used, tid, kTsThreads);
     train_finish(p, s_sum, l_kl, l_pair, l_bce, gs, skipped, lane);
 }
 
@@ -1364,7 +1358,7 @@ __global__ void __launch_bounds__(kTeThreads, 1) tdes_items_kernel(const TrainPa
             __syncthreads();
         if (grad && bt == 0)
             for (int i = tid; i < kTeWarps * 2 * kTsSlots * 32; i += kTeThreads) s_rows[i] = zero4;
-        const auto slot_of = [&](int t, int tok) { return grad ? hot_slot<kTsSlots>(s_hot, t, tok) + 1 : 0; };  // 0: none
+        const auto slot_of = [&](int t, int tok) { return grad ? hot_slot(s_hot, t, tok) + 1 : 0; };  // 0: none
 #pragma unroll
         for (int k = 0; k < 2; ++k)
             if (e_ok[k])
@@ -1424,8 +1418,8 @@ __global__ void __launch_bounds__(kTeThreads, 1) tdes_items_kernel(const TrainPa
                         if (q >= cnt) break;  // (uniform)
                         const float cf = __shfl_sync(0xFFFFFFFFu, coef, 4 * q);
                         const int4 e = s_edge[i + q];
-                        ctx_add_row<FULL, kTsSlots>(p, c, 0, e.x, (e.w & 15) - 1, mul4(cf, b[q]));
-                        ctx_add_row<FULL, kTsSlots>(p, c, 1, e.y, (e.w >> 4) - 1, mul4(cf, a[q]));
+                        ctx_add_row<FULL>(p, c, 0, e.x, (e.w & 15) - 1, mul4(cf, b[q]));
+                        ctx_add_row<FULL>(p, c, 1, e.y, (e.w >> 4) - 1, mul4(cf, a[q]));
                         gu = fma4(cf, add4(a[q], b[q]), gu);
                     }
                 }
@@ -1493,16 +1487,16 @@ __global__ void __launch_bounds__(kTeThreads, 1) tdes_items_kernel(const TrainPa
                         const int info = s_pinfo[i + q];
                         const int h1 = (info >> 8 & 15) - 1, h2 = (info >> 12 & 15) - 1, h3 = (info >> 16 & 15) - 1, h4 = (info >> 20 & 15) - 1;
                         if (e.x == e.z) {  // (uniform; an alternative keeps the pair's parent or its child: one addition for both)
-                            ctx_add_row<FULL, kTsSlots>(p, c, 0, e.x, h1, mul4(cf, sub4(b2[q], b1[q])));
+                            ctx_add_row<FULL>(p, c, 0, e.x, h1, mul4(cf, sub4(b2[q], b1[q])));
                         } else {
-                            ctx_add_row<FULL, kTsSlots>(p, c, 0, e.x, h1, mul4(-cf, b1[q]));
-                            ctx_add_row<FULL, kTsSlots>(p, c, 0, e.z, h3, mul4(cf, b2[q]));
+                            ctx_add_row<FULL>(p, c, 0, e.x, h1, mul4(-cf, b1[q]));
+                            ctx_add_row<FULL>(p, c, 0, e.z, h3, mul4(cf, b2[q]));
                         }
                         if (e.y == e.w) {
-                            ctx_add_row<FULL, kTsSlots>(p, c, 1, e.y, h2, mul4(cf, sub4(a2[q], a1[q])));
+                            ctx_add_row<FULL>(p, c, 1, e.y, h2, mul4(cf, sub4(a2[q], a1[q])));
                         } else {
-                            ctx_add_row<FULL, kTsSlots>(p, c, 1, e.y, h2, mul4(-cf, a1[q]));
-                            ctx_add_row<FULL, kTsSlots>(p, c, 1, e.w, h4, mul4(cf, a2[q]));
+                            ctx_add_row<FULL>(p, c, 1, e.y, h2, mul4(-cf, a1[q]));
+                            ctx_add_row<FULL>(p, c, 1, e.w, h4, mul4(cf, a2[q]));
                         }
                         const float4 s1 = add4(a1[q], b1[q]), s2 = add4(a2[q], b2[q]);
                         if ((info & 255) == d) {
@@ -1521,7 +1515,7 @@ __global__ void __launch_bounds__(kTeThreads, 1) tdes_items_kernel(const TrainPa
     }
     if (grad && n_batch > 0) {
         for (int i = tid; i < Lm / 4; i += kTeThreads) red_add4((float4*)p.gu + i, ((const float4*)s_gu)[i]);
-        flush_hot<kTsSlots>(p, s_hot, s_rows, (1u << kTeWarps) - 1, tid, kTeThreads);
+        flush_hot(p, s_hot, s_rows, (1u << kTeWarps) - 1, tid, kTeThreads);
     }
     train_finish(p, s_sum, 0.0, l_pair, l_bce, gs, skipped, lane);
     pdl_wait();  // (the end of this kernel stands for the end of both)
@@ -1537,7 +1531,7 @@ static size_t tdes_loss_smem(const graft_config& cfg) {
     if (cfg.m > 128) return lm * sizeof(float);  // gu
     return lm * (1 + rows_gu_copies(cfg)) * sizeof(float);
 }
-static size_t rows_hot_smem(const graft_config& cfg) { return tdes_loss_smem(cfg) + (size_t)kTsWarps * 2 * kTsFew * 512; }
+static size_t rows_hot_smem(const graft_config& cfg) { return tdes_loss_smem(cfg) + (size_t)kTsWarps * 2 * kTsSlots * 512; }
 template <bool HOT>
 static void (*rows_kernel(const graft_config& cfg))(const TrainParams) {
     if (cfg.m == 128) return cfg.K <= 8 ? tdes_loss_rows_kernel<8, true, HOT> : (cfg.K <= 16 ? tdes_loss_rows_kernel<16, true, HOT> : tdes_loss_rows_kernel<32, true, HOT>);

@@ -253,6 +253,33 @@ def test_full_size_tables():
     g.destroy()
 
 
+def _errors(n, seeds=3):
+    """Root mean square errors of gP, gC, gu and gs against 64 bits, over the results' size, on tokens by a power of 1.1 of their rank."""
+    V, L, K, m = 30000, 16, 32, 128
+    err = np.zeros(4)
+    for seed in range(seeds):
+        g, P, Ct, u, s, keep = _ctx(V, L, K, m, seed=70 + seed)
+        rng = np.random.default_rng(n + seed)
+        cdf = np.cumsum(np.arange(1, V + 1) ** -1.1)
+        tok = lambda *k: np.searchsorted(cdf, cdf[-1] * rng.random(k)).clip(max=V - 1).astype(np.int32)  # noqa: E731
+        dep = lambda k: rng.integers(1, L + 1, k, dtype=np.int32)  # noqa: E731
+        groups = dict(parent=tok(n), depth=dep(n), child=tok(n, K), logq=-rng.random((n, K), dtype=np.float32),
+                      ztgt=2 * rng.standard_normal((n, K), dtype=np.float32))
+        tr = dict(groups=groups, pairs=np.stack([f(4 * n) for f in (tok, tok, dep, tok, tok, dep)], 1),
+                  edges=np.stack([tok(8 * n), tok(8 * n), dep(8 * n), (dep(8 * n) < 3).astype(np.int32)], 1))
+        got = _run(g, V, L, m, tr)
+        ref = oracle.tdes_loss(P, Ct, u, s, tr["groups"], tr["pairs"], tr["edges"], **CFG)
+        err += [np.linalg.norm(got[k].astype(np.float64) - ref[k]) / np.linalg.norm(ref[k]) for k in ("gP", "gC", "gu", "gs")]
+        g.destroy()
+    return err / seeds
+
+
+def test_rows_of_frequent_tokens_keep_their_precision():
+    """Thousands of additions to one row one by one would each be rounded at the row's size: 1e-6 of gP.  One a CTA is 148."""
+    gP, gC, _, _ = _errors(2000)
+    assert gP <= 4e-7 and gC <= 5e-7, (gP, gC)
+
+
 @pytest.mark.parametrize("ng,npair,ne,V", [(2000, 4000, 8000, 40), (9000, 9000, 9000, 3000), (30, 40, 50, 300)])
 def test_first_call_under_capture(ng, npair, ne, V):
     """Kernels that are loaded with the first call that wants them."""
