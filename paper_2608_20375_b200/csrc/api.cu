@@ -158,7 +158,7 @@ graft_status graft_create(const graft_config* cfg, graft_ctx** out) {
     const size_t o_id = take(B * L * K * 4), o_lp = take(B * L * K * 4), o_lse = take(B * L * 4);
     const size_t o_rs = take(B * L * 4), o_edge = take(B * L * K * K * 4);
     const size_t o_es = take(B * L * K * K * 4), o_ei = take(B * L * K * K);
-    const size_t o_u = take(L * (size_t)cfg->m * 4), o_err = take(256), o_cos = take(B * L * 8), o_saba = take(B * sizeof(SabaResult)), o_fit = take(saba_fit_doubles() * 8), o_loss = take(kLossSums * 8), o_order = take(B * 4), o_ordn = take(256);
+    const size_t o_u = take(L * (size_t)cfg->m * 4), o_err = take(256), o_cos = take(B * L * 8), o_saba = take(B * sizeof(SabaResult)), o_fit = take(saba_fit_doubles() * 8), o_loss = take(tdes_loss_bytes(*cfg)), o_order = take(B * 4), o_ordn = take(256);
     ctx->ws_bytes = off;
     if (cudaMalloc(&ctx->ws, ctx->ws_bytes) != cudaSuccess) {
         cudaGetLastError();

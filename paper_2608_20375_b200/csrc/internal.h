@@ -93,7 +93,7 @@ struct graft_ctx {
     int* w_order_n;               // [2] sequences placed in it from either end, zero between rounds
     double* w_fit;                // graft_saba_fit: table of logarithms, arrival counter and normal equations (both zero between calls)
     bool loss_hot, loss_many;     // graft_tdes_loss's kernels for frequent tokens and for many traces are ready
-    double* w_loss;               // [kLossSums] sums of graft_tdes_loss and its arrival counter, zero between calls
+    double* w_loss;               // graft_tdes_loss: [kLossSums] sums and arrival counter, then shares of gu; zero between calls
     int32_t* w_errflag;           // [1] device-side internal error flag
     graft::VpPlan vp_plan;
     // scratch of the tensor-core table precompute (allocated on its first use: pieces of split tiles, W's parts,
@@ -184,7 +184,8 @@ cudaError_t tdes_loss_launch(graft_ctx* ctx, const graft_tdes_traces* tr, const 
                              cudaStream_t st);
 cudaError_t tdes_loss_configure(const graft_config& cfg);
 bool tdes_loss_supported(const graft_config& cfg);
-constexpr int kLossSums = 8;                       // graft_ctx::w_loss
+constexpr int kLossSums = 8;
+size_t tdes_loss_bytes(const graft_config& cfg);   // graft_ctx::w_loss
 constexpr int kFitLog = 257;                        // entries of the fit's table of logarithms
 void saba_fit_table(double* table);                // [2 kFitLog], on the host
 size_t saba_fit_doubles();                         // graft_ctx::w_fit

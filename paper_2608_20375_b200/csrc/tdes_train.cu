@@ -55,10 +55,11 @@ struct TrainParams {
     float lam_kl, lam_pair, lam_bce;
     double* loss;      // [4], zero at launch
     int32_t* skipped;  // [1] or NULL, zero at launch
-    double* acc;       // m <= 128: [5] loss sums, skipped items, arrival counter; zero between calls
+    double* acc;       // m <= 128: [6] loss sums, skipped items, arrival counter, gradient of the scale; zero between calls
     int gu_copies;     // m <= 128: copies of gu in shared memory: one per warp, or one
     int g_batch;       // m <= 128: groups of a batch
     int ctas;          // m <= 128: CTAs of the call, that arrive at acc
+    float* gu_parts;   // [kTgParts][L][m] or NULL: where the groups' kernel adds its share of gu, for the items' to collect; zero between calls
     float* gP;
     float* gC;
     float* gu;
@@ -553,10 +554,15 @@ __device__ __forceinline__ void train_finish(const TrainParams& p, TrainSums& s,
         atomicAdd(p.acc + 1, s.loss[1]);
         atomicAdd(p.acc + 2, s.loss[2]);
         if (s.skip) atomicAdd((int*)(p.acc + 3), s.skip);
-        if (p.gP != nullptr && s.gs != 0.f) atomicAdd(p.gs, s.gs);
+        if (p.gu_parts != nullptr)  // (two kernels' CTAs: twice as many roundings, unless in 64 bits)
+            atomicAdd(p.acc + 5, (double)s.gs);
+        else if (p.gP != nullptr && s.gs != 0.f)
+            atomicAdd(p.gs, s.gs);
         __threadfence();
         if (atomicAdd((unsigned int*)(p.acc + 4), 1u) == (unsigned)p.ctas - 1) {
             __threadfence();
+            const double scale = p.gu_parts != nullptr ? __ldcg(p.acc + 5) : 0.0;
+            const int skipped_all = __ldcg((const int*)(p.acc + 3));
             const double kl = __ldcg(p.acc + 0) / (double)(p.n_groups > 0 ? p.n_groups : 1);
             const double pr = __ldcg(p.acc + 1) / (double)(p.n_pairs > 0 ? p.n_pairs : 1);
             const double bc = __ldcg(p.acc + 2) / (double)(p.n_edges > 0 ? p.n_edges : 1);
@@ -564,8 +570,9 @@ __device__ __forceinline__ void train_finish(const TrainParams& p, TrainSums& s,
             p.loss[1] = pr;
             p.loss[2] = bc;
             p.loss[3] = (double)p.lam_kl * kl + (double)p.lam_pair * pr + (double)p.lam_bce * bc;
-            if (p.skipped) *p.skipped = __ldcg((const int*)(p.acc + 3));
-            for (int i = 0; i < 5; ++i) p.acc[i] = 0.0;
+            if (p.skipped) *p.skipped = skipped_all;
+            if (p.gu_parts != nullptr) atomicAdd(p.gs, (float)scale);
+            for (int i = 0; i < 6; ++i) p.acc[i] = 0.0;
         }
     }
 }
@@ -930,6 +937,10 @@ __global__ void __launch_bounds__(kTsThreads, 1) tdes_loss_rows_kernel(const Tra
 // a running softmax (163 - 167 against 150: the longer chain of a group costs what the second read does).
 constexpr int kTgGroups = 224;  // groups of a batch at most
 constexpr int kTgThreads = 768;
+// Sums of gu over the grid are rounded with every CTA's addition, and two kernels have twice as many CTAs: with the groups' adding
+// to four places by turns the error against 64 bits is that of one kernel (root mean square, before two kernels / two / so: 4,000
+// groups 1.82e-7 / 2.10e-7 / 1.76e-7, 32,768 1.85e-7 / 1.98e-7 / 1.83e-7).  Collecting them, and gs in 64 bits (2.4e-7 and 2e-8), are 0.4 us of 41 to 250.
+constexpr int kTgParts = 4;
 constexpr int kTgBinBits = 13, kTgBins = 1 << kTgBinBits;
 constexpr int kTeThreads = 512;
 constexpr int kTeWarps = kTeThreads / 32;
@@ -1227,7 +1238,8 @@ __global__ void __launch_bounds__(kTgThreads, 1) tdes_groups_kernel(const TrainP
     }
     if (grad) {
         __syncthreads();
-        for (int i = tid; i < Lm / 4; i += kTgThreads) red_add4((float4*)p.gu + i, ((const float4*)s_gu)[i]);
+        float4* gu = p.gu_parts != nullptr ? (float4*)p.gu_parts + (int)(blockIdx.x % kTgParts) * (Lm / 4) : (float4*)p.gu;
+        for (int i = tid; i < Lm / 4; i += kTgThreads) red_add4(gu + i, ((const float4*)s_gu)[i]);
     }
     __syncthreads();
     train_finish(p, s_sum, l_kl, 0.0, 0.0, gs, skipped, lane);
@@ -1513,14 +1525,30 @@ __global__ void __launch_bounds__(kTeThreads, 1) tdes_items_kernel(const TrainPa
         }
         __syncthreads();
     }
+    const int n4 = Lm / 4, col = (int)blockIdx.x + tid * (int)gridDim.x;
     if (grad && n_batch > 0) {
-        for (int i = tid; i < Lm / 4; i += kTeThreads) red_add4((float4*)p.gu + i, ((const float4*)s_gu)[i]);
+        for (int i = tid; i < n4; i += kTeThreads) red_add4((float4*)p.gu + i, ((const float4*)s_gu)[i]);
         flush_hot(p, s_hot, s_rows, (1u << kTeWarps) - 1, tid, kTeThreads);
     }
-    train_finish(p, s_sum, 0.0, l_pair, l_bce, gs, skipped, lane);
     pdl_wait();  // (the end of this kernel stands for the end of both)
+    // the groups' share of gu, a few columns a CTA: on its way while the losses are finished
+    const bool collect = grad && p.gu_parts != nullptr && col < n4;
+    float4 share[kTgParts];
+    if (collect) {
+#pragma unroll
+        for (int k = 0; k < kTgParts; ++k) share[k] = __ldcg((const float4*)p.gu_parts + k * n4 + col);
+    }
+    train_finish(p, s_sum, 0.0, l_pair, l_bce, gs, skipped, lane);
+    if (collect) {
+#pragma unroll
+        for (int k = 0; k < kTgParts; ++k) ((float4*)p.gu_parts)[k * n4 + col] = zero4;
+#pragma unroll
+        for (int k = kTgParts / 2; k >= 1; k /= 2)
+#pragma unroll
+            for (int q = 0; q < k; ++q) share[q] = add4(share[q], share[q + k]);
+        red_add4((float4*)p.gu + col, share[0]);
+    }
 }
-
 
 }  // namespace
 
@@ -1555,6 +1583,9 @@ static size_t items_smem(const graft_config& cfg) {
     return (size_t)(kTeEdges + kTePairs) * sizeof(int4) + kTePairs * sizeof(int) + (size_t)kTeWarps * 2 * kTsSlots * 512 + 2 * (size_t)cfg.L * cfg.m * sizeof(float);
 }
 
+size_t tdes_loss_bytes(const graft_config& cfg) {
+    return kLossSums * sizeof(double) + (cfg.m <= 128 ? (size_t)kTgParts * cfg.L * cfg.m * sizeof(float) : 0);
+}
 cudaError_t tdes_loss_launch(graft_ctx* ctx, const graft_tdes_traces* tr, const graft_tdes_loss_config* lc,
                              double* d_loss, int32_t* d_skipped, float* d_gP, float* d_gC, float* d_gu, float* d_gs,
                              cudaStream_t st) {
@@ -1597,6 +1628,7 @@ cudaError_t tdes_loss_launch(graft_ctx* ctx, const graft_tdes_traces* tr, const 
     const size_t smem = tdes_loss_smem(cfg);
     if (cfg.m <= 128 && items > 0) {
         p.acc = ctx->w_loss;
+        p.gu_parts = nullptr;
         p.gu_copies = rows_gu_copies(cfg);
         // a warp takes a group, eight pairs or eight edges at a time
         const long long work = (long long)tr->n_groups + (tr->n_pairs + 7ll) / 8 + (tr->n_edges + 7ll) / 8;
@@ -1628,6 +1660,7 @@ cudaError_t tdes_loss_launch(graft_ctx* ctx, const graft_tdes_traces* tr, const 
         }
         const int n_g = tr->n_groups > 0 ? ctx->num_sms : 0, n_i = tr->n_pairs + tr->n_edges > 0 ? ctx->num_sms : 0;
         p.ctas = n_g + n_i;
+        p.gu_parts = d_gP && n_g > 0 && n_i > 0 ? (float*)(ctx->w_loss + kLossSums) : nullptr;
         p.g_batch = groups_batch(cfg);
         cudaError_t e = cudaSuccess;
         if (n_g > 0) {
@@ -1647,7 +1680,7 @@ cudaError_t tdes_loss_launch(graft_ctx* ctx, const graft_tdes_traces* tr, const 
         // (thread blocks of a kernel that did start have arrived at sums that the other's would have brought back to zero)
         if (e != cudaSuccess) {
             cudaGetLastError();
-            cudaMemsetAsync(ctx->w_loss, 0, kLossSums * sizeof(double), st);
+            cudaMemsetAsync(ctx->w_loss, 0, tdes_loss_bytes(cfg), st);
         }
         return e;
     }

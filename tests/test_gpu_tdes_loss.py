@@ -280,6 +280,12 @@ def test_rows_of_frequent_tokens_keep_their_precision():
     assert gP <= 4e-7 and gC <= 5e-7, (gP, gC)
 
 
+def test_scale_gradient_of_many_traces():
+    """The sums of two kernels' CTAs, added up in 64 bits."""
+    _, _, _, gs = _errors(4000, seeds=4)
+    assert gs <= 1e-7, gs
+
+
 @pytest.mark.parametrize("ng,npair,ne,V", [(2000, 4000, 8000, 40), (9000, 9000, 9000, 3000), (30, 40, 50, 300)])
 def test_first_call_under_capture(ng, npair, ne, V):
     """Kernels that are loaded with the first call that wants them."""
