@@ -123,9 +123,10 @@ graft_status graft_set_tdes_tables(graft_ctx* ctx, const float* d_P, const float
 
 /* How many depths the edge-score kernel covers ahead of the expansion.  The scores of Eq. 4-6 are needed only for
  * depths that the best-first expansion reaches, which is not known in advance: depths [0, rows) are scored for every
- * sequence by a kernel of their own, deeper ones inside the tree kernel when an expansion gets there.  The trees do
- * not depend on the split at all: both scorers run the same arithmetic in the same order, so a score has the same
- * bits whichever kernel produced it.
+ * sequence by a kernel of their own, deeper ones inside the tree kernel when an expansion gets there.  Sequences whose drafter is
+ * confident have all depths scored ahead; and until this function is called, large batches score as few as four ahead for
+ * sequences whose drafter is not.  The trees do not depend on the split at all: both scorers run the same arithmetic in the
+ * same order, so a score has the same bits whichever kernel produced it.
  * rows in [0, L]; the default is min(L, 8), or L when the on-demand scorer's buffers do not fit in shared memory
  * (then any other value is GRAFT_ERR_INVALID_ARG).  Host-only call; takes effect from the next round.
  * (A tuning knob of this implementation; the paper scores all edges.) */

@@ -277,6 +277,7 @@ graft_status graft_set_edge_rows(graft_ctx* ctx, int32_t rows) {
     if (!ctx || rows < 0 || rows > ctx->cfg.L) return GRAFT_ERR_INVALID_ARG;
     if (rows < ctx->cfg.L && !tree_lazy_fits(ctx->cfg)) return GRAFT_ERR_INVALID_ARG;
     ctx->edge_rows = rows;
+    ctx->edge_rows_set = true;
     return GRAFT_OK;
 }
 
@@ -421,8 +422,8 @@ graft_status graft_build_trees(graft_ctx* ctx, int32_t batch, const void* d_logi
                   nullptr, neutral ? VpUse::neutral_round : VpUse::round, st) != cudaSuccess)
         return GRAFT_ERR_CUDA;
     if (ev) cudaEventRecord(ev[1], st);
-    // Edge scores of Eq. 4-6: the kernel scores the depths [0, edge_rows) for every sequence (all depths when the
-    // caller asks for the score array); the tree kernel scores deeper rows itself if an expansion gets that far.
+    // Edge scores of Eq. 4-6: the kernel scores the depths [0, edge_rows) (all depths when the caller asks for the score
+    // array), or as many of a sequence's as its tree will look at (rows_ahead); the tree kernel scores deeper rows itself if an expansion gets that far.
     // The depth-0 CTA of each sequence in that kernel also works out the sequence's budget (Sec. 3.3), which the tree
     // kernel then only reads; without an edge-score kernel the tree kernel does it itself.
     // Without edge scores (beta = 0) nothing needs that kernel: the tree kernel lays the rows out from log q.

@@ -20,9 +20,11 @@ namespace graft {
 // candidates trees are narrower and deeper (5 to 8 depths even at 0.01), and a depth's scores are cheap: 8.
 // (In two steps, so that a caller can have the load in flight beside its other loads: lane d's top-1 log-probability
 // of position d, 0 for d >= L; then the decision, taken by every lane of a warp together.)
-// Fewer than `rows` of them only where the scores take more CTAs than the SMs hold at once (four each): in one wave nothing is gained,
-// and the decision stands in front of the work (batch 16, 64: 0.7 us of a round).
-inline int rows_ahead_least(int batch, int rows, int num_sms) { return rows > 4 && (long long)batch * rows > 4ll * num_sms ? 4 : rows; }
+// Fewer than `rows` of them only where the caller has not asked for a number, and the scores take more CTAs than the SMs hold at once
+// (four each): in one wave nothing is gained, and the decision stands in front of the work (batch 16, 64: 0.7 us of a round).
+inline int rows_ahead_least(int batch, int rows, bool asked, int num_sms) {
+    return !asked && rows > 4 && (long long)batch * rows > 4ll * num_sms ? 4 : rows;
+}
 __device__ __forceinline__ float rows_ahead_load(const float* __restrict__ topk_lp_seq, int L, int K) {
     const int lane = threadIdx.x & 31;
     return lane < L ? topk_lp_seq[(size_t)lane * K] : 0.f;

@@ -74,7 +74,9 @@ struct graft_ctx {
     int32_t* hist_window;  // [max_batch, hist_w]
     int32_t* hist_count;   // [max_batch]
     float* hist_out;       // [max_batch]
-    int edge_rows;  // depths [0, edge_rows) are scored by the edge-score kernel, deeper ones on demand in the tree kernel
+    int edge_rows;  // depths [0, edge_rows) are scored by the edge-score kernel, deeper ones on demand in the tree kernel; but for
+                    // what rows_ahead says of a sequence
+    bool edge_rows_set;  // graft_set_edge_rows asked for them
     // scratch (one allocation)
     void* ws;
     size_t ws_bytes;

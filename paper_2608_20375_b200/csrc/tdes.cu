@@ -282,7 +282,7 @@ cudaError_t tdes_edges_launch(graft_ctx* ctx, int batch, const int32_t* d_topk_i
     p.root_edge = cfg.root_edge;
     p.rows = rows;
     // (the tree kernel takes the same decision if it can score on demand and the budget comes from here)
-    p.rows_least = !d_edge && d_saba_out && d_row_status && rows < cfg.L ? rows_ahead_least(batch, rows, ctx->num_sms) : rows;
+    p.rows_least = !d_edge && d_saba_out && d_row_status && rows < cfg.L ? rows_ahead_least(batch, rows, ctx->edge_rows_set, ctx->num_sms) : rows;
     const int rows_all = d_edge || rows == cfg.L ? rows : cfg.L;  // (rows < L only when the tree kernel can score on demand)
     p.saba_out = d_row_status ? d_saba_out : nullptr;
     p.order = p.saba_out && tree_ordered(ctx, batch) ? ctx->w_order : nullptr;

@@ -29,7 +29,7 @@ struct TreeParams {
     // Edge scores (Eq. 4-6): the rows of depths [0, rows_pre) come from the edge-score kernel through esort / eidx;
     // deeper rows are scored inside this kernel (lazy = 1), level by level, only if the expansion gets there.
     int rows_pre;
-    int rows_least;     // of those at least
+    int rows_least;     // of those at least: for every sequence
     const int32_t* order;  // [batch] which sequence's tree a CTA builds (more sequences than SMs), or NULL: its own number's
     int* order_n;          // [2] cleared for the next round
     int rows_adaptive;  // the edge-score kernel scored as many depths of a sequence as its tree will look at (rows_ahead)
@@ -721,7 +721,7 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
     // the sorted edge rows of this sequence: bulk copies through the TMA unit when the 16-byte rules allow it
     // (they land while warp 0 works out the budget), plain loads otherwise
     const int rows_pre = TIES ? L : p.rows_pre;
-    const int ne = rows_pre * K * K;  // entries that come from the edge-score kernel for every sequence
+    const int ne = rows_pre * K * K;  // entries that come from the edge-score kernel (what it left out is copied too, and not read)
     // (a bulk copy's source and size are multiples of 16 bytes: the child ranks are bytes, so the entries copied and the
     // entries between two sequences both have to be multiples of 16 -- L = 11, K = 10 with 8 rows ahead has 800 and 1100)
     const bool bulk = !TIES && ne > 0 && (ne % 16) == 0 && (L * K * K) % 16 == 0;
@@ -1213,8 +1213,10 @@ __global__ void __launch_bounds__(NT) tree_kernel(const TreeParams p) {
             n_grow = b1 - b0 <= NT && lv1 - lv0 <= NT ? grown : NT + 1;  // (a thread appended one node of the level at most)
             // theta only has to be a lower bound of its final value while the levels are built (it prunes), so
             // the exact B-th largest key is recomputed only when the table has grown noticeably, by a quarter -- by a sixteenth
-            // in front of the first row that is not scored ahead: scoring it costs four searches, and a tighter threshold
-            // often ends the tree there (a batch of 64 with mixed confidence: 6 % of the round)
+            // in front of row rows_pre: scoring a row on demand costs four searches, and a tighter threshold often ends the tree
+            // there (a batch of 64 with mixed confidence: 6 % of the round).  Where fewer rows are scored ahead than that
+            // (rows_ahead), a search in front of the first of the others gains and loses as often: budgets to 512 up to 1 % of
+            // the round, budgets to 64 minus 0.4 to 2 % at batch 256.
             if (ntot - 1 >= budget &&
                 (theta == 0u || ntot - n_at_select >= (!TIES && d + 1 == rows_pre ? ntot / 16 : ntot / 4))) {
                 sel_top = 0.0f + sm.es[0];  // the root's best child
@@ -1848,7 +1850,7 @@ cudaError_t tree_launch(graft_ctx* ctx, int batch, const int32_t* d_topk_id, con
     p.beta = ctx->tdes_set ? cfg.beta : 0.0f;
     const bool neutral = p.beta == 0.0f;  // (the candidates are staged whenever there is room; no row is scored)
     p.lazy = neutral ? tree_lazy_fits(cfg) : p.rows_pre < cfg.L ? 1 : 0;  // (only possible when tree_lazy_fits)
-    p.rows_least = rows_ahead_least(batch, p.rows_pre, ctx->num_sms);
+    p.rows_least = rows_ahead_least(batch, p.rows_pre, ctx->edge_rows_set || out->d_edge, ctx->num_sms);  // (d_edge: every row is scored)
     p.rows_adaptive = (p.lazy && p.rows_pre > 0 && d_saba_pre != nullptr) ? 1 : 0;
     p.lazy_m = tree_lazy_fits(cfg) ? cfg.m : 0;
     p.ncap = tree_node_cap(cfg.L, cfg.K, ctx->nmax, p.lazy_m);

@@ -313,3 +313,38 @@ def test_large_batches_build_the_trees_of_small_ones(K, m, fixed):
             assert np.array_equal(got[k], w[lo:hi]), (k, lo, hi)
     big.destroy()
     small.destroy()
+
+
+@pytest.mark.parametrize("K,m,L", [(32, 128, 12), (16, 64, 16), (9, 32, 7)])
+def test_large_batches_with_any_number_of_depths_scored_ahead(K, m, L):
+    """Asked for a number of depths, or for the score array, large batches build the same trees as when they choose for themselves."""
+    from paper_2608_20375_b200 import Graft
+    V, n = 2000, 170
+    gen = torch.Generator(device="cuda").manual_seed(K + L)
+    rand = lambda *s: torch.randn(s, generator=gen, device="cuda")  # noqa: E731
+    height = 16.0 * torch.rand((n, 1, 1), generator=gen, device="cuda")
+    rank = torch.rand((n, L, V), generator=gen, device="cuda").argsort(2).float()
+    logits = (2.0 * rand(n, L, V) + height / (1.0 + rank)).to(torch.bfloat16)
+    P, Ct, u = rand(V, m), rand(V, m), 0.5 * rand(L, m)
+    root = torch.randint(0, V, (n,), generator=gen, device="cuda", dtype=torch.int32)
+    prefix = torch.full_like(root, 200)
+    budget = torch.randint(1, 250, (n,), generator=gen, device="cuda", dtype=torch.int32)
+    g = Graft(V, L, K, m, 64, n, 16, 256, 16, 0.2, 1)
+    g.set_tdes_tables(P, Ct, u, 1.0)
+
+    def build(debug=False):
+        o = g.alloc_out(n, debug=debug)
+        g.build_trees(logits, None, root, None, prefix, budget, o)
+        torch.cuda.synchronize()
+        return o.cpu()
+
+    want = build()
+    with_edges = build(debug=True)
+    for rows in (0, 3, 5, 7, 12, L):
+        g.set_edge_rows(min(rows, L))
+        for got in (build(), build(debug=True)):
+            for k, w in want.items():
+                assert np.array_equal(got[k], w), (k, rows)
+            if "edge" in got:
+                assert np.array_equal(got["edge"], with_edges["edge"])
+    g.destroy()
