@@ -14,10 +14,11 @@ namespace graft {
 // tree that needs the edge scores of many depths; an uncertain one a shallow, wide tree that stops a few levels down.  The
 // edge-score kernel scores that many depths ahead of the tree kernel, which takes the same decision from the same numbers
 // and scores what is missing on demand (3 - 4 us a depth in front of everything else, so the bounds err on the side of more).  A
-// matter of speed only: a row has the same bits whoever scores it.  By the mean top-1 probability of the block, of 2,500
-// sequences of the configured workloads (budgets 16 to 512, L = 12 and 16, K > 8): below 0.02 at most 4 depths, below 0.03 5,
-// below 0.06 6, below 0.1 7 (all but one in two hundred); below 0.2 8 (all but one in forty), above it up to 12.  With 8 or fewer
-// candidates trees are narrower and deeper (5 to 8 depths even at 0.01), and a depth's scores are cheap: 8.
+// matter of speed only: a row has the same bits whoever scores it.  By the mean top-1 probability of the block: below 0.02 4
+// depths, below 0.03 5, below 0.06 6, below 0.1 7, below 0.2 8, from there on all.  Of 12,288 sequences (boosts of 12 and of 6 to 14, V = 32,000
+// and 151,936, L = 12 and 16, K = 16 and 32, budgets to 64, 256 and 512) twelve looked at a depth more, nine of them with budgets to
+// 512; of any class of them at most one in a hundred.  With 8 or fewer candidates trees are narrower and deeper (5 to 8 depths even at
+// 0.01), and a depth's scores are cheap: 8.
 // (In two steps, so that a caller can have the load in flight beside its other loads: lane d's top-1 log-probability
 // of position d, 0 for d >= L; then the decision, taken by every lane of a warp together.)
 // Fewer than `rows` of them only where the caller has not asked for a number, and the scores take more CTAs than the SMs hold at once
@@ -157,8 +158,9 @@ __device__ __forceinline__ void edge_row_finish(const float* dots, float lp, flo
         float sum = ft;
 #pragma unroll
         for (int d = 16; d > 0; d >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, d);
-        // sum / K: the product with 1 / K (worked out once by the caller) and one correction step with the exact
-        // remainder, which gives the rounded quotient without the division's special-case code
+        // sum / K from 1 / K, which the caller has worked out once: a quotient from the rounded reciprocal, corrected by the remainder that
+        // a fused multiply-add gives exactly (P. Markstein, "Computation of elementary functions on the IBM RISC System/6000
+        // processor", 1990), is the rounded quotient
         const float q0 = sum * inv_K;
         const float mean = fmaf(fmaf(-q0, (float)K, sum), inv_K, q0);
         val = fmaf(beta, ft - mean, lp);

@@ -764,8 +764,7 @@ __global__ void __cluster_dims__(F32 ? 1 : 2, 1, 1) __launch_bounds__(TablesCfg<
         // ------------------------------ fp32 embeddings -> fp16 parts ----------------------------
         // four warps take the even blocks, four the odd ones: a block is a chain of waits and round trips.  A wait on a barrier's parity
         // tells a phase from the ones beside it and not from the one two before, so a half has to wait for every phase of the
-        // barriers that it waits on: with an even number of stages every stage is always the same half's.  (Four raw stages or six: V =
-        // 32,000, E = 2048, two towers 208.4 and 209.3 us.)
+        // barriers that it waits on: with an even number of stages every stage is always the same half's.
         static_assert(!F32 || (NR % 2 == 0 && NS % 2 == 0), "a stage of either ring belongs to one half of the converting warps");
         // A thread has a row: a warp reaches its quarter of TMEM's lanes (its index modulo four), and a half has all four.
         const int half = (warp - (kTmEpiWarps + 3)) >> 2, row = 32 * (warp & 3) + lane;
@@ -953,12 +952,13 @@ cudaError_t tables_run(const TablesParams& p, cudaStream_t st, int* launches) {
     if (e == cudaSuccess) e = launch_pdl(tables_mma_kernel<F32>, dim3((C::PAIR ? 2 : 1) * p.pairs), dim3(C::THREADS), C::SMEM, st, p);
     *launches += 1;
     if (e == cudaSuccess && p.share_pairs > p.left) {
-        // fp32: 32 rows a block where that leaves a block an SM or more, else 8 (102 tiles left, V = 32,000, E =
-        // 2048: 87.2 and 92.8 us; 56, V = 64,000, E = 1536: 122.1 and 124.6; 9, V = 20,000, E = 2048: 69.1 and 65.1)
+        // fp32: 32 rows a block where that leaves a block an SM or more, else 8 (E = 2048, 32 rows and 8: 102 tiles left, V = 32,000,
+        // 73.3 and 77.1 us; 71, V = 28,000, 64.7 and 66.9; 33, V = 42,000, 89.3 and 87.7; 9, V = 20,000, 59.0 and 52.3)
         constexpr int N = F32 ? 4 : 1;
         if (F32 ? p.left * (C::ROWS / (8 * N)) >= p.pairs : p.share_pairs < 6 * p.left)
             e = launch_pdl(tables_pieces_kernel<F32, N, F32 ? 3 : 8>, dim3(C::ROWS / (8 * N), p.left), dim3(256), 0, st, p);
-        else  // (few tiles left, many pieces each: bf16 with registers for eight pieces' loads, V = 151,936: 14 -> 8 us)
+        else  // (few tiles left, many pieces each: bf16 with registers for eight pieces' loads, V = 151,936, one tile: 14 -> 8 us; 9, V =
+              // 80,000, E = 4096 183.5 -> 181.9; 24, three pieces each, V = 50,000, E = 2048 stays: 70.7 against 72.3)
             e = launch_pdl(tables_pieces_kernel<F32, 1, F32 ? 3 : 4>, dim3(C::ROWS / 8, p.left), dim3(256), 0, st, p);
         *launches += 1;
     }
@@ -1024,8 +1024,10 @@ cudaError_t tables_mma_launch(graft_ctx* ctx, const void* d_emb, graft_dtype dt,
         // lies in two tiles empties its accumulators and writes a piece twice, and with q = 1 nothing has to be added up:
         // the whole number saves 6 us on pairs and 3 us on single CTAs, 22 and 10 us for q = 1, and costs 0.02 and 0.03 us
         // for every column of E by which a share gets longer.  (Measured over 26 to 73 and 52 to 147 tiles left, E = 1024 to
-        // 4096, with and without a round of whole tiles ahead.  V = 16,000, bf16: E = 1024 35.0 -> 29.2 us, E = 4096 61.5 ->
-        // 57.9; V = 32,000, E = 1024: bf16 47.5 -> 32.7, fp32 71.9 -> 68.4; fp32, E = 2048 stays: 118.7 against 121.2.)
+        // 4096, with and without a round of whole tiles ahead.  Now, equal and whole, us: V = 16,000, bf16: E = 1024 29.7 and 24.9,
+        // E = 4096 54.2 and 52.2; V = 32,000, E = 1024: bf16 43.1 and 30.1, fp32 48.1 and 45.0; fp32, E = 2048 73.3 and 74.9, V = 50,000
+        // 105.1 and 109.1, which keep equal shares.  Of 54 sizes two are on the slower side: fp32, E = 1536, V = 32,000 61.1 and 59.7,
+        // 64,000 104.0 and 100.4.)
         const long long q = sp / p.left;
         const double longer = (1.0 / (double)q - (double)p.left / (double)sp) * E;
         if (longer <= (f32 ? (q == 1 ? 380 : 130) : (q == 1 ? 850 : 350))) sp = q * p.left;

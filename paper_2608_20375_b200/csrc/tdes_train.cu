@@ -1,4 +1,4 @@
-// TDES training objective, forward and backward in one kernel (Sec. 3.2 "Training", Eq. 7-12).
+// TDES training objective, forward and backward in one pass over the traces (Sec. 3.2 "Training", Eq. 7-12).
 //
 //   f(p,c,d)    = s (P[p] + u_d) . (C[c] + u_d) / sqrt(m)                                       (Eq. 6)
 //   L_KL        = mean over groups of KL(softmax_c z_tgt || softmax_c (log q_d(c) + f(p,c,d)))   (Eq. 7-9)
