@@ -326,9 +326,12 @@ __global__ void __launch_bounds__(kTrThreads) tdes_loss_kernel(const TrainParams
 // Many traces have kernels of their own, further down.
 constexpr int kTsThreads = 384;
 constexpr int kTsWarps = kTsThreads / 32;
-// References to rows from which the two kernels for many traces are used: with gradients (K = 32: 98 thousand 35.5 us by the
-// kernel below and 37.5 by the two, 130 thousand 39.6 and 39.7, 195 thousand 57.7 and 47.4) and for the losses alone (260
-// thousand 21.0 and 29.2, 520 thousand 35.4 and 37.4, a million 63.7 and 56.5).
+// References to rows from which the two kernels for many traces are used.  With gradients (K = 32, tokens by a power of 1.1 of their
+// rank, the kernel below and the two, us: 98 thousand 30.3 and 34.2, 130 thousand 33.8 and 37.3, 163 thousand 38.6 and 41.6, 195
+// thousand 47.2 and 43.9, 293 thousand 59.2 and 57.8; by 1.6 195 thousand 42.2 and 45.0, 293 thousand 53.3 and 58.4) the line lies
+// below where their times meet, because the two add to a row of gC less often (error against 64 bits, 163 thousand: 3.3e-7 and
+// 2.5e-7, 260 thousand 3.8e-7 and 2.6e-7).  For the losses alone: 260 thousand 21.0 and 29.2, 520 thousand 35.4 and 37.4, a million
+// 63.7 and 56.5.
 constexpr long long kTsMany = 131072, kTsManyLoss = 655360;
 // References to rows from which, with gradients, the frequent tokens' rows are summed up on chip (below it a step is over before a
 // sample is worth its 1.5 us: 65 thousand references 21.5 us).
