@@ -10,8 +10,9 @@
 // diagonal first, then Gauss-Jordan elimination with partial pivoting) and clears the accumulators for the next call.
 //
 // 28 bytes are read a tuple and some 55 fp64 operations done on it: with the next tuples' loads in flight and the table of logarithms
-// kept by the context a million tuples take 4.4 us (6.3 TB/s, the copy rate; 5.2 without), and a call costs 7 us however few:
-// launch, exchange, one round of atomics, the systems.  4 million tuples on a B200, one call after another: 30.0 -> 25.2 us, of
+// kept by the context a million tuples take 4.4 us (6.3 TB/s, the copy rate; 5.2 without), and a call costs 6 us however few:
+// launch, exchange, one round of atomics, the systems (half the threads a CTA for few rounds and the table fetched while the kernel ahead runs: 20,000
+// rounds captured 7.5 -> 6.3 us, 100 5.9 -> 5.4).  4 million tuples on a B200, one call after another: 30.0 -> 25.2 us, of
 // which 2.5 are the launch behind the call before (one CTA of 512 threads an SM and two of 256 are alike from 200,000 tuples on; the
 // CTAs' sums written out and added up in order by the last CTA instead of by atomics: 3 us slower at a million).  Before: 37.3 ->
 // 28.9 with logarithms from a table and a short series instead of log, one division for four quotients and whole numbers converted
@@ -26,7 +27,11 @@
 namespace graft {
 namespace {
 
-constexpr int kFitThreads = 512;  // one CTA an SM
+constexpr int kFitThreads = 512, kFitFew = 256;  // one CTA an SM
+// Turns of a thread (four rounds, or one where the arrays are not aligned) from which a CTA has the larger number: with few, warps that
+// have next to nothing to add up take their part in the exchange all the same.  256 and 512, captured, us: four rounds a turn, 20,000 rounds 6.8
+// and 7.4, 100,000 6.8 and 7.4, 130,000 7.3 both, 200,000 7.8 and 7.5; one, 20,000 6.3 and 6.6, 40,000 7.1 and 6.9, 400,000 12.2 and 9.3.
+constexpr long long kFitMany = 1 << 15;
 constexpr int kFitAcc = 25;  // gain: 10 (upper triangle of 4 x 4) + 4 + 1 count; cost: 6 + 3 + 1 count
 
 struct FitParams {
@@ -138,16 +143,17 @@ __device__ __forceinline__ void fit_accumulate(FitSums& t, float s0, float s1, f
 }
 
 // VEC: every array is 16-byte aligned, so a thread takes four consecutive rounds with seven 16-byte loads
-template <bool VEC>
-__global__ void __launch_bounds__(kFitThreads, 1) saba_fit_kernel(const FitParams p) {
-    constexpr int W = kFitThreads / 32;
+template <bool VEC, int T>
+__global__ void __launch_bounds__(T, 1) saba_fit_kernel(const FitParams p) {
+    constexpr int W = T / 32;
     __shared__ double2 s_log[kFitLog];
     __shared__ double s_acc[kFitAcc], s_warp[W][kFitAcc];
     __shared__ bool s_last;
     __shared__ int s_bad[2];
     pdl_launch_dependents();
+    for (int i = threadIdx.x; i < kFitLog; i += T) s_log[i] = p.log[i];  // (written once, by graft_create)
     pdl_wait();  // (the logs may come from the kernel ahead, and the one before this may still add up)
-    const long long tid = blockIdx.x * (long long)kFitThreads + threadIdx.x, nth = (long long)gridDim.x * kFitThreads;
+    const long long tid = blockIdx.x * (long long)T + threadIdx.x, nth = (long long)gridDim.x * T;
     const long long n4 = VEC ? p.n / 4 : 0;
     // the next four rounds are on their way while four are worked on, the first beside the table
     float4 a, b, c, ga, la;
@@ -159,7 +165,6 @@ __global__ void __launch_bounds__(kFitThreads, 1) saba_fit_kernel(const FitParam
         ga = __ldg((const float4*)p.gain + q), la = __ldg((const float4*)p.latency + q);
     };
     if (VEC) fetch(tid);
-    if (threadIdx.x < kFitLog) s_log[threadIdx.x] = p.log[threadIdx.x];
     __syncthreads();
     FitSums t;
 #pragma unroll
@@ -276,11 +281,15 @@ cudaError_t saba_fit_launch(graft_ctx* ctx, long long n, const float* d_state, c
     p.out = d_out;
     const bool vec = (((uintptr_t)d_state | (uintptr_t)d_budget | (uintptr_t)d_gain | (uintptr_t)d_prefix |
                        (uintptr_t)d_latency) & 15) == 0;
-    long long grid = ((vec ? n / 4 + 3 : n) + kFitThreads - 1) / kFitThreads;
+    const long long turns = vec ? n / 4 + 3 : n;
+    const int threads = turns < kFitMany ? kFitFew : kFitThreads;
+    long long grid = (turns + threads - 1) / threads;
     const long long cap = ctx->num_sms;
     if (grid > cap) grid = cap;
     if (grid < 1) grid = 1;
-    const cudaError_t e = launch_pdl(vec ? saba_fit_kernel<true> : saba_fit_kernel<false>, dim3((int)grid), dim3(kFitThreads), 0, st, p);
+    void (*kern)(const FitParams) = turns < kFitMany ? (vec ? saba_fit_kernel<true, kFitFew> : saba_fit_kernel<false, kFitFew>)
+                                                 : (vec ? saba_fit_kernel<true, kFitThreads> : saba_fit_kernel<false, kFitThreads>);
+    const cudaError_t e = launch_pdl(kern, dim3((int)grid), dim3(threads), 0, st, p);
     ctx->launches += 1;
     return e != cudaSuccess ? e : cudaGetLastError();
 }

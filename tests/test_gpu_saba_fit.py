@@ -110,3 +110,26 @@ def test_sizes_around_whole_turns_back_to_back(n):
         assert np.all(np.abs(got[i, :4] - ref["phi"]) <= RTOL * np.abs(ref["phi"]).max() * 10)
         assert np.all(np.abs(got[i, 4:7] - ref["c"]) <= RTOL * np.maximum(np.abs(ref["c"]), 1e-9) * 100)
     g.destroy()
+
+
+@pytest.mark.parametrize("n,odd", [(257, False), (1021, True), (131056, False), (131060, False), (131063, False), (32767, True), (32768, True)])
+def test_sizes_where_the_thread_blocks_change(n, odd):
+    """The last size of the smaller thread blocks and the first of the larger, with four rounds a turn and with one."""
+    g = _ctx()
+    lg = gi.saba_replay_logs(n, seed=n)
+    ref = oracle.saba_fit(**lg)
+    dev = {}
+    for k, v in lg.items():  # (four bytes behind a boundary: one round a turn)
+        flat = torch.from_numpy(np.ascontiguousarray(v)).reshape(-1)
+        buf = torch.zeros(flat.numel() + 1, dtype=flat.dtype, device="cuda")
+        part = buf[1:] if odd else buf[:-1]
+        part.copy_(flat)
+        dev[k] = part.view(v.shape)
+    out = torch.zeros((3, 10), dtype=torch.float64, device="cuda")
+    for i in range(3):
+        g.saba_fit(dev["state"], dev["budget"], dev["gain"], dev["prefix_len"], dev["latency"], out[i])
+    for got in out.cpu().numpy():
+        assert got[9] == 0.0 and got[7] == ref["n_gain"] and got[8] == ref["n_cost"]
+        assert np.all(np.abs(got[:4] - ref["phi"]) <= RTOL * np.abs(ref["phi"]).max() * 10)
+        assert np.all(np.abs(got[4:7] - ref["c"]) <= RTOL * np.maximum(np.abs(ref["c"]), 1e-9) * 100)
+    g.destroy()
