@@ -168,8 +168,17 @@ graft_status graft_create(const graft_config* cfg, graft_ctx** out) {
     }
     double fit_table[2 * kFitLog];
     saba_fit_table(fit_table);
-    if (cudaMemset(ctx->ws, 0, ctx->ws_bytes) != cudaSuccess ||
-        cudaMemcpy((char*)ctx->ws + o_fit, fit_table, sizeof fit_table, cudaMemcpyHostToDevice) != cudaSuccess) {
+    // (waited for on a stream of its own: a small copy from pageable memory may return before it has arrived, and the context's
+    // first call may come on a stream that does not wait for the default one)
+    cudaStream_t init = nullptr;
+    bool ready = cudaStreamCreateWithFlags(&init, cudaStreamNonBlocking) == cudaSuccess;
+    if (ready) {
+        ready = cudaMemsetAsync(ctx->ws, 0, ctx->ws_bytes, init) == cudaSuccess &&
+                cudaMemcpyAsync((char*)ctx->ws + o_fit, fit_table, sizeof fit_table, cudaMemcpyHostToDevice, init) == cudaSuccess;
+        ready = cudaStreamSynchronize(init) == cudaSuccess && ready;
+        cudaStreamDestroy(init);
+    }
+    if (!ready) {
         cudaGetLastError();
         cudaFree(ctx->ws);
         delete extra_of(ctx);

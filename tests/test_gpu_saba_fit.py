@@ -133,3 +133,27 @@ def test_sizes_where_the_thread_blocks_change(n, odd):
         assert np.all(np.abs(got[:4] - ref["phi"]) <= RTOL * np.abs(ref["phi"]).max() * 10)
         assert np.all(np.abs(got[4:7] - ref["c"]) <= RTOL * np.maximum(np.abs(ref["c"]), 1e-9) * 100)
     g.destroy()
+
+
+def test_first_call_on_a_stream_of_its_own_behind_a_busy_default_stream():
+    """A context is ready when its creation returns: the first call need not wait for the default stream, nor for what is queued there."""
+    lg = gi.saba_replay_logs(900, seed=3)
+    ref = oracle.saba_fit(**lg)
+    dev = {k: torch.from_numpy(np.ascontiguousarray(v)).cuda() for k, v in lg.items()}
+    out = torch.zeros((20, 10), dtype=torch.float64, device="cuda")
+    a = torch.ones((4096, 4096), device="cuda")
+    side = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    made = []
+    for i in range(20):
+        for _ in range(20):
+            a.mul_(1.0)
+        made.append(_ctx())
+        with torch.cuda.stream(side):
+            made[-1].saba_fit(dev["state"], dev["budget"], dev["gain"], dev["prefix_len"], dev["latency"], out[i])
+    torch.cuda.synchronize()
+    for got in out.cpu().numpy():
+        assert got[9] == 0.0 and got[7] == ref["n_gain"] and got[8] == ref["n_cost"]
+        assert np.all(np.abs(got[:4] - ref["phi"]) <= RTOL * np.abs(ref["phi"]).max() * 10)
+    for g in made:
+        g.destroy()
